@@ -291,3 +291,99 @@ def tolerance(case):
     # fp32 sums: 1.8e-3 to 2.2e-3 from the same attention in 64 bits (largest difference 0.043 of the root mean square);
     # hop by hop, with the running result rounded to bf16 after every merge, 4.2e-3 from the one-call result.
     return {"rel": 1.6e-2 if case["kind"] == "consumer" else 8e-3, "max": 0.15}
+
+
+def _placement(case, n_blocks, n_video):
+    """Rank of every block, as the library's placement functions define it."""
+    P, j = case["ranks"], torch.arange(n_blocks, dtype=torch.int64)
+    if case["placement"] == "contiguous":
+        return j * P // n_blocks
+    if case["placement"] == "shuffle":
+        return synth.shuffled_placement(n_blocks, P, seed=1).long()
+    first, frame = j * case["block"], case["grid_h"] * case["grid_w"]
+    return torch.where(first >= n_video, j % P, P * (first % frame) // frame)
+
+
+def _kept_blocks(case, q, k, n_cand):
+    """Kept KV blocks [heads][NB][NB] of q, k [heads][NB][b][d] (zeros behind the last token): fp32 sums in token and
+    channel order as the selection is defined, everything else in 64 bits."""
+    NB, b, n = q.shape[1], case["block"], case["tokens"]
+    count = torch.full((NB, 1), float(b), device=q.device)
+    count[-1] = n - (NB - 1) * b
+
+    def pooled(x):
+        acc = torch.zeros_like(x[:, :, 0], dtype=torch.float32)
+        for t in range(b):
+            acc = acc + x[:, :, t].float()
+        return (acc / count).double()
+
+    pq, pk = pooled(q), pooled(k)
+    score = torch.zeros(q.shape[0], NB, NB, dtype=torch.float32, device=q.device)
+    for c in range(q.shape[-1]):
+        score = (score.double() + pq[:, :, None, c] * pk[:, None, :, c]).float()
+    score = score[:, :, :n_cand]
+    kept = torch.ones(q.shape[0], NB, NB, dtype=torch.bool, device=q.device)
+    top, order = torch.sort(score, dim=-1, descending=True, stable=True)
+    if case["tau"]:
+        scale = torch.tensor(1.0 / math.sqrt(q.shape[-1])) * torch.tensor(1.4426950408889634)
+        weight = torch.floor(torch.exp2((top - top[..., :1]).double() * scale.double().item()) * 2.0 ** 26)
+        mass = torch.cumsum(weight, -1)
+        theta = torch.ceil(torch.tensor(case["tau"]).double().item() * mass[..., -1:])
+        last = torch.argmax((mass >= theta).to(torch.uint8), -1, keepdim=True)
+        kept[:, :, :n_cand] = score >= torch.gather(top, -1, last)
+    else:
+        topk = case["topk"] or max(1, (case["pct"] * n_cand + 99) // 100)
+        kept[:, :, :n_cand] = False
+        kept[:, :, :n_cand].scatter_(-1, order[..., :topk], True)
+    return kept
+
+
+def _attention(q, k, v, kept, tokens):
+    """One head: q, k, v [NB][b][d], kept [NB][NB] -> output [NB][b][d] and log-sum-exp [NB][b], in 64 bits."""
+    NB, b, d = q.shape
+    O = torch.zeros(NB, b, d, dtype=torch.float64, device=q.device)
+    lse = torch.full((NB, b), float("-inf"), dtype=torch.float64, device=q.device)
+    k, v = k.double(), v.double()
+    col = torch.arange(NB * b, device=q.device).view(NB, b) < tokens
+    n_kept = kept.sum(-1)
+    rows = torch.nonzero(n_kept, as_tuple=True)[0]
+    rows = rows[torch.argsort(n_kept[rows])]  # rows of similar length together
+    at = 0
+    while at < rows.numel():
+        most = int(n_kept[rows[min(at + 63, rows.numel() - 1)]])
+        r = rows[at:at + max(1, min(64, (1 << 28) // (most * b * max(b, d))))]
+        at += r.numel()
+        live, block = torch.sort(kept[r].to(torch.uint8), dim=-1, descending=True, stable=True)
+        live, block = live[:, :most].bool(), block[:, :most]
+        s = torch.matmul(q[r].double(), k[block].flatten(1, 2).transpose(1, 2)) / math.sqrt(d)
+        s.masked_fill_(~(live[..., None] & col[block]).flatten(1)[:, None], float("-inf"))
+        lse[r] = torch.logsumexp(s, -1)
+        O[r] = torch.matmul(torch.exp(s - lse[r][..., None]), v[block].flatten(1, 2))
+    return O, lse
+
+
+def exact(case, seed):
+    """The attention output and its log-sum-exp in 64 bits; everything else that a pass returns is whole numbers or bytes."""
+    kind, H, B, d, b = case["kind"], case["heads"], case["batch"], case["head_dim"], case["block"]
+    if kind in ("producer", "plan"):
+        return None
+    n_video = case["grid_t"] * case["grid_h"] * case["grid_w"]
+    n = n_video + case["n_text"]
+    NB = (n + b - 1) // b
+    n_cand = n_video // b if case["n_text"] else NB
+    nhd = case["layout"] == "NHD"
+    Q, K, V = _inputs(case, seed, H)
+    mine = torch.ones(NB, dtype=torch.bool, device=Q.device)
+    if kind != "layer":
+        mine = (_placement(case, NB, n_video) == case["rank"]).to(Q.device)
+    O = torch.zeros(Q.shape, dtype=torch.float64, device=Q.device)
+    lse = torch.full((B, H, n), float("-inf"), dtype=torch.float64, device=Q.device)
+    for bb in range(B):
+        for h in range(H):
+            q, k, v = ((x[bb, :, h] if nhd else x[bb, h]) for x in (Q, K, V))
+            q, k, v = (torch.nn.functional.pad(x, (0, 0, 0, NB * b - n)).view(NB, b, d) for x in (q, k, v))
+            kept = _kept_blocks(dict(case, tokens=n), q[None], k[None], n_cand)[0] & mine[:, None]
+            o, l = _attention(q, k, v, kept, n)
+            (O[bb, :, h] if nhd else O[bb, h]).copy_(o.flatten(0, 1)[:n])
+            lse[bb, h] = l.flatten()[:n]
+    return {"O": O, "lse": lse} if case["lse"] or kind != "layer" else {"O": O}
