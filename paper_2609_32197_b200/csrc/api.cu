@@ -121,14 +121,10 @@ WsLayout make_layout(const Geometry& g, int P) {
   off += align_up((int64_t)g.B * 8, 256);
   L.knorm = off;  // largest key norm of every KV block, fp32 [B][H][NB] (attention: bound on the scores of a tile)
   off += align_up((int64_t)g.B * g.H * g.NB * 4, 256);
-  L.own = off;
-  off += align_up((int64_t)P * g.Wd * 4, 256);
-  L.ent_base = off;
-  off += align_up((int64_t)g.B * P * 8, 256);
-  L.n_entries = off;
+  L.n_entries = off;  // blocks that anybody receives, int32
   off += 256;
-  L.entries = off;
-  off += align_up((int64_t)g.B * P * g.H * g.NB * (int64_t)sizeof(PackEntry), 256);
+  L.entries = off;  // destinations of every block, int64 [B][H][NB][P], and the list of those blocks, int32 [B][H][NB]
+  off += align_up((int64_t)g.B * P * g.H * g.NB * 16, 256);
   L.total = off;
   return L;
 }
@@ -417,7 +413,7 @@ int sparsp_demand_pack(const sparsp_shape* shape, const uint32_t* mask, const in
   SPARSP_TRY(launch_demand(g, mask, rank_of_block, n_ranks, flags, union_mask, cnt, seg_offset,
                            seg_total, volume_bytes, dst_base_bytes,
                            plan_only ? (int64_t)-1 : packed_capacity_bytes, ws, L, st));
-  if (!plan_only) SPARSP_TRY(launch_pack(*shape, g, K, V, packed, packed_capacity_bytes, n_ranks, ws, L, st));
+  if (!plan_only) SPARSP_TRY(launch_pack(*shape, g, K, V, packed, n_ranks, ws, L, st));
   return SPARSP_OK;
 }
 

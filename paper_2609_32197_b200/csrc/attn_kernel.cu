@@ -1146,21 +1146,23 @@ static EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
-// bf16 tensor viewed as (d, N, H, B) with a box of (64, rows, 1, 1) and 128-byte swizzle.
-static int make_tmap(CUtensorMap* out, const void* base, const sparsp_shape& s, const Geometry& g, int rows) {
+// bf16 tensor viewed as (d, N, H, B) with a box of (d, rows, 1, 1), or of (64, rows, 1, 1) and 128-byte swizzle.
+// A dimension of extent 1 takes a stride of its own choice (whatever the caller has there is never used).
+int make_tile_tmap(CUtensorMap* out, const void* base, const sparsp_shape& s, const Geometry& g, int rows,
+                   bool swizzled) {
   EncodeTiledFn enc = get_encode_fn();
   if (!enc) {
     set_error("cuTensorMapEncodeTiled is not available from the driver");
     return SPARSP_ERR_CUDA;
   }
   cuuint64_t dims[4] = {(cuuint64_t)g.d, (cuuint64_t)g.N, (cuuint64_t)g.H, (cuuint64_t)g.B};
-  const int64_t batch_stride = s.stride_batch > 0 ? s.stride_batch : g.N * s.stride_token;
-  cuuint64_t strides[3] = {(cuuint64_t)s.stride_token * 2, (cuuint64_t)s.stride_head * 2,
-                           (cuuint64_t)batch_stride * 2};
-  cuuint32_t box[4] = {64, (cuuint32_t)rows, 1, 1};
+  const int64_t head_stride = g.H > 1 ? s.stride_head : s.stride_token;
+  const int64_t batch_stride = g.B > 1 ? s.stride_batch : s.stride_token;
+  cuuint64_t strides[3] = {(cuuint64_t)s.stride_token * 2, (cuuint64_t)head_stride * 2, (cuuint64_t)batch_stride * 2};
+  cuuint32_t box[4] = {swizzled ? 64u : (cuuint32_t)g.d, (cuuint32_t)rows, 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzled ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_error("cuTensorMapEncodeTiled failed with %d", (int)r);
@@ -1201,9 +1203,9 @@ static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q
                          const void* packed, int64_t packed_capacity, const AttnParams& p, cudaStream_t st) {
   CUtensorMap tq, tk, tv, tp;
   int rc;
-  if ((rc = make_tmap(&tq, Q, s, g, BLK)) != SPARSP_OK) return rc;
-  if ((rc = make_tmap(&tk, K, s, g, BLK)) != SPARSP_OK) return rc;
-  if ((rc = make_tmap(&tv, V, s, g, BLK)) != SPARSP_OK) return rc;
+  if ((rc = make_tile_tmap(&tq, Q, s, g, BLK, true)) != SPARSP_OK) return rc;
+  if ((rc = make_tile_tmap(&tk, K, s, g, BLK, true)) != SPARSP_OK) return rc;
+  if ((rc = make_tile_tmap(&tv, V, s, g, BLK, true)) != SPARSP_OK) return rc;
   if (packed) {
     if ((rc = make_packed_tmap(&tp, packed, packed_capacity, g)) != SPARSP_OK) return rc;
   } else {

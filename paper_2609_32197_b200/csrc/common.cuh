@@ -1,6 +1,7 @@
 // Shared host-side plumbing of the SparSP library: geometry, error reporting, workspace layout.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -26,15 +27,8 @@ struct Geometry {
   int32_t B, H, d, b;
 };
 
-// One 16-byte record per packed entry, in pack order.
-struct PackEntry {
-  int64_t dst_byte;  // byte offset of the entry's K tile inside `packed`
-  int32_t bh;        // batch * H + head
-  int32_t j;         // KV block
-};
-
 struct WsLayout {
-  int64_t status, pooled_q, pooled_k, scores, pairs, slot, tile_base, knorm, own, ent_base, n_entries, entries, total;
+  int64_t status, pooled_q, pooled_k, scores, pairs, slot, tile_base, knorm, n_entries, entries, total;
 };
 
 void set_error(const char* fmt, ...);
@@ -58,6 +52,9 @@ inline int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
     if (e__ != cudaSuccess) return cuda_fail(e__, #call); \
   } while (0)
 
+int make_tile_tmap(CUtensorMap* out, const void* base, const sparsp_shape& s, const Geometry& g, int rows,
+                   bool swizzled);
+
 // launchers implemented in the kernel files -------------------------------------------------
 int launch_pool(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, float* pq,
                 float* pk, cudaStream_t st);
@@ -74,8 +71,8 @@ int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_o
                   int flags, uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total,
                   int64_t* volume, const int64_t* dst_base, int64_t capacity, char* ws,
                   const WsLayout& L, cudaStream_t st);
-int launch_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, void* packed,
-                int64_t capacity, int P, char* ws, const WsLayout& L, cudaStream_t st);
+int launch_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, void* packed, int P, char* ws,
+                const WsLayout& L, cudaStream_t st);
 int launch_pack_segment(const sparsp_shape& s, const Geometry& g, const uint32_t* U, const int32_t* rank, int P,
                         int consumer, int producer, const int64_t* seg_off, const int32_t* cnt, const void* K,
                         const void* V, void* dst, int64_t capacity, char* ws, const WsLayout& L, cudaStream_t st);

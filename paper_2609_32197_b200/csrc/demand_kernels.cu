@@ -1,549 +1,407 @@
 // Step 2: per-rank per-head unions of required KV blocks, demand counts, exchange volume,
-// pack-order offsets, the entry table, and the gather of K/V tiles into per-consumer buffers.
+// pack-order offsets, the destination table, and the gather of K/V tiles into per-consumer buffers.
 // Everything before the gather is small integer work on bit words; the gather is the HBM-bound part.
 #include <algorithm>
-#include <mutex>
 
+#include "block_sets.cuh"
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
 namespace sparsp {
 
-// One CTA per (batch, head) computes, for that head,
-//   own[p][w]     : bit j set iff rank_of_block[j] == p                      (CTA 0 also writes it out)
+// One CTA per (batch, head, rank r) computes
 //   U[b][r][h][w] = OR over the query blocks i of rank r of M[b][h][i][w]
-//   cnt[b][r][p][h] = popcount(U[b][r][h] & own[p])
-// The head's mask rows are read once, coalesced, and OR-ed into a [P][Wd] table in shared memory (at most
-// 64 ranks x 32 words = 8 KiB; OR does not depend on the order, so the bits are well defined); the ownership
-// words are rebuilt per CTA from the rank table (a few thousand compares) rather than fetched from an earlier
-// launch.  A rank value outside [0, P) is ignored.
-constexpr int kUnionThreads = 1024;
-static_assert(2 * kMaxRanks * (kMaxBlocks / 32) * 4 <= 48 * 1024, "union and ownership tables must fit shared memory");
+//   cnt[b][r][p][h] = popcount(U[b][r][h] & own[p]),  own[p] = the blocks of rank p
+// It reads the rows of its own query blocks only, whole words per lane (a row of up to 32 words is one coalesced
+// request, shorter rows share one), so a mask row is read once in all and B*H*P CTAs are in flight; the ownership
+// words are rebuilt per CTA from the rank table.  Latency-bound: the mask is a few MB.  (One CTA per (batch, head) with
+// shared-memory atomics for all ranks at once: 20.6 us on 24 heads x 929 blocks, 8 ranks, 24 CTAs on 148 SMs; this split
+// 8 us.)  OR does not depend on the order, so the bits are well defined.  A rank value outside [0, P) is ignored.
+constexpr int kUnionThreads = 512;
 
 __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32_t* __restrict__ mask,
                                                                     const int32_t* __restrict__ rank, int H, int NB,
-                                                                    int Wd, int P, uint32_t* __restrict__ own,
-                                                                    uint32_t* __restrict__ U,
-                                                                    int32_t* __restrict__ cnt) {
-  extern __shared__ uint32_t tab[];
-  uint32_t* u_s = tab;             // [P][Wd]
-  uint32_t* own_s = tab + P * Wd;  // [P][Wd]
-  const int bh = blockIdx.x, bb = bh / H, h = bh % H;
-  for (int idx = threadIdx.x; idx < P * Wd; idx += kUnionThreads) {
-    const int p = idx / Wd, w = idx - p * Wd;
-    uint32_t bits = 0;
-    for (int t = 0; t < 32; ++t) {
-      const int j = w * 32 + t;
-      if (j < NB && rank[j] == p) bits |= 1u << t;
-    }
-    own_s[idx] = bits;
-    u_s[idx] = 0u;
-    if (bh == 0) own[idx] = bits;
-  }
+                                                                    int Wd, int P, uint32_t* __restrict__ U,
+                                                                    int32_t* __restrict__ cnt,
+                                                                    int32_t* __restrict__ n_src) {
+  __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
+  __shared__ uint32_t u_s[kMaxWords];
+  __shared__ uint16_t rows_s[kMaxBlocks];
+  __shared__ int n_rows_s;
+  const int r = blockIdx.x % P, bh = blockIdx.x / P, bb = bh / H, h = bh % H;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = kUnionThreads / 32;
+  if (threadIdx.x == 0) n_rows_s = 0;
+  if (threadIdx.x < kMaxWords) u_s[threadIdx.x] = 0u;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && n_src) *n_src = 0;
+  own_words(rank, NB, Wd, P, own_s);
+  for (int i = threadIdx.x; i < NB; i += kUnionThreads)
+    if (rank[i] == r) rows_s[atomicAdd(&n_rows_s, 1)] = (uint16_t)i;
   __syncthreads();
+  int width = 1;  // lanes per row: the next power of two
+  while (width < Wd) width <<= 1;
+  const int per_warp = 32 / width, w = lane & (width - 1), sub = lane / width;
   const uint32_t* m = mask + (int64_t)bh * NB * Wd;
-  for (int idx = threadIdx.x; idx < NB * Wd; idx += kUnionThreads) {
-    const int i = idx / Wd, w = idx - i * Wd;
-    const uint32_t v = m[idx];
-    const int r = rank[i];
-    if (v != 0u && (unsigned)r < (unsigned)P) atomicOr(&u_s[r * Wd + w], v);
-  }
+  uint32_t acc = 0;
+  const int n_rows = n_rows_s;
+#pragma unroll 4
+  for (int k = warp * per_warp + sub; k < n_rows; k += n_warps * per_warp)
+    if (w < Wd) acc |= m[(int64_t)rows_s[k] * Wd + w];
+  for (int s = width; s < 32; s <<= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, s);
+  if (lane < Wd && acc) atomicOr(&u_s[lane], acc);
   __syncthreads();
-  for (int idx = threadIdx.x; idx < P * Wd; idx += kUnionThreads) {
-    const int r = idx / Wd, w = idx - r * Wd;
-    U[((int64_t)(bb * P + r) * H + h) * Wd + w] = u_s[idx];
-  }
-  for (int idx = threadIdx.x; idx < P * P; idx += kUnionThreads) {
-    const int r = idx / P, p = idx - r * P;
-    int c = 0;
-    for (int w = 0; w < Wd; ++w) c += __popc(u_s[r * Wd + w] & own_s[p * Wd + w]);
-    cnt[((int64_t)(bb * P + r) * P + p) * H + h] = c;
+  const uint32_t u = lane < Wd ? u_s[lane] : 0u;
+  if (warp == 0 && lane < Wd) U[((int64_t)(bb * P + r) * H + h) * Wd + lane] = u;
+  for (int p = warp; p < P; p += n_warps) {
+    const int c = __reduce_add_sync(0xffffffffu, lane < Wd ? __popc(u & own_s[p * Wd + lane]) : 0);
+    if (lane == 0) cnt[((int64_t)(bb * P + r) * P + p) * H + h] = c;
   }
 }
 
-static void launch_union_count(const uint32_t* mask, const int32_t* rank, const Geometry& g, int P, uint32_t* own,
-                               uint32_t* U, int32_t* cnt, cudaStream_t st) {
-  union_count_kernel<<<g.B * g.H, kUnionThreads, (size_t)2 * P * g.Wd * 4, st>>>(mask, rank, g.H, g.NB, g.Wd, P, own,
-                                                                                 U, cnt);
-}
+// Pack-order offsets, and where every packed tile goes.  A CTA per consumer scans its consumer's counts in pack
+// order (producer, then head) and writes offsets, total and volume.  With `dst` given there are consumers + batch items
+// CTAs per head: CTA (consumer, h) also fills its column of the destination table
+//   dst[(b*H + h)*NB + j][r] = byte offset in `packed` of consumer r's copy of block j, or -1
+// one warp per producer (the consumer's base is its caller-given dst_base or the sum of all earlier consumers' counts),
+// and CTA (B*P + b, h) appends the blocks that any consumer of batch item b receives to the list of sources, a head's
+// blocks together.  The order of the heads in that list is the order in which they arrive; it decides nothing but the
+// order of the copies.
+// Latency-bound integer work on a few MB, so every CTA repeats the scan (P*H counts) rather than wait for another
+// launch.  (A serial scan per consumer in one CTA and a launch for the entries: 13 + 7 us on 24 heads, 8 ranks, 18 + 4 us on 48
+// heads; offsets alone 2 us now, with destinations 9 us on 48 and 15 us on 24 heads; eight heads to a CTA, one warp each: 16-19 us.)
+constexpr int kPlanThreads = 256;
 
-// One thread per (b, r): exclusive scan of cnt over (p, h) in pack order, totals and volume; then
-// thread 0 turns the totals into table bases.  Sizes are tiny (P*H values per thread).
-__global__ void scan_kernel(const int32_t* __restrict__ cnt, int B, int H, int P, int include_local,
-                            int64_t entry_bytes, int64_t* __restrict__ seg_off,
-                            int64_t* __restrict__ seg_total, int64_t* __restrict__ volume,
-                            int64_t* __restrict__ ent_base, int64_t* __restrict__ n_entries) {
-  const int idx = threadIdx.x;
-  if (idx < B * P) {
-    const int r = idx % P;
-    int64_t cursor = 0, remote = 0;
-    for (int p = 0; p < P; ++p) {
-      for (int h = 0; h < H; ++h) {
-        const int64_t o = ((int64_t)idx * P + p) * H + h;
-        const int c = cnt[o];
-        seg_off[o] = cursor;
-        if (p != r) remote += c;
-        if (p != r || include_local) cursor += c;
-      }
-    }
-    seg_total[idx] = cursor;
-    volume[idx] = entry_bytes * remote;
-  }
+__device__ __forceinline__ int64_t block_sum(int64_t v, int64_t* warp_s) {
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
   __syncthreads();
-  if (idx == 0) {
-    int64_t base = 0;
-    for (int t = 0; t < B * P; ++t) {
-      ent_base[t] = base;
-      base += seg_total[t];
-    }
-    *n_entries = base;
-  }
+  if ((threadIdx.x & 31) == 0) warp_s[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int64_t t = 0;
+#pragma unroll
+  for (int k = 0; k < kPlanThreads / 32; ++k) t += warp_s[k];
+  return t;
 }
 
-// Entry table: one warp per (b, r, p, h) segment enumerates the set bits of U & own[p] in ascending
-// order and writes entry records at table index ent_base[b,r] + seg_off + t.
-__global__ void entries_kernel(const uint32_t* __restrict__ U, const uint32_t* __restrict__ own, int B,
-                               int H, int Wd, int P, int include_local, int64_t entry_bytes,
-                               const int64_t* __restrict__ seg_off, const int64_t* __restrict__ ent_base,
-                               const int64_t* __restrict__ dst_base, int64_t capacity,
-                               PackEntry* __restrict__ entries, int32_t* __restrict__ status) {
-  const int64_t seg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int64_t n_seg = (int64_t)B * P * P * H;
-  if (seg >= n_seg) return;
-  const int h = (int)(seg % H);
-  const int p = (int)((seg / H) % P);
-  const int r = (int)((seg / ((int64_t)H * P)) % P);
-  const int bb = (int)(seg / ((int64_t)H * P * P));
-  if (p == r && !include_local) return;
-  const uint32_t* u = U + ((int64_t)(bb * P + r) * H + h) * Wd;
-  const uint32_t* o = own + (int64_t)p * Wd;
-  const int64_t br = (int64_t)bb * P + r;
-  const int64_t first = seg_off[seg];
-  const int64_t base_byte = dst_base ? dst_base[br] : ent_base[br] * entry_bytes;
-  PackEntry* out = entries + ent_base[br] + first;
-  int running = 0;
-  for (int w0 = 0; w0 < Wd; w0 += 32) {
-    const int w = w0 + lane;
-    uint32_t bits = w < Wd ? (u[w] & o[w]) : 0u;
-    const int mine = __popc(bits);
-    int incl = mine;
+__global__ void __launch_bounds__(kPlanThreads) plan_kernel(
+    const int32_t* __restrict__ cnt, const uint32_t* __restrict__ U, const int32_t* __restrict__ rank, int BP, int H,
+    int NB, int Wd, int P, int include_local, int64_t entry_bytes, int64_t* __restrict__ seg_off,
+    int64_t* __restrict__ seg_total, int64_t* __restrict__ volume, const int64_t* __restrict__ dst_base,
+    int64_t capacity, int64_t* __restrict__ dst, int32_t* __restrict__ src, int32_t* __restrict__ n_src,
+    int32_t* __restrict__ status) {
+  __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
+  __shared__ int64_t seg_s[kMaxRanks];  // first entry of (producer, my head)
+  __shared__ int64_t warp_s[kPlanThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n_x = BP + (dst ? BP / P : 0), x = blockIdx.x % n_x, h = blockIdx.x / n_x;
+  if (dst) own_words(rank, NB, Wd, P, own_s);
+  if (x >= BP) {  // the blocks of this head that any consumer receives
+    __syncthreads();
+    if (warp != 0) return;
+    const int bb = x - BP;
+    uint32_t live = 0, owned = 0;
+    if (lane < Wd) {
+      for (int p = 0; p < P; ++p) owned |= own_s[p * Wd + lane];
+#pragma unroll 8
+      for (int r = 0; r < P; ++r)
+        live |= U[((int64_t)(bb * P + r) * H + h) * Wd + lane] & (include_local ? owned : owned & ~own_s[r * Wd + lane]);
+    }
+    int total, first = 0;
+    int at = bits_below(live, lane, &total);
+    if (lane == 0) first = atomicAdd(n_src, total);
+    at += __shfl_sync(0xffffffffu, first, 0);
+    for (; live; live &= live - 1) src[at++] = (bb * H + h) * NB + lane * 32 + __ffs(live) - 1;
+    return;
+  }
+
+  const int br = x, bb = br / P, r = br % P;
+  const int PH = P * H;
+  const bool writer = h == 0;
+  const int32_t* mine = cnt + (int64_t)br * PH;
+  int64_t cursor = 0, remote = 0;  // entries of earlier chunks of this consumer
+  for (int i0 = 0; i0 < PH; i0 += kPlanThreads) {
+    const int i = i0 + (int)threadIdx.x;
+    const int c = i < PH ? mine[i] : 0;
+    const int p = i / H;
+    const int counted = p != r || include_local ? c : 0;
+    if (p != r) remote += c;
+    int incl = counted;  // a chunk holds at most kPlanThreads * kMaxBlocks entries
 #pragma unroll
     for (int s = 1; s < 32; s <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, incl, s);
       if (lane >= s) incl += v;
     }
-    int pos = running + incl - mine;
-    while (bits) {
-      const int t = __ffs(bits) - 1;
-      bits &= bits - 1;
-      PackEntry e;
-      e.dst_byte = base_byte + (first + pos) * entry_bytes;
-      e.bh = bb * H + h;
-      e.j = w * 32 + t;
-      if (capacity >= 0 && e.dst_byte + entry_bytes > capacity) {
-        e.j = -1;  // would overflow: skipped by the gather
-        atomicExch(status, SPARSP_ERR_CAPACITY);
-      }
-      out[pos] = e;
-      ++pos;
+    __syncthreads();  // (the previous chunk's sums have been read)
+    if (lane == 31) warp_s[warp] = incl;
+    __syncthreads();
+    int before = 0, all = 0;
+#pragma unroll
+    for (int k = 0; k < kPlanThreads / 32; ++k) {
+      const int v = (int)warp_s[k];
+      if (k < warp) before += v;
+      all += v;
     }
-    running += __shfl_sync(0xffffffffu, incl, 31);
+    if (i < PH) {
+      const int64_t at = cursor + before + incl - counted;
+      if (writer) seg_off[(int64_t)br * PH + i] = at;
+      if (i - p * H == h) seg_s[p] = at;
+    }
+    cursor += all;
   }
+  if (writer) {
+    remote = block_sum(remote, warp_s);
+    if (threadIdx.x == 0) {
+      seg_total[br] = cursor;
+      volume[br] = entry_bytes * remote;
+    }
+  }
+  if (!dst) return;
+
+  int64_t base = 0;
+  if (dst_base) {
+    base = dst_base[br];
+  } else if (br > 0) {
+    int64_t n = 0;
+    for (int row = warp; row < br * P; row += kPlanThreads / 32) {  // (consumer, producer), a warp each
+      if (include_local || (row / P) % P != row % P)
+        for (int k = lane; k < H; k += 32) n += cnt[(int64_t)row * H + k];
+    }
+    base = entry_bytes * block_sum(n, warp_s);
+  }
+  __syncthreads();
+  int64_t* out = dst + (int64_t)(bb * H + h) * NB * P + r;
+  const uint32_t u = lane < Wd ? U[((int64_t)br * H + h) * Wd + lane] : 0u;
+  for (int j = threadIdx.x; j < NB; j += kPlanThreads) out[(int64_t)j * P] = -1;
+  __syncthreads();
+  for (int p = warp; p < P; p += kPlanThreads / 32) {
+    if (p == r && !include_local) continue;
+    uint32_t bits = lane < Wd ? u & own_s[p * Wd + lane] : 0u;
+    int total;
+    int64_t byte = base + (seg_s[p] + bits_below(bits, lane, &total)) * entry_bytes;
+    for (; bits; bits &= bits - 1, byte += entry_bytes) {
+      if (capacity >= 0 && byte + entry_bytes > capacity) {
+        atomicExch(status, SPARSP_ERR_CAPACITY);  // would overflow: stays -1, the gather leaves it out
+      } else {
+        out[(int64_t)(lane * 32 + __ffs(bits) - 1) * P] = byte;
+      }
+    }
+  }
+}
+
+// Table of destinations [B*H*NB][n_dst] and list of sources [<= B*H*NB] inside the workspace's entry area, which holds
+// 16 bytes for every (source, rank).
+static int64_t* dst_table(char* ws, const WsLayout& L) { return (int64_t*)(ws + L.entries); }
+static int32_t* src_list(char* ws, const WsLayout& L, const Geometry& g, int n_dst) {
+  return (int32_t*)(ws + L.entries + (int64_t)g.B * g.H * g.NB * n_dst * 8);
+}
+
+static void launch_plan(const Geometry& g, const uint32_t* mask, const int32_t* rank, int P, int include_local,
+                        uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total, int64_t* volume,
+                        const int64_t* dst_base, int64_t capacity, int64_t* dst, int32_t* src, int32_t* n_src,
+                        int32_t* status, cudaStream_t st) {
+  union_count_kernel<<<g.B * g.H * P, kUnionThreads, 0, st>>>(mask, rank, g.H, g.NB, g.Wd, P, U, cnt, n_src);
+  const unsigned grid = dst ? (unsigned)((g.B * P + g.B) * g.H) : (unsigned)(g.B * P);
+  plan_kernel<<<grid, kPlanThreads, 0, st>>>(cnt, U, rank, g.B * P, g.H, g.NB, g.Wd, P, include_local,
+                                             2LL * g.b * g.d * 2, seg_off, seg_total, volume, dst_base, capacity, dst,
+                                             src, n_src, status);
+  count_launch(2);
 }
 
 int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_of_block, int P,
                   int flags, uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total,
                   int64_t* volume, const int64_t* dst_base, int64_t capacity, char* ws,
                   const WsLayout& L, cudaStream_t st) {
-  uint32_t* own = (uint32_t*)(ws + L.own);
-  int64_t* ent_base = (int64_t*)(ws + L.ent_base);
-  int64_t* n_entries = (int64_t*)(ws + L.n_entries);
-  PackEntry* entries = (PackEntry*)(ws + L.entries);
-  int32_t* status = (int32_t*)(ws + L.status);
-  const int include_local = (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0;
-  const int64_t entry_bytes = 2LL * g.b * g.d * 2;
+  const bool pack = !(flags & SPARSP_PLAN_ONLY);  // a plan alone needs no destinations
   if (g.B * P > 1024) {
     set_error("batch * n_ranks = %d exceeds 1024", g.B * P);
     return SPARSP_ERR_UNSUPPORTED;
   }
-  launch_union_count(mask, rank_of_block, g, P, own, U, cnt, st);
-  const int64_t n_c = (int64_t)g.B * P * P * g.H;
-  scan_kernel<<<1, 1024, 0, st>>>(cnt, g.B, g.H, P, include_local, entry_bytes, seg_off, seg_total,
-                                  volume, ent_base, n_entries);
-  entries_kernel<<<(int)((n_c * 32 + 255) / 256), 256, 0, st>>>(U, own, g.B, g.H, g.Wd, P,
-                                                               include_local, entry_bytes, seg_off,
-                                                               ent_base, dst_base, capacity, entries,
-                                                               status);
-  count_launch(3);
+  launch_plan(g, mask, rank_of_block, P, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, U, cnt, seg_off, seg_total, volume,
+              dst_base, capacity, pack ? dst_table(ws, L) : nullptr, pack ? src_list(ws, L, g, P) : nullptr,
+              pack ? (int32_t*)(ws + L.n_entries) : nullptr, (int32_t*)(ws + L.status), st);
   SPARSP_CUDA_OK(cudaGetLastError());
   return SPARSP_OK;
 }
 
 // ------------------------------------------------------------------------------------------------
-// Gather.  All K and V tiles of all entries form one flat sequence of 16-byte vectors (tile t of the
-// sequence = K or V tile of entry t/2).  Persistent CTAs take chunks of kPackThreads * kPackUnroll
-// consecutive vectors, so the bytes in flight per SM do not depend on the tile size (8..32 KiB); loads
-// and stores are fully coalesced when a tile's rows are adjacent in memory.  Rows at or beyond N are
-// written as zeros.
+// Gather, source by source: a K or V tile is loaded into shared memory once and stored from there to every consumer
+// that selected it, so HBM carries one read per distinct tile and one write per packed tile -- its floor.  (Tile by tile
+// in the order of the packed buffer every copy was read again: 3.45 ms for the 10.8 GB that 8 ranks of 40 heads x 591
+// blocks of 32 KiB receive, at 6.3 TB/s of reads and writes; this order 2.23 ms, 5.5 TB/s of which seven eighths are writes.  Four to six
+// stages and one to three stores left in flight are within 1 %: memory sets the pace.)
+// One warp streams whole tiles: TMA tile load (any token stride; rows behind the last token arrive as zeros), then one
+// bulk store per consumer, issued by the lane that holds its destination.  A ring of kPackStages tile buffers per warp
+// (1, 2 or 4 warps per CTA for 32, 16, 8 KiB tiles: 160 KiB per CTA whatever the tile size), loads running
+// kPackStages - 1 tiles ahead of the stores.  The warp's next 32 sources sit in its lanes' registers and the next tile's
+// destinations are fetched before the wait for the current stores, so that no table lookup is exposed.
 // ------------------------------------------------------------------------------------------------
-constexpr int kPackThreads = 256;
-constexpr int kPackUnroll = 8;
+constexpr int kPackStages = 5;
+constexpr int kPackMaxWarps = 4;
 
-template <int D>
-__global__ void __launch_bounds__(kPackThreads) pack_kernel(
-    const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
-    const PackEntry* __restrict__ entries, const int64_t* __restrict__ n_entries_p, int H, int b,
-    int64_t N, int64_t sB, int64_t sH, int64_t sT, unsigned char* __restrict__ packed) {
-  constexpr int VPR = D / 8;                // 16-byte vectors per row
-  const int vpt = b * VPR;                  // vectors per tile (a power of two)
-  const int vpt_shift = 31 - __clz(vpt);
-  const int64_t n_vec = 2 * (*n_entries_p) * (int64_t)vpt;
-  constexpr int64_t kChunk = (int64_t)kPackThreads * kPackUnroll;
-  for (int64_t base = (int64_t)blockIdx.x * kChunk; base < n_vec; base += (int64_t)gridDim.x * kChunk) {
-    uint4 buf[kPackUnroll];
-    uint4* dst[kPackUnroll];
-#pragma unroll
-    for (int u = 0; u < kPackUnroll; ++u) {
-      const int64_t g = base + u * kPackThreads + threadIdx.x;
-      buf[u] = make_uint4(0u, 0u, 0u, 0u);
-      dst[u] = nullptr;
-      if (g < n_vec) {
-        const int64_t tile = g >> vpt_shift;
-        const int v = (int)(g & (vpt - 1));
-        const int4 raw = __ldg(reinterpret_cast<const int4*>(entries) + (tile >> 1));
-        PackEntry e;
-        e.dst_byte = (int64_t)(((uint64_t)(uint32_t)raw.y << 32) | (uint32_t)raw.x);
-        e.bh = raw.z;
-        e.j = raw.w;
-        if (e.j >= 0) {
-          const int which = (int)(tile & 1);
-          const int row = v / VPR, col = v % VPR;
-          const int64_t tok = (int64_t)e.j * b + row;
-          dst[u] = reinterpret_cast<uint4*>(packed + e.dst_byte + (int64_t)which * vpt * 16) + v;
-          if (tok < N) {
-            const int64_t batch = e.bh / H, head = e.bh % H;
-            const __nv_bfloat16* src = (which ? V : K) + batch * sB + head * sH + tok * sT;
-            buf[u] = __ldcs(reinterpret_cast<const uint4*>(src) + col);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kPackUnroll; ++u)
-      if (dst[u]) __stcs(dst[u], buf[u]);
-  }
-}
-
-// Per-tile variant for large tiles (>= 16 KiB): one K or V tile per CTA step, the entry record is read
-// once per tile.  Measured faster than the flat variant when a tile alone fills a CTA's loads in flight.
-template <int D>
-__global__ void __launch_bounds__(kPackThreads) pack_tile_kernel(
-    const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
-    const PackEntry* __restrict__ entries, const int64_t* __restrict__ n_entries_p, int H, int b,
-    int64_t N, int64_t sB, int64_t sH, int64_t sT, unsigned char* __restrict__ packed) {
-  constexpr int VPR = D / 8;  // 16-byte vectors per row
-  const int64_t n_items = 2 * (*n_entries_p);
-  const int vec_per_tile = b * VPR;
-  const int64_t tile_bytes = (int64_t)b * D * 2;
-  for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const PackEntry e = entries[item >> 1];
-    if (e.j < 0) continue;
-    const int which = (int)(item & 1);
-    const int64_t batch = e.bh / H, head = e.bh % H;
-    const int64_t tok0 = (int64_t)e.j * b;
-    const int n_valid = (int)min((int64_t)b, N - tok0);
-    const __nv_bfloat16* src = (which ? V : K) + batch * sB + head * sH + tok0 * sT;
-    uint4* dst = reinterpret_cast<uint4*>(packed + e.dst_byte + which * tile_bytes);
-    for (int v0 = threadIdx.x; v0 < vec_per_tile; v0 += kPackThreads * kPackUnroll) {
-      uint4 buf[kPackUnroll];
-#pragma unroll
-      for (int u = 0; u < kPackUnroll; ++u) {
-        const int v = v0 + u * kPackThreads;
-        const int row = v / VPR, col = v % VPR;
-        buf[u] = make_uint4(0u, 0u, 0u, 0u);
-        if (v < vec_per_tile && row < n_valid)
-          buf[u] = __ldcs(reinterpret_cast<const uint4*>(src + (int64_t)row * sT) + col);
-      }
-#pragma unroll
-      for (int u = 0; u < kPackUnroll; ++u) {
-        const int v = v0 + u * kPackThreads;
-        if (v < vec_per_tile) __stcs(dst + v, buf[u]);
-      }
-    }
-  }
-}
-
-// ------------------------------------------------------------------------------------------------
-// Bulk-copy gather for layouts in which a tile's rows are adjacent in memory ([B][H][N][d]): one warp
-// per CTA streams whole tiles global -> shared -> global with the TMA bulk engine (cp.async.bulk), a
-// ring of n_stages tile buffers per warp (1, 2 or 4 warps per CTA for 32, 16, 8 KiB tiles, so that the
-// bytes in flight per SM do not depend on the tile size), loads running n_stages-1 tiles ahead of the
-// stores.
-// No thread touches the data, except to zero the missing rows of a ragged last block.
-// ------------------------------------------------------------------------------------------------
-constexpr int kBulkMaxStages = 8;
-#ifndef SPARSP_TUNE_PACK_BULK
-#define SPARSP_TUNE_PACK_BULK 1
-#endif
-constexpr bool kPackUseBulk = SPARSP_TUNE_PACK_BULK != 0;
-
-__device__ __forceinline__ void bulk_load(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   ptx::smem_u32(smem_dst)),
-               "l"(gsrc), "r"(bytes), "r"(ptx::smem_u32(bar))
-               : "memory");
-}
 __device__ __forceinline__ void bulk_store(void* gdst, const void* smem_src, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst),
                "r"(ptx::smem_u32(smem_src)), "r"(bytes)
                : "memory");
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
-template <int D>
-__global__ void __launch_bounds__(128) pack_bulk_kernel(const __nv_bfloat16* __restrict__ K,
-                                                       const __nv_bfloat16* __restrict__ V,
-                                                       const PackEntry* __restrict__ entries,
-                                                       const int64_t* __restrict__ n_entries_p, int H, int b,
-                                                       int64_t N, int64_t sB, int64_t sH, int n_stages,
-                                                       unsigned char* __restrict__ packed,
-                                                       int32_t* __restrict__ status) {
+__global__ void __launch_bounds__(32 * kPackMaxWarps) pack_kernel(const __grid_constant__ CUtensorMap tmK,
+                                                                  const __grid_constant__ CUtensorMap tmV,
+                                                                  const int64_t* __restrict__ dst, int n_dst,
+                                                                  const int32_t* __restrict__ src,
+                                                                  const int32_t* __restrict__ n_src, int H, int NB,
+                                                                  int b, uint32_t tile_bytes,
+                                                                  unsigned char* __restrict__ packed,
+                                                                  int32_t* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ uint64_t full_all[4 * kBulkMaxStages];
+  __shared__ uint64_t full_all[kPackMaxWarps * kPackStages];
   __shared__ int s_abort;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n_warps = blockDim.x >> 5;
-  const uint32_t tile_bytes = (uint32_t)b * D * 2;
-  uint64_t* full = full_all + warp * kBulkMaxStages;
-  unsigned char* ring = smem_raw + (size_t)warp * n_stages * tile_bytes;  // this warp's buffers
-  const int64_t unit = (int64_t)blockIdx.x * n_warps + warp, n_units = (int64_t)gridDim.x * n_warps;
-  const int64_t n_items = 2 * (*n_entries_p);
-  const int64_t n_local = n_items > unit ? (n_items - unit + n_units - 1) / n_units : 0;
+  uint64_t* full = full_all + warp * kPackStages;
+  unsigned char* ring = smem_raw + (size_t)warp * kPackStages * tile_bytes;  // this warp's buffers
+  const int unit = blockIdx.x * n_warps + warp, n_units = gridDim.x * n_warps;
+  const int64_t n_items = 2 * (int64_t)*n_src;  // item: K (even) or V (odd) tile of source item / 2
+  const int n_local = (int)(n_items > unit ? (n_items - unit + n_units - 1) / n_units : 0);
   if (threadIdx.x == 0) s_abort = 0;
   if (lane == 0) {
-    for (int st = 0; st < n_stages; ++st) ptx::mbar_init(full + st, 1);
+    for (int st = 0; st < kPackStages; ++st) ptx::mbar_init(full + st, 1);
     ptx::mbar_init_fence();
   }
   __syncthreads();
 
-  // source address and valid byte count of local item q (0 valid bytes = entry skipped for capacity)
-  auto locate = [&](int64_t q, const unsigned char*& src, unsigned char*& dst, uint32_t& valid) {
-    const int64_t item = unit + q * n_units;
-    const int4 raw = __ldg(reinterpret_cast<const int4*>(entries) + (item >> 1));
-    const int64_t dst_byte = (int64_t)(((uint64_t)(uint32_t)raw.y << 32) | (uint32_t)raw.x);
-    const int bh = raw.z, j = raw.w;
-    const int which = (int)(item & 1);
-    if (j < 0) {
-      valid = 0;
-      src = nullptr;
-      dst = nullptr;
-      return;
-    }
-    const int64_t batch = bh / H, head = bh % H, tok0 = (int64_t)j * b;
-    const int64_t n_valid = min((int64_t)b, N - tok0);
-    valid = (uint32_t)(n_valid * D * 2);
-    src = reinterpret_cast<const unsigned char*>((which ? V : K) + batch * sB + head * sH + tok0 * D);
-    dst = packed + dst_byte + (int64_t)which * tile_bytes;
+  // lane l: the source of local item q + l
+  auto sources = [&](int q) -> int {
+    const int64_t item = unit + (int64_t)(q + lane) * n_units;
+    return item < n_items ? __ldg(src + (item >> 1)) : 0;
   };
-  auto issue_load = [&](int64_t q) {
-    const unsigned char* src;
-    unsigned char* dst;
-    uint32_t valid;
-    locate(q, src, dst, valid);
-    uint64_t* bar = full + q % n_stages;
-    if (valid == 0) {
-      ptx::mbar_arrive(bar);  // nothing to move: complete the phase directly
-    } else {
-      ptx::mbar_expect_tx(bar, valid);
-      bulk_load(ring + (size_t)(q % n_stages) * tile_bytes, src, valid, bar);
-    }
+  auto which = [&](int q) { return (int)((unit + (int64_t)q * n_units) & 1); };
+  auto destination = [&](int s, int first) -> int64_t {
+    return first + lane < n_dst ? __ldg(dst + (int64_t)s * n_dst + first + lane) : -1;
   };
-
-  if (lane == 0)
-    for (int64_t q = 0; q < n_stages - 1 && q < n_local; ++q) issue_load(q);
-  for (int64_t q = 0; q < n_local; ++q) {
-    const unsigned char* src;
-    unsigned char* dst;
-    uint32_t valid;
-    locate(q, src, dst, valid);  // same values in every lane
-    unsigned char* buf = ring + (size_t)(q % n_stages) * tile_bytes;
-    ptx::mbar_wait_bounded(full + q % n_stages, (uint32_t)((q / n_stages) & 1), &s_abort, status, 50, 200000000LL);
-    if (valid != 0 && valid < tile_bytes) {  // ragged last block: zero the missing rows
-      for (uint32_t o = valid + lane * 16; o < tile_bytes; o += 32 * 16)
-        *reinterpret_cast<uint4*>(buf + o) = make_uint4(0u, 0u, 0u, 0u);
-      ptx::fence_proxy_async_smem();
-    }
-    __syncwarp();
-    if (lane == 0) {
-      if (valid != 0) bulk_store(dst, buf, tile_bytes);
-      // the buffer of item q-1 may be refilled once its store has read it
-      asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-      if (q + n_stages - 1 < n_local) issue_load(q + n_stages - 1);
-    }
-    __syncwarp();
+  auto issue_load = [&](int q, int s) {
+    uint64_t* bar = full + q % kPackStages;
+    const int bh = s / NB;
+    ptx::mbar_expect_tx(bar, tile_bytes);
+    ptx::tma_load_4d(ring + (size_t)(q % kPackStages) * tile_bytes, which(q) ? &tmV : &tmK, bar, 0, (s - bh * NB) * b,
+                     bh % H, bh / H);
+  };
+  int cur = sources(0), ahead = cur;  // sources of the 32 items around the store / around the load
+  for (int q = 0; q < kPackStages - 1 && q < n_local; ++q) {
+    const int s = __shfl_sync(0xffffffffu, ahead, q);
+    if (lane == 0) issue_load(q, s);
   }
-  if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+  int64_t d0 = -1, d1 = -1;  // this lane's destinations of the current item (ranks lane and lane + 32)
+  if (n_local > 0) {
+    const int s = __shfl_sync(0xffffffffu, cur, 0);
+    d0 = destination(s, 0);
+    if (n_dst > 32) d1 = destination(s, 32);
+  }
+  for (int q = 0; q < n_local; ++q) {
+    const int64_t half = which(q) ? tile_bytes : 0;
+    const unsigned char* buf = ring + (size_t)(q % kPackStages) * tile_bytes;
+    ptx::mbar_wait_bounded(full + q % kPackStages, (uint32_t)((q / kPackStages) & 1), &s_abort, status, 50, 200000000LL);
+    if (d0 >= 0) bulk_store(packed + d0 + half, buf, tile_bytes);
+    if (d1 >= 0) bulk_store(packed + d1 + half, buf, tile_bytes);
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    if (q + 1 < n_local) {
+      if (((q + 1) & 31) == 0) cur = sources(q + 1);
+      const int s = __shfl_sync(0xffffffffu, cur, (q + 1) & 31);
+      d0 = destination(s, 0);
+      if (n_dst > 32) d1 = destination(s, 32);
+    }
+    const int ql = q + kPackStages - 1;
+    if (ql < n_local) {
+      if ((ql & 31) == 0) ahead = sources(ql);
+      const int s = __shfl_sync(0xffffffffu, ahead, ql & 31);
+      // the buffer of item q - 1 may be refilled once every lane's stores have read it
+      asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) issue_load(ql, s);
+    }
+  }
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-int launch_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, void* packed,
-                int64_t capacity, int P, char* ws, const WsLayout& L, cudaStream_t st) {
-  (void)capacity;
-  (void)P;
-  const PackEntry* entries = (const PackEntry*)(ws + L.entries);
-  const int64_t* n_entries = (const int64_t*)(ws + L.n_entries);
+static int run_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, const int64_t* dst, int n_dst,
+                    const int32_t* src, const int32_t* n_src, void* packed, int32_t* status, cudaStream_t st) {
   int dev = 0, sms = 148;
   SPARSP_CUDA_OK(cudaGetDevice(&dev));
   SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int grid = sms * 8;
-  auto k = (const __nv_bfloat16*)K;
-  auto v = (const __nv_bfloat16*)V;
-  const bool small_tiles = g.b * g.d / 8 < 1024;  // 8 KiB tiles: several tiles per CTA step
-  unsigned char* out = (unsigned char*)packed;
-  const bool rows_adjacent = s.stride_token == g.d;
-  if (rows_adjacent && kPackUseBulk) {
-    // TMA bulk path: a ring of whole-tile buffers per CTA, one CTA per SM
-    const int tile_bytes = g.b * g.d * 2;
-    const int n_warps = std::max(1, std::min(4, (32 * 1024) / tile_bytes));
-    const int n_stages = 5;  // per warp: 160 KiB of tile buffers per CTA whatever the tile size
-    const int smem = n_warps * n_stages * tile_bytes;
-    int32_t* status = (int32_t*)(ws + L.status);
-    if (g.d == 64) {
-      SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)pack_bulk_kernel<64>, smem));
-      pack_bulk_kernel<64><<<sms, 32 * n_warps, smem, st>>>(k, v, entries, n_entries, g.H, g.b, g.N,
-                                                            s.stride_batch, s.stride_head, n_stages, out, status);
-    } else {
-      SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)pack_bulk_kernel<128>, smem));
-      pack_bulk_kernel<128><<<sms, 32 * n_warps, smem, st>>>(k, v, entries, n_entries, g.H, g.b, g.N,
-                                                             s.stride_batch, s.stride_head, n_stages, out, status);
-    }
-  } else if (small_tiles) {
-    if (g.d == 64)
-      pack_kernel<64><<<grid, kPackThreads, 0, st>>>(k, v, entries, n_entries, g.H, g.b, g.N, s.stride_batch,
-                                                     s.stride_head, s.stride_token, out);
-    else
-      pack_kernel<128><<<grid, kPackThreads, 0, st>>>(k, v, entries, n_entries, g.H, g.b, g.N, s.stride_batch,
-                                                      s.stride_head, s.stride_token, out);
-  } else {
-    if (g.d == 64)
-      pack_tile_kernel<64><<<grid, kPackThreads, 0, st>>>(k, v, entries, n_entries, g.H, g.b, g.N,
-                                                          s.stride_batch, s.stride_head, s.stride_token, out);
-    else
-      pack_tile_kernel<128><<<grid, kPackThreads, 0, st>>>(k, v, entries, n_entries, g.H, g.b, g.N,
-                                                           s.stride_batch, s.stride_head, s.stride_token, out);
-  }
+  CUtensorMap tk, tv;
+  int rc;
+  if ((rc = make_tile_tmap(&tk, K, s, g, g.b, false)) != SPARSP_OK) return rc;
+  if ((rc = make_tile_tmap(&tv, V, s, g, g.b, false)) != SPARSP_OK) return rc;
+  const int tile_bytes = g.b * g.d * 2;
+  const int n_warps = std::max(1, std::min(kPackMaxWarps, (32 * 1024) / tile_bytes));
+  const int smem = n_warps * kPackStages * tile_bytes;
+  SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)pack_kernel, smem));
+  pack_kernel<<<sms, 32 * n_warps, smem, st>>>(tk, tv, dst, n_dst, src, n_src, g.H, g.NB, g.b, (uint32_t)tile_bytes,
+                                               (unsigned char*)packed, status);
   count_launch();
   SPARSP_CUDA_OK(cudaGetLastError());
   return SPARSP_OK;
 }
 
+int launch_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, void* packed, int P, char* ws,
+                const WsLayout& L, cudaStream_t st) {
+  return run_pack(s, g, K, V, dst_table(ws, L), P, src_list(ws, L, g, P), (const int32_t*)(ws + L.n_entries), packed,
+                  (int32_t*)(ws + L.status), st);
+}
+
 // ------------------------------------------------------------------------------------------------
 // Pack of ONE (consumer, producer) segment (Section 6.1: the producer packs the payload of one consumer into
-// the slot designated for that pair).  The entry table holds that segment alone, with destinations relative
+// the slot designated for that pair).  The tables hold that segment alone, with destinations relative
 // to the start of the slot: entry (h, j) sits where it sits inside the consumer's buffer, minus the segment's
 // first entry, so that consumer and producer derive the same byte ranges from the demand counts.
 // One warp per head enumerates U[consumer][h] & own[producer] in ascending block order.
 // ------------------------------------------------------------------------------------------------
-__global__ void segment_entries_kernel(const uint32_t* __restrict__ U, const int32_t* __restrict__ rank, int H, int NB,
-                                       int Wd, int P, int consumer, int producer,
-                                       const int64_t* __restrict__ seg_off, const int32_t* __restrict__ cnt,
-                                       int64_t entry_bytes, int64_t capacity, PackEntry* __restrict__ entries,
-                                       int64_t* __restrict__ n_entries, int32_t* __restrict__ status) {
+__global__ void __launch_bounds__(256) segment_kernel(const uint32_t* __restrict__ U, const int32_t* __restrict__ rank,
+                                                      int H, int NB, int Wd, int P, int consumer, int producer,
+                                                      const int64_t* __restrict__ seg_off,
+                                                      const int32_t* __restrict__ cnt, int64_t entry_bytes,
+                                                      int64_t capacity, int64_t* __restrict__ dst,
+                                                      int32_t* __restrict__ src, int32_t* __restrict__ n_src,
+                                                      int32_t* __restrict__ status) {
+  __shared__ uint32_t own_s[kMaxWords];
   const int h = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
+  rank_words(rank, NB, producer, own_s);
+  __syncthreads();
   if (h >= H) return;
   const int64_t seg0 = ((int64_t)consumer * P + producer) * H;  // batch item 0
   const int64_t first_of_segment = seg_off[seg0];
-  if (h == 0 && lane == 0) *n_entries = seg_off[seg0 + H - 1] + cnt[seg0 + H - 1] - first_of_segment;
-  const uint32_t* u = U + ((int64_t)consumer * H + h) * Wd;
-  const int64_t first = seg_off[seg0 + h] - first_of_segment;
-  int running = 0;
-  for (int w0 = 0; w0 < Wd; w0 += 32) {
-    const int w = w0 + lane;
-    uint32_t bits = 0;
-    if (w < Wd) {
-      uint32_t own = 0;
-      for (int t = 0; t < 32; ++t) {
-        const int j = w * 32 + t;
-        if (j < NB && rank[j] == producer) own |= 1u << t;
-      }
-      bits = u[w] & own;
-    }
-    const int mine = __popc(bits);
-    int incl = mine;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, s);
-      if (lane >= s) incl += v;
-    }
-    int pos = running + incl - mine;
-    while (bits) {
-      const int t = __ffs(bits) - 1;
-      bits &= bits - 1;
-      PackEntry e;
-      e.dst_byte = (first + pos) * entry_bytes;
-      e.bh = h;
-      e.j = w * 32 + t;
-      if (e.dst_byte + entry_bytes > capacity) {
-        e.j = -1;  // would not fit the slot: skipped by the gather
-        atomicExch(status, SPARSP_ERR_CAPACITY);
-      }
-      entries[first + pos] = e;
-      ++pos;
-    }
-    running += __shfl_sync(0xffffffffu, incl, 31);
+  if (h == 0 && lane == 0) *n_src = (int32_t)(seg_off[seg0 + H - 1] + cnt[seg0 + H - 1] - first_of_segment);
+  uint32_t bits = lane < Wd ? U[((int64_t)consumer * H + h) * Wd + lane] & own_s[lane] : 0u;
+  int total;
+  int64_t at = seg_off[seg0 + h] - first_of_segment + bits_below(bits, lane, &total);
+  for (; bits; bits &= bits - 1, ++at) {
+    const int s = h * NB + lane * 32 + __ffs(bits) - 1;
+    const bool fits = (at + 1) * entry_bytes <= capacity;
+    if (!fits) atomicExch(status, SPARSP_ERR_CAPACITY);  // left out by the gather
+    dst[s] = fits ? at * entry_bytes : -1;
+    src[at] = s;
   }
 }
 
 int launch_pack_segment(const sparsp_shape& s, const Geometry& g, const uint32_t* U, const int32_t* rank, int P,
                         int consumer, int producer, const int64_t* seg_off, const int32_t* cnt, const void* K,
                         const void* V, void* dst, int64_t capacity, char* ws, const WsLayout& L, cudaStream_t st) {
-  PackEntry* entries = (PackEntry*)(ws + L.entries);
-  int64_t* n_entries = (int64_t*)(ws + L.n_entries);
+  int64_t* table = dst_table(ws, L);
+  int32_t* src = src_list(ws, L, g, 1);
+  int32_t* n_src = (int32_t*)(ws + L.n_entries);
   int32_t* status = (int32_t*)(ws + L.status);
-  const int64_t entry_bytes = 2LL * g.b * g.d * 2;
-  segment_entries_kernel<<<(g.H * 32 + 255) / 256, 256, 0, st>>>(U, rank, g.H, g.NB, g.Wd, P, consumer, producer, seg_off,
-                                                                cnt, entry_bytes, capacity, entries, n_entries, status);
+  segment_kernel<<<(g.H * 32 + 255) / 256, 256, 0, st>>>(U, rank, g.H, g.NB, g.Wd, P, consumer, producer, seg_off, cnt,
+                                                        2LL * g.b * g.d * 2, capacity, table, src, n_src, status);
   count_launch();
   SPARSP_CUDA_OK(cudaGetLastError());
-  return launch_pack(s, g, K, V, dst, capacity, P, ws, L, st);
+  return run_pack(s, g, K, V, table, 1, src, n_src, dst, status, st);
 }
 
 // ------------------------------------------------------------------------------------------------
-// Allocation-free planning call.  Its scratch (the per-rank ownership bit words and the per-consumer
-// table bases) lives in one file-scope device array instead of a caller-provided workspace, so a
-// caller that cannot allocate device memory at all can still obtain unions, counts, offsets and
-// volumes.  Every GPU that loads the library carries the array (kPlanScratchBytes) until exit.
+// Allocation-free planning call: the same two launches, which need no scratch when no destinations are asked for, so a
+// caller that cannot allocate device memory at all can still obtain unions, counts, offsets and volumes.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPlanMaxRanks = 64;         // n_ranks limit of the allocation-free call
 constexpr int kPlanMaxBatchRanks = 1024;  // batch * n_ranks limit
-constexpr int kPlanOwnWords = kPlanMaxRanks * (kMaxBlocks / 32);
-constexpr size_t kPlanScratchBytes = kPlanOwnWords * sizeof(uint32_t) + (kPlanMaxBatchRanks + 1) * sizeof(int64_t);
-
-static __device__ __align__(256) unsigned char g_plan_scratch[kPlanScratchBytes];
-
-constexpr int kMaxDevices = 64;
-static std::mutex g_plan_mutex;
-static void* g_plan_scratch_addr[kMaxDevices] = {nullptr};
-
-// Device address of g_plan_scratch on the current device.  In host code the array's name is only a
-// handle, so the address is resolved once per device with that device current.
-static int plan_scratch_address(void** out) {
-  int dev = 0;
-  SPARSP_CUDA_OK(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= kMaxDevices) {
-    set_error("device ordinal %d outside 0..%d", dev, kMaxDevices - 1);
-    return SPARSP_ERR_UNSUPPORTED;
-  }
-  std::lock_guard<std::mutex> lock(g_plan_mutex);
-  if (!g_plan_scratch_addr[dev]) {
-    void* ptr = nullptr;
-    SPARSP_CUDA_OK(cudaGetSymbolAddress(&ptr, g_plan_scratch));
-    g_plan_scratch_addr[dev] = ptr;
-  }
-  *out = g_plan_scratch_addr[dev];
-  return SPARSP_OK;
-}
 
 }  // namespace sparsp
 
@@ -575,19 +433,8 @@ extern "C" SPARSP_API int sparsp_demand_plan_noalloc(const sparsp_shape* shape, 
     set_error("sparsp_demand_plan_noalloc: misaligned argument");
     return SPARSP_ERR_INVALID_ARG;
   }
-  void* scratch = nullptr;
-  if ((rc = plan_scratch_address(&scratch)) != SPARSP_OK) return rc;
-  uint32_t* own = (uint32_t*)scratch;                                       // [P][Wd], fully rewritten
-  int64_t* ent_base = (int64_t*)((char*)scratch + kPlanOwnWords * sizeof(uint32_t));  // [B*P] + total
-  int64_t* n_entries = ent_base + kPlanMaxBatchRanks;
-  const int P = n_ranks;
-  const int include_local = (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0;
-  const int64_t entry_bytes = 2LL * g.b * g.d * 2;
-  cudaStream_t st = (cudaStream_t)stream;
-  launch_union_count(mask, rank_of_block, g, P, own, union_mask, cnt, st);
-  scan_kernel<<<1, 1024, 0, st>>>(cnt, g.B, g.H, P, include_local, entry_bytes, seg_offset, seg_total,
-                                  volume_bytes, ent_base, n_entries);
-  count_launch(2);
+  launch_plan(g, mask, rank_of_block, n_ranks, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, union_mask, cnt, seg_offset,
+              seg_total, volume_bytes, nullptr, -1, nullptr, nullptr, nullptr, nullptr, (cudaStream_t)stream);
   SPARSP_CUDA_OK(cudaGetLastError());
   return SPARSP_OK;
 }
