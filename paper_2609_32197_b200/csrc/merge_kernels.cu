@@ -1,93 +1,155 @@
 // Consumer-side helpers of the demand-routed exchange: the mask of one hop (consumer rank's query
 // blocks x producer rank's KV blocks) and the log-sum-exp merge of per-hop partial attention results.
 // Both are small element-wise kernels; the merge is HBM-bound (reads two outputs, writes one).
+#include <algorithm>
+
+#include "block_sets.cuh"
 #include "common.cuh"
 
 namespace sparsp {
 
 // hop[b][h][i][w] = (rank[i] == consumer and head_begin <= h < head_end) ? mask[b][h][i][w] & own_producer[w] : 0.
-// Thread per word.
-__global__ void hop_mask_kernel(const uint32_t* __restrict__ mask, const int32_t* __restrict__ rank, int H, int NB,
-                                int Wd, int64_t n_words, int consumer, int producer, int head_begin, int head_end,
-                                uint32_t* __restrict__ hop) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n_words) return;
-  const int w = (int)(idx % Wd);
-  const int i = (int)((idx / Wd) % NB);
-  const int h = (int)((idx / ((int64_t)Wd * NB)) % H);
-  uint32_t out = 0;
-  if (rank[i] == consumer && h >= head_begin && h < head_end) {
-    uint32_t own = 0;
-    for (int t = 0; t < 32; ++t) {
-      const int j = w * 32 + t;
-      if (j < NB && rank[j] == producer) own |= 1u << t;
+// A lane handles one word of kHopRows rows (rows of fewer than 32 words share a warp); the producer's ownership words and
+// the consumer's rows are bits in shared memory, built once per CTA.  A mask is a few MB, so this is latency: 40 heads x
+// 591 rows x 19 words in 6.2 us (11.3 us with a thread per word that walked 32 ranks for its ownership bits).
+constexpr int kHopThreads = 256;
+constexpr int kHopRows = 4;
+
+__global__ void __launch_bounds__(kHopThreads) hop_mask_kernel(const uint32_t* __restrict__ mask,
+                                                               const int32_t* __restrict__ rank, int H, int NB, int Wd,
+                                                               int64_t n_rows, int consumer, int producer,
+                                                               int head_begin, int head_end,
+                                                               uint32_t* __restrict__ hop) {
+  __shared__ uint32_t own_s[kMaxWords], row_s[kMaxWords];
+  rank_words(rank, NB, producer, own_s);
+  rank_words(rank, NB, consumer, row_s);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int width = 1;  // lanes per row: the next power of two
+  while (width < Wd) width <<= 1;
+  const int per_warp = 32 / width, w = lane & (width - 1), sub = lane / width;
+  if (w >= Wd) return;
+  const int64_t first = ((int64_t)blockIdx.x * (kHopThreads / 32) + warp) * kHopRows * per_warp + sub;
+  uint32_t v[kHopRows];
+#pragma unroll
+  for (int k = 0; k < kHopRows; ++k) {
+    const int64_t row = first + k * per_warp;
+    v[k] = 0u;
+    if (row < n_rows) {
+      const int64_t bh = row / NB;
+      const int i = (int)(row - bh * NB), h = (int)(bh % H);
+      if (((row_s[i >> 5] >> (i & 31)) & 1u) && h >= head_begin && h < head_end) v[k] = mask[row * Wd + w];
     }
-    out = mask[idx] & own;
   }
-  hop[idx] = out;
+#pragma unroll
+  for (int k = 0; k < kHopRows; ++k) {
+    const int64_t row = first + k * per_warp;
+    if (row < n_rows) hop[row * Wd + w] = v[k] & own_s[w];
+  }
 }
 
-// One CTA per (token block, head, batch); a thread handles (row, 8 columns) units of the block.  O_a, O_b, O: bf16
-// with the shape's strides; lse: fp32 [B][H][N].  O may be O_a or O_b and lse may be lse_a or lse_b (no pointer is
-// declared restrict): a thread reads the 16 bytes it later writes, and only the row's first thread touches the
-// log-sum-exp values -- it reads both inputs, computes the weights and hands them to the row's other threads by
-// shuffle (the D/8 threads of a row are consecutive lanes of one warp) before it writes the merged value.
-// With `rank` given, only the blocks of `consumer` in heads [head_begin, head_begin + gridDim.y) are merged (one
-// chunk of one hop of one rank): a CTA of another rank's block returns at once, every other row stays untouched.
+// Log-sum-exp merge.  Unit of work: one (batch, head, token block); the CTAs walk the units, with `rank` given only those
+// of the blocks of `consumer` in heads [head_begin, head_end) (one chunk of one hop of one rank; every other row stays
+// untouched), which each CTA lists from the rank table.  O_a, O_b, O: bf16 with the shape's strides; lse: fp32 [B][H][N].
+// A thread handles 8 columns of a row, kMergeRows rows at a time with all their loads in flight: HBM-bound, 33 us for
+// 74 blocks of 128 rows x 20 heads x 256 bytes (40 us with a CTA per block, most of which found another rank's block, and
+// one row of loads in flight).
+// O may be O_a or O_b and lse may be lse_a or lse_b (no pointer is declared restrict): a thread reads the 16 bytes it later
+// writes, and the D/8 threads of a row are consecutive lanes of one warp, all of which have read the row's log-sum-exp
+// values before its first thread writes the merged one.
+// A row to which the second part adds nothing (lse_b = -inf: no kept block in this hop) has nothing to do when it is
+// merged in place.
+constexpr int kMergeThreads = 256;
+constexpr int kMergeRows = 4;
+
 template <int D>
-__global__ void __launch_bounds__(256) attn_merge_kernel(const __nv_bfloat16* Oa, const float* la,
-                                                         const __nv_bfloat16* Ob, const float* lb, __nv_bfloat16* O,
-                                                         float* lse, int H, int64_t N, int b, int64_t sB, int64_t sH,
-                                                         int64_t sT, const int32_t* __restrict__ rank, int consumer,
-                                                         int head_begin) {
+__global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __nv_bfloat16* Oa, const float* la,
+                                                                   const __nv_bfloat16* Ob, const float* lb,
+                                                                   __nv_bfloat16* O, float* lse, int B, int H, int NB,
+                                                                   int64_t N, int b, int64_t sB, int64_t sH, int64_t sT,
+                                                                   const int32_t* __restrict__ rank, int consumer,
+                                                                   int head_begin, int head_end) {
   constexpr int VPR = D / 8;
-  const int blk = blockIdx.x, head = head_begin + blockIdx.y, batch = blockIdx.z;
-  if (rank != nullptr && rank[blk] != consumer) return;
-  const int64_t tok0 = (int64_t)blk * b;
-  const int n_rows = (int)min((int64_t)b, N - tok0);
-  const int leader = (threadIdx.x & 31) & ~(VPR - 1);  // lane of the row's first thread
-  for (int u0 = 0; u0 < n_rows * VPR; u0 += blockDim.x) {  // blockDim.x is a multiple of VPR: a row never splits
-    const int u = u0 + threadIdx.x;
-    const int r = u / VPR, col = u % VPR;
-    const bool live = r < n_rows;
-    const int64_t row = ((int64_t)batch * H + head) * N + tok0 + r;
-    float wa = 0.0f, wb = 0.0f, out_lse = -INFINITY;
-    if (live && col == 0) {
-      const float a = la[row], c = lb[row];
-      const float m = fmaxf(a, c);
-      if (m > -INFINITY) {
-        const float ea = __expf(a - m), eb = __expf(c - m);
-        const float tot = ea + eb;
-        wa = ea / tot;
-        wb = eb / tot;
-        out_lse = m + __logf(tot);
-      }
-    }
-    wa = __shfl_sync(0xffffffffu, wa, leader);
-    wb = __shfl_sync(0xffffffffu, wb, leader);
-    if (!live) continue;
-    const int64_t off = (int64_t)batch * sB + (int64_t)head * sH + (tok0 + r) * sT + col * 8;
-    const uint4 va = *reinterpret_cast<const uint4*>(Oa + off);
-    const uint4 vb = *reinterpret_cast<const uint4*>(Ob + off);
-    const uint32_t xa[4] = {va.x, va.y, va.z, va.w}, xb[4] = {vb.x, vb.y, vb.z, vb.w};
-    uint32_t w[4];
+  constexpr int kPass = kMergeThreads / VPR;  // rows per pass of the CTA
+  __shared__ uint32_t words_s[kMaxWords];
+  __shared__ uint16_t own_s[kMaxBlocks];
+  int n_own = NB;
+  if (rank != nullptr) {
+    rank_words(rank, NB, consumer, words_s);
+    n_own = list_blocks(words_s, NB, own_s);
+  }
+  const int heads = head_end - head_begin;
+  const int64_t n_units = (int64_t)B * heads * n_own;
+  const int col = threadIdx.x % VPR, r0 = threadIdx.x / VPR;
+  const bool in_place = O == Oa && lse == la;
+  for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x) {
+    const int64_t bhi = u / n_own;
+    const int k = (int)(u - bhi * n_own);
+    const int blk = rank != nullptr ? own_s[k] : k;
+    const int batch = (int)(bhi / heads), head = head_begin + (int)(bhi - (int64_t)batch * heads);
+    const int64_t tok0 = (int64_t)blk * b;
+    const int n_rows = (int)min((int64_t)b, N - tok0);
+    const int64_t lrow = ((int64_t)batch * H + head) * N + tok0;
+    const int64_t orow = (int64_t)batch * sB + (int64_t)head * sH + tok0 * sT + col * 8;
+    for (int base = 0; base < n_rows; base += kPass * kMergeRows) {
+      float a[kMergeRows], c[kMergeRows];
+      uint4 va[kMergeRows], vb[kMergeRows];
+      bool live[kMergeRows];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float a0 = __uint_as_float(xa[e] << 16), a1 = __uint_as_float(xa[e] & 0xffff0000u);
-      const float b0 = __uint_as_float(xb[e] << 16), b1 = __uint_as_float(xb[e] & 0xffff0000u);
-      const __nv_bfloat162 h2 = __floats2bfloat162_rn(a0 * wa + b0 * wb, a1 * wa + b1 * wb);
-      w[e] = *reinterpret_cast<const uint32_t*>(&h2);
+      for (int t = 0; t < kMergeRows; ++t) {
+        const int r = base + t * kPass + r0;
+        live[t] = r < n_rows;
+        a[t] = live[t] ? la[lrow + r] : 0.0f;
+        c[t] = live[t] ? lb[lrow + r] : 0.0f;
+      }
+#pragma unroll
+      for (int t = 0; t < kMergeRows; ++t) {
+        const int64_t off = orow + (int64_t)(base + t * kPass + r0) * sT;
+        if (in_place && c[t] == -INFINITY && a[t] > -INFINITY) live[t] = false;
+        if (live[t]) {
+          va[t] = *reinterpret_cast<const uint4*>(Oa + off);
+          vb[t] = *reinterpret_cast<const uint4*>(Ob + off);
+        }
+      }
+      __syncwarp();  // every lane of a row has its log-sum-exp values
+#pragma unroll
+      for (int t = 0; t < kMergeRows; ++t) {
+        if (!live[t]) continue;
+        const int r = base + t * kPass + r0;
+        float wa = 0.0f, wb = 0.0f, out_lse = -INFINITY;
+        const float m = fmaxf(a[t], c[t]);
+        if (m > -INFINITY) {
+          const float ea = __expf(a[t] - m), eb = __expf(c[t] - m);
+          const float tot = ea + eb;
+          wa = ea / tot;
+          wb = eb / tot;
+          out_lse = m + __logf(tot);
+        }
+        const uint32_t xa[4] = {va[t].x, va[t].y, va[t].z, va[t].w}, xb[4] = {vb[t].x, vb[t].y, vb[t].z, vb[t].w};
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float a0 = __uint_as_float(xa[e] << 16), a1 = __uint_as_float(xa[e] & 0xffff0000u);
+          const float b0 = __uint_as_float(xb[e] << 16), b1 = __uint_as_float(xb[e] & 0xffff0000u);
+          const __nv_bfloat162 h2 = __floats2bfloat162_rn(a0 * wa + b0 * wb, a1 * wa + b1 * wb);
+          w[e] = *reinterpret_cast<const uint32_t*>(&h2);
+        }
+        *reinterpret_cast<uint4*>(O + orow + (int64_t)r * sT) = make_uint4(w[0], w[1], w[2], w[3]);
+        if (col == 0) lse[lrow + r] = out_lse;
+      }
+      __syncwarp();
     }
-    *reinterpret_cast<uint4*>(O + off) = make_uint4(w[0], w[1], w[2], w[3]);
-    if (col == 0) lse[row] = out_lse;
   }
 }
 
 int launch_hop_mask(const Geometry& g, const uint32_t* mask, const int32_t* rank, int consumer, int producer,
                     int head_begin, int head_end, uint32_t* hop, cudaStream_t st) {
-  const int64_t n_words = (int64_t)g.B * g.H * g.NB * g.Wd;
-  hop_mask_kernel<<<(unsigned)((n_words + 255) / 256), 256, 0, st>>>(mask, rank, g.H, g.NB, g.Wd, n_words, consumer,
-                                                                     producer, head_begin, head_end, hop);
+  const int64_t n_rows = (int64_t)g.B * g.H * g.NB;
+  int width = 1;
+  while (width < g.Wd) width <<= 1;
+  const int per_cta = kHopThreads / width * kHopRows;
+  hop_mask_kernel<<<(unsigned)((n_rows + per_cta - 1) / per_cta), kHopThreads, 0, st>>>(
+      mask, rank, g.H, g.NB, g.Wd, n_rows, consumer, producer, head_begin, head_end, hop);
   count_launch();
   SPARSP_CUDA_OK(cudaGetLastError());
   return SPARSP_OK;
@@ -97,16 +159,14 @@ int launch_attn_merge(const sparsp_shape& s, const Geometry& g, const void* Oa, 
                       const float* lb, void* O, float* lse, const int32_t* rank, int consumer, int head_begin,
                       int head_end, cudaStream_t st) {
   if (head_end <= head_begin) return SPARSP_OK;
-  dim3 grid((unsigned)g.NB, (unsigned)(head_end - head_begin), (unsigned)g.B);
-  auto a = (const __nv_bfloat16*)Oa;
-  auto b = (const __nv_bfloat16*)Ob;
-  auto o = (__nv_bfloat16*)O;
-  if (g.d == 64)
-    attn_merge_kernel<64><<<grid, 256, 0, st>>>(a, la, b, lb, o, lse, g.H, g.N, g.b, s.stride_batch, s.stride_head,
-                                                s.stride_token, rank, consumer, head_begin);
-  else
-    attn_merge_kernel<128><<<grid, 256, 0, st>>>(a, la, b, lb, o, lse, g.H, g.N, g.b, s.stride_batch, s.stride_head,
-                                                 s.stride_token, rank, consumer, head_begin);
+  int dev = 0, sms = 148;
+  SPARSP_CUDA_OK(cudaGetDevice(&dev));
+  SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const unsigned grid = (unsigned)std::min<int64_t>((int64_t)g.B * (head_end - head_begin) * g.NB, 4LL * sms);
+  auto kern = g.d == 64 ? attn_merge_kernel<64> : attn_merge_kernel<128>;
+  kern<<<grid, kMergeThreads, 0, st>>>((const __nv_bfloat16*)Oa, la, (const __nv_bfloat16*)Ob, lb, (__nv_bfloat16*)O, lse,
+                                       g.B, g.H, g.NB, g.N, g.b, s.stride_batch, s.stride_head, s.stride_token, rank,
+                                       consumer, head_begin, head_end);
   count_launch();
   SPARSP_CUDA_OK(cudaGetLastError());
   return SPARSP_OK;
