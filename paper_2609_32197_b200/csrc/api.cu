@@ -113,12 +113,14 @@ WsLayout make_layout(const Geometry& g, int P) {
   off += align_up(pooled, 256);
   L.scores = off;  // pooled-Q x pooled-K^T, fp32 [B][H][NB][NB]
   off += align_up((int64_t)g.B * g.H * g.NB * g.NB * 4, 256);
-  L.pairs = off;  // query-block pairs of the attention CTAs, int32 [B][H][ceil(NB/2)][2]
+  L.pairs = off;  // query blocks of the attention kernel's work items, int32 [B][H][ceil(NB/2)][2]
   off += align_up((int64_t)g.B * g.H * ((g.NB + 1) / 2) * 2 * 4, 256);
   L.slot = off;  // packed-buffer slot of every KV block for one consumer, int32 [B][H][NB]
   off += align_up((int64_t)g.B * g.H * g.NB * 4, 256);
   L.tile_base = off;  // first packed tile of that consumer per batch item, int64 [B]
   off += align_up((int64_t)g.B * 8, 256);
+  L.n_items = off;  // work items of the attention kernel per (batch, head), int32 [B][H]
+  off += align_up((int64_t)g.B * g.H * 4, 256);
   L.knorm = off;  // largest key norm of every KV block, fp32 [B][H][NB] (attention: bound on the scores of a tile)
   off += align_up((int64_t)g.B * g.H * g.NB * 4, 256);
   L.n_entries = off;  // blocks that anybody receives, int32

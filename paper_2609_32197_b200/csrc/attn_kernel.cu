@@ -42,6 +42,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "block_sets.cuh"
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -51,29 +52,25 @@ using namespace ptx;
 
 struct AttnParams {
   const uint32_t* mask;
-  // block 64: [B*H][ceil(NB/2)][2] query blocks of each item (second may be -1); block 128:
-  // [B*H][2*ceil(NB/2)] query block of each item (-1 = none), or NULL (item x handles block x)
+  // work items of every (batch, head), [B*H][2*ceil(NB/2)]: block 64: two query blocks per item (the second may be -1);
+  // block 128: one.  Only the first n_items[bh] items of a head exist: every one of them keeps at least one KV block.
   const int32_t* pairs;
-  // packed-source mode (NULL = every tile comes from K / V): slot[bh][j] = entry index of KV block j in
+  const int32_t* n_items;
+  // packed source only: slot[bh][j] = entry index of KV block j in
   // the consumer's packed buffer, or -1 if the consumer owns the block; tile_base = index of the
   // consumer's first tile in the packed tensor map (a device scalar)
   const int32_t* slot;
   const int64_t* tile_base;
-  // largest key norm (L2) of every KV block, [B*H][NB], or NULL: lets a softmax row skip the row-maximum pass
-  // of a tile whose scores provably stay within 2^kSkipMargin of the row's reference maximum
+  // K / V source only: largest key norm (L2) of every KV block that any row keeps, [B*H][NB]: lets a softmax row skip the
+  // row-maximum pass of a tile whose scores provably stay within 2^kSkipMargin of the row's reference maximum
   const float* knorm;
   __nv_bfloat16* O;
   float* lse;
   int32_t* status;
-  int32_t* work_counter;  // next work item to hand out; zeroed by the preparatory launch
-  // packed-source mode: number of work items per (batch, head) that can have rows at all (the consumer's query
-  // blocks come first in the pairs table), a device scalar; NULL = all per_bh items
-  const int32_t* active_per_bh;
+  int32_t* work_counter;  // items handed out beyond the first one of every CTA; zeroed by the preparatory launch
   int64_t N;
   int64_t sB, sH, sT;
-  int H, NB, Wd;
-  int per_bh;   // work items per (batch, head): NB (block 128) or ceil(NB/2) (block 64)
-  int n_items;  // B * H * per_bh
+  int BH, H, NB, Wd;
   float scale_log2;  // softmax scale * log2(e)
   long long wait_limit;
 };
@@ -195,7 +192,7 @@ __device__ __forceinline__ void named_bar_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-template <int D, int BLK>
+template <int D, int BLK, bool kPacked>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmP,
@@ -235,7 +232,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
   int* s_nent = reinterpret_cast<int*>(smem + C::kOffMisc + 8);   // [2]
   int* s_blk = reinterpret_cast<int*>(smem + C::kOffMisc + 16);   // [2][2] the item's query block(s); < 0 = absent
-  int* s_item = reinterpret_cast<int*>(smem + C::kOffMisc + 32);  // [2] the work item of each list buffer; < 0 = no more
+  int* s_item = reinterpret_cast<int*>(smem + C::kOffMisc + 32);  // [2] batch * H + head of the item in each list buffer; < 0 = no more
   int* s_rag = reinterpret_cast<int*>(smem + C::kOffMisc + 40);   // [2] the item's last tile reaches past the end of the sequence
   volatile int* s_frz = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 56);  // [4] per row group: reference frozen
   volatile int* s_pv_items = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 72);  // items whose P V are all issued
@@ -305,16 +302,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         for (int i = 0;; ++i) {
           const int buf = i & 1;
           mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 58, p.wait_limit);
-          const int it = s_item[buf];
-          if (it < 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
+          const int bh = s_item[buf];
+          if (bh < 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
           const int n_ent = s_nent[buf];
           const int n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
-          if (n_tiles > 0) {
-            const int bh = it / p.per_bh;
+          {
             const int batch = bh / p.H, head = bh % p.H;
             const uint16_t* entJ = sEntJ + buf * kMaxBlocks;
             const int32_t* entS = sSlot + buf * kMaxBlocks;
-            const int tile_base = p.slot ? (int)p.tile_base[batch] : 0;
+            const int tile_base = kPacked ? (int)p.tile_base[batch] : 0;
             for (int n = 0; n < n_tiles; ++n, ++vn) {
               const int st = vn % SV;
               mbar_wait_bounded_inline(v_empty + st, ((vn / SV) & 1) ^ 1, s_abort, 59, p.wait_limit);
@@ -323,7 +319,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   #pragma unroll
               for (int e = 0; e < C::kEPT; ++e) {
                 const int ent = min(n * C::kEPT + e, n_ent - 1);
-                const int slot = p.slot ? entS[ent] : -1;
+                const int slot = kPacked ? entS[ent] : -1;
                 if (slot < 0) {
                   const int tok = (int)entJ[ent] * BLK;
   #pragma unroll
@@ -343,20 +339,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     } else if (warp == 0) {
       // ================================ TMA producer: Q and K ===============================
       if (lane == 0) {
-        int kn = 0, qc = 0;  // K tiles loaded so far; items that had tiles
+        int kn = 0, qc = 0;  // K tiles loaded so far; items so far
         for (int i = 0;; ++i) {
           const int buf = i & 1;
           mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 51, p.wait_limit);
-          const int it = s_item[buf];
-          if (it < 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
+          const int bh = s_item[buf];
+          if (bh < 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
           const int n_ent = s_nent[buf];
           const int n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
-          if (n_tiles > 0) {
-            const int bh = it / p.per_bh;
+          {
             const int batch = bh / p.H, head = bh % p.H;
             const uint16_t* entJ = sEntJ + buf * kMaxBlocks;
             const int32_t* entS = sSlot + buf * kMaxBlocks;
-            const int tile_base = p.slot ? (int)p.tile_base[batch] : 0;
+            const int tile_base = kPacked ? (int)p.tile_base[batch] : 0;
             for (int n = 0; n < n_tiles; ++n, ++kn) {
               const int st = kn % SK;
               mbar_wait_bounded_inline(k_empty + st, ((kn / SK) & 1) ^ 1, s_abort, 57, p.wait_limit);
@@ -365,7 +360,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll
               for (int e = 0; e < C::kEPT; ++e) {
                 const int ent = min(n * C::kEPT + e, n_ent - 1);  // an absent second half re-reads the last entry
-                const int slot = p.slot ? entS[ent] : -1;
+                const int slot = kPacked ? entS[ent] : -1;
                 if (slot < 0) {
                   const int tok = (int)entJ[ent] * BLK;
 #pragma unroll
@@ -421,7 +416,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 53, p.wait_limit);
         if (s_item[buf] < 0) break;
         const int n_tiles = (s_nent[buf] + C::kEPT - 1) / C::kEPT;
-        if (n_tiles > 0) {
+        {
           // The tensor pipe works in issue order.  The first Q K^T of an item could be issued a tile or two
           // before the previous item ends, ahead of that item's last P V, and the epilogue (which waits for
           // that P V) would start ~1000 cycles later for nothing: the scores are not needed before the
@@ -515,34 +510,66 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     if (warp == 4) {
       // union of the item's (up to) two mask rows -> ascending entry list; flag bit q = kept by query
       // block blk[q].  Runs up to two items ahead of the consumers.
-      // Work items are handed out by a global counter (first come, first served), so CTAs whose items are
-      // short simply take more of them; the item number travels to the other roles with the list.
+      // Items are handed out head by head (a head's K and V stay in L2).  A CTA's first item is its own number, the
+      // following ones come from a global counter (first come, first served), so CTAs whose items are short simply take
+      // more of them; the head travels to the other roles with the list.
+      // Packed source: a head has few items, the consumer's; they are numbered without gaps, and since numbers only grow
+      // the place of an item is found by walking the heads' item counts forward, 32 heads at a time with a count per lane.
+      // K / V source: all query blocks count, and nearly always all of them keep something.
+      int hb = 0, hbase = 0, h_end;  // first head of the 32, items before it, items up to and including this lane's head
+      auto load_heads = [&]() {
+        h_end = hb + lane < p.BH ? p.n_items[hb + lane] : 0;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, h_end, s);
+          if (lane >= s) h_end += v;
+        }
+        h_end += hbase;
+      };
+      if (kPacked) load_heads();
       for (int i = 0;; ++i) {
         const int buf = i & 1;
         if (i >= 2) mbar_wait_bounded_inline(list_free + buf, ((i - 2) >> 1) & 1, s_abort, 50, p.wait_limit);
-        int it = 0;
-        if (lane == 0) it = atomicAdd(p.work_counter, 1);
-        it = __shfl_sync(0xffffffffu, it, 0);
-        // one consumer's call walks only the items of its own query blocks (the first `active` of every head)
-        const int active = p.active_per_bh ? *p.active_per_bh : p.per_bh;
-        if (it >= active * (p.n_items / p.per_bh) || *s_abort) {
+        int it = blockIdx.x;
+        if (i > 0) {
+          if (lane == 0) it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
+          it = __shfl_sync(0xffffffffu, it, 0);
+        }
+        int bh, x;
+        if (kPacked) {
+          uint32_t after;  // heads whose items end behind this one
+          while ((after = __ballot_sync(0xffffffffu, it < h_end)) == 0u && hb + 32 < p.BH) {
+            hbase = __shfl_sync(0xffffffffu, h_end, 31);
+            hb += 32;
+            load_heads();
+          }
+          const int f = __ffs(after) - 1;
+          bh = after ? hb + f : p.BH;
+          x = it - (f > 0 ? __shfl_sync(0xffffffffu, h_end, f - 1) : hbase);
+        } else {
+          const int per_bh = C::kStacked ? (p.NB + 1) / 2 : p.NB;
+          bh = it / per_bh;
+          x = it - bh * per_bh;
+          // Behind a head's last item are its query blocks that keep nothing: all CTAs go on with the next head.
+          while (bh < p.BH && x >= p.n_items[bh] && !*s_abort) {
+            if (lane == 0) {
+              atomicMax(p.work_counter, max((bh + 1) * per_bh - (int)gridDim.x, 0));
+              it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
+            }
+            it = __shfl_sync(0xffffffffu, it, 0);
+            bh = it / per_bh;
+            x = it - bh * per_bh;
+          }
+        }
+        if (bh >= p.BH || *s_abort) {
           if (lane == 0) {
             s_item[buf] = -1;
             mbar_arrive(list_ready + buf);
           }
           break;
         }
-        const int bh = it / active, x = it - bh * active;
-        it = bh * p.per_bh + x;  // the item's number in the full table, which the other roles derive the head from
-        int blk[2];
-        if (C::kStacked) {
-          const int32_t* pr = p.pairs + ((int64_t)bh * p.per_bh + x) * 2;
-          blk[0] = pr[0];
-          blk[1] = pr[1];
-        } else {
-          blk[0] = p.pairs ? p.pairs[(int64_t)bh * (2 * ((p.NB + 1) / 2)) + x] : x;
-          blk[1] = -1;
-        }
+        const int32_t* items = p.pairs + (int64_t)bh * (2 * ((p.NB + 1) / 2));
+        const int blk[2] = {C::kStacked ? items[2 * x] : items[x], C::kStacked ? items[2 * x + 1] : -1};
         uint16_t* entJ = sEntJ + buf * kMaxBlocks;
         uint8_t* entV = sEntV + buf * kMaxBlocks * 2;
         int32_t* entS = sSlot + buf * kMaxBlocks;
@@ -557,77 +584,94 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         // alternate in groups of two tiles (one of each per softmax warpgroup) while both last; then the rest
         // of the full tiles, the rest of the paired one-sided blocks and what is left of the longer one-sided
         // list.  With a single query block this is plain ascending order.
-        uint32_t cls[3] = {rb0 & rb1, rb0 & ~rb1, rb1 & ~rb0};
-        int before[3], total[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const int mine = __popc(cls[c]);
-          int incl = mine;
-#pragma unroll
-          for (int s = 1; s < 32; s <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, s);
-            if (lane >= s) incl += v;
-          }
-          before[c] = incl - mine;
-          total[c] = __shfl_sync(0xffffffffu, incl, 31);
+        // A mask word at a time, a lane per bit: next to busy softmax warps an instruction of this warp gets issued
+        // every several cycles, so the list is as late as it has instructions.
+        const uint32_t below = (1u << lane) - 1u;
+        int n_both = 0, n_mix = 0, n_grp = 0, running;
+        if (C::kStacked) {
+          n_both = __reduce_add_sync(0xffffffffu, __popc(rb0 & rb1));
+          const int n0 = __reduce_add_sync(0xffffffffu, __popc(rb0 & ~rb1)), n1 = __reduce_add_sync(0xffffffffu, __popc(rb1 & ~rb0));
+          n_mix = min(n0, n1);
+          // two full tiles (four blocks both keep), then two half-work tiles (two one-sided pairs), and so on
+          n_grp = min(n_both >> 2, n_mix >> 1);
+          running = n_both + n0 + n1;
+        } else {
+          running = __reduce_add_sync(0xffffffffu, __popc(rb0));
         }
-        const int n_both = total[0], n_mix = min(total[1], total[2]);
-        // two full tiles (four blocks both keep), then two half-work tiles (two one-sided pairs), and so on
-        const int n_grp = min(n_both >> 2, n_mix >> 1);
-        const int running = total[0] + total[1] + total[2];
-        float kn_max = 0.0f;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          uint32_t u = cls[c];
-          int idx = before[c];  // rank of the entry inside its class
-          while (u) {
-            const int t = __ffs(u) - 1;
-            u &= u - 1;
-            int pos;
-            if (c == 0) pos = idx < 4 * n_grp ? 8 * (idx >> 2) + (idx & 3) : 4 * n_grp + idx;
-            else if (idx < 2 * n_grp) pos = 8 * (idx >> 1) + 4 + 2 * (idx & 1) + (c - 1);
-            else if (idx < n_mix) pos = n_both + 2 * idx + (c - 1);
-            else pos = n_both + n_mix + idx;  // tail of the longer class
-            entJ[pos] = (uint16_t)(lane * 32 + t);
-            const int jb = lane * 32 + t;
-            const int nvalid = (int)min((int64_t)BLK, p.N - (int64_t)jb * BLK);
-            entV[pos * 2] = (uint8_t)(c != 2 ? nvalid : 0);      // keys valid for the first query block's rows
-            entV[pos * 2 + 1] = (uint8_t)(c != 1 ? nvalid : 0);  // ... for the second's
-            if (p.slot) entS[pos] = p.slot[(int64_t)bh * p.NB + lane * 32 + t];
-            if (p.knorm) {
-              const float kn = p.knorm[(int64_t)bh * p.NB + lane * 32 + t];
-              entN[pos] = kn;
-              kn_max = fmaxf(kn_max, kn);
+        int rag_pos = -1;               // where the sequence's ragged last block went
+        int at0 = 0, at1 = 0, at2 = 0;  // entries of each class so far
+        for (uint32_t todo = __ballot_sync(0xffffffffu, (rb0 | rb1) != 0u); todo; todo &= todo - 1) {
+          const int w = __ffs(todo) - 1;
+          const uint32_t w0 = __shfl_sync(0xffffffffu, rb0, w), w1 = C::kStacked ? __shfl_sync(0xffffffffu, rb1, w) : 0u;
+          const int jb = w * 32 + lane;
+          const int nvalid = (int)min((int64_t)BLK, p.N - (int64_t)jb * BLK);
+          if (C::kStacked) {
+            const uint32_t both = w0 & w1, only0 = w0 & ~w1, only1 = w1 & ~w0;
+            const bool in0 = (w0 >> lane) & 1u, in1 = (w1 >> lane) & 1u;
+            if (in0 || in1) {
+              int pos;
+              if (in0 && in1) {
+                const int idx = at0 + __popc(both & below);
+                pos = idx < 4 * n_grp ? 8 * (idx >> 2) + (idx & 3) : 4 * n_grp + idx;
+              } else {
+                const int c = in0 ? 0 : 1, idx = in0 ? at1 + __popc(only0 & below) : at2 + __popc(only1 & below);
+                if (idx < 2 * n_grp) pos = 8 * (idx >> 1) + 4 + 2 * (idx & 1) + c;
+                else if (idx < n_mix) pos = n_both + 2 * idx + c;
+                else pos = n_both + n_mix + idx;  // tail of the longer class
+              }
+              entJ[pos] = (uint16_t)jb;
+              // keys valid for the first query block's rows, for the second's
+              *reinterpret_cast<uint16_t*>(entV + pos * 2) = (uint16_t)((in0 ? nvalid : 0) | (in1 ? nvalid << 8 : 0));
+              if (nvalid < BLK) rag_pos = pos;
             }
-            ++idx;
+            at0 += __popc(both);
+            at1 += __popc(only0);
+            at2 += __popc(only1);
+          } else {
+            if ((w0 >> lane) & 1u) {
+              const int pos = at0 + __popc(w0 & below);
+              entJ[pos] = (uint16_t)jb;
+              entV[pos * 2] = (uint8_t)nvalid;
+              if (nvalid < BLK) rag_pos = pos;
+            }
+            at0 += __popc(w0);
+          }
+        }
+        __syncwarp();
+        // the softmax code lets only the LAST tile reach past the end of the sequence: if the last block of
+        // the sequence is ragged and in the list, it trades places with the last entry
+        rag_pos = __reduce_max_sync(0xffffffffu, rag_pos);
+        if (rag_pos >= 0) {
+          if (lane == 0) {
+            const int e = running - 1;
+            const uint16_t tj = entJ[rag_pos]; entJ[rag_pos] = entJ[e]; entJ[e] = tj;
+            for (int q = 0; q < 2; ++q) { const uint8_t tv = entV[rag_pos * 2 + q]; entV[rag_pos * 2 + q] = entV[e * 2 + q]; entV[e * 2 + q] = tv; }
+          }
+          __syncwarp();
+        }
+        // What the entries' blocks have in global memory, a lane per entry, two loads in flight
+        float kn_max = 0.0f;
+        for (int e = lane; e < running; e += 64) {
+          const int e2 = e + 32 < running ? e + 32 : e;
+          const int64_t at = (int64_t)bh * p.NB + entJ[e], at_2 = (int64_t)bh * p.NB + entJ[e2];
+          if (kPacked) {
+            const int32_t s1 = p.slot[at], s2 = p.slot[at_2];
+            entS[e] = s1;
+            entS[e2] = s2;
+          }
+          if (!kPacked) {
+            const float k1 = p.knorm[at], k2 = p.knorm[at_2];
+            entN[e] = k1;
+            entN[e2] = k2;
+            kn_max = fmaxf(kn_max, fmaxf(k1, k2));
           }
         }
 #pragma unroll
         for (int s = 16; s > 0; s >>= 1) kn_max = fmaxf(kn_max, __shfl_xor_sync(0xffffffffu, kn_max, s));
         __syncwarp();
-        // the softmax code lets only the LAST tile reach past the end of the sequence: if the last block of
-        // the sequence is ragged and in the list, it trades places with the last entry
-        bool last_ragged = false;
-        if ((int64_t)p.NB * BLK > p.N && running > 0) {
-          const int lw = (p.NB - 1) >> 5, lb = (p.NB - 1) & 31;
-          const uint32_t have = __shfl_sync(0xffffffffu, rb0 | rb1, lw);
-          if ((have >> lb) & 1u) {
-            last_ragged = true;
-            if (lane == 0) {
-              int r = 0;
-              while (r < running - 1 && entJ[r] != (uint16_t)(p.NB - 1)) ++r;
-              const int e = running - 1;
-              const uint16_t tj = entJ[r]; entJ[r] = entJ[e]; entJ[e] = tj;
-              for (int q = 0; q < 2; ++q) { const uint8_t tv = entV[r * 2 + q]; entV[r * 2 + q] = entV[e * 2 + q]; entV[e * 2 + q] = tv; }
-              if (p.slot) { const int32_t ts = entS[r]; entS[r] = entS[e]; entS[e] = ts; }
-              if (p.knorm) { const float tn = entN[r]; entN[r] = entN[e]; entN[e] = tn; }
-            }
-            __syncwarp();
-          }
-        }
         if (lane == 0) {
-          s_item[buf] = it;
-          s_rag[buf] = last_ragged ? 1 : 0;
+          s_item[buf] = bh;
+          s_rag[buf] = rag_pos >= 0 ? 1 : 0;
           s_nent[buf] = running;
           s_knmax[buf] = kn_max;
           s_blk[buf * 2] = blk[0];
@@ -653,20 +697,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     volatile int* frz = s_frz + rgrp;               // set by the warp that freezes the reference, cleared by the other
 
     int g0 = 0;  // number of the item's first tile
-    int qn = 0;  // items that had tiles (the phase of the Q barrier)
+    int qn = 0;  // items so far (the phase of the Q barrier)
     for (int i = 0;; ++i) {
       const int buf = i & 1;
       volatile float* ref = sRef + (i % 3) * 128;
       mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 56, p.wait_limit);
-      const int it = s_item[buf];
-      if (it < 0) break;
+      const int bh = s_item[buf];
+      if (bh < 0) break;
       const int n_ent = s_nent[buf];
       const int n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
       const uint8_t* entV = sEntV + buf * kMaxBlocks * 2 + (C::kStacked ? rh : 0);  // my query block's column
       const bool item_ragged = s_rag[buf] != 0;
       const float* entN = sEntN + buf * kMaxBlocks;
       const float kn_item = s_knmax[buf];
-      const int bh = it / p.per_bh;
       const int batch = bh / p.H, head = bh % p.H;
       // Once no score of any remaining tile of the item can exceed the row's reference maximum by more than
       // 2^kSkipMargin (Cauchy-Schwarz with the item's largest key norm), the reference is final: both warps of
@@ -675,40 +718,38 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       float q_bound = INFINITY;  // |q_row| * softmax scale * log2(e) (+0.1 %), once known
       float m_ref = -INFINITY;  // the row's reference maximum (log2 domain) as this thread last saw it
       float l_run = 0.0f;       // this thread's partial row sum, relative to m_ref
-      if (n_tiles > 0) {
-        if (p.knorm != nullptr && n_tiles >= 4) {
-          // The norm of my query row, read from the Q tile in shared memory while the item's first Q K^T runs (any
-          // order of its 16-byte units will do, so the swizzle does not matter).  Q stays there until the item's
-          // last Q K^T has completed; with four or more tiles that one cannot be issued before both warpgroups
-          // have released a score buffer, which they do after this.
-          mbar_wait_bounded_inline(q_full, qn & 1, s_abort, 42, p.wait_limit);
-          float ss[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // four chains, so that the additions do not wait for each other
+      if (!kPacked && n_tiles >= 4) {
+        // The norm of my query row, read from the Q tile in shared memory while the item's first Q K^T runs (any
+        // order of its 16-byte units will do, so the swizzle does not matter).  Q stays there until the item's
+        // last Q K^T has completed; with four or more tiles that one cannot be issued before both warpgroups
+        // have released a score buffer, which they do after this.
+        mbar_wait_bounded_inline(q_full, qn & 1, s_abort, 42, p.wait_limit);
+        float ss[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // four chains, so that the additions do not wait for each other
 #pragma unroll
-          for (int c = 0; c < D / 64; ++c) {
+        for (int c = 0; c < D / 64; ++c) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const uint4 v = *reinterpret_cast<const uint4*>(sQ + c * 16384 + row * 128 + (((k + lane) & 7) << 4));
-              const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+          for (int k = 0; k < 8; ++k) {
+            const uint4 v = *reinterpret_cast<const uint4*>(sQ + c * 16384 + row * 128 + (((k + lane) & 7) << 4));
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
-                ss[e] = fmaf(lo, lo, ss[e]);
-                ss[e] = fmaf(hi, hi, ss[e]);
-              }
+            for (int e = 0; e < 4; ++e) {
+              const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
+              ss[e] = fmaf(lo, lo, ss[e]);
+              ss[e] = fmaf(hi, hi, ss[e]);
             }
           }
-          q_bound = sqrtf((ss[0] + ss[1]) + (ss[2] + ss[3])) * p.scale_log2 * 1.001f;
-          // Both threads of a row compute the same bound from the same data, so both warps of a row group take this
-          // decision alike without talking to each other: the item runs on the fixed reference 0 from its first
-          // tile on -- no row maximum, no turns, no named barrier (neither warp arrives, neither waits).
-          if (__all_sync(0xffffffffu, q_bound * kn_item <= kStaticBound)) {
-            frozen = true;
-            m_ref = 0.0f;
-            ref[row] = 0.0f;  // (both threads of the row write the same value; the epilogue reads it)
-          }
         }
-        ++qn;
+        q_bound = sqrtf((ss[0] + ss[1]) + (ss[2] + ss[3])) * p.scale_log2 * 1.001f;
+        // Both threads of a row compute the same bound from the same data, so both warps of a row group take this
+        // decision alike without talking to each other: the item runs on the fixed reference 0 from its first
+        // tile on -- no row maximum, no turns, no named barrier (neither warp arrives, neither waits).
+        if (__all_sync(0xffffffffu, q_bound * kn_item <= kStaticBound)) {
+          frozen = true;
+          m_ref = 0.0f;
+          ref[row] = 0.0f;  // (both threads of the row write the same value; the epilogue reads it)
+        }
       }
+      ++qn;
 
       // One tile of this warpgroup.  kRagged = the sequence ends inside the tile (possible only for the item's
       // last tile): that variant carries the column masking, the common one stays small.
@@ -754,7 +795,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           // skipped: the exponentials stay below 2^kSkipMargin, harmless in fp32 / bf16, and the result does
           // not depend on the reference.
           bool skip = false;
-          if (!kRagged && p.knorm != nullptr) {
+          if (!kRagged && !kPacked) {
             float kn = entN[n * C::kEPT];
             if (C::kStacked) kn = fmaxf(kn, entN[min(n * 2 + 1, n_ent - 1)]);
             skip = __all_sync(0xffffffffu, q_bound * kn <= m_ref + kSkipMargin);
@@ -784,7 +825,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           // ---- my turn to look at / move the row's reference maximum (strictly in tile order) ----
           if (n > 0) named_bar_sync(bar_other, 64);
           const float m_cur = ref[row];
-          const int told = n > 0 ? *frz : 0;  // the row group's other warp froze the reference in its last turn
+          const int told = !kPacked && n > 0 ? *frz : 0;  // the row group's other warp froze the reference in its last turn
           if (m_cur != m_ref) {  // the other thread moved it since my last tile
             l_run *= ex2(m_ref - m_cur);  // m_ref = -inf: l_run is 0 and stays 0
             m_ref = m_cur;
@@ -796,7 +837,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           } else {
             // the first of the two warps to see the bound hold for the whole item says so, takes its last turn
             // without moving the reference (no score can make that necessary) and releases the other one more time
-            if (n + 1 < n_tiles && p.knorm != nullptr &&
+            if (!kPacked && n + 1 < n_tiles &&
                 __all_sync(0xffffffffu, q_bound * kn_item <= m_ref + kSkipMargin)) {
               frozen = true;
               if (lane == 0) *frz = 1;
@@ -908,11 +949,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       // ---- item epilogue: warpgroup x writes the column half x of every row -------------------------
       sStat[(buf * 2 + wg) * 128 + row] = make_float2(m_ref, l_run);
       named_bar_sync(9, 256);  // all of the item's decisions and P stores are done
-      if (n_tiles > 0) {
-        const int last = g0 + n_tiles - 1;
-        mbar_wait_bounded_inline(o_full + (last & 3), (last >> 2) & 1, s_abort, 40, p.wait_limit);
-        tc_fence_after();
-      }
+      const int last = g0 + n_tiles - 1;
+      mbar_wait_bounded_inline(o_full + (last & 3), (last >> 2) & 1, s_abort, 40, p.wait_limit);
+      tc_fence_after();
       {
         constexpr int HW = D / 2;
         const float m_fin = ref[row];
@@ -921,28 +960,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         // the barrier above, and the item before this one (its last user) is finished for all of them
         sRef[((i + 2) % 3) * 128 + row] = -INFINITY;
         float l = (st0.y > 0.0f ? st0.y * ex2(st0.x - m_fin) : 0.0f) + (st1.y > 0.0f ? st1.y * ex2(st1.x - m_fin) : 0.0f);
-        if (C::kSumMma) {  // the row sum is a tensor-memory column (CTA-uniform branch: the load is warp-collective)
-          l = 0.0f;
-          if (n_tiles > 0) {
-            uint32_t sums[16];
-            tmem_ld16(tmem_base + C::kColL + lane_off, sums);
-            tmem_ld_wait();
-            l = __uint_as_float(sums[0]);
-          }
+        if (C::kSumMma) {  // the row sum is a tensor-memory column
+          uint32_t sums[16];
+          tmem_ld16(tmem_base + C::kColL + lane_off, sums);
+          tmem_ld_wait();
+          l = __uint_as_float(sums[0]);
         }
         const float inv_l = l > 0.0f ? 1.0f / l : 0.0f;
         const int qb = C::kStacked ? s_blk[buf * 2 + rh] : s_blk[buf * 2];
         const int64_t tok = qb >= 0 ? (int64_t)qb * BLK + (C::kStacked ? (row & 63) : row) : p.N;
         __nv_bfloat16* orow = p.O + (int64_t)batch * p.sB + (int64_t)head * p.sH + tok * p.sT + wg * HW;
         uint32_t o[HW];
-        if (n_tiles > 0) {  // CTA-uniform: tensor-memory loads are warp-collective
 #pragma unroll
-          for (int c = 0; c < HW / 32; ++c) tmem_ld32(tO + wg * HW + c * 32, o + c * 32);
-          tmem_ld_wait();
-        } else {
-#pragma unroll
-          for (int e = 0; e < HW; ++e) o[e] = 0u;
-        }
+        for (int c = 0; c < HW / 32; ++c) tmem_ld32(tO + wg * HW + c * 32, o + c * 32);
+        tmem_ld_wait();
         // the accumulator is in registers: the next item's first P V may overwrite it
         tc_fence_before();
         __syncwarp();
@@ -987,21 +1018,55 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 }
 
 // ------------------------------------------------------------------------------------------------
-// Pairing pass: which two query blocks of a head share a CTA.  Blocks i and i+D are paired in
-// stripes (i mod 2D < D), leftovers pair up consecutively.  With `search` the offset D in 1..NB/2 that
-// maximises the summed overlap |M[i] & M[i+D]| of the kept lists is chosen per (batch, head) --
-// video attention is multi-diagonal, so the best partner of a block is typically the same position a
-// fixed number of blocks away; the more two stacked blocks share, the less of a 128-row tile's work
-// is masked away.  Without `search`, D = 1 (neighbours).  One CTA per (batch, head).
+// Preparation of an attention call, one launch for passes that do not depend on each other:
+//   CTAs [0, B*H)  fix the work items of one (batch, head) each (and, packed source, its table of packed slots);
+//   the rest       one warp per block: the largest key norm of the KV block, and the output rows of a query block that
+//                  keeps nothing (zeros, log-sum-exp -inf), so that such blocks never become work items.
+//
+// Block 64: which two query blocks share a Q tile.  Blocks i and i+D (positions in the consumer's ascending list of
+// blocks with a packed source, block numbers otherwise) are paired in stripes (i mod 2D < D), leftovers pair up
+// consecutively; the offset D in 1..n/2 that maximises the summed overlap |M[i] & M[i+D]| of the kept lists is chosen per
+// (batch, head) -- video attention is multi-diagonal, so the best partner of a block is typically the same position a
+// fixed number of blocks away; the more two stacked blocks share, the less of a 128-row tile's work is masked away.
+// (Mask rows in shared memory have an odd pitch: the threads' offsets differ by one row, a pitch of 32 words would put
+// them all on one bank.)
+// Items of one (batch, head) are handed out longest list first: the items still running when the queue
+// runs dry are then the short ones, which matters when list lengths vary (threshold selection, unions of two
+// stacked blocks).  Key = (list length << 10) | (1023 - index): equal lengths keep their index order.
+// Latency-bound integer work next to the key norms, which read K once: 132 us for the 774 MB of 40 heads x 75600 keys
+// (158 us when a lane's loads waited for each other), 7 us for 26 heads x 6034 keys (24 us).
 // ------------------------------------------------------------------------------------------------
-constexpr int kPairThreads = 256;
+constexpr int kPrepThreads = 256;
 constexpr int kPairSample = 8;
 
-// Sorts n keys (n a power of two, <= 1024) in shared memory into descending order; all kPairThreads threads call it.
+struct PrepParams {
+  const uint32_t* mask;
+  int32_t* pairs;
+  int32_t* n_items;
+  int32_t* work_counter;
+  const __nv_bfloat16* K;
+  __nv_bfloat16* O;
+  float* lse;
+  float* knorm;
+  int64_t sB, sH, sT, N;
+  int BH, H, NB, Wd, b;
+  // packed source only
+  const int32_t* rank;
+  const uint32_t* U;
+  const int64_t* seg_off;
+  const int64_t* seg_total;
+  const int64_t* dst_base;
+  int64_t tile_bytes;
+  int32_t* slot;
+  int64_t* tile_base;
+  int P, consumer;
+};
+
+// Sorts n keys (n a power of two, <= 1024) in shared memory into descending order; all threads call it.
 __device__ __forceinline__ void sort_keys_descending(uint32_t* keys, int n) {
   for (int k = 2; k <= n; k <<= 1) {
     for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < n; t += kPairThreads) {
+      for (int t = threadIdx.x; t < n; t += kPrepThreads) {
         const int u = t ^ j;
         if (u > t) {
           const uint32_t a = keys[t], b = keys[u];
@@ -1016,115 +1081,229 @@ __device__ __forceinline__ void sort_keys_descending(uint32_t* keys, int n) {
   }
 }
 
-// Work items of one (batch, head) are handed out longest list first: the items still running when the queue
-// runs dry are then the short ones, which matters when list lengths vary (threshold selection, unions of two
-// stacked blocks).  Key = (list length << 10) | (1023 - index): equal lengths keep their index order.
 __device__ __forceinline__ int next_pow2(int n) {
   int v = 1;
   while (v < n) v <<= 1;
   return v;
 }
 
-// block 128: order[x] = the query block that item x of this (batch, head) handles
-__device__ __forceinline__ void order_body(const uint32_t* __restrict__ mask, int NB, int Wd,
-                                           int32_t* __restrict__ pairs, int bh) {
-  __shared__ uint32_t s_keys[1024];
-  const int n2 = next_pow2(NB);
-  const uint32_t* rows = mask + (int64_t)bh * NB * Wd;
-  for (int i = threadIdx.x; i < n2; i += kPairThreads) {
-    uint32_t key = 0;
-    if (i < NB) {
-      int len = 0;
-      for (int w = 0; w < Wd; ++w) len += __popc(rows[(int64_t)i * Wd + w]);
-      key = ((uint32_t)len << 10) | (uint32_t)(1023 - i);
+// Work items of one (batch, head) among the n query blocks list[0..n) (NULL = all blocks); returns their number.
+__device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uint16_t* list, int n, unsigned char* smem_raw) {
+  __shared__ uint32_t s_keys[kMaxBlocks];
+  __shared__ uint32_t s_pair[kMaxBlocks / 2];  // positions of an item's two blocks, (second or 0xffff) << 16 | first
+  __shared__ unsigned int s_best;              // (score << 10) | (1023 - D): max = best score, smallest D
+  const uint32_t* rows = p.mask + (int64_t)bh * p.NB * p.Wd;
+  auto block = [&](int pos) -> int { return list ? list[pos] : pos; };
+  int n_keys;
+  if (p.b == 64) {
+    uint32_t* m = reinterpret_cast<uint32_t*>(smem_raw);  // [n][pitch]
+    const int Wd = p.Wd, pitch = Wd | 1;
+    if (threadIdx.x == 0) s_best = 1023u - 1u;  // default D = 1
+    for (int idx = threadIdx.x; idx < n * Wd; idx += kPrepThreads) {
+      const int i = idx / Wd, w = idx - i * Wd;
+      m[i * pitch + w] = rows[(int64_t)block(i) * Wd + w];
     }
-    s_keys[i] = key;
-  }
-  __syncthreads();
-  sort_keys_descending(s_keys, n2);
-  int32_t* out = pairs + (int64_t)bh * ((NB + 1) / 2) * 2;
-  for (int x = threadIdx.x; x < NB; x += kPairThreads) out[x] = 1023 - (int)(s_keys[x] & 1023u);
-}
-
-__device__ __forceinline__ void pair_body(const uint32_t* __restrict__ mask, int NB, int Wd, int search,
-                                          int32_t* __restrict__ pairs, int bh, unsigned char* smem_raw) {
-  uint32_t* m = reinterpret_cast<uint32_t*>(smem_raw);  // [NB][Wd]
-  __shared__ unsigned int s_best;                        // (score << 10) | (1023 - D): max = best score, smallest D
-  if (threadIdx.x == 0) s_best = (0u << 10) | (1023u - 1u);  // default D = 1
-  if (search) {
-    const uint32_t* src = mask + (int64_t)bh * NB * Wd;
-    for (int idx = threadIdx.x; idx < NB * Wd; idx += kPairThreads) m[idx] = src[idx];
     __syncthreads();
-    for (int d = 1 + threadIdx.x; d <= NB / 2; d += kPairThreads) {
+    for (int d = 1 + threadIdx.x; d <= n / 2; d += kPrepThreads) {
       unsigned int score = 0;
-      for (int i = 0; i + d < NB; i += kPairSample)  // every kPairSample-th row is enough to rank offsets
-        for (int w = 0; w < Wd; ++w) score += __popc(m[i * Wd + w] & m[(i + d) * Wd + w]);
+      for (int i = 0; i + d < n; i += kPairSample)  // every kPairSample-th row is enough to rank offsets
+        for (int w = 0; w < Wd; ++w) score += __popc(m[i * pitch + w] & m[(i + d) * pitch + w]);
       atomicMax(&s_best, (score << 10) | (unsigned int)(1023 - d));
     }
-  }
-  __syncthreads();
-  const int D = 1023 - (int)(s_best & 1023u);
-  // stripes: rows with (i mod 2D) < D pair with i + D; the rows of the last partial stripe that have
-  // no partner form one consecutive run and pair up as neighbours
-  const int full = NB / (2 * D), R = NB % (2 * D);
-  const int np_last = max(R - D, 0), lo_end = min(R, D);
-  int32_t* out = pairs + (int64_t)bh * ((NB + 1) / 2) * 2;
-  for (int i = threadIdx.x; i < NB; i += kPairThreads) {
-    const int st = i / (2 * D), pos = i % (2 * D);
-    if (st < full) {
-      if (pos < D) {
-        out[2 * (st * D + pos)] = i;
-        out[2 * (st * D + pos) + 1] = i + D;
-      }
-    } else if (pos < np_last) {
-      out[2 * (full * D + pos)] = i;
-      out[2 * (full * D + pos) + 1] = i + D;
-    } else if (pos < lo_end) {
-      const int k = pos - np_last, n_left = lo_end - np_last;
-      if ((k & 1) == 0) {
-        const int c = full * D + np_last + k / 2;
-        out[2 * c] = i;
-        out[2 * c + 1] = (k + 1 < n_left) ? i + 1 : -1;
+    __syncthreads();
+    const int D = 1023 - (int)(s_best & 1023u);
+    // stripes: positions with (i mod 2D) < D pair with i + D; the positions of the last partial stripe that have
+    // no partner form one consecutive run and pair up as neighbours
+    const int full = n / (2 * D), R = n % (2 * D);
+    const int np_last = max(R - D, 0), lo_end = min(R, D);
+    for (int i = threadIdx.x; i < n; i += kPrepThreads) {
+      const int st = i / (2 * D), pos = i % (2 * D);
+      if (st < full) {
+        if (pos < D) s_pair[st * D + pos] = (uint32_t)(i + D) << 16 | (uint32_t)i;
+      } else if (pos < np_last) {
+        s_pair[full * D + pos] = (uint32_t)(i + D) << 16 | (uint32_t)i;
+      } else if (pos < lo_end) {
+        const int k = pos - np_last, n_left = lo_end - np_last;
+        if ((k & 1) == 0)
+          s_pair[full * D + np_last + k / 2] = (k + 1 < n_left ? (uint32_t)(i + 1) : 0xffffu) << 16 | (uint32_t)i;
       }
     }
-  }
-  // longest union first
-  __shared__ uint32_t s_keys[512];
-  const int n_pairs = (NB + 1) / 2, n2 = next_pow2(n_pairs);
-  const uint32_t* rows = mask + (int64_t)bh * NB * Wd;
-  __syncthreads();  // the pairs written above are visible to the whole block
-  for (int c = threadIdx.x; c < n2; c += kPairThreads) {
-    uint32_t key = 0;
-    if (c < n_pairs) {
-      const int a = out[2 * c], b = out[2 * c + 1];
-      int len = 0;
-      for (int w = 0; w < Wd; ++w)
-        len += __popc(rows[(int64_t)a * Wd + w] | (b >= 0 ? rows[(int64_t)b * Wd + w] : 0u));
-      key = ((uint32_t)len << 10) | (uint32_t)(1023 - c);
+    __syncthreads();
+    n_keys = (n + 1) / 2;
+    for (int c = threadIdx.x; c < next_pow2(n_keys); c += kPrepThreads) {
+      uint32_t key = 0;
+      if (c < n_keys) {
+        const int a = (int)(s_pair[c] & 0xffffu), b2 = (int)(s_pair[c] >> 16);
+        int len = 0;
+        for (int w = 0; w < Wd; ++w) len += __popc(m[a * pitch + w] | (b2 != 0xffff ? m[b2 * pitch + w] : 0u));
+        key = ((uint32_t)len << 10) | (uint32_t)(1023 - c);
+      }
+      s_keys[c] = key;
     }
-    s_keys[c] = key;
+  } else {
+    n_keys = n;
+    for (int i = threadIdx.x; i < next_pow2(n_keys); i += kPrepThreads) {
+      uint32_t key = 0;
+      if (i < n) {
+        const uint32_t* row = rows + (int64_t)block(i) * p.Wd;
+        int len = 0;
+#pragma unroll 8
+        for (int w = 0; w < p.Wd; ++w) len += __popc(row[w]);
+        key = ((uint32_t)len << 10) | (uint32_t)(1023 - i);
+      }
+      s_keys[i] = key;
+    }
   }
   __syncthreads();
-  sort_keys_descending(s_keys, n2);
-  int pa[2], pb[2];  // at most 512 pairs for 256 threads
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int x = threadIdx.x + r * kPairThreads;
-    if (x < n_pairs) {
+  sort_keys_descending(s_keys, next_pow2(n_keys));
+  int32_t* out = p.pairs + (int64_t)bh * (2 * ((p.NB + 1) / 2));
+  int n_live = 0;
+  for (int x0 = 0; x0 < n_keys; x0 += kPrepThreads) {
+    const int x = x0 + (int)threadIdx.x;
+    const bool live = x < n_keys && (s_keys[x] >> 10) != 0u;
+    if (live) {
       const int c = 1023 - (int)(s_keys[x] & 1023u);
-      pa[r] = out[2 * c];
-      pb[r] = out[2 * c + 1];
+      if (p.b == 64) {
+        const int a = (int)(s_pair[c] & 0xffffu), b2 = (int)(s_pair[c] >> 16);
+        out[2 * x] = block(a);
+        out[2 * x + 1] = b2 != 0xffff ? block(b2) : -1;
+      } else {
+        out[x] = block(c);
+      }
     }
+    n_live += __syncthreads_count(live);
   }
+  return n_live;
+}
+
+// slot[bh][j] = entry index of block j inside the consumer's packed buffer (pack order: producer ascending,
+// head ascending, block ascending), for every block of the consumer's union that another rank owns; -1 elsewhere.
+__device__ __forceinline__ void make_slots(const PrepParams& p, int bh) {
+  __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int bb = bh / p.H, h = bh % p.H;
+  const int64_t br = (int64_t)bb * p.P + p.consumer;
+  int32_t* out = p.slot + (int64_t)bh * p.NB;
+  for (int j = threadIdx.x; j < p.NB; j += kPrepThreads) out[j] = -1;
+  own_words(p.rank, p.NB, p.Wd, p.P, own_s);
   __syncthreads();
+  const uint32_t u = lane < p.Wd ? p.U[(br * p.H + h) * p.Wd + lane] : 0u;
+  for (int prod = warp; prod < p.P; prod += kPrepThreads / 32) {
+    if (prod == p.consumer) continue;
+    uint32_t bits = lane < p.Wd ? u & own_s[prod * p.Wd + lane] : 0u;
+    int total;
+    int at = (int)p.seg_off[(br * p.P + prod) * p.H + h] + bits_below(bits, lane, &total);
+    for (; bits; bits &= bits - 1, ++at) out[lane * 32 + __ffs(bits) - 1] = at;
+  }
+}
+
+// The output rows of query block i: zeros and a log-sum-exp of -inf.  One warp.
+template <int D>
+__device__ __forceinline__ void clear_rows(const PrepParams& p, int64_t bh, int i) {
+  constexpr int LPT = D / 8;
+  const int lane = threadIdx.x & 31;
+  const int64_t tok0 = (int64_t)i * p.b;
+  const int n = (int)min((int64_t)p.b, p.N - tok0);
+  __nv_bfloat16* o = p.O + (bh / p.H) * p.sB + (bh % p.H) * p.sH + tok0 * p.sT + (lane % LPT) * 8;
+  for (int r = lane / LPT; r < n; r += 32 / LPT)
+    *reinterpret_cast<uint4*>(o + (int64_t)r * p.sT) = make_uint4(0u, 0u, 0u, 0u);
+  if (p.lse)
+    for (int r = lane; r < n; r += 32) p.lse[bh * p.N + tok0 + r] = -INFINITY;
+}
+
+// Largest L2 norm of the keys of block j (times 1.001): with the norm of a query row it bounds the scores of a tile.
+// One warp, d/8 lanes per token, kNormLoads 16-byte loads of every lane in flight.
+constexpr int kNormLoads = 16;
+template <int D>
+__device__ __forceinline__ float block_norm(const PrepParams& p, int64_t bh, int j) {
+  constexpr int LPT = D / 8;     // lanes per token
+  constexpr int TPW = 32 / LPT;  // tokens per warp load
+  const int lane = threadIdx.x & 31;
+  const int64_t tok0 = (int64_t)j * p.b;
+  const int n = (int)min((int64_t)p.b, p.N - tok0);
+  const __nv_bfloat16* base = p.K + (bh / p.H) * p.sB + (bh % p.H) * p.sH + tok0 * p.sT + (lane % LPT) * 8;
+  float best = 0.0f;
+  for (int t0 = lane / LPT; t0 < p.b; t0 += TPW * kNormLoads) {  // (p.b is a multiple of TPW: the lanes stay together)
+    uint4 v[kNormLoads];
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int x = threadIdx.x + r * kPairThreads;
-    if (x < n_pairs) {
-      out[2 * x] = pa[r];
-      out[2 * x + 1] = pb[r];
+    for (int k = 0; k < kNormLoads; ++k) {
+      const int t = t0 + k * TPW;
+      v[k] = t < n ? *reinterpret_cast<const uint4*>(base + (int64_t)t * p.sT) : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int k = 0; k < kNormLoads; ++k) {
+      const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+      float ss = 0.0f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
+        ss = fmaf(lo, lo, ss);
+        ss = fmaf(hi, hi, ss);
+      }
+#pragma unroll
+      for (int sft = 1; sft < LPT; sft <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, sft);
+      best = fmaxf(best, ss);
     }
   }
+#pragma unroll
+  for (int sft = LPT; sft < 32; sft <<= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, sft));
+  return sqrtf(best) * 1.001f;
+}
+
+template <int D, bool kPacked>
+__global__ void __launch_bounds__(kPrepThreads) attn_prep_kernel(const PrepParams p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *p.work_counter = 0;  // the attention kernel's work queue
+  if ((int)blockIdx.x < p.BH) {
+    const int bh = blockIdx.x;
+    int n_live;
+    if (kPacked) {
+      __shared__ uint32_t s_words[kMaxWords];
+      __shared__ uint16_t s_list[kMaxBlocks];
+      rank_words(p.rank, p.NB, p.consumer, s_words);
+      const int n = list_blocks(s_words, p.NB, s_list);
+      n_live = make_items(p, bh, s_list, n, smem_raw);
+      if (n_live > 0) make_slots(p, bh);
+      if (bh % p.H == 0 && warp == 0) {  // first tile of the consumer's buffer for this batch item
+        const int64_t br = (int64_t)(bh / p.H) * p.P + p.consumer;
+        int64_t first = 0;
+        if (p.dst_base) {
+          first = p.dst_base[br] / p.tile_bytes;
+        } else {
+          for (int64_t t = lane; t < br; t += 32) first += 2 * p.seg_total[t];
+#pragma unroll
+          for (int s = 16; s >= 1; s >>= 1) first += __shfl_xor_sync(0xffffffffu, first, s);
+        }
+        if (lane == 0) p.tile_base[bh / p.H] = first;
+      }
+    } else {
+      n_live = make_items(p, bh, nullptr, p.NB, smem_raw);
+    }
+    if (threadIdx.x == 0) p.n_items[bh] = n_live;
+    return;
+  }
+  const int64_t unit = (int64_t)((int)blockIdx.x - p.BH) * (kPrepThreads / 32) + warp;  // (batch, head, block)
+  if (unit >= (int64_t)p.BH * p.NB) return;
+  const int64_t bh = unit / p.NB;
+  const int j = (int)(unit - bh * p.NB);
+  if (kPacked && p.rank[j] != p.consumer) return;
+  const uint32_t row = lane < p.Wd ? p.mask[unit * p.Wd + lane] : 0u;
+  if (!__any_sync(0xffffffffu, row != 0u)) clear_rows<D>(p, bh, j);
+  if (kPacked) return;  // remote keys live in the packed buffer: every tile takes its row maximum
+  // A block that nobody keeps needs no norm.  Its own row nearly always keeps it; otherwise the column decides.
+  const int w = j >> 5;
+  bool kept = (__shfl_sync(0xffffffffu, row, w) >> (j & 31)) & 1u;
+  if (!kept) {
+    const uint32_t* col = p.mask + bh * p.NB * p.Wd + w;
+    uint32_t any = 0;
+#pragma unroll 4
+    for (int i = lane; i < p.NB; i += 32) any |= col[(int64_t)i * p.Wd];
+    kept = __any_sync(0xffffffffu, (any >> (j & 31)) & 1u);
+  }
+  if (!kept) return;
+  const float norm = block_norm<D>(p, bh, j);
+  if (lane == 0) p.knorm[unit] = norm;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1198,7 +1377,7 @@ static int make_packed_tmap(CUtensorMap* out, const void* packed, int64_t capaci
   return SPARSP_OK;
 }
 
-template <int D, int BLK>
+template <int D, int BLK, bool kPacked>
 static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, const void* V,
                          const void* packed, int64_t packed_capacity, const AttnParams& p, cudaStream_t st) {
   CUtensorMap tq, tk, tv, tp;
@@ -1206,28 +1385,27 @@ static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q
   if ((rc = make_tile_tmap(&tq, Q, s, g, BLK, true)) != SPARSP_OK) return rc;
   if ((rc = make_tile_tmap(&tk, K, s, g, BLK, true)) != SPARSP_OK) return rc;
   if ((rc = make_tile_tmap(&tv, V, s, g, BLK, true)) != SPARSP_OK) return rc;
-  if (packed) {
+  if (kPacked) {
     if ((rc = make_packed_tmap(&tp, packed, packed_capacity, g)) != SPARSP_OK) return rc;
   } else {
-    tp = tk;  // never used without a slot table
+    tp = tk;  // never used
   }
-  auto kern = attn_fwd_kernel<D, BLK>;
+  auto kern = attn_fwd_kernel<D, BLK, kPacked>;
   const int smem = AttnCfg<D, BLK>::kDynamic;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
   // work item = one 128-row Q tile (a 128-token block, or a pair of 64-token blocks); one persistent CTA per SM
-  AttnParams pp = p;
-  pp.per_bh = BLK == 128 ? g.NB : (g.NB + 1) / 2;
-  pp.n_items = g.B * g.H * pp.per_bh;
+  const int64_t most = (int64_t)g.B * g.H * (BLK == 128 ? g.NB : (g.NB + 1) / 2);
   int dev = 0, sms = 0;
   SPARSP_CUDA_OK(cudaGetDevice(&dev));
   SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  dim3 grid((unsigned)std::min(pp.n_items, sms));
-  kern<<<grid, kAttnThreads, smem, st>>>(tq, tk, tv, tp, pp);
+  const unsigned grid = (unsigned)std::min<int64_t>(most, sms);
+  kern<<<grid, kAttnThreads, smem, st>>>(tq, tk, tv, tp, p);
   count_launch();
   SPARSP_CUDA_OK(cudaGetLastError());
   return SPARSP_OK;
 }
 
+template <bool kPacked>
 static int launch_attn_common(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, const void* V,
                               const void* packed, int64_t packed_capacity, AttnParams p, float scale, void* O,
                               float* lse, char* ws, const WsLayout& L, cudaStream_t st) {
@@ -1239,219 +1417,98 @@ static int launch_attn_common(const sparsp_shape& s, const Geometry& g, const vo
   p.sB = s.stride_batch;
   p.sH = s.stride_head;
   p.sT = s.stride_token;
+  p.BH = g.B * g.H;
   p.H = g.H;
   p.NB = g.NB;
   p.Wd = g.Wd;
   const float sc = scale > 0.0f ? scale : 1.0f / sqrtf((float)g.d);
   p.scale_log2 = sc * 1.4426950408889634f;
   p.wait_limit = 200000000LL;  // about 0.1 s of SM clocks
-  if (g.d == 64 && g.b == 64) return launch_attn_t<64, 64>(s, g, Q, K, V, packed, packed_capacity, p, st);
-  if (g.d == 64 && g.b == 128) return launch_attn_t<64, 128>(s, g, Q, K, V, packed, packed_capacity, p, st);
-  if (g.d == 128 && g.b == 64) return launch_attn_t<128, 64>(s, g, Q, K, V, packed, packed_capacity, p, st);
-  return launch_attn_t<128, 128>(s, g, Q, K, V, packed, packed_capacity, p, st);
+  if (g.d == 64 && g.b == 64) return launch_attn_t<64, 64, kPacked>(s, g, Q, K, V, packed, packed_capacity, p, st);
+  if (g.d == 64 && g.b == 128) return launch_attn_t<64, 128, kPacked>(s, g, Q, K, V, packed, packed_capacity, p, st);
+  if (g.d == 128 && g.b == 64) return launch_attn_t<128, 64, kPacked>(s, g, Q, K, V, packed, packed_capacity, p, st);
+  return launch_attn_t<128, 128, kPacked>(s, g, Q, K, V, packed, packed_capacity, p, st);
 }
 
-// Largest L2 norm of the keys of every KV block (times 1.001), fp32 [B*H][NB]: with the norm of a query row it
-// bounds the scores of a tile.  One warp per (batch, head, block); d/8 lanes read one token (16 bytes each).
-template <int D>
-__device__ __forceinline__ void knorm_body(const __nv_bfloat16* __restrict__ K, int64_t sB, int64_t sH, int64_t sT,
-                                           int H, int NB, int b, int64_t N, int64_t n_units, float* __restrict__ out,
-                                           int64_t unit) {
-  constexpr int LPT = D / 8;       // lanes per token
-  constexpr int TPW = 32 / LPT;    // tokens per warp pass
-  if (unit >= n_units) return;
-  const int lane = threadIdx.x & 31;
-  const int j = (int)(unit % NB);
-  const int64_t bh = unit / NB;
-  const int64_t batch = bh / H, head = bh % H;
-  const __nv_bfloat16* base = K + batch * sB + head * sH;
-  float best = 0.0f;
-#pragma unroll 8
-  for (int t0 = 0; t0 < b; t0 += TPW) {
-    const int64_t tok = (int64_t)j * b + t0 + lane / LPT;
-    float ss = 0.0f;
-    if (tok < N && t0 + lane / LPT < b) {
-      const uint4 v = *reinterpret_cast<const uint4*>(base + tok * sT + (lane % LPT) * 8);
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
-        ss = fmaf(lo, lo, ss);
-        ss = fmaf(hi, hi, ss);
-      }
-    }
-#pragma unroll
-    for (int sft = 1; sft < LPT; sft <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, sft);
-    best = fmaxf(best, ss);
-  }
-#pragma unroll
-  for (int sft = LPT; sft < 32; sft <<= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, sft));
-  if (lane == 0) out[unit] = sqrtf(best) * 1.001f;
+template <bool kPacked>
+static int launch_prep(const Geometry& g, const PrepParams& p, cudaStream_t st) {
+  auto kern = g.d == 64 ? attn_prep_kernel<64, kPacked> : attn_prep_kernel<128, kPacked>;
+  const int smem = g.b == 64 ? g.NB * (g.Wd | 1) * 4 : 0;
+  SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
+  constexpr int kWarps = kPrepThreads / 32;
+  const int64_t blocks = p.BH + ((int64_t)p.BH * g.NB + kWarps - 1) / kWarps;
+  kern<<<(unsigned)blocks, kPrepThreads, smem, st>>>(p);
+  count_launch();
+  SPARSP_CUDA_OK(cudaGetLastError());
+  return SPARSP_OK;
 }
 
-// One launch for the two passes that precede the attention kernel and do not depend on each other: blocks
-// [0, n_pair) fix the work items of one (batch, head) each (block 64: which query blocks are stacked; both block
-// sizes: longest list first), the rest take the largest
-// key norm of every KV block (times 1.001), fp32 [B*H][NB], one warp per block and d/8 lanes per token: with the
-// norm of a query row it bounds the scores of a tile.
-template <int D>
-__global__ void __launch_bounds__(kPairThreads) attn_prep_kernel(const uint32_t* __restrict__ mask, int NB, int Wd,
-                                                                 int32_t* __restrict__ pairs, int n_pair,
-                                                                 const __nv_bfloat16* __restrict__ K, int64_t sB,
-                                                                 int64_t sH, int64_t sT, int H, int b, int64_t N,
-                                                                 int64_t n_units, float* __restrict__ knorm,
-                                                                 int32_t* __restrict__ work_counter) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (blockIdx.x == 0 && threadIdx.x == 0) *work_counter = 0;  // the attention kernel's work queue
-  if ((int)blockIdx.x < n_pair) {
-    if (b == 64) pair_body(mask, NB, Wd, 1, pairs, (int)blockIdx.x, smem_raw);
-    else order_body(mask, NB, Wd, pairs, (int)blockIdx.x);
-  } else {
-    const int64_t unit = ((int64_t)(blockIdx.x - n_pair) * kPairThreads + threadIdx.x) >> 5;
-    knorm_body<D>(K, sB, sH, sT, H, NB, b, N, n_units, knorm, unit);
-  }
+static PrepParams prep_params(const sparsp_shape& s, const Geometry& g, const void* K, const uint32_t* mask, void* O,
+                              float* lse, char* ws, const WsLayout& L) {
+  PrepParams p = {};
+  p.mask = mask;
+  p.pairs = (int32_t*)(ws + L.pairs);
+  p.n_items = (int32_t*)(ws + L.n_items);
+  p.work_counter = (int32_t*)(ws + L.status) + kWorkCounterWord;
+  p.K = (const __nv_bfloat16*)K;
+  p.O = (__nv_bfloat16*)O;
+  p.lse = lse;
+  p.sB = s.stride_batch;
+  p.sH = s.stride_head;
+  p.sT = s.stride_token;
+  p.N = g.N;
+  p.BH = g.B * g.H;
+  p.H = g.H;
+  p.NB = g.NB;
+  p.Wd = g.Wd;
+  p.b = g.b;
+  return p;
 }
 
 int launch_attn(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, const void* V,
                 const uint32_t* mask, float scale, void* O, float* lse, char* ws, const WsLayout& L,
                 cudaStream_t st) {
-  int32_t* pairs = (int32_t*)(ws + L.pairs);  // block 64: the two stacked blocks of each item; block 128: its block
-  float* knorm = (float*)(ws + L.knorm);
-  {
-    const int n_pair = g.B * g.H;
-    const size_t smem = g.b == 64 ? (size_t)g.NB * g.Wd * 4 : 0;
-    const int64_t n_units = (int64_t)g.B * g.H * g.NB;
-    const unsigned blocks = (unsigned)(n_pair + (n_units * 32 + kPairThreads - 1) / kPairThreads);
-    const int64_t sB = s.stride_batch > 0 ? s.stride_batch : 0;
-    if (g.d == 64) {
-      SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)attn_prep_kernel<64>, (int)smem));
-      attn_prep_kernel<64><<<blocks, kPairThreads, smem, st>>>(mask, g.NB, g.Wd, pairs, n_pair, (const __nv_bfloat16*)K, sB,
-                                                             s.stride_head, s.stride_token, g.H, g.b, g.N, n_units, knorm,
-                                                             (int32_t*)(ws + L.status) + kWorkCounterWord);
-    } else {
-      SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)attn_prep_kernel<128>, (int)smem));
-      attn_prep_kernel<128><<<blocks, kPairThreads, smem, st>>>(mask, g.NB, g.Wd, pairs, n_pair, (const __nv_bfloat16*)K, sB,
-                                                              s.stride_head, s.stride_token, g.H, g.b, g.N, n_units, knorm,
-                                                             (int32_t*)(ws + L.status) + kWorkCounterWord);
-    }
-    count_launch();
-  }
-  AttnParams p;
+  PrepParams pre = prep_params(s, g, K, mask, O, lse, ws, L);
+  pre.knorm = (float*)(ws + L.knorm);
+  const int rc = launch_prep<false>(g, pre, st);
+  if (rc != SPARSP_OK) return rc;
+  AttnParams p = {};
   p.mask = mask;
-  p.pairs = pairs;
-  p.slot = nullptr;
-  p.tile_base = nullptr;
-  p.active_per_bh = nullptr;
-  p.knorm = knorm;
-  return launch_attn_common(s, g, Q, K, V, nullptr, 0, p, scale, O, lse, ws, L, st);
+  p.pairs = pre.pairs;
+  p.n_items = pre.n_items;
+  p.knorm = pre.knorm;
+  return launch_attn_common<false>(s, g, Q, K, V, nullptr, 0, p, scale, O, lse, ws, L, st);
 }
 
 // ------------------------------------------------------------------------------------------------
-// Packed-source attention for one consumer rank: pairs are formed among the consumer's own query
+// Packed-source attention for one consumer rank: items are formed among the consumer's own query
 // blocks, and every kept KV block the consumer does not own is read from the consumer's packed buffer.
 // ------------------------------------------------------------------------------------------------
-// pairs of the consumer's blocks (ascending, neighbours in that order); the rest of the table is (-1, -1)
-// Also leaves the number of work items per (batch, head) that hold any of the consumer's blocks.
-__global__ void pair_rank_kernel(const int32_t* __restrict__ rank, int NB, int consumer, int stacked,
-                                 int32_t* __restrict__ pairs, int32_t* __restrict__ active_per_bh) {
-  const int n_pairs = (NB + 1) / 2;
-  int32_t* out = pairs + (int64_t)blockIdx.x * n_pairs * 2;
-  for (int i = threadIdx.x; i < 2 * n_pairs; i += blockDim.x) out[i] = -1;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int k = 0;
-    for (int i = 0; i < NB; ++i)
-      if (rank[i] == consumer) out[k++] = i;  // pair c = entries 2c and 2c+1
-    if (blockIdx.x == 0) *active_per_bh = stacked ? (k + 1) / 2 : k;
-  }
-}
-
-// slot[bh][j] = entry index of block j inside the consumer's packed buffer (pack order: producer ascending,
-// head ascending, block ascending), for every block of the consumer's union that another rank owns.  One warp
-// per (batch, producer, head).  The table must have been filled with -1.  Also writes tile_base[b].
-__global__ void slot_kernel(const uint32_t* __restrict__ U, const int32_t* __restrict__ rank,
-                            const int64_t* __restrict__ seg_off, const int64_t* __restrict__ seg_total,
-                            const int64_t* __restrict__ dst_base, int B, int H, int NB, int Wd, int P, int consumer,
-                            int64_t tile_bytes, int32_t* __restrict__ slot, int64_t* __restrict__ tile_base,
-                            int32_t* __restrict__ work_counter) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *work_counter = 0;  // the attention kernel's work queue
-  const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (wid < B && lane == 0) {  // first tile of the consumer's buffer for batch item wid
-    const int64_t br = wid * P + consumer;
-    int64_t base;
-    if (dst_base) {
-      base = dst_base[br];
-    } else {
-      base = 0;
-      for (int64_t t = 0; t < br; ++t) base += seg_total[t] * 2 * tile_bytes;
-    }
-    tile_base[wid] = base / tile_bytes;
-  }
-  const int64_t n_seg = (int64_t)B * P * H;
-  if (wid >= n_seg) return;
-  const int h = (int)(wid % H);
-  const int prod = (int)((wid / H) % P);
-  const int bb = (int)(wid / ((int64_t)H * P));
-  if (prod == consumer) return;
-  const uint32_t* u = U + ((int64_t)(bb * P + consumer) * H + h) * Wd;
-  const int64_t first = seg_off[((int64_t)(bb * P + consumer) * P + prod) * H + h];
-  int32_t* out = slot + (int64_t)(bb * H + h) * NB;
-  int running = 0;
-  for (int w0 = 0; w0 < Wd; w0 += 32) {
-    const int w = w0 + lane;
-    uint32_t bits = 0;
-    if (w < Wd) {
-      uint32_t own = 0;
-      for (int t = 0; t < 32; ++t) {
-        const int j = w * 32 + t;
-        if (j < NB && rank[j] == prod) own |= 1u << t;
-      }
-      bits = u[w] & own;
-    }
-    const int mine = __popc(bits);
-    int incl = mine;
-#pragma unroll
-    for (int sft = 1; sft < 32; sft <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, sft);
-      if (lane >= sft) incl += v;
-    }
-    int pos = running + incl - mine;
-    while (bits) {
-      const int t = __ffs(bits) - 1;
-      bits &= bits - 1;
-      out[w * 32 + t] = (int32_t)(first + pos);
-      ++pos;
-    }
-    running += __shfl_sync(0xffffffffu, incl, 31);
-  }
-}
-
 int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, const void* V,
                        const uint32_t* mask, const int32_t* rank, int P, int consumer, const uint32_t* U,
                        const int64_t* seg_off, const int64_t* seg_total, const void* packed, int64_t capacity,
                        const int64_t* dst_base, float scale, void* O, float* lse, char* ws, const WsLayout& L,
                        cudaStream_t st) {
-  int32_t* pairs = (int32_t*)(ws + L.pairs);
-  int32_t* slot = (int32_t*)(ws + L.slot);
-  int64_t* tile_base = (int64_t*)(ws + L.tile_base);
-  const int64_t tile_bytes = (int64_t)g.b * g.d * 2;
-  SPARSP_CUDA_OK(cudaMemsetAsync(slot, 0xFF, (size_t)g.B * g.H * g.NB * 4, st));
-  int32_t* active = (int32_t*)(ws + L.status) + kWorkCounterWord + 1;
-  pair_rank_kernel<<<g.B * g.H, 128, 0, st>>>(rank, g.NB, consumer, g.b == 64 ? 1 : 0, pairs, active);
-  const int64_t n_warps = std::max<int64_t>((int64_t)g.B * P * g.H, g.B);
-  slot_kernel<<<(unsigned)((n_warps * 32 + 255) / 256), 256, 0, st>>>(U, rank, seg_off, seg_total, dst_base, g.B, g.H,
-                                                                    g.NB, g.Wd, P, consumer, tile_bytes, slot,
-                                                                    tile_base, (int32_t*)(ws + L.status) + kWorkCounterWord);
-  count_launch(2);
-  AttnParams p;
+  PrepParams pre = prep_params(s, g, K, mask, O, lse, ws, L);
+  pre.rank = rank;
+  pre.U = U;
+  pre.seg_off = seg_off;
+  pre.seg_total = seg_total;
+  pre.dst_base = dst_base;
+  pre.tile_bytes = (int64_t)g.b * g.d * 2;
+  pre.slot = (int32_t*)(ws + L.slot);
+  pre.tile_base = (int64_t*)(ws + L.tile_base);
+  pre.P = P;
+  pre.consumer = consumer;
+  const int rc = launch_prep<true>(g, pre, st);
+  if (rc != SPARSP_OK) return rc;
+  AttnParams p = {};
   p.mask = mask;
-  p.pairs = pairs;
-  p.slot = slot;
-  p.tile_base = tile_base;
-  p.active_per_bh = active;
-  p.knorm = nullptr;  // remote keys live in the packed buffer: every tile takes its row maximum
-  return launch_attn_common(s, g, Q, K, V, packed, capacity, p, scale, O, lse, ws, L, st);
+  p.pairs = pre.pairs;
+  p.n_items = pre.n_items;
+  p.slot = pre.slot;
+  p.tile_base = pre.tile_base;
+  return launch_attn_common<true>(s, g, Q, K, V, packed, capacity, p, scale, O, lse, ws, L, st);
 }
 
 }  // namespace sparsp
