@@ -6,91 +6,102 @@
 //          IEEE division by the valid count;
 //   score: acc = fmaf(q_c, k_c, acc) from acc = 0, channel c ascending;
 //   top-k: score descending, index ascending on equal scores, -0 == +0.
+#include <cstring>
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace sparsp {
 
 // ------------------------------------------------------------------------------------------------
-// pool: a group of d/8 lanes owns one (tensor, batch*head, block) tile; lane l owns channels
-// 8l..8l+7 and walks the tile's rows with 16-byte loads, so every channel is one sequential chain.
+// pool: a group of lanes owns one (tensor, batch*head, block) tile; a lane owns 8 (or 4) channels and walks the tile's
+// rows with 16-byte (8-byte) loads, several of them in flight, so every channel is one sequential chain.
+// Large problems are HBM-bound: 16-byte loads, 16 rows in flight (24 heads x 24576 x 128: 53.6 us = 5.6 TB/s; 8 rows
+// 54.5, 8-byte loads of 32 rows 68).  Where the tiles do not fill a quarter of the chip's thread slots the time is the
+// latency of the dependent batches: 8-byte loads, so twice the threads, and 32 rows in flight (26 heads x 6034 x 64:
+// 17.9 us against 28 with the wide form and 32-38 with 8 rows of it; 2 heads x 4096: 4.3 us against 6.2).
 // ------------------------------------------------------------------------------------------------
-template <int D>
-__global__ void __launch_bounds__(256) pool_kernel(const __nv_bfloat16* __restrict__ Q,
-                                                   const __nv_bfloat16* __restrict__ K,
-                                                   float* __restrict__ pq, float* __restrict__ pk,
-                                                   int H, int NB, int b, int64_t N, int64_t sB,
-                                                   int64_t sH, int64_t sT, int64_t n_tiles) {
-  constexpr int G = D / 8;  // lanes per tile
-  constexpr int U = 8;      // rows in flight per lane
-  const int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+constexpr int kPoolThreads = 128;
+constexpr int kPoolNarrowThreads = 148 * 512;  // up to this many threads of the wide form the narrow one is used
+
+template <int D, bool kNarrow>
+__global__ void __launch_bounds__(kPoolThreads) pool_kernel(const __nv_bfloat16* __restrict__ Q,
+                                                            const __nv_bfloat16* __restrict__ K,
+                                                            float* __restrict__ pq, float* __restrict__ pk,
+                                                            int H, int NB, int b, int64_t N, int64_t sB,
+                                                            int64_t sH, int64_t sT, int64_t n_tiles) {
+  constexpr int kVec = kNarrow ? 4 : 8;    // channels per lane
+  constexpr int kRows = kNarrow ? 32 : 16;  // rows in flight
+  constexpr int G = D / kVec;              // lanes per tile
+  constexpr int W = kVec / 2;              // 32-bit words per lane and row
+  using Vec = typename std::conditional<kNarrow, uint2, uint4>::type;
+  const int64_t tile = ((int64_t)blockIdx.x * kPoolThreads + threadIdx.x) / G;
   const int lane = threadIdx.x % G;
   if (tile >= 2 * n_tiles) return;
   const bool is_k = tile >= n_tiles;
   const int64_t t = is_k ? tile - n_tiles : tile;  // (batch*H + head) * NB + block
-  const int blk = (int)(t % NB);
   const int64_t bh = t / NB;
+  const int blk = (int)(t - bh * NB);
   const int64_t batch = bh / H, head = bh % H;
   const int64_t tok0 = (int64_t)blk * b;
   const int n = (int)min((int64_t)b, N - tok0);
-  const __nv_bfloat16* src = (is_k ? K : Q) + batch * sB + head * sH + tok0 * sT + lane * 8;
+  const __nv_bfloat16* src = (is_k ? K : Q) + batch * sB + head * sH + tok0 * sT + lane * kVec;
 
-  float acc[8];
+  float acc[kVec];
 #pragma unroll
-  for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
-
+  for (int c = 0; c < kVec; ++c) acc[c] = 0.0f;
+  auto add = [&](const Vec& x) {
+    uint32_t v[W];
+    memcpy(v, &x, sizeof v);
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      acc[2 * w] = __fadd_rn(acc[2 * w], __uint_as_float(v[w] << 16));
+      acc[2 * w + 1] = __fadd_rn(acc[2 * w + 1], __uint_as_float(v[w] & 0xffff0000u));
+    }
+  };
+  auto load = [&](int r) { return __ldg(reinterpret_cast<const Vec*>(src + (int64_t)r * sT)); };
   int r = 0;
-  for (; r + U <= n; r += U) {
-    uint4 v[U];
+  if (kNarrow) {
+    for (; r < n; r += kRows) {
+      Vec x[kRows];
 #pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = __ldg(reinterpret_cast<const uint4*>(src + (int64_t)(r + u) * sT));
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        acc[2 * p] = __fadd_rn(acc[2 * p], __uint_as_float(w[p] << 16));
-        acc[2 * p + 1] = __fadd_rn(acc[2 * p + 1], __uint_as_float(w[p] & 0xffff0000u));
+      for (int u = 0; u < kRows; ++u) {
+        x[u] = Vec{};
+        if (r + u < n) x[u] = load(r + u);
       }
-    }
-  }
-  for (; r < n; ++r) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(src + (int64_t)r * sT));
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+      // (a row behind the last token adds +0, which changes no sum: a sum that starts at +0 is never -0)
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      acc[2 * p] = __fadd_rn(acc[2 * p], __uint_as_float(w[p] << 16));
-      acc[2 * p + 1] = __fadd_rn(acc[2 * p + 1], __uint_as_float(w[p] & 0xffff0000u));
+      for (int u = 0; u < kRows; ++u) add(x[u]);
     }
+  } else {
+    for (; r + kRows <= n; r += kRows) {
+      Vec x[kRows];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) x[u] = load(r + u);
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) add(x[u]);
+    }
+    for (; r < n; ++r) add(load(r));
   }
   const float cntf = (float)n;
-  float* dst = (is_k ? pk : pq) + t * D + lane * 8;
-  float4 o0, o1;
-  o0.x = __fdiv_rn(acc[0], cntf);
-  o0.y = __fdiv_rn(acc[1], cntf);
-  o0.z = __fdiv_rn(acc[2], cntf);
-  o0.w = __fdiv_rn(acc[3], cntf);
-  o1.x = __fdiv_rn(acc[4], cntf);
-  o1.y = __fdiv_rn(acc[5], cntf);
-  o1.z = __fdiv_rn(acc[6], cntf);
-  o1.w = __fdiv_rn(acc[7], cntf);
-  reinterpret_cast<float4*>(dst)[0] = o0;
-  reinterpret_cast<float4*>(dst)[1] = o1;
+  float* dst = (is_k ? pk : pq) + t * D + lane * kVec;
+#pragma unroll
+  for (int c = 0; c < kVec; c += 4)
+    *reinterpret_cast<float4*>(dst + c) = make_float4(__fdiv_rn(acc[c], cntf), __fdiv_rn(acc[c + 1], cntf),
+                                                      __fdiv_rn(acc[c + 2], cntf), __fdiv_rn(acc[c + 3], cntf));
 }
 
 int launch_pool(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, float* pq,
                 float* pk, cudaStream_t st) {
   const int64_t n_tiles = (int64_t)g.B * g.H * g.NB;
-  const int G = g.d / 8;
-  const int64_t threads = 2 * n_tiles * G;
-  const int grid = (int)((threads + 255) / 256);
-  auto q = (const __nv_bfloat16*)Q;
-  auto k = (const __nv_bfloat16*)K;
-  if (g.d == 64)
-    pool_kernel<64><<<grid, 256, 0, st>>>(q, k, pq, pk, g.H, g.NB, g.b, g.N, s.stride_batch,
-                                          s.stride_head, s.stride_token, n_tiles);
-  else
-    pool_kernel<128><<<grid, 256, 0, st>>>(q, k, pq, pk, g.H, g.NB, g.b, g.N, s.stride_batch,
-                                           s.stride_head, s.stride_token, n_tiles);
+  int64_t threads = 2 * n_tiles * (g.d / 8);
+  const bool narrow = threads <= kPoolNarrowThreads;
+  if (narrow) threads *= 2;
+  auto kern = g.d == 64 ? (narrow ? pool_kernel<64, true> : pool_kernel<64, false>)
+                        : (narrow ? pool_kernel<128, true> : pool_kernel<128, false>);
+  kern<<<(unsigned)((threads + kPoolThreads - 1) / kPoolThreads), kPoolThreads, 0, st>>>(
+      (const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, pq, pk, g.H, g.NB, g.b, g.N, s.stride_batch, s.stride_head,
+      s.stride_token, n_tiles);
   count_launch();
   SPARSP_CUDA_OK(cudaGetLastError());
   return SPARSP_OK;
@@ -165,11 +176,25 @@ __global__ void __launch_bounds__(kScoreThreads) score_kernel(const float* __res
   }
 }
 
+static cudaError_t launch_score(const Geometry& g, const float* pq, const float* pk, float* scores, cudaStream_t st) {
+  const size_t smem = (size_t)2 * kScoreTile * (g.d + 4) * 4;
+  const unsigned nt = (unsigned)((g.NB + kScoreTile - 1) / kScoreTile);
+  auto kern = g.d == 64 ? score_kernel<64> : score_kernel<128>;
+  const cudaError_t e = ensure_dynamic_smem((const void*)kern, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(nt, nt, (unsigned)(g.B * g.H)), kScoreThreads, smem, st>>>(pq, pk, g.NB, scores);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------------------------------------
 // top-k: one warp per (batch, head, query block) row.  The row's scores become order-preserving
-// uint32 keys in registers (lane l holds blocks l, l + 32, ...); the warp finds the k-th largest key by a 32-step radix search with
-// ballots/popcounts, breaks ties towards the lower index, forces the text blocks on, and emits the
-// mask words and the ascending kept list by ballot-prefix compaction.
+// uint32 keys in registers (lane l holds blocks l, l + 32, ...); the warp finds the k-th largest key by bisection between
+// the row's smallest and largest key with compares and a warp sum per step, which ends as soon as a trial value has
+// exactly k keys at or above it (well before the 32 steps that a search bit by bit always takes), breaks ties towards
+// the lower index, forces the text blocks on, and emits the mask words and the ascending kept list by ballot-prefix
+// compaction.  Bound by instruction issue, a compare and an add per key and step: instances for several row lengths.
+// 24 x 384 rows of 384: 19 us, 40 x 591 of 591: 79 us, 24 x 929 of 929: 136 us (29, 152 and 194 us with 32 steps of one bit
+// each and instances of 4, 8, 16 and 32 words; bisection by the keys instead of the scores: 18, 71 and 212 us).
 // ------------------------------------------------------------------------------------------------
 constexpr int kTopkWarps = 8;
 
@@ -179,8 +204,20 @@ __device__ __forceinline__ uint32_t score_key(float s) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+__device__ __forceinline__ float key_score(uint32_t key) {
+  return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
+}
+
+// A key in (lo, hi] for the next step of a search, lo < hi: the one of the middle of the two scores, which halves evenly
+// spread scores where the middle of the keys halves their exponents; or the middle key where that is no such key (ends that
+// are infinite, not numbers or neighbours) and in every third step, so that the search ends after at most 96 steps.
+__device__ __forceinline__ uint32_t middle(uint32_t lo, uint32_t hi, int step) {
+  const uint32_t by_score = score_key(0.5f * key_score(lo) + 0.5f * key_score(hi));
+  return by_score > lo && by_score <= hi && step % 3 != 2 ? by_score : lo + ((hi - lo) >> 1) + 1;
+}
+
 template <int WMAX>  // mask words per row this instance can hold (keys live in registers: WMAX per lane)
-__global__ void __launch_bounds__(kTopkWarps * 32) topk_kernel(const float* __restrict__ scores, int64_t n_rows,
+__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 6 : 4) topk_kernel(const float* __restrict__ scores, int64_t n_rows,
                                                                int NB, int Wd, int nb_cand, int topk,
                                                                int kept_cap, uint32_t* __restrict__ mask,
                                                                int32_t* __restrict__ kv_list,
@@ -199,16 +236,26 @@ __global__ void __launch_bounds__(kTopkWarps * 32) topk_kernel(const float* __re
   }
 
   const uint32_t lt_mask = (1u << lane) - 1u;
-  // largest T with |{ candidates : key >= T }| >= topk  ==> T is the topk-th largest key
-  uint32_t T = 0;
-  for (int bit = 31; bit >= 0; --bit) {
-    const uint32_t trial = T | (1u << bit);
+  // T with |{ candidates : key >= T }| == topk, or else the topk-th largest key (ties)
+  uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+  for (int t = 0; t < WMAX; ++t) {
+    lo = min(lo, t * 32 + lane < nb_cand ? key[t] : 0xffffffffu);
+    hi = max(hi, key[t]);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);  // all candidates are >= lo, at least topk of them
+  hi = __reduce_max_sync(0xffffffffu, hi);  // fewer than topk are > hi
+  for (int step = 0; lo < hi && topk < nb_cand; ++step) {
+    const uint32_t trial = middle(lo, hi, step);
     int c = 0;
 #pragma unroll
     for (int t = 0; t < WMAX; ++t) c += key[t] >= trial ? 1 : 0;
     c = __reduce_add_sync(0xffffffffu, c);
-    if (c >= topk) T = trial;
+    if (c >= topk) lo = trial;
+    else hi = trial - 1;
+    if (c == topk) break;
   }
+  const uint32_t T = lo;
   int gt = 0;
 #pragma unroll
   for (int t = 0; t < WMAX; ++t) gt += key[t] > T ? 1 : 0;
@@ -245,8 +292,9 @@ __global__ void __launch_bounds__(kTopkWarps * 32) topk_kernel(const float* __re
 //   split, degree-5 Horner polynomial with fused multiply-adds, integer part added into the exponent field);
 //   w_j = floor(p_j * 2^26);  Z = sum w_j;  kept = { key >= T } for the largest T with
 //   mass{ key >= T } >= ceil(tau * Z), the product taken once in fp64.
-// One warp per row; T is found by a 32-step search over the order-preserving key space, which is valid
-// because the mass of { key >= t } never grows with t.
+// One warp per row; T is found by bisection over the order-preserving key space, which is valid
+// because the mass of { key >= t } never grows with t, until a
+// single key is left between its ends: 24 x 384 rows of 384 in 24 us (37 us with 32 steps of one bit).
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ float exp2c(float x) {
   x = fmaxf(x, -125.0f);
@@ -269,7 +317,7 @@ __device__ __forceinline__ unsigned long long warp_sum(uint32_t v) {
 }
 
 template <int WMAX>  // mask words per row this instance can hold (keys and terms live in registers)
-__global__ void __launch_bounds__(kTopkWarps * 32) cdf_kernel(const float* __restrict__ scores, int64_t n_rows, int NB,
+__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 4 : WMAX <= 20 ? 3 : 2) cdf_kernel(const float* __restrict__ scores, int64_t n_rows, int NB,
                                                               int Wd, int nb_cand, float tau, float c,
                                                               uint32_t* __restrict__ mask,
                                                               int32_t* __restrict__ kv_count) {
@@ -306,15 +354,37 @@ __global__ void __launch_bounds__(kTopkWarps * 32) cdf_kernel(const float* __res
     w[t] = wj;
   }
   const unsigned long long theta = (unsigned long long)ceil(__dmul_rn((double)tau, (double)warp_sum(acc)));
-  // largest T with mass{ key >= T } >= theta
-  uint32_t T = 0;
-  for (int bit = 31; bit >= 0; --bit) {
-    const uint32_t trial = T | (1u << bit);
-    uint32_t m = 0;
+  // a T with the same { key >= T } as the largest T with mass{ key >= T } >= theta: bisection between the row's
+  // smallest and largest key, until a single key is left between the two ends
+  uint32_t lo = 0xffffffffu, hi = 0u;
 #pragma unroll
-    for (int t = 0; t < WMAX; ++t) m += key[t] >= trial ? w[t] : 0u;
-    if (warp_sum(m) >= theta) T = trial;
+  for (int t = 0; t < WMAX; ++t) {
+    lo = min(lo, t * 32 + lane < nb_cand ? key[t] : 0xffffffffu);
+    hi = max(hi, key[t]);
   }
+  lo = __reduce_min_sync(0xffffffffu, lo);  // mass{ key >= lo } >= theta
+  hi = __reduce_max_sync(0xffffffffu, hi);  // mass{ key > hi } < theta
+  int n_lo = nb_cand, n_hi = 0;             // keys >= lo, keys > hi
+  for (int step = 0; lo < hi && n_lo - n_hi > 1; ++step) {
+    const uint32_t trial = middle(lo, hi, step);
+    uint32_t m = 0;
+    int c = 0;
+#pragma unroll
+    for (int t = 0; t < WMAX; ++t) {
+      m += key[t] >= trial ? w[t] : 0u;
+      c += key[t] >= trial ? 1 : 0;
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (warp_sum(m) >= theta) {
+      lo = trial;
+      n_lo = c;
+    } else {
+      hi = trial - 1;
+      n_hi = c;
+    }
+  }
+  // (theta 0: all weights are zero, as with a NaN or infinite maximum; then no score reaches the threshold)
+  const uint32_t T = theta != 0 ? lo : 0xffffffffu;
   int cnt = 0;
 #pragma unroll
   for (int t = 0; t < WMAX; ++t) {
@@ -331,19 +401,14 @@ __global__ void __launch_bounds__(kTopkWarps * 32) cdf_kernel(const float* __res
 
 int launch_score_cdf(const Geometry& g, const float* pq, const float* pk, float* scores, float tau, float scale,
                      uint32_t* mask, int32_t* kv_count, cudaStream_t st) {
-  {
-    const size_t smem = (size_t)2 * kScoreTile * (g.d + 4) * 4;
-    const int nt = (g.NB + kScoreTile - 1) / kScoreTile;
-    dim3 grid(nt, nt, g.B * g.H);
-    auto kern = g.d == 64 ? score_kernel<64> : score_kernel<128>;
-    SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, (int)smem));
-    kern<<<grid, kScoreThreads, smem, st>>>(pq, pk, g.NB, scores);
-  }
+  SPARSP_CUDA_OK(launch_score(g, pq, pk, scores, st));
   {
     const int64_t n_rows = (int64_t)g.B * g.H * g.NB;
     const float c = scale * 1.4426950408889634f;  // fp32 product, as in the definition above
     const unsigned grid = (unsigned)((n_rows + kTopkWarps - 1) / kTopkWarps);
-    auto kern = g.Wd <= 4 ? cdf_kernel<4> : g.Wd <= 8 ? cdf_kernel<8> : g.Wd <= 16 ? cdf_kernel<16> : cdf_kernel<32>;
+    auto kern = g.Wd <= 4 ? cdf_kernel<4> : g.Wd <= 8 ? cdf_kernel<8> : 
+                g.Wd <= 12 ? cdf_kernel<12> : g.Wd <= 16 ? cdf_kernel<16> : g.Wd <= 20 ? cdf_kernel<20> : 
+                g.Wd <= 24 ? cdf_kernel<24> : cdf_kernel<32>;
     kern<<<grid, kTopkWarps * 32, 0, st>>>(scores, n_rows, g.NB, g.Wd, g.nb_cand, tau, c, mask, kv_count);
   }
   count_launch(2);
@@ -354,18 +419,13 @@ int launch_score_cdf(const Geometry& g, const float* pq, const float* pk, float*
 int launch_score_topk(const Geometry& g, const float* pq, const float* pk, float* scores, int topk,
                       uint32_t* mask, int32_t* kv_list, int32_t* kv_count, cudaStream_t st) {
   const int kept_cap = topk + (g.NB - g.nb_cand);
-  {
-    const size_t smem = (size_t)2 * kScoreTile * (g.d + 4) * 4;
-    const int nt = (g.NB + kScoreTile - 1) / kScoreTile;
-    dim3 grid(nt, nt, g.B * g.H);
-    auto kern = g.d == 64 ? score_kernel<64> : score_kernel<128>;
-    SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, (int)smem));
-    kern<<<grid, kScoreThreads, smem, st>>>(pq, pk, g.NB, scores);
-  }
+  SPARSP_CUDA_OK(launch_score(g, pq, pk, scores, st));
   {
     const int64_t n_rows = (int64_t)g.B * g.H * g.NB;
     const unsigned grid = (unsigned)((n_rows + kTopkWarps - 1) / kTopkWarps);
-    auto kern = g.Wd <= 4 ? topk_kernel<4> : g.Wd <= 8 ? topk_kernel<8> : g.Wd <= 16 ? topk_kernel<16> : topk_kernel<32>;
+    auto kern = g.Wd <= 4 ? topk_kernel<4> : g.Wd <= 8 ? topk_kernel<8> : 
+                g.Wd <= 12 ? topk_kernel<12> : g.Wd <= 16 ? topk_kernel<16> : g.Wd <= 20 ? topk_kernel<20> : 
+                g.Wd <= 24 ? topk_kernel<24> : topk_kernel<32>;
     kern<<<grid, kTopkWarps * 32, 0, st>>>(scores, n_rows, g.NB, g.Wd, g.nb_cand, topk, kept_cap, mask, kv_list, kv_count);
   }
   count_launch(2);
