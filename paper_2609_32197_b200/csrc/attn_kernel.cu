@@ -285,6 +285,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     tmem_alloc(s_tmem, kTmemCols);
     tmem_relinquish();
   }
+  enter_grid();  // (barriers, tensor memory and constants are set up while the preparatory launch still runs)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1252,6 +1253,7 @@ __device__ __forceinline__ float block_norm(const PrepParams& p, int64_t bh, int
 
 template <int D, bool kPacked>
 __global__ void __launch_bounds__(kPrepThreads) attn_prep_kernel(const PrepParams p) {
+  enter_grid();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (blockIdx.x == 0 && threadIdx.x == 0) *p.work_counter = 0;  // the attention kernel's work queue
@@ -1399,9 +1401,7 @@ static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q
   SPARSP_CUDA_OK(cudaGetDevice(&dev));
   SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const unsigned grid = (unsigned)std::min<int64_t>(most, sms);
-  kern<<<grid, kAttnThreads, smem, st>>>(tq, tk, tv, tp, p);
-  count_launch();
-  SPARSP_CUDA_OK(cudaGetLastError());
+  SPARSP_CUDA_OK(launch_kernel(kern, grid, kAttnThreads, smem, st, tq, tk, tv, tp, p));
   return SPARSP_OK;
 }
 
@@ -1437,9 +1437,7 @@ static int launch_prep(const Geometry& g, const PrepParams& p, cudaStream_t st) 
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
   constexpr int kWarps = kPrepThreads / 32;
   const int64_t blocks = p.BH + ((int64_t)p.BH * g.NB + kWarps - 1) / kWarps;
-  kern<<<(unsigned)blocks, kPrepThreads, smem, st>>>(p);
-  count_launch();
-  SPARSP_CUDA_OK(cudaGetLastError());
+  SPARSP_CUDA_OK(launch_kernel(kern, (unsigned)blocks, kPrepThreads, smem, st, p));
   return SPARSP_OK;
 }
 

@@ -44,6 +44,43 @@ WsLayout make_layout(const Geometry& g, int n_ranks);
 // what was set per (kernel, device) so that the driver call is made only when the limit must grow.
 cudaError_t ensure_dynamic_smem(const void* func, int bytes);
 
+// Launches a kernel that may start while the launches before it in the stream still run (programmatic stream
+// serialisation): its CTAs take their places and set themselves up as soon as the previous kernel's have all started, and
+// wait in enter_grid() before they touch memory, so that the latency of a launch is hidden behind the kernel before it.
+// Every kernel launched here calls enter_grid() first thing, in every thread.
+template <typename T>
+struct same_type {
+  using type = T;
+};
+template <typename... P>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                 typename same_type<P>::type... args) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+#ifdef __CUDACC__
+// First statement of a kernel started by launch_kernel: lets the next launch begin, then waits until all work before this
+// launch has completed.  No thread returns or touches global memory before it.  Pointers that the compiler
+// may take for read-only are passed through it, so that no load through them can be moved ahead of the wait.
+template <typename... P>
+__device__ __forceinline__ void enter_grid(P&... pointers) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  ((void)([](auto& p) { asm volatile("" : "+l"(p)::"memory"); }(pointers)), ...);
+}
+#endif
+
 inline int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 #define SPARSP_CUDA_OK(call)                              \

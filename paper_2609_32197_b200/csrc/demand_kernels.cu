@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
                                                                     int Wd, int P, uint32_t* __restrict__ U,
                                                                     int32_t* __restrict__ cnt,
                                                                     int32_t* __restrict__ n_src) {
+  enter_grid(mask, rank);
   __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
   __shared__ uint32_t u_s[kMaxWords];
   __shared__ uint16_t rows_s[kMaxBlocks];
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(
     int64_t* __restrict__ seg_total, int64_t* __restrict__ volume, const int64_t* __restrict__ dst_base,
     int64_t capacity, int64_t* __restrict__ dst, int32_t* __restrict__ src, int32_t* __restrict__ n_src,
     int32_t* __restrict__ status) {
+  enter_grid(cnt, U, rank, dst_base);
   __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
   __shared__ int64_t seg_s[kMaxRanks];  // first entry of (producer, my head)
   __shared__ int64_t warp_s[kPlanThreads / 32];
@@ -194,16 +196,17 @@ static int32_t* src_list(char* ws, const WsLayout& L, const Geometry& g, int n_d
   return (int32_t*)(ws + L.entries + (int64_t)g.B * g.H * g.NB * n_dst * 8);
 }
 
-static void launch_plan(const Geometry& g, const uint32_t* mask, const int32_t* rank, int P, int include_local,
+static cudaError_t launch_plan(const Geometry& g, const uint32_t* mask, const int32_t* rank, int P, int include_local,
                         uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total, int64_t* volume,
                         const int64_t* dst_base, int64_t capacity, int64_t* dst, int32_t* src, int32_t* n_src,
                         int32_t* status, cudaStream_t st) {
-  union_count_kernel<<<g.B * g.H * P, kUnionThreads, 0, st>>>(mask, rank, g.H, g.NB, g.Wd, P, U, cnt, n_src);
+  cudaError_t e = launch_kernel(union_count_kernel, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P, U,
+                                cnt, n_src);
+  if (e != cudaSuccess) return e;
   const unsigned grid = dst ? (unsigned)((g.B * P + g.B) * g.H) : (unsigned)(g.B * P);
-  plan_kernel<<<grid, kPlanThreads, 0, st>>>(cnt, U, rank, g.B * P, g.H, g.NB, g.Wd, P, include_local,
+  return launch_kernel(plan_kernel, grid, kPlanThreads, 0, st, cnt, U, rank, g.B * P, g.H, g.NB, g.Wd, P, include_local,
                                              2LL * g.b * g.d * 2, seg_off, seg_total, volume, dst_base, capacity, dst,
                                              src, n_src, status);
-  count_launch(2);
 }
 
 int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_of_block, int P,
@@ -215,10 +218,9 @@ int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_o
     set_error("batch * n_ranks = %d exceeds 1024", g.B * P);
     return SPARSP_ERR_UNSUPPORTED;
   }
-  launch_plan(g, mask, rank_of_block, P, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, U, cnt, seg_off, seg_total, volume,
+  SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, P, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, U, cnt, seg_off, seg_total, volume,
               dst_base, capacity, pack ? dst_table(ws, L) : nullptr, pack ? src_list(ws, L, g, P) : nullptr,
-              pack ? (int32_t*)(ws + L.n_entries) : nullptr, (int32_t*)(ws + L.status), st);
-  SPARSP_CUDA_OK(cudaGetLastError());
+              pack ? (int32_t*)(ws + L.n_entries) : nullptr, (int32_t*)(ws + L.status), st));
   return SPARSP_OK;
 }
 
@@ -259,14 +261,15 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps) pack_kernel(const __grid_c
   uint64_t* full = full_all + warp * kPackStages;
   unsigned char* ring = smem_raw + (size_t)warp * kPackStages * tile_bytes;  // this warp's buffers
   const int unit = blockIdx.x * n_warps + warp, n_units = gridDim.x * n_warps;
-  const int64_t n_items = 2 * (int64_t)*n_src;  // item: K (even) or V (odd) tile of source item / 2
-  const int n_local = (int)(n_items > unit ? (n_items - unit + n_units - 1) / n_units : 0);
   if (threadIdx.x == 0) s_abort = 0;
   if (lane == 0) {
     for (int st = 0; st < kPackStages; ++st) ptx::mbar_init(full + st, 1);
     ptx::mbar_init_fence();
   }
+  enter_grid(dst, src, n_src);
   __syncthreads();
+  const int64_t n_items = 2 * (int64_t)*n_src;  // item: K (even) or V (odd) tile of source item / 2
+  const int n_local = (int)(n_items > unit ? (n_items - unit + n_units - 1) / n_units : 0);
 
   // lane l: the source of local item q + l
   auto sources = [&](int q) -> int {
@@ -334,10 +337,8 @@ static int run_pack(const sparsp_shape& s, const Geometry& g, const void* K, con
   const int n_warps = std::max(1, std::min(kPackMaxWarps, (32 * 1024) / tile_bytes));
   const int smem = n_warps * kPackStages * tile_bytes;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)pack_kernel, smem));
-  pack_kernel<<<sms, 32 * n_warps, smem, st>>>(tk, tv, dst, n_dst, src, n_src, g.H, g.NB, g.b, (uint32_t)tile_bytes,
-                                               (unsigned char*)packed, status);
-  count_launch();
-  SPARSP_CUDA_OK(cudaGetLastError());
+  SPARSP_CUDA_OK(launch_kernel(pack_kernel, sms, 32 * n_warps, smem, st, tk, tv, dst, n_dst, src, n_src, g.H, g.NB, g.b, (uint32_t)tile_bytes,
+                                               (unsigned char*)packed, status));
   return SPARSP_OK;
 }
 
@@ -361,6 +362,7 @@ __global__ void __launch_bounds__(256) segment_kernel(const uint32_t* __restrict
                                                       int64_t capacity, int64_t* __restrict__ dst,
                                                       int32_t* __restrict__ src, int32_t* __restrict__ n_src,
                                                       int32_t* __restrict__ status) {
+  enter_grid(U, rank, seg_off, cnt);
   __shared__ uint32_t own_s[kMaxWords];
   const int h = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
@@ -389,10 +391,8 @@ int launch_pack_segment(const sparsp_shape& s, const Geometry& g, const uint32_t
   int32_t* src = src_list(ws, L, g, 1);
   int32_t* n_src = (int32_t*)(ws + L.n_entries);
   int32_t* status = (int32_t*)(ws + L.status);
-  segment_kernel<<<(g.H * 32 + 255) / 256, 256, 0, st>>>(U, rank, g.H, g.NB, g.Wd, P, consumer, producer, seg_off, cnt,
-                                                        2LL * g.b * g.d * 2, capacity, table, src, n_src, status);
-  count_launch();
-  SPARSP_CUDA_OK(cudaGetLastError());
+  SPARSP_CUDA_OK(launch_kernel(segment_kernel, (g.H * 32 + 255) / 256, 256, 0, st, U, rank, g.H, g.NB, g.Wd, P, consumer, producer, seg_off, cnt,
+                                                        2LL * g.b * g.d * 2, capacity, table, src, n_src, status));
   return run_pack(s, g, K, V, table, 1, src, n_src, dst, status, st);
 }
 
@@ -433,8 +433,7 @@ extern "C" SPARSP_API int sparsp_demand_plan_noalloc(const sparsp_shape* shape, 
     set_error("sparsp_demand_plan_noalloc: misaligned argument");
     return SPARSP_ERR_INVALID_ARG;
   }
-  launch_plan(g, mask, rank_of_block, n_ranks, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, union_mask, cnt, seg_offset,
-              seg_total, volume_bytes, nullptr, -1, nullptr, nullptr, nullptr, nullptr, (cudaStream_t)stream);
-  SPARSP_CUDA_OK(cudaGetLastError());
+  SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, n_ranks, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, union_mask, cnt, seg_offset,
+              seg_total, volume_bytes, nullptr, -1, nullptr, nullptr, nullptr, nullptr, (cudaStream_t)stream));
   return SPARSP_OK;
 }

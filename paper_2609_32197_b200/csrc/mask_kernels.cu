@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(kPoolThreads) pool_kernel(const __nv_bfloat16*
                                                             float* __restrict__ pq, float* __restrict__ pk,
                                                             int H, int NB, int b, int64_t N, int64_t sB,
                                                             int64_t sH, int64_t sT, int64_t n_tiles) {
+  enter_grid(Q, K);
   constexpr int kVec = kNarrow ? 4 : 8;    // channels per lane
   constexpr int kRows = kNarrow ? 32 : 16;  // rows in flight
   constexpr int G = D / kVec;              // lanes per tile
@@ -99,11 +100,9 @@ int launch_pool(const sparsp_shape& s, const Geometry& g, const void* Q, const v
   if (narrow) threads *= 2;
   auto kern = g.d == 64 ? (narrow ? pool_kernel<64, true> : pool_kernel<64, false>)
                         : (narrow ? pool_kernel<128, true> : pool_kernel<128, false>);
-  kern<<<(unsigned)((threads + kPoolThreads - 1) / kPoolThreads), kPoolThreads, 0, st>>>(
-      (const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, pq, pk, g.H, g.NB, g.b, g.N, s.stride_batch, s.stride_head,
-      s.stride_token, n_tiles);
-  count_launch();
-  SPARSP_CUDA_OK(cudaGetLastError());
+  SPARSP_CUDA_OK(launch_kernel(kern, (unsigned)((threads + kPoolThreads - 1) / kPoolThreads), kPoolThreads, 0, st,
+                               (const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, pq, pk, g.H, g.NB, g.b, g.N,
+                               s.stride_batch, s.stride_head, s.stride_token, n_tiles));
   return SPARSP_OK;
 }
 
@@ -121,6 +120,7 @@ template <int D>
 __global__ void __launch_bounds__(kScoreThreads) score_kernel(const float* __restrict__ pq,
                                                               const float* __restrict__ pk, int NB,
                                                               float* __restrict__ scores) {
+  enter_grid(pq, pk);
   constexpr int LD = D + 4;  // row pitch in floats: 16 bytes of skew per row
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* sQ = reinterpret_cast<float*>(smem_raw);  // [64][LD]
@@ -182,8 +182,7 @@ static cudaError_t launch_score(const Geometry& g, const float* pq, const float*
   auto kern = g.d == 64 ? score_kernel<64> : score_kernel<128>;
   const cudaError_t e = ensure_dynamic_smem((const void*)kern, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(nt, nt, (unsigned)(g.B * g.H)), kScoreThreads, smem, st>>>(pq, pk, g.NB, scores);
-  return cudaGetLastError();
+  return launch_kernel(kern, dim3(nt, nt, (unsigned)(g.B * g.H)), kScoreThreads, smem, st, pq, pk, g.NB, scores);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -222,6 +221,7 @@ __global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 6 : 4) topk_kern
                                                                int kept_cap, uint32_t* __restrict__ mask,
                                                                int32_t* __restrict__ kv_list,
                                                                int32_t* __restrict__ kv_count) {
+  enter_grid(scores);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * kTopkWarps + warp;  // (batch*H + head) * NB + i
   if (row >= n_rows) return;
@@ -321,6 +321,7 @@ __global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 4 : WMAX <= 20 ?
                                                               int Wd, int nb_cand, float tau, float c,
                                                               uint32_t* __restrict__ mask,
                                                               int32_t* __restrict__ kv_count) {
+  enter_grid(scores);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * kTopkWarps + warp;  // (batch*H + head) * NB + i
   if (row >= n_rows) return;
@@ -409,10 +410,8 @@ int launch_score_cdf(const Geometry& g, const float* pq, const float* pk, float*
     auto kern = g.Wd <= 4 ? cdf_kernel<4> : g.Wd <= 8 ? cdf_kernel<8> : 
                 g.Wd <= 12 ? cdf_kernel<12> : g.Wd <= 16 ? cdf_kernel<16> : g.Wd <= 20 ? cdf_kernel<20> : 
                 g.Wd <= 24 ? cdf_kernel<24> : cdf_kernel<32>;
-    kern<<<grid, kTopkWarps * 32, 0, st>>>(scores, n_rows, g.NB, g.Wd, g.nb_cand, tau, c, mask, kv_count);
+    SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, g.NB, g.Wd, g.nb_cand, tau, c, mask, kv_count));
   }
-  count_launch(2);
-  SPARSP_CUDA_OK(cudaGetLastError());
   return SPARSP_OK;
 }
 
@@ -426,10 +425,8 @@ int launch_score_topk(const Geometry& g, const float* pq, const float* pk, float
     auto kern = g.Wd <= 4 ? topk_kernel<4> : g.Wd <= 8 ? topk_kernel<8> : 
                 g.Wd <= 12 ? topk_kernel<12> : g.Wd <= 16 ? topk_kernel<16> : g.Wd <= 20 ? topk_kernel<20> : 
                 g.Wd <= 24 ? topk_kernel<24> : topk_kernel<32>;
-    kern<<<grid, kTopkWarps * 32, 0, st>>>(scores, n_rows, g.NB, g.Wd, g.nb_cand, topk, kept_cap, mask, kv_list, kv_count);
+    SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, g.NB, g.Wd, g.nb_cand, topk, kept_cap, mask, kv_list, kv_count));
   }
-  count_launch(2);
-  SPARSP_CUDA_OK(cudaGetLastError());
   return SPARSP_OK;
 }
 

@@ -20,6 +20,7 @@ __global__ void __launch_bounds__(kHopThreads) hop_mask_kernel(const uint32_t* _
                                                                int64_t n_rows, int consumer, int producer,
                                                                int head_begin, int head_end,
                                                                uint32_t* __restrict__ hop) {
+  enter_grid(mask, rank);
   __shared__ uint32_t own_s[kMaxWords], row_s[kMaxWords];
   rank_words(rank, NB, producer, own_s);
   rank_words(rank, NB, consumer, row_s);
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __nv_bf
                                                                    int64_t N, int b, int64_t sB, int64_t sH, int64_t sT,
                                                                    const int32_t* __restrict__ rank, int consumer,
                                                                    int head_begin, int head_end) {
+  enter_grid(rank);
   constexpr int VPR = D / 8;
   constexpr int kPass = kMergeThreads / VPR;  // rows per pass of the CTA
   __shared__ uint32_t words_s[kMaxWords];
@@ -148,10 +150,8 @@ int launch_hop_mask(const Geometry& g, const uint32_t* mask, const int32_t* rank
   int width = 1;
   while (width < g.Wd) width <<= 1;
   const int per_cta = kHopThreads / width * kHopRows;
-  hop_mask_kernel<<<(unsigned)((n_rows + per_cta - 1) / per_cta), kHopThreads, 0, st>>>(
-      mask, rank, g.H, g.NB, g.Wd, n_rows, consumer, producer, head_begin, head_end, hop);
-  count_launch();
-  SPARSP_CUDA_OK(cudaGetLastError());
+  SPARSP_CUDA_OK(launch_kernel(hop_mask_kernel, (unsigned)((n_rows + per_cta - 1) / per_cta), kHopThreads, 0, st, 
+      mask, rank, g.H, g.NB, g.Wd, n_rows, consumer, producer, head_begin, head_end, hop));
   return SPARSP_OK;
 }
 
@@ -164,11 +164,9 @@ int launch_attn_merge(const sparsp_shape& s, const Geometry& g, const void* Oa, 
   SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const unsigned grid = (unsigned)std::min<int64_t>((int64_t)g.B * (head_end - head_begin) * g.NB, 4LL * sms);
   auto kern = g.d == 64 ? attn_merge_kernel<64> : attn_merge_kernel<128>;
-  kern<<<grid, kMergeThreads, 0, st>>>((const __nv_bfloat16*)Oa, la, (const __nv_bfloat16*)Ob, lb, (__nv_bfloat16*)O, lse,
+  SPARSP_CUDA_OK(launch_kernel(kern, grid, kMergeThreads, 0, st, (const __nv_bfloat16*)Oa, la, (const __nv_bfloat16*)Ob, lb, (__nv_bfloat16*)O, lse,
                                        g.B, g.H, g.NB, g.N, g.b, s.stride_batch, s.stride_head, s.stride_token, rank,
-                                       consumer, head_begin, head_end);
-  count_launch();
-  SPARSP_CUDA_OK(cudaGetLastError());
+                                       consumer, head_begin, head_end));
   return SPARSP_OK;
 }
 
