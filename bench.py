@@ -211,10 +211,19 @@ class Config:
         total_entries = int(self.do["seg_total"].sum().item())
         self.packed = torch.empty(max(total_entries * self.entry, 16), dtype=torch.uint8, device=dev)
         self.volume = int(self.do["volume_bytes"].sum().item())
+        self.sources = self.distinct_tiles() * self.entry
         self.flops, self.kept_pairs = kept_flops_and_counts(self.mo["mask"], self.N, self.b, self.d)
         self.input_bytes = 3 * self.Q.numel() * 2
         # a working set that fits L2 would turn "HBM GB/s" into an L2 figure: flush L2 between iterations
         self.flush = torch.empty(2 * L2_BYTES, dtype=torch.uint8, device=dev) if self.input_bytes < 2 * L2_BYTES else None
+
+    def distinct_tiles(self):
+        """(KV block, head) pairs that at least one rank receives: what the gather cannot do without reading."""
+        own = torch.zeros(self.P, 32 * self.do["union_mask"].shape[-1], dtype=torch.bool, device=self.rank_d.device)
+        own[self.rank_d.long(), torch.arange(self.NB, device=own.device)] = True
+        bits = (self.do["union_mask"].unsqueeze(-1) >> torch.arange(32, device=own.device, dtype=torch.int32)) & 1
+        taken = bits.bool().flatten(-2) & ~own[None, :, None]  # [B][P][H][32 * words]
+        return int(taken.any(1).sum().item())
 
     def step_mask(self):
         b, mo = self.binding, self.mo
@@ -333,7 +342,7 @@ def graph_replay(cfg, steps):
 def figures(cfg, t, peaks, traffic_table):
     """The per-kernel figures of one measured configuration."""
     attn_tflops = cfg.flops / (t["attn"] * 1e-3) / 1e12
-    pack_bytes = 2.0 * cfg.volume
+    pack_bytes = float(cfg.volume + cfg.sources)  # every packed byte written, every distinct tile read once
     pack_gbs = pack_bytes / (t["pack"] * 1e-3) / 1e9 if cfg.volume else 0.0
     traffic = traffic_table.get((cfg.wl.name, cfg.k)) if cfg.tau <= 0 and cfg.H == cfg.wl.heads else None
     return {
@@ -352,7 +361,7 @@ def figures(cfg, t, peaks, traffic_table):
                      "unit": "TFLOP/s", "frac": attn_tflops / peaks["bf16_tflops"],
                      "traffic": traffic[0] if traffic else None,
                      "traffic_source": traffic[1] if traffic else "no ncu capture of this configuration"},
-        "roofline_pack": {"bound": "hbm", "kernel": "pack_bulk_kernel", "achieved": pack_gbs, "peak": peaks["hbm_gbs"],
+        "roofline_pack": {"bound": "hbm", "kernel": "pack_kernel", "achieved": pack_gbs, "peak": peaks["hbm_gbs"],
                           "peak_source": peaks["source"], "unit": "GB/s", "frac": pack_gbs / peaks["hbm_gbs"],
                           "algorithmic_bytes": pack_bytes},
     }
