@@ -70,3 +70,38 @@ def test_rows_and_heads_that_keep_nothing(oracle_mod, binding, d, b, layout, H, 
     check(O, lse, torch.nonzero(mine)[:, 0])
     assert bool((pu.from_layout(O, layout).cpu()[:, ~mine] == 5.0).all()) and bool((lse[0].cpu()[:, ~mine] == 5.0).all())
     assert binding.sparsp_status(ws) == binding.SPARSP_OK
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_stacked_blocks_of_a_packed_source_are_neighbours(binding, d):
+    """64-token blocks: the rows of two neighbours in the consumer's list come out bit for bit the same whatever the
+    consumer's other blocks keep, also where one of those keeps exactly what the first of the two keeps (the order in which
+    a row meets its scores, and with it every rounding, depends on the block it is stacked with)."""
+    H, NB, P, b = 2, 16, 2, 64
+    N = NB * b
+    rng = np.random.default_rng(d)
+    Q, K, V = (torch.tensor(rng.standard_normal((1, H, N, d)) * s).to(torch.bfloat16).cuda() for s in (3.0, 1.0, 1.0))
+    rank_d = torch.arange(NB, dtype=torch.int32).remainder(P).cuda()  # the consumer's list: blocks 0, 2, 4, ...
+    shape = binding.make_shape(H, d, (1, 1, N), 0, b)
+    ws = binding.make_workspace(shape, P)
+    first, second = 0b0101010101010101, 0b0011001101100110  # half of the first's blocks, and others
+
+    def rows_of_the_first_two(others):
+        words = np.zeros((H, NB, 1), np.uint32)
+        words[:, 0, 0], words[:, 2, 0] = first, second
+        for pos in range(2, NB // 2):
+            words[:, 2 * pos, 0] = others[pos]
+        mask_d = torch.as_tensor(words.view(np.int32)).cuda()
+        dm = pu.gpu_demand_pack(binding, shape, mask_d, rank_d, P, 0, K, V, ws)
+        O, lse = torch.zeros_like(Q), torch.zeros(1, H, N, device="cuda")
+        binding.sparsp_sparse_attn_fwd_packed(shape, Q, K, V, mask_d, rank_d, P, 0, dm["union_mask"], dm["seg_offset"],
+                                              dm["seg_total"], dm["packed"], dm["packed"].numel(), None, 0.0, O, lse, ws)
+        assert binding.sparsp_status(ws) == binding.SPARSP_OK
+        mine = torch.cat([torch.arange(b), torch.arange(2 * b, 3 * b)]).cuda()
+        return O[:, :, mine].view(torch.int16), lse[:, :, mine].view(torch.int32)
+
+    apart = [1 << (2 * (pos % 2) + 1) for pos in range(NB // 2)]
+    want = rows_of_the_first_two(apart)
+    for twin in (2, 3, 4):
+        got = rows_of_the_first_two(apart[:twin] + [first] + apart[twin + 1:])
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1]), twin
