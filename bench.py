@@ -174,6 +174,18 @@ def kept_flops_and_counts(mask_i32, N, b, d):
     return 4.0 * d * pairs, kept
 
 
+def distinct_tiles(union_i32, rank_of_block):
+    """(batch item, head, KV block) triples that at least one rank receives from another: the tiles that a gather cannot do
+    without reading.  union_i32: [B][P][H][words] bit words, rank_of_block: [NB]."""
+    import torch
+    P, Wd = union_i32.shape[1], union_i32.shape[-1]
+    own = torch.zeros(P, 32 * Wd, dtype=torch.bool, device=union_i32.device)
+    own[rank_of_block.long(), torch.arange(rank_of_block.numel(), device=own.device)] = True
+    bits = (union_i32.unsqueeze(-1) >> torch.arange(32, device=own.device, dtype=torch.int32)) & 1
+    received = bits.bool().flatten(-2) & ~own[None, :, None]  # [B][P][H][32 * words]
+    return int(received.any(1).sum().item())
+
+
 # ------------------------------------------------------------------------------------------------
 # our arm
 # ------------------------------------------------------------------------------------------------
@@ -211,19 +223,11 @@ class Config:
         total_entries = int(self.do["seg_total"].sum().item())
         self.packed = torch.empty(max(total_entries * self.entry, 16), dtype=torch.uint8, device=dev)
         self.volume = int(self.do["volume_bytes"].sum().item())
-        self.sources = self.distinct_tiles() * self.entry
+        self.sources = distinct_tiles(self.do["union_mask"], self.rank_d) * self.entry
         self.flops, self.kept_pairs = kept_flops_and_counts(self.mo["mask"], self.N, self.b, self.d)
         self.input_bytes = 3 * self.Q.numel() * 2
         # a working set that fits L2 would turn "HBM GB/s" into an L2 figure: flush L2 between iterations
         self.flush = torch.empty(2 * L2_BYTES, dtype=torch.uint8, device=dev) if self.input_bytes < 2 * L2_BYTES else None
-
-    def distinct_tiles(self):
-        """(KV block, head) pairs that at least one rank receives: what the gather cannot do without reading."""
-        own = torch.zeros(self.P, 32 * self.do["union_mask"].shape[-1], dtype=torch.bool, device=self.rank_d.device)
-        own[self.rank_d.long(), torch.arange(self.NB, device=own.device)] = True
-        bits = (self.do["union_mask"].unsqueeze(-1) >> torch.arange(32, device=own.device, dtype=torch.int32)) & 1
-        taken = bits.bool().flatten(-2) & ~own[None, :, None]  # [B][P][H][32 * words]
-        return int(taken.any(1).sum().item())
 
     def step_mask(self):
         b, mo = self.binding, self.mo
