@@ -11,7 +11,8 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsparsp.so")
 SOURCES = ["api.cu", "mask_kernels.cu", "demand_kernels.cu", "attn_kernel.cu", "merge_kernels.cu",
            "placement_kernels.cu", "diag_kernels.cu", "exchange.cu"]
-HEADERS = ["block_sets.cuh", "common.cuh", "sm100_ptx.cuh", os.path.join("..", "..", "include", "sparsp.h")]
+HEADERS = ["block_sets.cuh", "common.cuh", "item_queue.cuh", "sm100_ptx.cuh",
+           os.path.join("..", "..", "include", "sparsp.h")]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
 

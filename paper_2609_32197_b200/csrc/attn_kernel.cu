@@ -44,6 +44,7 @@
 
 #include "block_sets.cuh"
 #include "common.cuh"
+#include "item_queue.cuh"
 #include "sm100_ptx.cuh"
 
 namespace sparsp {
@@ -544,19 +545,17 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           bh = after ? hb + f : p.BH;
           x = it - (f > 0 ? __shfl_sync(0xffffffffu, h_end, f - 1) : hbase);
         } else {
-          const int per_bh = C::kStacked ? (p.NB + 1) / 2 : p.NB;
-          bh = it / per_bh;
-          x = it - bh * per_bh;
           // Behind a head's last item are its query blocks that keep nothing: all CTAs go on with the next head.
-          while (bh < p.BH && x >= p.n_items[bh] && !*s_abort) {
+          auto leave_head = [&](int first) {
+            int to = 0;
             if (lane == 0) {
-              atomicMax(p.work_counter, max((bh + 1) * per_bh - (int)gridDim.x, 0));
-              it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
+              atomicMax(p.work_counter, max(first - (int)gridDim.x, 0));
+              to = (int)gridDim.x + atomicAdd(p.work_counter, 1);
             }
-            it = __shfl_sync(0xffffffffu, it, 0);
-            bh = it / per_bh;
-            x = it - bh * per_bh;
-          }
+            return __shfl_sync(0xffffffffu, to, 0);
+          };
+          bh = find_item(it, C::kStacked ? (p.NB + 1) / 2 : p.NB, p.BH, p.n_items, leave_head,
+                         [&] { return *s_abort != 0; }, &x);
         }
         if (bh >= p.BH) return;
         const int32_t* items = p.pairs + (int64_t)bh * (2 * ((p.NB + 1) / 2));
