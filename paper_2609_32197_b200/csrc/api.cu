@@ -22,6 +22,7 @@ void set_error(const char* fmt, ...) {
 
 int cuda_fail(cudaError_t e, const char* what) {
   set_error("CUDA error %d (%s) in %s", (int)e, cudaGetErrorString(e), what);
+  (void)cudaGetLastError();  // the runtime keeps a refused launch's code for the next check, of some other call
   return SPARSP_ERR_CUDA;
 }
 

@@ -65,8 +65,9 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int threads, s
   cfg.stream = st;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  count_launch();
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e == cudaSuccess) count_launch();
+  return e;
 }
 
 #ifdef __CUDACC__

@@ -30,8 +30,8 @@ __global__ void __launch_bounds__(32) wait_timeout_kernel(int32_t* __restrict__ 
 int launch_wait_timeout(char* ws, const WsLayout& L, long long limit_cycles, cudaStream_t st) {
   int32_t* status = (int32_t*)(ws + L.status);
   wait_timeout_kernel<<<1, 32, 0, st>>>(status, limit_cycles, status + 4);
-  count_launch();
   SPARSP_CUDA_OK(cudaGetLastError());
+  count_launch();
   return SPARSP_OK;
 }
 

@@ -42,8 +42,8 @@ int launch_permute_tokens(const sparsp_shape& s, const Geometry& g, const void* 
     permute_tokens_kernel<128><<<grid, 256, 0, st>>>((const __nv_bfloat16*)X, (__nv_bfloat16*)Y, block_of_slot,
                                                      token_offset_of_slot, g.b, g.N, s.stride_batch, s.stride_head,
                                                      s.stride_token, inverse);
-  count_launch();
   SPARSP_CUDA_OK(cudaGetLastError());
+  count_launch();
   return SPARSP_OK;
 }
 
@@ -80,8 +80,8 @@ int launch_sharing(const Geometry& g, const uint32_t* mask, const int32_t* rank,
   const int64_t warps = (int64_t)g.B * P * g.H * g.Wd;
   sharing_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(mask, rank, g.B, g.H, g.NB, g.Wd, P,
                                                                     (unsigned long long*)hist);
-  count_launch();
   SPARSP_CUDA_OK(cudaGetLastError());
+  count_launch();
   return SPARSP_OK;
 }
 
