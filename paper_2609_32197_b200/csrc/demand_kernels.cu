@@ -12,6 +12,8 @@ namespace sparsp {
 // One CTA per (batch, head, rank r) computes
 //   U[b][r][h][w] = OR over the query blocks i of rank r of M[b][h][i][w]
 //   cnt[b][r][p][h] = popcount(U[b][r][h] & own[p]),  own[p] = the blocks of rank p
+// and, with `received` given, received[b][r][h], the number of entries packed for consumer r in head h: what the plan's
+// CTAs need of the consumers before theirs.
 // It reads the rows of its own query blocks only, whole words per lane (a row of up to 32 words is one coalesced
 // request, shorter rows share one), so a mask row is read once in all and B*H*P CTAs are in flight; the ownership
 // words are rebuilt per CTA from the rank table.  Latency-bound: the mask is a few MB.  (One CTA per (batch, head) with
@@ -22,7 +24,8 @@ constexpr int kUnionThreads = 512;
 __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32_t* __restrict__ mask,
                                                                     const int32_t* __restrict__ rank, int H, int NB,
                                                                     int Wd, int P, uint32_t* __restrict__ U,
-                                                                    int32_t* __restrict__ cnt,
+                                                                    int include_local, int32_t* __restrict__ cnt,
+                                                                    int32_t* __restrict__ received,
                                                                     int32_t* __restrict__ n_src) {
   enter_grid(mask, rank);
   __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
@@ -56,19 +59,28 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
     const int c = __reduce_add_sync(0xffffffffu, lane < Wd ? __popc(u & own_s[p * Wd + lane]) : 0);
     if (lane == 0) cnt[((int64_t)(bb * P + r) * P + p) * H + h] = c;
   }
+  if (received && warp == n_warps - 1) {  // (up to 15 ranks this warp has no counts to take)
+    uint32_t packed = 0;
+    if (lane < Wd)
+      for (int p = 0; p < P; ++p) packed |= p != r || include_local ? own_s[p * Wd + lane] : 0u;
+    const int c = __reduce_add_sync(0xffffffffu, __popc(u & packed));
+    if (lane == 0) received[(int64_t)(bb * P + r) * H + h] = c;
+  }
 }
 
 // Pack-order offsets, and where every packed tile goes.  A CTA per consumer scans its consumer's counts in pack
 // order (producer, then head) and writes offsets, total and volume.  With `dst` given there are consumers + batch items
 // CTAs per head: CTA (consumer, h) also fills its column of the destination table
 //   dst[(b*H + h)*NB + j][r] = byte offset in `packed` of consumer r's copy of block j, or -1
-// one warp per producer (the consumer's base is its caller-given dst_base or the sum of all earlier consumers' counts),
-// and CTA (B*P + b, h) appends the blocks that any consumer of batch item b receives to the list of sources, a head's
+// one warp per producer (the consumer's base is its caller-given dst_base or the sum of `received` over all earlier
+// consumers), and CTA (B*P + b, h) appends the blocks that any consumer of batch item b receives to the list of sources, a head's
 // blocks together.  The order of the heads in that list is the order in which they arrive; it decides nothing but the
 // order of the copies.
-// Latency-bound integer work on a few MB, so every CTA repeats the scan (P*H counts) rather than wait for another
-// launch.  (A serial scan per consumer in one CTA and a launch for the entries: 13 + 7 us on 24 heads, 8 ranks, 18 + 4 us on 48
-// heads; offsets alone 2 us now, with destinations 9 us on 48 and 15 us on 24 heads; eight heads to a CTA, one warp each: 16-19 us.)
+// Latency-bound integer work on a few MB, so every CTA repeats the scan (P*H counts) and the sum (at most B*P*H values)
+// rather than wait for another launch.  (A serial scan per consumer in one CTA and a launch for the entries: 13 + 7 us on 24
+// heads, 8 ranks, 18 + 4 us on 48 heads; offsets alone 2 us now, with destinations 9 us on 48 and 15 us on 24 heads; eight
+// heads to a CTA, one warp each: 16-19 us.  Union, plan and an empty gather at the limit, 16 batch items x 64 ranks x 24
+// heads: 0.55 ms; 72 ms with the sum over the counts of every producer, 2.9 ms with the serial scan.)
 constexpr int kPlanThreads = 256;
 
 __device__ __forceinline__ int64_t block_sum(int64_t v, int64_t* warp_s) {
@@ -84,12 +96,12 @@ __device__ __forceinline__ int64_t block_sum(int64_t v, int64_t* warp_s) {
 }
 
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(
-    const int32_t* __restrict__ cnt, const uint32_t* __restrict__ U, const int32_t* __restrict__ rank, int BP, int H,
-    int NB, int Wd, int P, int include_local, int64_t entry_bytes, int64_t* __restrict__ seg_off,
-    int64_t* __restrict__ seg_total, int64_t* __restrict__ volume, const int64_t* __restrict__ dst_base,
-    int64_t capacity, int64_t* __restrict__ dst, int32_t* __restrict__ src, int32_t* __restrict__ n_src,
-    int32_t* __restrict__ status) {
-  enter_grid(cnt, U, rank, dst_base);
+    const int32_t* __restrict__ cnt, const int32_t* __restrict__ received, const uint32_t* __restrict__ U,
+    const int32_t* __restrict__ rank, int BP, int H, int NB, int Wd, int P, int include_local, int64_t entry_bytes,
+    int64_t* __restrict__ seg_off, int64_t* __restrict__ seg_total, int64_t* __restrict__ volume,
+    const int64_t* __restrict__ dst_base, int64_t capacity, int64_t* __restrict__ dst, int32_t* __restrict__ src,
+    int32_t* __restrict__ n_src, int32_t* __restrict__ status) {
+  enter_grid(cnt, received, U, rank, dst_base);
   __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
   __shared__ int64_t seg_s[kMaxRanks];  // first entry of (producer, my head)
   __shared__ int64_t warp_s[kPlanThreads / 32];
@@ -163,10 +175,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(
     base = dst_base[br];
   } else if (br > 0) {
     int64_t n = 0;
-    for (int row = warp; row < br * P; row += kPlanThreads / 32) {  // (consumer, producer), a warp each
-      if (include_local || (row / P) % P != row % P)
-        for (int k = lane; k < H; k += 32) n += cnt[(int64_t)row * H + k];
-    }
+    for (int k = threadIdx.x; k < br * H; k += kPlanThreads) n += received[k];
     base = entry_bytes * block_sum(n, warp_s);
   }
   __syncthreads();
@@ -195,18 +204,24 @@ static int64_t* dst_table(char* ws, const WsLayout& L) { return (int64_t*)(ws + 
 static int32_t* src_list(char* ws, const WsLayout& L, const Geometry& g, int n_dst) {
   return (int32_t*)(ws + L.entries + (int64_t)g.B * g.H * g.NB * n_dst * 8);
 }
+// Entries per (consumer, head) [B*P*H] behind them: tables and list take 8 P + 4 of the 16 P bytes for a block, these 4 P for
+// a head.
+static int32_t* received_table(char* ws, const WsLayout& L, const Geometry& g, int P) {
+  return src_list(ws, L, g, P) + (int64_t)g.B * g.H * g.NB;
+}
 
+// dst, src, n_src, received: NULL for a plan without destinations.
 static cudaError_t launch_plan(const Geometry& g, const uint32_t* mask, const int32_t* rank, int P, int include_local,
-                        uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total, int64_t* volume,
-                        const int64_t* dst_base, int64_t capacity, int64_t* dst, int32_t* src, int32_t* n_src,
-                        int32_t* status, cudaStream_t st) {
+                               uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total, int64_t* volume,
+                               const int64_t* dst_base, int64_t capacity, int64_t* dst, int32_t* src, int32_t* n_src,
+                               int32_t* received, int32_t* status, cudaStream_t st) {
   cudaError_t e = launch_kernel(union_count_kernel, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P, U,
-                                cnt, n_src);
+                                include_local, cnt, received, n_src);
   if (e != cudaSuccess) return e;
   const unsigned grid = dst ? (unsigned)((g.B * P + g.B) * g.H) : (unsigned)(g.B * P);
-  return launch_kernel(plan_kernel, grid, kPlanThreads, 0, st, cnt, U, rank, g.B * P, g.H, g.NB, g.Wd, P, include_local,
-                                             2LL * g.b * g.d * 2, seg_off, seg_total, volume, dst_base, capacity, dst,
-                                             src, n_src, status);
+  return launch_kernel(plan_kernel, grid, kPlanThreads, 0, st, cnt, received, U, rank, g.B * P, g.H, g.NB, g.Wd, P,
+                       include_local, 2LL * g.b * g.d * 2, seg_off, seg_total, volume, dst_base, capacity, dst, src, n_src,
+                       status);
 }
 
 int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_of_block, int P,
@@ -218,9 +233,10 @@ int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_o
     set_error("batch * n_ranks = %d exceeds 1024", g.B * P);
     return SPARSP_ERR_UNSUPPORTED;
   }
-  SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, P, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, U, cnt, seg_off, seg_total, volume,
-              dst_base, capacity, pack ? dst_table(ws, L) : nullptr, pack ? src_list(ws, L, g, P) : nullptr,
-              pack ? (int32_t*)(ws + L.n_entries) : nullptr, (int32_t*)(ws + L.status), st));
+  SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, P, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, U, cnt, seg_off,
+                             seg_total, volume, dst_base, capacity, pack ? dst_table(ws, L) : nullptr,
+                             pack ? src_list(ws, L, g, P) : nullptr, pack ? (int32_t*)(ws + L.n_entries) : nullptr,
+                             pack ? received_table(ws, L, g, P) : nullptr, (int32_t*)(ws + L.status), st));
   return SPARSP_OK;
 }
 
@@ -433,7 +449,8 @@ extern "C" SPARSP_API int sparsp_demand_plan_noalloc(const sparsp_shape* shape, 
     set_error("sparsp_demand_plan_noalloc: misaligned argument");
     return SPARSP_ERR_INVALID_ARG;
   }
-  SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, n_ranks, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, union_mask, cnt, seg_offset,
-              seg_total, volume_bytes, nullptr, -1, nullptr, nullptr, nullptr, nullptr, (cudaStream_t)stream));
+  SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, n_ranks, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, union_mask, cnt,
+                             seg_offset, seg_total, volume_bytes, nullptr, -1, nullptr, nullptr, nullptr, nullptr, nullptr,
+                             (cudaStream_t)stream));
   return SPARSP_OK;
 }
