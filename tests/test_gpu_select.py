@@ -58,6 +58,27 @@ def test_threshold_rows_of_every_instance(oracle_mod, binding, NB):
         assert np.array_equal(cnt[0].cpu().numpy(), ref["kv_count"])
 
 
+@pytest.mark.parametrize("NB", [31, 129, 257, 385, 513, 641, 769, 1024])
+def test_threshold_rows_with_infinite_scores(oracle_mod, binding, NB):
+    """Odd query blocks score one block -inf: the search starts at an infinite end.  Even ones score it +inf: no difference to
+    that maximum is a number or finite, all weights are zero, and no block reaches the threshold."""
+    b, d = 64, 64
+    Q, K = _inputs(NB, b, d, NB + 2, True)
+    shape = binding.make_shape(2, d, (1, 1, NB * b), 0, b)
+    ws = binding.make_workspace(shape, 1)
+    g = binding.sparsp_geometry(shape)
+    Qd, Kd = Q.cuda(), K.cuda()
+    for tau, scale in ((1e-6, 0.0), (0.5, 40.0), (0.93, 3.0), (1.0, 0.0)):
+        mask = torch.zeros(1, 2, NB, g.n_words, dtype=torch.int32, device="cuda")
+        cnt = torch.zeros(1, 2, NB, dtype=torch.int32, device="cuda")
+        binding.sparsp_block_mask_cdf(shape, Qd, Kd, tau, scale, mask, cnt, None, None, ws)
+        ref = oracle_mod.block_mask_cdf(Q, K, b, tau, 0, scale)
+        got, count = pu.u32(mask[0]), cnt[0].cpu().numpy()
+        assert np.array_equal(got[:, 1::2], ref["mask"][:, 1::2]), (tau, scale)
+        assert np.array_equal(count[:, 1::2], ref["kv_count"][:, 1::2])
+        assert not got[:, ::2].any() and not count[:, ::2].any()
+
+
 @pytest.mark.parametrize("d,b", [(64, 64), (128, 128)])
 @pytest.mark.parametrize("layout", ["HND", "NHD"])
 def test_pool_at_the_change_of_form(oracle_mod, binding, d, b, layout):
