@@ -109,3 +109,39 @@ def test_calls_wait_for_the_callers_kernels_and_these_for_the_calls(binding, d, 
             writer.wait_event(done)
             layer.leave()
         _same(layer.outputs(), want)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_calls_behind_a_join_are_captured(binding, d):
+    """The inputs come from two streams that join before the first call; they are overwritten on the other stream behind the last one.
+    All of it is captured once and replayed."""
+    layer = _Layer(binding, d)
+    layer.arrive()
+    torch.cuda.synchronize()
+    layer.calls()
+    want = layer.outputs()
+    layer.leave()
+    torch.cuda.synchronize()
+    main, side = torch.cuda.Stream(), torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=main):
+        begin, arrived, done, left = (torch.cuda.Event() for _ in range(4))
+        begin.record()
+        with torch.cuda.stream(side):
+            side.wait_event(begin)
+            for x, y in zip((layer.Q, layer.K), layer.src):
+                x.copy_(y)
+            arrived.record()
+        layer.V.copy_(layer.src[2])
+        layer.rank.copy_(layer.rank_src)
+        main.wait_event(arrived)
+        layer.calls()
+        done.record()
+        with torch.cuda.stream(side):
+            side.wait_event(done)
+            layer.leave()
+            left.record()
+        main.wait_event(left)
+    for _ in range(2):
+        graph.replay()
+        _same(layer.outputs(), want)
