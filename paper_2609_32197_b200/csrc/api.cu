@@ -126,8 +126,8 @@ WsLayout make_layout(const Geometry& g, int P) {
   off += align_up((int64_t)g.B * g.H * g.NB * 4, 256);
   L.n_entries = off;  // blocks that anybody receives, int32
   off += 256;
-  // destinations of every block, int64 [B][H][NB][P], the list of those blocks, int32 [B][H][NB], and the entries of every
-  // (consumer, head), int32 [B][P][H]
+  // destinations of every block, int64 [B][H][NB][P], the list of those blocks, int32 [B][H][NB], and the entries of
+  // every (consumer, head), int32 [B][P][H]
   L.entries = off;
   off += align_up((int64_t)g.B * P * g.H * g.NB * 16, 256);
   L.total = off;

@@ -62,8 +62,8 @@ struct AttnParams {
   // consumer's first tile in the packed tensor map (a device scalar)
   const int32_t* slot;
   const int64_t* tile_base;
-  // K / V source only: largest key norm (L2) of every KV block that any row keeps, [B*H][NB]: lets a softmax row skip the
-  // row-maximum pass of a tile whose scores provably stay within 2^kSkipMargin of the row's reference maximum
+  // K / V source only: largest key norm (L2) of every KV block that any row keeps, [B*H][NB]: lets a softmax row skip
+  // the row-maximum pass of a tile whose scores provably stay within 2^kSkipMargin of the row's reference maximum
   const float* knorm;
   __nv_bfloat16* O;
   float* lse;
@@ -228,12 +228,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   uint64_t* o_full = p_full + 2;
   uint64_t* o_drained = o_full + 4;      // the item's accumulator has been read out by all 8 softmax warps
   uint64_t* list_ready = o_drained + 1;  // [2] list buffer filled
-  uint64_t* list_free = list_ready + 2;  // [2] list buffer no longer needed by its 11 readers
+  uint64_t* list_free = list_ready + 2;  // [2] list buffer no longer needed by its kListReaders
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
   int* s_nent = reinterpret_cast<int*>(smem + C::kOffMisc + 8);   // [2]
   int* s_blk = reinterpret_cast<int*>(smem + C::kOffMisc + 16);   // [2][2] the item's query block(s); < 0 = absent
-  int* s_item = reinterpret_cast<int*>(smem + C::kOffMisc + 32);  // [2] batch * H + head of the item in each list buffer; < 0 = no more
+  int* s_item = reinterpret_cast<int*>(smem + C::kOffMisc + 32);  // [2] batch * H + head of each list buffer; < 0: none
   int* s_rag = reinterpret_cast<int*>(smem + C::kOffMisc + 40);   // [2] the item's last tile reaches past the end of the sequence
   volatile int* s_frz = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 56);  // [4] per row group: reference frozen
   volatile int* s_pv_items = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 72);  // items whose P V are all issued
@@ -515,10 +515,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       // Items are handed out head by head (a head's K and V stay in L2).  A CTA's first item is its own number, the
       // following ones come from a global counter (first come, first served), so CTAs whose items are short simply take
       // more of them; the head travels to the other roles with the list.
-      // Packed source: a head has few items, the consumer's; they are numbered without gaps, and since numbers only grow
-      // the place of an item is found by walking the heads' item counts forward, 32 heads at a time with a count per lane.
-      // K / V source: all query blocks count, and nearly always all of them keep something.
-      int hb = 0, hbase = 0, h_end;  // first head of the 32, items before it, items up to and including this lane's head
+      // Packed source: a head has few items, the consumer's; they are numbered without gaps, and since numbers only
+      // grow the place of an item is found by walking the heads' item counts forward, 32 heads at a time with a count
+      // per lane. K / V source: all query blocks count, and nearly always all of them keep something.
+      int hb = 0, hbase = 0, h_end;  // first head of the 32, items before it, items up to and including this lane's
       auto load_heads = [&]() {
         h_end = hb + lane < p.BH ? p.n_items[hb + lane] : 0;
 #pragma unroll
@@ -570,10 +570,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (lane == 0) it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
         return __shfl_sync(0xffffffffu, it, 0);
       };
-      // When the next item is taken: for stacked items of a packed source with d = 128, whose lists are short and slow to
-      // build, right after the list before it, while its buffer is still in use (one-call attention of 24 heads x 24576, 4
-      // ranks: 371 -> 348 us).  Everywhere else once there is a buffer for it: an item taken early is one that a CTA with
-      // nothing left to do cannot take (26 heads x 6034, 40 heads x 75600 hop by hop: 3 % slower when taken early).
+      // When the next item is taken: for stacked items of a packed source with d = 128, whose lists are short and slow
+      // to build, right after the list before it, while its buffer is still in use (24 heads x 24576, 4 ranks: one call
+      // 434 us against 483, with a shuffled placement 421 against 462, hop by hop 796 against 811; 12 heads x 9504: 64.5
+      // against 66.4).  Everywhere else once there is a buffer for it: an item taken early is one that a CTA with nothing
+      // left to do cannot take (packed source, d = 64, 24 heads x 24576: one call 339 us against 345-358 early, hop by
+      // hop 641 against 654; 48 heads x 17776, 8 ranks: 265 against 271-280; K / V source, 26 heads x 6034 and 40 heads
+      // x 75600 hop by hop: 3 % slower early).
       constexpr bool kEarly = kPacked && C::kStacked && D == 128;
       if (kEarly) fetch(blockIdx.x);
       for (int i = 0;; ++i) {
@@ -604,7 +607,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         int n_both = 0, n_mix = 0, n_grp = 0, running;
         if (C::kStacked) {
           n_both = __reduce_add_sync(0xffffffffu, __popc(rb0 & rb1));
-          const int n0 = __reduce_add_sync(0xffffffffu, __popc(rb0 & ~rb1)), n1 = __reduce_add_sync(0xffffffffu, __popc(rb1 & ~rb0));
+          const int n0 = __reduce_add_sync(0xffffffffu, __popc(rb0 & ~rb1));
+          const int n1 = __reduce_add_sync(0xffffffffu, __popc(rb1 & ~rb0));
           n_mix = min(n0, n1);
           // two full tiles (four blocks both keep), then two half-work tiles (two one-sided pairs), and so on
           n_grp = min(n_both >> 2, n_mix >> 1);
@@ -616,7 +620,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         int at0 = 0, at1 = 0, at2 = 0;  // entries of each class so far
         for (uint32_t todo = __ballot_sync(0xffffffffu, (rb0 | rb1) != 0u); todo; todo &= todo - 1) {
           const int w = __ffs(todo) - 1;
-          const uint32_t w0 = __shfl_sync(0xffffffffu, rb0, w), w1 = C::kStacked ? __shfl_sync(0xffffffffu, rb1, w) : 0u;
+          const uint32_t w0 = __shfl_sync(0xffffffffu, rb0, w);
+          const uint32_t w1 = C::kStacked ? __shfl_sync(0xffffffffu, rb1, w) : 0u;
           const int jb = w * 32 + lane;
           const int nvalid = (int)min((int64_t)BLK, p.N - (int64_t)jb * BLK);
           if (C::kStacked) {
@@ -659,7 +664,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           if (lane == 0) {
             const int e = running - 1;
             const uint16_t tj = entJ[rag_pos]; entJ[rag_pos] = entJ[e]; entJ[e] = tj;
-            for (int q = 0; q < 2; ++q) { const uint8_t tv = entV[rag_pos * 2 + q]; entV[rag_pos * 2 + q] = entV[e * 2 + q]; entV[e * 2 + q] = tv; }
+            for (int q = 0; q < 2; ++q) {
+              const uint8_t tv = entV[rag_pos * 2 + q];
+              entV[rag_pos * 2 + q] = entV[e * 2 + q];
+              entV[e * 2 + q] = tv;
+            }
           }
           __syncwarp();
         }
@@ -1038,17 +1047,17 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 //   the rest       one warp per block: the largest key norm of the KV block, and the output rows of a query block that
 //                  keeps nothing (zeros, log-sum-exp -inf), so that such blocks never become work items.
 //
-// Block 64: which two query blocks share a Q tile.  K / V source: blocks i and i+D are paired in stripes (i mod 2D < D),
-// leftovers pair up consecutively; the offset D in 1..n/2 that maximises the summed overlap |M[i] & M[i+D]| of the kept
-// lists is chosen per (batch, head) -- video attention is multi-diagonal, so the best partner of a block is typically the
-// same position a fixed number of blocks away; the more two stacked blocks share, the less of a 128-row tile's work is
-// masked away.
+// Block 64: which two query blocks share a Q tile.  K / V source: blocks i and i+D are paired in stripes (i mod 2D <
+// D), leftovers pair up consecutively; the offset D in 1..n/2 that maximises the summed overlap |M[i] & M[i+D]| of the
+// kept lists is chosen per (batch, head) -- video attention is multi-diagonal, so the best partner of a block is
+// typically the same position a fixed number of blocks away; the more two stacked blocks share, the less of a 128-row
+// tile's work is masked away.
 // Packed source: neighbours in the consumer's ascending list of blocks (D = 1).  Its rows take their reference from the
-// first tiles, and neighbours keep each other's blocks: there a row nearly always meets its largest score at once, whose
-// exponential is then exactly 1.  Chosen by overlap the partner is far away, the largest term is some rounded 2^x, and the
-// output is further from 64 bits (24 heads x 24576, 4 ranks: 2.01e-3 against 1.95e-3, log-sum-exp 3.7e-4 against 3.2e-4).
-// (Mask rows in shared memory have an odd pitch: the threads' offsets differ by one row, a pitch of 32 words would put
-// them all on one bank.)
+// first tiles, and neighbours keep each other's blocks: there a row nearly always meets its largest score at once,
+// whose exponential is then exactly 1.  Chosen by overlap the partner is far away, the largest term is some rounded
+// 2^x, and the output is further from 64 bits (24 heads x 24576, 4 ranks: 2.01e-3 against 1.95e-3, log-sum-exp 3.7e-4
+// against 3.2e-4). (Mask rows in shared memory have an odd pitch: the threads' offsets differ by one row, a pitch of 32
+// words would put them all on one bank.)
 // Items of one (batch, head) are handed out longest list first: the items still running when the queue
 // runs dry are then the short ones, which matters when list lengths vary (threshold selection, unions of two
 // stacked blocks).  Key = (list length << 10) | (1023 - index): equal lengths keep their index order.
@@ -1108,7 +1117,8 @@ __device__ __forceinline__ int next_pow2(int n) {
 
 // Work items of one (batch, head) among the n query blocks list[0..n) (packed source; NULL: all blocks, K / V source);
 // returns their number.
-__device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uint16_t* list, int n, unsigned char* smem_raw) {
+__device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uint16_t* list, int n,
+                                          unsigned char* smem_raw) {
   __shared__ uint32_t s_keys[kMaxBlocks];
   __shared__ uint32_t s_pair[kMaxBlocks / 2];  // positions of an item's two blocks, (second or 0xffff) << 16 | first
   __shared__ unsigned int s_best;              // (score << 10) | (1023 - D): max = best score, smallest D
@@ -1362,8 +1372,8 @@ int make_tile_tmap(CUtensorMap* out, const void* base, const sparsp_shape& s, co
   cuuint32_t box[4] = {swizzled ? 64u : (cuuint32_t)g.d, (cuuint32_t)rows, 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzled ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzled ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_error("cuTensorMapEncodeTiled failed with %d", (int)r);
     return SPARSP_ERR_CUDA;

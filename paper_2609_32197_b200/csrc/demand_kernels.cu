@@ -17,8 +17,8 @@ namespace sparsp {
 // It reads the rows of its own query blocks only, whole words per lane (a row of up to 32 words is one coalesced
 // request, shorter rows share one), so a mask row is read once in all and B*H*P CTAs are in flight; the ownership
 // words are rebuilt per CTA from the rank table.  Latency-bound: the mask is a few MB.  (One CTA per (batch, head) with
-// shared-memory atomics for all ranks at once: 20.6 us on 24 heads x 929 blocks, 8 ranks, 24 CTAs on 148 SMs; this split
-// 8 us.)  OR does not depend on the order, so the bits are well defined.  A rank value outside [0, P) is ignored.
+// shared-memory atomics for all ranks at once: 20.6 us on 24 heads x 929 blocks, 8 ranks, 24 CTAs on 148 SMs; this
+// split 8 us.)  OR does not depend on the order, so the bits are well defined.  A rank value outside [0, P) is ignored.
 constexpr int kUnionThreads = 512;
 
 __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32_t* __restrict__ mask,
@@ -73,14 +73,14 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
 // CTAs per head: CTA (consumer, h) also fills its column of the destination table
 //   dst[(b*H + h)*NB + j][r] = byte offset in `packed` of consumer r's copy of block j, or -1
 // one warp per producer (the consumer's base is its caller-given dst_base or the sum of `received` over all earlier
-// consumers), and CTA (B*P + b, h) appends the blocks that any consumer of batch item b receives to the list of sources, a head's
-// blocks together.  The order of the heads in that list is the order in which they arrive; it decides nothing but the
-// order of the copies.
+// consumers), and CTA (B*P + b, h) appends the blocks that any consumer of batch item b receives to the list of
+// sources, a head's blocks together.  The order of the heads in that list is the order in which they arrive; it decides
+// nothing but the order of the copies.
 // Latency-bound integer work on a few MB, so every CTA repeats the scan (P*H counts) and the sum (at most B*P*H values)
-// rather than wait for another launch.  (A serial scan per consumer in one CTA and a launch for the entries: 13 + 7 us on 24
-// heads, 8 ranks, 18 + 4 us on 48 heads; offsets alone 2 us now, with destinations 9 us on 48 and 15 us on 24 heads; eight
-// heads to a CTA, one warp each: 16-19 us.  Union, plan and an empty gather at the limit, 16 batch items x 64 ranks x 24
-// heads: 0.55 ms; 72 ms with the sum over the counts of every producer, 2.9 ms with the serial scan.)
+// rather than wait for another launch.  (A serial scan per consumer in one CTA and a launch for the entries: 13 + 7 us
+// on 24 heads, 8 ranks, 18 + 4 us on 48 heads; offsets alone 2 us now, with destinations 9 us on 48 and 15 us on 24
+// heads; eight heads to a CTA, one warp each: 16-19 us.  Union, plan and an empty gather at the limit, 16 batch items x
+// 64 ranks x 24 heads: 0.55 ms; 72 ms with the sum over the counts of every producer, 2.9 ms with the serial scan.)
 constexpr int kPlanThreads = 256;
 
 __device__ __forceinline__ int64_t block_sum(int64_t v, int64_t* warp_s) {
@@ -117,7 +117,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(
       for (int p = 0; p < P; ++p) owned |= own_s[p * Wd + lane];
 #pragma unroll 8
       for (int r = 0; r < P; ++r)
-        live |= U[((int64_t)(bb * P + r) * H + h) * Wd + lane] & (include_local ? owned : owned & ~own_s[r * Wd + lane]);
+        live |= U[((int64_t)(bb * P + r) * H + h) * Wd + lane] &
+                (include_local ? owned : owned & ~own_s[r * Wd + lane]);
     }
     int total, first = 0;
     int at = bits_below(live, lane, &total);
@@ -204,8 +205,8 @@ static int64_t* dst_table(char* ws, const WsLayout& L) { return (int64_t*)(ws + 
 static int32_t* src_list(char* ws, const WsLayout& L, const Geometry& g, int n_dst) {
   return (int32_t*)(ws + L.entries + (int64_t)g.B * g.H * g.NB * n_dst * 8);
 }
-// Entries per (consumer, head) [B*P*H] behind them: tables and list take 8 P + 4 of the 16 P bytes for a block, these 4 P for
-// a head.
+// Entries per (consumer, head) [B*P*H] behind them: tables and list take 8 P + 4 of the 16 P bytes for a block, these 4
+// P for a head.
 static int32_t* received_table(char* ws, const WsLayout& L, const Geometry& g, int P) {
   return src_list(ws, L, g, P) + (int64_t)g.B * g.H * g.NB;
 }
@@ -215,13 +216,13 @@ static cudaError_t launch_plan(const Geometry& g, const uint32_t* mask, const in
                                uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total, int64_t* volume,
                                const int64_t* dst_base, int64_t capacity, int64_t* dst, int32_t* src, int32_t* n_src,
                                int32_t* received, int32_t* status, cudaStream_t st) {
-  cudaError_t e = launch_kernel(union_count_kernel, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P, U,
-                                include_local, cnt, received, n_src);
+  cudaError_t e = launch_kernel(union_count_kernel, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P,
+                                U, include_local, cnt, received, n_src);
   if (e != cudaSuccess) return e;
   const unsigned grid = dst ? (unsigned)((g.B * P + g.B) * g.H) : (unsigned)(g.B * P);
   return launch_kernel(plan_kernel, grid, kPlanThreads, 0, st, cnt, received, U, rank, g.B * P, g.H, g.NB, g.Wd, P,
-                       include_local, 2LL * g.b * g.d * 2, seg_off, seg_total, volume, dst_base, capacity, dst, src, n_src,
-                       status);
+                       include_local, 2LL * g.b * g.d * 2, seg_off, seg_total, volume, dst_base, capacity, dst, src,
+                       n_src, status);
 }
 
 int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_of_block, int P,
@@ -242,15 +243,15 @@ int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_o
 
 // ------------------------------------------------------------------------------------------------
 // Gather, source by source: a K or V tile is loaded into shared memory once and stored from there to every consumer
-// that selected it, so HBM carries one read per distinct tile and one write per packed tile -- its floor.  (Tile by tile
-// in the order of the packed buffer every copy was read again: 3.45 ms for the 10.8 GB that 8 ranks of 40 heads x 591
-// blocks of 32 KiB receive, at 6.3 TB/s of reads and writes; this order 2.23 ms, 5.5 TB/s of which seven eighths are writes.  Four to six
-// stages and one to three stores left in flight are within 1 %: memory sets the pace.)
+// that selected it, so HBM carries one read per distinct tile and one write per packed tile -- its floor.  (Tile by
+// tile in the order of the packed buffer every copy was read again: 3.45 ms for the 10.8 GB that 8 ranks of 40 heads x
+// 591 blocks of 32 KiB receive, at 6.3 TB/s of reads and writes; this order 2.23 ms, 5.5 TB/s of which seven eighths
+// are writes.  Four to six stages and one to three stores left in flight are within 1 %: memory sets the pace.)
 // One warp streams whole tiles: TMA tile load (any token stride; rows behind the last token arrive as zeros), then one
 // bulk store per consumer, issued by the lane that holds its destination.  A ring of kPackStages tile buffers per warp
 // (1, 2 or 4 warps per CTA for 32, 16, 8 KiB tiles: 160 KiB per CTA whatever the tile size), loads running
-// kPackStages - 1 tiles ahead of the stores.  The warp's next 32 sources sit in its lanes' registers and the next tile's
-// destinations are fetched before the wait for the current stores, so that no table lookup is exposed.
+// kPackStages - 1 tiles ahead of the stores.  The warp's next 32 sources sit in its lanes' registers and the next
+// tile's destinations are fetched before the wait for the current stores, so that no table lookup is exposed.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPackStages = 5;
 constexpr int kPackMaxWarps = 4;
@@ -340,8 +341,9 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps) pack_kernel(const __grid_c
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-static int run_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, const int64_t* dst, int n_dst,
-                    const int32_t* src, const int32_t* n_src, void* packed, int32_t* status, cudaStream_t st) {
+static int run_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, const int64_t* dst,
+                    int n_dst, const int32_t* src, const int32_t* n_src, void* packed, int32_t* status,
+                    cudaStream_t st) {
   int dev = 0, sms = 148;
   SPARSP_CUDA_OK(cudaGetDevice(&dev));
   SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -353,8 +355,8 @@ static int run_pack(const sparsp_shape& s, const Geometry& g, const void* K, con
   const int n_warps = std::max(1, std::min(kPackMaxWarps, (32 * 1024) / tile_bytes));
   const int smem = n_warps * kPackStages * tile_bytes;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)pack_kernel, smem));
-  SPARSP_CUDA_OK(launch_kernel(pack_kernel, sms, 32 * n_warps, smem, st, tk, tv, dst, n_dst, src, n_src, g.H, g.NB, g.b, (uint32_t)tile_bytes,
-                                               (unsigned char*)packed, status));
+  SPARSP_CUDA_OK(launch_kernel(pack_kernel, sms, 32 * n_warps, smem, st, tk, tv, dst, n_dst, src, n_src, g.H, g.NB, g.b,
+                               (uint32_t)tile_bytes, (unsigned char*)packed, status));
   return SPARSP_OK;
 }
 
@@ -407,8 +409,9 @@ int launch_pack_segment(const sparsp_shape& s, const Geometry& g, const uint32_t
   int32_t* src = src_list(ws, L, g, 1);
   int32_t* n_src = (int32_t*)(ws + L.n_entries);
   int32_t* status = (int32_t*)(ws + L.status);
-  SPARSP_CUDA_OK(launch_kernel(segment_kernel, (g.H * 32 + 255) / 256, 256, 0, st, U, rank, g.H, g.NB, g.Wd, P, consumer, producer, seg_off, cnt,
-                                                        2LL * g.b * g.d * 2, capacity, table, src, n_src, status));
+  SPARSP_CUDA_OK(launch_kernel(segment_kernel, (g.H * 32 + 255) / 256, 256, 0, st, U, rank, g.H, g.NB, g.Wd, P,
+                               consumer, producer, seg_off, cnt, 2LL * g.b * g.d * 2, capacity, table, src, n_src,
+                               status));
   return run_pack(s, g, K, V, table, 1, src, n_src, dst, status, st);
 }
 
@@ -450,7 +453,7 @@ extern "C" SPARSP_API int sparsp_demand_plan_noalloc(const sparsp_shape* shape, 
     return SPARSP_ERR_INVALID_ARG;
   }
   SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, n_ranks, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, union_mask, cnt,
-                             seg_offset, seg_total, volume_bytes, nullptr, -1, nullptr, nullptr, nullptr, nullptr, nullptr,
-                             (cudaStream_t)stream));
+                             seg_offset, seg_total, volume_bytes, nullptr, -1, nullptr, nullptr, nullptr, nullptr,
+                             nullptr, (cudaStream_t)stream));
   return SPARSP_OK;
 }

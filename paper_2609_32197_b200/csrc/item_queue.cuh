@@ -1,5 +1,5 @@
-// Which work item a number of the attention kernel's queue stands for (K / V source).  Plain integer code, apart from the
-// kernel so that it can be run on a host as well.
+// Which work item a number of the attention kernel's queue stands for (K / V source).  Plain integer code, apart from
+// the kernel so that it can be run on a host as well.
 #pragma once
 
 #include <stdint.h>
@@ -13,9 +13,9 @@
 namespace sparsp {
 
 // Numbers run head by head, per_head to a head, of which only the first n_items[head] are items.  Returns the head of
-// number `it` and its place *x among the head's items, or n_heads if there are no more.  A number behind a head's last item
-// is exchanged: next(first number of the next head) hands out another one.  stop() ends the search without an item: the
-// items' table is not written behind a head's last one, so nobody may look a place there up.
+// number `it` and its place *x among the head's items, or n_heads if there are no more.  A number behind a head's last
+// item is exchanged: next(first number of the next head) hands out another one.  stop() ends the search without an
+// item: the items' table is not written behind a head's last one, so nobody may look a place there up.
 template <typename Next, typename Stop>
 SPARSP_QUEUE_FN int find_item(int it, int per_head, int n_heads, const int32_t* n_items, Next next, Stop stop, int* x) {
   int head = it / per_head;

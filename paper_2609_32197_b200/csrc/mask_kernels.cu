@@ -16,10 +16,12 @@ namespace sparsp {
 // ------------------------------------------------------------------------------------------------
 // pool: a group of lanes owns one (tensor, batch*head, block) tile; a lane owns 8 (or 4) channels and walks the tile's
 // rows with 16-byte (8-byte) loads, several of them in flight, so every channel is one sequential chain.
-// Large problems are HBM-bound: 16-byte loads, 16 rows in flight (24 heads x 24576 x 128: 53.6 us = 5.6 TB/s; 8 rows
-// 54.5, 8-byte loads of 32 rows 68).  Where the tiles do not fill a quarter of the chip's thread slots the time is the
-// latency of the dependent batches: 8-byte loads, so twice the threads, and 32 rows in flight (26 heads x 6034 x 64:
-// 17.9 us against 28 with the wide form and 32-38 with 8 rows of it; 2 heads x 4096: 4.3 us against 6.2).
+// Large problems are HBM-bound: 16-byte loads, unrolled over 16 rows (24 heads x 24576 x 128: 53.6 us = 5.6 TB/s; over
+// 8 rows 54.5, 8-byte loads of 32 rows 68), of which the compiler keeps what fits 51 registers in flight, about 8.
+// Where the tiles do not fill a quarter of the chip's thread slots (148 SMs; the measured crossover, not a property of
+// the kernel) the time is the latency of the dependent batches: 8-byte loads, so twice the threads, and 32 rows in
+// flight (95 registers; 26 heads x 6034 x 64: 17.9 us against 28 with the wide form and 32-38 with 8 rows of it; 2
+// heads x 4096: 4.3 us against 6.2).
 // ------------------------------------------------------------------------------------------------
 constexpr int kPoolThreads = 128;
 constexpr int kPoolNarrowThreads = 148 * 512;  // up to this many threads of the wide form the narrow one is used
@@ -187,13 +189,16 @@ static cudaError_t launch_score(const Geometry& g, const float* pq, const float*
 
 // ------------------------------------------------------------------------------------------------
 // top-k: one warp per (batch, head, query block) row.  The row's scores become order-preserving
-// uint32 keys in registers (lane l holds blocks l, l + 32, ...); the warp finds the k-th largest key by bisection between
-// the row's smallest and largest key with compares and a warp sum per step, which ends as soon as a trial value has
-// exactly k keys at or above it (well before the 32 steps that a search bit by bit always takes), breaks ties towards
-// the lower index, forces the text blocks on, and emits the mask words and the ascending kept list by ballot-prefix
-// compaction.  Bound by instruction issue, a compare and an add per key and step: instances for several row lengths.
-// 24 x 384 rows of 384: 19 us, 40 x 591 of 591: 79 us, 24 x 929 of 929: 136 us (29, 152 and 194 us with 32 steps of one bit
-// each and instances of 4, 8, 16 and 32 words; bisection by the keys instead of the scores: 18, 71 and 212 us).
+// uint32 keys in registers (lane l holds blocks l, l + 32, ...); the warp finds the k-th largest key by bisection
+// between the row's smallest and largest key with compares and a warp sum per step, which ends as soon as a trial value
+// has exactly k keys at or above it (well before the 32 steps that a search bit by bit always takes), breaks ties
+// towards the lower index, forces the text blocks on, and emits the mask words and the ascending kept list by
+// ballot-prefix compaction.  Bound by instruction issue, a compare and an add per key and step: instances for several
+// row lengths. 24 x 384 rows of 384: 19 us, 40 x 591 of 591: 79 us, 24 x 929 of 929: 136 us (29, 152 and 194 us with 32
+// steps of one bit each and instances of 4, 8, 16 and 32 words; bisection by the keys instead of the scores: 18, 71 and
+// 212 us).  Four CTAs per SM
+// although the instances of 24 and 32 words spill for it: pool, score and selection of 24 x 929 rows 273 us, 296 with
+// three and 340 with two; of 40 x 700 rows 267, 284 and 285.
 // ------------------------------------------------------------------------------------------------
 constexpr int kTopkWarps = 8;
 
@@ -207,20 +212,19 @@ __device__ __forceinline__ float key_score(uint32_t key) {
   return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
 }
 
-// A key in (lo, hi] for the next step of a search, lo < hi: the one of the middle of the two scores, which halves evenly
-// spread scores where the middle of the keys halves their exponents; or the middle key where that is no such key (ends that
-// are infinite, not numbers or neighbours) and in every third step, so that the search ends after at most 96 steps.
+// A key in (lo, hi] for the next step of a search, lo < hi: the one of the middle of the two scores, which halves
+// evenly spread scores where the middle of the keys halves their exponents; or the middle key where that is no such key
+// (ends that are infinite, not numbers or neighbours) and in every third step, so that the search ends after at most 96
+// steps.
 __device__ __forceinline__ uint32_t middle(uint32_t lo, uint32_t hi, int step) {
   const uint32_t by_score = score_key(0.5f * key_score(lo) + 0.5f * key_score(hi));
   return by_score > lo && by_score <= hi && step % 3 != 2 ? by_score : lo + ((hi - lo) >> 1) + 1;
 }
 
 template <int WMAX>  // mask words per row this instance can hold (keys live in registers: WMAX per lane)
-__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 6 : 4) topk_kernel(const float* __restrict__ scores, int64_t n_rows,
-                                                               int NB, int Wd, int nb_cand, int topk,
-                                                               int kept_cap, uint32_t* __restrict__ mask,
-                                                               int32_t* __restrict__ kv_list,
-                                                               int32_t* __restrict__ kv_count) {
+__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 6 : 4)
+    topk_kernel(const float* __restrict__ scores, int64_t n_rows, int NB, int Wd, int nb_cand, int topk, int kept_cap,
+                uint32_t* __restrict__ mask, int32_t* __restrict__ kv_list, int32_t* __restrict__ kv_count) {
   enter_grid(scores);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * kTopkWarps + warp;  // (batch*H + head) * NB + i
@@ -317,10 +321,9 @@ __device__ __forceinline__ unsigned long long warp_sum(uint32_t v) {
 }
 
 template <int WMAX>  // mask words per row this instance can hold (keys and terms live in registers)
-__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 4 : WMAX <= 20 ? 3 : 2) cdf_kernel(const float* __restrict__ scores, int64_t n_rows, int NB,
-                                                              int Wd, int nb_cand, float tau, float c,
-                                                              uint32_t* __restrict__ mask,
-                                                              int32_t* __restrict__ kv_count) {
+__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 4 : WMAX <= 20 ? 3 : 2)
+    cdf_kernel(const float* __restrict__ scores, int64_t n_rows, int NB, int Wd, int nb_cand, float tau, float c,
+               uint32_t* __restrict__ mask, int32_t* __restrict__ kv_count) {
   enter_grid(scores);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * kTopkWarps + warp;  // (batch*H + head) * NB + i
@@ -407,10 +410,11 @@ int launch_score_cdf(const Geometry& g, const float* pq, const float* pk, float*
     const int64_t n_rows = (int64_t)g.B * g.H * g.NB;
     const float c = scale * 1.4426950408889634f;  // fp32 product, as in the definition above
     const unsigned grid = (unsigned)((n_rows + kTopkWarps - 1) / kTopkWarps);
-    auto kern = g.Wd <= 4 ? cdf_kernel<4> : g.Wd <= 8 ? cdf_kernel<8> : 
-                g.Wd <= 12 ? cdf_kernel<12> : g.Wd <= 16 ? cdf_kernel<16> : g.Wd <= 20 ? cdf_kernel<20> : 
+    auto kern = g.Wd <= 4 ? cdf_kernel<4> : g.Wd <= 8 ? cdf_kernel<8> :
+                g.Wd <= 12 ? cdf_kernel<12> : g.Wd <= 16 ? cdf_kernel<16> : g.Wd <= 20 ? cdf_kernel<20> :
                 g.Wd <= 24 ? cdf_kernel<24> : cdf_kernel<32>;
-    SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, g.NB, g.Wd, g.nb_cand, tau, c, mask, kv_count));
+    SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, g.NB, g.Wd, g.nb_cand, tau, c,
+                                 mask, kv_count));
   }
   return SPARSP_OK;
 }
@@ -422,10 +426,11 @@ int launch_score_topk(const Geometry& g, const float* pq, const float* pk, float
   {
     const int64_t n_rows = (int64_t)g.B * g.H * g.NB;
     const unsigned grid = (unsigned)((n_rows + kTopkWarps - 1) / kTopkWarps);
-    auto kern = g.Wd <= 4 ? topk_kernel<4> : g.Wd <= 8 ? topk_kernel<8> : 
-                g.Wd <= 12 ? topk_kernel<12> : g.Wd <= 16 ? topk_kernel<16> : g.Wd <= 20 ? topk_kernel<20> : 
+    auto kern = g.Wd <= 4 ? topk_kernel<4> : g.Wd <= 8 ? topk_kernel<8> :
+                g.Wd <= 12 ? topk_kernel<12> : g.Wd <= 16 ? topk_kernel<16> : g.Wd <= 20 ? topk_kernel<20> :
                 g.Wd <= 24 ? topk_kernel<24> : topk_kernel<32>;
-    SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, g.NB, g.Wd, g.nb_cand, topk, kept_cap, mask, kv_list, kv_count));
+    SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, g.NB, g.Wd, g.nb_cand, topk,
+                                 kept_cap, mask, kv_list, kv_count));
   }
   return SPARSP_OK;
 }
