@@ -32,29 +32,35 @@ __device__ __forceinline__ void own_words(const int32_t* __restrict__ rank, int 
   }
 }
 
-// words[kMaxWords]: the blocks of rank r.  The caller synchronises the block afterwards.
+// words[kMaxWords]: the blocks of rank r, a warp per word with its loads in flight.  The caller synchronises the block
+// afterwards.
 __device__ __forceinline__ void rank_words(const int32_t* __restrict__ rank, int NB, int r, uint32_t* words) {
-  if (threadIdx.x < kMaxWords) words[threadIdx.x] = 0u;
-  __syncthreads();
-  for (int j = threadIdx.x; j < NB; j += blockDim.x)
-    if (rank[j] == r) atomicOr(&words[j >> 5], 1u << (j & 31));
+  const int lane = threadIdx.x & 31, n = (NB + 31) >> 5;
+  if (threadIdx.x >= n && threadIdx.x < kMaxWords) words[threadIdx.x] = 0u;
+#pragma unroll 4
+  for (int w = threadIdx.x >> 5; w < n; w += blockDim.x >> 5) {
+    const int j = w * 32 + lane;
+    const uint32_t word = __ballot_sync(0xffffffffu, (j < NB ? rank[j] : ~r) == r);
+    if (lane == 0) words[w] = word;
+  }
 }
 
 // list[]: the blocks of the set in ascending order; returns their number.  Synchronises before and after.
 __device__ __forceinline__ int list_blocks(const uint32_t* words, int NB, uint16_t* list) {
+  __shared__ int before_s[kMaxWords + 1];  // blocks of the set in lower words; all of them
   __syncthreads();
-  int n = 0;
-  for (int w = 0; w < (NB + 31) / 32; ++w) n += __popc(words[w]);
-  for (int j = threadIdx.x; j < NB; j += blockDim.x) {
-    const uint32_t word = words[j >> 5];
-    if ((word >> (j & 31)) & 1u) {
-      int pos = __popc(word & ((1u << (j & 31)) - 1u));
-      for (int w = 0; w < (j >> 5); ++w) pos += __popc(words[w]);
-      list[pos] = (uint16_t)j;
-    }
+  if (threadIdx.x < kMaxWords) {
+    int total;
+    before_s[threadIdx.x] = bits_below(words[threadIdx.x], threadIdx.x, &total);
+    if (threadIdx.x == 0) before_s[kMaxWords] = total;
   }
   __syncthreads();
-  return n;
+  for (int j = threadIdx.x; j < NB; j += blockDim.x) {
+    const uint32_t word = words[j >> 5];
+    if ((word >> (j & 31)) & 1u) list[before_s[j >> 5] + __popc(word & ((1u << (j & 31)) - 1u))] = (uint16_t)j;
+  }
+  __syncthreads();
+  return before_s[kMaxWords];
 }
 
 }  // namespace sparsp

@@ -9,9 +9,9 @@
 namespace sparsp {
 
 // hop[b][h][i][w] = (rank[i] == consumer and head_begin <= h < head_end) ? mask[b][h][i][w] & own_producer[w] : 0.
-// A lane handles one word of kHopRows rows (rows of fewer than 32 words share a warp); the producer's ownership words and
-// the consumer's rows are bits in shared memory, built once per CTA.  A mask is a few MB, so this is latency: 40 heads x
-// 591 rows x 19 words in 6.2 us (11.3 us with a thread per word that walked 32 ranks for its ownership bits).
+// A lane handles one word of kHopRows rows (rows of fewer than 32 words share a warp); the producer's ownership words
+// and the consumer's rows are bits in shared memory, built once per CTA.  A mask is a few MB, so this is latency: 40
+// heads x 591 rows x 19 words in 6.2 us (11.3 us with a thread per word that walked 32 ranks for its ownership bits).
 constexpr int kHopThreads = 256;
 constexpr int kHopRows = 4;
 
@@ -49,27 +49,30 @@ __global__ void __launch_bounds__(kHopThreads) hop_mask_kernel(const uint32_t* _
   }
 }
 
-// Log-sum-exp merge.  Unit of work: one (batch, head, token block); the CTAs walk the units, with `rank` given only those
-// of the blocks of `consumer` in heads [head_begin, head_end) (one chunk of one hop of one rank; every other row stays
-// untouched), which each CTA lists from the rank table.  O_a, O_b, O: bf16 with the shape's strides; lse: fp32 [B][H][N].
-// A thread handles 8 columns of a row, kMergeRows rows at a time with all their loads in flight: HBM-bound, 33 us for
-// 74 blocks of 128 rows x 20 heads x 256 bytes (40 us with a CTA per block, most of which found another rank's block, and
-// one row of loads in flight).
-// O may be O_a or O_b and lse may be lse_a or lse_b (no pointer is declared restrict): a thread reads the 16 bytes it later
-// writes, and the D/8 threads of a row are consecutive lanes of one warp, all of which have read the row's log-sum-exp
-// values before its first thread writes the merged one.
+// Log-sum-exp merge.  Unit of work: one (batch, head, token block).  Without `rank` a CTA each; with `rank` given only
+// those of the blocks of `consumer` in heads [head_begin, head_end) (one chunk of one hop of one rank; every other row
+// stays untouched), which each CTA lists from the rank table and then walks.  O_a, O_b, O: bf16 with the shape's
+// strides; lse: fp32 [B][H][N].
+// A thread handles 8 columns of a row, kMergeRows rows at a time with all their loads in flight: a block of 64 tokens
+// has two rows for each thread at d = 64 (40 registers, 6 CTAs per SM), four or eight everywhere else (80 registers, 3
+// CTAs).  HBM-bound, us as it is / with four rows and 4 CTAs per SM, of which 3 fit, whatever the shape / with a CTA
+// per block and a row of loads in flight: 40 heads x 591 blocks of 128 x 128 as a whole 350 / 460 / 360, an eighth of
+// its blocks 60 / 71 / 73; 24 x 384 of 64 x 128 75 / 91 / 75, a quarter of them 13 / 14 / 17; 48 x 279 of 64 x 64 62 /
+// 97 / 65, an eighth 11 / 15 / 13.  (Listing 1024 blocks takes longer than the merge of few heads in L2: half of the
+// blocks of 8 heads x 1024 of 64 x 64 22 / 34 / 18.)
+// O may be O_a or O_b and lse may be lse_a or lse_b (no pointer is declared restrict): a thread reads the 16 bytes it
+// later writes, and the D/8 threads of a row are consecutive lanes of one warp, all of which have read the row's
+// log-sum-exp values before its first thread writes the merged one.
 // A row to which the second part adds nothing (lse_b = -inf: no kept block in this hop) has nothing to do when it is
 // merged in place.
 constexpr int kMergeThreads = 256;
-constexpr int kMergeRows = 4;
+constexpr int merge_ctas_per_sm(int rows) { return rows == 2 ? 6 : 3; }
 
-template <int D>
-__global__ void __launch_bounds__(kMergeThreads) attn_merge_kernel(const __nv_bfloat16* Oa, const float* la,
-                                                                   const __nv_bfloat16* Ob, const float* lb,
-                                                                   __nv_bfloat16* O, float* lse, int B, int H, int NB,
-                                                                   int64_t N, int b, int64_t sB, int64_t sH, int64_t sT,
-                                                                   const int32_t* __restrict__ rank, int consumer,
-                                                                   int head_begin, int head_end) {
+template <int D, int kMergeRows>
+__global__ void __launch_bounds__(kMergeThreads, merge_ctas_per_sm(kMergeRows))
+    attn_merge_kernel(const __nv_bfloat16* Oa, const float* la, const __nv_bfloat16* Ob, const float* lb,
+                      __nv_bfloat16* O, float* lse, int B, int H, int NB, int64_t N, int b, int64_t sB, int64_t sH,
+                      int64_t sT, const int32_t* __restrict__ rank, int consumer, int head_begin, int head_end) {
   enter_grid(rank);
   constexpr int VPR = D / 8;
   constexpr int kPass = kMergeThreads / VPR;  // rows per pass of the CTA
@@ -150,8 +153,8 @@ int launch_hop_mask(const Geometry& g, const uint32_t* mask, const int32_t* rank
   int width = 1;
   while (width < g.Wd) width <<= 1;
   const int per_cta = kHopThreads / width * kHopRows;
-  SPARSP_CUDA_OK(launch_kernel(hop_mask_kernel, (unsigned)((n_rows + per_cta - 1) / per_cta), kHopThreads, 0, st, 
-      mask, rank, g.H, g.NB, g.Wd, n_rows, consumer, producer, head_begin, head_end, hop));
+  SPARSP_CUDA_OK(launch_kernel(hop_mask_kernel, (unsigned)((n_rows + per_cta - 1) / per_cta), kHopThreads, 0, st, mask,
+                               rank, g.H, g.NB, g.Wd, n_rows, consumer, producer, head_begin, head_end, hop));
   return SPARSP_OK;
 }
 
@@ -162,11 +165,17 @@ int launch_attn_merge(const sparsp_shape& s, const Geometry& g, const void* Oa, 
   int dev = 0, sms = 148;
   SPARSP_CUDA_OK(cudaGetDevice(&dev));
   SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const unsigned grid = (unsigned)std::min<int64_t>((int64_t)g.B * (head_end - head_begin) * g.NB, 4LL * sms);
-  auto kern = g.d == 64 ? attn_merge_kernel<64> : attn_merge_kernel<128>;
-  SPARSP_CUDA_OK(launch_kernel(kern, grid, kMergeThreads, 0, st, (const __nv_bfloat16*)Oa, la, (const __nv_bfloat16*)Ob, lb, (__nv_bfloat16*)O, lse,
-                                       g.B, g.H, g.NB, g.N, g.b, s.stride_batch, s.stride_head, s.stride_token, rank,
-                                       consumer, head_begin, head_end));
+  const int rows = g.d == 64 && g.b == 64 ? 2 : 4;
+  auto kern = g.d == 128 ? attn_merge_kernel<128, 4> : rows == 2 ? attn_merge_kernel<64, 2> : attn_merge_kernel<64, 4>;
+  const int64_t units = (int64_t)g.B * (head_end - head_begin) * g.NB;
+  // Walkers: as many CTAs as fit the chip (twice as many: half of the blocks of 8 heads x 1024 of 64 x 64 22.8 us for
+  // 21.9); in the four-row form twice as many (an attention of 40 heads x 75600 hop by hop 3.00 ms, as many 3.07, four
+  // times 3.045).
+  const int64_t walkers = (rows == 2 ? 1LL : 2LL) * merge_ctas_per_sm(rows) * sms;
+  const unsigned grid = (unsigned)(rank ? std::min(units, walkers) : units);
+  SPARSP_CUDA_OK(launch_kernel(kern, grid, kMergeThreads, 0, st, (const __nv_bfloat16*)Oa, la, (const __nv_bfloat16*)Ob,
+                               lb, (__nv_bfloat16*)O, lse, g.B, g.H, g.NB, g.N, g.b, s.stride_batch, s.stride_head,
+                               s.stride_token, rank, consumer, head_begin, head_end));
   return SPARSP_OK;
 }
 
