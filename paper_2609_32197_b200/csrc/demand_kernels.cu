@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
 
 // Pack-order offsets, and where every packed tile goes.  A CTA per consumer scans its consumer's counts in pack
 // order (producer, then head) and writes offsets, total and volume.  With `dst` given there are consumers + batch items
-// CTAs per head: CTA (consumer, h) also fills its column of the destination table
+// CTAs per `heads` heads: CTA (consumer, h) also fills its column of the destination table
 //   dst[(b*H + h)*NB + j][r] = byte offset in `packed` of consumer r's copy of block j, or -1
 // one warp per producer (the consumer's base is its caller-given dst_base or the sum of `received` over all earlier
 // consumers), and CTA (B*P + b, h) appends the blocks that any consumer of batch item b receives to the list of
@@ -81,7 +81,13 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
 // on 24 heads, 8 ranks, 18 + 4 us on 48 heads; offsets alone 2 us now, with destinations 9 us on 48 and 15 us on 24
 // heads; eight heads to a CTA, one warp each: 16-19 us.  Union, plan and an empty gather at the limit, 16 batch items x
 // 64 ranks x 24 heads: 0.55 ms; 72 ms with the sum over the counts of every producer, 2.9 ms with the serial scan.)
+// A CTA takes one head up to 64 heads, and so many beyond that there are about 64 CTAs per consumer: the scans repeated
+// per head would grow with the square of the heads (plan and gather of 2000 heads x 4 blocks, 8 ranks: 184 us, 1447
+// with a head per CTA, 731 with the serial scan; 300 heads x 20 blocks 34, 63 and 122).
 constexpr int kPlanThreads = 256;
+constexpr int kPlanMaxHeads = 32;
+
+static int plan_heads(int H) { return H <= 64 ? 1 : std::min(kPlanMaxHeads, (H + 63) / 64); }
 
 __device__ __forceinline__ int64_t block_sum(int64_t v, int64_t* warp_s) {
 #pragma unroll
@@ -97,40 +103,42 @@ __device__ __forceinline__ int64_t block_sum(int64_t v, int64_t* warp_s) {
 
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(
     const int32_t* __restrict__ cnt, const int32_t* __restrict__ received, const uint32_t* __restrict__ U,
-    const int32_t* __restrict__ rank, int BP, int H, int NB, int Wd, int P, int include_local, int64_t entry_bytes,
-    int64_t* __restrict__ seg_off, int64_t* __restrict__ seg_total, int64_t* __restrict__ volume,
-    const int64_t* __restrict__ dst_base, int64_t capacity, int64_t* __restrict__ dst, int32_t* __restrict__ src,
-    int32_t* __restrict__ n_src, int32_t* __restrict__ status) {
+    const int32_t* __restrict__ rank, int BP, int H, int heads, int NB, int Wd, int P, int include_local,
+    int64_t entry_bytes, int64_t* __restrict__ seg_off, int64_t* __restrict__ seg_total,
+    int64_t* __restrict__ volume, const int64_t* __restrict__ dst_base, int64_t capacity, int64_t* __restrict__ dst,
+    int32_t* __restrict__ src, int32_t* __restrict__ n_src, int32_t* __restrict__ status) {
   enter_grid(cnt, received, U, rank, dst_base);
   __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
-  __shared__ int64_t seg_s[kMaxRanks];  // first entry of (producer, my head)
+  extern __shared__ int64_t seg_s[];  // [heads][P] first entry of (my head, producer)
   __shared__ int64_t warp_s[kPlanThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int n_x = BP + (dst ? BP / P : 0), x = blockIdx.x % n_x, h = blockIdx.x / n_x;
+  const int n_x = BP + (dst ? BP / P : 0), x = blockIdx.x % n_x;
+  const int h0 = blockIdx.x / n_x * heads, h1 = min(h0 + heads, H);  // my heads
   if (dst) own_words(rank, NB, Wd, P, own_s);
-  if (x >= BP) {  // the blocks of this head that any consumer receives
+  if (x >= BP) {  // the blocks of my heads that any consumer receives, a warp per head
     __syncthreads();
-    if (warp != 0) return;
     const int bb = x - BP;
-    uint32_t live = 0, owned = 0;
-    if (lane < Wd) {
-      for (int p = 0; p < P; ++p) owned |= own_s[p * Wd + lane];
+    for (int h = h0 + warp; h < h1; h += kPlanThreads / 32) {
+      uint32_t live = 0, owned = 0;
+      if (lane < Wd) {
+        for (int p = 0; p < P; ++p) owned |= own_s[p * Wd + lane];
 #pragma unroll 8
-      for (int r = 0; r < P; ++r)
-        live |= U[((int64_t)(bb * P + r) * H + h) * Wd + lane] &
-                (include_local ? owned : owned & ~own_s[r * Wd + lane]);
+        for (int r = 0; r < P; ++r)
+          live |= U[((int64_t)(bb * P + r) * H + h) * Wd + lane] &
+                  (include_local ? owned : owned & ~own_s[r * Wd + lane]);
+      }
+      int total, first = 0;
+      int at = bits_below(live, lane, &total);
+      if (lane == 0) first = atomicAdd(n_src, total);
+      at += __shfl_sync(0xffffffffu, first, 0);
+      for (; live; live &= live - 1) src[at++] = (bb * H + h) * NB + lane * 32 + __ffs(live) - 1;
     }
-    int total, first = 0;
-    int at = bits_below(live, lane, &total);
-    if (lane == 0) first = atomicAdd(n_src, total);
-    at += __shfl_sync(0xffffffffu, first, 0);
-    for (; live; live &= live - 1) src[at++] = (bb * H + h) * NB + lane * 32 + __ffs(live) - 1;
     return;
   }
 
   const int br = x, bb = br / P, r = br % P;
   const int PH = P * H;
-  const bool writer = h == 0;
+  const bool writer = h0 == 0;
   const int32_t* mine = cnt + (int64_t)br * PH;
   int64_t cursor = 0, remote = 0;  // entries of earlier chunks of this consumer
   for (int i0 = 0; i0 < PH; i0 += kPlanThreads) {
@@ -158,7 +166,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(
     if (i < PH) {
       const int64_t at = cursor + before + incl - counted;
       if (writer) seg_off[(int64_t)br * PH + i] = at;
-      if (i - p * H == h) seg_s[p] = at;
+      const int h = i - p * H;
+      if (h >= h0 && h < h1) seg_s[(h - h0) * P + p] = at;
     }
     cursor += all;
   }
@@ -179,21 +188,22 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(
     for (int k = threadIdx.x; k < br * H; k += kPlanThreads) n += received[k];
     base = entry_bytes * block_sum(n, warp_s);
   }
-  __syncthreads();
-  int64_t* out = dst + (int64_t)(bb * H + h) * NB * P + r;
-  const uint32_t u = lane < Wd ? U[((int64_t)br * H + h) * Wd + lane] : 0u;
-  for (int j = threadIdx.x; j < NB; j += kPlanThreads) out[(int64_t)j * P] = -1;
-  __syncthreads();
-  for (int p = warp; p < P; p += kPlanThreads / 32) {
-    if (p == r && !include_local) continue;
-    uint32_t bits = lane < Wd ? u & own_s[p * Wd + lane] : 0u;
-    int total;
-    int64_t byte = base + (seg_s[p] + bits_below(bits, lane, &total)) * entry_bytes;
-    for (; bits; bits &= bits - 1, byte += entry_bytes) {
-      if (capacity >= 0 && byte + entry_bytes > capacity) {
-        atomicExch(status, SPARSP_ERR_CAPACITY);  // would overflow: stays -1, the gather leaves it out
-      } else {
-        out[(int64_t)(lane * 32 + __ffs(bits) - 1) * P] = byte;
+  for (int h = h0; h < h1; ++h) {
+    int64_t* out = dst + (int64_t)(bb * H + h) * NB * P + r;
+    const uint32_t u = lane < Wd ? U[((int64_t)br * H + h) * Wd + lane] : 0u;
+    for (int j = threadIdx.x; j < NB; j += kPlanThreads) out[(int64_t)j * P] = -1;
+    __syncthreads();
+    for (int p = warp; p < P; p += kPlanThreads / 32) {
+      if (p == r && !include_local) continue;
+      uint32_t bits = lane < Wd ? u & own_s[p * Wd + lane] : 0u;
+      int total;
+      int64_t byte = base + (seg_s[(h - h0) * P + p] + bits_below(bits, lane, &total)) * entry_bytes;
+      for (; bits; bits &= bits - 1, byte += entry_bytes) {
+        if (capacity >= 0 && byte + entry_bytes > capacity) {
+          atomicExch(status, SPARSP_ERR_CAPACITY);  // would overflow: stays -1, the gather leaves it out
+        } else {
+          out[(int64_t)(lane * 32 + __ffs(bits) - 1) * P] = byte;
+        }
       }
     }
   }
@@ -219,10 +229,11 @@ static cudaError_t launch_plan(const Geometry& g, const uint32_t* mask, const in
   cudaError_t e = launch_kernel(union_count_kernel, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P,
                                 U, include_local, cnt, received, n_src);
   if (e != cudaSuccess) return e;
-  const unsigned grid = dst ? (unsigned)((g.B * P + g.B) * g.H) : (unsigned)(g.B * P);
-  return launch_kernel(plan_kernel, grid, kPlanThreads, 0, st, cnt, received, U, rank, g.B * P, g.H, g.NB, g.Wd, P,
-                       include_local, 2LL * g.b * g.d * 2, seg_off, seg_total, volume, dst_base, capacity, dst, src,
-                       n_src, status);
+  const int heads = dst ? plan_heads(g.H) : 1;
+  const unsigned grid = dst ? (unsigned)((g.B * P + g.B) * ((g.H + heads - 1) / heads)) : (unsigned)(g.B * P);
+  return launch_kernel(plan_kernel, grid, kPlanThreads, (size_t)heads * P * 8, st, cnt, received, U, rank, g.B * P, g.H,
+                       heads, g.NB, g.Wd, P, include_local, 2LL * g.b * g.d * 2, seg_off, seg_total, volume, dst_base,
+                       capacity, dst, src, n_src, status);
 }
 
 int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_of_block, int P,

@@ -196,9 +196,8 @@ static cudaError_t launch_score(const Geometry& g, const float* pq, const float*
 // ballot-prefix compaction.  Bound by instruction issue, a compare and an add per key and step: instances for several
 // row lengths. 24 x 384 rows of 384: 19 us, 40 x 591 of 591: 79 us, 24 x 929 of 929: 136 us (29, 152 and 194 us with 32
 // steps of one bit each and instances of 4, 8, 16 and 32 words; bisection by the keys instead of the scores: 18, 71 and
-// 212 us).  Four CTAs per SM
-// although the instances of 24 and 32 words spill for it: pool, score and selection of 24 x 929 rows 273 us, 296 with
-// three and 340 with two; of 40 x 700 rows 267, 284 and 285.
+// 212 us).  Four CTAs per SM although the instances of 24 and 32 words spill for it: pool, score and selection of 24 x
+// 929 rows 273 us, 296 with three and 340 with two; of 40 x 700 rows 267, 284 and 285.
 // ------------------------------------------------------------------------------------------------
 constexpr int kTopkWarps = 8;
 

@@ -1,4 +1,4 @@
-"""Planning and packing at the largest accepted batch * ranks: 16 batch items of 64 ranks."""
+"""Planning and packing at the largest accepted batch * ranks, 16 batch items of 64 ranks, and with many heads."""
 import pytest
 import torch
 
@@ -13,15 +13,17 @@ def binding():
 
 
 @pytest.mark.parametrize("local", [False, True])
-@pytest.mark.parametrize("H,NB", [(24, 64), (3, 97)])
-def test_plan_and_bytes_at_the_limit(binding, local, H, NB):
+@pytest.mark.parametrize("B,P,H,NB,limit_ms", [(16, 64, 24, 64, 2.0), (16, 64, 3, 97, 2.0), (3, 64, 130, 5, 2.0),
+                                               (2, 3, 64, 33, 2.0), (2, 3, 65, 33, 2.0), (1, 8, 2000, 4, 0.4)])
+def test_plan_and_bytes_at_the_limit(binding, local, B, P, H, NB, limit_ms):
     """Every table against the definitions in tensor form, and the time of the call with destinations: the plan's CTAs (25
-    thousand at 24 heads) read the entries of the consumers before theirs per head, not per producer and head."""
-    B, P, b, d = 16, 64, 64, 64
+    thousand at 16 x 64 x 24) read the entries of the consumers before theirs per head, not per producer and head, and a CTA
+    that scans a consumer's counts does so for a group of heads where there are many."""
+    b, d = 64, 64
     N = NB * b - 7
     g = torch.Generator(device="cuda").manual_seed(H)
     K, V = (torch.randn(B, H, N, d, device="cuda", generator=g).to(torch.bfloat16) for _ in range(2))
-    M = torch.rand(B, H, NB, NB, device="cuda", generator=g) < 0.03
+    M = torch.rand(B, H, NB, NB, device="cuda", generator=g) < (0.03 if NB > 10 else 0.2)
     rank = torch.randint(0, P, (NB,), device="cuda", generator=g, dtype=torch.int32)
     shape = binding.make_shape(H, d, (1, 1, N), 0, b, batch=B)
     ws = binding.make_workspace(shape, P)
@@ -71,5 +73,5 @@ def test_plan_and_bytes_at_the_limit(binding, local, H, NB):
         end.record()
         torch.cuda.synchronize()
         times.append(start.elapsed_time(end))
-    # a read and a write of every packed byte at 1 TB/s, and 2 ms for the tables
-    assert min(times) < 2.0 + 2 * packed.numel() / 1e9, times
+    # a read and a write of every packed byte at 1 TB/s, and some time for the tables
+    assert min(times) < limit_ms + 2 * packed.numel() / 1e9, times
