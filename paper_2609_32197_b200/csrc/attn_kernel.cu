@@ -572,9 +572,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       };
       // When the next item is taken: for stacked items of a packed source with d = 128, whose lists are short and slow
       // to build, right after the list before it, while its buffer is still in use (24 heads x 24576, 4 ranks: one call
-      // 434 us against 483, with a shuffled placement 421 against 462, hop by hop 796 against 811; 12 heads x 9504: 64.5
-      // against 66.4).  Everywhere else once there is a buffer for it: an item taken early is one that a CTA with nothing
-      // left to do cannot take (packed source, d = 64, 24 heads x 24576: one call 339 us against 345-358 early, hop by
+      // 434 us against 483, with a shuffled placement 421 against 462, hop by hop 796 against 811; 12 heads x 9504:
+      // 64.5 against 66.4).  Everywhere else once there is a buffer for it: an item taken early is one that a CTA with
+      // nothing left to do cannot take (packed source, d = 64, 24 heads x 24576: one call 339 us against 345-358 early, hop by
       // hop 641 against 654; 48 heads x 17776, 8 ranks: 265 against 271-280; K / V source, 26 heads x 6034 and 40 heads
       // x 75600 hop by hop: 3 % slower early).
       constexpr bool kEarly = kPacked && C::kStacked && D == 128;
@@ -1053,11 +1053,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 // typically the same position a fixed number of blocks away; the more two stacked blocks share, the less of a 128-row
 // tile's work is masked away.
 // Packed source: neighbours in the consumer's ascending list of blocks (D = 1).  Its rows take their reference from the
-// first tiles, and neighbours keep each other's blocks: there a row nearly always meets its largest score at once,
-// whose exponential is then exactly 1.  Chosen by overlap the partner is far away, the largest term is some rounded
-// 2^x, and the output is further from 64 bits (24 heads x 24576, 4 ranks: 2.01e-3 against 1.95e-3, log-sum-exp 3.7e-4
-// against 3.2e-4). (Mask rows in shared memory have an odd pitch: the threads' offsets differ by one row, a pitch of 32
-// words would put them all on one bank.)
+// first tiles, and the blocks that two neighbours both keep, which come first, are on video inputs little more than the
+// two themselves: a row meets its largest score at once, whose exponential is then exactly 1.  Chosen by overlap the
+// partner is far away, the largest term is some rounded 2^x, and the output is further from 64 bits (24 heads x 24576,
+// 4 ranks: 2.01e-3 against 1.95e-3, log-sum-exp 3.7e-4 against 3.2e-4; 347 us against 433).
+// (Mask rows in shared memory have an odd pitch: the threads' offsets differ by one row, a pitch of 32 words would put
+// them all on one bank.)
 // Items of one (batch, head) are handed out longest list first: the items still running when the queue
 // runs dry are then the short ones, which matters when list lengths vary (threshold selection, unions of two
 // stacked blocks).  Key = (list length << 10) | (1023 - index): equal lengths keep their index order.
