@@ -17,26 +17,26 @@
 //   warp 0      TMA producer of Q (per item) and of the K ring
 //   warp 1      issues every Q K^T          warp 2      issues every P V
 //   warp 3      TMA producer of the V ring
-//   warp 4      builds the kept / union list of the NEXT items (two list buffers; warps 5-7 idle)
+//   warp 4      builds the kept / union list of the NEXT items (two list buffers)
+//   warps 5-7   clear the output rows of query blocks that keep nothing
 //   warps 8-11  softmax of the even tiles   warps 12-15 softmax of the odd tiles
 // (A producer is one thread running a chain of dependent instructions next to busy softmax warps: it gets
 // an instruction issued every ~8 cycles, so K and V loads have a warp each and keep per-tile work minimal.)
-// A softmax thread owns one query row of its tile: the whole 128-column row of S sits in registers.  The
-// two threads that own the same row (one per warpgroup) share the row's reference maximum through shared
-// memory and take their decisions strictly in tile order (a pair of 64-thread named barriers per row
-// group hands the turn back and forth); each keeps its own partial row sum.
-// Online softmax is base-2 in fp32; O is rescaled lazily, only when a row's maximum has grown by more
-// than 2^8 since the reference last moved -- the thread that decides so first waits for every P V
-// issued so far, then rescales the row of O.
-// Norm bounds shorten most tiles: |q_row| * (largest key norm of a block) * scale bounds the block's scores, so
-// a tile whose bound stays within 2^64 of the row's reference skips its row-maximum pass, and once the bound
-// with the item's largest key norm holds, the reference is final and the two warps of a row group stop taking
-// turns for the rest of the item (load scores -> exponentials -> store P).
-// And if that bound is at most 2^80 in absolute terms -- ordinary inputs -- the item needs no reference at all: every
-// softmax thread takes its row's norm from the Q tile while the first Q K^T runs, and an item whose bounds hold runs
-// on the fixed reference 0 from its first tile on.
-// The block-64 pairing and the order of a head's items (longest list first) come from attn_prep_kernel,
-// which also takes the key norms.
+// A softmax thread owns one query row of its tile: the whole 128-column row of S sits in registers.  Ordinary items run
+// without a row maximum: load scores -> exponentials -> store P, relative to 0 (K / V source) or to the row's maximum
+// over the item's first tile (packed source), which the warpgroup of that tile hands to the other one; the tensor pipe
+// takes the row sums.  Whether that was right is seen from the finished row sums and the exponents on the way, and an
+// item that left the range is computed again (kRefZero ... below).  Only an item that fails relative to its first tile as
+// well takes its maxima as it goes: the two threads that own the same row (one per warpgroup) then share the reference
+// through shared memory and take their decisions strictly in tile order (a pair of 64-thread named barriers per row group
+// hands the turn back and forth), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since
+// the reference last moved -- the thread that decides so first waits for every P V issued so far.
+// (The range used to be proved beforehand, by Cauchy-Schwarz from key norms that a pass over K took ahead of every call
+// and row norms taken from the Q tile of every item, and not at all for a packed source, whose tiles all took their
+// maximum in turns.  us per call then and now: one hop of 40 heads x 75600 over 8 ranks, 7 tiles an item, 97-112 -> 75;
+// 24 x 24576 from one rank's whole buffer 437-445 -> 415-425; 13 heads x 2 x 6034 92-101 -> 85-93; all of 40 x 75600
+// 10.1-10.5 -> 9.7-10.2 ms.)
+// The block-64 pairing and the order of a head's items (longest list first) come from attn_prep_kernel.
 // Every mbarrier wait is bounded; a wait that runs out sets SPARSP_ERR_TIMEOUT in the status word
 // and raises a CTA-wide flag that makes all later waits fall through, so the CTA still drains.
 #include <algorithm>
@@ -62,9 +62,8 @@ struct AttnParams {
   // consumer's first tile in the packed tensor map (a device scalar)
   const int32_t* slot;
   const int64_t* tile_base;
-  // K / V source only: largest key norm (L2) of every KV block that any row keeps, [B*H][NB]: lets a softmax row skip
-  // the row-maximum pass of a tile whose scores provably stay within 2^kSkipMargin of the row's reference maximum
-  const float* knorm;
+  const int32_t* rank;  // packed source: owner of every block, and the rank whose rows are computed
+  int consumer;
   __nv_bfloat16* O;
   float* lse;
   int32_t* status;
@@ -77,30 +76,38 @@ struct AttnParams {
 };
 
 constexpr int kAttnThreads = 512;  // four warpgroups: two of utility warps, softmax of the even tiles, softmax of the odd tiles
-// register budget per thread after the warpgroups re-balance (128*48 + 128*32 + 256*216 = 512*128)
+// register budget per thread after the warpgroups re-balance (2*128*48 + 256*208 = 512*128; nothing spills in the softmax
+// warps, and the list builder, which spilled with 32, hardly does)
 #ifndef SPARSP_REGS_UTILITY
 #define SPARSP_REGS_UTILITY 48
-#define SPARSP_REGS_UTILITY2 32
-#define SPARSP_REGS_SOFTMAX 216
+#define SPARSP_REGS_UTILITY2 48
+#define SPARSP_REGS_SOFTMAX 208
 #endif
 constexpr int kTmemCols = 512;
 constexpr int kWorkCounterWord = 8;  // word of the workspace header that holds the attention work counter
 constexpr float kGrowThreshold = 8.0f;
-constexpr float kSkipMargin = 64.0f;  // 2^64 * (keys of a sequence) * |V| stays far inside fp32
-// If |q_row| * (largest key norm of the item) * scale * log2(e) <= kStaticBound for all rows of a warp, every score of
-// the item lies in [-kStaticBound, kStaticBound] (log2 domain) and the fixed reference 0 serves the whole item:
-// exponentials between 2^-80 and 2^80 are normal numbers in fp32 and bf16 with full relative precision, and
-// 2^80 * (keys of a sequence) * |V| stays inside fp32.
-constexpr float kStaticBound = 80.0f;
+// Where an item's softmax rows take the reference that is subtracted from their scores (log2 domain) from:
+//   kRefZero   nowhere, it is 0;
+//   kRefFirst  the row's maximum over the item's first tile (0 for a row that keeps nothing of it);
+//   kRefWide   the same, with exponents below the range raised to its lower end;
+//   kRefExact  the row's running maximum, moved lazily and strictly in tile order.
+// The first three never look at another score, so they are right only for rows whose scores stay near the reference.
+// That is seen at the end of the item: no exponential left the range of normal numbers on the FMA pipe (kMaxExponent;
+// the special-function unit saturates to 0 and infinity by itself), and the row sum lies within [kMinSum, kMaxSum].
+// Then every term is a normal fp32 and bf16 number of full relative precision, or at most 2^-36 of the sum, and
+// kMaxSum * |V| is far inside fp32.  An item with a row that fails, one with scores that are no numbers included, is
+// computed again, as kRefWide and then as kRefExact (at once where the range was missed by far), and the later items of
+// its CTA start one kind further on.  Ordinary scores pass: with unit-variance
+// Q and K at d = 128 they are within +-16.
+constexpr int kRefZero = 0, kRefFirst = 1, kRefWide = 2, kRefExact = 3;
+constexpr float kMaxExponent = 126.0f;
+constexpr float kMinSum = 8.077935669463161e-28f;  // 2^-90
+constexpr float kMaxSum = 1.2676506002282294e30f;  // 2^100
+constexpr int kZeroMinTiles = 4;  // K / V source: shorter items take kRefFirst, whose largest terms are exact
 // Tuning switch (compile-time): how many of the exponentials go to the FMA pipe instead of the
 // special-function unit (every n-th pair; 0 = none).
 #ifndef SPARSP_TUNE_POLY
 #define SPARSP_TUNE_POLY 3
-#endif
-// d = 128: take the row sum on the tensor pipe as well (an extra N = 16 MMA per 16 keys against a small block of
-// ones), at the price of the second P buffer, whose tensor-memory columns the 16 sum columns need (1 = on)
-#ifndef SPARSP_SUM_MMA_128
-#define SPARSP_SUM_MMA_128 1
 #endif
 // ... at d = 64 (measured there: every 3rd pair is 3 % faster than every 4th, every 2nd 4 % slower; at d = 128, with the
 // row sum on the tensor pipe, every 3rd is 1-2 % faster than every 4th and every 2nd 2 % slower)
@@ -128,18 +135,15 @@ struct AttnCfg {
   // d = 128: the row sum also comes from the tensor pipe, through a separate N = 16 MMA per 16
   // keys against a [16 keys][column 0 = 1] block (2 KB, 128-byte swizzle like a V box), into 16 tensor-memory columns
   // of its own -- which exist only if P keeps ONE buffer instead of two (tensor memory is full otherwise)
-  static constexpr bool kSum128 = (D == 128 && SPARSP_SUM_MMA_128 != 0);
-  static constexpr bool kSumMma = kOnes || kSum128;  // the softmax warps keep no row sums
+  static constexpr bool kSum128 = (D == 128);
   static constexpr int kNumP = kSum128 ? 1 : 2;
   static constexpr int kOffOnes = kOffV + kStagesV * kTileBytes;  // bf16 [128][64], 128-byte swizzle like a V box
-  static constexpr int kOffEntJ = kOffOnes + (kOnes ? 128 * 128 : (kSum128 ? 2048 : 0));  // uint16 [2][1024] kept / union list
+  static constexpr int kOffEntJ = kOffOnes + (kOnes ? 128 * 128 : 2048);  // uint16 [2][1024] kept / union list
   static constexpr int kOffEntV = kOffEntJ + 2 * 2 * kMaxBlocks;  // uint8 [2][1024][2] keys of the entry valid for query block q (0 = not kept)
   static constexpr int kOffSlot = kOffEntV + 2 * 2 * kMaxBlocks;  // int32 [2][1024] packed-buffer slot per entry
-  static constexpr int kOffEntN = kOffSlot + 2 * 4 * kMaxBlocks;  // float [2][1024] largest key norm of the entry's block
-  static constexpr int kOffStat = kOffEntN + 2 * 4 * kMaxBlocks;  // float2 [2 items][2 warpgroups][128]
-  static constexpr int kOffRef = kOffStat + 2 * 2 * 128 * 8;      // float [3 items][128] reference maximum per row
-  static constexpr int kOffBars = kOffRef + 3 * 128 * 4;
-  static constexpr int kNumBars = 2 + 2 * (kStagesK + kStagesV) + 10 + 1 + 4;
+  static constexpr int kOffRef = kOffSlot + 2 * 4 * kMaxBlocks;  // float [4 items][128] reference per row
+  static constexpr int kOffBars = kOffRef + 4 * 128 * 4;
+  static constexpr int kNumBars = 2 + 2 * (kStagesK + kStagesV) + 10 + 1 + 4 + 4;
   static constexpr int kColS = 0;    // S buffers: columns [0, 256)
   static constexpr int kColP = 256;  // P: two buffers in columns [256, 384), or one in [256, 320) with the row sums in [320, 336)
   static constexpr int kColO = 384;  // accumulator: columns [384, 384 + d)
@@ -171,15 +175,27 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
   return d;
 }
 
+// max(|a|, |b|, |c|), not a number if any of them is none.
+__device__ __forceinline__ float max_abs3(float a, float b, float c) {
+  float d;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // 2^x for a pair of fp32 values on the FMA/ALU pipes (no special-function unit): round-to-nearest
 // split x = i + f, f in [-0.5, 0.5], cubic minimax polynomial for 2^f (relative error 7.5e-5, far
-// below bf16 rounding), exponent added into the bit pattern.  x is clamped at -126 (result >= 2^-126).
-__device__ __forceinline__ float2 exp2_poly2(float2 x) {
+// below bf16 rounding), exponent added into the bit pattern.  The result is right for |i| <= 126; *i_max collects the
+// largest |i|.  kClamp: x is clamped at -126 first (result >= 2^-126).
+template <bool kClamp>
+__device__ __forceinline__ float2 exp2_poly2(float2 x, float* i_max) {
   const float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
-  x.x = fmaxf(x.x, -126.0f);
-  x.y = fmaxf(x.y, -126.0f);
+  if (kClamp) {
+    x.x = fmaxf(x.x, -126.0f);
+    x.y = fmaxf(x.y, -126.0f);
+  }
   const float2 t = fadd2(x, make_float2(kMagic, kMagic));
   const float2 fi = fadd2(t, make_float2(-kMagic, -kMagic));
+  *i_max = max_abs3(fi.x, fi.y, *i_max);
   const float2 f = fadd2(x, make_float2(-fi.x, -fi.y));
   float2 q = ffma2(f, make_float2(0.0551716685f, 0.0551716685f), make_float2(0.2426111251f, 0.2426111251f));
   q = ffma2(q, f, make_float2(0.6932609677f, 0.6932609677f));
@@ -187,6 +203,21 @@ __device__ __forceinline__ float2 exp2_poly2(float2 x) {
   q.x = __int_as_float(__float_as_int(q.x) + (__float_as_int(t.x) << 23));
   q.y = __int_as_float(__float_as_int(q.y) + (__float_as_int(t.y) << 23));
   return q;
+}
+
+// The output rows of query block i: zeros and a log-sum-exp of -inf.  One warp.
+template <int D, int BLK>
+__device__ __forceinline__ void clear_rows(const AttnParams& p, int64_t bh, int i) {
+  constexpr int LPT = D / 8;  // lanes per row
+  const int lane = threadIdx.x & 31;
+  const int64_t tok0 = (int64_t)i * BLK;
+  const int n = (int)min((int64_t)BLK, p.N - tok0);
+  __nv_bfloat16* o = p.O + (bh / p.H) * p.sB + (bh % p.H) * p.sH + tok0 * p.sT + (lane % LPT) * 8;
+#pragma unroll 4
+  for (int r = lane / LPT; r < n; r += 32 / LPT)
+    *reinterpret_cast<uint4*>(o + (int64_t)r * p.sT) = make_uint4(0u, 0u, 0u, 0u);
+  if (p.lse)
+    for (int r = lane; r < n; r += 32) p.lse[bh * p.N + tok0 + r] = -INFINITY;
 }
 
 __device__ __forceinline__ void named_bar_sync(int id, int n) {
@@ -209,9 +240,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   uint16_t* sEntJ = reinterpret_cast<uint16_t*>(smem + C::kOffEntJ);  // [2][kMaxBlocks]
   uint8_t* sEntV = smem + C::kOffEntV;                                // [2][kMaxBlocks][2]
   int32_t* sSlot = reinterpret_cast<int32_t*>(smem + C::kOffSlot);    // [2][kMaxBlocks]
-  float* sEntN = reinterpret_cast<float*>(smem + C::kOffEntN);        // [2][kMaxBlocks]
-  float2* sStat = reinterpret_cast<float2*>(smem + C::kOffStat);      // [2][2][128]
-  volatile float* sRef = reinterpret_cast<volatile float*>(smem + C::kOffRef);  // [3][128]
+  volatile float* sRef = reinterpret_cast<volatile float*>(smem + C::kOffRef);  // [4][128]
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kOffBars);
   uint64_t* q_full = bars;          // the item's Q tile has landed
   uint64_t* q_free = bars + 1;      // every Q K^T of the item has completed: Q may be overwritten
@@ -229,15 +258,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   uint64_t* o_drained = o_full + 4;      // the item's accumulator has been read out by all 8 softmax warps
   uint64_t* list_ready = o_drained + 1;  // [2] list buffer filled
   uint64_t* list_free = list_ready + 2;  // [2] list buffer no longer needed by its kListReaders
+  // [4] the four warps that own an item's first tile have left the reference that it gives in sRef.  Four, because
+  // the other warpgroup, which waits for it, may be up to three tiles and as many items behind.
+  uint64_t* ref_ready = list_free + 2;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
   int* s_nent = reinterpret_cast<int*>(smem + C::kOffMisc + 8);   // [2]
   int* s_blk = reinterpret_cast<int*>(smem + C::kOffMisc + 16);   // [2][2] the item's query block(s); < 0 = absent
   int* s_item = reinterpret_cast<int*>(smem + C::kOffMisc + 32);  // [2] batch * H + head of each list buffer; < 0: none
   int* s_rag = reinterpret_cast<int*>(smem + C::kOffMisc + 40);   // [2] the item's last tile reaches past the end of the sequence
-  volatile int* s_frz = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 56);  // [4] per row group: reference frozen
-  volatile int* s_pv_items = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 72);  // items whose P V are all issued
-  float* s_knmax = reinterpret_cast<float*>(smem + C::kOffMisc + 48);  // [2] largest key norm bound among the item's entries
+  int* s_ref = reinterpret_cast<int*>(smem + C::kOffMisc + 48);   // [2] where the rows' reference comes from
+  int* s_none = reinterpret_cast<int*>(smem + C::kOffMisc + 56);  // [2] bit q: query block q keeps nothing
+  volatile int* s_failed = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 64);  // [2] a row of the item left the range: 1, by far: 2
   constexpr int kListReaders = 12;  // two producers, two issuers, eight softmax warps
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -266,13 +298,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     }
     for (int s = 0; s < 4; ++s) mbar_init(o_full + s, 1);
     mbar_init(o_drained, 8);
+    for (int s = 0; s < 4; ++s) mbar_init(ref_ready + s, 4);
     mbar_init_fence();
     *s_abort = 0;
-    *s_pv_items = 0;
-    for (int r = 0; r < 4; ++r) s_frz[r] = 0;
   }
-  if (tid < 384) sRef[tid] = -INFINITY;  // 3 x 128 entries
-  if (C::kSumMma) {
+  {
     // key row r holds column 64 + c at byte r*128 + ((c/8 ^ (r & 7)) << 4) + (c%8)*2 (the swizzle of a TMA box);
     // 128 key rows at d = 64 (one block for a whole tile), 16 at d = 128 (every group of 16 keys uses the same)
     uint4* ones = reinterpret_cast<uint4*>(smem + C::kOffOnes);
@@ -419,22 +449,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (s_item[buf] < 0) break;
         const int n_tiles = (s_nent[buf] + C::kEPT - 1) / C::kEPT;
         {
-          // The tensor pipe works in issue order.  The first Q K^T of an item could be issued a tile or two
-          // before the previous item ends, ahead of that item's last P V, and the epilogue (which waits for
-          // that P V) would start ~1000 cycles later for nothing: the scores are not needed before the
-          // epilogue is over.  So they wait until the previous item's P V are all issued.
-          if (i > 0) {
-            const long long t0 = clock64();
-            while (*s_pv_items < i) {
-              if (*s_abort) break;
-              if (clock64() - t0 > p.wait_limit) {
-                *s_abort = 14;
-                break;
-              }
-            }
-          }
-          mbar_wait_bounded_inline(q_full, qc & 1, s_abort, 11, p.wait_limit);
-          ++qc;
+          mbar_wait_bounded_inline(q_full, qc++ & 1, s_abort, 11, p.wait_limit);
           for (int n = 0; n < n_tiles; ++n, ++g) {
             mbar_wait_bounded_inline(k_full + g % SK, (g / SK) & 1, s_abort, 12, p.wait_limit);
             // S buffer g%2 is free once the softmax warps have loaded the scores of tile g-2
@@ -499,10 +514,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           }
           __syncwarp();
         }
-        if (lane == 0) {
-          *s_pv_items = i + 1;
-          mbar_arrive(list_free + buf);
-        }
+        if (lane == 0) mbar_arrive(list_free + buf);
         __syncwarp();
       }
     }
@@ -532,6 +544,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       int bh = p.BH, blk0 = -1, blk1 = -1;
       uint32_t rb0 = 0u, rb1 = 0u;  // the item's mask rows, a word per lane (NB <= 1024: at most 32 words)
       // Takes an item: its head (BH = no more items), query block(s) and mask rows.
+      auto load_rows = [&]() {
+        const uint32_t* rows = p.mask + (int64_t)bh * p.NB * p.Wd;
+        rb0 = lane < p.Wd ? rows[blk0 * p.Wd + lane] : 0u;
+        rb1 = lane < p.Wd && blk1 >= 0 ? rows[blk1 * p.Wd + lane] : 0u;
+      };
       auto fetch = [&](int it) {
         int x;
         if (kPacked) {
@@ -561,9 +578,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         const int32_t* items = p.pairs + (int64_t)bh * (2 * ((p.NB + 1) / 2));
         blk0 = C::kStacked ? items[2 * x] : items[x];
         blk1 = C::kStacked ? items[2 * x + 1] : -1;
-        const uint32_t* rows = p.mask + (int64_t)bh * p.NB * p.Wd;
-        rb0 = lane < p.Wd ? rows[blk0 * p.Wd + lane] : 0u;
-        rb1 = lane < p.Wd && blk1 >= 0 ? rows[blk1 * p.Wd + lane] : 0u;
+        load_rows();
       };
       auto next_item = [&]() {
         int it = 0;
@@ -579,21 +594,42 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       // x 75600 hop by hop: 3 % slower early).
       constexpr bool kEarly = kPacked && C::kStacked && D == 128;
       if (kEarly) fetch(blockIdx.x);
+      int kind = kPacked ? kRefFirst : kRefZero;  // what new items take their reference from
       for (int i = 0;; ++i) {
         const int buf = i & 1;
-        if (i >= 2) mbar_wait_bounded_inline(list_free + buf, ((i - 2) >> 1) & 1, s_abort, 50, p.wait_limit);
-        if (!kEarly) fetch(i == 0 ? (int)blockIdx.x : next_item());
-        if (bh >= p.BH || *s_abort) {
+        int again = -1;  // list buffer of an item that failed and is computed again now (rare)
+        if (i >= 2) {
+          mbar_wait_bounded_inline(list_free + buf, ((i - 2) >> 1) & 1, s_abort, 50, p.wait_limit);
+          if (s_failed[buf]) again = buf;
+        }
+        if (again < 0 && !kEarly) fetch(i == 0 ? (int)blockIdx.x : next_item());
+        if (again < 0 && bh >= p.BH && i >= 1) {  // no more items: what became of the last one?
+          mbar_wait_bounded_inline(list_free + (buf ^ 1), ((i - 1) >> 1) & 1, s_abort, 60, p.wait_limit);
+          if (s_failed[buf ^ 1]) again = buf ^ 1;
+        }
+        if (__any_sync(0xffffffffu, *s_abort != 0) || (again < 0 && bh >= p.BH)) {
           if (lane == 0) {
             s_item[buf] = -1;
             mbar_arrive(list_ready + buf);
           }
           break;
         }
+        const int next_bh = bh, next_blk0 = blk0, next_blk1 = blk1;
+        int ref_of = kind;
+        if (again >= 0) {
+          bh = s_item[again];
+          blk0 = s_blk[again * 2];
+          blk1 = s_blk[again * 2 + 1];
+          const bool far = s_failed[again] == 2;
+          ref_of = far ? kRefExact : max(s_ref[again] + 1, kRefWide);
+          kind = far ? kRefExact : min(kind + 1, ref_of);
+          load_rows();
+          __syncwarp();  // (every lane has looked)
+          if (lane == 0) s_failed[again] = 0;
+        }
         uint16_t* entJ = sEntJ + buf * kMaxBlocks;
         uint8_t* entV = sEntV + buf * kMaxBlocks * 2;
         int32_t* entS = sSlot + buf * kMaxBlocks;
-        float* entN = sEntN + buf * kMaxBlocks;
         // Entry order (any order gives the same attention).  Blocks BOTH query blocks keep make full tiles; a
         // block only the first keeps is put next to a block only the second keeps, so that such a tile costs
         // every softmax row one 64-key half instead of costing half of the rows two.  A full tile is bound by
@@ -604,7 +640,36 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         // A mask word at a time, a lane per bit: next to busy softmax warps an instruction of this warp gets issued
         // every several cycles, so the list is as late as it has instructions.
         const uint32_t below = (1u << lane) - 1u;
-        int n_both = 0, n_mix = 0, n_grp = 0, running;
+        // Packed source: the item's own query blocks come first.  There a row meets the largest score that it is likely
+        // to meet, so the reference it takes from the first tile makes that term's exponential exactly 1 (24 heads x
+        // 24576, 4 ranks: 1.87e-3 from 64 bits; 2.00e-3 with the first tile as it comes, 1.95e-3 with a reference that
+        // follows the maximum).
+        int lead = 0, own_of = 0;  // entries ahead of the classes; bit q: one of them is kept by query block q
+        int rag_pos = -1;          // where the sequence's ragged last block went
+        if (kPacked) {
+#pragma unroll
+          for (int q = 0; q < (C::kStacked ? 2 : 1); ++q) {
+            const int j = q ? blk1 : blk0;
+            if (j < 0) continue;
+            const uint32_t f0 = __shfl_sync(0xffffffffu, rb0, j >> 5), f1 = __shfl_sync(0xffffffffu, rb1, j >> 5);
+            const uint32_t f = ((f0 >> (j & 31)) & 1u) | ((f1 >> (j & 31)) & 1u) << 1;
+            if (f == 0u) continue;
+            if (lane == (j >> 5)) {
+              rb0 &= ~(1u << (j & 31));
+              rb1 &= ~(1u << (j & 31));
+            }
+            own_of |= (int)f;
+            const int nvalid = (int)min((int64_t)BLK, p.N - (int64_t)j * BLK);
+            if (lane == 0) {
+              entJ[lead] = (uint16_t)j;
+              entV[lead * 2] = (uint8_t)(f & 1u ? nvalid : 0);
+              entV[lead * 2 + 1] = (uint8_t)(f & 2u ? nvalid : 0);
+            }
+            if (nvalid < BLK) rag_pos = lead;
+            ++lead;
+          }
+        }
+        int n_both = 0, n_mix = 0, n_grp = 0, running, none = 0;
         if (C::kStacked) {
           n_both = __reduce_add_sync(0xffffffffu, __popc(rb0 & rb1));
           const int n0 = __reduce_add_sync(0xffffffffu, __popc(rb0 & ~rb1));
@@ -612,11 +677,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           n_mix = min(n0, n1);
           // two full tiles (four blocks both keep), then two half-work tiles (two one-sided pairs), and so on
           n_grp = min(n_both >> 2, n_mix >> 1);
-          running = n_both + n0 + n1;
+          running = lead + n_both + n0 + n1;
+          none = (n_both + n0 == 0 ? 1 : 0) | (n_both + n1 == 0 ? 2 : 0);
+          none &= ~own_of;
         } else {
-          running = __reduce_add_sync(0xffffffffu, __popc(rb0));
+          running = lead + __reduce_add_sync(0xffffffffu, __popc(rb0));
         }
-        int rag_pos = -1;               // where the sequence's ragged last block went
         int at0 = 0, at1 = 0, at2 = 0;  // entries of each class so far
         for (uint32_t todo = __ballot_sync(0xffffffffu, (rb0 | rb1) != 0u); todo; todo &= todo - 1) {
           const int w = __ffs(todo) - 1;
@@ -638,6 +704,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                 else if (idx < n_mix) pos = n_both + 2 * idx + c;
                 else pos = n_both + n_mix + idx;  // tail of the longer class
               }
+              pos += lead;
               entJ[pos] = (uint16_t)jb;
               // keys valid for the first query block's rows, for the second's
               *reinterpret_cast<uint16_t*>(entV + pos * 2) = (uint16_t)((in0 ? nvalid : 0) | (in1 ? nvalid << 8 : 0));
@@ -648,7 +715,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             at2 += __popc(only1);
           } else {
             if ((w0 >> lane) & 1u) {
-              const int pos = at0 + __popc(w0 & below);
+              const int pos = lead + at0 + __popc(w0 & below);
               entJ[pos] = (uint16_t)jb;
               entV[pos * 2] = (uint8_t)nvalid;
               if (nvalid < BLK) rag_pos = pos;
@@ -672,37 +739,56 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           }
           __syncwarp();
         }
-        // What the entries' blocks have in global memory, a lane per entry, two loads in flight
-        float kn_max = 0.0f;
-        for (int e = lane; e < running; e += 64) {
-          const int e2 = e + 32 < running ? e + 32 : e;
-          const int64_t at = (int64_t)bh * p.NB + entJ[e], at_2 = (int64_t)bh * p.NB + entJ[e2];
-          if (kPacked) {
-            const int32_t s1 = p.slot[at], s2 = p.slot[at_2];
+        if (kPacked) {  // where the entries' blocks are, a lane per entry, two loads in flight
+          for (int e = lane; e < running; e += 64) {
+            const int e2 = e + 32 < running ? e + 32 : e;
+            const int32_t s1 = p.slot[(int64_t)bh * p.NB + entJ[e]], s2 = p.slot[(int64_t)bh * p.NB + entJ[e2]];
             entS[e] = s1;
             entS[e2] = s2;
           }
-          if (!kPacked) {
-            const float k1 = p.knorm[at], k2 = p.knorm[at_2];
-            entN[e] = k1;
-            entN[e2] = k2;
-            kn_max = fmaxf(kn_max, fmaxf(k1, k2));
-          }
+          __syncwarp();
         }
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) kn_max = fmaxf(kn_max, __shfl_xor_sync(0xffffffffu, kn_max, s));
-        __syncwarp();
+        if (ref_of == kRefZero && running < (kZeroMinTiles - 1) * C::kEPT + 1) ref_of = kRefFirst;
         if (lane == 0) {
           s_item[buf] = bh;
           s_rag[buf] = rag_pos >= 0 ? 1 : 0;
           s_nent[buf] = running;
-          s_knmax[buf] = kn_max;
+          s_ref[buf] = ref_of;
+          s_none[buf] = none;
           s_blk[buf * 2] = blk0;
           s_blk[buf * 2 + 1] = blk1;
+          s_failed[buf] = 0;
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(list_ready + buf);
-        if (kEarly) fetch(next_item());
+        if (again >= 0) {  // back to the item that was at hand, if there was one
+          bh = next_bh;
+          blk0 = next_blk0;
+          blk1 = next_blk1;
+          if (kEarly && bh < p.BH) load_rows();
+        } else if (kEarly) {
+          fetch(next_item());
+        }
+      }
+    } else {
+      // ============== rows of query blocks that keep nothing, which are no work items ==============
+      // They have nothing to do with the items, so three idle warps write them while the others work: 677 MB of an
+      // attention of 40 heads x 75600 to one rank's own blocks.  A lane looks at a query block of its own, since a look
+      // is one or two loads that wait for each other; neighbours go to different warps.
+      const int64_t n_rows = (int64_t)p.BH * p.NB, warps = (int64_t)gridDim.x * 3, mine = (int64_t)blockIdx.x * 3 + warp - 5;
+      for (int64_t u0 = mine; u0 < n_rows; u0 += 32 * warps) {
+        const int64_t u = u0 + lane * warps;  // (batch, head, block)
+        bool empty = u < n_rows && (!kPacked || p.rank[u % p.NB] == p.consumer);
+        if (empty) {
+          uint32_t any = 0;
+#pragma unroll 8
+          for (int w = 0; w < p.Wd; ++w) any |= p.mask[u * p.Wd + w];
+          empty = any == 0u;
+        }
+        for (uint32_t todo = __ballot_sync(0xffffffffu, empty); todo; todo &= todo - 1) {
+          const int64_t v = u0 + (__ffs(todo) - 1) * warps;
+          clear_rows<D, BLK>(p, v / p.NB, (int)(v % p.NB));
+        }
       }
     }
   } else {
@@ -718,67 +804,36 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     const uint32_t tO = tmem_base + C::kColO + lane_off;
     const int bar_mine = 1 + wg * 4 + rgrp;         // I arrive here after my decision
     const int bar_other = 1 + (1 - wg) * 4 + rgrp;  // the row group's other warp arrives here after its decision
-    volatile int* frz = s_frz + rgrp;               // set by the warp that freezes the reference, cleared by the other
-
-    int g0 = 0;  // number of the item's first tile
-    int qn = 0;  // items so far (the phase of the Q barrier)
+    int g0 = 0;       // number of the item's first tile
+    int n_first = 0;  // items so far whose reference came from their first tile
     for (int i = 0;; ++i) {
       const int buf = i & 1;
-      volatile float* ref = sRef + (i % 3) * 128;
       mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 56, p.wait_limit);
       const int bh = s_item[buf];
       if (bh < 0) break;
       const int n_ent = s_nent[buf];
       const int n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
+      const int first = (wg - g0) & 1;  // my first tile
+      const int ref_of = s_ref[buf];
       const uint8_t* entV = sEntV + buf * kMaxBlocks * 2 + (C::kStacked ? rh : 0);  // my query block's column
       const bool item_ragged = s_rag[buf] != 0;
-      const float* entN = sEntN + buf * kMaxBlocks;
-      const float kn_item = s_knmax[buf];
-      const int batch = bh / p.H, head = bh % p.H;
-      // Once no score of any remaining tile of the item can exceed the row's reference maximum by more than
-      // 2^kSkipMargin (Cauchy-Schwarz with the item's largest key norm), the reference is final: both warps of
-      // the row group stop taking turns and the rest of the item is load -> exponentials -> store.
-      bool frozen = false;
-      float q_bound = INFINITY;  // |q_row| * softmax scale * log2(e) (+0.1 %), once known
-      float m_ref = -INFINITY;  // the row's reference maximum (log2 domain) as this thread last saw it
-      float l_run = 0.0f;       // this thread's partial row sum, relative to m_ref
-      if (!kPacked && n_tiles >= 4) {
-        // The norm of my query row, read from the Q tile in shared memory while the item's first Q K^T runs (any
-        // order of its 16-byte units will do, so the swizzle does not matter).  Q stays there until the item's
-        // last Q K^T has completed; with four or more tiles that one cannot be issued before both warpgroups
-        // have released a score buffer, which they do after this.
-        mbar_wait_bounded_inline(q_full, qn & 1, s_abort, 42, p.wait_limit);
-        float ss[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // four chains, so that the additions do not wait for each other
-#pragma unroll
-        for (int c = 0; c < D / 64; ++c) {
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const uint4 v = *reinterpret_cast<const uint4*>(sQ + c * 16384 + row * 128 + (((k + lane) & 7) << 4));
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
-              ss[e] = fmaf(lo, lo, ss[e]);
-              ss[e] = fmaf(hi, hi, ss[e]);
-            }
-          }
-        }
-        q_bound = sqrtf((ss[0] + ss[1]) + (ss[2] + ss[3])) * p.scale_log2 * 1.001f;
-        // Both threads of a row compute the same bound from the same data, so both warps of a row group take this
-        // decision alike without talking to each other: the item runs on the fixed reference 0 from its first
-        // tile on -- no row maximum, no turns, no named barrier (neither warp arrives, neither waits).
-        if (__all_sync(0xffffffffu, q_bound * kn_item <= kStaticBound)) {
-          frozen = true;
-          m_ref = 0.0f;
-          ref[row] = 0.0f;  // (both threads of the row write the same value; the epilogue reads it)
-        }
-      }
-      ++qn;
+      volatile float* ref = sRef + (i & 3) * 128;
+      float m_ref = ref_of == kRefZero ? 0.0f : -INFINITY;  // the row's reference as this thread last saw it
+      float i_max = 0.0f;  // largest binary exponent that was taken on the FMA pipe, in magnitude
+      uint64_t* ref_bar = ref_ready + (n_first & 3);
+      const uint32_t ref_phase = (n_first >> 2) & 1;
+      const bool from_first = ref_of == kRefFirst || ref_of == kRefWide;
+      if (from_first) ++n_first;
+      auto learn_ref = [&]() {  // the warpgroup that does not own the first tile
+        mbar_wait_bounded_inline(ref_bar, ref_phase, s_abort, 43, p.wait_limit);
+        m_ref = ref[row];
+      };
 
-      // One tile of this warpgroup.  kRagged = the sequence ends inside the tile (possible only for the item's
-      // last tile): that variant carries the column masking, the common one stays small.
-      auto do_tile = [&](auto ragged_tag, const int n) {
-        constexpr bool kRagged = decltype(ragged_tag)::value;
+      // One tile of this warpgroup.  kGeneral = the sequence may end inside the tile (possible only for the item's last
+      // tile), or the item is computed again, or (K / V source) the reference comes from the first tile and this is it:
+      // that variant carries the column masking and the turns, the common one stays small.
+      auto do_tile = [&](auto general_tag, const int n) {
+        constexpr bool kGeneral = decltype(general_tag)::value;
         const int g = g0 + n;
         // kept / valid key columns of each 64-column half of the tile (warp-uniform), as the list builder left them
         int vh[2];
@@ -802,7 +857,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(s_free + wg);
 
-        if (kRagged) {
+        if (kGeneral) {
           // the sequence ends inside this tile: columns past the end count as -inf
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
@@ -812,23 +867,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             }
           }
         }
-        if (!frozen) {
-          // Cauchy-Schwarz: no score of this tile exceeds |q| * max |k| * scale.  If that bound stays within
-          // 2^kSkipMargin of the row's reference maximum (which only grows, so the value this thread saw last
-          // will do) for all 32 rows of the warp, the reference need not move and the row-maximum pass is
-          // skipped: the exponentials stay below 2^kSkipMargin, harmless in fp32 / bf16, and the result does
-          // not depend on the reference.
-          bool skip = false;
-          if (!kRagged && !kPacked) {
-            float kn = entN[n * C::kEPT];
-            if (C::kStacked) kn = fmaxf(kn, entN[min(n * 2 + 1, n_ent - 1)]);
-            skip = __all_sync(0xffffffffu, q_bound * kn <= m_ref + kSkipMargin);
-          }
-
+        auto row_max = [&]() {
           // one flat instruction stream per 64-key half; an absent half (not kept by this row's query block)
           // is skipped
           float mx = -INFINITY;
-          if (!skip)
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const float* svh = sv + h * 64;
@@ -844,98 +886,80 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
               mx = fmaxf(mx, fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)));
             }
           }
-          mx *= p.scale_log2;
-
+          return mx * p.scale_log2;
+        };
+        if (kGeneral && ref_of == kRefExact) {
+          const float mx = row_max();
           // ---- my turn to look at / move the row's reference maximum (strictly in tile order) ----
-          if (n > 0) named_bar_sync(bar_other, 64);
-          const float m_cur = ref[row];
-          const int told = !kPacked && n > 0 ? *frz : 0;  // the row group's other warp froze the reference in its last turn
-          if (m_cur != m_ref) {  // the other thread moved it since my last tile
-            l_run *= ex2(m_ref - m_cur);  // m_ref = -inf: l_run is 0 and stays 0
-            m_ref = m_cur;
+          if (n > 0) {
+            named_bar_sync(bar_other, 64);
+            m_ref = ref[row];  // (the other thread may have moved it since my last tile)
           }
-          if (told) {
-            frozen = true;
-            __syncwarp();
-            if (lane == 0) *frz = 0;  // nobody looks at it again before the next item's turns
-          } else {
-            // the first of the two warps to see the bound hold for the whole item says so, takes its last turn
-            // without moving the reference (no score can make that necessary) and releases the other one more time
-            if (!kPacked && n + 1 < n_tiles &&
-                __all_sync(0xffffffffu, q_bound * kn_item <= m_ref + kSkipMargin)) {
-              frozen = true;
-              if (lane == 0) *frz = 1;
-            }
-            const float m_new = fmaxf(m_ref, mx);
-            const bool grow = !frozen && (m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY));
-            if (!skip && __any_sync(0xffffffffu, grow)) {
-              const float alpha = grow ? ex2(m_ref - m_new) : 1.0f;  // m_ref = -inf -> 0
-              if (n > 0) {
-                // every P V of the item issued so far must have landed in O before the row is rescaled; they
-                // complete in order, so the one of tile g-1 suffices
-                mbar_wait_bounded_inline(o_full + ((g - 1) & 3), ((g - 1) >> 2) & 1, s_abort, 38, p.wait_limit);
-                tc_fence_after();
+          const float m_new = fmaxf(m_ref, mx);
+          const bool grow = m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY);
+          if (__any_sync(0xffffffffu, grow)) {
+            const float alpha = grow ? ex2(m_ref - m_new) : 1.0f;  // m_ref = -inf -> 0
+            if (n > 0) {
+              // every P V of the item issued so far must have landed in O before the row is rescaled; they
+              // complete in order, so the one of tile g-1 suffices
+              mbar_wait_bounded_inline(o_full + ((g - 1) & 3), ((g - 1) >> 2) & 1, s_abort, 38, p.wait_limit);
+              tc_fence_after();
 #pragma unroll 1
-                for (int c = 0; c < C::kAccCols / 16; ++c) {  // the row's accumulator, 16 columns at a time (rare: kept small)
-                  uint32_t o[16];
-                  tmem_ld16(tO + c * 16, o);
-                  tmem_ld_wait();
+              for (int c = 0; c < C::kAccCols / 16; ++c) {  // the row's accumulator, 16 columns at a time (rare: kept small)
+                uint32_t o[16];
+                tmem_ld16(tO + c * 16, o);
+                tmem_ld_wait();
 #pragma unroll
-                  for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                  tmem_st16(tO + c * 16, o);
-                }
-                if (C::kSum128) {  // the row sums live in columns of their own
-                  uint32_t o[16];
-                  tmem_ld16(tmem_base + C::kColL + lane_off, o);
-                  tmem_ld_wait();
+                for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                tmem_st16(tO + c * 16, o);
+              }
+              if (C::kSum128) {  // the row sums live in columns of their own
+                uint32_t o[16];
+                tmem_ld16(tmem_base + C::kColL + lane_off, o);
+                tmem_ld_wait();
 #pragma unroll
-                  for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                  tmem_st16(tmem_base + C::kColL + lane_off, o);
-                }
-                tmem_st_wait();
-                tc_fence_before();
+                for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                tmem_st16(tmem_base + C::kColL + lane_off, o);
               }
-              l_run *= alpha;
-              if (grow) {
-                m_ref = m_new;
-                ref[row] = m_new;
-              }
+              tmem_st_wait();
+              tc_fence_before();
             }
-            if (n + 1 < n_tiles) {
-              asm volatile("bar.arrive %0, %1;" ::"r"(bar_mine), "r"(64) : "memory");
-            }
+            if (grow) m_ref = m_new;
+          }
+          if (n == 0 || m_ref != ref[row]) ref[row] = m_ref;
+          if (n + 1 < n_tiles) asm volatile("bar.arrive %0, %1;" ::"r"(bar_mine), "r"(64) : "memory");
+        }
+        if ((kGeneral || kPacked) && from_first && n <= 1) {
+          if (n == 0) {
+            const float mx = row_max();
+            m_ref = mx > -INFINITY ? mx : 0.0f;  // (keeps nothing of this tile, or is no number)
+            ref[row] = m_ref;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(ref_bar);
+          } else {
+            learn_ref();
           }
         }
 
         // exponentials of keys [64h, 64h+64) -> packed bf16 columns [32h, 32h+32) of the P buffer
-        float2 lsum2 = make_float2(0.0f, 0.0f);
-        const float neg_m = -m_ref;
         uint32_t pk[64];
-        const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nm2 = make_float2(neg_m, neg_m);
+        const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nm2 = make_float2(-m_ref, -m_ref);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const float* svh = sv + h * 64;
           uint32_t* pkh = pk + h * 32;
-          if (vh[h] > 0) {  // then the row has a finite reference maximum
+          if (vh[h] > 0) {  // then the row has a finite reference
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
               const float2 x = ffma2(make_float2(svh[2 * e], svh[2 * e + 1]), sc2, nm2);
               constexpr int kPoly = C::kOnes ? SPARSP_TUNE_POLY_D64 : SPARSP_TUNE_POLY;
               const float2 pp = (kPoly > 0 && (e % (kPoly > 0 ? kPoly : 1)) == 1)
-                                    ? exp2_poly2(x)
+                                    ? exp2_poly2<kGeneral>(x, &i_max)
                                     : make_float2(ex2(x.x), ex2(x.y));
               const __nv_bfloat162 h2 = __floats2bfloat162_rn(pp.x, pp.y);
               pkh[e] = *reinterpret_cast<const uint32_t*>(&h2);
-              if (!C::kSumMma) {
-                // the row sum adds the bf16 values that P V multiplies, not the unrounded exponentials: with a
-                // reference that is not the row's maximum the largest term is an arbitrary 2^x, and a sum of
-                // unrounded terms would differ from the numerator's weights by up to 2^-9 of a peaked row
-                asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}"
-                    : "+f"(lsum2.x), "+f"(lsum2.y)
-                    : "r"(pkh[e]));
-              }
             }
-            if (kRagged && vh[h] < 64) {
+            if (kGeneral && vh[h] < 64) {
               // columns past the end of the sequence: exactly zero in P (the polynomial path returns
               // 2^-126 for them, which the row sum may keep)
 #pragma unroll
@@ -946,7 +970,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             for (int e = 0; e < 32; ++e) pkh[e] = 0u;
           }
         }
-        l_run += lsum2.x + lsum2.y;
         // my P buffer was last read by the P V of tile g-2; a single P buffer by that of tile g-1
         constexpr int kBack = C::kNumP == 2 ? 2 : 1;
         if (g >= kBack) {
@@ -960,51 +983,53 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(p_full + wg);
       };
-      for (int n = (wg - g0) & 1; n < n_tiles; n += 2) {
+      for (int n = first; n < n_tiles; n += 2) {
         // the list builder puts the sequence's last block (the only one that can be ragged) into the last tile
-        const bool ragged = item_ragged && n == n_tiles - 1;
-        if (ragged) {
+        if (ref_of >= kRefWide || (item_ragged && n == n_tiles - 1) || (!kPacked && from_first && n <= 1)) {
           do_tile(std::true_type{}, n);
         } else {
           do_tile(std::false_type{}, n);
         }
       }
 
+      g0 += n_tiles;
       // ---- item epilogue: warpgroup x writes the column half x of every row -------------------------
-      sStat[(buf * 2 + wg) * 128 + row] = make_float2(m_ref, l_run);
-      named_bar_sync(9, 256);  // all of the item's decisions and P stores are done
-      const int last = g0 + n_tiles - 1;
+      if (ref_of == kRefExact) {
+        named_bar_sync(9, 256);  // all of the item's decisions are done
+        m_ref = ref[row];
+      } else if (from_first && first >= n_tiles) {
+        learn_ref();
+      }
+      const int last = g0 - 1;
       mbar_wait_bounded_inline(o_full + (last & 3), (last >> 2) & 1, s_abort, 40, p.wait_limit);
       tc_fence_after();
       {
         constexpr int HW = D / 2;
-        const float m_fin = ref[row];
-        const float2 st0 = sStat[(buf * 2) * 128 + row], st1 = sStat[(buf * 2 + 1) * 128 + row];
-        // this reference buffer serves the item after next: no warp can be there before every warp has passed
-        // the barrier above, and the item before this one (its last user) is finished for all of them
-        sRef[((i + 2) % 3) * 128 + row] = -INFINITY;
-        float l = (st0.y > 0.0f ? st0.y * ex2(st0.x - m_fin) : 0.0f) + (st1.y > 0.0f ? st1.y * ex2(st1.x - m_fin) : 0.0f);
-        if (C::kSumMma) {  // the row sum is a tensor-memory column
-          uint32_t sums[16];
-          tmem_ld16(tmem_base + C::kColL + lane_off, sums);
-          tmem_ld_wait();
-          l = __uint_as_float(sums[0]);
-        }
-        const float inv_l = l > 0.0f ? 1.0f / l : 0.0f;
         const int qb = C::kStacked ? s_blk[buf * 2 + rh] : s_blk[buf * 2];
-        const int64_t tok = qb >= 0 ? (int64_t)qb * BLK + (C::kStacked ? (row & 63) : row) : p.N;
+        // (a block that keeps nothing is stacked with one that does: other warps write its rows)
+        const bool none = qb < 0 || ((s_none[buf] >> (C::kStacked ? rh : 0)) & 1);
+        const int64_t tok = none ? p.N : (int64_t)qb * BLK + (C::kStacked ? (row & 63) : row);
+        const int batch = bh / p.H, head = bh % p.H;
         __nv_bfloat16* orow = p.O + (int64_t)batch * p.sB + (int64_t)head * p.sH + tok * p.sT + wg * HW;
-        uint32_t o[HW];
+        uint32_t sum, o[HW];
+        tmem_ld1(tmem_base + C::kColL + lane_off, &sum);
 #pragma unroll
         for (int c = 0; c < HW / 32; ++c) tmem_ld32(tO + wg * HW + c * 32, o + c * 32);
         tmem_ld_wait();
+        const float l = __uint_as_float(sum);  // the row sum is a tensor-memory column
+        const bool failed = ref_of != kRefExact && tok < p.N && !(i_max <= kMaxExponent && l >= kMinSum && l <= kMaxSum);
+        const bool any_failed = __any_sync(0xffffffffu, failed);
+        const bool any_far = __any_sync(0xffffffffu, failed && i_max > 2.0f * kMaxExponent);
         // the accumulator is in registers: the next item's first P V may overwrite it
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
+          if (any_far) s_failed[buf] = 2;
+          else if (any_failed && s_failed[buf] == 0) s_failed[buf] = 1;
           mbar_arrive(o_drained);
           mbar_arrive(list_free + buf);
         }
+        const float inv_l = l > 0.0f ? 1.0f / l : 0.0f;
         if (tok < p.N) {
           // a thread's row segment is 2 HW contiguous bytes but the rows of a warp are sT elements apart, so every
           // store instruction touches 32 lines: 32-byte stores (when the layout allows) halve their number
@@ -1029,9 +1054,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           }
         }
         if (p.lse && wg == 0 && tok < p.N)
-          p.lse[(int64_t)bh * p.N + tok] = l > 0.0f ? (m_fin + log2f(l)) * 0.6931471805599453f : -INFINITY;
+          p.lse[(int64_t)bh * p.N + tok] = l > 0.0f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
       }
-      g0 += n_tiles;
     }
   }
 
@@ -1042,28 +1066,22 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 }
 
 // ------------------------------------------------------------------------------------------------
-// Preparation of an attention call, one launch for passes that do not depend on each other:
-//   CTAs [0, B*H)  fix the work items of one (batch, head) each (and, packed source, its table of packed slots);
-//   the rest       one warp per block: the largest key norm of the KV block, and the output rows of a query block that
-//                  keeps nothing (zeros, log-sum-exp -inf), so that such blocks never become work items.
+// Preparation of an attention call: a CTA per (batch, head) fixes its work items and, packed source, its table of packed
+// slots.  A query block that keeps nothing never becomes a work item.
 //
 // Block 64: which two query blocks share a Q tile.  K / V source: blocks i and i+D are paired in stripes (i mod 2D <
 // D), leftovers pair up consecutively; the offset D in 1..n/2 that maximises the summed overlap |M[i] & M[i+D]| of the
 // kept lists is chosen per (batch, head) -- video attention is multi-diagonal, so the best partner of a block is
 // typically the same position a fixed number of blocks away; the more two stacked blocks share, the less of a 128-row
 // tile's work is masked away.
-// Packed source: neighbours in the consumer's ascending list of blocks (D = 1).  Its rows take their reference from the
-// first tiles, and the blocks that two neighbours both keep, which come first, are on video inputs little more than the
-// two themselves: a row meets its largest score at once, whose exponential is then exactly 1.  Chosen by overlap the
-// partner is far away, the largest term is some rounded 2^x, and the output is further from 64 bits (24 heads x 24576,
-// 4 ranks: 2.01e-3 against 1.95e-3, log-sum-exp 3.7e-4 against 3.2e-4; 347 us against 433).
+// Packed source: neighbours in the consumer's ascending list of blocks (D = 1), so that a row's result does not depend on
+// what the consumer's other blocks keep.
 // (Mask rows in shared memory have an odd pitch: the threads' offsets differ by one row, a pitch of 32 words would put
 // them all on one bank.)
 // Items of one (batch, head) are handed out longest list first: the items still running when the queue
 // runs dry are then the short ones, which matters when list lengths vary (threshold selection, unions of two
 // stacked blocks).  Key = (list length << 10) | (1023 - index): equal lengths keep their index order.
-// Latency-bound integer work next to the key norms, which read K once: 132 us for the 774 MB of 40 heads x 75600 keys
-// (158 us when a lane's loads waited for each other), 7 us for 26 heads x 6034 keys (24 us).
+// Latency-bound integer work.
 // ------------------------------------------------------------------------------------------------
 constexpr int kPrepThreads = 256;
 constexpr int kPairSample = 8;
@@ -1073,11 +1091,6 @@ struct PrepParams {
   int32_t* pairs;
   int32_t* n_items;
   int32_t* work_counter;
-  const __nv_bfloat16* K;
-  __nv_bfloat16* O;
-  float* lse;
-  float* knorm;
-  int64_t sB, sH, sT, N;
   int BH, H, NB, Wd, b;
   // packed source only
   const int32_t* rank;
@@ -1228,114 +1241,37 @@ __device__ __forceinline__ void make_slots(const PrepParams& p, int bh) {
   }
 }
 
-// The output rows of query block i: zeros and a log-sum-exp of -inf.  One warp.
-template <int D>
-__device__ __forceinline__ void clear_rows(const PrepParams& p, int64_t bh, int i) {
-  constexpr int LPT = D / 8;
-  const int lane = threadIdx.x & 31;
-  const int64_t tok0 = (int64_t)i * p.b;
-  const int n = (int)min((int64_t)p.b, p.N - tok0);
-  __nv_bfloat16* o = p.O + (bh / p.H) * p.sB + (bh % p.H) * p.sH + tok0 * p.sT + (lane % LPT) * 8;
-  for (int r = lane / LPT; r < n; r += 32 / LPT)
-    *reinterpret_cast<uint4*>(o + (int64_t)r * p.sT) = make_uint4(0u, 0u, 0u, 0u);
-  if (p.lse)
-    for (int r = lane; r < n; r += 32) p.lse[bh * p.N + tok0 + r] = -INFINITY;
-}
-
-// Largest L2 norm of the keys of block j (times 1.001): with the norm of a query row it bounds the scores of a tile.
-// One warp, d/8 lanes per token, kNormLoads 16-byte loads of every lane in flight.
-constexpr int kNormLoads = 16;
-template <int D>
-__device__ __forceinline__ float block_norm(const PrepParams& p, int64_t bh, int j) {
-  constexpr int LPT = D / 8;     // lanes per token
-  constexpr int TPW = 32 / LPT;  // tokens per warp load
-  const int lane = threadIdx.x & 31;
-  const int64_t tok0 = (int64_t)j * p.b;
-  const int n = (int)min((int64_t)p.b, p.N - tok0);
-  const __nv_bfloat16* base = p.K + (bh / p.H) * p.sB + (bh % p.H) * p.sH + tok0 * p.sT + (lane % LPT) * 8;
-  float best = 0.0f;
-  for (int t0 = lane / LPT; t0 < p.b; t0 += TPW * kNormLoads) {  // (p.b is a multiple of TPW: the lanes stay together)
-    uint4 v[kNormLoads];
-#pragma unroll
-    for (int k = 0; k < kNormLoads; ++k) {
-      const int t = t0 + k * TPW;
-      v[k] = t < n ? *reinterpret_cast<const uint4*>(base + (int64_t)t * p.sT) : make_uint4(0u, 0u, 0u, 0u);
-    }
-#pragma unroll
-    for (int k = 0; k < kNormLoads; ++k) {
-      const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-      float ss = 0.0f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
-        ss = fmaf(lo, lo, ss);
-        ss = fmaf(hi, hi, ss);
-      }
-#pragma unroll
-      for (int sft = 1; sft < LPT; sft <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, sft);
-      best = fmaxf(best, ss);
-    }
-  }
-#pragma unroll
-  for (int sft = LPT; sft < 32; sft <<= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, sft));
-  return sqrtf(best) * 1.001f;
-}
-
-template <int D, bool kPacked>
+template <bool kPacked>
 __global__ void __launch_bounds__(kPrepThreads) attn_prep_kernel(const PrepParams p) {
   enter_grid();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (blockIdx.x == 0 && threadIdx.x == 0) *p.work_counter = 0;  // the attention kernel's work queue
-  if ((int)blockIdx.x < p.BH) {
-    const int bh = blockIdx.x;
-    int n_live;
-    if (kPacked) {
-      __shared__ uint32_t s_words[kMaxWords];
-      __shared__ uint16_t s_list[kMaxBlocks];
-      rank_words(p.rank, p.NB, p.consumer, s_words);
-      const int n = list_blocks(s_words, p.NB, s_list);
-      n_live = make_items(p, bh, s_list, n, smem_raw);
-      if (n_live > 0) make_slots(p, bh);
-      if (bh % p.H == 0 && warp == 0) {  // first tile of the consumer's buffer for this batch item
-        const int64_t br = (int64_t)(bh / p.H) * p.P + p.consumer;
-        int64_t first = 0;
-        if (p.dst_base) {
-          first = p.dst_base[br] / p.tile_bytes;
-        } else {
-          for (int64_t t = lane; t < br; t += 32) first += 2 * p.seg_total[t];
+  const int bh = blockIdx.x;
+  int n_live;
+  if (kPacked) {
+    __shared__ uint32_t s_words[kMaxWords];
+    __shared__ uint16_t s_list[kMaxBlocks];
+    rank_words(p.rank, p.NB, p.consumer, s_words);
+    const int n = list_blocks(s_words, p.NB, s_list);
+    n_live = make_items(p, bh, s_list, n, smem_raw);
+    if (n_live > 0) make_slots(p, bh);
+    if (bh % p.H == 0 && warp == 0) {  // first tile of the consumer's buffer for this batch item
+      const int64_t br = (int64_t)(bh / p.H) * p.P + p.consumer;
+      int64_t first = 0;
+      if (p.dst_base) {
+        first = p.dst_base[br] / p.tile_bytes;
+      } else {
+        for (int64_t t = lane; t < br; t += 32) first += 2 * p.seg_total[t];
 #pragma unroll
-          for (int s = 16; s >= 1; s >>= 1) first += __shfl_xor_sync(0xffffffffu, first, s);
-        }
-        if (lane == 0) p.tile_base[bh / p.H] = first;
+        for (int s = 16; s >= 1; s >>= 1) first += __shfl_xor_sync(0xffffffffu, first, s);
       }
-    } else {
-      n_live = make_items(p, bh, nullptr, p.NB, smem_raw);
+      if (lane == 0) p.tile_base[bh / p.H] = first;
     }
-    if (threadIdx.x == 0) p.n_items[bh] = n_live;
-    return;
+  } else {
+    n_live = make_items(p, bh, nullptr, p.NB, smem_raw);
   }
-  const int64_t unit = (int64_t)((int)blockIdx.x - p.BH) * (kPrepThreads / 32) + warp;  // (batch, head, block)
-  if (unit >= (int64_t)p.BH * p.NB) return;
-  const int64_t bh = unit / p.NB;
-  const int j = (int)(unit - bh * p.NB);
-  if (kPacked && p.rank[j] != p.consumer) return;
-  const uint32_t row = lane < p.Wd ? p.mask[unit * p.Wd + lane] : 0u;
-  if (!__any_sync(0xffffffffu, row != 0u)) clear_rows<D>(p, bh, j);
-  if (kPacked) return;  // remote keys live in the packed buffer: every tile takes its row maximum
-  // A block that nobody keeps needs no norm.  Its own row nearly always keeps it; otherwise the column decides.
-  const int w = j >> 5;
-  bool kept = (__shfl_sync(0xffffffffu, row, w) >> (j & 31)) & 1u;
-  if (!kept) {
-    const uint32_t* col = p.mask + bh * p.NB * p.Wd + w;
-    uint32_t any = 0;
-#pragma unroll 4
-    for (int i = lane; i < p.NB; i += 32) any |= col[(int64_t)i * p.Wd];
-    kept = __any_sync(0xffffffffu, (any >> (j & 31)) & 1u);
-  }
-  if (!kept) return;
-  const float norm = block_norm<D>(p, bh, j);
-  if (lane == 0) p.knorm[unit] = norm;
+  if (threadIdx.x == 0) p.n_items[bh] = n_live;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1462,29 +1398,19 @@ static int launch_attn_common(const sparsp_shape& s, const Geometry& g, const vo
 
 template <bool kPacked>
 static int launch_prep(const Geometry& g, const PrepParams& p, cudaStream_t st) {
-  auto kern = g.d == 64 ? attn_prep_kernel<64, kPacked> : attn_prep_kernel<128, kPacked>;
+  auto kern = attn_prep_kernel<kPacked>;
   const int smem = g.b == 64 ? g.NB * (g.Wd | 1) * 4 : 0;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
-  constexpr int kWarps = kPrepThreads / 32;
-  const int64_t blocks = p.BH + ((int64_t)p.BH * g.NB + kWarps - 1) / kWarps;
-  SPARSP_CUDA_OK(launch_kernel(kern, (unsigned)blocks, kPrepThreads, smem, st, p));
+  SPARSP_CUDA_OK(launch_kernel(kern, (unsigned)p.BH, kPrepThreads, smem, st, p));
   return SPARSP_OK;
 }
 
-static PrepParams prep_params(const sparsp_shape& s, const Geometry& g, const void* K, const uint32_t* mask, void* O,
-                              float* lse, char* ws, const WsLayout& L) {
+static PrepParams prep_params(const Geometry& g, const uint32_t* mask, char* ws, const WsLayout& L) {
   PrepParams p = {};
   p.mask = mask;
   p.pairs = (int32_t*)(ws + L.pairs);
   p.n_items = (int32_t*)(ws + L.n_items);
   p.work_counter = (int32_t*)(ws + L.status) + kWorkCounterWord;
-  p.K = (const __nv_bfloat16*)K;
-  p.O = (__nv_bfloat16*)O;
-  p.lse = lse;
-  p.sB = s.stride_batch;
-  p.sH = s.stride_head;
-  p.sT = s.stride_token;
-  p.N = g.N;
   p.BH = g.B * g.H;
   p.H = g.H;
   p.NB = g.NB;
@@ -1496,15 +1422,13 @@ static PrepParams prep_params(const sparsp_shape& s, const Geometry& g, const vo
 int launch_attn(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, const void* V,
                 const uint32_t* mask, float scale, void* O, float* lse, char* ws, const WsLayout& L,
                 cudaStream_t st) {
-  PrepParams pre = prep_params(s, g, K, mask, O, lse, ws, L);
-  pre.knorm = (float*)(ws + L.knorm);
+  PrepParams pre = prep_params(g, mask, ws, L);
   const int rc = launch_prep<false>(g, pre, st);
   if (rc != SPARSP_OK) return rc;
   AttnParams p = {};
   p.mask = mask;
   p.pairs = pre.pairs;
   p.n_items = pre.n_items;
-  p.knorm = pre.knorm;
   return launch_attn_common<false>(s, g, Q, K, V, nullptr, 0, p, scale, O, lse, ws, L, st);
 }
 
@@ -1517,7 +1441,7 @@ int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, 
                        const int64_t* seg_off, const int64_t* seg_total, const void* packed, int64_t capacity,
                        const int64_t* dst_base, float scale, void* O, float* lse, char* ws, const WsLayout& L,
                        cudaStream_t st) {
-  PrepParams pre = prep_params(s, g, K, mask, O, lse, ws, L);
+  PrepParams pre = prep_params(g, mask, ws, L);
   pre.rank = rank;
   pre.U = U;
   pre.seg_off = seg_off;
@@ -1536,6 +1460,8 @@ int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, 
   p.n_items = pre.n_items;
   p.slot = pre.slot;
   p.tile_base = pre.tile_base;
+  p.rank = rank;
+  p.consumer = consumer;
   return launch_attn_common<true>(s, g, Q, K, V, packed, capacity, p, scale, O, lse, ws, L, st);
 }
 

@@ -28,7 +28,7 @@ struct Geometry {
 };
 
 struct WsLayout {
-  int64_t status, pooled_q, pooled_k, scores, pairs, slot, tile_base, n_items, knorm, n_entries, entries, total;
+  int64_t status, pooled_q, pooled_k, scores, pairs, slot, tile_base, n_items, n_entries, entries, total;
 };
 
 void set_error(const char* fmt, ...);

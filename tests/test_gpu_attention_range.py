@@ -1,0 +1,85 @@
+"""Items whose scores leave the range that the attention kernel assumes are computed again: relative to their first tile,
+then with the running maximum.  Rows of all three kinds among many items per CTA, the last items of the call among them,
+against a masked softmax in 64 bits."""
+import math
+
+import pytest
+import torch
+
+import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def binding():
+    from paper_2609_32197_b200 import binding as b
+    b.lib()
+    return b
+
+
+def _reference(Q, K, V, kept, b):
+    """[H][N][d] in 64 bits: softmax over the keys of kept [H][NB][NB] blocks, and the log-sum-exp."""
+    N, d = Q.shape[1:]
+    O, lse = torch.empty_like(Q, dtype=torch.float64), torch.empty(Q.shape[:2], dtype=torch.float64, device="cuda")
+    for h in range(Q.shape[0]):
+        s = Q[h].double() @ K[h].double().T / math.sqrt(d)
+        tokens = kept[h].repeat_interleave(b, 0).repeat_interleave(b, 1)[:N, :N]
+        s.masked_fill_(~tokens, float("-inf"))
+        lse[h] = torch.logsumexp(s, -1)
+        O[h] = torch.exp(s - lse[h][:, None]) @ V[h].double()
+    return O, lse
+
+
+@pytest.mark.parametrize("d,b", [(64, 64), (128, 64), (64, 128), (128, 128)])
+@pytest.mark.parametrize("large", ["some", "last", "all"])
+@pytest.mark.parametrize("keep", [2, 9])  # lists of one to three and of four to nine tiles
+def test_items_that_leave_the_range(binding, d, b, large, keep):
+    H, NB = (24, 40) if b == 64 else (16, 32)
+    N = NB * b - 9
+    g = torch.Generator(device="cuda").manual_seed(d + b + keep)
+    Q, K, V = (torch.randn(H, N, d, generator=g, device="cuda") for _ in range(3))
+    # scores of a unit row spread over +-6 log2 units; times 40 over +-240 (far from 0, at times near the first tile's
+    # maximum), times 400 over thousands
+    block = torch.arange(N, device="cuda") // b
+    factor = torch.ones(H, N, device="cuda")
+    if large == "all":
+        factor[:] = 40.0
+    elif large == "last":
+        factor[-1] = 40.0
+    else:
+        factor[3::7, :][:, block % 5 == 2] = 40.0
+        factor[2::9, :][:, block % 11 == 3] = 400.0
+        factor[5] = 3.0
+    Q, K, V = (x.to(torch.bfloat16) for x in (Q * factor[..., None], K, V))
+    kept = torch.rand(H, NB, NB, generator=g, device="cuda").argsort(-1).argsort(-1) < keep
+    words = torch.zeros(H, NB, (NB + 31) // 32, dtype=torch.int64, device="cuda")
+    for j in range(NB):
+        words[:, :, j // 32] |= kept[:, :, j].long() << (j % 32)
+    mask = torch.where(words >= 1 << 31, words - (1 << 32), words).to(torch.int32)[None].contiguous()
+    want, want_lse = _reference(Q, K, V, kept, b)
+    shape = binding.make_shape(H, d, (1, 1, N), 0, b)
+    P = 3
+    ws = binding.make_workspace(shape, P)
+
+    def check(O, lse, rows):
+        err = (O[0].double() - want)[:, rows].abs()
+        assert err.max() <= pu.ATTN_MAX_ABS * max(1.0, float(want.abs().max()) / 4.0), float(err.max())
+        # an fp32 number of up to thousands: eight units in the last place on top of the tolerance
+        tol = 2e-2 + want_lse.abs() * 2.0 ** -20
+        assert bool(((lse[0].double() - want_lse).abs() <= tol)[:, rows].all())
+
+    O, lse = torch.full_like(Q, 7.0)[None], torch.full((1, H, N), 7.0, device="cuda")
+    binding.sparsp_sparse_attn_fwd(shape, Q, K, V, mask, 0.0, O, lse, ws)
+    assert binding.sparsp_status(ws) == binding.SPARSP_OK
+    check(O, lse, torch.arange(N, device="cuda"))
+
+    rank = torch.arange(NB, dtype=torch.int32, device="cuda").remainder(P)
+    dm = pu.gpu_demand_pack(binding, shape, mask, rank, P, 0, K, V, ws)
+    for consumer in (0, 2):
+        O.fill_(7.0)
+        lse.fill_(7.0)
+        binding.sparsp_sparse_attn_fwd_packed(shape, Q, K, V, mask, rank, P, consumer, dm["union_mask"], dm["seg_offset"],
+                                              dm["seg_total"], dm["packed"], dm["packed"].numel(), None, 0.0, O, lse, ws)
+        assert binding.sparsp_status(ws) == binding.SPARSP_OK
+        check(O, lse, torch.nonzero(rank.repeat_interleave(b)[:N] == consumer)[:, 0])
