@@ -1066,8 +1066,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 }
 
 // ------------------------------------------------------------------------------------------------
-// Preparation of an attention call: a CTA per (batch, head) fixes its work items and, packed source, its table of packed
-// slots.  A query block that keeps nothing never becomes a work item.
+// Preparation of an attention call: a CTA per (batch, head) fixes its work items and, packed source, another one its table
+// of packed slots.  A query block that keeps nothing never becomes a work item.
 //
 // Block 64: which two query blocks share a Q tile.  K / V source: blocks i and i+D are paired in stripes (i mod 2D <
 // D), leftovers pair up consecutively; the offset D in 1..n/2 that maximises the summed overlap |M[i] & M[i+D]| of the
@@ -1081,9 +1081,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 // Items of one (batch, head) are handed out longest list first: the items still running when the queue
 // runs dry are then the short ones, which matters when list lengths vary (threshold selection, unions of two
 // stacked blocks).  Key = (list length << 10) | (1023 - index): equal lengths keep their index order.
-// Latency-bound integer work.
+// Latency-bound integer work, so what matters is how many loads and barriers wait for each other: rows are counted by a
+// warp each with eight in flight, up to 256 items are put in order without rounds, offsets are scored by all threads, and
+// slots have CTAs of their own and no shared-memory atomics.  One hop of 40 heads x 591 blocks, 8 ranks 5.9 us (23 with
+// 256 threads, a thread per row, a bitonic sort for any number and the slots behind the items), 24 x 384 stacked blocks
+// 15.5, 2 x 64 4.5 (attention calls 72 -> 66-74, 617 -> 594 and 21.2 -> 19.4 us).
 // ------------------------------------------------------------------------------------------------
-constexpr int kPrepThreads = 256;
+constexpr int kPrepThreads = 512;
 constexpr int kPairSample = 8;
 
 struct PrepParams {
@@ -1104,8 +1108,23 @@ struct PrepParams {
   int P, consumer;
 };
 
-// Sorts n keys (n a power of two, <= 1024) in shared memory into descending order; all threads call it.
+// Sorts n keys (n a power of two, <= 1024; distinct but for zeros) in shared memory into descending order; all threads call it.
 __device__ __forceinline__ void sort_keys_descending(uint32_t* keys, int n) {
+  if (n <= kPrepThreads / 2) {
+    // Few keys: a key's place is the number of larger ones, counted by two threads.  No rounds that wait for each other.
+    const int k = threadIdx.x >> 1;
+    const uint32_t key = k < n ? keys[k] : 0u;
+    int place = 0;
+    if (key != 0u)
+      for (int j = threadIdx.x & 1; j < n; j += 2) place += keys[j] > key ? 1 : 0;
+    place += __shfl_xor_sync(0xffffffffu, place, 1);
+    __syncthreads();
+    if (k < n && (threadIdx.x & 1) == 0) keys[k] = 0u;
+    __syncthreads();
+    if (key != 0u && (threadIdx.x & 1) == 0) keys[place] = key;
+    __syncthreads();
+    return;
+  }
   for (int k = 2; k <= n; k <<= 1) {
     for (int j = k >> 1; j > 0; j >>= 1) {
       for (int t = threadIdx.x; t < n; t += kPrepThreads) {
@@ -1135,6 +1154,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
                                           unsigned char* smem_raw) {
   __shared__ uint32_t s_keys[kMaxBlocks];
   __shared__ uint32_t s_pair[kMaxBlocks / 2];  // positions of an item's two blocks, (second or 0xffff) << 16 | first
+  __shared__ unsigned int s_score[kMaxBlocks / 2];
   __shared__ unsigned int s_best;              // (score << 10) | (1023 - D): max = best score, smallest D
   const uint32_t* rows = p.mask + (int64_t)bh * p.NB * p.Wd;
   auto block = [&](int pos) -> int { return list ? list[pos] : pos; };
@@ -1148,11 +1168,21 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
       m[i * pitch + w] = rows[(int64_t)block(i) * Wd + w];
     }
     __syncthreads();
-    for (int d = 1 + threadIdx.x; !list && d <= n / 2; d += kPrepThreads) {
-      unsigned int score = 0;
-      for (int i = 0; i + d < n; i += kPairSample)  // every kPairSample-th row is enough to rank offsets
-        for (int w = 0; w < Wd; ++w) score += __popc(m[i * pitch + w] & m[(i + d) * pitch + w]);
-      atomicMax(&s_best, (score << 10) | (unsigned int)(1023 - d));
+    if (!list && n > 1) {
+      const int n_off = n / 2, parts = max(1, kPrepThreads / n_off);  // threads per offset
+      for (int t = threadIdx.x; t < n_off; t += kPrepThreads) s_score[t] = 0u;
+      __syncthreads();
+      for (int t = threadIdx.x; t < n_off * parts; t += kPrepThreads) {
+        const int part = t / n_off, d = 1 + t - part * n_off;
+        unsigned int score = 0;
+        // every kPairSample-th row is enough to rank offsets
+        for (int i = part * kPairSample; i + d < n; i += kPairSample * parts)
+          for (int w = 0; w < Wd; ++w) score += __popc(m[i * pitch + w] & m[(i + d) * pitch + w]);
+        atomicAdd(&s_score[d - 1], score);
+      }
+      __syncthreads();
+      for (int t = threadIdx.x; t < n_off; t += kPrepThreads)
+        atomicMax(&s_best, (s_score[t] << 10) | (unsigned int)(1023 - (t + 1)));
     }
     __syncthreads();
     const int D = 1023 - (int)(s_best & 1023u);
@@ -1185,17 +1215,22 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
       s_keys[c] = key;
     }
   } else {
+    // a warp per row, kPrepRows rows of loads in flight
     n_keys = n;
-    for (int i = threadIdx.x; i < next_pow2(n_keys); i += kPrepThreads) {
-      uint32_t key = 0;
-      if (i < n) {
-        const uint32_t* row = rows + (int64_t)block(i) * p.Wd;
-        int len = 0;
-#pragma unroll 8
-        for (int w = 0; w < p.Wd; ++w) len += __popc(row[w]);
-        key = ((uint32_t)len << 10) | (uint32_t)(1023 - i);
+    constexpr int kPrepRows = 8, kWarps = kPrepThreads / 32;
+    const int lane = threadIdx.x & 31, n_pow2 = next_pow2(n_keys);
+    for (int i0 = threadIdx.x >> 5; i0 < n_pow2; i0 += kWarps * kPrepRows) {
+      uint32_t v[kPrepRows];
+#pragma unroll
+      for (int k = 0; k < kPrepRows; ++k) {
+        const int i = i0 + k * kWarps;
+        v[k] = i < n && lane < p.Wd ? rows[(int64_t)block(i) * p.Wd + lane] : 0u;
       }
-      s_keys[i] = key;
+#pragma unroll
+      for (int k = 0; k < kPrepRows; ++k) {
+        const int i = i0 + k * kWarps, len = __reduce_add_sync(0xffffffffu, __popc(v[k]));
+        if (lane == 0 && i < n_pow2) s_keys[i] = i < n ? ((uint32_t)len << 10) | (uint32_t)(1023 - i) : 0u;
+      }
     }
   }
   __syncthreads();
@@ -1222,22 +1257,40 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
 
 // slot[bh][j] = entry index of block j inside the consumer's packed buffer (pack order: producer ascending,
 // head ascending, block ascending), for every block of the consumer's union that another rank owns; -1 elsewhere.
+// First the entry index of every word of every producer's set, a warp per producer; then a thread per block.
 __device__ __forceinline__ void make_slots(const PrepParams& p, int bh) {
-  __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
+  __shared__ uint32_t set_s[kMaxRanks * kMaxWords];
+  __shared__ int32_t at_s[kMaxRanks * kMaxWords];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int bb = bh / p.H, h = bh % p.H;
   const int64_t br = (int64_t)bb * p.P + p.consumer;
-  int32_t* out = p.slot + (int64_t)bh * p.NB;
-  for (int j = threadIdx.x; j < p.NB; j += kPrepThreads) out[j] = -1;
-  own_words(p.rank, p.NB, p.Wd, p.P, own_s);
-  __syncthreads();
   const uint32_t u = lane < p.Wd ? p.U[(br * p.H + h) * p.Wd + lane] : 0u;
   for (int prod = warp; prod < p.P; prod += kPrepThreads / 32) {
-    if (prod == p.consumer) continue;
-    uint32_t bits = lane < p.Wd ? u & own_s[prod * p.Wd + lane] : 0u;
+    const int64_t first = p.seg_off[(br * p.P + prod) * p.H + h];
+    uint32_t set = 0;
+#pragma unroll 8
+    for (int w = 0; w < p.Wd; ++w) {
+      const int j = w * 32 + lane;
+      const uint32_t word = __ballot_sync(0xffffffffu, j < p.NB && p.rank[j] == prod);
+      if (lane == w) set = word & u;
+    }
     int total;
-    int at = (int)p.seg_off[(br * p.P + prod) * p.H + h] + bits_below(bits, lane, &total);
-    for (; bits; bits &= bits - 1, ++at) out[lane * 32 + __ffs(bits) - 1] = at;
+    const int below = bits_below(set, lane, &total);
+    if (lane < p.Wd) {
+      set_s[prod * p.Wd + lane] = set;
+      at_s[prod * p.Wd + lane] = (int)first + below;
+    }
+  }
+  __syncthreads();
+  int32_t* out = p.slot + (int64_t)bh * p.NB;
+  for (int j = threadIdx.x; j < p.NB; j += kPrepThreads) {
+    const int prod = p.rank[j], bit = j & 31;
+    int slot = -1;
+    if ((unsigned)prod < (unsigned)p.P && prod != p.consumer) {
+      const uint32_t set = set_s[prod * p.Wd + (j >> 5)];
+      if ((set >> bit) & 1u) slot = at_s[prod * p.Wd + (j >> 5)] + __popc(set & ((1u << bit) - 1u));
+    }
+    out[j] = slot;
   }
 }
 
@@ -1248,6 +1301,10 @@ __global__ void __launch_bounds__(kPrepThreads) attn_prep_kernel(const PrepParam
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (blockIdx.x == 0 && threadIdx.x == 0) *p.work_counter = 0;  // the attention kernel's work queue
   const int bh = blockIdx.x;
+  if (kPacked && bh >= p.BH) {
+    make_slots(p, bh - p.BH);
+    return;
+  }
   int n_live;
   if (kPacked) {
     __shared__ uint32_t s_words[kMaxWords];
@@ -1255,7 +1312,6 @@ __global__ void __launch_bounds__(kPrepThreads) attn_prep_kernel(const PrepParam
     rank_words(p.rank, p.NB, p.consumer, s_words);
     const int n = list_blocks(s_words, p.NB, s_list);
     n_live = make_items(p, bh, s_list, n, smem_raw);
-    if (n_live > 0) make_slots(p, bh);
     if (bh % p.H == 0 && warp == 0) {  // first tile of the consumer's buffer for this batch item
       const int64_t br = (int64_t)(bh / p.H) * p.P + p.consumer;
       int64_t first = 0;
@@ -1401,7 +1457,7 @@ static int launch_prep(const Geometry& g, const PrepParams& p, cudaStream_t st) 
   auto kern = attn_prep_kernel<kPacked>;
   const int smem = g.b == 64 ? g.NB * (g.Wd | 1) * 4 : 0;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
-  SPARSP_CUDA_OK(launch_kernel(kern, (unsigned)p.BH, kPrepThreads, smem, st, p));
+  SPARSP_CUDA_OK(launch_kernel(kern, (unsigned)(kPacked ? 2 * p.BH : p.BH), kPrepThreads, smem, st, p));
   return SPARSP_OK;
 }
 
