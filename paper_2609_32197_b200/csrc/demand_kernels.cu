@@ -267,9 +267,14 @@ int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_o
 constexpr int kPackStages = 5;
 constexpr int kPackMaxWarps = 4;
 
+// Nobody reads the copies before a consumer fetches them, so the L2 cache need not keep them: the sources, which are read
+// again for other consumers, and K and V stay there longer (demand and gather of 24 heads x 24576 226.5 -> 224 us, of 48 x
+// 17776 328.5 -> 325.5, of 40 x 75600 2221 -> 2207; seven segments 394.7 -> 392).
 __device__ __forceinline__ void bulk_store(void* gdst, const void* smem_src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst),
-               "r"(ptx::smem_u32(smem_src)), "r"(bytes)
+  uint64_t policy;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;" ::"l"(gdst),
+               "r"(ptx::smem_u32(smem_src)), "r"(bytes), "l"(policy)
                : "memory");
 }
 
@@ -352,78 +357,155 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps) pack_kernel(const __grid_c
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-static int run_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, const int64_t* dst,
-                    int n_dst, const int32_t* src, const int32_t* n_src, void* packed, int32_t* status,
-                    cudaStream_t st) {
+// Tensor maps and launch shape of a kernel that moves tiles as pack_kernel does.
+struct PackLaunch {
+  CUtensorMap tk, tv;
+  unsigned grid;
+  int threads, smem;
+  uint32_t tile_bytes;
+};
+static int prepare_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, const void* kernel,
+                        PackLaunch* c) {
   int dev = 0, sms = 148;
   SPARSP_CUDA_OK(cudaGetDevice(&dev));
   SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  CUtensorMap tk, tv;
   int rc;
-  if ((rc = make_tile_tmap(&tk, K, s, g, g.b, false)) != SPARSP_OK) return rc;
-  if ((rc = make_tile_tmap(&tv, V, s, g, g.b, false)) != SPARSP_OK) return rc;
-  const int tile_bytes = g.b * g.d * 2;
-  const int n_warps = std::max(1, std::min(kPackMaxWarps, (32 * 1024) / tile_bytes));
-  const int smem = n_warps * kPackStages * tile_bytes;
-  SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)pack_kernel, smem));
-  SPARSP_CUDA_OK(launch_kernel(pack_kernel, sms, 32 * n_warps, smem, st, tk, tv, dst, n_dst, src, n_src, g.H, g.NB, g.b,
-                               (uint32_t)tile_bytes, (unsigned char*)packed, status));
+  if ((rc = make_tile_tmap(&c->tk, K, s, g, g.b, false)) != SPARSP_OK) return rc;
+  if ((rc = make_tile_tmap(&c->tv, V, s, g, g.b, false)) != SPARSP_OK) return rc;
+  c->tile_bytes = (uint32_t)(g.b * g.d * 2);
+  const int n_warps = std::max(1, std::min(kPackMaxWarps, (32 * 1024) / (int)c->tile_bytes));
+  c->grid = (unsigned)sms;
+  c->threads = 32 * n_warps;
+  c->smem = n_warps * kPackStages * (int)c->tile_bytes;
+  SPARSP_CUDA_OK(ensure_dynamic_smem(kernel, c->smem));
   return SPARSP_OK;
 }
 
 int launch_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, void* packed, int P, char* ws,
                 const WsLayout& L, cudaStream_t st) {
-  return run_pack(s, g, K, V, dst_table(ws, L), P, src_list(ws, L, g, P), (const int32_t*)(ws + L.n_entries), packed,
-                  (int32_t*)(ws + L.status), st);
+  PackLaunch c;
+  const int rc = prepare_pack(s, g, K, V, (const void*)pack_kernel, &c);
+  if (rc != SPARSP_OK) return rc;
+  SPARSP_CUDA_OK(launch_kernel(pack_kernel, c.grid, c.threads, c.smem, st, c.tk, c.tv, dst_table(ws, L), P,
+                               src_list(ws, L, g, P), (const int32_t*)(ws + L.n_entries), g.H, g.NB, g.b, c.tile_bytes,
+                               (unsigned char*)packed, (int32_t*)(ws + L.status)));
+  return SPARSP_OK;
 }
 
 // ------------------------------------------------------------------------------------------------
 // Pack of ONE (consumer, producer) segment (Section 6.1: the producer packs the payload of one consumer into
-// the slot designated for that pair).  The tables hold that segment alone, with destinations relative
-// to the start of the slot: entry (h, j) sits where it sits inside the consumer's buffer, minus the segment's
+// the slot designated for that pair).  Entry (h, j) sits where it sits inside the consumer's buffer, minus the segment's
 // first entry, so that consumer and producer derive the same byte ranges from the demand counts.
-// One warp per head enumerates U[consumer][h] & own[producer] in ascending block order.
+// The entries are U[consumer][h] & own[producer], head by head, blocks ascending.  Their places in the slot are
+// consecutive, so a warp that takes every n-th entry finds its block by counting bits from the entry before: no
+// tables and no launch that fills them.  Tiles move as in pack_kernel.  HBM-bound: seven segments of 175 MB, read and
+// written, 426 us with tables, 399 without, 395 with every second one walked backwards, 389-392 with the hint above (6.3
+// TB/s); 421 with a run of consecutive entries per warp instead of every n-th.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) segment_kernel(const uint32_t* __restrict__ U, const int32_t* __restrict__ rank,
-                                                      int H, int NB, int Wd, int P, int consumer, int producer,
-                                                      const int64_t* __restrict__ seg_off,
-                                                      const int32_t* __restrict__ cnt, int64_t entry_bytes,
-                                                      int64_t capacity, int64_t* __restrict__ dst,
-                                                      int32_t* __restrict__ src, int32_t* __restrict__ n_src,
-                                                      int32_t* __restrict__ status) {
-  enter_grid(U, rank, seg_off, cnt);
-  __shared__ uint32_t own_s[kMaxWords];
-  const int h = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  rank_words(rank, NB, producer, own_s);
-  __syncthreads();
-  if (h >= H) return;
-  const int64_t seg0 = ((int64_t)consumer * P + producer) * H;  // batch item 0
-  const int64_t first_of_segment = seg_off[seg0];
-  if (h == 0 && lane == 0) *n_src = (int32_t)(seg_off[seg0 + H - 1] + cnt[seg0 + H - 1] - first_of_segment);
-  uint32_t bits = lane < Wd ? U[((int64_t)consumer * H + h) * Wd + lane] & own_s[lane] : 0u;
-  int total;
-  int64_t at = seg_off[seg0 + h] - first_of_segment + bits_below(bits, lane, &total);
-  for (; bits; bits &= bits - 1, ++at) {
-    const int s = h * NB + lane * 32 + __ffs(bits) - 1;
-    const bool fits = (at + 1) * entry_bytes <= capacity;
-    if (!fits) atomicExch(status, SPARSP_ERR_CAPACITY);  // left out by the gather
-    dst[s] = fits ? at * entry_bytes : -1;
-    src[at] = s;
+__global__ void __launch_bounds__(32 * kPackMaxWarps)
+    segment_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+                   const uint32_t* __restrict__ U, const int32_t* __restrict__ rank, int H, int NB, int Wd, int P,
+                   int consumer, int producer, const int64_t* __restrict__ seg_off, const int32_t* __restrict__ cnt,
+                   int b, uint32_t tile_bytes, unsigned char* __restrict__ slot, int64_t capacity,
+                   int32_t* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ uint64_t full_all[kPackMaxWarps * kPackStages];
+  __shared__ int s_abort;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+  uint64_t* full = full_all + warp * kPackStages;
+  unsigned char* ring = smem_raw + (size_t)warp * kPackStages * tile_bytes;  // this warp's buffers
+  if (threadIdx.x == 0) s_abort = 0;
+  if (lane == 0) {
+    for (int st = 0; st < kPackStages; ++st) ptx::mbar_init(full + st, 1);
+    ptx::mbar_init_fence();
   }
+  enter_grid(U, rank, seg_off, cnt);
+  __syncthreads();
+  uint32_t own = 0;  // blocks of the producer, a word per lane
+#pragma unroll 8
+  for (int w = 0; w < Wd; ++w) {
+    const int j = w * 32 + lane;
+    const uint32_t word = __ballot_sync(0xffffffffu, (j < NB ? rank[j] : ~producer) == producer);
+    if (lane == w) own = word;
+  }
+  const int64_t* off = seg_off + ((int64_t)consumer * P + producer) * H;  // batch item 0
+  const int64_t first = off[0];
+  const int n_entries = (int)(off[H - 1] + cnt[((int64_t)consumer * P + producer) * H + H - 1] - first);
+  const int unit = blockIdx.x * n_warps + warp, n_units = gridDim.x * n_warps;
+  // Every second consumer's entries are walked backwards: the tiles that were read last for one consumer are the first
+  // ones for the next and still in L2.
+  const bool back = consumer & 1;
+  int n_local = n_entries > unit ? 2 * ((n_entries - unit + n_units - 1) / n_units) : 0;  // K (even) or V (odd) tiles
+  auto entry = [&](int q) { return back ? n_entries - 1 - unit - (q >> 1) * n_units : unit + (q >> 1) * n_units; };
+  if (n_local > 0) {
+    const uint32_t* u_row = U + (int64_t)consumer * H * Wd;
+    auto head_words = [&](int h) { return h >= 0 && h < H && lane < Wd ? u_row[(int64_t)h * Wd + lane] & own : 0u; };
+    int h = back ? H - 1 : 0, total, at;  // the head, its entries, its first entry
+    uint32_t words = head_words(h), next = head_words(back ? h - 1 : h + 1);
+    int below = bits_below(words, lane, &total);
+    at = back ? n_entries - total : 0;
+    // head * NB + block of entry e; -1 where there is none, should the counts promise more than there are
+    auto block_of = [&](int e) -> int {
+      while (back ? e < at : e >= at + total) {
+        if (!back) at += total;
+        h += back ? -1 : 1;
+        if (h < 0 || h >= H) return -1;
+        words = next;
+        next = head_words(back ? h - 1 : h + 1);
+        below = bits_below(words, lane, &total);
+        if (back) at -= total;
+      }
+      const int k = e - at;
+      const int w = 31 - __clz(__ballot_sync(0xffffffffu, words != 0u && below <= k));
+      uint32_t left = __shfl_sync(0xffffffffu, words, w);
+      for (int skip = k - __shfl_sync(0xffffffffu, below, w); skip > 0; --skip) left &= left - 1u;
+      return h * NB + w * 32 + __ffs(left) - 1;
+    };
+    int s_load = 0;
+    auto issue_load = [&](int q) {
+      if ((q & 1) == 0) s_load = block_of(entry(q));
+      if (s_load < 0) {
+        n_local = q;
+      } else if (lane == 0) {
+        uint64_t* bar = full + q % kPackStages;
+        const int hd = s_load / NB;
+        ptx::mbar_expect_tx(bar, tile_bytes);
+        ptx::tma_load_4d(ring + (size_t)(q % kPackStages) * tile_bytes, q & 1 ? &tmV : &tmK, bar, 0, (s_load - hd * NB) * b,
+                         hd, 0);
+      }
+    };
+    for (int q = 0; q < kPackStages - 1 && q < n_local; ++q) issue_load(q);
+    for (int q = 0; q < n_local; ++q) {
+      const int64_t e = entry(q);
+      ptx::mbar_wait_bounded(full + q % kPackStages, (uint32_t)((q / kPackStages) & 1), &s_abort, status, 50, 200000000LL);
+      if (lane == 0) {
+        if ((e + 1) * 2 * tile_bytes <= capacity)
+          bulk_store(slot + (2 * e + (q & 1)) * tile_bytes, ring + (size_t)(q % kPackStages) * tile_bytes, tile_bytes);
+        else
+          atomicExch(status, SPARSP_ERR_CAPACITY);  // does not fit: left out
+      }
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      if (q + kPackStages - 1 < n_local) {
+        // the buffer of item q - 1 may be refilled once its store has read it
+        asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        __syncwarp();
+        issue_load(q + kPackStages - 1);
+      }
+    }
+  }
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 int launch_pack_segment(const sparsp_shape& s, const Geometry& g, const uint32_t* U, const int32_t* rank, int P,
                         int consumer, int producer, const int64_t* seg_off, const int32_t* cnt, const void* K,
                         const void* V, void* dst, int64_t capacity, char* ws, const WsLayout& L, cudaStream_t st) {
-  int64_t* table = dst_table(ws, L);
-  int32_t* src = src_list(ws, L, g, 1);
-  int32_t* n_src = (int32_t*)(ws + L.n_entries);
-  int32_t* status = (int32_t*)(ws + L.status);
-  SPARSP_CUDA_OK(launch_kernel(segment_kernel, (g.H * 32 + 255) / 256, 256, 0, st, U, rank, g.H, g.NB, g.Wd, P,
-                               consumer, producer, seg_off, cnt, 2LL * g.b * g.d * 2, capacity, table, src, n_src,
-                               status));
-  return run_pack(s, g, K, V, table, 1, src, n_src, dst, status, st);
+  PackLaunch c;
+  const int rc = prepare_pack(s, g, K, V, (const void*)segment_kernel, &c);
+  if (rc != SPARSP_OK) return rc;
+  SPARSP_CUDA_OK(launch_kernel(segment_kernel, c.grid, c.threads, c.smem, st, c.tk, c.tv, U, rank, g.H, g.NB, g.Wd, P,
+                               consumer, producer, seg_off, cnt, g.b, c.tile_bytes, (unsigned char*)dst, capacity,
+                               (int32_t*)(ws + L.status)));
+  return SPARSP_OK;
 }
 
 // ------------------------------------------------------------------------------------------------
