@@ -1,6 +1,6 @@
 """Items whose scores leave the range that the attention kernel assumes are computed again: relative to their first tile,
 then with the running maximum.  Rows of all three kinds among many items per CTA, the last items of the call among them,
-against a masked softmax in 64 bits."""
+against a masked softmax in 64 bits.  And 64-token blocks where every one has an SM of its own, at the edge of that rule."""
 import math
 
 import pytest
@@ -83,3 +83,34 @@ def test_items_that_leave_the_range(binding, d, b, large, keep):
                                               dm["seg_total"], dm["packed"], dm["packed"].numel(), None, 0.0, O, lse, ws)
         assert binding.sparsp_status(ws) == binding.SPARSP_OK
         check(O, lse, torch.nonzero(rank.repeat_interleave(b)[:N] == consumer)[:, 0])
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("layout", ["HND", "NHD"])
+@pytest.mark.parametrize("spare", [-1, 0, 1])
+def test_as_many_blocks_as_multiprocessors(binding, d, layout, spare):
+    sms, b, B = torch.cuda.get_device_properties(0).multi_processor_count, 64, 2
+    H, NB = 1, (sms + 2 * spare) // B  # two batch items
+    N = NB * b - 21
+    g = torch.Generator(device="cuda").manual_seed(d + NB)
+    Q, K, V = (torch.randn(B, N, d, generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    kept = torch.rand(B, NB, NB, generator=g, device="cuda") < 0.3
+    kept[:, 5] = False                 # a block that keeps nothing
+    kept[:, 7] = False
+    kept[:, 7, NB - 1] = True          # the ragged block alone
+    words = torch.zeros(B, H, NB, (NB + 31) // 32, dtype=torch.int64, device="cuda")
+    for j in range(NB):
+        words[:, 0, :, j // 32] |= kept[:, :, j].long() << (j % 32)
+    mask = torch.where(words >= 1 << 31, words - (1 << 32), words).to(torch.int32).contiguous()
+    want, want_lse = _reference(Q, K, V, kept, b)
+    shape = binding.make_shape(H, d, (1, 1, N), 0, b, batch=B, layout=layout)
+    ws = binding.make_workspace(shape, 2)
+    q, k, v = ((x[:, None] if layout == "HND" else x[:, :, None]).contiguous() for x in (Q, K, V))
+    O, lse = torch.full_like(q, 7.0), torch.full((B, H, N), 7.0, device="cuda")
+    binding.sparsp_sparse_attn_fwd(shape, q, k, v, mask, 0.0, O, lse, ws)
+    assert binding.sparsp_status(ws) == binding.SPARSP_OK
+    rows = kept.any(-1).repeat_interleave(b, 1)[:, :N]
+    out = O.reshape(B, N, d).double()
+    assert (out - want)[rows].abs().max() <= pu.ATTN_MAX_ABS
+    assert (lse[:, 0].double() - want_lse)[rows].abs().max() <= 2e-2
+    assert bool((out[~rows] == 0).all()) and bool((lse[:, 0][~rows] == float("-inf")).all())
