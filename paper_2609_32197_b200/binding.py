@@ -37,6 +37,22 @@ EXPORTS = [
 ]
 SPARSP_XCHG_HOST_MEMORY = 1
 
+# Argument types of the calls that a layer makes (s: shape, p: pointer, i / l: 32 / 64-bit integer, f: float), so that ctypes
+# converts plain values itself: a ctypes object per argument costs more than the call.
+_SIGNATURES = {
+    "sparsp_block_mask": "sppippppppp",
+    "sparsp_block_mask_cdf": "sppffpppppp",
+    "sparsp_demand_pack": "sppiipppppppplppp",
+    "sparsp_demand_plan_noalloc": "sppiipppppp",
+    "sparsp_sparse_attn_fwd": "sppppfpppp",
+    "sparsp_sparse_attn_fwd_packed": "spppppiipppplpfpppp",
+    "sparsp_hop_mask": "sppiiipp",
+    "sparsp_hop_chunk_mask": "sppiiiiipp",
+    "sparsp_attn_merge": "sppppppp",
+    "sparsp_attn_merge_rows": "spppppppiiiip",
+    "sparsp_pack_segment": "sppiiippppplpp",
+}
+
 
 class SparspError(RuntimeError):
     def __init__(self, code: int, text: str):
@@ -74,6 +90,10 @@ def lib() -> ctypes.CDLL:
         L.sparsp_resolve_topk.restype = ctypes.c_int32
         for name in EXPORTS:
             getattr(L, name)  # AttributeError if a declared symbol is not exported
+        kinds = {"s": ctypes.POINTER(sparsp_shape), "p": ctypes.c_void_p, "i": ctypes.c_int32, "l": ctypes.c_int64,
+                 "f": ctypes.c_float}
+        for name, args in _SIGNATURES.items():
+            getattr(L, name).argtypes = [kinds[a] for a in args]
         _lib = L
     return _lib
 
@@ -89,9 +109,18 @@ def _ptr(t):
     return ctypes.c_void_p(t.data_ptr())
 
 
+def _data(t):
+    """Data pointer of a tensor as a plain value, None for None."""
+    return None if t is None else t.data_ptr()
+
+
+def _stream_handle():
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
 def _stream():
     # the handle itself: torch.cuda.current_stream() builds a Stream object around it, 3 us per call
-    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return ctypes.c_void_p(_stream_handle())
 
 
 @dataclass
@@ -202,75 +231,68 @@ def make_workspace(shape: sparsp_shape, n_ranks: int, device="cuda") -> torch.Te
 
 
 def sparsp_block_mask(shape, Q, K, topk_video, mask, kv_list, kv_count, pooled_q, pooled_k, workspace):
-    _check(lib().sparsp_block_mask(ctypes.byref(shape), _ptr(Q), _ptr(K), ctypes.c_int32(topk_video),
-                                   _ptr(mask), _ptr(kv_list), _ptr(kv_count), _ptr(pooled_q),
-                                   _ptr(pooled_k), _ptr(workspace), _stream()))
+    _check(lib().sparsp_block_mask(shape, _data(Q), _data(K), topk_video, _data(mask), _data(kv_list),
+                                   _data(kv_count), _data(pooled_q), _data(pooled_k), _data(workspace),
+                                   _stream_handle()))
 
 
 def sparsp_block_mask_cdf(shape, Q, K, tau, score_scale, mask, kv_count, pooled_q, pooled_k, workspace):
-    _check(lib().sparsp_block_mask_cdf(ctypes.byref(shape), _ptr(Q), _ptr(K), ctypes.c_float(tau),
-                                       ctypes.c_float(score_scale), _ptr(mask), _ptr(kv_count), _ptr(pooled_q),
-                                       _ptr(pooled_k), _ptr(workspace), _stream()))
+    _check(lib().sparsp_block_mask_cdf(shape, _data(Q), _data(K), tau, score_scale, _data(mask), _data(kv_count),
+                                       _data(pooled_q), _data(pooled_k), _data(workspace), _stream_handle()))
 
 
 def sparsp_demand_pack(shape, mask, rank_of_block, n_ranks, flags, K, V, union_mask, cnt, seg_offset,
                        seg_total, volume_bytes, packed, packed_capacity_bytes, dst_base_bytes, workspace):
-    _check(lib().sparsp_demand_pack(ctypes.byref(shape), _ptr(mask), _ptr(rank_of_block),
-                                    ctypes.c_int32(n_ranks), ctypes.c_int32(flags), _ptr(K), _ptr(V),
-                                    _ptr(union_mask), _ptr(cnt), _ptr(seg_offset), _ptr(seg_total),
-                                    _ptr(volume_bytes), _ptr(packed), ctypes.c_int64(packed_capacity_bytes),
-                                    _ptr(dst_base_bytes), _ptr(workspace), _stream()))
+    _check(lib().sparsp_demand_pack(shape, _data(mask), _data(rank_of_block), n_ranks, flags, _data(K), _data(V),
+                                    _data(union_mask), _data(cnt), _data(seg_offset), _data(seg_total),
+                                    _data(volume_bytes), _data(packed), packed_capacity_bytes, _data(dst_base_bytes),
+                                    _data(workspace), _stream_handle()))
 
 
 def sparsp_demand_plan_noalloc(shape, mask, rank_of_block, n_ranks, flags, union_mask, cnt, seg_offset, seg_total,
                                volume_bytes):
     """Planning half of sparsp_demand_pack for callers that cannot allocate device memory: no workspace
     argument, the scratch is a small array inside the library.  Outputs as for SPARSP_PLAN_ONLY."""
-    _check(lib().sparsp_demand_plan_noalloc(ctypes.byref(shape), _ptr(mask), _ptr(rank_of_block),
-                                            ctypes.c_int32(n_ranks), ctypes.c_int32(flags), _ptr(union_mask),
-                                            _ptr(cnt), _ptr(seg_offset), _ptr(seg_total), _ptr(volume_bytes),
-                                            _stream()))
+    _check(lib().sparsp_demand_plan_noalloc(shape, _data(mask), _data(rank_of_block), n_ranks, flags,
+                                            _data(union_mask), _data(cnt), _data(seg_offset), _data(seg_total),
+                                            _data(volume_bytes), _stream_handle()))
 
 
 def sparsp_sparse_attn_fwd(shape, Q, K, V, mask, softmax_scale, O, lse, workspace):
-    _check(lib().sparsp_sparse_attn_fwd(ctypes.byref(shape), _ptr(Q), _ptr(K), _ptr(V), _ptr(mask),
-                                        ctypes.c_float(softmax_scale), _ptr(O), _ptr(lse), _ptr(workspace),
-                                        _stream()))
+    _check(lib().sparsp_sparse_attn_fwd(shape, _data(Q), _data(K), _data(V), _data(mask), softmax_scale, _data(O),
+                                        _data(lse), _data(workspace), _stream_handle()))
 
 
 def sparsp_sparse_attn_fwd_packed(shape, Q, K, V, mask, rank_of_block, n_ranks, consumer, union_mask, seg_offset,
                                   seg_total, packed, packed_capacity_bytes, dst_base_bytes, softmax_scale, O, lse,
                                   workspace):
-    _check(lib().sparsp_sparse_attn_fwd_packed(ctypes.byref(shape), _ptr(Q), _ptr(K), _ptr(V), _ptr(mask),
-                                               _ptr(rank_of_block), ctypes.c_int32(n_ranks), ctypes.c_int32(consumer),
-                                               _ptr(union_mask), _ptr(seg_offset), _ptr(seg_total), _ptr(packed),
-                                               ctypes.c_int64(packed_capacity_bytes), _ptr(dst_base_bytes),
-                                               ctypes.c_float(softmax_scale), _ptr(O), _ptr(lse), _ptr(workspace),
-                                               _stream()))
+    _check(lib().sparsp_sparse_attn_fwd_packed(shape, _data(Q), _data(K), _data(V), _data(mask), _data(rank_of_block),
+                                               n_ranks, consumer, _data(union_mask), _data(seg_offset),
+                                               _data(seg_total), _data(packed), packed_capacity_bytes,
+                                               _data(dst_base_bytes), softmax_scale, _data(O), _data(lse),
+                                               _data(workspace), _stream_handle()))
 
 
 def sparsp_hop_mask(shape, mask, rank_of_block, n_ranks, consumer, producer, hop_mask):
-    _check(lib().sparsp_hop_mask(ctypes.byref(shape), _ptr(mask), _ptr(rank_of_block), ctypes.c_int32(n_ranks),
-                                 ctypes.c_int32(consumer), ctypes.c_int32(producer), _ptr(hop_mask), _stream()))
+    _check(lib().sparsp_hop_mask(shape, _data(mask), _data(rank_of_block), n_ranks, consumer, producer,
+                                 _data(hop_mask), _stream_handle()))
 
 
 def sparsp_hop_chunk_mask(shape, mask, rank_of_block, n_ranks, consumer, producer, head_begin, head_end, hop_mask):
-    _check(lib().sparsp_hop_chunk_mask(ctypes.byref(shape), _ptr(mask), _ptr(rank_of_block), ctypes.c_int32(n_ranks),
-                                       ctypes.c_int32(consumer), ctypes.c_int32(producer), ctypes.c_int32(head_begin),
-                                       ctypes.c_int32(head_end), _ptr(hop_mask), _stream()))
+    _check(lib().sparsp_hop_chunk_mask(shape, _data(mask), _data(rank_of_block), n_ranks, consumer, producer,
+                                       head_begin, head_end, _data(hop_mask), _stream_handle()))
 
 
 def sparsp_attn_merge(shape, O_a, lse_a, O_b, lse_b, O, lse):
-    _check(lib().sparsp_attn_merge(ctypes.byref(shape), _ptr(O_a), _ptr(lse_a), _ptr(O_b), _ptr(lse_b), _ptr(O),
-                                   _ptr(lse), _stream()))
+    _check(lib().sparsp_attn_merge(shape, _data(O_a), _data(lse_a), _data(O_b), _data(lse_b), _data(O), _data(lse),
+                                   _stream_handle()))
 
 
 def sparsp_attn_merge_rows(shape, O_a, lse_a, O_b, lse_b, O, lse, rank_of_block, n_ranks, consumer, head_begin,
                            head_end):
-    _check(lib().sparsp_attn_merge_rows(ctypes.byref(shape), _ptr(O_a), _ptr(lse_a), _ptr(O_b), _ptr(lse_b), _ptr(O),
-                                        _ptr(lse), _ptr(rank_of_block), ctypes.c_int32(n_ranks),
-                                        ctypes.c_int32(consumer), ctypes.c_int32(head_begin), ctypes.c_int32(head_end),
-                                        _stream()))
+    _check(lib().sparsp_attn_merge_rows(shape, _data(O_a), _data(lse_a), _data(O_b), _data(lse_b), _data(O),
+                                        _data(lse), _data(rank_of_block), n_ranks, consumer, head_begin, head_end,
+                                        _stream_handle()))
 
 
 def _addr(x):
@@ -294,10 +316,9 @@ def _stream_of(stream):
 def sparsp_pack_segment(shape, union_mask, rank_of_block, n_ranks, consumer, producer, cnt, seg_offset, K, V, dst,
                         dst_capacity_bytes, workspace):
     """dst: a tensor or a raw device address (a slot of the producer's window)."""
-    _check(lib().sparsp_pack_segment(ctypes.byref(shape), _ptr(union_mask), _ptr(rank_of_block),
-                                     ctypes.c_int32(n_ranks), ctypes.c_int32(consumer), ctypes.c_int32(producer),
-                                     _ptr(cnt), _ptr(seg_offset), _ptr(K), _ptr(V), _addr(dst),
-                                     ctypes.c_int64(dst_capacity_bytes), _ptr(workspace), _stream()))
+    _check(lib().sparsp_pack_segment(shape, _data(union_mask), _data(rank_of_block), n_ranks, consumer, producer,
+                                     _data(cnt), _data(seg_offset), _data(K), _data(V), _addr(dst),
+                                     dst_capacity_bytes, _data(workspace), _stream_handle()))
 
 
 def sparsp_xchg_flag_bytes(n_ranks: int, window: int) -> int:
