@@ -413,11 +413,11 @@ int sparsp_demand_pack(const sparsp_shape* shape, const uint32_t* mask, const in
   char* ws = (char*)workspace;
   const WsLayout L = make_layout(g, n_ranks);
   cudaStream_t st = (cudaStream_t)stream;
-  SPARSP_TRY(launch_demand(g, mask, rank_of_block, n_ranks, flags, union_mask, cnt, seg_offset,
-                           seg_total, volume_bytes, dst_base_bytes,
-                           plan_only ? (int64_t)-1 : packed_capacity_bytes, ws, L, st));
-  if (!plan_only) SPARSP_TRY(launch_pack(*shape, g, K, V, packed, n_ranks, ws, L, st));
-  return SPARSP_OK;
+  if (plan_only)
+    return launch_demand(g, mask, rank_of_block, n_ranks, flags, union_mask, cnt, seg_offset, seg_total, volume_bytes, ws,
+                         L, st);
+  return launch_demand_pack(*shape, g, mask, rank_of_block, n_ranks, flags, K, V, union_mask, cnt, seg_offset, seg_total,
+                            volume_bytes, packed, packed_capacity_bytes, dst_base_bytes, ws, L, st);
 }
 
 int sparsp_pack_segment(const sparsp_shape* shape, const uint32_t* union_mask, const int32_t* rank_of_block,

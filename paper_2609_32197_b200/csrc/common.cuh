@@ -105,12 +105,13 @@ int launch_score_cdf(const Geometry& g, const float* pq, const float* pk, float*
                      uint32_t* mask, int32_t* kv_count, cudaStream_t st);
 int launch_score_topk(const Geometry& g, const float* pq, const float* pk, float* scores, int topk,
                       uint32_t* mask, int32_t* kv_list, int32_t* kv_count, cudaStream_t st);
-int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_of_block, int P,
-                  int flags, uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total,
-                  int64_t* volume, const int64_t* dst_base, int64_t capacity, char* ws,
-                  const WsLayout& L, cudaStream_t st);
-int launch_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, void* packed, int P, char* ws,
-                const WsLayout& L, cudaStream_t st);
+int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_of_block, int P, int flags, uint32_t* U,
+                  int32_t* cnt, int64_t* seg_off, int64_t* seg_total, int64_t* volume, char* ws, const WsLayout& L,
+                  cudaStream_t st);
+int launch_demand_pack(const sparsp_shape& s, const Geometry& g, const uint32_t* mask, const int32_t* rank, int P,
+                       int flags, const void* K, const void* V, uint32_t* U, int32_t* cnt, int64_t* seg_off,
+                       int64_t* seg_total, int64_t* volume, void* packed, int64_t capacity, const int64_t* dst_base,
+                       char* ws, const WsLayout& L, cudaStream_t st);
 int launch_pack_segment(const sparsp_shape& s, const Geometry& g, const uint32_t* U, const int32_t* rank, int P,
                         int consumer, int producer, const int64_t* seg_off, const int32_t* cnt, const void* K,
                         const void* V, void* dst, int64_t capacity, char* ws, const WsLayout& L, cudaStream_t st);

@@ -221,13 +221,18 @@ static int32_t* received_table(char* ws, const WsLayout& L, const Geometry& g, i
   return src_list(ws, L, g, P) + (int64_t)g.B * g.H * g.NB;
 }
 
+static cudaError_t launch_union(const Geometry& g, const uint32_t* mask, const int32_t* rank, int P, int include_local,
+                                uint32_t* U, int32_t* cnt, int32_t* received, int32_t* n_src, cudaStream_t st) {
+  return launch_kernel(union_count_kernel, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P, U,
+                       include_local, cnt, received, n_src);
+}
+
 // dst, src, n_src, received: NULL for a plan without destinations.
 static cudaError_t launch_plan(const Geometry& g, const uint32_t* mask, const int32_t* rank, int P, int include_local,
                                uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total, int64_t* volume,
                                const int64_t* dst_base, int64_t capacity, int64_t* dst, int32_t* src, int32_t* n_src,
                                int32_t* received, int32_t* status, cudaStream_t st) {
-  cudaError_t e = launch_kernel(union_count_kernel, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P,
-                                U, include_local, cnt, received, n_src);
+  const cudaError_t e = launch_union(g, mask, rank, P, include_local, U, cnt, received, n_src, st);
   if (e != cudaSuccess) return e;
   const int heads = dst ? plan_heads(g.H) : 1;
   const unsigned grid = dst ? (unsigned)((g.B * P + g.B) * ((g.H + heads - 1) / heads)) : (unsigned)(g.B * P);
@@ -236,19 +241,20 @@ static cudaError_t launch_plan(const Geometry& g, const uint32_t* mask, const in
                        capacity, dst, src, n_src, status);
 }
 
-int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_of_block, int P,
-                  int flags, uint32_t* U, int32_t* cnt, int64_t* seg_off, int64_t* seg_total,
-                  int64_t* volume, const int64_t* dst_base, int64_t capacity, char* ws,
-                  const WsLayout& L, cudaStream_t st) {
-  const bool pack = !(flags & SPARSP_PLAN_ONLY);  // a plan alone needs no destinations
-  if (g.B * P > 1024) {
-    set_error("batch * n_ranks = %d exceeds 1024", g.B * P);
-    return SPARSP_ERR_UNSUPPORTED;
-  }
+static int check_consumers(const Geometry& g, int P) {
+  if (g.B * P <= 1024) return SPARSP_OK;
+  set_error("batch * n_ranks = %d exceeds 1024", g.B * P);
+  return SPARSP_ERR_UNSUPPORTED;
+}
+
+int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_of_block, int P, int flags, uint32_t* U,
+                  int32_t* cnt, int64_t* seg_off, int64_t* seg_total, int64_t* volume, char* ws, const WsLayout& L,
+                  cudaStream_t st) {
+  const int rc = check_consumers(g, P);
+  if (rc != SPARSP_OK) return rc;
   SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, P, (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, U, cnt, seg_off,
-                             seg_total, volume, dst_base, capacity, pack ? dst_table(ws, L) : nullptr,
-                             pack ? src_list(ws, L, g, P) : nullptr, pack ? (int32_t*)(ws + L.n_entries) : nullptr,
-                             pack ? received_table(ws, L, g, P) : nullptr, (int32_t*)(ws + L.status), st));
+                             seg_total, volume, nullptr, -1, nullptr, nullptr, nullptr, nullptr,
+                             (int32_t*)(ws + L.status), st));
   return SPARSP_OK;
 }
 
@@ -357,15 +363,15 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps) pack_kernel(const __grid_c
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// Tensor maps and launch shape of a kernel that moves tiles as pack_kernel does.
+// Tensor maps and grid of a kernel that moves tiles as pack_kernel does, and its shared memory.
 struct PackLaunch {
   CUtensorMap tk, tv;
   unsigned grid;
-  int threads, smem;
   uint32_t tile_bytes;
 };
+static int pack_warps(int tile_bytes) { return std::max(1, std::min(kPackMaxWarps, (32 * 1024) / tile_bytes)); }
 static int prepare_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, const void* kernel,
-                        PackLaunch* c) {
+                        int smem, PackLaunch* c) {
   int dev = 0, sms = 148;
   SPARSP_CUDA_OK(cudaGetDevice(&dev));
   SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -373,22 +379,195 @@ static int prepare_pack(const sparsp_shape& s, const Geometry& g, const void* K,
   if ((rc = make_tile_tmap(&c->tk, K, s, g, g.b, false)) != SPARSP_OK) return rc;
   if ((rc = make_tile_tmap(&c->tv, V, s, g, g.b, false)) != SPARSP_OK) return rc;
   c->tile_bytes = (uint32_t)(g.b * g.d * 2);
-  const int n_warps = std::max(1, std::min(kPackMaxWarps, (32 * 1024) / (int)c->tile_bytes));
   c->grid = (unsigned)sms;
-  c->threads = 32 * n_warps;
-  c->smem = n_warps * kPackStages * (int)c->tile_bytes;
-  SPARSP_CUDA_OK(ensure_dynamic_smem(kernel, c->smem));
+  SPARSP_CUDA_OK(ensure_dynamic_smem(kernel, smem));
   return SPARSP_OK;
 }
 
-int launch_pack(const sparsp_shape& s, const Geometry& g, const void* K, const void* V, void* packed, int P, char* ws,
-                const WsLayout& L, cudaStream_t st) {
-  PackLaunch c;
-  const int rc = prepare_pack(s, g, K, V, (const void*)pack_kernel, &c);
+// ------------------------------------------------------------------------------------------------
+// Offsets and gather in one launch, for plans of up to kScanMax counts: every CTA scans the counts of all consumers into
+// shared memory (their flat order is the order of the packed buffers), and a copy's place is its segment's first entry
+// plus the blocks of the segment below it, counted in the union words by the lane of its consumer.  No tables, no list of
+// sources and no launch that makes them.  The first CTAs also write the offsets, totals and volumes.  Tiles move as in
+// pack_kernel, a block's K and V together (an entry is one store), kGatherStages - 1 blocks of loads in flight.
+// us of the whole call before (tables, n-th source of the list for the n-th warp) / with the tables gone / with blocks from
+// a counter as well: 40 heads x 75600, 8 ranks 2176 / 2148 / 1931 (6.4 TB/s), 24 x 118800 1714 / 1692 / 1522, 48 x 17776
+// 322 / 329 / 298, 24 x 24576, 4 ranks 223 / 212 / 197, 2 x 13 x 6034, 3 ranks 18.0 / 15.7 / 15.5, 2 x 4096 18.3 / 13.4 /
+// 13.7.  What held it back was not memory but warps whose blocks happened to have many consumers.
+// The counts and a table of owners have to fit beside the rings, and every CTA scans all of them: a few us at 6144.
+// ------------------------------------------------------------------------------------------------
+constexpr int kScanMax = 6144;
+constexpr int kGatherStages = 3, kGatherThreads = 128;
+constexpr int kGatherSmem = 232448 - 7 * 1024;  // dynamic shared memory, next to less than 7 KB of its own
+
+__global__ void __launch_bounds__(kGatherThreads)
+    gather_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+                  const uint32_t* __restrict__ U, const int32_t* __restrict__ rank, const int32_t* __restrict__ cnt, int B,
+                  int H, int NB, int Wd, int P, int include_local, int b, uint32_t tile_bytes, int n_copy,
+                  int64_t* __restrict__ seg_off, int64_t* __restrict__ seg_total, int64_t* __restrict__ volume,
+                  const int64_t* __restrict__ dst_base, int64_t capacity, unsigned char* __restrict__ packed,
+                  int32_t* __restrict__ n_taken, int32_t* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ uint64_t full_all[kPackMaxWarps * kGatherStages];
+  __shared__ int64_t dst_all[kPackMaxWarps][kGatherStages][kMaxRanks];
+  __shared__ int warp_s[kGatherThreads / 32];
+  __shared__ int s_abort;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int PH = P * H, T = B * P * PH;
+  const int64_t entry_bytes = 2LL * tile_bytes;
+  int32_t* off_s = reinterpret_cast<int32_t*>(smem_raw + (size_t)n_copy * kGatherStages * entry_bytes);  // [T + 1]
+  uint32_t* own_s = reinterpret_cast<uint32_t*>(off_s + T + 1);                                          // [P][Wd]
+  if (threadIdx.x == 0) s_abort = 0;
+  if (threadIdx.x < kPackMaxWarps * kGatherStages) {
+    ptx::mbar_init(full_all + threadIdx.x, 1);
+    ptx::mbar_init_fence();
+  }
+  enter_grid(U, rank, cnt, dst_base);
+  own_words(rank, NB, Wd, P, own_s);
+  // exclusive scan of the counts, a quarter per warp
+  {
+    constexpr int kWarps = kGatherThreads / 32;
+    const int chunk = (T + 32 * kWarps - 1) / (32 * kWarps) * 32;
+    const int i1 = min(T, (warp + 1) * chunk);
+    int running = 0;
+#pragma unroll 4
+    for (int i0 = warp * chunk; i0 < i1; i0 += 32) {
+      const int i = i0 + lane;
+      const int br = i / PH, q = (i - br * PH) / H;
+      const int c = i < i1 && (q != br % P || include_local) ? cnt[i] : 0;
+      int incl = c;
+#pragma unroll
+      for (int s = 1; s < 32; s <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, s);
+        if (lane >= s) incl += v;
+      }
+      if (i < i1) off_s[i] = running + incl - c;
+      running += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) warp_s[warp] = running;
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int k = 0; k < kWarps; ++k) {
+      before += k < warp ? warp_s[k] : 0;
+      all += warp_s[k];
+    }
+    for (int i = warp * chunk + lane; i < i1; i += 32) off_s[i] += before;
+    if (threadIdx.x == 0) off_s[T] = all;
+    __syncthreads();
+  }
+  for (int br = blockIdx.x; br < B * P; br += gridDim.x) {
+    const int first = off_s[br * PH], total = off_s[(br + 1) * PH] - first, own = (br % P) * H;
+    for (int i = threadIdx.x; i < PH; i += kGatherThreads) seg_off[(int64_t)br * PH + i] = off_s[br * PH + i] - first;
+    if (threadIdx.x == 0) {
+      seg_total[br] = total;
+      volume[br] = entry_bytes * (total - (off_s[br * PH + own + H] - off_s[br * PH + own]));
+    }
+  }
+  if (warp >= n_copy) return;
+
+  uint64_t* full = full_all + warp * kGatherStages;
+  unsigned char* ring = smem_raw + (size_t)warp * kGatherStages * entry_bytes;
+  int64_t(*dst_s)[kMaxRanks] = dst_all[warp];
+  const int n_units = gridDim.x * n_copy;
+  // Blocks are copied to between none and all consumers, so a warp takes its next one, (batch, head, block), from a counter,
+  // and the number after that while it looks the block up.
+  int next = blockIdx.x * n_copy + warp;
+  const int n_blocks = B * H * NB;
+  // where consumer r's copy of block j goes, -1 if it gets none
+  auto destination = [&](int bb, int h, int j, int p, int r) -> int64_t {
+    if (r >= P || (r == p && !include_local)) return -1;
+    const int br = bb * P + r;
+    const uint32_t* u = U + ((int64_t)br * H + h) * Wd;
+    const uint32_t* own = own_s + p * Wd;
+    const int w = j >> 5;
+    const uint32_t word = u[w];
+    if (!((word >> (j & 31)) & 1u)) return -1;
+    int below = __popc(word & own[w] & ((1u << (j & 31)) - 1u));
+#pragma unroll 8
+    for (int k = 0; k < w; ++k) below += __popc(u[k] & own[k]);
+    int64_t byte = (int64_t)(off_s[(br * P + p) * H + h] + below) * entry_bytes;
+    if (dst_base) byte += dst_base[br] - (int64_t)off_s[br * PH] * entry_bytes;
+    if (capacity >= 0 && byte + entry_bytes > capacity) {
+      atomicExch(status, SPARSP_ERR_CAPACITY);  // would overflow: left out
+      return -1;
+    }
+    return byte;
+  };
+  // Loads the next block that anybody receives into stage st; false: there is none left.
+  auto load_next = [&](int st) -> bool {
+    while (next < n_blocks) {
+      int after = 0;
+      if (lane == 0) after = n_units + atomicAdd(n_taken, 1);
+      const int bh = next / NB, j = next - bh * NB, p = rank[j];
+      const int bb = bh / H, h = bh - bb * H;
+      const bool owned = (unsigned)p < (unsigned)P;
+      const int64_t d0 = owned ? destination(bb, h, j, p, lane) : -1;
+      const int64_t d1 = owned && P > 32 ? destination(bb, h, j, p, lane + 32) : -1;
+      next = __shfl_sync(0xffffffffu, after, 0);
+      if (!__any_sync(0xffffffffu, d0 >= 0 || d1 >= 0)) continue;
+      dst_s[st][lane] = d0;
+      dst_s[st][lane + 32] = d1;
+      if (lane == 0) {
+        unsigned char* buf = ring + (size_t)st * entry_bytes;
+        ptx::mbar_expect_tx(full + st, 2 * tile_bytes);
+        ptx::tma_load_4d(buf, &tmK, full + st, 0, j * b, h, bb);
+        ptx::tma_load_4d(buf + tile_bytes, &tmV, full + st, 0, j * b, h, bb);
+      }
+      return true;
+    }
+    return false;
+  };
+  int n = 0;  // blocks loaded
+  while (n < kGatherStages - 1 && load_next(n)) ++n;
+  for (int q = 0; q < n; ++q) {
+    const int st = q % kGatherStages;
+    const unsigned char* buf = ring + (size_t)st * entry_bytes;
+    ptx::mbar_wait_bounded(full + st, (uint32_t)((q / kGatherStages) & 1), &s_abort, status, 50, 200000000LL);
+    const int64_t d0 = dst_s[st][lane], d1 = dst_s[st][lane + 32];
+    // (an entry is the K tile and the V tile behind it, here as there)
+    if (d0 >= 0) bulk_store(packed + d0, buf, (uint32_t)entry_bytes);
+    if (d1 >= 0) bulk_store(packed + d1, buf, (uint32_t)entry_bytes);
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    if (n == q + kGatherStages - 1) {
+      // the stage of block q - 1 may be refilled once every lane's stores have read it
+      asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+      __syncwarp();
+      if (load_next(n % kGatherStages)) ++n;
+    }
+  }
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
+int launch_demand_pack(const sparsp_shape& s, const Geometry& g, const uint32_t* mask, const int32_t* rank, int P,
+                       int flags, const void* K, const void* V, uint32_t* U, int32_t* cnt, int64_t* seg_off,
+                       int64_t* seg_total, int64_t* volume, void* packed, int64_t capacity, const int64_t* dst_base,
+                       char* ws, const WsLayout& L, cudaStream_t st) {
+  int rc = check_consumers(g, P);
   if (rc != SPARSP_OK) return rc;
-  SPARSP_CUDA_OK(launch_kernel(pack_kernel, c.grid, c.threads, c.smem, st, c.tk, c.tv, dst_table(ws, L), P,
-                               src_list(ws, L, g, P), (const int32_t*)(ws + L.n_entries), g.H, g.NB, g.b, c.tile_bytes,
-                               (unsigned char*)packed, (int32_t*)(ws + L.status)));
+  const int local = (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0;
+  int32_t* status = (int32_t*)(ws + L.status);
+  const int64_t T = (int64_t)g.B * P * P * g.H, tile_bytes = 2LL * g.b * g.d;
+  const int n_copy = pack_warps((int)tile_bytes);
+  const int64_t smem = n_copy * kGatherStages * 2 * tile_bytes + (T + 1) * 4 + (int64_t)P * g.Wd * 4;
+  PackLaunch c;
+  if (T <= kScanMax && smem <= kGatherSmem) {
+    if ((rc = prepare_pack(s, g, K, V, (const void*)gather_kernel, (int)smem, &c)) != SPARSP_OK) return rc;
+    int32_t* n_taken = (int32_t*)(ws + L.n_entries);  // zeroed by the union's launch
+    SPARSP_CUDA_OK(launch_union(g, mask, rank, P, local, U, cnt, nullptr, n_taken, st));
+    SPARSP_CUDA_OK(launch_kernel(gather_kernel, c.grid, kGatherThreads, (size_t)smem, st, c.tk, c.tv, U, rank, cnt, g.B,
+                                 g.H, g.NB, g.Wd, P, local, g.b, c.tile_bytes, n_copy, seg_off, seg_total, volume,
+                                 dst_base, capacity, (unsigned char*)packed, n_taken, status));
+    return SPARSP_OK;
+  }
+  const int ring = n_copy * kPackStages * (int)tile_bytes;
+  if ((rc = prepare_pack(s, g, K, V, (const void*)pack_kernel, ring, &c)) != SPARSP_OK) return rc;
+  int64_t* dst = dst_table(ws, L);
+  int32_t* src = src_list(ws, L, g, P);
+  int32_t* n_src = (int32_t*)(ws + L.n_entries);
+  SPARSP_CUDA_OK(launch_plan(g, mask, rank, P, local, U, cnt, seg_off, seg_total, volume, dst_base, capacity, dst, src,
+                             n_src, received_table(ws, L, g, P), status, st));
+  SPARSP_CUDA_OK(launch_kernel(pack_kernel, c.grid, 32 * n_copy, (size_t)ring, st, c.tk, c.tv, dst, P, src, n_src, g.H,
+                               g.NB, g.b, c.tile_bytes, (unsigned char*)packed, status));
   return SPARSP_OK;
 }
 
@@ -500,9 +679,10 @@ int launch_pack_segment(const sparsp_shape& s, const Geometry& g, const uint32_t
                         int consumer, int producer, const int64_t* seg_off, const int32_t* cnt, const void* K,
                         const void* V, void* dst, int64_t capacity, char* ws, const WsLayout& L, cudaStream_t st) {
   PackLaunch c;
-  const int rc = prepare_pack(s, g, K, V, (const void*)segment_kernel, &c);
+  const int n_warps = pack_warps(g.b * g.d * 2), smem = n_warps * kPackStages * g.b * g.d * 2;
+  const int rc = prepare_pack(s, g, K, V, (const void*)segment_kernel, smem, &c);
   if (rc != SPARSP_OK) return rc;
-  SPARSP_CUDA_OK(launch_kernel(segment_kernel, c.grid, c.threads, c.smem, st, c.tk, c.tv, U, rank, g.H, g.NB, g.Wd, P,
+  SPARSP_CUDA_OK(launch_kernel(segment_kernel, c.grid, 32 * n_warps, (size_t)smem, st, c.tk, c.tv, U, rank, g.H, g.NB, g.Wd, P,
                                consumer, producer, seg_off, cnt, g.b, c.tile_bytes, (unsigned char*)dst, capacity,
                                (int32_t*)(ws + L.status)));
   return SPARSP_OK;
