@@ -317,7 +317,7 @@ def time_steps(cfg, steps, warmup, barrier, local_gpu):
 
 
 def graph_replay(cfg, steps):
-    """The same step captured ONCE in a CUDA graph (the three calls, eight launches) and replayed: what the launch
+    """The same step captured ONCE in a CUDA graph (the three calls, seven launches) and replayed: what the launch
     gaps between the library's kernels cost.  Per-replay CUDA events; the L2 flush (small workloads) stays outside
     the timed pairs.  Returns ms per step."""
     import torch

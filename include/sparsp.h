@@ -346,7 +346,7 @@ SPARSP_API int sparsp_xchg_destroy(sparsp_xchg* x);
  *   union_mask, cnt, seg_offset   outputs of sparsp_demand_pack / sparsp_demand_plan_noalloc made WITHOUT
  *                                 SPARSP_INCLUDE_LOCAL (DEVICE)
  *   dst                           DEVICE, 16-byte aligned (a slot of the producer's window)
- *   workspace                     this rank's own (the call rewrites the workspace's entry table) */
+ *   workspace                     this rank's own */
 SPARSP_API int sparsp_pack_segment(const sparsp_shape* shape, const uint32_t* union_mask, const int32_t* rank_of_block,
                                    int32_t n_ranks, int32_t consumer, int32_t producer, const int32_t* cnt,
                                    const int64_t* seg_offset, const void* K, const void* V, void* dst,

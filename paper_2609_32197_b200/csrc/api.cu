@@ -122,7 +122,7 @@ WsLayout make_layout(const Geometry& g, int P) {
   off += align_up((int64_t)g.B * 8, 256);
   L.n_items = off;  // work items of the attention kernel per (batch, head), int32 [B][H]
   off += align_up((int64_t)g.B * g.H * 4, 256);
-  L.n_entries = off;  // blocks that anybody receives, int32
+  L.n_entries = off;  // blocks that anybody receives, or that the gather has handed out, int32
   off += 256;
   // destinations of every block, int64 [B][H][NB][P], the list of those blocks, int32 [B][H][NB], and the entries of
   // every (consumer, head), int32 [B][P][H]
