@@ -47,7 +47,8 @@ cudaError_t ensure_dynamic_smem(const void* func, int bytes);
 // Launches a kernel that may start while the launches before it in the stream still run (programmatic stream
 // serialisation): its CTAs take their places and set themselves up as soon as the previous kernel's have all started,
 // and wait in enter_grid() before they touch memory, so that the latency of a launch is hidden behind the kernel before
-// it. Every kernel launched here calls enter_grid() first thing, in every thread.
+// it. Every kernel launched here calls enter_grid() first thing, in every thread, or
+// wait_previous_grids() where the next launch is to begin only as its CTAs end.
 template <typename T>
 struct same_type {
   using type = T;
@@ -71,14 +72,19 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int threads, s
 }
 
 #ifdef __CUDACC__
-// First statement of a kernel started by launch_kernel: lets the next launch begin, then waits until all work before
-// this launch has completed.  No thread returns or touches global memory before it.  Pointers that the compiler
-// may take for read-only are passed through it, so that no load through them can be moved ahead of the wait.
+// Waits until all work before this launch has completed.  No thread returns or touches global memory before it.
+// Pointers that the compiler may take for read-only are passed through it, so that no load through them can be moved
+// ahead of the wait.
+template <typename... P>
+__device__ __forceinline__ void wait_previous_grids(P&... pointers) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  ((void)([](auto& p) { asm volatile("" : "+l"(p)::"memory"); }(pointers)), ...);
+}
+// First statement of a kernel started by launch_kernel: lets the next launch begin, then waits as above.
 template <typename... P>
 __device__ __forceinline__ void enter_grid(P&... pointers) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  ((void)([](auto& p) { asm volatile("" : "+l"(p)::"memory"); }(pointers)), ...);
+  wait_previous_grids(pointers...);
 }
 #endif
 
