@@ -26,8 +26,8 @@
 // without a row maximum: load scores -> exponentials -> store P, relative to 0 (K / V source) or to the row's maximum
 // over the item's first tile (packed source), which the warpgroup of that tile hands to the other one; the tensor pipe
 // takes the row sums.  Whether that was right is seen from the finished row sums and the exponents on the way, and an
-// item that left the range is computed again (kRefZero ... below).  Only an item that fails relative to its first tile as
-// well takes its maxima as it goes: the two threads that own the same row (one per warpgroup) then share the reference
+// item that left the range is computed again (kRefZero ... below).  Only such an item, and rows whose first scores are out
+// of range, take their maxima as they go: the two threads that own the same row (one per warpgroup) then share the reference
 // through shared memory and take their decisions strictly in tile order (a pair of 64-thread named barriers per row group
 // hands the turn back and forth), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since
 // the reference last moved -- the thread that decides so first waits for every P V issued so far.
@@ -90,20 +90,26 @@ constexpr float kGrowThreshold = 8.0f;
 // Where an item's softmax rows take the reference that is subtracted from their scores (log2 domain) from:
 //   kRefZero   nowhere, it is 0;
 //   kRefFirst  the row's maximum over the item's first tile (0 for a row that keeps nothing of it);
-//   kRefWide   the same, with exponents below the range raised to its lower end;
 //   kRefExact  the row's running maximum, moved lazily and strictly in tile order.
-// The first three never look at another score, so they are right only for rows whose scores stay near the reference.
-// That is seen at the end of the item: no exponential left the range of normal numbers on the FMA pipe (kMaxExponent;
-// the special-function unit saturates to 0 and infinity by itself), and the row sum lies within [kMinSum, kMaxSum].
-// Then every term is a normal fp32 and bf16 number of full relative precision, or at most 2^-36 of the sum, and
-// kMaxSum * |V| is far inside fp32.  An item with a row that fails, one with scores that are no numbers included, is
-// computed again, as kRefWide and then as kRefExact (at once where the range was missed by far), and the later items of
-// its CTA start one kind further on.  Ordinary scores pass: with unit-variance
-// Q and K at d = 128 they are within +-16.
-constexpr int kRefZero = 0, kRefFirst = 1, kRefWide = 2, kRefExact = 3;
+// The first two look at no score behind the first tile, so they are right only for rows whose scores stay near the
+// reference.  That is seen at the end of the item: no exponential left the range of normal numbers on the FMA pipe
+// (kMaxExponent; the special-function unit saturates to 0 and infinity by itself), the row sum lies within
+// [kMinSum, kMaxSum].  Then every term is a normal fp32 and bf16 number of full relative precision, or at most 2^-36 of the
+// sum, and kMaxSum * |V| is far inside fp32.  An item with a row that fails, one with scores that are no numbers included, is
+// computed again as kRefExact.
+// So that this is rare, the four warps of the item's first tile look at it first: rows whose first scores are far from 0
+// take the running maximum from the start, the 32 rows of a warp together (kZeroSample: every eighth score; kFirstSample:
+// the maximum that the reference is anyway).  Ordinary scores pass both: with unit-variance Q and K at d = 128 they are
+// within +-16.  (us per call of 13 heads x 2 x 6034 tokens, Q times 1, 4 and 60: 88, 140 and 133; looking for +-64 only 183
+// with Q times 4; with range proofs from the norms of rows and keys instead of all this 91, 131 and 140.)
+// All of this follows from the item alone, so a call repeats itself bit for bit whichever CTA takes which item.  (A CTA that
+// remembered failures and began its next items further on was right too, but let rows of ordinary heads change in their
+// last bit from call to call.)
+constexpr int kRefZero = 0, kRefFirst = 1, kRefExact = 2;
 constexpr float kMaxExponent = 126.0f;
 constexpr float kMinSum = 8.077935669463161e-28f;  // 2^-90
 constexpr float kMaxSum = 1.2676506002282294e30f;  // 2^100
+constexpr float kZeroSample = 48.0f, kFirstSample = 64.0f;
 constexpr int kZeroMinTiles = 4;  // K / V source: shorter items take kRefFirst, whose largest terms are exact
 // Tuning switch (compile-time): how many of the exponentials go to the FMA pipe instead of the
 // special-function unit (every n-th pair; 0 = none).
@@ -150,7 +156,7 @@ struct AttnCfg {
   static constexpr int kColO = 384;  // accumulator: columns [384, 384 + d)
   static constexpr int kColL = kOnes ? kColO + D : 320;  // row sums (column 0 of 16), where the tensor pipe takes them
   static constexpr int kOffMisc = kOffBars + 8 * kNumBars;
-  static constexpr int kTotal = kOffMisc + 80;
+  static constexpr int kTotal = kOffMisc + 96;
   static constexpr int kDynamic = kTotal + 1024;  // slack for the 1024-byte alignment of the base
   static_assert(kDynamic <= 232448, "shared memory budget");
 };
@@ -185,9 +191,9 @@ __device__ __forceinline__ float max_abs3(float a, float b, float c) {
 
 // 2^x for a pair of fp32 values on the FMA/ALU pipes (no special-function unit): round-to-nearest
 // split x = i + f, f in [-0.5, 0.5], cubic minimax polynomial for 2^f (relative error 7.5e-5, far
-// below bf16 rounding), exponent added into the bit pattern.  The result is right for |i| <= 126; *i_max collects the
-// largest |i|.  kClamp: x is clamped at -126 first (result >= 2^-126).
-template <bool kClamp>
+// below bf16 rounding), exponent added into the bit pattern.  The result is right for |i| <= 126.
+// kTrack: *i_max collects the largest |i|.  kClamp: x is clamped at -126 first (result >= 2^-126).
+template <bool kClamp, bool kTrack>
 __device__ __forceinline__ float2 exp2_poly2(float2 x, float* i_max) {
   const float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
   if (kClamp) {
@@ -196,7 +202,7 @@ __device__ __forceinline__ float2 exp2_poly2(float2 x, float* i_max) {
   }
   const float2 t = fadd2(x, make_float2(kMagic, kMagic));
   const float2 fi = fadd2(t, make_float2(-kMagic, -kMagic));
-  *i_max = max_abs3(fi.x, fi.y, *i_max);
+  if (kTrack) *i_max = max_abs3(fi.x, fi.y, *i_max);
   const float2 f = fadd2(x, make_float2(-fi.x, -fi.y));
   float2 q = ffma2(f, make_float2(0.0551716685f, 0.0551716685f), make_float2(0.2426111251f, 0.2426111251f));
   q = ffma2(q, f, make_float2(0.6932609677f, 0.6932609677f));
@@ -259,8 +265,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   uint64_t* o_drained = o_full + 4;      // the item's accumulator has been read out by all 8 softmax warps
   uint64_t* list_ready = o_drained + 1;  // [2] list buffer filled
   uint64_t* list_free = list_ready + 2;  // [2] list buffer no longer needed by its kListReaders
-  // [4] the four warps that own an item's first tile have left the reference that it gives in sRef.  Four, because
-  // the other warpgroup, which waits for it, may be up to three tiles and as many items behind.
+  // [4] the four warps that own an item's first tile have left what it says in s_exact and, if that is the reference, in
+  // sRef.  Four, because the other warpgroup, which waits for it, may be up to three tiles and as many items behind.
   uint64_t* ref_ready = list_free + 2;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
@@ -270,7 +276,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   int* s_rag = reinterpret_cast<int*>(smem + C::kOffMisc + 40);   // [2] the item's last tile reaches past the end of the sequence
   int* s_ref = reinterpret_cast<int*>(smem + C::kOffMisc + 48);   // [2] where the rows' reference comes from
   int* s_none = reinterpret_cast<int*>(smem + C::kOffMisc + 56);  // [2] bit q: query block q keeps nothing
-  volatile int* s_failed = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 64);  // [2] a row of the item left the range: 1, by far: 2
+  volatile int* s_failed = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 64);  // [2] the item is to be computed again
+  // [4 items][4 row groups] the group's rows take the running maximum
+  volatile uint8_t* s_exact = reinterpret_cast<volatile uint8_t*>(smem + C::kOffMisc + 80);
   constexpr int kListReaders = 12;  // two producers, two issuers, eight softmax warps
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -596,10 +604,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       // x 75600 hop by hop: 3 % slower early).
       constexpr bool kEarly = kPacked && C::kStacked && D == 128;
       if (kEarly) fetch(blockIdx.x);
-      int kind = kPacked ? kRefFirst : kRefZero;  // what new items take their reference from
       for (int i = 0;; ++i) {
         const int buf = i & 1;
-        int again = -1;  // list buffer of an item that failed and is computed again now (rare)
+        int again = -1;  // list buffer of an item that is computed again now (rare)
         if (i >= 2) {
           mbar_wait_bounded_inline(list_free + buf, ((i - 2) >> 1) & 1, s_abort, 50, p.wait_limit);
           if (s_failed[buf]) again = buf;
@@ -617,14 +624,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           break;
         }
         const int next_bh = bh, next_blk0 = blk0, next_blk1 = blk1;
-        int ref_of = kind;
         if (again >= 0) {
           bh = s_item[again];
           blk0 = s_blk[again * 2];
           blk1 = s_blk[again * 2 + 1];
-          const bool far = s_failed[again] == 2;
-          ref_of = far ? kRefExact : max(s_ref[again] + 1, kRefWide);
-          kind = far ? kRefExact : min(kind + 1, ref_of);
           load_rows();
           __syncwarp();  // (every lane has looked)
           if (lane == 0) s_failed[again] = 0;
@@ -750,7 +753,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           }
           __syncwarp();
         }
-        if (ref_of == kRefZero && running < (kZeroMinTiles - 1) * C::kEPT + 1) ref_of = kRefFirst;
+        int ref_of = kPacked || running <= (kZeroMinTiles - 1) * C::kEPT ? kRefFirst : kRefZero;
+        if (again >= 0) ref_of = kRefExact;
         if (lane == 0) {
           s_item[buf] = bh;
           s_rag[buf] = rag_pos >= 0 ? 1 : 0;
@@ -807,7 +811,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     const int bar_mine = 1 + wg * 4 + rgrp;         // I arrive here after my decision
     const int bar_other = 1 + (1 - wg) * 4 + rgrp;  // the row group's other warp arrives here after its decision
     int g0 = 0;       // number of the item's first tile
-    int n_first = 0;  // items so far whose reference came from their first tile
     for (int i = 0;; ++i) {
       const int buf = i & 1;
       mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 56, p.wait_limit);
@@ -822,20 +825,64 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       volatile float* ref = sRef + (i & 3) * 128;
       float m_ref = ref_of == kRefZero ? 0.0f : -INFINITY;  // the row's reference as this thread last saw it
       float i_max = 0.0f;  // largest binary exponent that was taken on the FMA pipe, in magnitude
-      uint64_t* ref_bar = ref_ready + (n_first & 3);
-      const uint32_t ref_phase = (n_first >> 2) & 1;
-      const bool from_first = ref_of == kRefFirst || ref_of == kRefWide;
-      if (from_first) ++n_first;
+      bool exact = ref_of == kRefExact;  // this row group takes the running maximum
       auto learn_ref = [&]() {  // the warpgroup that does not own the first tile
-        mbar_wait_bounded_inline(ref_bar, ref_phase, s_abort, 43, p.wait_limit);
-        m_ref = ref[row];
+        mbar_wait_bounded_inline(ref_ready + (i & 3), (i >> 2) & 1, s_abort, 43, p.wait_limit);
+        exact = s_exact[(i & 3) * 4 + rgrp] != 0;
+        if (ref_of == kRefFirst && !exact) m_ref = ref[row];
+      };
+      // the row's largest score of a tile: one flat instruction stream per 64-key half, an absent half (not kept by this
+      // row's query block) is skipped
+      auto row_max = [&](const float* sv, const int* vh) {
+        float mx = -INFINITY;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float* svh = sv + h * 64;
+          if (vh[h] > 0) {
+            float m0 = svh[0], m1 = svh[1], m2 = svh[2], m3 = svh[3];
+#pragma unroll
+            for (int e = 4; e < 64; e += 4) {
+              m0 = fmaxf(m0, svh[e]);
+              m1 = fmaxf(m1, svh[e + 1]);
+              m2 = fmaxf(m2, svh[e + 2]);
+              m3 = fmaxf(m3, svh[e + 3]);
+            }
+            mx = fmaxf(mx, fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)));
+          }
+        }
+        return mx * p.scale_log2;
+      };
+      // the warpgroup that does
+      auto look_at_first = [&](auto careful_tag, const float* sv, const int* vh) {
+        if ((decltype(careful_tag)::value || kPacked) && ref_of == kRefFirst) {
+          const float mx = row_max(sv, vh);
+          m_ref = mx > -INFINITY ? mx : 0.0f;  // (keeps nothing of this tile, or is no number)
+          ref[row] = m_ref;
+          exact = __any_sync(0xffffffffu, !(fabsf(m_ref) <= kFirstSample));
+        } else {
+          float most = 0.0f;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (vh[h] > 0) {
+#pragma unroll
+              for (int e = h * 64; e < h * 64 + 64; e += 16) most = max_abs3(sv[e], sv[e + 8], most);
+            }
+          }
+          exact = __any_sync(0xffffffffu, !(most * p.scale_log2 <= kZeroSample));
+        }
+        if (exact) m_ref = -INFINITY;
+        __syncwarp();
+        if (lane == 0) {
+          s_exact[(i & 3) * 4 + rgrp] = exact ? 1 : 0;
+          mbar_arrive(ref_ready + (i & 3));
+        }
       };
 
-      // One tile of this warpgroup.  kGeneral = the sequence may end inside the tile (possible only for the item's last
-      // tile), or the item is computed again, or (K / V source) the reference comes from the first tile and this is it:
-      // that variant carries the column masking and the turns, the common one stays small.
-      auto do_tile = [&](auto general_tag, const int n) {
-        constexpr bool kGeneral = decltype(general_tag)::value;
+      // One tile of this warpgroup.  kRagged = the sequence ends inside the tile (possible only for the item's last one), or
+      // (K / V source) the reference comes from the first tile and this is it: that variant carries the column masking;
+      // kExact: the one with the turns.  The common variant stays small.
+      auto do_tile = [&](auto ragged_tag, auto exact_tag, const int n) {
+        constexpr bool kRagged = decltype(ragged_tag)::value, kExact = decltype(exact_tag)::value;
         const int g = g0 + n;
         // kept / valid key columns of each 64-column half of the tile (warp-uniform), as the list builder left them
         int vh[2];
@@ -847,19 +894,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           vh[0] = min(nv, 64);
           vh[1] = max(nv - 64, 0);
         }
-
         mbar_wait_bounded_inline(s_full + wg, (g >> 1) & 1, s_abort, 30 + wg, p.wait_limit);
         tc_fence_after();
         float sv[128];
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, reinterpret_cast<uint32_t*>(sv) + c * 32);
         tmem_ld_wait();
-        // S is in registers: the Q K^T of tile g+2 may overwrite the buffer
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(s_free + wg);
-
-        if (kGeneral) {
+        if (kRagged) {
           // the sequence ends inside this tile: columns past the end count as -inf
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
@@ -869,29 +910,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             }
           }
         }
-        auto row_max = [&]() {
-          // one flat instruction stream per 64-key half; an absent half (not kept by this row's query block)
-          // is skipped
-          float mx = -INFINITY;
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float* svh = sv + h * 64;
-            if (vh[h] > 0) {
-              float m0 = svh[0], m1 = svh[1], m2 = svh[2], m3 = svh[3];
-#pragma unroll
-              for (int e = 4; e < 64; e += 4) {
-                m0 = fmaxf(m0, svh[e]);
-                m1 = fmaxf(m1, svh[e + 1]);
-                m2 = fmaxf(m2, svh[e + 2]);
-                m3 = fmaxf(m3, svh[e + 3]);
-              }
-              mx = fmaxf(mx, fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)));
-            }
-          }
-          return mx * p.scale_log2;
-        };
-        if (kGeneral && ref_of == kRefExact) {
-          const float mx = row_max();
+        if (!kExact && n <= 1) {
+          if (n == 0) look_at_first(ragged_tag, sv, vh);
+          else learn_ref();
+          if (exact) return;  // the variant with the turns takes the tile
+        }
+        // S is in registers: the Q K^T of tile g+2 may overwrite the buffer
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(s_free + wg);
+
+        if (kExact) {
+          const float mx = row_max(sv, vh);
           // ---- my turn to look at / move the row's reference maximum (strictly in tile order) ----
           if (n > 0) {
             named_bar_sync(bar_other, 64);
@@ -926,21 +956,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
               tmem_st_wait();
               tc_fence_before();
             }
-            if (grow) m_ref = m_new;
+            if (grow) {
+              m_ref = m_new;
+              ref[row] = m_new;
+            }
           }
-          if (n == 0 || m_ref != ref[row]) ref[row] = m_ref;
+          if (n == 0 && m_ref == -INFINITY) ref[row] = m_ref;
           if (n + 1 < n_tiles) asm volatile("bar.arrive %0, %1;" ::"r"(bar_mine), "r"(64) : "memory");
-        }
-        if ((kGeneral || kPacked) && from_first && n <= 1) {
-          if (n == 0) {
-            const float mx = row_max();
-            m_ref = mx > -INFINITY ? mx : 0.0f;  // (keeps nothing of this tile, or is no number)
-            ref[row] = m_ref;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(ref_bar);
-          } else {
-            learn_ref();
-          }
         }
 
         // exponentials of keys [64h, 64h+64) -> packed bf16 columns [32h, 32h+32) of the P buffer
@@ -956,12 +978,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
               const float2 x = ffma2(make_float2(svh[2 * e], svh[2 * e + 1]), sc2, nm2);
               constexpr int kPoly = C::kOnes ? SPARSP_TUNE_POLY_D64 : SPARSP_TUNE_POLY;
               const float2 pp = (kPoly > 0 && (e % (kPoly > 0 ? kPoly : 1)) == 1)
-                                    ? exp2_poly2<kGeneral>(x, &i_max)
+                                    ? exp2_poly2<kRagged || kExact, !kExact>(x, &i_max)
                                     : make_float2(ex2(x.x), ex2(x.y));
               const __nv_bfloat162 h2 = __floats2bfloat162_rn(pp.x, pp.y);
               pkh[e] = *reinterpret_cast<const uint32_t*>(&h2);
             }
-            if (kGeneral && vh[h] < 64) {
+            if (kRagged && vh[h] < 64) {
               // columns past the end of the sequence: exactly zero in P (the polynomial path returns
               // 2^-126 for them, which the row sum may keep)
 #pragma unroll
@@ -985,22 +1007,26 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(p_full + wg);
       };
-      for (int n = first; n < n_tiles; n += 2) {
-        // the list builder puts the sequence's last block (the only one that can be ragged) into the last tile
-        if (ref_of >= kRefWide || (item_ragged && n == n_tiles - 1) || (!kPacked && from_first && n <= 1)) {
-          do_tile(std::true_type{}, n);
-        } else {
-          do_tile(std::false_type{}, n);
+      if (exact && first == 0 && lane == 0) mbar_arrive(ref_ready + (i & 3));  // (nothing to learn: the barriers keep step)
+      int n = first;
+      // the list builder puts the sequence's last block (the only one that can be ragged) into the last tile
+      const int n_rag = item_ragged ? n_tiles - 1 : -1;
+      if (!exact) {
+        for (; n < n_tiles; n += 2) {
+          if (n == n_rag || (!kPacked && ref_of == kRefFirst && n <= 1)) do_tile(std::true_type{}, std::false_type{}, n);
+          else do_tile(std::false_type{}, std::false_type{}, n);
+          if (exact) break;  // what the first tile says
         }
       }
+      if (exact)
+        for (; n < n_tiles; n += 2) do_tile(std::true_type{}, std::true_type{}, n);
 
       g0 += n_tiles;
       // ---- item epilogue: warpgroup x writes the column half x of every row -------------------------
-      if (ref_of == kRefExact) {
-        named_bar_sync(9, 256);  // all of the item's decisions are done
+      if (first >= n_tiles && ref_of != kRefExact) learn_ref();
+      if (exact) {
+        named_bar_sync(9 + rgrp, 64);  // all decisions about the row group are done
         m_ref = ref[row];
-      } else if (from_first && first >= n_tiles) {
-        learn_ref();
       }
       const int last = g0 - 1;
       mbar_wait_bounded_inline(o_full + (last & 3), (last >> 2) & 1, s_abort, 40, p.wait_limit);
@@ -1019,15 +1045,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         for (int c = 0; c < HW / 32; ++c) tmem_ld32(tO + wg * HW + c * 32, o + c * 32);
         tmem_ld_wait();
         const float l = __uint_as_float(sum);  // the row sum is a tensor-memory column
-        const bool failed = ref_of != kRefExact && tok < p.N && !(i_max <= kMaxExponent && l >= kMinSum && l <= kMaxSum);
-        const bool any_failed = __any_sync(0xffffffffu, failed);
-        const bool any_far = __any_sync(0xffffffffu, failed && i_max > 2.0f * kMaxExponent);
+        const bool failed = !exact && tok < p.N && !(i_max <= kMaxExponent && l >= kMinSum && l <= kMaxSum);
+        if (__any_sync(0xffffffffu, failed) && lane == 0) s_failed[buf] = 1;
         // the accumulator is in registers: the next item's first P V may overwrite it
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          if (any_far) s_failed[buf] = 2;
-          else if (any_failed && s_failed[buf] == 0) s_failed[buf] = 1;
           mbar_arrive(o_drained);
           mbar_arrive(list_free + buf);
         }
@@ -1076,8 +1099,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 // kept lists is chosen per (batch, head) -- video attention is multi-diagonal, so the best partner of a block is
 // typically the same position a fixed number of blocks away; the more two stacked blocks share, the less of a 128-row
 // tile's work is masked away.
-// Packed source: neighbours in the consumer's ascending list of blocks (D = 1), so that a row's result does not depend on
-// what the consumer's other blocks keep.
+// Packed source: neighbours in the consumer's ascending list of blocks (D = 1), so that a row's result depends on its
+// neighbour's list at most, not on what the consumer's other blocks keep.
 // (Mask rows in shared memory have an odd pitch: the threads' offsets differ by one row, a pitch of 32 words would put
 // them all on one bank.)
 // Items of one (batch, head) are handed out longest list first: the items still running when the queue

@@ -114,3 +114,79 @@ def test_as_many_blocks_as_multiprocessors(binding, d, layout, spare):
     assert (out - want)[rows].abs().max() <= pu.ATTN_MAX_ABS
     assert (lse[:, 0].double() - want_lse)[rows].abs().max() <= 2e-2
     assert bool((out[~rows] == 0).all()) and bool((lse[:, 0][~rows] == float("-inf")).all())
+
+
+def _mask(kept):
+    """[H][NB][NB] -> mask words [1][H][NB][Wd]."""
+    words = torch.zeros(*kept.shape[:2], (kept.shape[2] + 31) // 32, dtype=torch.int64, device="cuda")
+    for j in range(kept.shape[2]):
+        words[:, :, j // 32] |= kept[:, :, j].long() << (j % 32)
+    return torch.where(words >= 1 << 31, words - (1 << 32), words).to(torch.int32)[None].contiguous()
+
+
+class _Calls:
+    """The three calls that make an output, on [H][N][d] inputs in a layout: K / V source, packed, one hop of it."""
+
+    def __init__(self, binding, kept, d, b, N, layout="HND", P=3, consumer=1):
+        self.b, self.layout, self.P, self.consumer, self.N = binding, layout, P, consumer, N
+        H, NB = kept.shape[:2]
+        self.shape = binding.make_shape(H, d, (1, 1, N), 0, b, layout=layout)
+        self.ws, self.mask = binding.make_workspace(self.shape, P), _mask(kept)
+        self.rank = torch.arange(NB, dtype=torch.int32, device="cuda").remainder(P)
+        self.mine = (self.rank == consumer).repeat_interleave(b)[:N]
+
+    def place(self, x):
+        return pu.to_layout(x, self.layout)
+
+    def run(self, source, Q, K, V):
+        """O [H][N][d] and lse [H][N] as int16 / fp32; rows that a packed call leaves alone come back as 7."""
+        bd, (q, k, v) = self.b, (self.place(x) for x in (Q, K, V))
+        O = torch.full_like(q, 7.0)
+        lse = torch.full((1, Q.shape[0], self.N), 7.0, device="cuda")
+        if source == "kv":
+            bd.sparsp_sparse_attn_fwd(self.shape, q, k, v, self.mask, 0.0, O, lse, self.ws)
+        else:
+            mask = self.mask
+            dm = pu.gpu_demand_pack(bd, self.shape, mask, self.rank, self.P, 0, k, v, self.ws)
+            if source == "hop":
+                mask = torch.empty_like(mask)
+                bd.sparsp_hop_mask(self.shape, self.mask, self.rank, self.P, self.consumer, 0, mask)
+            bd.sparsp_sparse_attn_fwd_packed(self.shape, q, k, v, mask, self.rank, self.P, self.consumer, dm["union_mask"],
+                                             dm["seg_offset"], dm["seg_total"], dm["packed"], dm["packed"].numel(), None,
+                                             0.0, O, lse, self.ws)
+        assert bd.sparsp_status(self.ws) == bd.SPARSP_OK
+        return pu.from_layout(O, self.layout).contiguous(), lse[0]
+
+
+def _same_bits(a, b):
+    return torch.equal(a[0].view(torch.int16), b[0].view(torch.int16)) and torch.equal(a[1].view(torch.int32),
+                                                                                       b[1].view(torch.int32))
+
+
+def _mixed_heads(H, N, d, NB, b, seed):
+    """Heads within the range, far out of it, and with single blocks of rows or keys that are."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    Q, K, V = (torch.randn(H, N, d, generator=g, device="cuda") for _ in range(3))
+    block = torch.arange(N, device="cuda") // b
+    Q[1::4] *= 40.0
+    Q[2::5][:, block % 9 == 4] *= 300.0
+    K[3::6][:, block % 13 == 6] *= 60.0
+    return [x.to(torch.bfloat16) for x in (Q, K, V)], g
+
+
+@pytest.mark.parametrize("d,b,layout", [(64, 64, "HND"), (128, 64, "NHD"), (64, 128, "NHD"), (128, 128, "HND")])
+@pytest.mark.parametrize("source", ["kv", "packed", "hop"])
+def test_a_row_does_not_depend_on_who_computes_it(binding, d, b, layout, source):
+    """Many items per multiprocessor, some of which are computed again: a repeated call gives the same bits, and so does one
+    with the heads in another order, in which other items meet in a CTA."""
+    H, NB = 60, 60 if b == 64 else 45
+    N = NB * b - 9
+    (Q, K, V), g = _mixed_heads(H, N, d, NB, b, d + b)
+    kept = torch.rand(H, NB, NB, generator=g, device="cuda") < 0.3
+    kept[:, 4] = False
+    first = _Calls(binding, kept, d, b, N, layout).run(source, Q, K, V)
+    for _ in range(3):
+        assert _same_bits(first, _Calls(binding, kept, d, b, N, layout).run(source, Q, K, V))
+    order = torch.randperm(H, generator=g, device="cuda")
+    other = _Calls(binding, kept[order], d, b, N, layout).run(source, Q[order], K[order], V[order])
+    assert _same_bits((first[0][order], first[1][order]), other)
