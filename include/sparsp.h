@@ -198,6 +198,7 @@ SPARSP_API int sparsp_demand_pack(const sparsp_shape* shape, const uint32_t* mas
  *   softmax_scale  in   0 means 1/sqrt(d)
  *   O              out  bf16, strided like Q; rows of tokens >= N are not written
  *   lse            out  fp32 [B][H][N], natural-log sum-exp of the scaled logits; may be NULL
+ * A row with a score among its kept ones that is NaN or +infinity is NaN throughout, its lse included.
  */
 SPARSP_API int sparsp_sparse_attn_fwd(const sparsp_shape* shape, const void* Q, const void* K, const void* V,
                            const uint32_t* mask, float softmax_scale, void* O, float* lse,

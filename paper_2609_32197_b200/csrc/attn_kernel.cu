@@ -189,16 +189,23 @@ __device__ __forceinline__ float max_abs3(float a, float b, float c) {
   return d;
 }
 
+// The larger of the two, not a number if one of them is none.
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+
 // 2^x for a pair of fp32 values on the FMA/ALU pipes (no special-function unit): round-to-nearest
 // split x = i + f, f in [-0.5, 0.5], cubic minimax polynomial for 2^f (relative error 7.5e-5, far
-// below bf16 rounding), exponent added into the bit pattern.  The result is right for |i| <= 126.
-// kTrack: *i_max collects the largest |i|.  kClamp: x is clamped at -126 first (result >= 2^-126).
+// below bf16 rounding), exponent added into the bit pattern.  The result is right for |i| <= 126, and infinite in bf16 where
+// x is not a number.  kTrack: *i_max collects the largest |i|.  kClamp: x is clamped at -126 first (result >= 2^-126).
 template <bool kClamp, bool kTrack>
 __device__ __forceinline__ float2 exp2_poly2(float2 x, float* i_max) {
   const float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
   if (kClamp) {
-    x.x = fmaxf(x.x, -126.0f);
-    x.y = fmaxf(x.y, -126.0f);
+    x.x = max_nan(x.x, -126.0f);
+    x.y = max_nan(x.y, -126.0f);
   }
   const float2 t = fadd2(x, make_float2(kMagic, kMagic));
   const float2 fi = fadd2(t, make_float2(-kMagic, -kMagic));
@@ -1078,8 +1085,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             }
           }
         }
-        if (p.lse && wg == 0 && tok < p.N)
-          p.lse[(int64_t)bh * p.N + tok] = l > 0.0f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
+        if (p.lse && wg == 0 && tok < p.N)  // (a score that is no number makes the row's sum none, or infinite)
+          p.lse[(int64_t)bh * p.N + tok] = !(l < INFINITY) ? NAN : l > 0.0f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
       }
     }
   }

@@ -190,3 +190,31 @@ def test_a_row_does_not_depend_on_who_computes_it(binding, d, b, layout, source)
     order = torch.randperm(H, generator=g, device="cuda")
     other = _Calls(binding, kept[order], d, b, N, layout).run(source, Q[order], K[order], V[order])
     assert _same_bits((first[0][order], first[1][order]), other)
+
+
+@pytest.mark.parametrize("d,b", [(64, 64), (128, 64), (64, 128), (128, 128)])
+@pytest.mark.parametrize("source", ["kv", "packed", "hop"])
+@pytest.mark.parametrize("key", [0, 2, 63])  # by the special-function unit, by the polynomial, the last of a half tile
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_scores_that_are_no_numbers(binding, d, b, source, key, value):
+    """A row that keeps a key whose score is NaN or +infinity is NaN throughout; all other rows are what they are."""
+    H, NB = 8, 24
+    N = NB * b - 9
+    g = torch.Generator(device="cuda").manual_seed(d + b + key)
+    Q, K, V = (torch.randn(H, N, d, generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    Q[..., 0] = 1.0  # (so that an infinite key gives every row the score +infinity)
+    kept = torch.rand(H, NB, NB, generator=g, device="cuda") < 0.3
+    c = _Calls(binding, kept, d, b, N)
+    plain = c.run(source, Q, K, V)
+    bad = 9  # a block of rank 0
+    K[:, bad * b + key, 0] = value
+    O, lse = c.run(source, Q, K, V)
+    none = kept[:, :, bad].repeat_interleave(b, 1)[:, :N]
+    rows = c.mine if source != "kv" else torch.ones_like(c.mine)
+    assert bool(torch.isnan(O[none & rows]).all()) and bool(torch.isnan(lse[none & rows]).all())
+    keep = ~none & rows
+    # (another row of its item may have made the item be computed again: two roundings of the same result)
+    assert (O.double() - plain[0].double())[keep].abs().max() <= 2 * pu.ATTN_MAX_ABS
+    finite = keep & torch.isfinite(plain[1])
+    assert bool(torch.isfinite(lse[finite]).all()) and (lse - plain[1])[finite].abs().max() <= 2e-2
+    assert torch.equal(lse[keep & ~finite], plain[1][keep & ~finite])
