@@ -94,9 +94,10 @@ constexpr float kGrowThreshold = 8.0f;
 // The first two look at no score behind the first tile, so they are right only for rows whose scores stay near the
 // reference.  That is seen at the end of the item: no exponential left the range of normal numbers on the FMA pipe
 // (kMaxExponent; the special-function unit saturates to 0 and infinity by itself), the row sum lies within
-// [kMinSum, kMaxSum].  Then every term is a normal fp32 and bf16 number of full relative precision, or at most 2^-36 of the
-// sum, and kMaxSum * |V| is far inside fp32.  An item with a row that fails, one with scores that are no numbers included, is
-// computed again as kRefExact.
+// [kMinSum, kMaxSum], and no output column ran out of fp32 where the sum is so large that a finite V could do that (above
+// kSafeSumZero or kSafeSumFirst; below them it takes |V| > 2^63 or 2^102, and the running maximum allows no more than the
+// latter).  Then every term is a normal fp32 and bf16 number of full relative precision, or at most 2^-36 of the sum.  An
+// item with a row that fails, one with scores that are no numbers included, is computed again as kRefExact.
 // So that this is rare, the four warps of the item's first tile look at it first: rows whose first scores are far from 0
 // take the running maximum from the start, the 32 rows of a warp together (kZeroSample: every eighth score; kFirstSample:
 // the maximum that the reference is anyway).  Ordinary scores pass both: with unit-variance Q and K at d = 128 they are
@@ -109,6 +110,8 @@ constexpr int kRefZero = 0, kRefFirst = 1, kRefExact = 2;
 constexpr float kMaxExponent = 126.0f;
 constexpr float kMinSum = 8.077935669463161e-28f;  // 2^-90
 constexpr float kMaxSum = 1.2676506002282294e30f;  // 2^100
+constexpr float kSafeSumZero = 1.8446744073709552e19f;  // 2^64
+constexpr float kSafeSumFirst = 33554432.0f;            // 2^25: kGrowThreshold and 2^17 keys
 constexpr float kZeroSample = 48.0f, kFirstSample = 64.0f;
 constexpr int kZeroMinTiles = 4;  // K / V source: shorter items take kRefFirst, whose largest terms are exact
 // Tuning switch (compile-time): how many of the exponentials go to the FMA pipe instead of the
@@ -1052,8 +1055,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         for (int c = 0; c < HW / 32; ++c) tmem_ld32(tO + wg * HW + c * 32, o + c * 32);
         tmem_ld_wait();
         const float l = __uint_as_float(sum);  // the row sum is a tensor-memory column
-        const bool failed = !exact && tok < p.N && !(i_max <= kMaxExponent && l >= kMinSum && l <= kMaxSum);
-        if (__any_sync(0xffffffffu, failed) && lane == 0) s_failed[buf] = 1;
+        // (an ordinary item asks one question here)
+        const float safe = ref_of == kRefZero ? kSafeSumZero : kSafeSumFirst;
+        const bool asks = !exact && tok < p.N && !(i_max <= kMaxExponent && l >= kMinSum && l <= safe);
+        if (__any_sync(0xffffffffu, asks)) {
+          bool failed = asks && !(i_max <= kMaxExponent && l >= kMinSum && l <= kMaxSum);
+          if (asks) {
+            float most = 0.0f;  // has a column run out of fp32?
+#pragma unroll
+            for (int e = 0; e < HW; e += 2) most = max_abs3(__uint_as_float(o[e]), __uint_as_float(o[e + 1]), most);
+            failed = failed || !(most < INFINITY);
+          }
+          if (__any_sync(0xffffffffu, failed) && lane == 0) s_failed[buf] = 1;
+        }
         // the accumulator is in registers: the next item's first P V may overwrite it
         tc_fence_before();
         __syncwarp();

@@ -138,13 +138,13 @@ class _Calls:
     def place(self, x):
         return pu.to_layout(x, self.layout)
 
-    def run(self, source, Q, K, V):
+    def run(self, source, Q, K, V, scale=0.0):
         """O [H][N][d] and lse [H][N] as int16 / fp32; rows that a packed call leaves alone come back as 7."""
         bd, (q, k, v) = self.b, (self.place(x) for x in (Q, K, V))
         O = torch.full_like(q, 7.0)
         lse = torch.full((1, Q.shape[0], self.N), 7.0, device="cuda")
         if source == "kv":
-            bd.sparsp_sparse_attn_fwd(self.shape, q, k, v, self.mask, 0.0, O, lse, self.ws)
+            bd.sparsp_sparse_attn_fwd(self.shape, q, k, v, self.mask, scale, O, lse, self.ws)
         else:
             mask = self.mask
             dm = pu.gpu_demand_pack(bd, self.shape, mask, self.rank, self.P, 0, k, v, self.ws)
@@ -153,7 +153,7 @@ class _Calls:
                 bd.sparsp_hop_mask(self.shape, self.mask, self.rank, self.P, self.consumer, 0, mask)
             bd.sparsp_sparse_attn_fwd_packed(self.shape, q, k, v, mask, self.rank, self.P, self.consumer, dm["union_mask"],
                                              dm["seg_offset"], dm["seg_total"], dm["packed"], dm["packed"].numel(), None,
-                                             0.0, O, lse, self.ws)
+                                             scale, O, lse, self.ws)
         assert bd.sparsp_status(self.ws) == bd.SPARSP_OK
         return pu.from_layout(O, self.layout).contiguous(), lse[0]
 
@@ -190,6 +190,36 @@ def test_a_row_does_not_depend_on_who_computes_it(binding, d, b, layout, source)
     order = torch.randperm(H, generator=g, device="cuda")
     other = _Calls(binding, kept[order], d, b, N, layout).run(source, Q[order], K[order], V[order])
     assert _same_bits((first[0][order], first[1][order]), other)
+
+
+@pytest.mark.parametrize("d,b", [(64, 64), (128, 64), (64, 128), (128, 128)])
+@pytest.mark.parametrize("source", ["kv", "packed", "hop"])
+@pytest.mark.parametrize("most", [20.0, 90.0])
+def test_large_values_of_v(binding, d, b, source, most):
+    """Row sums up to 2^97 relative to a reference that is far too low, times |V| of 2^40: out of fp32, the result is not.
+    A score is 0 but for one block's keys, whose score is `most` for every row (log2 units, softmax scale ln 2)."""
+    H, NB = 4, 24
+    N = NB * b - 9
+    g = torch.Generator(device="cuda").manual_seed(d)
+    Q, K = (torch.zeros(H, N, d, device="cuda") for _ in range(2))
+    Q[..., 0] = 1.0
+    block = torch.arange(N, device="cuda") // b
+    K[:, block == 18, 0] = most
+    V = torch.randn(H, N, d, generator=g, device="cuda") * 2.0 ** 40
+    Q, K, V = (x.to(torch.bfloat16) for x in (Q, K, V))
+    kept = torch.zeros(H, NB, NB, dtype=torch.bool, device="cuda")
+    kept[:, :, ::3] = True  # rank 0's, block 18 among them, and a row's own
+    kept[:, torch.arange(NB), torch.arange(NB)] = True
+    c = _Calls(binding, kept, d, b, N)
+    O, lse = c.run(source, Q, K, V, scale=math.log(2.0))
+    s = Q.double() @ K.double().transpose(1, 2) * math.log(2.0)
+    tokens = (kept & (c.rank == 0) if source == "hop" else kept).repeat_interleave(b, 1).repeat_interleave(b, 2)[:, :N, :N]
+    s.masked_fill_(~tokens, float("-inf"))
+    want = torch.softmax(s, -1) @ V.double()
+    rows = c.mine if source != "kv" else torch.ones_like(c.mine)
+    # weights and result are rounded to bf16: 2^-9 each, of values that are at most the largest |V|
+    assert (O.double() - want)[:, rows].abs().max() <= 2.0 ** -8 * V.double().abs().max()
+    assert (lse.double() - torch.logsumexp(s, -1))[:, rows].abs().max() <= 2e-2
 
 
 @pytest.mark.parametrize("d,b", [(64, 64), (128, 64), (64, 128), (128, 128)])
