@@ -196,7 +196,8 @@ SPARSP_API int sparsp_demand_pack(const sparsp_shape* shape, const uint32_t* mas
  * accumulation and fp32 online softmax.  Every row must keep at least one block.
  *   mask           in   uint32 [B][H][NB][Wd]
  *   softmax_scale  in   0 means 1/sqrt(d)
- *   O              out  bf16, strided like Q; rows of tokens >= N are not written
+ *   O              out  bf16, strided like Q; rows of tokens >= N are not written.  O may be Q itself (the same
+ *                  pointer), which it then replaces
  *   lse            out  fp32 [B][H][N], natural-log sum-exp of the scaled logits; may be NULL
  * A row with a score among its kept ones that is NaN or +infinity is NaN throughout, its lse included.
  */

@@ -71,6 +71,7 @@ struct AttnParams {
   int64_t N;
   int64_t sB, sH, sT;
   int BH, H, NB, Wd;
+  int in_place;      // O is Q: no row of an item is written before all of them are known to be right
   int single;        // block 64, K / V source: every item is one query block (an int of `pairs` each), none are stacked
   float scale_log2;  // softmax scale * log2(e)
   long long wait_limit;
@@ -1046,7 +1047,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         const int qb = C::kStacked ? s_blk[buf * 2 + rh] : s_blk[buf * 2];
         // (a block that keeps nothing is stacked with one that does: other warps write its rows)
         const bool none = qb < 0 || ((s_none[buf] >> (C::kStacked ? rh : 0)) & 1);
-        const int64_t tok = none ? p.N : (int64_t)qb * BLK + (C::kStacked ? (row & 63) : row);
+        int64_t tok = none ? p.N : (int64_t)qb * BLK + (C::kStacked ? (row & 63) : row);
         const int batch = bh / p.H, head = bh % p.H;
         __nv_bfloat16* orow = p.O + (int64_t)batch * p.sB + (int64_t)head * p.sH + tok * p.sT + wg * HW;
         uint32_t sum, o[HW];
@@ -1058,7 +1059,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         // (an ordinary item asks one question here)
         const float safe = ref_of == kRefZero ? kSafeSumZero : kSafeSumFirst;
         const bool asks = !exact && tok < p.N && !(i_max <= kMaxExponent && l >= kMinSum && l <= safe);
-        if (__any_sync(0xffffffffu, asks)) {
+        const bool slow = __any_sync(0xffffffffu, asks) || p.in_place;
+        if (slow) {
           bool failed = asks && !(i_max <= kMaxExponent && l >= kMinSum && l <= kMaxSum);
           if (asks) {
             float most = 0.0f;  // has a column run out of fp32?
@@ -1067,6 +1069,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             failed = failed || !(most < INFINITY);
           }
           if (__any_sync(0xffffffffu, failed) && lane == 0) s_failed[buf] = 1;
+          if (p.in_place) {  // the rows of an item that is computed again are still its queries
+            named_bar_sync(13, 256);
+            if (s_failed[buf]) tok = p.N;
+          }
         }
         // the accumulator is in registers: the next item's first P V may overwrite it
         tc_fence_before();
@@ -1485,6 +1491,7 @@ static int launch_attn_common(const sparsp_shape& s, const Geometry& g, const vo
                               float* lse, char* ws, const WsLayout& L, cudaStream_t st) {
   p.O = (__nv_bfloat16*)O;
   p.lse = lse;
+  p.in_place = O == Q;
   p.status = (int32_t*)(ws + L.status);
   p.work_counter = p.status + kWorkCounterWord;
   p.N = g.N;

@@ -138,10 +138,11 @@ class _Calls:
     def place(self, x):
         return pu.to_layout(x, self.layout)
 
-    def run(self, source, Q, K, V, scale=0.0):
+    def run(self, source, Q, K, V, scale=0.0, in_place=False):
         """O [H][N][d] and lse [H][N] as int16 / fp32; rows that a packed call leaves alone come back as 7."""
         bd, (q, k, v) = self.b, (self.place(x) for x in (Q, K, V))
-        O = torch.full_like(q, 7.0)
+        q = q.clone()
+        O = q if in_place else torch.full_like(q, 7.0)
         lse = torch.full((1, Q.shape[0], self.N), 7.0, device="cuda")
         if source == "kv":
             bd.sparsp_sparse_attn_fwd(self.shape, q, k, v, self.mask, scale, O, lse, self.ws)
@@ -190,6 +191,20 @@ def test_a_row_does_not_depend_on_who_computes_it(binding, d, b, layout, source)
     order = torch.randperm(H, generator=g, device="cuda")
     other = _Calls(binding, kept[order], d, b, N, layout).run(source, Q[order], K[order], V[order])
     assert _same_bits((first[0][order], first[1][order]), other)
+
+
+@pytest.mark.parametrize("d,b", [(64, 64), (128, 64), (64, 128), (128, 128)])
+@pytest.mark.parametrize("source", ["kv", "packed", "hop"])
+def test_output_may_take_the_place_of_the_queries(binding, d, b, source):
+    H, NB = 20, 30
+    N = NB * b - 9
+    (Q, K, V), g = _mixed_heads(H, N, d, NB, b, 3 * d + b)
+    kept = torch.rand(H, NB, NB, generator=g, device="cuda") < 0.3
+    kept[:, 4] = False
+    c = _Calls(binding, kept, d, b, N)
+    apart, together = c.run(source, Q, K, V), c.run(source, Q, K, V, in_place=True)
+    rows = c.mine if source != "kv" else torch.ones_like(c.mine)
+    assert _same_bits((apart[0][:, rows], apart[1]), (together[0][:, rows], together[1]))
 
 
 @pytest.mark.parametrize("d,b", [(64, 64), (128, 64), (64, 128), (128, 128)])
