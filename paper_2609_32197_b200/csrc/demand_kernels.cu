@@ -387,18 +387,58 @@ static int prepare_pack(const sparsp_shape& s, const Geometry& g, const void* K,
 // ------------------------------------------------------------------------------------------------
 // Offsets and gather in one launch, for plans of up to kScanMax counts: every CTA scans the counts of all consumers into
 // shared memory (their flat order is the order of the packed buffers), and a copy's place is its segment's first entry
-// plus the blocks of the segment below it, counted in the union words by the lane of its consumer.  No tables, no list of
-// sources and no launch that makes them.  The first CTAs also write the offsets, totals and volumes.  Tiles move as in
-// pack_kernel, a block's K and V together (an entry is one store), kGatherStages - 1 blocks of loads in flight.
-// us of the whole call before (tables, n-th source of the list for the n-th warp) / with the tables gone / with blocks from
-// a counter as well: 40 heads x 75600, 8 ranks 2176 / 2148 / 1931 (6.4 TB/s), 24 x 118800 1714 / 1692 / 1522, 48 x 17776
-// 322 / 329 / 298, 24 x 24576, 4 ranks 223 / 212 / 197, 2 x 13 x 6034, 3 ranks 18.0 / 15.7 / 15.5, 2 x 4096 18.3 / 13.4 /
-// 13.7.  What held it back was not memory but warps whose blocks happened to have many consumers.
-// The counts and a table of owners have to fit beside the rings, and every CTA scans all of them: a few us at 6144.
+// plus the blocks of the segment below it, counted in the union words by the lane of its consumer.  The other half of its
+// warps meanwhile numbers the blocks that anybody receives, of all heads, so that only those are handed out.  No tables, no
+// list of sources in memory and no launch that makes them.  The first CTAs also write the offsets, totals and volumes.  Tiles
+// move as in pack_kernel, a block's K and V together (an entry is one store), kGatherStages - 1 blocks of loads in flight.
+// us of the whole call with tables and the n-th source of the list for the n-th warp / this way: 40 heads x 75600, 8 ranks
+// 2176 / 1931 (6.4 TB/s), 24 x 118800 1714 / 1522, 48 x 17776 322 / 287, 24 x 24576, 4 ranks 223 / 200, 2 x 13 x 6034, 3
+// ranks 18.0 / 13.9, 2 x 4096 18.3 / 10.3.  What held it back was not memory but warps whose blocks happened to have many
+// consumers.  Where little is wanted, with tables / this way / with every block handed out and looked up, wanted or not: 40
+// heads x 591 blocks of 128 x 128, a band of two blocks either side, 8 ranks 38 / 38 / 158, one rank 12.6 / 11 / 96, two heads
+// of all 129 / 115 / 231.
+// The counts, the words of live blocks and a table of owners have to fit beside the rings, and every CTA scans all of them: a
+// few us at 6144 counts (24 heads, 16 ranks 1712 / 1483; one more head, by tables, 1784 / 1770).
 // ------------------------------------------------------------------------------------------------
 constexpr int kScanMax = 6144;
-constexpr int kGatherStages = 3, kGatherThreads = 128;
+constexpr int kGatherStages = 3, kGatherThreads = 512;
 constexpr int kGatherSmem = 232448 - 7 * 1024;  // dynamic shared memory, next to less than 7 KB of its own
+
+// out[i] = sum of value(0 .. i - 1) for i <= n, in two steps with a barrier between them and one behind: n_warps warps, of
+// which this one is `warp`, scan a part each, then add what lies before it.
+template <int kUnroll, typename F>
+__device__ __forceinline__ void scan_part(int n, int warp, int n_warps, int32_t* out, int* warp_s, F value) {
+  const int lane = threadIdx.x & 31;
+  const int chunk = (n + 32 * n_warps - 1) / (32 * n_warps) * 32;
+  const int i1 = min(n, (warp + 1) * chunk);
+  int running = 0;
+#pragma unroll kUnroll
+  for (int i0 = warp * chunk; i0 < i1; i0 += 32) {
+    const int i = i0 + lane;
+    const int c = i < i1 ? value(i) : 0;
+    int incl = c;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, s);
+      if (lane >= s) incl += v;
+    }
+    if (i < i1) out[i] = running + incl - c;
+    running += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  if (lane == 0) warp_s[warp] = running;
+}
+__device__ __forceinline__ void scan_rest(int n, int warp, int n_warps, int32_t* out, const int* warp_s) {
+  const int lane = threadIdx.x & 31;
+  const int chunk = (n + 32 * n_warps - 1) / (32 * n_warps) * 32;
+  const int i1 = min(n, (warp + 1) * chunk);
+  int before = 0, all = 0;
+  for (int k = 0; k < n_warps; ++k) {
+    before += k < warp ? warp_s[k] : 0;
+    all += warp_s[k];
+  }
+  for (int i = warp * chunk + lane; i < i1; i += 32) out[i] += before;
+  if (warp == 0 && lane == 0) out[n] = all;
+}
 
 __global__ void __launch_bounds__(kGatherThreads)
     gather_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
@@ -412,11 +452,15 @@ __global__ void __launch_bounds__(kGatherThreads)
   __shared__ int64_t dst_all[kPackMaxWarps][kGatherStages][kMaxRanks];
   __shared__ int warp_s[kGatherThreads / 32];
   __shared__ int s_abort;
+  static_assert(sizeof(full_all) + sizeof(dst_all) + sizeof(warp_s) + sizeof(s_abort) + 128 <= 232448 - kGatherSmem,
+                "shared memory budget");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int PH = P * H, T = B * P * PH;
+  const int PH = P * H, T = B * P * PH, n_words = B * H * Wd;
   const int64_t entry_bytes = 2LL * tile_bytes;
   int32_t* off_s = reinterpret_cast<int32_t*>(smem_raw + (size_t)n_copy * kGatherStages * entry_bytes);  // [T + 1]
-  uint32_t* own_s = reinterpret_cast<uint32_t*>(off_s + T + 1);                                          // [P][Wd]
+  int32_t* pos_s = off_s + T + 1;                                        // [n_words + 1] live blocks before each word's
+  uint32_t* live_s = reinterpret_cast<uint32_t*>(pos_s + n_words + 1);   // [B*H][Wd] blocks that any consumer receives
+  uint32_t* own_s = live_s + n_words;                                    // [P][Wd]
   if (threadIdx.x == 0) s_abort = 0;
   if (threadIdx.x < kPackMaxWarps * kGatherStages) {
     ptx::mbar_init(full_all + threadIdx.x, 1);
@@ -427,37 +471,33 @@ __global__ void __launch_bounds__(kGatherThreads)
   // gather by tables; of 2 x 4096 39.2, 38.8 and 41).
   wait_previous_grids(U, rank, cnt, dst_base);
   own_words(rank, NB, Wd, P, own_s);
-  // exclusive scan of the counts, a quarter per warp
-  {
-    constexpr int kWarps = kGatherThreads / 32;
-    const int chunk = (T + 32 * kWarps - 1) / (32 * kWarps) * 32;
-    const int i1 = min(T, (warp + 1) * chunk);
-    int running = 0;
-#pragma unroll 4
-    for (int i0 = warp * chunk; i0 < i1; i0 += 32) {
-      const int i = i0 + lane;
+  __syncthreads();
+  // One half of the warps scans the counts, the other the words of live blocks.
+  constexpr int kHalf = kGatherThreads / 64;
+  if (warp < kHalf) {
+    scan_part<4>(T, warp, kHalf, off_s, warp_s, [&](int i) {
       const int br = i / PH, q = (i - br * PH) / H;
-      const int c = i < i1 && (q != br % P || include_local) ? cnt[i] : 0;
-      int incl = c;
-#pragma unroll
-      for (int s = 1; s < 32; s <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, s);
-        if (lane >= s) incl += v;
+      return q != br % P || include_local ? cnt[i] : 0;
+    });
+  } else {
+    scan_part<1>(n_words, warp - kHalf, kHalf, pos_s, warp_s + kHalf, [&](int i) {
+      const int bh = i / Wd, w = i - bh * Wd, bb = bh / H;
+      const uint32_t* u = U + ((int64_t)bb * P * H + bh - bb * H) * Wd + w;
+      uint32_t live = 0, owned = 0;
+#pragma unroll 8
+      for (int r = 0; r < P; ++r) {
+        const uint32_t own = own_s[r * Wd + w];
+        live |= u[(int64_t)r * H * Wd] & (include_local ? ~0u : ~own);
+        owned |= own;
       }
-      if (i < i1) off_s[i] = running + incl - c;
-      running += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) warp_s[warp] = running;
-    __syncthreads();
-    int before = 0, all = 0;
-    for (int k = 0; k < kWarps; ++k) {
-      before += k < warp ? warp_s[k] : 0;
-      all += warp_s[k];
-    }
-    for (int i = warp * chunk + lane; i < i1; i += 32) off_s[i] += before;
-    if (threadIdx.x == 0) off_s[T] = all;
-    __syncthreads();
+      live_s[i] = live & owned;
+      return __popc(live & owned);
+    });
   }
+  __syncthreads();
+  if (warp < kHalf) scan_rest(T, warp, kHalf, off_s, warp_s);
+  else scan_rest(n_words, warp - kHalf, kHalf, pos_s, warp_s + kHalf);
+  __syncthreads();
   for (int br = blockIdx.x; br < B * P; br += gridDim.x) {
     const int first = off_s[br * PH], total = off_s[(br + 1) * PH] - first, own = (br % P) * H;
     for (int i = threadIdx.x; i < PH; i += kGatherThreads) seg_off[(int64_t)br * PH + i] = off_s[br * PH + i] - first;
@@ -472,13 +512,14 @@ __global__ void __launch_bounds__(kGatherThreads)
   unsigned char* ring = smem_raw + (size_t)warp * kGatherStages * entry_bytes;
   int64_t(*dst_s)[kMaxRanks] = dst_all[warp];
   const int n_units = gridDim.x * n_copy;
-  // Blocks are copied to between none and all consumers, so a warp takes its next one, (batch, head, block), from a counter,
-  // and the number after that while it looks the block up.
+  // Blocks are copied to between one and all consumers, so a warp takes its next one, a number among those that anybody
+  // receives, from a counter, and the number after that while it looks the block up.
   int next = blockIdx.x * n_copy + warp;
-  const int n_blocks = B * H * NB;
+  const int n_blocks = pos_s[n_words];
+  int word = 0;  // the one that holds the last block taken (numbers only grow)
   // where consumer r's copy of block j goes, -1 if it gets none
   auto destination = [&](int bb, int h, int j, int p, int r) -> int64_t {
-    if (r >= P || (r == p && !include_local)) return -1;
+    if (r == p && !include_local) return -1;
     const int br = bb * P + r;
     const uint32_t* u = U + ((int64_t)br * H + h) * Wd;
     const uint32_t* own = own_s + p * Wd;
@@ -496,20 +537,29 @@ __global__ void __launch_bounds__(kGatherThreads)
     }
     return byte;
   };
-  // Loads the next block that anybody receives into stage st; false: there is none left.
+  // Loads the next block into stage st; false: there is none left.
   auto load_next = [&](int st) -> bool {
     while (next < n_blocks) {
       int after = 0;
       if (lane == 0) after = n_units + atomicAdd(n_taken, 1);
-      const int bh = next / NB, j = next - bh * NB, p = rank[j];
+      for (int full_words = 32; full_words == 32; word += full_words)  // words whose blocks have lower numbers
+        full_words = __popc(__ballot_sync(0xffffffffu, word + lane < n_words && pos_s[word + lane + 1] <= next));
+      uint32_t left = live_s[word];
+      for (int skip = next - pos_s[word]; skip > 0; --skip) left &= left - 1u;
+      const int bit = __ffs(left) - 1, bh = word / Wd, w = word - bh * Wd, j = w * 32 + bit;
+      // its owner, looked for by a lane per rank
+      int p = __ffs(__ballot_sync(0xffffffffu, lane < P && ((own_s[lane * Wd + w] >> bit) & 1u))) - 1;
+      if (p < 0) p = 31 + __ffs(__ballot_sync(0xffffffffu, lane + 32 < P && ((own_s[(lane + 32) * Wd + w] >> bit) & 1u)));
       const int bb = bh / H, h = bh - bb * H;
-      const bool owned = (unsigned)p < (unsigned)P;
-      const int64_t d0 = owned ? destination(bb, h, j, p, lane) : -1;
-      const int64_t d1 = owned && P > 32 ? destination(bb, h, j, p, lane + 32) : -1;
+      bool any = false;
+#pragma unroll 1
+      for (int r = lane; r < P; r += 32) {
+        const int64_t d = destination(bb, h, j, p, r);
+        dst_s[st][r] = d;
+        any = any || d >= 0;
+      }
       next = __shfl_sync(0xffffffffu, after, 0);
-      if (!__any_sync(0xffffffffu, d0 >= 0 || d1 >= 0)) continue;
-      dst_s[st][lane] = d0;
-      dst_s[st][lane + 32] = d1;
+      if (!__any_sync(0xffffffffu, any)) continue;  // (no room for any of its copies)
       if (lane == 0) {
         unsigned char* buf = ring + (size_t)st * entry_bytes;
         ptx::mbar_expect_tx(full + st, 2 * tile_bytes);
@@ -521,21 +571,25 @@ __global__ void __launch_bounds__(kGatherThreads)
     return false;
   };
   int n = 0;  // blocks loaded
-  while (n < kGatherStages - 1 && load_next(n)) ++n;
-  for (int q = 0; q < n; ++q) {
-    const int st = q % kGatherStages;
-    const unsigned char* buf = ring + (size_t)st * entry_bytes;
-    ptx::mbar_wait_bounded(full + st, (uint32_t)((q / kGatherStages) & 1), &s_abort, status, 50, 200000000LL);
-    const int64_t d0 = dst_s[st][lane], d1 = dst_s[st][lane + 32];
-    // (an entry is the K tile and the V tile behind it, here as there)
-    if (d0 >= 0) bulk_store(packed + d0, buf, (uint32_t)entry_bytes);
-    if (d1 >= 0) bulk_store(packed + d1, buf, (uint32_t)entry_bytes);
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    if (n == q + kGatherStages - 1) {
+  bool more = true;
+  for (int q = 1 - kGatherStages; q < 0 || q < n; ++q) {
+    if (q >= 0) {
+      const int st = q % kGatherStages;
+      const unsigned char* buf = ring + (size_t)st * entry_bytes;
+      ptx::mbar_wait_bounded(full + st, (uint32_t)((q / kGatherStages) & 1), &s_abort, status, 50, 200000000LL);
+      // (an entry is the K tile and the V tile behind it, here as there)
+      for (int r = lane; r < P; r += 32) {
+        const int64_t d = dst_s[st][r];
+        if (d >= 0) bulk_store(packed + d, buf, (uint32_t)entry_bytes);
+      }
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+    if (more) {
       // the stage of block q - 1 may be refilled once every lane's stores have read it
       asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
       __syncwarp();
-      if (load_next(n % kGatherStages)) ++n;
+      more = load_next(n % kGatherStages);
+      n += more ? 1 : 0;
     }
   }
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -551,7 +605,8 @@ int launch_demand_pack(const sparsp_shape& s, const Geometry& g, const uint32_t*
   int32_t* status = (int32_t*)(ws + L.status);
   const int64_t T = (int64_t)g.B * P * P * g.H, tile_bytes = 2LL * g.b * g.d;
   const int n_copy = pack_warps((int)tile_bytes);
-  const int64_t smem = n_copy * kGatherStages * 2 * tile_bytes + (T + 1) * 4 + (int64_t)P * g.Wd * 4;
+  const int64_t n_words = (int64_t)g.B * g.H * g.Wd;
+  const int64_t smem = n_copy * kGatherStages * 2 * tile_bytes + (T + 1 + 2 * n_words + 1 + (int64_t)P * g.Wd) * 4;
   PackLaunch c;
   if (T <= kScanMax && smem <= kGatherSmem) {
     if ((rc = prepare_pack(s, g, K, V, (const void*)gather_kernel, (int)smem, &c)) != SPARSP_OK) return rc;
