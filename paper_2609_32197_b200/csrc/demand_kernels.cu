@@ -2,6 +2,7 @@
 // pack-order offsets, the destination table, and the gather of K/V tiles into per-consumer buffers.
 // Everything before the gather is small integer work on bit words; the gather is the HBM-bound part.
 #include <algorithm>
+#include <climits>
 
 #include "block_sets.cuh"
 #include "common.cuh"
@@ -634,11 +635,14 @@ int launch_demand_pack(const sparsp_shape& s, const Geometry& g, const uint32_t*
 // the slot designated for that pair).  Entry (h, j) sits where it sits inside the consumer's buffer, minus the segment's
 // first entry, so that consumer and producer derive the same byte ranges from the demand counts.
 // The entries are U[consumer][h] & own[producer], head by head, blocks ascending.  Their places in the slot are
-// consecutive, so a warp that takes every n-th entry finds its block by counting bits from the entry before: no
+// consecutive, so a warp that takes every n-th entry finds its head in the offsets and its block by counting bits: no
 // tables and no launch that fills them.  Tiles move as in pack_kernel.  HBM-bound: seven segments of 175 MB, read and
-// written, 426 us with tables, 399 without, 395 with every second one walked backwards, 389-392 with the hint above (6.3
-// TB/s); 421 with a run of consecutive entries per warp instead of every n-th.
+// written, 426 us with tables, 382-384 this way (6.4 TB/s); 421 with a run of consecutive entries per warp instead of
+// every n-th.  Three tiles per warp: with two loads in flight reads and writes alternate best (four 390, five 394).  Small
+// segments, 80 entries of 40 heads / 400 of 200: 9.2 / 9.0 us with tables, 6.2 / 6.2; walking from head to head 18 / 52.
 // ------------------------------------------------------------------------------------------------
+constexpr int kSegmentStages = 3;
+
 __global__ void __launch_bounds__(32 * kPackMaxWarps)
     segment_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                    const uint32_t* __restrict__ U, const int32_t* __restrict__ rank, int H, int NB, int Wd, int P,
@@ -646,14 +650,14 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps)
                    int b, uint32_t tile_bytes, unsigned char* __restrict__ slot, int64_t capacity,
                    int32_t* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ uint64_t full_all[kPackMaxWarps * kPackStages];
+  __shared__ uint64_t full_all[kPackMaxWarps * kSegmentStages];
   __shared__ int s_abort;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-  uint64_t* full = full_all + warp * kPackStages;
-  unsigned char* ring = smem_raw + (size_t)warp * kPackStages * tile_bytes;  // this warp's buffers
+  uint64_t* full = full_all + warp * kSegmentStages;
+  unsigned char* ring = smem_raw + (size_t)warp * kSegmentStages * tile_bytes;  // this warp's buffers
   if (threadIdx.x == 0) s_abort = 0;
   if (lane == 0) {
-    for (int st = 0; st < kPackStages; ++st) ptx::mbar_init(full + st, 1);
+    for (int st = 0; st < kSegmentStages; ++st) ptx::mbar_init(full + st, 1);
     ptx::mbar_init_fence();
   }
   enter_grid(U, rank, seg_off, cnt);
@@ -676,23 +680,46 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps)
   auto entry = [&](int q) { return back ? n_entries - 1 - unit - (q >> 1) * n_units : unit + (q >> 1) * n_units; };
   if (n_local > 0) {
     const uint32_t* u_row = U + (int64_t)consumer * H * Wd;
-    auto head_words = [&](int h) { return h >= 0 && h < H && lane < Wd ? u_row[(int64_t)h * Wd + lane] & own : 0u; };
-    int h = back ? H - 1 : 0, total, at;  // the head, its entries, its first entry
-    uint32_t words = head_words(h), next = head_words(back ? h - 1 : h + 1);
-    int below = bits_below(words, lane, &total);
-    at = back ? n_entries - total : 0;
-    // head * NB + block of entry e; -1 where there is none, should the counts promise more than there are
-    auto block_of = [&](int e) -> int {
-      while (back ? e < at : e >= at + total) {
-        if (!back) at += total;
-        h += back ? -1 : 1;
-        if (h < 0 || h >= H) return -1;
-        words = next;
-        next = head_words(back ? h - 1 : h + 1);
-        below = bits_below(words, lane, &total);
-        if (back) at -= total;
+    // the head that entry e belongs to, the last one that begins at or before it
+    auto head_of = [&](int e) -> int {
+      int lo = 0, end = H;
+      while (end - lo > 1) {
+        const int step = (end - lo + 31) / 32, h = lo + lane * step;
+        const int c = __popc(__ballot_sync(0xffffffffu, h < end && off[h] - first <= e));
+        lo += max(c - 1, 0) * step;
+        end = min(end, lo + step);
       }
-      const int k = e - at;
+      return lo;
+    };
+    auto head_words = [&](int h) { return lane < Wd ? u_row[(int64_t)h * Wd + lane] & own : 0u; };
+    // The head of the next entry to load, its first entry, and its words on their way.  Where the heads begin is kept a lane
+    // per head, 32 of them in the direction of the walk, so that a look needs no load.
+    int h, at, h0, x_at;
+    uint32_t words;
+    auto keep_heads = [&](int from) {
+      h0 = from;
+      const int x = back ? h0 - lane : h0 + lane;
+      x_at = x >= 0 && x < H ? (int)(off[x] - first) : back ? 0 : INT_MAX;
+    };
+    auto look_up = [&](int e) {
+      uint32_t begun = __ballot_sync(0xffffffffu, x_at <= e);  // of the heads kept: from one on (back), or up to one
+      if (begun == (back ? 0u : ~0u)) {
+        keep_heads(head_of(e));
+        begun = __ballot_sync(0xffffffffu, x_at <= e);
+      }
+      const int found = back ? __ffs(begun) - 1 : __popc(begun) - 1;
+      h = back ? h0 - found : h0 + found;
+      at = __shfl_sync(0xffffffffu, x_at, found);
+      words = head_words(h);
+    };
+    keep_heads(head_of(entry(0)));
+    look_up(entry(0));
+    // head * NB + block of entry e, which has been looked up; -1 where there is none, should the counts promise more than
+    // there are
+    auto block_of = [&](int e) -> int {
+      int total;
+      const int below = bits_below(words, lane, &total), k = e - at;
+      if (k >= total) return -1;
       const int w = 31 - __clz(__ballot_sync(0xffffffffu, words != 0u && below <= k));
       uint32_t left = __shfl_sync(0xffffffffu, words, w);
       for (int skip = k - __shfl_sync(0xffffffffu, below, w); skip > 0; --skip) left &= left - 1u;
@@ -703,30 +730,33 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps)
       if ((q & 1) == 0) s_load = block_of(entry(q));
       if (s_load < 0) {
         n_local = q;
-      } else if (lane == 0) {
-        uint64_t* bar = full + q % kPackStages;
+        return;
+      }
+      if (lane == 0) {
+        uint64_t* bar = full + q % kSegmentStages;
         const int hd = s_load / NB;
         ptx::mbar_expect_tx(bar, tile_bytes);
-        ptx::tma_load_4d(ring + (size_t)(q % kPackStages) * tile_bytes, q & 1 ? &tmV : &tmK, bar, 0, (s_load - hd * NB) * b,
+        ptx::tma_load_4d(ring + (size_t)(q % kSegmentStages) * tile_bytes, q & 1 ? &tmV : &tmK, bar, 0, (s_load - hd * NB) * b,
                          hd, 0);
       }
+      if ((q & 1) && q + 1 < n_local) look_up(entry(q + 1));
     };
-    for (int q = 0; q < kPackStages - 1 && q < n_local; ++q) issue_load(q);
+    for (int q = 0; q < kSegmentStages - 1 && q < n_local; ++q) issue_load(q);
     for (int q = 0; q < n_local; ++q) {
       const int64_t e = entry(q);
-      ptx::mbar_wait_bounded(full + q % kPackStages, (uint32_t)((q / kPackStages) & 1), &s_abort, status, 50, 200000000LL);
+      ptx::mbar_wait_bounded(full + q % kSegmentStages, (uint32_t)((q / kSegmentStages) & 1), &s_abort, status, 50, 200000000LL);
       if (lane == 0) {
         if ((e + 1) * 2 * tile_bytes <= capacity)
-          bulk_store(slot + (2 * e + (q & 1)) * tile_bytes, ring + (size_t)(q % kPackStages) * tile_bytes, tile_bytes);
+          bulk_store(slot + (2 * e + (q & 1)) * tile_bytes, ring + (size_t)(q % kSegmentStages) * tile_bytes, tile_bytes);
         else
           atomicExch(status, SPARSP_ERR_CAPACITY);  // does not fit: left out
       }
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-      if (q + kPackStages - 1 < n_local) {
+      if (q + kSegmentStages - 1 < n_local) {
         // the buffer of item q - 1 may be refilled once its store has read it
         asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
         __syncwarp();
-        issue_load(q + kPackStages - 1);
+        issue_load(q + kSegmentStages - 1);
       }
     }
   }
@@ -737,7 +767,7 @@ int launch_pack_segment(const sparsp_shape& s, const Geometry& g, const uint32_t
                         int consumer, int producer, const int64_t* seg_off, const int32_t* cnt, const void* K,
                         const void* V, void* dst, int64_t capacity, char* ws, const WsLayout& L, cudaStream_t st) {
   PackLaunch c;
-  const int n_warps = pack_warps(g.b * g.d * 2), smem = n_warps * kPackStages * g.b * g.d * 2;
+  const int n_warps = pack_warps(g.b * g.d * 2), smem = n_warps * kSegmentStages * g.b * g.d * 2;
   const int rc = prepare_pack(s, g, K, V, (const void*)segment_kernel, smem, &c);
   if (rc != SPARSP_OK) return rc;
   SPARSP_CUDA_OK(launch_kernel(segment_kernel, c.grid, 32 * n_warps, (size_t)smem, st, c.tk, c.tv, U, rank, g.H, g.NB, g.Wd, P,

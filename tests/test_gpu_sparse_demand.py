@@ -1,5 +1,5 @@
-"""Demand in few heads and blocks, or none: the gather hands out only blocks that anybody receives.  And the gather at the edge
-of its shared memory, where the one by tables begins."""
+"""Demand in few heads and blocks, or none: the gather hands out only blocks that anybody receives, and a segment's walk goes
+straight to the heads that have entries.  And the gather at the edge of its shared memory, where the one by tables begins."""
 import numpy as np
 import pytest
 import torch
@@ -65,3 +65,31 @@ def test_edge_of_the_shared_memory(oracle_mod, binding, H, P, NB):
     rng = np.random.default_rng(NB)
     M = rng.random((H, NB, NB)) < 0.004
     _pack(oracle_mod, binding, M, P, (rng.permutation(NB) % P).astype(np.int32), 64, 64, False)
+
+
+@pytest.mark.parametrize("heads", ["first", "last", "around a search step", "every other"])
+@pytest.mark.parametrize("H,NB", [(1, 40), (33, 9), (70, 33), (1030, 5)])
+def test_segments_of_few_heads(oracle_mod, binding, heads, H, NB):
+    P, d, b = 3, 64, 64
+    entry = 4 * b * d
+    rng = np.random.default_rng(H)
+    live = {"first": [0], "last": [H - 1], "around a search step": [h for h in (30, 31, 32, 33, 65, 1023, 1024) if h < H],
+            "every other": list(range(1, H, 2))}[heads]
+    M = np.zeros((H, NB, NB), bool)
+    M[live] = rng.random((len(live), NB, NB)) < 0.5
+    rank = (rng.permutation(NB) % P).astype(np.int32)
+    K, V, shape, rank_d, ws, got = _pack(oracle_mod, binding, M, P, rank, d, b, False)
+    cnt, seg, total = got["cnt"][0].cpu(), got["seg_offset"][0].cpu(), got["seg_total"][0].cpu()
+    start = torch.cat([torch.zeros(1, dtype=torch.int64), total.cumsum(0)]) * entry
+    for r in range(P):
+        for p in range(P):
+            n = int(cnt[r, p].sum())
+            if p == r:
+                continue
+            first = int(start[r]) + int(seg[r, p, 0]) * entry
+            slot = torch.full(((n + 1) * entry,), 0xEE, dtype=torch.uint8, device="cuda")
+            binding.sparsp_pack_segment(shape, got["union_mask"], rank_d, P, r, p, got["cnt"], got["seg_offset"], K, V, slot,
+                                        n * entry, ws)
+            assert binding.sparsp_status(ws) == binding.SPARSP_OK
+            assert torch.equal(slot[:n * entry], got["packed"][first:first + n * entry])
+            assert bool((slot[n * entry:] == 0xEE).all())
