@@ -263,3 +263,29 @@ def test_scores_that_are_no_numbers(binding, d, b, source, key, value):
     finite = keep & torch.isfinite(plain[1])
     assert bool(torch.isfinite(lse[finite]).all()) and (lse - plain[1])[finite].abs().max() <= 2e-2
     assert torch.equal(lse[keep & ~finite], plain[1][keep & ~finite])
+
+
+@pytest.mark.parametrize("d,b", [(64, 64), (128, 128)])
+@pytest.mark.parametrize("shift", [0, 8])
+def test_rows_that_keep_nothing(binding, d, b, shift):
+    """32-byte stores where the output begins on such a boundary, 16-byte ones where it does not."""
+    H, NB = 6, 21
+    N = NB * b - 9
+    g = torch.Generator(device="cuda").manual_seed(d)
+    Q, K, V = (torch.randn(H, N, d, generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    kept = torch.rand(H, NB, NB, generator=g, device="cuda") < 0.2
+    kept[:, ::2] = False
+    kept[:, -1] = False
+    kept[2] = False
+    shape = binding.make_shape(H, d, (1, 1, N), 0, b)
+    ws = binding.make_workspace(shape, 1)
+    buf = torch.full((Q.numel() + 16,), 7.0, dtype=torch.bfloat16, device="cuda")
+    O, lse = buf[shift:shift + Q.numel()].view_as(Q), torch.full((1, H, N), 7.0, device="cuda")
+    binding.sparsp_sparse_attn_fwd(shape, Q, K, V, _mask(kept), 0.0, O, lse, ws)
+    assert binding.sparsp_status(ws) == binding.SPARSP_OK
+    rows = kept.any(-1).repeat_interleave(b, 1)[:, :N]
+    want, want_lse = _reference(Q, K, V, kept, b)
+    assert bool((O[~rows] == 0).all()) and bool((lse[0][~rows] == float("-inf")).all())
+    assert (O.double() - want)[rows].abs().max() <= pu.ATTN_MAX_ABS
+    assert (lse[0].double() - want_lse)[rows].abs().max() <= 2e-2
+    assert bool((buf[:shift] == 7.0).all()) and bool((buf[shift + Q.numel():] == 7.0).all())
