@@ -365,7 +365,7 @@ def figures(cfg, t, peaks, traffic_table):
                      "unit": "TFLOP/s", "frac": attn_tflops / peaks["bf16_tflops"],
                      "traffic": traffic[0] if traffic else None,
                      "traffic_source": traffic[1] if traffic else "no ncu capture of this configuration"},
-        "roofline_pack": {"bound": "hbm", "kernel": "pack_kernel", "achieved": pack_gbs, "peak": peaks["hbm_gbs"],
+        "roofline_pack": {"bound": "hbm", "kernel": "gather_kernel", "achieved": pack_gbs, "peak": peaks["hbm_gbs"],
                           "peak_source": peaks["source"], "unit": "GB/s", "frac": pack_gbs / peaks["hbm_gbs"],
                           "algorithmic_bytes": pack_bytes},
     }

@@ -282,9 +282,9 @@ def test_degenerate_shapes(oracle_mod, binding):
 @pytest.mark.parametrize("d,b", [(128, 128), (64, 64), (128, 64)])
 @pytest.mark.parametrize("jump", [30.0, 100.0])
 def test_scores_far_above_the_first_tile(oracle_mod, binding, d, b, jump):
-    """The kernel skips a tile's row-maximum pass when a norm bound shows the scores stay within 2^64 of the
-    row's reference.  Here the first kept block scores 0 and a later one `jump` (log2 units) higher: 30 stays
-    inside the bound (exponentials up to 2^30 against the old reference), 100 does not (reference must move).
+    """The kernel takes an item relative to 0 or to its first tile's row maxima and sees at its end whether that was right.
+    Here the first kept block scores 0 and a later one `jump` (log2 units) higher: 30 stays inside the range (exponentials
+    up to 2^30), 100 does not (the row sum is beyond it, and the item is computed again with its running maximum).
     Both must give the oracle's result: the mean of V over the high-scoring block, to 2^-jump."""
     H = 2
     NB = 6
@@ -331,11 +331,10 @@ def test_scores_far_above_the_first_tile(oracle_mod, binding, d, b, jump):
 @pytest.mark.parametrize("outlier", [False, True])
 @pytest.mark.parametrize("v_sigma", [1.0, 0.5])
 def test_long_lists_with_final_reference_and_ragged_tail(oracle_mod, binding, d, b, outlier, v_sigma):
-    """Lists long enough (13 kept blocks per row, a different random set per row) that the kernel stops
-    updating a row's reference once the item's largest key norm bounds all remaining scores, with the ragged
-    last block of the sequence in every list.  With `outlier` one block holds keys of 40 times the norm
-    (orthogonal to the queries, so its scores stay ordinary): the item-wide bound then fails while the
-    per-tile bound holds for the other tiles, and the reference keeps being checked tile by tile."""
+    """Lists long enough (13 kept blocks per row, a different random set per row) that the kernel takes them relative to a
+    reference that is final from the first tile on, with the ragged last block of the sequence in every list.  With
+    `outlier` one block holds keys of 40 times the norm (orthogonal to the queries, so its scores stay ordinary): nothing
+    but the scores themselves may decide."""
     H, NB = 2, 20
     N = NB * b - 37
     rng = np.random.default_rng(23 + d + b)
@@ -417,8 +416,8 @@ def test_demand_plan_with_the_most_ranks_and_blocks(oracle_mod, binding):
 @pytest.mark.parametrize("seed", [1, 2, 3, 4, 5, 6])
 @pytest.mark.parametrize("v_sigma", [1.0, 0.5])
 def test_random_norm_profiles(oracle_mod, binding, seed, v_sigma):
-    """Random shapes with key blocks and query rows scaled by random factors (0.1 ... 20): tiles whose norm
-    bound holds, tiles where it fails, references that become final early, late or never, all in one launch."""
+    """Random shapes with key blocks and query rows scaled by random factors (0.1 ... 20): items that stay in the range,
+    items that leave it, rows that take the running maximum from their first tile on, all in one launch."""
     rng = np.random.default_rng(100 + seed)
     d = int(rng.choice([64, 128]))
     b = int(rng.choice([64, 128]))
@@ -454,11 +453,11 @@ def test_random_norm_profiles(oracle_mod, binding, seed, v_sigma):
 @pytest.mark.parametrize("d,b", [(128, 128), (64, 64), (128, 64), (64, 128)])
 @pytest.mark.parametrize("level", [30.0, 74.0])
 def test_fixed_reference_at_the_edge_of_its_bound(oracle_mod, binding, d, b, level):
-    """An item whose norm bound |q| |k| scale log2(e) stays under 2^80 runs on the fixed reference 0.  Here every score
-    is about +level or -level (log2 units; 74 is just inside the bound): query blocks that keep only the low-scoring
-    blocks work with exponentials around 2^-74 throughout, blocks that keep only the high ones with 2^+74, the rest
-    with both at once.  All must give the oracle's rows (and log-sum-exp), which for the one-sided blocks are close
-    to the mean of V over the kept keys."""
+    """A long item runs on the fixed reference 0 unless its first scores are far from it.  Here every score is about
+    +level or -level (log2 units; 30 is near, 74 is far): at 30, query blocks that keep only the low-scoring blocks work
+    with exponentials around 2^-30 throughout, blocks that keep only the high ones with 2^+30, the rest with both at once;
+    at 74 all take the running maximum.  All must give the oracle's rows (and log-sum-exp), which for the one-sided blocks
+    are close to the mean of V over the kept keys."""
     H, NB = 2, 12
     N = NB * b - 7                                    # ragged last block
     rng = np.random.default_rng(29)

@@ -1,7 +1,7 @@
 """Seeded random sweep of the whole path against the oracle: head dim, block size, head count, rank count, grid, text
 length, layout, k, placement and input statistics are all drawn per case.  Three kinds of case: the generator's
 structured inputs; unstructured inputs with per-token norm profiles (log-normal, up to e^1.5 spread: stress for the
-norm bounds and the frozen reference of the attention kernel); and the same with an ARBITRARY mask handed to the
+range checks and the fixed reference of the attention kernel); and the same with an ARBITRARY mask handed to the
 demand / pack / attention calls (random density per row, some rows empty, some full), which the selection step never
 produces but the calls must handle.  Integers and bytes bit-exact, attention within the stated tolerance on every row."""
 import numpy as np
