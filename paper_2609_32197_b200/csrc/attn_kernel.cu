@@ -28,9 +28,9 @@
 // takes the row sums.  Whether that was right is seen from the finished row sums and the exponents on the way, and an
 // item that left the range is computed again (kRefZero ... below).  Only such an item, and rows whose first scores are out
 // of range, take their maxima as they go: the two threads that own the same row (one per warpgroup) then share the reference
-// through shared memory and take their decisions strictly in tile order (a pair of 64-thread named barriers per row group
-// hands the turn back and forth), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since
-// the reference last moved -- the thread that decides so first waits for every P V issued so far.
+// through shared memory and take their decisions strictly in tile order (two mbarriers per row group hand the turn back and
+// forth), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since the reference last moved --
+// the thread that decides so first waits for every P V issued so far.
 // (The range used to be proved beforehand, by Cauchy-Schwarz from key norms that a pass over K took ahead of every call
 // and row norms taken from the Q tile of every item, and not at all for a packed source, whose tiles all took their
 // maximum in turns.  us per call then and now: one hop of 40 heads x 75600 over 8 ranks, 7 tiles an item, 97-112 -> 75;
@@ -102,7 +102,7 @@ constexpr float kGrowThreshold = 8.0f;
 // So that this is rare, the four warps of the item's first tile look at it first: rows whose first scores are far from 0
 // take the running maximum from the start, the 32 rows of a warp together (kZeroSample: every eighth score; kFirstSample:
 // the maximum that the reference is anyway).  Ordinary scores pass both: with unit-variance Q and K at d = 128 they are
-// within +-16.  (us per call of 13 heads x 2 x 6034 tokens, Q times 1, 4 and 60: 88, 140 and 133; looking for +-64 only 183
+// within +-16.  (us per call of 13 heads x 2 x 6034 tokens, Q times 1, 4 and 60: 87, 144 and 136; looking for +-64 only 183
 // with Q times 4; with range proofs from the norms of rows and keys instead of all this 91, 131 and 140.)
 // All of this follows from the item alone, so a call repeats itself bit for bit whichever CTA takes which item.  (A CTA that
 // remembered failures and began its next items further on was right too, but let rows of ordinary heads change in their
@@ -154,7 +154,7 @@ struct AttnCfg {
   static constexpr int kOffSlot = kOffEntV + 2 * 2 * kMaxBlocks;  // int32 [2][1024] packed-buffer slot per entry
   static constexpr int kOffRef = kOffSlot + 2 * 4 * kMaxBlocks;  // float [4 items][128] reference per row
   static constexpr int kOffBars = kOffRef + 4 * 128 * 4;
-  static constexpr int kNumBars = 2 + 2 * (kStagesK + kStagesV) + 10 + 1 + 4 + 4;
+  static constexpr int kNumBars = 2 + 2 * (kStagesK + kStagesV) + 10 + 1 + 4 + 4 + 8 + 1;
   static constexpr int kColS = 0;    // S buffers: columns [0, 256)
   static constexpr int kColP = 256;  // P: two buffers in columns [256, 384), or one in [256, 320) with the row sums in [320, 336)
   static constexpr int kColO = 384;  // accumulator: columns [384, 384 + d)
@@ -247,10 +247,6 @@ __device__ __forceinline__ void clear_rows(const AttnParams& p, int bh, int i) {
     for (int r = lane; r < n; r += 32) p.lse[bh * p.N + tok0 + r] = -INFINITY;
 }
 
-__device__ __forceinline__ void named_bar_sync(int id, int n) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-
 template <int D, int BLK, bool kPacked>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -288,6 +284,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // [4] the four warps that own an item's first tile have left what it says in s_exact and, if that is the reference, in
   // sRef.  Four, because the other warpgroup, which waits for it, may be up to three tiles and as many items behind.
   uint64_t* ref_ready = list_free + 2;
+  // [2][4] the warpgroup's warp of a row group has decided about the running maximum of a tile.  (Not named barriers, which
+  // cannot be bounded: after a wait that has run out two warps need not agree on who takes turns.  Every lane arrives: with
+  // one lane behind a __syncwarp and the count of waits in shared memory 13 heads x 2 x 6034, Q times 8, took 138 us, not 132.)
+  uint64_t* turn = ref_ready + 4;
+  uint64_t* placed = turn + 8;     // in-place calls: the eight softmax warps know whether the item is to be computed again
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
   int* s_nent = reinterpret_cast<int*>(smem + C::kOffMisc + 8);   // [2]
@@ -328,6 +329,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     for (int s = 0; s < 4; ++s) mbar_init(o_full + s, 1);
     mbar_init(o_drained, 8);
     for (int s = 0; s < 4; ++s) mbar_init(ref_ready + s, 4);
+    for (int s = 0; s < 8; ++s) mbar_init(turn + s, 32);
+    mbar_init(placed, 8);
     mbar_init_fence();
     *s_abort = 0;
   }
@@ -831,9 +834,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     const uint32_t tS = tmem_base + C::kColS + wg * 128 + lane_off;
     const uint32_t tP = tmem_base + C::kColP + (C::kNumP == 2 ? wg * 64 : 0) + lane_off;
     const uint32_t tO = tmem_base + C::kColO + lane_off;
-    const int bar_mine = 1 + wg * 4 + rgrp;         // I arrive here after my decision
-    const int bar_other = 1 + (1 - wg) * 4 + rgrp;  // the row group's other warp arrives here after its decision
+    const int mine = wg * 4 + rgrp, other = (1 - wg) * 4 + rgrp;  // the two warps of a row group
     int g0 = 0;       // number of the item's first tile
+    int turns = 0;    // waits for the other warp of the row group so far
     for (int i = 0;; ++i) {
       const int buf = i & 1;
       mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 56, p.wait_limit);
@@ -853,6 +856,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         mbar_wait_bounded_inline(ref_ready + (i & 3), (i >> 2) & 1, s_abort, 43, p.wait_limit);
         exact = s_exact[(i & 3) * 4 + rgrp] != 0;
         if (ref_of == kRefFirst && !exact) m_ref = ref[row];
+      };
+      auto take_turn = [&]() {  // the other warp has decided about the tile before, and may have moved the reference
+        mbar_wait_bounded_inline(turn + other, turns++ & 1, s_abort, 44, p.wait_limit);
+        m_ref = ref[row];
       };
       // the row's largest score of a tile: one flat instruction stream per 64-key half, an absent half (not kept by this
       // row's query block) is skipped
@@ -946,10 +953,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (kExact) {
           const float mx = row_max(sv, vh);
           // ---- my turn to look at / move the row's reference maximum (strictly in tile order) ----
-          if (n > 0) {
-            named_bar_sync(bar_other, 64);
-            m_ref = ref[row];  // (the other thread may have moved it since my last tile)
-          }
+          if (n > 0) take_turn();
           const float m_new = fmaxf(m_ref, mx);
           const bool grow = m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY);
           if (__any_sync(0xffffffffu, grow)) {
@@ -985,7 +989,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             }
           }
           if (n == 0 && m_ref == -INFINITY) ref[row] = m_ref;
-          if (n + 1 < n_tiles) asm volatile("bar.arrive %0, %1;" ::"r"(bar_mine), "r"(64) : "memory");
+          mbar_arrive(turn + mine);
         }
 
         // exponentials of keys [64h, 64h+64) -> packed bf16 columns [32h, 32h+32) of the P buffer
@@ -1047,10 +1051,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       g0 += n_tiles;
       // ---- item epilogue: warpgroup x writes the column half x of every row -------------------------
       if (first >= n_tiles && ref_of != kRefExact) learn_ref();
-      if (exact) {
-        named_bar_sync(9 + rgrp, 64);  // all decisions about the row group are done
-        m_ref = ref[row];
-      }
+      if (exact && ((n_tiles - 1 - first) & 1)) take_turn();  // (the last tile was the other warp's)
       const int last = g0 - 1;
       mbar_wait_bounded_inline(o_full + (last & 3), (last >> 2) & 1, s_abort, 40, p.wait_limit);
       tc_fence_after();
@@ -1082,7 +1083,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           }
           if (__any_sync(0xffffffffu, failed) && lane == 0) s_failed[buf] = 1;
           if (p.in_place) {  // the rows of an item that is computed again are still its queries
-            named_bar_sync(13, 256);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(placed);
+            mbar_wait_bounded_inline(placed, i & 1, s_abort, 45, p.wait_limit);
             if (s_failed[buf]) tok = p.N;
           }
         }
