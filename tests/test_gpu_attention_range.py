@@ -1,6 +1,8 @@
-"""Items whose scores leave the range that the attention kernel assumes are computed again: relative to their first tile,
-then with the running maximum.  Rows of all three kinds among many items per CTA, the last items of the call among them,
-against a masked softmax in 64 bits.  And 64-token blocks where every one has an SM of its own, at the edge of that rule."""
+"""Rows whose first scores are out of the range that the attention kernel assumes take their running maximum, and items
+whose scores leave it later are computed again.  Rows of all kinds among many items per CTA, the last items of the call among
+them, against a masked softmax in 64 bits; the same bits whoever computes them; the output in the place of the queries; large
+values; scores that are no numbers; rows that keep nothing.  And 64-token blocks where every one has an SM of its own, at the
+edge of that rule."""
 import math
 
 import pytest
