@@ -8,13 +8,20 @@
 //                zeroed in P.
 // The kernel is persistent: one CTA per SM takes items from a global counter; the next item's kept
 // list, Q tile and first K/V tiles overlap the current item's last tiles, its first Q K^T the epilogue.
+// Where an item ends, only the warpgroup of its last tile waits for the accumulator and writes the rows; the other one is
+// already at the next item, whose Q tile has a buffer of its own: the next one of the K ring, which gets the finished
+// item's Q buffer in exchange.  (Both warpgroups writing half of the columns, the Q tile behind the last Q K^T in a buffer
+// that is always Q's: 13 heads x 2 x 6034 tokens, 9 tiles an item, 86.9 us a call, now 78.2; 16 x 18600 with 6 to 30 tiles
+// 306 / 282; 40 x 75600, 59 tiles, 10.05 / 9.82 ms; one hop of it over 8 ranks, 2 to 8 tiles, 64.1 / 61.1.  Tried on top and
+// no better: rows through shared memory and a TMA store, lists for one or two items more, tiles dealt so that the
+// warpgroups take turns at writing.)
 // The scores S = Q K^T are double-buffered in tensor memory (S: 2 x 128 fp32 columns; P: 64 columns of packed bf16,
 // two buffers at d = 64, one at d = 128 where 16 columns hold the row sums instead; O: d columns), so that the tensor pipe always has the next
 // tiles' MMAs queued while the softmax of the current tile runs: Q K^T of tile g+2 starts as soon as the
 // scores of tile g have been READ, and P V of tile g is issued as soon as P_g is written.  Tiles are
 // numbered g = 0, 1, 2, ... across the CTA's items; every ring, buffer and barrier phase follows g.
 // Warp roles (512 threads = 4 warpgroups; the first two hand most of their registers to the other two):
-//   warp 0      TMA producer of Q (per item) and of the K ring
+//   warp 0      TMA producer of Q (per item) and K, which share a ring of buffers
 //   warp 1      issues every Q K^T          warp 2      issues every P V
 //   warp 3      TMA producer of the V ring
 //   warp 4      builds the kept / union list of the NEXT items (two list buffers)
@@ -116,15 +123,45 @@ constexpr float kSafeSumFirst = 33554432.0f;            // 2^25: kGrowThreshold 
 constexpr float kZeroSample = 48.0f, kFirstSample = 64.0f;
 constexpr int kZeroMinTiles = 4;  // K / V source: shorter items take kRefFirst, whose largest terms are exact
 // Tuning switch (compile-time): how many of the exponentials go to the FMA pipe instead of the
-// special-function unit (every n-th pair; 0 = none).
+// special-function unit (every n-th pair; 0 = none).  us per attention call with every 3rd / 4th / 6th / none:
+//   d = 128, K / V source    40 heads x 75600, 10 % kept 9884 / 9816 / 9903 / 10596, 24 x 24576 of 64-token blocks with
+//                            threshold lists 671 / 665 / 681 / 690, 2 x 13560 38.9 / 37.8 / 37.8 / 37.3
+//   ... packed source, 128-token blocks (hops: 2 to 8 tiles an item)    62.5 / 61.4 / 61.2 / 60.5; with none lists as long
+//                            as those above would be 5-10 % slower
+//   d = 64                   48 x 17776 1393 / 1410 / 1429 / 1488, 13 x 2 x 6034 77.8 / 80.0 / 79.5 / 84.2, every 2nd 85
 #ifndef SPARSP_TUNE_POLY
-#define SPARSP_TUNE_POLY 3
+#define SPARSP_TUNE_POLY 4
 #endif
-// ... at d = 64 (measured there: every 3rd pair is 3 % faster than every 4th, every 2nd 4 % slower; at d = 128, with the
-// row sum on the tensor pipe, every 3rd is 1-2 % faster than every 4th and every 2nd 2 % slower)
+#ifndef SPARSP_TUNE_POLY_HOP
+#define SPARSP_TUNE_POLY_HOP 6
+#endif
 #ifndef SPARSP_TUNE_POLY_D64
 #define SPARSP_TUNE_POLY_D64 3
 #endif
+
+// Lists that the list builder keeps: the current item's and the next one's.  (With 3 or 4 a CTA takes items that one with
+// nothing left to do cannot take any more: 9 heads x 10602 tokens 60.8 us a call, 62.2 with 3, 63.2 with 4.)
+constexpr int kLists = 2;
+// One list entry: a KV block and which of the item's two query blocks keep it (64-token blocks); for a packed source the
+// tile index of a remote block in its place.  (A word, or half of one, for both of a tile's entries: with the block, the
+// valid keys per query block and the slot in three arrays 48 heads x 17776 took 2 % longer.)
+template <bool kPacked>
+struct Entry;
+template <>
+struct Entry<false> {
+  using type = uint16_t;
+  static constexpr int kFlagShift = 14;  // bits 14, 15: kept by the first, the second query block
+};
+template <>
+struct Entry<true> {
+  using type = uint32_t;
+  static constexpr int kFlagShift = 30;
+  static constexpr uint32_t kRemote = 1u << 29;  // bits 0-28 are the block's K tile in the packed buffer (its V tile is next)
+  static constexpr uint32_t kValue = kRemote - 1u;
+};
+// Item header, one load for each role: x = batch * H + head; y = entries | kHead... flags (0: there are no more items);
+// z = query blocks, first | second << 16 (0xffff: none); w = batch.
+constexpr int kHeadEntries = 0xffff, kHeadRagged = 1 << 16, kHeadRefShift = 17, kHeadNoneShift = 19;
 
 template <int D, int BLK>
 struct AttnCfg {
@@ -134,9 +171,11 @@ struct AttnCfg {
   static constexpr int kStagesV = (D == 64) ? 4 : 2;
   static constexpr int kQBytes = 128 * D * 2;
   static constexpr int kTileBytes = 128 * D * 2;  // one K or V tile
-  static constexpr int kOffQ = 0;
-  static constexpr int kOffK = kOffQ + kQBytes;
-  static constexpr int kOffV = kOffK + kStagesK * kTileBytes;
+  // Q tile and K ring share kStagesK + 1 buffers: an item's Q tile takes the next buffer of the ring for as long as the item
+  // lasts, the buffer of the item before it joins the ring behind (QKRing).
+  static constexpr int kBufsQK = kStagesK + 1;
+  static constexpr int kOffQK = 0;
+  static constexpr int kOffV = kOffQK + kBufsQK * kTileBytes;
   // d = 64 leaves room in tensor memory for 16 more accumulator columns: P V then runs with N = 80, its B
   // operand continuing, 64 columns on, into a constant [128 keys][column 64 = 1, the rest 0] block in shared
   // memory, so that accumulator column 64 is the row sum of P -- taken by the tensor pipe from the very
@@ -149,18 +188,17 @@ struct AttnCfg {
   static constexpr bool kSum128 = (D == 128);
   static constexpr int kNumP = kSum128 ? 1 : 2;
   static constexpr int kOffOnes = kOffV + kStagesV * kTileBytes;  // bf16 [128][64], 128-byte swizzle like a V box
-  static constexpr int kOffEntJ = kOffOnes + (kOnes ? 128 * 128 : 2048);  // uint16 [2][1024] kept / union list
-  static constexpr int kOffEntV = kOffEntJ + 2 * 2 * kMaxBlocks;  // uint8 [2][1024][2] keys of the entry valid for query block q (0 = not kept)
-  static constexpr int kOffSlot = kOffEntV + 2 * 2 * kMaxBlocks;  // int32 [2][1024] packed-buffer slot per entry
-  static constexpr int kOffRef = kOffSlot + 2 * 4 * kMaxBlocks;  // float [4 items][128] reference per row
+  static constexpr int kOffEnt = kOffOnes + (kOnes ? 128 * 128 : 2048);  // entries [kLists][1024]
+  static constexpr int kOffRef = kOffEnt + kLists * kMaxBlocks * 4;  // float [4 items][128] reference per row
   static constexpr int kOffBars = kOffRef + 4 * 128 * 4;
-  static constexpr int kNumBars = 2 + 2 * (kStagesK + kStagesV) + 10 + 1 + 4 + 4 + 8 + 1;
+  static constexpr int kNumBars = 2 * (kBufsQK + kStagesV) + 10 + 1 + 2 * kLists + 4 + 8 + 1;
   static constexpr int kColS = 0;    // S buffers: columns [0, 256)
   static constexpr int kColP = 256;  // P: two buffers in columns [256, 384), or one in [256, 320) with the row sums in [320, 336)
   static constexpr int kColO = 384;  // accumulator: columns [384, 384 + d)
   static constexpr int kColL = kOnes ? kColO + D : 320;  // row sums (column 0 of 16), where the tensor pipe takes them
-  static constexpr int kOffMisc = kOffBars + 8 * kNumBars;
-  static constexpr int kTotal = kOffMisc + 96;
+  static constexpr int kOffHead = (kOffBars + 8 * kNumBars + 15) / 16 * 16;  // int4 [kLists]
+  static constexpr int kOffMisc = kOffHead + 16 * kLists;
+  static constexpr int kTotal = kOffMisc + 64;
   static constexpr int kDynamic = kTotal + 1024;  // slack for the 1024-byte alignment of the base
   static_assert(kDynamic <= 232448, "shared memory budget");
 };
@@ -253,23 +291,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmP,
                     const AttnParams p) {
   using C = AttnCfg<D, BLK>;
-  constexpr int SK = C::kStagesK, SV = C::kStagesV;
+  constexpr int SV = C::kStagesV;
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
-  unsigned char* sQ = smem + C::kOffQ;
-  unsigned char* sK = smem + C::kOffK;
+  unsigned char* sQK = smem + C::kOffQK;
   unsigned char* sV = smem + C::kOffV;
-  uint16_t* sEntJ = reinterpret_cast<uint16_t*>(smem + C::kOffEntJ);  // [2][kMaxBlocks]
-  uint8_t* sEntV = smem + C::kOffEntV;                                // [2][kMaxBlocks][2]
-  int32_t* sSlot = reinterpret_cast<int32_t*>(smem + C::kOffSlot);    // [2][kMaxBlocks]
+  using E = Entry<kPacked>;
+  using EntT = typename E::type;
+  EntT* sEnt = reinterpret_cast<EntT*>(smem + C::kOffEnt);  // [kLists][kMaxBlocks]
   volatile float* sRef = reinterpret_cast<volatile float*>(smem + C::kOffRef);  // [4][128]
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kOffBars);
-  uint64_t* q_full = bars;          // the item's Q tile has landed
-  uint64_t* q_free = bars + 1;      // every Q K^T of the item has completed: Q may be overwritten
-  uint64_t* k_full = bars + 2;
-  uint64_t* k_empty = k_full + SK;
-  uint64_t* v_full = k_empty + SK;
+  uint64_t* qk_full = bars;                  // a Q or K tile has landed
+  uint64_t* qk_empty = qk_full + C::kBufsQK;  // ... and every Q K^T that reads it has completed
+  uint64_t* v_full = qk_empty + C::kBufsQK;
   uint64_t* v_empty = v_full + SV;
   uint64_t* s_full = v_empty + SV;  // [2] S buffer written by a Q K^T
   uint64_t* s_free = s_full + 2;    // [2] S buffer read into registers by its 4 softmax warps
@@ -278,28 +313,23 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // phase a barrier is in from the one before: a softmax thread that wants P V g-1 or g-2 has itself seen
   // P V g-4 complete, and P V g+2 cannot complete before that thread has stored P_g.
   uint64_t* o_full = p_full + 2;
-  uint64_t* o_drained = o_full + 4;      // the item's accumulator has been read out by all 8 softmax warps
-  uint64_t* list_ready = o_drained + 1;  // [2] list buffer filled
-  uint64_t* list_free = list_ready + 2;  // [2] list buffer no longer needed by its kListReaders
+  uint64_t* o_drained = o_full + 4;      // the item's accumulator has been read out by the four warps that write it
+  uint64_t* list_ready = o_drained + 1;  // [kLists] list buffer filled
+  uint64_t* list_free = list_ready + kLists;  // [kLists] list buffer no longer needed by its kListReaders
   // [4] the four warps that own an item's first tile have left what it says in s_exact and, if that is the reference, in
   // sRef.  Four, because the other warpgroup, which waits for it, may be up to three tiles and as many items behind.
-  uint64_t* ref_ready = list_free + 2;
+  uint64_t* ref_ready = list_free + kLists;
   // [2][4] the warpgroup's warp of a row group has decided about the running maximum of a tile.  (Not named barriers, which
   // cannot be bounded: after a wait that has run out two warps need not agree on who takes turns.  Every lane arrives: with
   // one lane behind a __syncwarp and the count of waits in shared memory 13 heads x 2 x 6034, Q times 8, took 138 us, not 132.)
   uint64_t* turn = ref_ready + 4;
   uint64_t* placed = turn + 8;     // in-place calls: the eight softmax warps know whether the item is to be computed again
+  int4* s_head = reinterpret_cast<int4*>(smem + C::kOffHead);  // [kLists] item headers
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
-  int* s_nent = reinterpret_cast<int*>(smem + C::kOffMisc + 8);   // [2]
-  int* s_blk = reinterpret_cast<int*>(smem + C::kOffMisc + 16);   // [2][2] the item's query block(s); < 0 = absent
-  int* s_item = reinterpret_cast<int*>(smem + C::kOffMisc + 32);  // [2] batch * H + head of each list buffer; < 0: none
-  int* s_rag = reinterpret_cast<int*>(smem + C::kOffMisc + 40);   // [2] the item's last tile reaches past the end of the sequence
-  int* s_ref = reinterpret_cast<int*>(smem + C::kOffMisc + 48);   // [2] where the rows' reference comes from
-  int* s_none = reinterpret_cast<int*>(smem + C::kOffMisc + 56);  // [2] bit q: query block q keeps nothing
-  volatile int* s_failed = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 64);  // [2] the item is to be computed again
   // [4 items][4 row groups] the group's rows take the running maximum
-  volatile uint8_t* s_exact = reinterpret_cast<volatile uint8_t*>(smem + C::kOffMisc + 80);
+  volatile uint8_t* s_exact = reinterpret_cast<volatile uint8_t*>(smem + C::kOffMisc + 16);
+  volatile int* s_failed = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 32);  // [kLists] the item is to be computed again
   constexpr int kListReaders = 12;  // two producers, two issuers, eight softmax warps
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -309,11 +339,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     prefetch_tmap(&tmQ);
     prefetch_tmap(&tmK);
     prefetch_tmap(&tmV);
-    mbar_init(q_full, 1);
-    mbar_init(q_free, 1);
-    for (int s = 0; s < SK; ++s) {
-      mbar_init(k_full + s, 1);
-      mbar_init(k_empty + s, 1);
+    for (int s = 0; s < C::kBufsQK; ++s) {
+      mbar_init(qk_full + s, 1);
+      mbar_init(qk_empty + s, 1);
     }
     for (int s = 0; s < SV; ++s) {
       mbar_init(v_full + s, 1);
@@ -323,11 +351,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       mbar_init(s_full + s, 1);
       mbar_init(s_free + s, 4);
       mbar_init(p_full + s, 4);
+    }
+    for (int s = 0; s < kLists; ++s) {
       mbar_init(list_ready + s, 1);
       mbar_init(list_free + s, kListReaders);
     }
     for (int s = 0; s < 4; ++s) mbar_init(o_full + s, 1);
-    mbar_init(o_drained, 8);
+    mbar_init(o_drained, 4);
     for (int s = 0; s < 4; ++s) mbar_init(ref_ready + s, 4);
     for (int s = 0; s < 8; ++s) mbar_init(turn + s, 32);
     mbar_init(placed, 8);
@@ -359,43 +389,46 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   // under which limit)
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SPARSP_REGS_UTILITY));
+    // K (of_v = 0) or V tile n of an item's list; an absent second half re-reads the last entry
+    auto load_kv = [&](const CUtensorMap* tm, uint64_t* bar, unsigned char* dst, const EntT* ent, int n, int n_ent, int head,
+                       int batch, int of_v) {
+#pragma unroll
+      for (int e = 0; e < C::kEPT; ++e) {
+        const uint32_t v = ent[min(n * C::kEPT + e, n_ent - 1)];
+        bool remote = false;
+        if constexpr (kPacked) {
+          remote = (v & E::kRemote) != 0u;
+          if (remote) {
+            // a remote block's K tile and V tile are consecutive tiles of the consumer's packed buffer
+#pragma unroll
+            for (int c = 0; c < D / 64; ++c)
+              tma_load_4d(dst + c * 16384 + e * (BLK * 128), &tmP, bar, c * 64, 0, (int)(v & E::kValue) + of_v, 0);
+          }
+        }
+        if (!remote) {
+          const int tok = (int)(v & (kMaxBlocks - 1)) * BLK;
+#pragma unroll
+          for (int c = 0; c < D / 64; ++c) tma_load_4d(dst + c * 16384 + e * (BLK * 128), tm, bar, c * 64, tok, head, batch);
+        }
+      }
+    };
     if (warp == 3) {
       // ================================ TMA producer: V =====================================
       if (lane == 0) {
         int vn = 0;  // V tiles loaded so far
         for (int i = 0;; ++i) {
-          const int buf = i & 1;
-          mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 58, p.wait_limit);
-          const int bh = s_item[buf];
-          if (bh < 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
-          const int n_ent = s_nent[buf];
-          const int n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
-          {
-            const int batch = bh / p.H, head = bh % p.H;
-            const uint16_t* entJ = sEntJ + buf * kMaxBlocks;
-            const int32_t* entS = sSlot + buf * kMaxBlocks;
-            const int tile_base = kPacked ? (int)p.tile_base[batch] : 0;
-            for (int n = 0; n < n_tiles; ++n, ++vn) {
-              const int st = vn % SV;
-              mbar_wait_bounded_inline(v_empty + st, ((vn / SV) & 1) ^ 1, s_abort, 59, p.wait_limit);
-              unsigned char* dst = sV + st * C::kTileBytes;
-              mbar_expect_tx(v_full + st, C::kTileBytes);
-  #pragma unroll
-              for (int e = 0; e < C::kEPT; ++e) {
-                const int ent = min(n * C::kEPT + e, n_ent - 1);
-                const int slot = kPacked ? entS[ent] : -1;
-                if (slot < 0) {
-                  const int tok = (int)entJ[ent] * BLK;
-  #pragma unroll
-                  for (int c = 0; c < D / 64; ++c)
-                    tma_load_4d(dst + c * 16384 + e * (BLK * 128), &tmV, v_full + st, c * 64, tok, head, batch);
-                } else {
-  #pragma unroll
-                  for (int c = 0; c < D / 64; ++c)
-                    tma_load_4d(dst + c * 16384 + e * (BLK * 128), &tmP, v_full + st, c * 64, 0, tile_base + 2 * slot + 1, 0);
-                }
-              }
-            }
+          const int buf = i % kLists;
+          mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 58, p.wait_limit);
+          const int4 hd = s_head[buf];
+          if (hd.y == 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
+          const int n_ent = hd.y & kHeadEntries, n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
+          const int batch = hd.w, head = hd.x - batch * p.H;
+          const EntT* ent = sEnt + buf * kMaxBlocks;
+          for (int n = 0; n < n_tiles; ++n, ++vn) {
+            const int st = vn % SV;
+            mbar_wait_bounded_inline(v_empty + st, ((vn / SV) & 1) ^ 1, s_abort, 59, p.wait_limit);
+            mbar_expect_tx(v_full + st, C::kTileBytes);
+            load_kv(&tmV, v_full + st, sV + st * C::kTileBytes, ent, n, n_ent, head, batch, 1);
           }
           mbar_arrive(list_free + buf);
         }
@@ -403,58 +436,35 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     } else if (warp == 0) {
       // ================================ TMA producer: Q and K ===============================
       if (lane == 0) {
-        int kn = 0, qc = 0;  // K tiles loaded so far; items so far
+        QKRing<C::kStagesK> at;
         for (int i = 0;; ++i) {
-          const int buf = i & 1;
-          mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 51, p.wait_limit);
-          const int bh = s_item[buf];
-          if (bh < 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
-          const int n_ent = s_nent[buf];
-          const int n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
+          const int buf = i % kLists;
+          mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 51, p.wait_limit);
+          const int4 hd = s_head[buf];
+          if (hd.y == 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
+          const int n_ent = hd.y & kHeadEntries, n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
+          const int batch = hd.w, head = hd.x - batch * p.H;
+          const EntT* ent = sEnt + buf * kMaxBlocks;
           {
-            const int batch = bh / p.H, head = bh % p.H;
-            const uint16_t* entJ = sEntJ + buf * kMaxBlocks;
-            const int32_t* entS = sSlot + buf * kMaxBlocks;
-            const int tile_base = kPacked ? (int)p.tile_base[batch] : 0;
-            for (int n = 0; n < n_tiles; ++n, ++kn) {
-              const int st = kn % SK;
-              mbar_wait_bounded_inline(k_empty + st, ((kn / SK) & 1) ^ 1, s_abort, 57, p.wait_limit);
-              unsigned char* dst = sK + st * C::kTileBytes;
-              mbar_expect_tx(k_full + st, C::kTileBytes);
+            // a Q tile is 128 rows: one 128-token block, or two 64-token blocks stacked (an absent second
+            // block re-reads the first: finite data whose rows are never used)
+            const uint32_t b = at.next_q();
+            mbar_wait_bounded_inline(qk_empty + b, at.use(b) ^ 1u, s_abort, 52, p.wait_limit);
+            mbar_expect_tx(qk_full + b, C::kTileBytes);
 #pragma unroll
-              for (int e = 0; e < C::kEPT; ++e) {
-                const int ent = min(n * C::kEPT + e, n_ent - 1);  // an absent second half re-reads the last entry
-                const int slot = kPacked ? entS[ent] : -1;
-                if (slot < 0) {
-                  const int tok = (int)entJ[ent] * BLK;
+            for (int q = 0; q < C::kEPT; ++q) {
+              const int b1 = (int)((uint32_t)hd.z >> 16), bq = q && b1 != 0xffff ? b1 : hd.z & 0xffff;
 #pragma unroll
-                  for (int c = 0; c < D / 64; ++c)
-                    tma_load_4d(dst + c * 16384 + e * (BLK * 128), &tmK, k_full + st, c * 64, tok, head, batch);
-                } else {
-                  // remote block: its K tile and V tile are consecutive tiles of the consumer's packed buffer
-#pragma unroll
-                  for (int c = 0; c < D / 64; ++c)
-                    tma_load_4d(dst + c * 16384 + e * (BLK * 128), &tmP, k_full + st, c * 64, 0, tile_base + 2 * slot, 0);
-                }
-              }
-              if (n == 0) {
-                // the item's first K tile is on its way; now the Q tile, which may be overwritten once every
-                // Q K^T of the previous item has completed
-                if (qc > 0) mbar_wait_bounded_inline(q_free, (qc - 1) & 1, s_abort, 52, p.wait_limit);
-                ++qc;
-                mbar_expect_tx(q_full, C::kQBytes);
-                // a Q tile is 128 rows: one 128-token block, or two 64-token blocks stacked (an absent second
-                // block re-reads the first: finite data whose rows are never used)
-#pragma unroll
-                for (int q = 0; q < C::kEPT; ++q) {
-                  const int bq = s_blk[buf * 2 + q] >= 0 ? s_blk[buf * 2 + q] : s_blk[buf * 2];
-                  const int tok = max(bq, 0) * BLK;
-#pragma unroll
-                  for (int c = 0; c < D / 64; ++c)
-                    tma_load_4d(sQ + c * 16384 + q * (BLK * 128), &tmQ, q_full, c * 64, tok, head, batch);
-                }
-              }
+              for (int c = 0; c < D / 64; ++c)
+                tma_load_4d(sQK + b * C::kTileBytes + c * 16384 + q * (BLK * 128), &tmQ, qk_full + b, c * 64, bq * BLK, head,
+                            batch);
             }
+          }
+          for (int n = 0; n < n_tiles; ++n) {
+            const uint32_t b = at.next_k();
+            mbar_wait_bounded_inline(qk_empty + b, at.use(b) ^ 1u, s_abort, 57, p.wait_limit);
+            mbar_expect_tx(qk_full + b, C::kTileBytes);
+            load_kv(&tmK, qk_full + b, sQK + b * C::kTileBytes, ent, n, n_ent, head, batch, 0);
           }
           mbar_arrive(list_free + buf);
         }
@@ -464,41 +474,39 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       // The whole warp runs the loop (uniform control flow and operands); one elected lane issues.
       const bool leader = elect_one();
       constexpr uint32_t kIdescQK = make_idesc_bf16(128, 128, 0, 0);
-      const uint64_t descQ = make_smem_desc(smem_u32(sQ), 16, 1024);
-      const uint64_t descK = make_smem_desc(smem_u32(sK), 16, 1024);
-      const uint32_t hiQK = (uint32_t)(descK >> 32);
-      uint32_t qlo[D / 16], klo[D / 16];
+      const uint64_t desc0 = make_smem_desc(smem_u32(sQK), 16, 1024);
+      const uint32_t hi = (uint32_t)(desc0 >> 32);
+      uint32_t lo[D / 16];
 #pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) {
-        const uint32_t off = (uint32_t)(((kk / 4) * 16384 + (kk % 4) * 32) >> 4);
-        qlo[kk] = (uint32_t)descQ + off;
-        klo[kk] = (uint32_t)descK + off;
-      }
-      int g = 0, qc = 0;
+      for (int kk = 0; kk < D / 16; ++kk) lo[kk] = (uint32_t)desc0 + (uint32_t)(((kk / 4) * 16384 + (kk % 4) * 32) >> 4);
+      QKRing<C::kStagesK> at;
+      int g = 0;
       for (int i = 0;; ++i) {
-        const int buf = i & 1;
-        mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 53, p.wait_limit);
-        if (s_item[buf] < 0) break;
-        const int n_tiles = (s_nent[buf] + C::kEPT - 1) / C::kEPT;
-        {
-          mbar_wait_bounded_inline(q_full, qc++ & 1, s_abort, 11, p.wait_limit);
-          for (int n = 0; n < n_tiles; ++n, ++g) {
-            mbar_wait_bounded_inline(k_full + g % SK, (g / SK) & 1, s_abort, 12, p.wait_limit);
-            // S buffer g%2 is free once the softmax warps have loaded the scores of tile g-2
-            if (g >= 2) mbar_wait_bounded_inline(s_free + (g & 1), ((g - 2) >> 1) & 1, s_abort, 24, p.wait_limit);
-            tc_fence_after();
-            const uint32_t stage_off = (uint32_t)(((g % SK) * C::kTileBytes) >> 4);
-            const uint32_t tS = tmem_base + C::kColS + (g & 1) * 128;
-            if (leader) {
+        const int buf = i % kLists;
+        mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 53, p.wait_limit);
+        const int y = s_head[buf].y;
+        if (y == 0) break;
+        const int n_tiles = ((y & kHeadEntries) + C::kEPT - 1) / C::kEPT;
+        const uint32_t bq = at.next_q();
+        mbar_wait_bounded_inline(qk_full + bq, at.use(bq), s_abort, 11, p.wait_limit);
+        const uint32_t q_off = bq * (C::kTileBytes >> 4);
+        for (int n = 0; n < n_tiles; ++n, ++g) {
+          const uint32_t bk = at.next_k();
+          mbar_wait_bounded_inline(qk_full + bk, at.use(bk), s_abort, 12, p.wait_limit);
+          // S buffer g%2 is free once the softmax warps have loaded the scores of tile g-2
+          if (g >= 2) mbar_wait_bounded_inline(s_free + (g & 1), ((g - 2) >> 1) & 1, s_abort, 24, p.wait_limit);
+          tc_fence_after();
+          const uint32_t k_off = bk * (C::kTileBytes >> 4);
+          const uint32_t tS = tmem_base + C::kColS + (g & 1) * 128;
+          if (leader) {
 #pragma unroll
-              for (int kk = 0; kk < D / 16; ++kk)
-                mma_ss_lohi(tS, qlo[kk], hiQK, klo[kk] + stage_off, hiQK, kIdescQK, kk > 0 ? 1u : 0u);
-              mma_commit(s_full + (g & 1));
-              mma_commit(k_empty + g % SK);
-              if (n == n_tiles - 1) mma_commit(q_free);
-            }
-            __syncwarp();
+            for (int kk = 0; kk < D / 16; ++kk)
+              mma_ss_lohi(tS, lo[kk] + q_off, hi, lo[kk] + k_off, hi, kIdescQK, kk > 0 ? 1u : 0u);
+            mma_commit(s_full + (g & 1));
+            mma_commit(qk_empty + bk);
+            if (n == n_tiles - 1) mma_commit(qk_empty + bq);
           }
+          __syncwarp();
         }
         if (lane == 0) mbar_arrive(list_free + buf);
         __syncwarp();
@@ -520,10 +528,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       const uint32_t tL = tmem_base + C::kColL;
       int g = 0;
       for (int i = 0;; ++i) {
-        const int buf = i & 1;
-        mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 54, p.wait_limit);
-        if (s_item[buf] < 0) break;
-        const int n_tiles = (s_nent[buf] + C::kEPT - 1) / C::kEPT;
+        const int buf = i % kLists;
+        mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 54, p.wait_limit);
+        const int y = s_head[buf].y;
+        if (y == 0) break;
+        const int n_tiles = ((y & kHeadEntries) + C::kEPT - 1) / C::kEPT;
         // the previous item's accumulator must have been read out before this item's first P V overwrites it
         if (i > 0) mbar_wait_bounded_inline(o_drained, (i - 1) & 1, s_abort, 55, p.wait_limit);
         for (int n = 0; n < n_tiles; ++n, ++g) {
@@ -575,6 +584,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       if (kPacked) load_heads();
       const bool stacked = C::kStacked && (kPacked || !p.single);
       int bh = p.BH, blk0 = -1, blk1 = -1;
+      const int ragged_block = p.N % BLK ? p.NB - 1 : -1;
       uint32_t rb0 = 0u, rb1 = 0u;  // the item's mask rows, a word per lane (NB <= 1024: at most 32 words)
       // Takes an item: its head (BH = no more items), query block(s) and mask rows.
       auto load_rows = [&]() {
@@ -618,46 +628,41 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (lane == 0) it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
         return __shfl_sync(0xffffffffu, it, 0);
       };
-      // When the next item is taken: for stacked items of a packed source with d = 128, whose lists are short and slow
-      // to build, right after the list before it, while its buffer is still in use (24 heads x 24576, 4 ranks: one call
-      // 434 us against 483, with a shuffled placement 421 against 462, hop by hop 796 against 811; 12 heads x 9504:
-      // 64.5 against 66.4).  Everywhere else once there is a buffer for it: an item taken early is one that a CTA with
-      // nothing left to do cannot take (packed source, d = 64, 24 heads x 24576: one call 339 us against 345-358 early, hop by
-      // hop 641 against 654; 48 heads x 17776, 8 ranks: 265 against 271-280; K / V source, 26 heads x 6034 and 40 heads
-      // x 75600 hop by hop: 3 % slower early).
-      constexpr bool kEarly = kPacked && C::kStacked && D == 128;
-      if (kEarly) fetch(blockIdx.x);
+      // An item that has failed is handed out again.  Its verdict is there once its list buffer is free: before the buffer is
+      // used again, or, when there are no more items, one outstanding item after the other.
+      int checked = 0;  // items whose verdict has been seen
+      auto verdict = [&]() -> int {
+        const int b = checked % kLists;
+        mbar_wait_bounded_inline(list_free + b, (checked / kLists) & 1, s_abort, 50, p.wait_limit);
+        ++checked;
+        return s_failed[b] ? b : -1;
+      };
       for (int i = 0;; ++i) {
-        const int buf = i & 1;
+        const int buf = i % kLists;
         int again = -1;  // list buffer of an item that is computed again now (rare)
-        if (i >= 2) {
-          mbar_wait_bounded_inline(list_free + buf, ((i - 2) >> 1) & 1, s_abort, 50, p.wait_limit);
-          if (s_failed[buf]) again = buf;
-        }
-        if (again < 0 && !kEarly) fetch(i == 0 ? (int)blockIdx.x : next_item());
-        if (again < 0 && bh >= p.BH && i >= 1) {  // no more items: what became of the last one?
-          mbar_wait_bounded_inline(list_free + (buf ^ 1), ((i - 1) >> 1) & 1, s_abort, 60, p.wait_limit);
-          if (s_failed[buf ^ 1]) again = buf ^ 1;
-        }
+        if (checked <= i - kLists) again = verdict();
+        if (again < 0) fetch(i == 0 ? (int)blockIdx.x : next_item());
+        while (again < 0 && bh >= p.BH && checked < i) again = verdict();
         if (__any_sync(0xffffffffu, *s_abort != 0) || (again < 0 && bh >= p.BH)) {
           if (lane == 0) {
-            s_item[buf] = -1;
+            s_head[buf].y = 0;
             mbar_arrive(list_ready + buf);
           }
           break;
         }
-        const int next_bh = bh, next_blk0 = blk0, next_blk1 = blk1;
+        const int next_bh = bh;
         if (again >= 0) {
-          bh = s_item[again];
-          blk0 = s_blk[again * 2];
-          blk1 = s_blk[again * 2 + 1];
+          bh = s_head[again].x;
+          const int z = s_head[again].z;
+          blk0 = z & 0xffff;
+          blk1 = (int)((uint32_t)z >> 16) == 0xffff ? -1 : (int)((uint32_t)z >> 16);
           load_rows();
           __syncwarp();  // (every lane has looked)
           if (lane == 0) s_failed[again] = 0;
         }
-        uint16_t* entJ = sEntJ + buf * kMaxBlocks;
-        uint8_t* entV = sEntV + buf * kMaxBlocks * 2;
-        int32_t* entS = sSlot + buf * kMaxBlocks;
+        EntT* ent = sEnt + buf * kMaxBlocks;
+        const int batch = bh / p.H;
+        const int tile_base = kPacked ? (int)p.tile_base[batch] : 0;
         // Entry order (any order gives the same attention).  Blocks BOTH query blocks keep make full tiles; a
         // block only the first keeps is put next to a block only the second keeps, so that such a tile costs
         // every softmax row one 64-key half instead of costing half of the rows two.  A full tile is bound by
@@ -687,13 +692,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
               rb1 &= ~(1u << (j & 31));
             }
             own_of |= (int)f;
-            const int nvalid = (int)min((int64_t)BLK, p.N - (int64_t)j * BLK);
-            if (lane == 0) {
-              entJ[lead] = (uint16_t)j;
-              entV[lead * 2] = (uint8_t)(f & 1u ? nvalid : 0);
-              entV[lead * 2 + 1] = (uint8_t)(f & 2u ? nvalid : 0);
-            }
-            if (nvalid < BLK) rag_pos = lead;
+            if (lane == 0) ent[lead] = (EntT)((uint32_t)j | f << E::kFlagShift);
+            if (j == ragged_block) rag_pos = lead;
             ++lead;
           }
         }
@@ -717,7 +717,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           const uint32_t w0 = __shfl_sync(0xffffffffu, rb0, w);
           const uint32_t w1 = C::kStacked ? __shfl_sync(0xffffffffu, rb1, w) : 0u;
           const int jb = w * 32 + lane;
-          const int nvalid = (int)min((int64_t)BLK, p.N - (int64_t)jb * BLK);
           if (C::kStacked) {
             const uint32_t both = w0 & w1, only0 = w0 & ~w1, only1 = w1 & ~w0;
             const bool in0 = (w0 >> lane) & 1u, in1 = (w1 >> lane) & 1u;
@@ -733,10 +732,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                 else pos = n_both + n_mix + idx;  // tail of the longer class
               }
               pos += lead;
-              entJ[pos] = (uint16_t)jb;
-              // keys valid for the first query block's rows, for the second's
-              *reinterpret_cast<uint16_t*>(entV + pos * 2) = (uint16_t)((in0 ? nvalid : 0) | (in1 ? nvalid << 8 : 0));
-              if (nvalid < BLK) rag_pos = pos;
+              ent[pos] = (EntT)((uint32_t)jb | ((in0 ? 1u : 0u) | (in1 ? 2u : 0u)) << E::kFlagShift);
+              if (jb == ragged_block) rag_pos = pos;
             }
             at0 += __popc(both);
             at1 += __popc(only0);
@@ -744,9 +741,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           } else {
             if ((w0 >> lane) & 1u) {
               const int pos = lead + at0 + __popc(w0 & below);
-              entJ[pos] = (uint16_t)jb;
-              entV[pos * 2] = (uint8_t)nvalid;
-              if (nvalid < BLK) rag_pos = pos;
+              ent[pos] = (EntT)((uint32_t)jb | 1u << E::kFlagShift);
+              if (jb == ragged_block) rag_pos = pos;
             }
             at0 += __popc(w0);
           }
@@ -758,46 +754,37 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (rag_pos >= 0) {
           if (lane == 0) {
             const int e = running - 1;
-            const uint16_t tj = entJ[rag_pos]; entJ[rag_pos] = entJ[e]; entJ[e] = tj;
-            for (int q = 0; q < 2; ++q) {
-              const uint8_t tv = entV[rag_pos * 2 + q];
-              entV[rag_pos * 2 + q] = entV[e * 2 + q];
-              entV[e * 2 + q] = tv;
-            }
+            const EntT t = ent[rag_pos];
+            ent[rag_pos] = ent[e];
+            ent[e] = t;
           }
           __syncwarp();
         }
-        if (kPacked) {  // where the entries' blocks are, a lane per entry, two loads in flight
+        if (C::kStacked && (running & 1) && lane == 0) ent[running] = 0;
+        if constexpr (kPacked) {  // where the entries' blocks are, a lane per entry, two loads in flight
+          const int32_t* slot = p.slot + (int64_t)bh * p.NB;
+          auto placed_at = [&](uint32_t v, int32_t sl) {
+            return sl < 0 ? v : (v & ~E::kValue) | E::kRemote | ((uint32_t)(tile_base + 2 * sl) & E::kValue);
+          };
           for (int e = lane; e < running; e += 64) {
-            const int e2 = e + 32 < running ? e + 32 : e;
-            const int32_t s1 = p.slot[(int64_t)bh * p.NB + entJ[e]], s2 = p.slot[(int64_t)bh * p.NB + entJ[e2]];
-            entS[e] = s1;
-            entS[e2] = s2;
+            const bool two = e + 32 < running;
+            const uint32_t v1 = ent[e], v2 = two ? ent[e + 32] : v1;
+            const int32_t s1 = slot[v1 & (kMaxBlocks - 1)], s2 = slot[v2 & (kMaxBlocks - 1)];
+            ent[e] = placed_at(v1, s1);
+            if (two) ent[e + 32] = placed_at(v2, s2);
           }
           __syncwarp();
         }
         int ref_of = kPacked || running <= (kZeroMinTiles - 1) * C::kEPT ? kRefFirst : kRefZero;
         if (again >= 0) ref_of = kRefExact;
         if (lane == 0) {
-          s_item[buf] = bh;
-          s_rag[buf] = rag_pos >= 0 ? 1 : 0;
-          s_nent[buf] = running;
-          s_ref[buf] = ref_of;
-          s_none[buf] = none;
-          s_blk[buf * 2] = blk0;
-          s_blk[buf * 2 + 1] = blk1;
+          s_head[buf] = make_int4(bh, running | (rag_pos >= 0 ? kHeadRagged : 0) | ref_of << kHeadRefShift | none << kHeadNoneShift,
+                                  blk0 | (blk1 < 0 ? 0xffff : blk1) << 16, batch);
           s_failed[buf] = 0;
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(list_ready + buf);
-        if (again >= 0) {  // back to the item that was at hand, if there was one
-          bh = next_bh;
-          blk0 = next_blk0;
-          blk1 = next_blk1;
-          if (kEarly && bh < p.BH) load_rows();
-        } else if (kEarly) {
-          fetch(next_item());
-        }
+        if (again >= 0) bh = next_bh;  // (>= BH where there are no more items)
       }
     } else {
       // ============== rows of query blocks that keep nothing, which are no work items ==============
@@ -838,16 +825,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     int g0 = 0;       // number of the item's first tile
     int turns = 0;    // waits for the other warp of the row group so far
     for (int i = 0;; ++i) {
-      const int buf = i & 1;
-      mbar_wait_bounded_inline(list_ready + buf, (i >> 1) & 1, s_abort, 56, p.wait_limit);
-      const int bh = s_item[buf];
-      if (bh < 0) break;
-      const int n_ent = s_nent[buf];
+      const int buf = i % kLists;
+      mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 56, p.wait_limit);
+      const int4 hd = s_head[buf];
+      if (hd.y == 0) break;
+      const int n_ent = hd.y & kHeadEntries;
       const int n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
       const int first = (wg - g0) & 1;  // my first tile
-      const int ref_of = s_ref[buf];
-      const uint8_t* entV = sEntV + buf * kMaxBlocks * 2 + (C::kStacked ? rh : 0);  // my query block's column
-      const bool item_ragged = s_rag[buf] != 0;
+      const int ref_of = (hd.y >> kHeadRefShift) & 3;
+      const EntT* ent = sEnt + buf * kMaxBlocks;
+      const bool item_ragged = (hd.y & kHeadRagged) != 0;
       volatile float* ref = sRef + (i & 3) * 128;
       float m_ref = ref_of == kRefZero ? 0.0f : -INFINITY;  // the row's reference as this thread last saw it
       float i_max = 0.0f;  // largest binary exponent that was taken on the FMA pipe, in magnitude
@@ -917,12 +904,29 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         // kept / valid key columns of each 64-column half of the tile (warp-uniform), as the list builder left them
         int vh[2];
         if (C::kStacked) {
-          vh[0] = entV[(n * 2) * 2];
-          vh[1] = n * 2 + 1 < n_ent ? entV[(n * 2 + 1) * 2] : 0;
+          // both entries at once; an odd list ends with one that nobody keeps
+          if constexpr (kPacked) {
+            const uint2 v = reinterpret_cast<const uint2*>(ent)[n];
+            vh[0] = (v.x >> (E::kFlagShift + rh)) & 1u ? 64 : 0;
+            vh[1] = (v.y >> (E::kFlagShift + rh)) & 1u ? 64 : 0;
+          } else {
+            const uint32_t v = reinterpret_cast<const uint32_t*>(ent)[n] >> (E::kFlagShift + rh);
+            vh[0] = v & 1u ? 64 : 0;
+            vh[1] = v & 0x10000u ? 64 : 0;
+          }
         } else {
-          const int nv = entV[n * 2];
-          vh[0] = min(nv, 64);
-          vh[1] = max(nv - 64, 0);
+          vh[0] = vh[1] = 64;
+        }
+        if (kRagged && item_ragged && n == n_tiles - 1) {
+          // the list's last entry is the block in which the sequence ends
+          const int valid = (int)(p.N - (int64_t)(p.NB - 1) * BLK);
+          if (C::kStacked) {
+            if (n_ent & 1) vh[0] = min(vh[0], valid);
+            else vh[1] = min(vh[1], valid);
+          } else {
+            vh[0] = min(valid, 64);
+            vh[1] = max(valid - 64, 0);
+          }
         }
         mbar_wait_bounded_inline(s_full + wg, (g >> 1) & 1, s_abort, 30 + wg, p.wait_limit);
         tc_fence_after();
@@ -1003,7 +1007,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
               const float2 x = ffma2(make_float2(svh[2 * e], svh[2 * e + 1]), sc2, nm2);
-              constexpr int kPoly = C::kOnes ? SPARSP_TUNE_POLY_D64 : SPARSP_TUNE_POLY;
+              constexpr int kPoly = D == 64 ? SPARSP_TUNE_POLY_D64 : kPacked && BLK == 128 ? SPARSP_TUNE_POLY_HOP : SPARSP_TUNE_POLY;
               const float2 pp = (kPoly > 0 && (e % (kPoly > 0 ? kPoly : 1)) == 1)
                                     ? exp2_poly2<kRagged || kExact, !kExact>(x, &i_max)
                                     : make_float2(ex2(x.x), ex2(x.y));
@@ -1049,60 +1053,66 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         for (; n < n_tiles; n += 2) do_tile(std::true_type{}, std::true_type{}, n);
 
       g0 += n_tiles;
-      // ---- item epilogue: warpgroup x writes the column half x of every row -------------------------
+      // ---- item epilogue: the warpgroup of the item's last tile writes the rows, the other one goes on ----
       if (first >= n_tiles && ref_of != kRefExact) learn_ref();
-      if (exact && ((n_tiles - 1 - first) & 1)) take_turn();  // (the last tile was the other warp's)
       const int last = g0 - 1;
-      mbar_wait_bounded_inline(o_full + (last & 3), (last >> 2) & 1, s_abort, 40, p.wait_limit);
-      tc_fence_after();
-      {
-        constexpr int HW = D / 2;
-        const int qb = C::kStacked ? s_blk[buf * 2 + rh] : s_blk[buf * 2];
+      if ((last & 1) != wg) {
+        if (exact) take_turn();  // (the last tile was the other warp's)
+        if (__any_sync(0xffffffffu, !exact && !(i_max <= kMaxExponent)) && lane == 0) s_failed[buf] = 1;
+        __syncwarp();
+        if (p.in_place) {
+          if (lane == 0) mbar_arrive(placed);
+          mbar_wait_bounded_inline(placed, i & 1, s_abort, 45, p.wait_limit);
+        }
+        if (lane == 0) mbar_arrive(list_free + buf);
+      } else {
+        const int qb = C::kStacked && rh ? (int)((uint32_t)hd.z >> 16) : hd.z & 0xffff;
         // (a block that keeps nothing is stacked with one that does: other warps write its rows)
-        const bool none = qb < 0 || ((s_none[buf] >> (C::kStacked ? rh : 0)) & 1);
+        const bool none = qb == 0xffff || ((hd.y >> (kHeadNoneShift + (C::kStacked ? rh : 0))) & 1);
         int64_t tok = none ? p.N : (int64_t)qb * BLK + (C::kStacked ? (row & 63) : row);
-        const int batch = bh / p.H, head = bh % p.H;
-        __nv_bfloat16* orow = p.O + (int64_t)batch * p.sB + (int64_t)head * p.sH + tok * p.sT + wg * HW;
-        uint32_t sum, o[HW];
+        __nv_bfloat16* orow = p.O + (int64_t)hd.w * p.sB + (int64_t)(hd.x - hd.w * p.H) * p.sH + tok * p.sT;
+        float* lrow = p.lse ? p.lse + (int64_t)hd.x * p.N + tok : nullptr;
+        // a thread's row is 2 D contiguous bytes but the rows of a warp are sT elements apart, so every
+        // store instruction touches 32 lines: 32-byte stores (when the layout allows) halve their number
+        int wide = ((reinterpret_cast<uintptr_t>(orow) | (uintptr_t)(p.sT * 2)) & 31) == 0, mine_to_write = tok < p.N;
+        // (worked out while the last P V runs, not behind it)
+        asm volatile("" : "+l"(orow), "+l"(lrow), "+r"(wide), "+r"(mine_to_write));
+        mbar_wait_bounded_inline(o_full + (last & 3), (last >> 2) & 1, s_abort, 40, p.wait_limit);
+        tc_fence_after();
+        uint32_t sum, o[D];
         tmem_ld1(tmem_base + C::kColL + lane_off, &sum);
 #pragma unroll
-        for (int c = 0; c < HW / 32; ++c) tmem_ld32(tO + wg * HW + c * 32, o + c * 32);
+        for (int c = 0; c < D / 32; ++c) tmem_ld32(tO + c * 32, o + c * 32);
         tmem_ld_wait();
+        // the accumulator is in registers: the next item's first P V may overwrite it
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(o_drained);
         const float l = __uint_as_float(sum);  // the row sum is a tensor-memory column
         // (an ordinary item asks one question here)
         const float safe = ref_of == kRefZero ? kSafeSumZero : kSafeSumFirst;
-        const bool asks = !exact && tok < p.N && !(i_max <= kMaxExponent && l >= kMinSum && l <= safe);
-        const bool slow = __any_sync(0xffffffffu, asks) || p.in_place;
-        if (slow) {
+        const bool asks = !exact && mine_to_write && !(i_max <= kMaxExponent && l >= kMinSum && l <= safe);
+        if (__any_sync(0xffffffffu, asks) || p.in_place) {
           bool failed = asks && !(i_max <= kMaxExponent && l >= kMinSum && l <= kMaxSum);
           if (asks) {
             float most = 0.0f;  // has a column run out of fp32?
 #pragma unroll
-            for (int e = 0; e < HW; e += 2) most = max_abs3(__uint_as_float(o[e]), __uint_as_float(o[e + 1]), most);
+            for (int e = 0; e < D; e += 2) most = max_abs3(__uint_as_float(o[e]), __uint_as_float(o[e + 1]), most);
             failed = failed || !(most < INFINITY);
           }
           if (__any_sync(0xffffffffu, failed) && lane == 0) s_failed[buf] = 1;
+          __syncwarp();
           if (p.in_place) {  // the rows of an item that is computed again are still its queries
-            __syncwarp();
             if (lane == 0) mbar_arrive(placed);
             mbar_wait_bounded_inline(placed, i & 1, s_abort, 45, p.wait_limit);
-            if (s_failed[buf]) tok = p.N;
+            if (s_failed[buf]) mine_to_write = 0;
           }
         }
-        // the accumulator is in registers: the next item's first P V may overwrite it
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(o_drained);
-          mbar_arrive(list_free + buf);
-        }
+        if (lane == 0) mbar_arrive(list_free + buf);
         const float inv_l = l > 0.0f ? 1.0f / l : 0.0f;
-        if (tok < p.N) {
-          // a thread's row segment is 2 HW contiguous bytes but the rows of a warp are sT elements apart, so every
-          // store instruction touches 32 lines: 32-byte stores (when the layout allows) halve their number
-          const bool wide = ((reinterpret_cast<uintptr_t>(orow) | (uintptr_t)(p.sT * 2)) & 31) == 0;
+        if (mine_to_write) {
 #pragma unroll
-          for (int v = 0; v < HW / 16; ++v) {
+          for (int v = 0; v < D / 16; ++v) {
             uint32_t w[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -1120,8 +1130,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             }
           }
         }
-        if (p.lse && wg == 0 && tok < p.N)  // (a score that is no number makes the row's sum none, or infinite)
-          p.lse[(int64_t)bh * p.N + tok] = !(l < INFINITY) ? NAN : l > 0.0f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
+        if (lrow && mine_to_write)  // (a score that is no number makes the row's sum none, or infinite)
+          *lrow = !(l < INFINITY) ? NAN : l > 0.0f ? (m_ref + log2f(l)) * 0.6931471805599453f : -INFINITY;
       }
     }
   }

@@ -1,5 +1,5 @@
-// Which work item a number of the attention kernel's queue stands for (K / V source).  Plain integer code, apart from
-// the kernel so that it can be run on a host as well.
+// Which work item a number of the attention kernel's queue stands for (K / V source), and which buffer a tile of an item
+// lies in.  Plain integer code, apart from the kernel so that it can be run on a host as well.
 #pragma once
 
 #include <stdint.h>
@@ -28,5 +28,30 @@ SPARSP_QUEUE_FN int find_item(int it, int per_head, int n_heads, const int32_t* 
   }
   return head;
 }
+
+// Which of the kRing + 1 shared buffers the next Q or K tile lies in, and the parity of its use: the producer and the Q K^T
+// issuer both follow the same sequence of tiles.  A nibble per buffer, the next one lowest.
+template <int kRing>
+struct QKRing {
+  uint32_t ring = kRing == 4 ? 0x3210u : 0x210u;
+  uint32_t q = kRing;     // the item's Q tile (before the first item: the buffer that is not in the ring)
+  uint32_t uses = 0u;     // bit b: parity of the uses of buffer b so far
+  SPARSP_QUEUE_FN uint32_t use(uint32_t b) {  // parity of this use
+    const uint32_t par = (uses >> b) & 1u;
+    uses ^= 1u << b;
+    return par;
+  }
+  SPARSP_QUEUE_FN uint32_t next_q() {
+    const uint32_t b = ring & 15u;
+    ring = (ring >> 4) | q << (4 * (kRing - 1));
+    q = b;
+    return b;
+  }
+  SPARSP_QUEUE_FN uint32_t next_k() {
+    const uint32_t b = ring & 15u;
+    ring = (ring >> 4) | b << (4 * (kRing - 1));
+    return b;
+  }
+};
 
 }  // namespace sparsp
