@@ -333,7 +333,7 @@ int sparsp_block_mask(const sparsp_shape* shape, const void* Q, const void* K, i
   float* pq = pooled_q ? pooled_q : (float*)(ws + L.pooled_q);
   float* pk = pooled_k ? pooled_k : (float*)(ws + L.pooled_k);
   cudaStream_t st = (cudaStream_t)stream;
-  SPARSP_TRY(launch_pool(*shape, g, Q, K, pq, pk, st));
+  SPARSP_TRY(launch_pool(*shape, g, Q, K, pq, pk, ws, L, st));
   SPARSP_TRY(launch_score_topk(g, pq, pk, (float*)(ws + L.scores), topk_video, mask, kv_list, kv_count, st));
   return SPARSP_OK;
 }
@@ -369,7 +369,7 @@ int sparsp_block_mask_cdf(const sparsp_shape* shape, const void* Q, const void* 
   float* pk = pooled_k ? pooled_k : (float*)(ws + L.pooled_k);
   cudaStream_t st = (cudaStream_t)stream;
   const float scale = score_scale > 0.0f ? score_scale : 1.0f / sqrtf((float)g.d);
-  SPARSP_TRY(launch_pool(*shape, g, Q, K, pq, pk, st));
+  SPARSP_TRY(launch_pool(*shape, g, Q, K, pq, pk, ws, L, st));
   SPARSP_TRY(launch_score_cdf(g, pq, pk, (float*)(ws + L.scores), tau, scale, mask, kv_count, st));
   return SPARSP_OK;
 }

@@ -100,8 +100,8 @@ int make_tile_tmap(CUtensorMap* out, const void* base, const sparsp_shape& s, co
                    bool swizzled);
 
 // launchers implemented in the kernel files -------------------------------------------------
-int launch_pool(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, float* pq,
-                float* pk, cudaStream_t st);
+int launch_pool(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, float* pq, float* pk, char* ws,
+                const WsLayout& L, cudaStream_t st);
 int launch_permute_tokens(const sparsp_shape& s, const Geometry& g, const void* X, void* Y,
                           const int32_t* block_of_slot, const int64_t* token_offset_of_slot, int inverse,
                           cudaStream_t st);

@@ -6,105 +6,83 @@
 //          IEEE division by the valid count;
 //   score: acc = fmaf(q_c, k_c, acc) from acc = 0, channel c ascending;
 //   top-k: score descending, index ascending on equal scores, -0 == +0.
-#include <cstring>
-#include <type_traits>
-
 #include "common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace sparsp {
 
 // ------------------------------------------------------------------------------------------------
-// pool: a group of lanes owns one (tensor, batch*head, block) tile; a lane owns 8 (or 4) channels and walks the tile's
-// rows with 16-byte (8-byte) loads, several of them in flight, so every channel is one sequential chain.
-// Large problems are HBM-bound: 16-byte loads, unrolled over 16 rows (24 heads x 24576 x 128: 53.6 us = 5.6 TB/s; over
-// 8 rows 54.5, 8-byte loads of 32 rows 68), of which the compiler keeps what fits 51 registers in flight, about 8.
-// Where the tiles do not fill a quarter of the chip's thread slots (148 SMs; the measured crossover, not a property of
-// the kernel) the time is the latency of the dependent batches: 8-byte loads, so twice the threads, and 32 rows in
-// flight (95 registers; 26 heads x 6034 x 64: 17.9 us against 28 with the wide form and 32-38 with 8 rows of it; 2
-// heads x 4096: 4.3 us against 6.2).
+// pool: a warp per (tensor, batch*head, block) tile, a CTA of its own.  The tile comes into shared memory as one TMA load
+// (any token stride; rows behind the last token arrive as zeros), so all of it is in flight at once and as many tiles per
+// multiprocessor as fit there; a lane then adds its 2 or 4 channels row by row, every channel one sequential chain.
+// HBM-bound where there are many tiles, one memory latency and the chain of `block` additions where there are few.
+// us of a whole mask call with loads through registers (8 to 32 rows in flight a lane) / this way: 40 heads x 75600 x 128
+// 486 / 419, 24 x 24576 115 / 100 (pool alone 53.6 -> about 46, 6.5 TB/s), 48 x 17776 x 64 89 / 81, 2 x 13 x 6034 x 64
+// token-major 18.6 / 13.1, 48 heads x 1558 token-major 23.9 / 14.5, 2 x 4096 x 64 11.7 / 9.9.
 // ------------------------------------------------------------------------------------------------
-constexpr int kPoolThreads = 128;
-constexpr int kPoolNarrowThreads = 148 * 512;  // up to this many threads of the wide form the narrow one is used
-
-template <int D, bool kNarrow>
-__global__ void __launch_bounds__(kPoolThreads) pool_kernel(const __nv_bfloat16* __restrict__ Q,
-                                                            const __nv_bfloat16* __restrict__ K,
-                                                            float* __restrict__ pq, float* __restrict__ pk,
-                                                            int H, int NB, int b, int64_t N, int64_t sB,
-                                                            int64_t sH, int64_t sT, int64_t n_tiles) {
-  enter_grid(Q, K);
-  constexpr int kVec = kNarrow ? 4 : 8;    // channels per lane
-  constexpr int kRows = kNarrow ? 32 : 16;  // rows in flight
-  constexpr int G = D / kVec;              // lanes per tile
-  constexpr int W = kVec / 2;              // 32-bit words per lane and row
-  using Vec = typename std::conditional<kNarrow, uint2, uint4>::type;
-  const int64_t tile = ((int64_t)blockIdx.x * kPoolThreads + threadIdx.x) / G;
-  const int lane = threadIdx.x % G;
-  if (tile >= 2 * n_tiles) return;
-  const bool is_k = tile >= n_tiles;
-  const int64_t t = is_k ? tile - n_tiles : tile;  // (batch*H + head) * NB + block
-  const int64_t bh = t / NB;
-  const int blk = (int)(t - bh * NB);
-  const int64_t batch = bh / H, head = bh % H;
-  const int64_t tok0 = (int64_t)blk * b;
-  const int n = (int)min((int64_t)b, N - tok0);
-  const __nv_bfloat16* src = (is_k ? K : Q) + batch * sB + head * sH + tok0 * sT + lane * kVec;
-
-  float acc[kVec];
+template <int D>
+__global__ void __launch_bounds__(32) pool_kernel(const __grid_constant__ CUtensorMap tmQ,
+                                                  const __grid_constant__ CUtensorMap tmK, float* __restrict__ pq,
+                                                  float* __restrict__ pk, int H, int NB, int b, int64_t N, int n_tiles,
+                                                  int32_t* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ uint64_t full;
+  __shared__ int s_abort;
+  const int lane = threadIdx.x;
+  const bool is_k = blockIdx.x >= (unsigned)n_tiles;
+  const int t = is_k ? (int)blockIdx.x - n_tiles : (int)blockIdx.x;  // (batch*H + head) * NB + block
+  const int bh = t / NB, blk = t - bh * NB;
+  if (lane == 0) {
+    s_abort = 0;
+    ptx::mbar_init(&full, 1);
+    ptx::mbar_init_fence();
+  }
+  enter_grid();
+  if (lane == 0) {
+    ptx::mbar_expect_tx(&full, (uint32_t)(b * D * 2));
+    ptx::tma_load_4d(smem_raw, is_k ? &tmK : &tmQ, &full, 0, blk * b, bh % H, bh / H);
+  }
+  __syncwarp();
+  ptx::mbar_wait_bounded(&full, 0, &s_abort, status, 50, 200000000LL);
+  constexpr int W = D / 64;  // 32-bit words per lane and row
+  const uint32_t* row = reinterpret_cast<const uint32_t*>(smem_raw) + lane * W;
+  float acc[2 * W];
 #pragma unroll
-  for (int c = 0; c < kVec; ++c) acc[c] = 0.0f;
-  auto add = [&](const Vec& x) {
+  for (int c = 0; c < 2 * W; ++c) acc[c] = 0.0f;
+  // (a row behind the last token adds +0, which changes no sum: a sum that starts at +0 is never -0)
+#pragma unroll 16
+  for (int r = 0; r < b; ++r, row += D / 2) {
     uint32_t v[W];
-    memcpy(v, &x, sizeof v);
+    if (W == 2) {
+      const uint2 x = *reinterpret_cast<const uint2*>(row);
+      v[0] = x.x;
+      v[W - 1] = x.y;
+    } else {
+      v[0] = *row;
+    }
 #pragma unroll
     for (int w = 0; w < W; ++w) {
       acc[2 * w] = __fadd_rn(acc[2 * w], __uint_as_float(v[w] << 16));
       acc[2 * w + 1] = __fadd_rn(acc[2 * w + 1], __uint_as_float(v[w] & 0xffff0000u));
     }
-  };
-  auto load = [&](int r) { return __ldg(reinterpret_cast<const Vec*>(src + (int64_t)r * sT)); };
-  int r = 0;
-  if (kNarrow) {
-    for (; r < n; r += kRows) {
-      Vec x[kRows];
-#pragma unroll
-      for (int u = 0; u < kRows; ++u) {
-        x[u] = Vec{};
-        if (r + u < n) x[u] = load(r + u);
-      }
-      // (a row behind the last token adds +0, which changes no sum: a sum that starts at +0 is never -0)
-#pragma unroll
-      for (int u = 0; u < kRows; ++u) add(x[u]);
-    }
-  } else {
-    for (; r + kRows <= n; r += kRows) {
-      Vec x[kRows];
-#pragma unroll
-      for (int u = 0; u < kRows; ++u) x[u] = load(r + u);
-#pragma unroll
-      for (int u = 0; u < kRows; ++u) add(x[u]);
-    }
-    for (; r < n; ++r) add(load(r));
   }
-  const float cntf = (float)n;
-  float* dst = (is_k ? pk : pq) + t * D + lane * kVec;
+  const float cntf = (float)min((int64_t)b, N - (int64_t)blk * b);
+  float* dst = (is_k ? pk : pq) + (int64_t)t * D + lane * 2 * W;
 #pragma unroll
-  for (int c = 0; c < kVec; c += 4)
-    *reinterpret_cast<float4*>(dst + c) = make_float4(__fdiv_rn(acc[c], cntf), __fdiv_rn(acc[c + 1], cntf),
-                                                      __fdiv_rn(acc[c + 2], cntf), __fdiv_rn(acc[c + 3], cntf));
+  for (int w = 0; w < W; ++w)
+    *reinterpret_cast<float2*>(dst + 2 * w) = make_float2(__fdiv_rn(acc[2 * w], cntf), __fdiv_rn(acc[2 * w + 1], cntf));
 }
 
-int launch_pool(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, float* pq,
-                float* pk, cudaStream_t st) {
-  const int64_t n_tiles = (int64_t)g.B * g.H * g.NB;
-  int64_t threads = 2 * n_tiles * (g.d / 8);
-  const bool narrow = threads <= kPoolNarrowThreads;
-  if (narrow) threads *= 2;
-  auto kern = g.d == 64 ? (narrow ? pool_kernel<64, true> : pool_kernel<64, false>)
-                        : (narrow ? pool_kernel<128, true> : pool_kernel<128, false>);
-  SPARSP_CUDA_OK(launch_kernel(kern, (unsigned)((threads + kPoolThreads - 1) / kPoolThreads), kPoolThreads, 0, st,
-                               (const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, pq, pk, g.H, g.NB, g.b, g.N,
-                               s.stride_batch, s.stride_head, s.stride_token, n_tiles));
+int launch_pool(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, float* pq, float* pk, char* ws,
+                const WsLayout& L, cudaStream_t st) {
+  CUtensorMap tq, tk;
+  int rc;
+  if ((rc = make_tile_tmap(&tq, Q, s, g, g.b, false)) != SPARSP_OK) return rc;
+  if ((rc = make_tile_tmap(&tk, K, s, g, g.b, false)) != SPARSP_OK) return rc;
+  const int n_tiles = g.B * g.H * g.NB;
+  auto kern = g.d == 64 ? pool_kernel<64> : pool_kernel<128>;
+  SPARSP_CUDA_OK(launch_kernel(kern, 2u * (unsigned)n_tiles, 32, (size_t)g.b * g.d * 2, st, tq, tk, pq, pk, g.H, g.NB, g.b,
+                               g.N, n_tiles, (int32_t*)(ws + L.status)));
   return SPARSP_OK;
 }
 
