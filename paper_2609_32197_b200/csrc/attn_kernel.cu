@@ -79,7 +79,6 @@ struct AttnParams {
   int64_t sB, sH, sT;
   int BH, H, NB, Wd;
   int in_place;      // O is Q: no row of an item is written before all of them are known to be right
-  int single;        // block 64, K / V source: every item is one query block (an int of `pairs` each), none are stacked
   float scale_log2;  // softmax scale * log2(e)
   long long wait_limit;
 };
@@ -162,6 +161,10 @@ struct Entry<true> {
 // Item header, one load for each role: x = batch * H + head; y = entries | kHead... flags (0: there are no more items);
 // z = query blocks, first | second << 16 (0xffff: none); w = batch.
 constexpr int kHeadEntries = 0xffff, kHeadRagged = 1 << 16, kHeadRefShift = 17, kHeadNoneShift = 19;
+
+// Where items and their K / V tiles come from: a queue of items and the sequence's own K and V; the same, but every query
+// block has a CTA of its own and is its item (64-token blocks: not stacked); a queue and a consumer's packed buffer.
+enum class Source { kQueue, kDirect, kPacked };
 
 template <int D, int BLK>
 struct AttnCfg {
@@ -285,12 +288,13 @@ __device__ __forceinline__ void clear_rows(const AttnParams& p, int bh, int i) {
     for (int r = lane; r < n; r += 32) p.lse[bh * p.N + tok0 + r] = -INFINITY;
 }
 
-template <int D, int BLK, bool kPacked>
+template <int D, int BLK, Source kSource>
 __global__ void __launch_bounds__(kAttnThreads, 1)
     attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmP,
                     const AttnParams p) {
   using C = AttnCfg<D, BLK>;
+  constexpr bool kPacked = kSource == Source::kPacked, kDirect = kSource == Source::kDirect;
   constexpr int SV = C::kStagesV;
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem =
@@ -582,7 +586,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         h_end += hbase;
       };
       if (kPacked) load_heads();
-      const bool stacked = C::kStacked && (kPacked || !p.single);
       int bh = p.BH, blk0 = -1, blk1 = -1;
       const int ragged_block = p.N % BLK ? p.NB - 1 : -1;
       uint32_t rb0 = 0u, rb1 = 0u;  // the item's mask rows, a word per lane (NB <= 1024: at most 32 words)
@@ -593,6 +596,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         rb1 = lane < p.Wd && blk1 >= 0 ? rows[blk1 * p.Wd + lane] : 0u;
       };
       auto fetch = [&](int it) {
+        if (kDirect) {  // my item is the query block of my number, if it keeps anything
+          bh = it / p.NB;
+          blk0 = it - bh * p.NB;
+          if (bh < p.BH) load_rows();
+          if (!__any_sync(0xffffffffu, rb0 != 0u)) bh = p.BH;
+          return;
+        }
         int x;
         if (kPacked) {
           uint32_t after;  // heads whose items end behind this one
@@ -614,16 +624,17 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             }
             return __shfl_sync(0xffffffffu, to, 0);
           };
-          bh = find_item(it, stacked ? (p.NB + 1) / 2 : p.NB, p.BH, p.n_items, leave_head,
+          bh = find_item(it, C::kStacked ? (p.NB + 1) / 2 : p.NB, p.BH, p.n_items, leave_head,
                          [&] { return *s_abort != 0; }, &x);
         }
         if (bh >= p.BH) return;
         const int32_t* items = p.pairs + (int64_t)bh * (2 * ((p.NB + 1) / 2));
-        blk0 = stacked ? items[2 * x] : items[x];
-        blk1 = stacked ? items[2 * x + 1] : -1;
+        blk0 = C::kStacked ? items[2 * x] : items[x];
+        blk1 = C::kStacked ? items[2 * x + 1] : -1;
         load_rows();
       };
       auto next_item = [&]() {
+        if (kDirect) return p.BH * p.NB;
         int it = 0;
         if (lane == 0) it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
         return __shfl_sync(0xffffffffu, it, 0);
@@ -1173,7 +1184,6 @@ struct PrepParams {
   int32_t* n_items;
   int32_t* work_counter;
   int BH, H, NB, Wd, b;
-  int single;  // block 64: no block shares a Q tile
   // packed source only
   const int32_t* rank;
   const uint32_t* U;
@@ -1238,7 +1248,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
   auto block = [&](int pos) -> int { return list ? list[pos] : pos; };
   int n_keys;
   bool live = false;  // any of my keys is an item's
-  if (p.b == 64 && !p.single) {
+  if (p.b == 64) {
     uint32_t* m = reinterpret_cast<uint32_t*>(smem_raw);  // [n][pitch]
     const int Wd = p.Wd, pitch = Wd | 1;
     if (threadIdx.x == 0) s_best = 1023u - 1u;  // default D = 1
@@ -1323,7 +1333,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
     const bool is_item = x < n_keys && (s_keys[x] >> 10) != 0u;
     if (is_item) {
       const int c = 1023 - (int)(s_keys[x] & 1023u);
-      if (p.b == 64 && !p.single) {
+      if (p.b == 64) {
         const int a = (int)(s_pair[c] & 0xffffu), b2 = (int)(s_pair[c] >> 16);
         out[2 * x] = block(a);
         out[2 * x + 1] = b2 != 0xffff ? block(b2) : -1;
@@ -1488,7 +1498,7 @@ static int make_packed_tmap(CUtensorMap* out, const void* packed, int64_t capaci
   return SPARSP_OK;
 }
 
-template <int D, int BLK, bool kPacked>
+template <int D, int BLK, Source kSource>
 static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, const void* V,
                          const void* packed, int64_t packed_capacity, const AttnParams& p, cudaStream_t st) {
   CUtensorMap tq, tk, tv, tp;
@@ -1496,16 +1506,16 @@ static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q
   if ((rc = make_tile_tmap(&tq, Q, s, g, BLK, true)) != SPARSP_OK) return rc;
   if ((rc = make_tile_tmap(&tk, K, s, g, BLK, true)) != SPARSP_OK) return rc;
   if ((rc = make_tile_tmap(&tv, V, s, g, BLK, true)) != SPARSP_OK) return rc;
-  if (kPacked) {
+  if (kSource == Source::kPacked) {
     if ((rc = make_packed_tmap(&tp, packed, packed_capacity, g)) != SPARSP_OK) return rc;
   } else {
     tp = tk;  // never used
   }
-  auto kern = attn_fwd_kernel<D, BLK, kPacked>;
+  auto kern = attn_fwd_kernel<D, BLK, kSource>;
   const int smem = AttnCfg<D, BLK>::kDynamic;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
   // work item = one 128-row Q tile (a 128-token block, a pair of 64-token blocks, or one of them); one persistent CTA per SM
-  const int64_t most = (int64_t)g.B * g.H * (BLK == 128 || p.single ? g.NB : (g.NB + 1) / 2);
+  const int64_t most = (int64_t)g.B * g.H * (BLK == 128 || kSource == Source::kDirect ? g.NB : (g.NB + 1) / 2);
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
   const unsigned grid = (unsigned)std::min<int64_t>(most, sms);
@@ -1513,7 +1523,7 @@ static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q
   return SPARSP_OK;
 }
 
-template <bool kPacked>
+template <Source kSource>
 static int launch_attn_common(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, const void* V,
                               const void* packed, int64_t packed_capacity, AttnParams p, float scale, void* O,
                               float* lse, char* ws, const WsLayout& L, cudaStream_t st) {
@@ -1533,10 +1543,10 @@ static int launch_attn_common(const sparsp_shape& s, const Geometry& g, const vo
   const float sc = scale > 0.0f ? scale : 1.0f / sqrtf((float)g.d);
   p.scale_log2 = sc * 1.4426950408889634f;
   p.wait_limit = 200000000LL;  // about 0.1 s of SM clocks
-  if (g.d == 64 && g.b == 64) return launch_attn_t<64, 64, kPacked>(s, g, Q, K, V, packed, packed_capacity, p, st);
-  if (g.d == 64 && g.b == 128) return launch_attn_t<64, 128, kPacked>(s, g, Q, K, V, packed, packed_capacity, p, st);
-  if (g.d == 128 && g.b == 64) return launch_attn_t<128, 64, kPacked>(s, g, Q, K, V, packed, packed_capacity, p, st);
-  return launch_attn_t<128, 128, kPacked>(s, g, Q, K, V, packed, packed_capacity, p, st);
+  if (g.d == 64 && g.b == 64) return launch_attn_t<64, 64, kSource>(s, g, Q, K, V, packed, packed_capacity, p, st);
+  if (g.d == 64 && g.b == 128) return launch_attn_t<64, 128, kSource>(s, g, Q, K, V, packed, packed_capacity, p, st);
+  if (g.d == 128 && g.b == 64) return launch_attn_t<128, 64, kSource>(s, g, Q, K, V, packed, packed_capacity, p, st);
+  return launch_attn_t<128, 128, kSource>(s, g, Q, K, V, packed, packed_capacity, p, st);
 }
 
 template <bool kPacked>
@@ -1565,21 +1575,23 @@ static PrepParams prep_params(const Geometry& g, const uint32_t* mask, char* ws,
 int launch_attn(const sparsp_shape& s, const Geometry& g, const void* Q, const void* K, const void* V,
                 const uint32_t* mask, float scale, void* O, float* lse, char* ws, const WsLayout& L,
                 cudaStream_t st) {
-  PrepParams pre = prep_params(g, mask, ws, L);
-  // Two query blocks share a Q tile for the sake of throughput.  Where every block can have an SM of its own there is none
-  // to be had, and an item is done sooner with its own list than with the union of two (2 heads x 64 blocks, 16 kept: 15.8
-  // us a call against 19.4).
-  int sms = 0;
-  SPARSP_CUDA_OK(sm_count(&sms));
-  pre.single = g.b == 64 && (int64_t)g.B * g.H * g.NB <= sms;
-  const int rc = launch_prep<false>(g, pre, st);
-  if (rc != SPARSP_OK) return rc;
   AttnParams p = {};
   p.mask = mask;
+  // Where every query block can have an SM of its own, its CTA needs no queue, no order and no partner for it: one launch.
+  // Two query blocks share a Q tile for the sake of throughput, and alone one is done sooner with its own list than with the
+  // union of two.  (us a call with the launch that makes items, stacked / single / without it: 2 heads x 64 blocks of 64 x 64,
+  // 16 kept 19.4 / 14.9 / 11.5; 7 x 21 of 64 x 128 - / 15.7 / 10.4.  An instance of the kernel of its own, because the
+  // question inside the queue's made 64-token blocks 1-2 % slower.)
+  int sms = 0;
+  SPARSP_CUDA_OK(sm_count(&sms));
+  if ((int64_t)g.B * g.H * g.NB <= sms)
+    return launch_attn_common<Source::kDirect>(s, g, Q, K, V, nullptr, 0, p, scale, O, lse, ws, L, st);
+  const PrepParams pre = prep_params(g, mask, ws, L);
+  const int rc = launch_prep<false>(g, pre, st);
+  if (rc != SPARSP_OK) return rc;
   p.pairs = pre.pairs;
   p.n_items = pre.n_items;
-  p.single = pre.single;
-  return launch_attn_common<false>(s, g, Q, K, V, nullptr, 0, p, scale, O, lse, ws, L, st);
+  return launch_attn_common<Source::kQueue>(s, g, Q, K, V, nullptr, 0, p, scale, O, lse, ws, L, st);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1612,7 +1624,7 @@ int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, 
   p.tile_base = pre.tile_base;
   p.rank = rank;
   p.consumer = consumer;
-  return launch_attn_common<true>(s, g, Q, K, V, packed, capacity, p, scale, O, lse, ws, L, st);
+  return launch_attn_common<Source::kPacked>(s, g, Q, K, V, packed, capacity, p, scale, O, lse, ws, L, st);
 }
 
 }  // namespace sparsp
