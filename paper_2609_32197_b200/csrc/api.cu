@@ -42,6 +42,18 @@ cudaError_t ensure_dynamic_smem(const void* func, int bytes) {
   return cudaSuccess;
 }
 
+cudaError_t sm_count(int* sms) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::atomic<int>* slot = dev >= 0 && dev < 64 ? known + dev : nullptr;
+  if (slot && (*sms = slot->load(std::memory_order_relaxed)) > 0) return cudaSuccess;
+  e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess && slot) slot->store(*sms, std::memory_order_relaxed);
+  return e;
+}
+
 int make_geometry(const sparsp_shape* s, Geometry* g) {
   if (!s) {
     set_error("shape is NULL");

@@ -17,6 +17,7 @@ namespace sparsp {
 constexpr int kMaxBlocks = 1024;  // NB limit (score rows are held in shared memory)
 constexpr int kMaxRanks = 64;
 constexpr int kStatusWords = 64;  // workspace header: word 0 = status code, 1.. = detail
+constexpr int kPlanTicketWord = 16, kPlanTickets = 48;  // words of the header that count a plan's finished CTAs, 0 between launches
 
 struct Geometry {
   int64_t N;         // tokens
@@ -43,6 +44,9 @@ WsLayout make_layout(const Geometry& g, int n_ranks);
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` on the current device; remembers
 // what was set per (kernel, device) so that the driver call is made only when the limit must grow.
 cudaError_t ensure_dynamic_smem(const void* func, int bytes);
+
+// Multiprocessors of the current device; asked of the driver once per device.
+cudaError_t sm_count(int* sms);
 
 // Launches a kernel that may start while the launches before it in the stream still run (programmatic stream
 // serialisation): its CTAs take their places and set themselves up as soon as the previous kernel's have all started,

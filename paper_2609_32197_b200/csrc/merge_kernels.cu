@@ -162,9 +162,8 @@ int launch_attn_merge(const sparsp_shape& s, const Geometry& g, const void* Oa, 
                       const float* lb, void* O, float* lse, const int32_t* rank, int consumer, int head_begin,
                       int head_end, cudaStream_t st) {
   if (head_end <= head_begin) return SPARSP_OK;
-  int dev = 0, sms = 148;
-  SPARSP_CUDA_OK(cudaGetDevice(&dev));
-  SPARSP_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  int sms = 0;
+  SPARSP_CUDA_OK(sm_count(&sms));
   const int rows = g.d == 64 && g.b == 64 ? 2 : 4;
   auto kern = g.d == 128 ? attn_merge_kernel<128, 4> : rows == 2 ? attn_merge_kernel<64, 2> : attn_merge_kernel<64, 4>;
   const int64_t units = (int64_t)g.B * (head_end - head_begin) * g.NB;
