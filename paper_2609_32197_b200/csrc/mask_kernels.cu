@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kScoreThreads) score_kernel(const float* __res
                                                               float* __restrict__ scores) {
   enter_grid(pq, pk);
   constexpr int LD = D + 4;  // row pitch in floats: 16 bytes of skew per row
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   float* sQ = reinterpret_cast<float*>(smem_raw);  // [64][LD]
   float* sK = sQ + kScoreTile * LD;                // [64][LD]
   const int64_t bh = blockIdx.z;
@@ -198,23 +198,22 @@ __device__ __forceinline__ uint32_t middle(uint32_t lo, uint32_t hi, int step) {
   return by_score > lo && by_score <= hi && step % 3 != 2 ? by_score : lo + ((hi - lo) >> 1) + 1;
 }
 
-template <int WMAX>  // mask words per row this instance can hold (keys live in registers: WMAX per lane)
-__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 6 : 4)
-    topk_kernel(const float* __restrict__ scores, int64_t n_rows, int NB, int Wd, int nb_cand, int topk, int kept_cap,
-                uint32_t* __restrict__ mask, int32_t* __restrict__ kv_list, int32_t* __restrict__ kv_count) {
-  enter_grid(scores);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * kTopkWarps + warp;  // (batch*H + head) * NB + i
-  if (row >= n_rows) return;
-  const float* srow = scores + row * NB;
-  // lane l holds the keys of blocks l, l + 32, ...; a block that is not a candidate (text, padding) holds 0,
-  // which no trial threshold (>= 1) counts
+struct TopkParams {
+  int NB, Wd, nb_cand, topk, kept_cap;
+  uint32_t* mask;
+  int32_t *kv_list, *kv_count;
+};
+
+// One warp, one row: score(t) is the score of block t * 32 + lane, asked for candidates only.
+template <int WMAX, typename Score>
+__device__ __forceinline__ void select_row(const TopkParams& p, int64_t row, Score score) {
+  const int lane = threadIdx.x & 31, NB = p.NB, Wd = p.Wd, nb_cand = p.nb_cand, topk = p.topk, kept_cap = p.kept_cap;
+  uint32_t* mask = p.mask;
+  int32_t *kv_list = p.kv_list, *kv_count = p.kv_count;
+  // a block that is not a candidate (text, padding) holds the key 0, which no trial threshold (>= 1) counts
   uint32_t key[WMAX];
 #pragma unroll
-  for (int t = 0; t < WMAX; ++t) {
-    const int j = t * 32 + lane;
-    key[t] = (t < Wd && j < nb_cand) ? score_key(__ldcs(srow + j)) : 0u;
-  }
+  for (int t = 0; t < WMAX; ++t) key[t] = (t < Wd && t * 32 + lane < nb_cand) ? score_key(score(t)) : 0u;
 
   const uint32_t lt_mask = (1u << lane) - 1u;
   // T with |{ candidates : key >= T }| == topk, or else the topk-th largest key (ties)
@@ -265,6 +264,21 @@ __global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 6 : 4)
   if (kv_count && lane == 0) kv_count[row] = out_pos;
 }
 
+template <int WMAX, typename Params>
+__device__ __forceinline__ void select_stored_row(const Params& p, const float* scores, int64_t n_rows) {
+  const int64_t row = (int64_t)blockIdx.x * kTopkWarps + (threadIdx.x >> 5);  // (batch*H + head) * NB + i
+  if (row >= n_rows) return;
+  const float* srow = scores + row * p.NB + (threadIdx.x & 31);
+  select_row<WMAX>(p, row, [&](int t) { return __ldcs(srow + t * 32); });
+}
+
+template <int WMAX>  // mask words per row this instance can hold (keys live in registers: WMAX per lane)
+__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 6 : 4)
+    topk_kernel(const float* __restrict__ scores, int64_t n_rows, const TopkParams p) {
+  enter_grid(scores);
+  select_stored_row<WMAX>(p, scores, n_rows);
+}
+
 // ------------------------------------------------------------------------------------------------
 // CDF-threshold selection (Section 8.1): per row, softmax over the candidate scores, keep the smallest
 // top set by score (whole groups of equal scores) whose mass reaches tau.  The mass is counted in integers, so
@@ -297,15 +311,19 @@ __device__ __forceinline__ unsigned long long warp_sum(uint32_t v) {
   return ((unsigned long long)hi << 16) + lo;
 }
 
-template <int WMAX>  // mask words per row this instance can hold (keys and terms live in registers)
-__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 4 : WMAX <= 20 ? 3 : 2)
-    cdf_kernel(const float* __restrict__ scores, int64_t n_rows, int NB, int Wd, int nb_cand, float tau, float c,
-               uint32_t* __restrict__ mask, int32_t* __restrict__ kv_count) {
-  enter_grid(scores);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * kTopkWarps + warp;  // (batch*H + head) * NB + i
-  if (row >= n_rows) return;
-  const float* srow = scores + row * NB;
+struct CdfParams {
+  int NB, Wd, nb_cand;
+  float tau, c;
+  uint32_t* mask;
+  int32_t* kv_count;
+};
+
+template <int WMAX, typename Score>
+__device__ __forceinline__ void select_row(const CdfParams& p, int64_t row, Score score) {
+  const int lane = threadIdx.x & 31, NB = p.NB, Wd = p.Wd, nb_cand = p.nb_cand;
+  const float tau = p.tau, c = p.c;
+  uint32_t* mask = p.mask;
+  int32_t* kv_count = p.kv_count;
   // lane l holds blocks l, l + 32, ...  A block that is not a candidate holds key 0 (no trial threshold, all
   // >= 1, selects it) and the weight 0.
   uint32_t key[WMAX];
@@ -315,7 +333,7 @@ __global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 4 : WMAX <= 20 ?
   for (int t = 0; t < WMAX; ++t) {
     const int j = t * 32 + lane;
     const bool cand = t < Wd && j < nb_cand;
-    const float s = cand ? __ldcs(srow + j) : -INFINITY;
+    const float s = cand ? score(t) : -INFINITY;
     w[t] = __float_as_uint(s);
     key[t] = cand ? score_key(s) : 0u;
     mx = fmaxf(mx, s);
@@ -380,35 +398,111 @@ __global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 4 : WMAX <= 20 ?
   if (kv_count && lane == 0) kv_count[row] = cnt;
 }
 
+template <int WMAX>  // mask words per row this instance can hold (keys and terms live in registers)
+__global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 4 : WMAX <= 20 ? 3 : 2)
+    cdf_kernel(const float* __restrict__ scores, int64_t n_rows, const CdfParams p) {
+  enter_grid(scores);
+  select_stored_row<WMAX>(p, scores, n_rows);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Scores and selection of short rows (up to 128 blocks) in one launch: a CTA keeps the pooled K of its head in shared memory
+// and takes a few rows of it, a warp each, whose scores never leave the registers they are selected from.  Same chains, same
+// selection.  What bounds it is the latency of the launch, of bringing pooled K in (16 warps, more than have a row) and of one
+// row: few rows a CTA while all CTAs run at once, more where pooled K would be read too often.  us of a whole mask call, two
+// launches / this way: 2 heads x 64 blocks of d = 64 9.7 / 7.6, 7 x 21 of d = 128 13.5 / 7.7, 2 x 68 15.2 / 9.6, 5 x 108 18.3 /
+// 12.0, 26 x 48 of d = 64 13.2 / 10.6, 48 x 128 of d = 128 85 / 82.  (8 warps and rows whatever the size: 7.6, 7.6, 12.8, 15.1,
+// 10.9, 84.  Rows of up to 256 blocks: 7 x 147 21.1 -> 18.5, but 2 x 200 14.2 -> 17.5 and 24 x 256 60 -> 79.)
+// ------------------------------------------------------------------------------------------------
+constexpr int kShortWords = 4;
+constexpr int kShortWarps = 16;
+
+template <int D, typename Params>
+__global__ void __launch_bounds__(kShortWarps * 32)
+    short_rows_kernel(const float* __restrict__ pq, const float* __restrict__ pk, int rows, const Params p) {
+  enter_grid(pq, pk);
+  constexpr int LD = D + 4;  // row pitch in floats: 16 bytes of skew per row
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  float* sK = reinterpret_cast<float*>(smem_raw);  // [NB][LD]
+  float* sQ = sK + p.NB * LD;                      // [rows][D]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, NB = p.NB;
+  const int64_t row0 = (int64_t)blockIdx.y * NB;   // of my head
+  const int first = blockIdx.x * rows, n_rows = min(rows, NB - first);
+  const float4* k4 = reinterpret_cast<const float4*>(pk + row0 * D);
+  const float4* q4 = reinterpret_cast<const float4*>(pq + (row0 + first) * D);
+  for (int idx = threadIdx.x; idx < n_rows * (D / 4); idx += kShortWarps * 32)
+    reinterpret_cast<float4*>(sQ)[idx] = __ldg(q4 + idx);
+#pragma unroll 8
+  for (int idx = threadIdx.x; idx < NB * (D / 4); idx += kShortWarps * 32)
+    *reinterpret_cast<float4*>(sK + idx / (D / 4) * LD + idx % (D / 4) * 4) = __ldg(k4 + idx);
+  __syncthreads();
+  if (warp >= n_rows) return;
+  float score[kShortWords];
+#pragma unroll
+  for (int t = 0; t < kShortWords; ++t) score[t] = 0.0f;
+  const float* q = sQ + warp * D;
+#pragma unroll 4
+  for (int c = 0; c < D; c += 4) {
+    const float4 qv = *reinterpret_cast<const float4*>(q + c);
+#pragma unroll
+    for (int t = 0; t < kShortWords; ++t) {
+      if (t * 32 < NB) {  // (lanes behind the last block take its row)
+        const float4 kv = *reinterpret_cast<const float4*>(sK + min(t * 32 + lane, NB - 1) * LD + c);
+        score[t] = __fmaf_rn(qv.x, kv.x, score[t]);
+        score[t] = __fmaf_rn(qv.y, kv.y, score[t]);
+        score[t] = __fmaf_rn(qv.z, kv.z, score[t]);
+        score[t] = __fmaf_rn(qv.w, kv.w, score[t]);
+      }
+    }
+  }
+  select_row<kShortWords>(p, row0 + first + warp, [&](int t) { return score[t]; });
+}
+
+template <typename Params>
+static cudaError_t launch_short_rows(const Geometry& g, const float* pq, const float* pk, const Params& p, cudaStream_t st) {
+  const int64_t BH = (int64_t)g.B * g.H;
+  auto groups = [&](int rows) { return (g.NB + rows - 1) / rows; };
+  const int rows = BH * groups(4) <= 148 ? 4 : BH * groups(8) <= 2 * 148 ? 8 : kShortWarps;
+  const size_t smem = (size_t)(g.NB * (g.d + 4) + rows * g.d) * 4;
+  auto kern = g.d == 64 ? short_rows_kernel<64, Params> : short_rows_kernel<128, Params>;
+  const cudaError_t e = ensure_dynamic_smem((const void*)kern, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(kern, dim3((unsigned)groups(rows), (unsigned)BH), kShortWarps * 32, smem, st, pq, pk, rows, p);
+}
+static bool rows_are_short(const Geometry& g) { return g.Wd <= kShortWords && (int64_t)g.B * g.H <= 65535; }
+
 int launch_score_cdf(const Geometry& g, const float* pq, const float* pk, float* scores, float tau, float scale,
                      uint32_t* mask, int32_t* kv_count, cudaStream_t st) {
-  SPARSP_CUDA_OK(launch_score(g, pq, pk, scores, st));
-  {
-    const int64_t n_rows = (int64_t)g.B * g.H * g.NB;
-    const float c = scale * 1.4426950408889634f;  // fp32 product, as in the definition above
-    const unsigned grid = (unsigned)((n_rows + kTopkWarps - 1) / kTopkWarps);
-    auto kern = g.Wd <= 4 ? cdf_kernel<4> : g.Wd <= 8 ? cdf_kernel<8> :
-                g.Wd <= 12 ? cdf_kernel<12> : g.Wd <= 16 ? cdf_kernel<16> : g.Wd <= 20 ? cdf_kernel<20> :
-                g.Wd <= 24 ? cdf_kernel<24> : cdf_kernel<32>;
-    SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, g.NB, g.Wd, g.nb_cand, tau, c,
-                                 mask, kv_count));
+  const float c = scale * 1.4426950408889634f;  // fp32 product, as in the definition above
+  const CdfParams p = {g.NB, g.Wd, g.nb_cand, tau, c, mask, kv_count};
+  if (rows_are_short(g)) {
+    SPARSP_CUDA_OK(launch_short_rows(g, pq, pk, p, st));
+    return SPARSP_OK;
   }
+  SPARSP_CUDA_OK(launch_score(g, pq, pk, scores, st));
+  const int64_t n_rows = (int64_t)g.B * g.H * g.NB;
+  const unsigned grid = (unsigned)((n_rows + kTopkWarps - 1) / kTopkWarps);
+  auto kern = g.Wd <= 4 ? cdf_kernel<4> : g.Wd <= 8 ? cdf_kernel<8> :
+              g.Wd <= 12 ? cdf_kernel<12> : g.Wd <= 16 ? cdf_kernel<16> : g.Wd <= 20 ? cdf_kernel<20> :
+              g.Wd <= 24 ? cdf_kernel<24> : cdf_kernel<32>;
+  SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, p));
   return SPARSP_OK;
 }
 
 int launch_score_topk(const Geometry& g, const float* pq, const float* pk, float* scores, int topk,
                       uint32_t* mask, int32_t* kv_list, int32_t* kv_count, cudaStream_t st) {
-  const int kept_cap = topk + (g.NB - g.nb_cand);
-  SPARSP_CUDA_OK(launch_score(g, pq, pk, scores, st));
-  {
-    const int64_t n_rows = (int64_t)g.B * g.H * g.NB;
-    const unsigned grid = (unsigned)((n_rows + kTopkWarps - 1) / kTopkWarps);
-    auto kern = g.Wd <= 4 ? topk_kernel<4> : g.Wd <= 8 ? topk_kernel<8> :
-                g.Wd <= 12 ? topk_kernel<12> : g.Wd <= 16 ? topk_kernel<16> : g.Wd <= 20 ? topk_kernel<20> :
-                g.Wd <= 24 ? topk_kernel<24> : topk_kernel<32>;
-    SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, g.NB, g.Wd, g.nb_cand, topk,
-                                 kept_cap, mask, kv_list, kv_count));
+  const TopkParams p = {g.NB, g.Wd, g.nb_cand, topk, topk + (g.NB - g.nb_cand), mask, kv_list, kv_count};
+  if (rows_are_short(g)) {
+    SPARSP_CUDA_OK(launch_short_rows(g, pq, pk, p, st));
+    return SPARSP_OK;
   }
+  SPARSP_CUDA_OK(launch_score(g, pq, pk, scores, st));
+  const int64_t n_rows = (int64_t)g.B * g.H * g.NB;
+  const unsigned grid = (unsigned)((n_rows + kTopkWarps - 1) / kTopkWarps);
+  auto kern = g.Wd <= 4 ? topk_kernel<4> : g.Wd <= 8 ? topk_kernel<8> :
+              g.Wd <= 12 ? topk_kernel<12> : g.Wd <= 16 ? topk_kernel<16> : g.Wd <= 20 ? topk_kernel<20> :
+              g.Wd <= 24 ? topk_kernel<24> : topk_kernel<32>;
+  SPARSP_CUDA_OK(launch_kernel(kern, grid, kTopkWarps * 32, 0, st, scores, n_rows, p));
   return SPARSP_OK;
 }
 
