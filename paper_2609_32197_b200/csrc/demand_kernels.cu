@@ -504,6 +504,12 @@ static int prepare_pack(const sparsp_shape& s, const Geometry& g, const void* K,
 // few us at 6144 counts (24 heads, 16 ranks 1712 / 1483; one more head, by tables, 1784 / 1770).
 // ------------------------------------------------------------------------------------------------
 constexpr int kScanMax = 6144;
+// Masks of up to kMaskMax words are read by every CTA, which makes the unions and counts for itself (kFromMask): no launch of
+// the union before it.  A warp then gets every n-th block, of which there are few enough for that.  us of the whole call with
+// the union's launch / without: 2 heads x 64 blocks, 4 ranks 10.2 / 8.1; 7 x 21 of d = 128, 7 ranks 11.5 / 8.5; 48 x 13 of 128
+// x 128, 7 ranks 27.0 / 23.0; 2 x 13 x 48, 3 ranks 13.3 / 11.6; 40 x 40, 8 ranks 29.9 / 28.4 (3200 words); beyond the line 24 x
+// 80 (5760 words) 20.2 / 22.7, 9 x 166 (8964) 27.9 / 31.2; 16 x 64 of 128 x 128 in 7 blocks a warp 43.8 / 44.3.
+constexpr int kMaskMax = 4096, kFromMaskBlocks = 6;
 constexpr int kGatherStages = 3, kGatherThreads = 512;
 constexpr int kGatherSmem = 232448 - 7 * 1024;  // dynamic shared memory, next to less than 7 KB of its own
 
@@ -543,9 +549,11 @@ __device__ __forceinline__ void scan_rest(int n, int warp, int n_warps, int32_t*
   if (warp == 0 && lane == 0) out[n] = all;
 }
 
+template <bool kFromMask>
 __global__ void __launch_bounds__(kGatherThreads)
     gather_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                  const uint32_t* __restrict__ U, const int32_t* __restrict__ rank, const int32_t* __restrict__ cnt, int B,
+                  const uint32_t* __restrict__ mask, uint32_t* __restrict__ U_out, const int32_t* __restrict__ rank,
+                  int32_t* __restrict__ cnt_out, int B,
                   int H, int NB, int Wd, int P, int include_local, int b, uint32_t tile_bytes, int n_copy,
                   int64_t* __restrict__ seg_off, int64_t* __restrict__ seg_total, int64_t* __restrict__ volume,
                   const int64_t* __restrict__ dst_base, int64_t capacity, unsigned char* __restrict__ packed,
@@ -564,6 +572,7 @@ __global__ void __launch_bounds__(kGatherThreads)
   int32_t* pos_s = off_s + T + 1;                                        // [n_words + 1] live blocks before each word's
   uint32_t* live_s = reinterpret_cast<uint32_t*>(pos_s + n_words + 1);   // [B*H][Wd] blocks that any consumer receives
   uint32_t* own_s = live_s + n_words;                                    // [P][Wd]
+  uint32_t* union_s = own_s + P * Wd;                                    // kFromMask: [B*P][H][Wd]
   if (threadIdx.x == 0) s_abort = 0;
   if (threadIdx.x < kPackMaxWarps * kGatherStages) {
     ptx::mbar_init(full_all + threadIdx.x, 1);
@@ -572,15 +581,48 @@ __global__ void __launch_bounds__(kGatherThreads)
   // The launches behind this one begin when its CTAs end: an attention that takes its places while CTAs are still copying
   // makes the step longer (mask, demand and gather, attention of 2 x 13 x 6034 tokens 138 us, 131 this way, 141 with the
   // gather by tables; of 2 x 4096 39.2, 38.8 and 41).
-  wait_previous_grids(U, rank, cnt, dst_base);
+  const uint32_t* U = U_out;
+  const int32_t* cnt = cnt_out;
+  wait_previous_grids(mask, U, rank, cnt, dst_base);
+  if (kFromMask)
+    for (int i = threadIdx.x; i < n_words * P; i += kGatherThreads) union_s[i] = 0u;
   own_words(rank, NB, Wd, P, own_s);
+  if (kFromMask) {
+    const int n_mask = B * H * NB * Wd;
+    constexpr int kFlight = 8;
+    for (int i0 = threadIdx.x; i0 < n_mask; i0 += kFlight * kGatherThreads) {
+      uint32_t v[kFlight];
+#pragma unroll
+      for (int u = 0; u < kFlight; ++u) v[u] = i0 + u * kGatherThreads < n_mask ? mask[i0 + u * kGatherThreads] : 0u;
+#pragma unroll
+      for (int u = 0; u < kFlight; ++u) {
+        if (v[u] == 0u) continue;
+        const int i = i0 + u * kGatherThreads, row = i / Wd, w = i - row * Wd, bh = row / NB, bb = bh / H;
+        const int r = rank[row - bh * NB];
+        if ((unsigned)r < (unsigned)P) atomicOr(&union_s[((bb * P + r) * H + bh - bb * H) * Wd + w], v[u]);
+      }
+    }
+    U = union_s;
+  }
   __syncthreads();
+  if (kFromMask)
+    for (int i = blockIdx.x * kGatherThreads + threadIdx.x; i < n_words * P; i += gridDim.x * kGatherThreads)
+      U_out[i] = union_s[i];
   // One half of the warps scans the counts, the other the words of live blocks.
   constexpr int kHalf = kGatherThreads / 64;
   if (warp < kHalf) {
     scan_part<4>(T, warp, kHalf, off_s, warp_s, [&](int i) {
       const int br = i / PH, q = (i - br * PH) / H;
-      return q != br % P || include_local ? cnt[i] : 0;
+      int c;
+      if (kFromMask) {
+        const uint32_t* u = U + ((int64_t)br * H + i % H) * Wd;
+        c = 0;
+        for (int w = 0; w < Wd; ++w) c += __popc(u[w] & own_s[q * Wd + w]);
+        if (blockIdx.x == 0) cnt_out[i] = c;
+      } else {
+        c = cnt[i];
+      }
+      return q != br % P || include_local ? c : 0;
     });
   } else {
     scan_part<1>(n_words, warp - kHalf, kHalf, pos_s, warp_s + kHalf, [&](int i) {
@@ -644,7 +686,8 @@ __global__ void __launch_bounds__(kGatherThreads)
   auto load_next = [&](int st) -> bool {
     while (next < n_blocks) {
       int after = 0;
-      if (lane == 0) after = n_units + atomicAdd(n_taken, 1);
+      if (kFromMask) after = next + n_units;
+      else if (lane == 0) after = n_units + atomicAdd(n_taken, 1);
       for (int full_words = 32; full_words == 32; word += full_words)  // words whose blocks have lower numbers
         full_words = __popc(__ballot_sync(0xffffffffu, word + lane < n_words && pos_s[word + lane + 1] <= next));
       uint32_t left = live_s[word];
@@ -709,13 +752,17 @@ int launch_demand_pack(const sparsp_shape& s, const Geometry& g, const uint32_t*
   const int64_t T = (int64_t)g.B * P * P * g.H, tile_bytes = 2LL * g.b * g.d;
   const int n_copy = pack_warps((int)tile_bytes);
   const int64_t n_words = (int64_t)g.B * g.H * g.Wd;
-  const int64_t smem = n_copy * kGatherStages * 2 * tile_bytes + (T + 1 + 2 * n_words + 1 + (int64_t)P * g.Wd) * 4;
+  int64_t smem = n_copy * kGatherStages * 2 * tile_bytes + (T + 1 + 2 * n_words + 1 + (int64_t)P * g.Wd) * 4;
+  const bool from_mask = n_words * g.NB <= kMaskMax && (int64_t)g.B * g.H * g.NB <= kFromMaskBlocks * 148 * n_copy &&
+                         smem + n_words * P * 4 <= kGatherSmem;
   PackLaunch c;
   if (T <= kScanMax && smem <= kGatherSmem) {
-    if ((rc = prepare_pack(s, g, K, V, (const void*)gather_kernel, (int)smem, &c)) != SPARSP_OK) return rc;
+    auto kern = from_mask ? gather_kernel<true> : gather_kernel<false>;
+    if (from_mask) smem += n_words * P * 4;
+    if ((rc = prepare_pack(s, g, K, V, (const void*)kern, (int)smem, &c)) != SPARSP_OK) return rc;
     int32_t* n_taken = (int32_t*)(ws + L.n_entries);  // zeroed by the union's launch
-    SPARSP_CUDA_OK(launch_union(g, mask, rank, P, local, U, cnt, nullptr, n_taken, st));
-    SPARSP_CUDA_OK(launch_kernel(gather_kernel, c.grid, kGatherThreads, (size_t)smem, st, c.tk, c.tv, U, rank, cnt, g.B,
+    if (!from_mask) SPARSP_CUDA_OK(launch_union(g, mask, rank, P, local, U, cnt, nullptr, n_taken, st));
+    SPARSP_CUDA_OK(launch_kernel(kern, c.grid, kGatherThreads, (size_t)smem, st, c.tk, c.tv, mask, U, rank, cnt, g.B,
                                  g.H, g.NB, g.Wd, P, local, g.b, c.tile_bytes, n_copy, seg_off, seg_total, volume,
                                  dst_base, capacity, (unsigned char*)packed, n_taken, status));
     return SPARSP_OK;
