@@ -71,6 +71,11 @@ struct AttnParams {
   const int64_t* tile_base;
   const int32_t* rank;  // packed source: owner of every block, and the rank whose rows are computed
   int consumer;
+  // kPackedDirect: what slot and tile_base are made of
+  int P;
+  const uint32_t* U;
+  const int64_t *seg_off, *seg_total, *dst_base;
+  int64_t tile_bytes;
   __nv_bfloat16* O;
   float* lse;
   int32_t* status;
@@ -162,9 +167,12 @@ struct Entry<true> {
 // z = query blocks, first | second << 16 (0xffff: none); w = batch.
 constexpr int kHeadEntries = 0xffff, kHeadRagged = 1 << 16, kHeadRefShift = 17, kHeadNoneShift = 19;
 
-// Where items and their K / V tiles come from: a queue of items and the sequence's own K and V; the same, but every query
-// block has a CTA of its own and is its item (64-token blocks: not stacked); a queue and a consumer's packed buffer.
-enum class Source { kQueue, kDirect, kPacked };
+// Where items and their K / V tiles come from.
+//   kQueue         a queue of items made by the preparatory launch, the sequence's own K and V
+//   kDirect        the same K and V, but every query block has a CTA of its own and is its item (64-token blocks: not stacked)
+//   kPacked        a queue of the consumer's items, a packed buffer and the consumer's own K and V
+//   kPackedDirect  the same tiles, but the CTAs number the consumer's items and places in the buffer for themselves
+enum class Source { kQueue, kDirect, kPacked, kPackedDirect };
 
 template <int D, int BLK>
 struct AttnCfg {
@@ -203,7 +211,11 @@ struct AttnCfg {
   static constexpr int kOffMisc = kOffHead + 16 * kLists;
   static constexpr int kTotal = kOffMisc + 64;
   static constexpr int kDynamic = kTotal + 1024;  // slack for the 1024-byte alignment of the base
-  static_assert(kDynamic <= 232448, "shared memory budget");
+  // kPackedDirect: uint32 own[P][Wd], int32 first[P][Wd] (places of a head's blocks), uint32 union[32], uint8 rank[1024]
+  static constexpr int kOffOwn = kTotal, kOffFirst = kOffOwn + kMaxRanks * kMaxWords * 4;
+  static constexpr int kOffUnion = kOffFirst + kMaxRanks * kMaxWords * 4, kOffRank = kOffUnion + kMaxWords * 4;
+  static constexpr int kDynamicDirect = kOffRank + kMaxBlocks + 1024;
+  static_assert(kDynamicDirect <= 232448, "shared memory budget");
 };
 
 // Packed fp32 pairs (one instruction for two lanes' worth of fused multiply-add / add).
@@ -294,7 +306,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmP,
                     const AttnParams p) {
   using C = AttnCfg<D, BLK>;
-  constexpr bool kPacked = kSource == Source::kPacked, kDirect = kSource == Source::kDirect;
+  constexpr bool kDirect = kSource == Source::kDirect, kPackedDirect = kSource == Source::kPackedDirect;
+  constexpr bool kPacked = kSource == Source::kPacked || kPackedDirect;
   constexpr int SV = C::kStagesV;
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem =
@@ -382,7 +395,29 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     tmem_alloc(s_tmem, kTmemCols);
     tmem_relinquish();
   }
-  enter_grid();  // (barriers, tensor memory and constants are set up while the preparatory launch still runs)
+  enter_grid();  // (barriers, tensor memory and constants are set up while the launch before still runs)
+  uint32_t* sOwn = reinterpret_cast<uint32_t*>(smem + C::kOffOwn);
+  uint8_t* sRank = smem + C::kOffRank;
+  if constexpr (kPackedDirect) {
+    constexpr int kWarps = kAttnThreads / 32, kRounds = kMaxWords / kWarps;
+    int rk[kRounds];
+#pragma unroll
+    for (int t = 0; t < kRounds; ++t) {
+      const int j = (warp + t * kWarps) * 32 + lane;
+      rk[t] = j < p.NB ? p.rank[j] : -1;
+    }
+#pragma unroll
+    for (int t = 0; t < kRounds; ++t) {
+      const int w = warp + t * kWarps;
+      if (w < p.Wd) {
+        sRank[w * 32 + lane] = (uint8_t)((unsigned)rk[t] < (unsigned)p.P ? rk[t] : 0xff);
+        for (int r = 0; r < p.P; ++r) {
+          const uint32_t word = __ballot_sync(0xffffffffu, rk[t] == r);
+          if (lane == 0) sOwn[r * p.Wd + w] = word;
+        }
+      }
+    }
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -585,7 +620,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         }
         h_end += hbase;
       };
-      if (kPacked) load_heads();
+      if (kSource == Source::kPacked) load_heads();
+      // kPackedDirect: the consumer's blocks, a word per lane, and how many of them lie in lower words
+      uint32_t own = 0u;
+      int n_own = 0, own_before = 0, number = 0, first_of = -1, base_of = -1, own_base = 0;
+      if constexpr (kPackedDirect) {
+        own = lane < p.Wd ? sOwn[p.consumer * p.Wd + lane] : 0u;
+        own_before = bits_below(own, lane, &n_own);
+      }
+      auto own_block = [&](int x) {  // the consumer's x-th block
+        const int w = 31 - __clz(__ballot_sync(0xffffffffu, own != 0u && own_before <= x));
+        uint32_t left = __shfl_sync(0xffffffffu, own, w);
+        for (int skip = x - __shfl_sync(0xffffffffu, own_before, w); skip > 0; --skip) left &= left - 1u;
+        return w * 32 + __ffs(left) - 1;
+      };
       int bh = p.BH, blk0 = -1, blk1 = -1;
       const int ragged_block = p.N % BLK ? p.NB - 1 : -1;
       uint32_t rb0 = 0u, rb1 = 0u;  // the item's mask rows, a word per lane (NB <= 1024: at most 32 words)
@@ -602,6 +650,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           if (bh < p.BH) load_rows();
           if (!__any_sync(0xffffffffu, rb0 != 0u)) bh = p.BH;
           return;
+        }
+        if constexpr (kPackedDirect) {  // every gridDim.x-th one; those that keep nothing are left out
+          const int per_head = (n_own + C::kEPT - 1) / C::kEPT;
+          for (number = it;; number += (int)gridDim.x) {
+            bh = per_head > 0 ? min(number / per_head, p.BH) : p.BH;
+            if (bh >= p.BH) return;
+            const int x = (number - bh * per_head) * C::kEPT;
+            blk0 = own_block(x);
+            blk1 = C::kStacked && x + 1 < n_own ? own_block(x + 1) : -1;
+            load_rows();
+            if (__any_sync(0xffffffffu, (rb0 | rb1) != 0u)) return;
+          }
         }
         int x;
         if (kPacked) {
@@ -635,6 +695,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       };
       auto next_item = [&]() {
         if (kDirect) return p.BH * p.NB;
+        if (kPackedDirect) return number + (int)gridDim.x;
         int it = 0;
         if (lane == 0) it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
         return __shfl_sync(0xffffffffu, it, 0);
@@ -673,7 +734,39 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         }
         EntT* ent = sEnt + buf * kMaxBlocks;
         const int batch = bh / p.H;
-        const int tile_base = kPacked ? (int)p.tile_base[batch] : 0;
+        if constexpr (kPackedDirect) {
+          if (batch != base_of) {  // the consumer's first tile
+            const int64_t br = (int64_t)batch * p.P + p.consumer;
+            int64_t first = 0;
+            if (p.dst_base) {
+              first = p.dst_base[br] / p.tile_bytes;
+            } else {
+              for (int64_t t = lane; t < br; t += 32) first += 2 * p.seg_total[t];
+#pragma unroll
+              for (int s = 16; s >= 1; s >>= 1) first += __shfl_xor_sync(0xffffffffu, first, s);
+            }
+            own_base = (int)first;
+            base_of = batch;
+          }
+          if (bh != first_of) {  // places of the head's blocks: of every producer, the entries before each word's
+            const int64_t br = (int64_t)batch * p.P + p.consumer, h = bh - batch * p.H;
+            const uint32_t u = lane < p.Wd ? p.U[(br * p.H + h) * p.Wd + lane] : 0u;
+            const int64_t* off = p.seg_off + br * p.P * p.H + h;
+            const int o0 = lane < p.P ? (int)off[(int64_t)lane * p.H] : 0;
+            const int o1 = lane + 32 < p.P ? (int)off[(int64_t)(lane + 32) * p.H] : 0;
+            int32_t* first = reinterpret_cast<int32_t*>(smem + C::kOffFirst);
+            for (int r = 0; r < p.P; ++r) {
+              int total;
+              const int below = bits_below(lane < p.Wd ? u & sOwn[r * p.Wd + lane] : 0u, lane, &total);
+              const int o = __shfl_sync(0xffffffffu, r < 32 ? o0 : o1, r & 31);
+              if (lane < p.Wd) first[r * p.Wd + lane] = o + below;
+            }
+            if (lane < p.Wd) reinterpret_cast<uint32_t*>(smem + C::kOffUnion)[lane] = u;
+            __syncwarp();
+            first_of = bh;
+          }
+        }
+        const int tile_base = kPackedDirect ? own_base : kPacked ? (int)p.tile_base[batch] : 0;
         // Entry order (any order gives the same attention).  Blocks BOTH query blocks keep make full tiles; a
         // block only the first keeps is put next to a block only the second keeps, so that such a tile costs
         // every softmax row one 64-key half instead of costing half of the rows two.  A full tile is bound by
@@ -774,13 +867,24 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (C::kStacked && (running & 1) && lane == 0) ent[running] = 0;
         if constexpr (kPacked) {  // where the entries' blocks are, a lane per entry, two loads in flight
           const int32_t* slot = p.slot + (int64_t)bh * p.NB;
+          auto slot_of = [&](int j) -> int32_t {
+            if constexpr (kPackedDirect) {
+              const int r = sRank[j], w = j >> 5;
+              if (r >= p.P || r == p.consumer) return -1;
+              const uint32_t set = reinterpret_cast<const uint32_t*>(smem + C::kOffUnion)[w] & sOwn[r * p.Wd + w];
+              if (!((set >> (j & 31)) & 1u)) return -1;
+              return reinterpret_cast<const int32_t*>(smem + C::kOffFirst)[r * p.Wd + w] + __popc(set & ((1u << (j & 31)) - 1u));
+            } else {
+              return slot[j];
+            }
+          };
           auto placed_at = [&](uint32_t v, int32_t sl) {
             return sl < 0 ? v : (v & ~E::kValue) | E::kRemote | ((uint32_t)(tile_base + 2 * sl) & E::kValue);
           };
           for (int e = lane; e < running; e += 64) {
             const bool two = e + 32 < running;
             const uint32_t v1 = ent[e], v2 = two ? ent[e + 32] : v1;
-            const int32_t s1 = slot[v1 & (kMaxBlocks - 1)], s2 = slot[v2 & (kMaxBlocks - 1)];
+            const int32_t s1 = slot_of(v1 & (kMaxBlocks - 1)), s2 = slot_of(v2 & (kMaxBlocks - 1));
             ent[e] = placed_at(v1, s1);
             if (two) ent[e + 32] = placed_at(v2, s2);
           }
@@ -1500,13 +1604,13 @@ static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q
   if ((rc = make_tile_tmap(&tq, Q, s, g, BLK, true)) != SPARSP_OK) return rc;
   if ((rc = make_tile_tmap(&tk, K, s, g, BLK, true)) != SPARSP_OK) return rc;
   if ((rc = make_tile_tmap(&tv, V, s, g, BLK, true)) != SPARSP_OK) return rc;
-  if (kSource == Source::kPacked) {
+  if (kSource == Source::kPacked || kSource == Source::kPackedDirect) {
     if ((rc = make_packed_tmap(&tp, packed, packed_capacity, g)) != SPARSP_OK) return rc;
   } else {
     tp = tk;  // never used
   }
   auto kern = attn_fwd_kernel<D, BLK, kSource>;
-  const int smem = AttnCfg<D, BLK>::kDynamic;
+  const int smem = kSource == Source::kPackedDirect ? AttnCfg<D, BLK>::kDynamicDirect : AttnCfg<D, BLK>::kDynamic;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
   // work item = one 128-row Q tile (a 128-token block, a pair of 64-token blocks, or one of them); one persistent CTA per SM
   const int64_t most = (int64_t)g.B * g.H * (BLK == 128 || kSource == Source::kDirect ? g.NB : (g.NB + 1) / 2);
@@ -1597,6 +1701,27 @@ int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, 
                        const int64_t* seg_off, const int64_t* seg_total, const void* packed, int64_t capacity,
                        const int64_t* dst_base, float scale, void* O, float* lse, char* ws, const WsLayout& L,
                        cudaStream_t st) {
+  AttnParams p = {};
+  p.mask = mask;
+  p.rank = rank;
+  p.consumer = consumer;
+  // Where the consumer has hardly more items than there are SMs (if it has its share of the blocks; otherwise the CTAs just
+  // take more of them), their order and a queue are worth less than the launch that makes them: us a call over a whole
+  // buffer, with the launch / without, 1 head x 43 blocks, 5 ranks 18.5 / 16.4; 4 x 97 of 64 x 128, 8 ranks 20.0 / 17.9; 8 x 128,
+  // 4 ranks (1.7 items an SM) 37.6 / 33.4; 9 hops of 6 x 140 with all that belongs to them 238 / 214.  With 2.2 items an SM it
+  // depends: 80.5 / 77.3 for a whole buffer of 10 x 128, but 222 / 227 for its hops, half of whose items are empty.
+  int sms = 0;
+  SPARSP_CUDA_OK(sm_count(&sms));
+  const int64_t blocks = (g.NB + P - 1) / P, per_item = 128 / g.b;
+  if ((int64_t)g.B * g.H * ((blocks + per_item - 1) / per_item) <= 2 * sms) {
+    p.P = P;
+    p.U = U;
+    p.seg_off = seg_off;
+    p.seg_total = seg_total;
+    p.dst_base = dst_base;
+    p.tile_bytes = (int64_t)g.b * g.d * 2;
+    return launch_attn_common<Source::kPackedDirect>(s, g, Q, K, V, packed, capacity, p, scale, O, lse, ws, L, st);
+  }
   PrepParams pre = prep_params(g, mask, ws, L);
   pre.rank = rank;
   pre.U = U;
@@ -1610,14 +1735,10 @@ int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, 
   pre.consumer = consumer;
   const int rc = launch_prep<true>(g, pre, st);
   if (rc != SPARSP_OK) return rc;
-  AttnParams p = {};
-  p.mask = mask;
   p.pairs = pre.pairs;
   p.n_items = pre.n_items;
   p.slot = pre.slot;
   p.tile_base = pre.tile_base;
-  p.rank = rank;
-  p.consumer = consumer;
   return launch_attn_common<Source::kPacked>(s, g, Q, K, V, packed, capacity, p, scale, O, lse, ws, L, st);
 }
 
