@@ -11,7 +11,8 @@ namespace sparsp {
 // hop[b][h][i][w] = (rank[i] == consumer and head_begin <= h < head_end) ? mask[b][h][i][w] & own_producer[w] : 0.
 // A lane handles one word of kHopRows rows (rows of fewer than 32 words share a warp); the producer's ownership words
 // and the consumer's rows are bits in shared memory, built once per CTA.  A mask is a few MB, so this is latency: 40
-// heads x 591 rows x 19 words in 6.2 us (11.3 us with a thread per word that walked 32 ranks for its ownership bits).
+// heads x 591 rows x 19 words in 5.0 us (11.3 us with a thread per word that walked 32 ranks for its ownership bits, 7.5 with
+// a pass over the ranks for each of the two sets, 6.5 with eight rows a lane).
 constexpr int kHopThreads = 256;
 constexpr int kHopRows = 4;
 
@@ -22,10 +23,26 @@ __global__ void __launch_bounds__(kHopThreads) hop_mask_kernel(const uint32_t* _
                                                                uint32_t* __restrict__ hop) {
   enter_grid(mask, rank);
   __shared__ uint32_t own_s[kMaxWords], row_s[kMaxWords];
-  rank_words(rank, NB, producer, own_s);
-  rank_words(rank, NB, consumer, row_s);
-  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  {
+    constexpr int kLooks = kMaxWords / (kHopThreads / 32);  // words a warp looks at, all loads in flight
+    int owner[kLooks];
+#pragma unroll
+    for (int t = 0; t < kLooks; ++t) {
+      const int j = (warp + t * (kHopThreads / 32)) * 32 + lane;
+      owner[t] = j < NB ? rank[j] : -1;
+    }
+#pragma unroll
+    for (int t = 0; t < kLooks; ++t) {
+      const uint32_t own = __ballot_sync(0xffffffffu, owner[t] == producer);
+      const uint32_t row = __ballot_sync(0xffffffffu, owner[t] == consumer);
+      if (lane == 0) {
+        own_s[warp + t * (kHopThreads / 32)] = own;
+        row_s[warp + t * (kHopThreads / 32)] = row;
+      }
+    }
+  }
+  __syncthreads();
   int width = 1;  // lanes per row: the next power of two
   while (width < Wd) width <<= 1;
   const int per_warp = 32 / width, w = lane & (width - 1), sub = lane / width;
