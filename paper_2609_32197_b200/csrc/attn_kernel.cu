@@ -15,28 +15,36 @@
 // 306 / 282; 40 x 75600, 59 tiles, 10.05 / 9.82 ms; one hop of it over 8 ranks, 2 to 8 tiles, 64.1 / 61.1.  Tried on top and
 // no better: rows through shared memory and a TMA store, lists for one or two items more, tiles dealt so that the
 // warpgroups take turns at writing.)
-// The scores S = Q K^T are double-buffered in tensor memory (S: 2 x 128 fp32 columns; P: 64 columns of packed bf16,
-// two buffers at d = 64, one at d = 128 where 16 columns hold the row sums instead; O: d columns), so that the tensor pipe always has the next
-// tiles' MMAs queued while the softmax of the current tile runs: Q K^T of tile g+2 starts as soon as the
-// scores of tile g have been READ, and P V of tile g is issued as soon as P_g is written.  Tiles are
-// numbered g = 0, 1, 2, ... across the CTA's items; every ring, buffer and barrier phase follows g.
-// Warp roles (512 threads = 4 warpgroups; the first two hand most of their registers to the other two):
+// Every softmax warpgroup has a buffer of its own for scores S = Q K^T in tensor memory (128 fp32 columns), so that the tensor
+// pipe always has the next tiles' MMAs queued while the softmax of the current tile runs.  Tiles are numbered g = 0, 1, 2, ...
+// across the CTA's items; every ring, buffer and barrier phase follows g.
+//   d = 128: two warpgroups.  S 2 x 128 columns, P 64 columns of packed bf16, O 128 columns, 16 columns for the row sums.
+//            Q K^T of tile g+2 starts as soon as the scores of tile g have been READ.  A tile moves 160 KB through shared memory
+//            (64 KB of TMA writes, 96 KB of operands), 1250 clocks at 128 bytes a clock; ordinary tiles take 1400.
+//   d = 64:  three warpgroups.  A tile is half of that and its 16384 exponentials bound it, with two warps a scheduler more by
+//            their latencies (1495 clocks) than by the special-function unit (683), so there is a third one.  S 3 x 128
+//            columns, P in the place of the scores it was made from, O 64 + 16 columns; Q K^T of tile g+3 starts when P V of
+//            tile g has read P.  Two warpgroups with P buffers of their own / three: 13 heads x 2 x 6034 tokens 78.7 / 76.0 us
+//            a call, 48 x 17776 1380 / 1321, 16 x 18600 with threshold lists 282 / 258, 27 x 27403 from a packed buffer 279 / 244.
+// P V of tile g is issued as soon as P_g is written.
+// Warp roles (512 or 640 threads = 4 or 5 warpgroups; the first two hand most of their registers to the others):
 //   warp 0      TMA producer of Q (per item) and K, which share a ring of buffers
 //   warp 1      issues every Q K^T          warp 2      issues every P V
 //   warp 3      TMA producer of the V ring
 //   warp 4      builds the kept / union list of the NEXT items (two list buffers)
 //   warps 5-7   clear the output rows of query blocks that keep nothing
-//   warps 8-11  softmax of the even tiles   warps 12-15 softmax of the odd tiles
+//   warps 8-    softmax: warpgroup w of kWGs takes the tiles with g % kWGs = w
 // (A producer is one thread running a chain of dependent instructions next to busy softmax warps: it gets
 // an instruction issued every ~8 cycles, so K and V loads have a warp each and keep per-tile work minimal.)
-// A softmax thread owns one query row of its tile: the whole 128-column row of S sits in registers.  Ordinary items run
+// A softmax thread owns one query row of its tile: at d = 128 the whole 128-column row of S sits in registers, at d = 64, with
+// fewer registers a thread, 32 columns and the next 32 on their way.  Ordinary items run
 // without a row maximum: load scores -> exponentials -> store P, relative to 0 (K / V source) or to the row's maximum
-// over the item's first tile (packed source), which the warpgroup of that tile hands to the other one; the tensor pipe
+// over the item's first tile (packed source), which the warpgroup of that tile hands to the others; the tensor pipe
 // takes the row sums.  Whether that was right is seen from the finished row sums and the exponents on the way, and an
 // item that left the range is computed again (kRefZero ... below).  Only such an item, and rows whose first scores are out
-// of range, take their maxima as they go: the two threads that own the same row (one per warpgroup) then share the reference
-// through shared memory and take their decisions strictly in tile order (two mbarriers per row group hand the turn back and
-// forth), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since the reference last moved --
+// of range, take their maxima as they go: the threads that own the same row (one per warpgroup) then share the reference
+// through shared memory and take their decisions strictly in tile order (mbarriers of the row group hand the turn from one to
+// the next), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since the reference last moved --
 // the thread that decides so first waits for every P V issued so far.
 // (The range used to be proved beforehand, by Cauchy-Schwarz from key norms that a pass over K took ahead of every call
 // and row norms taken from the Q tile of every item, and not at all for a packed source, whose tiles all took their
@@ -88,9 +96,8 @@ struct AttnParams {
   long long wait_limit;
 };
 
-constexpr int kAttnThreads = 512;  // four warpgroups: two of utility warps, softmax of the even tiles, softmax of the odd tiles
-// register budget per thread after the warpgroups re-balance (2*128*48 + 256*208 = 512*128; nothing spills in the softmax
-// warps, and the list builder, which spilled with 32, hardly does)
+// register budget per thread after the warpgroups re-balance (d = 128: 256 * 48 + 256 * 208 = 512 * 128; d = 64: 256 * 48 + 384 *
+// 128 = 640 * 96, which is what a block of 640 threads is launched with; hardly anything spills)
 #ifndef SPARSP_REGS_UTILITY
 #define SPARSP_REGS_UTILITY 48
 #define SPARSP_REGS_UTILITY2 48
@@ -180,7 +187,6 @@ struct AttnCfg {
   static constexpr int kEPT = 128 / BLK;         // kept-list entries per 128-key KV tile
   static constexpr int kStagesK = (D == 64) ? 4 : 3;
   static constexpr int kStagesV = (D == 64) ? 4 : 2;
-  static constexpr int kQBytes = 128 * D * 2;
   static constexpr int kTileBytes = 128 * D * 2;  // one K or V tile
   // Q tile and K ring share kStagesK + 1 buffers: an item's Q tile takes the next buffer of the ring for as long as the item
   // lasts, the buffer of the item before it joins the ring behind (QKRing).
@@ -197,14 +203,20 @@ struct AttnCfg {
   // keys against a [16 keys][column 0 = 1] block (2 KB, 128-byte swizzle like a V box), into 16 tensor-memory columns
   // of its own -- which exist only if P keeps ONE buffer instead of two (tensor memory is full otherwise)
   static constexpr bool kSum128 = (D == 128);
-  static constexpr int kNumP = kSum128 ? 1 : 2;
+  // Softmax warpgroups, each of which takes every kWGs-th tile and has an S buffer.  Three: P takes the place of the scores it
+  // was made from.  Two: one P buffer for both.
+  static constexpr int kWGs = D == 64 ? 3 : 2;
+  static constexpr bool kInPlaceP = kWGs == 3;
+  static constexpr int kThreads = (2 + kWGs) * 128;  // two warpgroups of utility warps before them
+  static constexpr int kRegsSoftmax = kWGs == 3 ? 128 : SPARSP_REGS_SOFTMAX;
+  static constexpr int kListReaders = 4 + 4 * kWGs;  // two producers, two issuers, the softmax warps
   static constexpr int kOffOnes = kOffV + kStagesV * kTileBytes;  // bf16 [128][64], 128-byte swizzle like a V box
   static constexpr int kOffEnt = kOffOnes + (kOnes ? 128 * 128 : 2048);  // entries [kLists][1024]
   static constexpr int kOffRef = kOffEnt + kLists * kMaxBlocks * 4;  // float [4 items][128] reference per row
   static constexpr int kOffBars = kOffRef + 4 * 128 * 4;
-  static constexpr int kNumBars = 2 * (kBufsQK + kStagesV) + 10 + 1 + 2 * kLists + 4 + 8 + 1;
-  static constexpr int kColS = 0;    // S buffers: columns [0, 256)
-  static constexpr int kColP = 256;  // P: two buffers in columns [256, 384), or one in [256, 320) with the row sums in [320, 336)
+  static constexpr int kNumBars = 2 * (kBufsQK + kStagesV) + 3 * kWGs + 4 + 1 + 2 * kLists + 4 + 8 * kWGs + 1;
+  static constexpr int kColS = 0;    // S buffers: 128 columns each
+  static constexpr int kColP = 256;  // d = 128: P in columns [256, 320), row sums in [320, 336)
   static constexpr int kColO = 384;  // accumulator: columns [384, 384 + d)
   static constexpr int kColL = kOnes ? kColO + D : 320;  // row sums (column 0 of 16), where the tensor pipe takes them
   static constexpr int kOffHead = (kOffBars + 8 * kNumBars + 15) / 16 * 16;  // int4 [kLists]
@@ -301,7 +313,7 @@ __device__ __forceinline__ void clear_rows(const AttnParams& p, int bh, int i) {
 }
 
 template <int D, int BLK, Source kSource>
-__global__ void __launch_bounds__(kAttnThreads, 1)
+__global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
     attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmP,
                     const AttnParams p) {
@@ -324,30 +336,30 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   uint64_t* v_full = qk_empty + C::kBufsQK;
   uint64_t* v_empty = v_full + SV;
   uint64_t* s_full = v_empty + SV;  // [2] S buffer written by a Q K^T
-  uint64_t* s_free = s_full + 2;    // [2] S buffer read into registers by its 4 softmax warps
-  uint64_t* p_full = s_free + 2;    // [2] P of an even / odd tile written by its 4 softmax warps
-  // [4] the P V of tile g arrives on o_full[g % 4].  Four barriers, because a parity wait can only tell the
-  // phase a barrier is in from the one before: a softmax thread that wants P V g-1 or g-2 has itself seen
-  // P V g-4 complete, and P V g+2 cannot complete before that thread has stored P_g.
-  uint64_t* o_full = p_full + 2;
+  uint64_t* s_free = s_full + C::kWGs;  // [kWGs] S buffer read into registers by its 4 softmax warps (not where P takes its place)
+  uint64_t* p_full = s_free + C::kWGs;  // [kWGs] P of a tile written by its 4 softmax warps
+  // [4] the P V of tile g arrives on o_full[g % 4].  Four barriers, because a parity wait can only tell the phase a barrier is
+  // in from the one before.  d = 128: a softmax thread that wants P V g-1 has itself seen P V g-3 complete, and P V g+2 cannot
+  // complete before that thread has stored P_g.  d = 64: P V g-3 was complete when the Q K^T whose scores it holds was issued.
+  uint64_t* o_full = p_full + C::kWGs;
   uint64_t* o_drained = o_full + 4;      // the item's accumulator has been read out by the four warps that write it
   uint64_t* list_ready = o_drained + 1;  // [kLists] list buffer filled
   uint64_t* list_free = list_ready + kLists;  // [kLists] list buffer no longer needed by its kListReaders
   // [4] the four warps that own an item's first tile have left what it says in s_exact and, if that is the reference, in
-  // sRef.  Four, because the other warpgroup, which waits for it, may be up to three tiles and as many items behind.
+  // sRef.  Four, because a warpgroup that waits for it may be up to three tiles and as many items behind.
   uint64_t* ref_ready = list_free + kLists;
-  // [2][4] the warpgroup's warp of a row group has decided about the running maximum of a tile.  (Not named barriers, which
+  // [2][kWGs][4] the warpgroup's warp of a row group has decided about the running maximum of a tile.  Two in turn, because it may
+  // decide about the first tile of the next item before the warp behind it has noticed.  (Not named barriers, which
   // cannot be bounded: after a wait that has run out two warps need not agree on who takes turns.  Every lane arrives: with
   // one lane behind a __syncwarp and the count of waits in shared memory 13 heads x 2 x 6034, Q times 8, took 138 us, not 132.)
   uint64_t* turn = ref_ready + 4;
-  uint64_t* placed = turn + 8;     // in-place calls: the eight softmax warps know whether the item is to be computed again
+  uint64_t* placed = turn + 8 * C::kWGs;  // in-place calls: all softmax warps know whether the item is to be computed again
   int4* s_head = reinterpret_cast<int4*>(smem + C::kOffHead);  // [kLists] item headers
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
   // [4 items][4 row groups] the group's rows take the running maximum
   volatile uint8_t* s_exact = reinterpret_cast<volatile uint8_t*>(smem + C::kOffMisc + 16);
   volatile int* s_failed = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 32);  // [kLists] the item is to be computed again
-  constexpr int kListReaders = 12;  // two producers, two issuers, eight softmax warps
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -364,20 +376,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       mbar_init(v_full + s, 1);
       mbar_init(v_empty + s, 1);
     }
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < C::kWGs; ++s) {
       mbar_init(s_full + s, 1);
       mbar_init(s_free + s, 4);
       mbar_init(p_full + s, 4);
     }
     for (int s = 0; s < kLists; ++s) {
       mbar_init(list_ready + s, 1);
-      mbar_init(list_free + s, kListReaders);
+      mbar_init(list_free + s, C::kListReaders);
     }
     for (int s = 0; s < 4; ++s) mbar_init(o_full + s, 1);
     mbar_init(o_drained, 4);
     for (int s = 0; s < 4; ++s) mbar_init(ref_ready + s, 4);
-    for (int s = 0; s < 8; ++s) mbar_init(turn + s, 32);
-    mbar_init(placed, 8);
+    for (int s = 0; s < 8 * C::kWGs; ++s) mbar_init(turn + s, 32);
+    mbar_init(placed, 4 * C::kWGs);
     mbar_init_fence();
     *s_abort = 0;
   }
@@ -385,7 +397,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     // key row r holds column 64 + c at byte r*128 + ((c/8 ^ (r & 7)) << 4) + (c%8)*2 (the swizzle of a TMA box);
     // 128 key rows at d = 64 (one block for a whole tile), 16 at d = 128 (every group of 16 keys uses the same)
     uint4* ones = reinterpret_cast<uint4*>(smem + C::kOffOnes);
-    for (int idx = tid; idx < (C::kOnes ? 128 : 16) * 8; idx += kAttnThreads) {
+    for (int idx = tid; idx < (C::kOnes ? 128 : 16) * 8; idx += C::kThreads) {
       const int r = idx >> 3, chunk = idx & 7;
       ones[idx] = make_uint4(chunk == (r & 7) ? 0x3F80u : 0u, 0u, 0u, 0u);  // bf16 1.0 in element 0 of logical chunk 0
     }
@@ -399,7 +411,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   uint32_t* sOwn = reinterpret_cast<uint32_t*>(smem + C::kOffOwn);
   uint8_t* sRank = smem + C::kOffRank;
   if constexpr (kPackedDirect) {
-    constexpr int kWarps = kAttnThreads / 32, kRounds = kMaxWords / kWarps;
+    constexpr int kWarps = C::kThreads / 32, kRounds = (kMaxWords + kWarps - 1) / kWarps;
     int rk[kRounds];
 #pragma unroll
     for (int t = 0; t < kRounds; ++t) {
@@ -423,7 +435,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
 
-  // the utility warpgroup hands most of its registers to the two softmax warpgroups (the re-balancing
+  // the utility warpgroups hand most of their registers to the softmax warpgroups (the re-balancing
   // instruction sits inside each role's branch so that the register allocator sees which code runs
   // under which limit)
   if (warp < 4) {
@@ -519,7 +531,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll
       for (int kk = 0; kk < D / 16; ++kk) lo[kk] = (uint32_t)desc0 + (uint32_t)(((kk / 4) * 16384 + (kk % 4) * 32) >> 4);
       QKRing<C::kStagesK> at;
-      int g = 0;
+      int g = 0, w = 0;     // tiles so far, the next one's warpgroup
+      uint32_t round = 0u;  // parity of that warpgroup's tiles so far
       for (int i = 0;; ++i) {
         const int buf = i % kLists;
         mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 53, p.wait_limit);
@@ -532,20 +545,30 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         for (int n = 0; n < n_tiles; ++n, ++g) {
           const uint32_t bk = at.next_k();
           mbar_wait_bounded_inline(qk_full + bk, at.use(bk), s_abort, 12, p.wait_limit);
-          // S buffer g%2 is free once the softmax warps have loaded the scores of tile g-2
-          if (g >= 2) mbar_wait_bounded_inline(s_free + (g & 1), ((g - 2) >> 1) & 1, s_abort, 24, p.wait_limit);
+          // an S buffer is free once its warpgroup has loaded the scores of its tile before, or the P V has read the P that
+          // took their place
+          if (g >= C::kWGs) {
+            if (C::kInPlaceP)
+              mbar_wait_bounded_inline(o_full + ((g - C::kWGs) & 3), ((g - C::kWGs) >> 2) & 1, s_abort, 24, p.wait_limit);
+            else
+              mbar_wait_bounded_inline(s_free + w, round ^ 1u, s_abort, 24, p.wait_limit);
+          }
           tc_fence_after();
           const uint32_t k_off = bk * (C::kTileBytes >> 4);
-          const uint32_t tS = tmem_base + C::kColS + (g & 1) * 128;
+          const uint32_t tS = tmem_base + C::kColS + w * 128;
           if (leader) {
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
               mma_ss_lohi(tS, lo[kk] + q_off, hi, lo[kk] + k_off, hi, kIdescQK, kk > 0 ? 1u : 0u);
-            mma_commit(s_full + (g & 1));
+            mma_commit(s_full + w);
             mma_commit(qk_empty + bk);
             if (n == n_tiles - 1) mma_commit(qk_empty + bq);
           }
           __syncwarp();
+          if (++w == C::kWGs) {
+            w = 0;
+            round ^= 1u;
+          }
         }
         if (lane == 0) mbar_arrive(list_free + buf);
         __syncwarp();
@@ -565,7 +588,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       constexpr uint32_t kIdescSum = make_idesc_bf16(128, 16, 0, 1);
       const uint64_t descOnes = make_smem_desc(smem_u32(smem + C::kOffOnes), 16384u, 1024);
       const uint32_t tL = tmem_base + C::kColL;
-      int g = 0;
+      int g = 0, w = 0;
+      uint32_t round = 0u;
       for (int i = 0;; ++i) {
         const int buf = i % kLists;
         mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 54, p.wait_limit);
@@ -575,12 +599,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         // the previous item's accumulator must have been read out before this item's first P V overwrites it
         if (i > 0) mbar_wait_bounded_inline(o_drained, (i - 1) & 1, s_abort, 55, p.wait_limit);
         for (int n = 0; n < n_tiles; ++n, ++g) {
-          mbar_wait_bounded_inline(p_full + (g & 1), (g >> 1) & 1, s_abort, 20, p.wait_limit);
+          mbar_wait_bounded_inline(p_full + w, round, s_abort, 20, p.wait_limit);
           mbar_wait_bounded_inline(v_full + g % SV, (g / SV) & 1, s_abort, 22, p.wait_limit);
           tc_fence_after();
           uint32_t stage_off = (uint32_t)(((g % SV) * C::kTileBytes) >> 4);
           if (C::kOnes) stage_off -= stage_off << 16;  // start address up, distance to the ones block down
-          const uint32_t tP = tmem_base + C::kColP + (C::kNumP == 2 ? (g & 1) * 64 : 0);
+          const uint32_t tP = tmem_base + (C::kInPlaceP ? C::kColS + w * 128 : C::kColP);
           if (leader) {
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {
@@ -593,6 +617,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             mma_commit(v_empty + g % SV);
           }
           __syncwarp();
+          if (++w == C::kWGs) {
+            w = 0;
+            round ^= 1u;
+          }
         }
         if (lane == 0) mbar_arrive(list_free + buf);
         __syncwarp();
@@ -926,19 +954,21 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       }
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SPARSP_REGS_SOFTMAX));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsSoftmax));
     // ================================ softmax warpgroups ==================================
-    const int wg = (warp >> 2) - 2;  // 0: even tiles g, 1: odd tiles; also the S (and, where there are two, P) buffer this warpgroup uses
+    const int wg = (warp >> 2) - 2;  // takes the tiles with g % kWGs = wg, in S buffer wg
     const int rgrp = warp & 3;       // tensor-memory lane group this warp may access
     const int row = rgrp * 32 + lane;
     const int rh = row >> 6;         // which query block of a stacked Q tile the row belongs to
     const uint32_t lane_off = (uint32_t)(rgrp * 32) << 16;
     const uint32_t tS = tmem_base + C::kColS + wg * 128 + lane_off;
-    const uint32_t tP = tmem_base + C::kColP + (C::kNumP == 2 ? wg * 64 : 0) + lane_off;
+    const uint32_t tP = C::kInPlaceP ? tS : tmem_base + C::kColP + lane_off;
     const uint32_t tO = tmem_base + C::kColO + lane_off;
-    const int mine = wg * 4 + rgrp, other = (1 - wg) * 4 + rgrp;  // the two warps of a row group
-    int g0 = 0;       // number of the item's first tile
-    int turns = 0;    // waits for the other warp of the row group so far
+    // the warps of a row group: mine, and the one that takes the tiles before mine
+    const int mine = wg * 4 + rgrp, before = (wg == 0 ? C::kWGs - 1 : wg - 1) * 4 + rgrp;
+    int g0 = 0, w0 = 0;     // number of the item's first tile, its warpgroup
+    uint32_t round = 0u;    // parity of my tiles so far
+    int turns = 0, given = 0;  // turns taken over from the warp before and handed to the one behind so far
     for (int i = 0;; ++i) {
       const int buf = i % kLists;
       mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 56, p.wait_limit);
@@ -946,7 +976,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       if (hd.y == 0) break;
       const int n_ent = hd.y & kHeadEntries;
       const int n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
-      const int first = (wg - g0) & 1;  // my first tile
+      const int first = wg >= w0 ? wg - w0 : wg - w0 + C::kWGs;  // my first tile
       const int ref_of = (hd.y >> kHeadRefShift) & 3;
       const EntT* ent = sEnt + buf * kMaxBlocks;
       const bool item_ragged = (hd.y & kHeadRagged) != 0;
@@ -960,9 +990,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         if (ref_of == kRefFirst && !exact) m_ref = ref[row];
       };
       auto take_turn = [&]() {  // the other warp has decided about the tile before, and may have moved the reference
-        mbar_wait_bounded_inline(turn + other, turns++ & 1, s_abort, 44, p.wait_limit);
+        mbar_wait_bounded_inline(turn + before + (turns & 1) * 4 * C::kWGs, (turns >> 1) & 1, s_abort, 44, p.wait_limit);
+        ++turns;
         m_ref = ref[row];
       };
+      auto give_turn = [&]() { mbar_arrive(turn + mine + (given++ & 1) * 4 * C::kWGs); };
       // the row's largest score of a tile: one flat instruction stream per 64-key half, an absent half (not kept by this
       // row's query block) is skipped
       auto row_max = [&](const float* sv, const int* vh) {
@@ -1010,12 +1042,239 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         }
       };
 
+      // the row's reference follows its running maximum; the accumulator is rescaled
+      auto move_ref = [&](const float mx, const int n) {
+        const int g = g0 + n;
+        const float m_new = fmaxf(m_ref, mx);
+        const bool grow = m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY);
+        if (__any_sync(0xffffffffu, grow)) {
+          const float alpha = grow ? ex2(m_ref - m_new) : 1.0f;  // m_ref = -inf -> 0
+          if (n > 0) {
+            // every P V of the item issued so far must have landed in O before the row is rescaled; they
+            // complete in order, so the one of tile g-1 suffices
+            mbar_wait_bounded_inline(o_full + ((g - 1) & 3), ((g - 1) >> 2) & 1, s_abort, 38, p.wait_limit);
+            tc_fence_after();
+#pragma unroll 1
+            for (int c = 0; c < C::kAccCols / 16; ++c) {  // the row's accumulator, 16 columns at a time (rare: kept small)
+              uint32_t o[16];
+              tmem_ld16(tO + c * 16, o);
+              tmem_ld_wait();
+#pragma unroll
+              for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+              tmem_st16(tO + c * 16, o);
+            }
+            if (C::kSum128) {  // the row sums live in columns of their own
+              uint32_t o[16];
+              tmem_ld16(tmem_base + C::kColL + lane_off, o);
+              tmem_ld_wait();
+#pragma unroll
+              for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+              tmem_st16(tmem_base + C::kColL + lane_off, o);
+            }
+            tmem_st_wait();
+            tc_fence_before();
+          }
+          if (grow) {
+            m_ref = m_new;
+            ref[row] = m_new;
+          }
+        }
+      };
+      // A tile whose P takes the place of its scores: 32 columns at a time, the next ones on their way from tensor memory.
+      auto in_place_tile = [&](auto ragged_tag, auto exact_tag, const int n, const int* vh) {
+        constexpr bool kRagged = decltype(ragged_tag)::value, kExact = decltype(exact_tag)::value;
+        float va[32], vb[32];
+        auto load = [&](float(&v)[32], const int q) { tmem_ld32(tS + q * 32, reinterpret_cast<uint32_t*>(v)); };
+        auto loaded = [&](float(&v)[32]) {  // nothing of v is looked at ahead of the wait before this
+#pragma unroll
+          for (int e = 0; e < 32; ++e) asm volatile("" : "+f"(v[e]));
+        };
+        auto cut = [&](float(&v)[32], const int q) {  // columns past the end of the sequence count as -inf
+          if (kRagged && vh[q >> 1] < 64) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] = (q & 1) * 32 + e < vh[q >> 1] ? v[e] : -INFINITY;
+          }
+        };
+        if (kExact || n == 0) {  // a look at the whole tile first
+          float mx = -INFINITY, most = 0.0f;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (vh[q >> 1] > 0) {
+              load(va, q);
+              tmem_ld_wait();
+              cut(va, q);
+              if (kExact || ((kRagged || kPacked) && ref_of == kRefFirst)) {
+                float m0 = va[0], m1 = va[1];
+#pragma unroll
+                for (int e = 2; e < 32; e += 2) {
+                  m0 = fmaxf(m0, va[e]);
+                  m1 = fmaxf(m1, va[e + 1]);
+                }
+                mx = fmaxf(mx, fmaxf(m0, m1));
+              } else {
+#pragma unroll
+                for (int e = 0; e < 32; e += 16) most = max_abs3(va[e], va[e + 8], most);
+              }
+            }
+          }
+          mx *= p.scale_log2;
+          if (kExact) {
+            if (n > 0) take_turn();
+            move_ref(mx, n);
+            if (n == 0 && m_ref == -INFINITY) ref[row] = m_ref;
+            if (n + 1 < n_tiles) give_turn();
+          } else {
+            if ((kRagged || kPacked) && ref_of == kRefFirst) {
+              m_ref = mx > -INFINITY ? mx : 0.0f;  // (keeps nothing of this tile, or is no number)
+              ref[row] = m_ref;
+              exact = __any_sync(0xffffffffu, !(fabsf(m_ref) <= kFirstSample));
+            } else {
+              exact = __any_sync(0xffffffffu, !(most * p.scale_log2 <= kZeroSample));
+            }
+            if (exact) m_ref = -INFINITY;
+            __syncwarp();
+            if (lane == 0) {
+              s_exact[(i & 3) * 4 + rgrp] = exact ? 1 : 0;
+              mbar_arrive(ref_ready + (i & 3));
+            }
+          }
+        } else if (n < C::kWGs) {
+          learn_ref();
+        }
+        if (!kExact && n < C::kWGs && exact) return;  // the variant with the turns takes the tile
+        const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nm2 = make_float2(-m_ref, -m_ref);
+        auto exponentials = [&](float(&v)[32], const int q) {
+          uint32_t pk[16];
+          cut(v, q);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const float2 x = ffma2(make_float2(v[2 * e], v[2 * e + 1]), sc2, nm2);
+            constexpr int kPoly = SPARSP_TUNE_POLY_D64;
+            const float2 pp = (kPoly > 0 && (((q & 1) * 16 + e) % (kPoly > 0 ? kPoly : 1)) == 1)
+                                  ? exp2_poly2<kRagged || kExact, !kExact>(x, &i_max)
+                                  : make_float2(ex2(x.x), ex2(x.y));
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(pp.x, pp.y);
+            pk[e] = *reinterpret_cast<const uint32_t*>(&h2);
+          }
+          if (kRagged && vh[q >> 1] < 64) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              const int c = (q & 1) * 32 + 2 * e;
+              pk[e] = c + 1 < vh[q >> 1] ? pk[e] : (c < vh[q >> 1] ? (pk[e] & 0xffffu) : 0u);
+            }
+          }
+          tmem_st16(tP + q * 16, pk);
+        };
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (vh[h] > 0) {
+            load(va, 2 * h);
+            tmem_ld_wait();
+            load(vb, 2 * h + 1);
+            exponentials(va, 2 * h);
+            tmem_ld_wait();
+            loaded(vb);
+            exponentials(vb, 2 * h + 1);
+          } else {
+            uint32_t none[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) none[e] = 0u;
+            tmem_st16(tP + 2 * h * 16, none);
+            tmem_st16(tP + (2 * h + 1) * 16, none);
+          }
+        }
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(p_full + wg);
+        round ^= 1u;
+      };
+
+      // A tile whose P goes to a buffer of its own: the whole row of scores in registers, the S buffer is free at once.
+      auto own_buffer_tile = [&](auto ragged_tag, auto exact_tag, const int n, const int* vh) {
+        constexpr bool kRagged = decltype(ragged_tag)::value, kExact = decltype(exact_tag)::value;
+        const int g = g0 + n;
+        float sv[128];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, reinterpret_cast<uint32_t*>(sv) + c * 32);
+        tmem_ld_wait();
+        if (kRagged) {
+          // the sequence ends inside this tile: columns past the end count as -inf
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (vh[h] > 0 && vh[h] < 64) {
+#pragma unroll
+              for (int e = 0; e < 64; ++e) sv[h * 64 + e] = e < vh[h] ? sv[h * 64 + e] : -INFINITY;
+            }
+          }
+        }
+        if (!kExact && n < C::kWGs) {
+          if (n == 0) look_at_first(ragged_tag, sv, vh);
+          else learn_ref();
+          if (exact) return;  // the variant with the turns takes the tile
+        }
+        // S is in registers: the Q K^T of tile g+2 may overwrite the buffer
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(s_free + wg);
+
+        if (kExact) {
+          const float mx = row_max(sv, vh);
+          // ---- my turn to look at / move the row's reference maximum (strictly in tile order) ----
+          if (n > 0) take_turn();
+          move_ref(mx, n);
+          if (n == 0 && m_ref == -INFINITY) ref[row] = m_ref;
+          if (n + 1 < n_tiles) give_turn();
+        }
+
+        // exponentials of keys [64h, 64h+64) -> packed bf16 columns [32h, 32h+32) of the P buffer
+        uint32_t pk[64];
+        const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nm2 = make_float2(-m_ref, -m_ref);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float* svh = sv + h * 64;
+          uint32_t* pkh = pk + h * 32;
+          if (vh[h] > 0) {  // then the row has a finite reference
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+              const float2 x = ffma2(make_float2(svh[2 * e], svh[2 * e + 1]), sc2, nm2);
+              constexpr int kPoly = kPacked && BLK == 128 ? SPARSP_TUNE_POLY_HOP : SPARSP_TUNE_POLY;
+              const float2 pp = (kPoly > 0 && (e % (kPoly > 0 ? kPoly : 1)) == 1)
+                                    ? exp2_poly2<kRagged || kExact, !kExact>(x, &i_max)
+                                    : make_float2(ex2(x.x), ex2(x.y));
+              const __nv_bfloat162 h2 = __floats2bfloat162_rn(pp.x, pp.y);
+              pkh[e] = *reinterpret_cast<const uint32_t*>(&h2);
+            }
+            if (kRagged && vh[h] < 64) {
+              // columns past the end of the sequence: exactly zero in P (the polynomial path returns
+              // 2^-126 for them, which the row sum may keep)
+#pragma unroll
+              for (int e = 0; e < 32; ++e) pkh[e] = 2 * e + 1 < vh[h] ? pkh[e] : (2 * e < vh[h] ? (pkh[e] & 0xffffu) : 0u);
+            }
+          } else {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) pkh[e] = 0u;
+          }
+        }
+        // the P buffer was last read by the P V of tile g-1
+        if (g >= 1) {
+          mbar_wait_bounded_inline(o_full + ((g - 1) & 3), ((g - 1) >> 2) & 1, s_abort, 34 + wg, p.wait_limit);
+          tc_fence_after();
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tmem_st16(tP + c * 16, pk + c * 16);
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(p_full + wg);
+        round ^= 1u;
+      };
+
       // One tile of this warpgroup.  kRagged = the sequence ends inside the tile (possible only for the item's last one), or
       // (K / V source) the reference comes from the first tile and this is it: that variant carries the column masking;
       // kExact: the one with the turns.  The common variant stays small.
       auto do_tile = [&](auto ragged_tag, auto exact_tag, const int n) {
-        constexpr bool kRagged = decltype(ragged_tag)::value, kExact = decltype(exact_tag)::value;
-        const int g = g0 + n;
+        constexpr bool kRagged = decltype(ragged_tag)::value;
         // kept / valid key columns of each 64-column half of the tile (warp-uniform), as the list builder left them
         int vh[2];
         if (C::kStacked) {
@@ -1043,136 +1302,30 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             vh[1] = max(valid - 64, 0);
           }
         }
-        mbar_wait_bounded_inline(s_full + wg, (g >> 1) & 1, s_abort, 30 + wg, p.wait_limit);
+        mbar_wait_bounded_inline(s_full + wg, round, s_abort, 30 + wg, p.wait_limit);
         tc_fence_after();
-        float sv[128];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, reinterpret_cast<uint32_t*>(sv) + c * 32);
-        tmem_ld_wait();
-        if (kRagged) {
-          // the sequence ends inside this tile: columns past the end count as -inf
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            if (vh[h] > 0 && vh[h] < 64) {
-#pragma unroll
-              for (int e = 0; e < 64; ++e) sv[h * 64 + e] = e < vh[h] ? sv[h * 64 + e] : -INFINITY;
-            }
-          }
-        }
-        if (!kExact && n <= 1) {
-          if (n == 0) look_at_first(ragged_tag, sv, vh);
-          else learn_ref();
-          if (exact) return;  // the variant with the turns takes the tile
-        }
-        // S is in registers: the Q K^T of tile g+2 may overwrite the buffer
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(s_free + wg);
-
-        if (kExact) {
-          const float mx = row_max(sv, vh);
-          // ---- my turn to look at / move the row's reference maximum (strictly in tile order) ----
-          if (n > 0) take_turn();
-          const float m_new = fmaxf(m_ref, mx);
-          const bool grow = m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY);
-          if (__any_sync(0xffffffffu, grow)) {
-            const float alpha = grow ? ex2(m_ref - m_new) : 1.0f;  // m_ref = -inf -> 0
-            if (n > 0) {
-              // every P V of the item issued so far must have landed in O before the row is rescaled; they
-              // complete in order, so the one of tile g-1 suffices
-              mbar_wait_bounded_inline(o_full + ((g - 1) & 3), ((g - 1) >> 2) & 1, s_abort, 38, p.wait_limit);
-              tc_fence_after();
-#pragma unroll 1
-              for (int c = 0; c < C::kAccCols / 16; ++c) {  // the row's accumulator, 16 columns at a time (rare: kept small)
-                uint32_t o[16];
-                tmem_ld16(tO + c * 16, o);
-                tmem_ld_wait();
-#pragma unroll
-                for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                tmem_st16(tO + c * 16, o);
-              }
-              if (C::kSum128) {  // the row sums live in columns of their own
-                uint32_t o[16];
-                tmem_ld16(tmem_base + C::kColL + lane_off, o);
-                tmem_ld_wait();
-#pragma unroll
-                for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                tmem_st16(tmem_base + C::kColL + lane_off, o);
-              }
-              tmem_st_wait();
-              tc_fence_before();
-            }
-            if (grow) {
-              m_ref = m_new;
-              ref[row] = m_new;
-            }
-          }
-          if (n == 0 && m_ref == -INFINITY) ref[row] = m_ref;
-          mbar_arrive(turn + mine);
-        }
-
-        // exponentials of keys [64h, 64h+64) -> packed bf16 columns [32h, 32h+32) of the P buffer
-        uint32_t pk[64];
-        const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nm2 = make_float2(-m_ref, -m_ref);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float* svh = sv + h * 64;
-          uint32_t* pkh = pk + h * 32;
-          if (vh[h] > 0) {  // then the row has a finite reference
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              const float2 x = ffma2(make_float2(svh[2 * e], svh[2 * e + 1]), sc2, nm2);
-              constexpr int kPoly = D == 64 ? SPARSP_TUNE_POLY_D64 : kPacked && BLK == 128 ? SPARSP_TUNE_POLY_HOP : SPARSP_TUNE_POLY;
-              const float2 pp = (kPoly > 0 && (e % (kPoly > 0 ? kPoly : 1)) == 1)
-                                    ? exp2_poly2<kRagged || kExact, !kExact>(x, &i_max)
-                                    : make_float2(ex2(x.x), ex2(x.y));
-              const __nv_bfloat162 h2 = __floats2bfloat162_rn(pp.x, pp.y);
-              pkh[e] = *reinterpret_cast<const uint32_t*>(&h2);
-            }
-            if (kRagged && vh[h] < 64) {
-              // columns past the end of the sequence: exactly zero in P (the polynomial path returns
-              // 2^-126 for them, which the row sum may keep)
-#pragma unroll
-              for (int e = 0; e < 32; ++e) pkh[e] = 2 * e + 1 < vh[h] ? pkh[e] : (2 * e < vh[h] ? (pkh[e] & 0xffffu) : 0u);
-            }
-          } else {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) pkh[e] = 0u;
-          }
-        }
-        // my P buffer was last read by the P V of tile g-2; a single P buffer by that of tile g-1
-        constexpr int kBack = C::kNumP == 2 ? 2 : 1;
-        if (g >= kBack) {
-          mbar_wait_bounded_inline(o_full + ((g - kBack) & 3), ((g - kBack) >> 2) & 1, s_abort, 34 + wg, p.wait_limit);
-          tc_fence_after();
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_st16(tP + c * 16, pk + c * 16);
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(p_full + wg);
+        if constexpr (C::kInPlaceP) in_place_tile(ragged_tag, exact_tag, n, vh);
+        else own_buffer_tile(ragged_tag, exact_tag, n, vh);
       };
       if (exact && first == 0 && lane == 0) mbar_arrive(ref_ready + (i & 3));  // (nothing to learn: the barriers keep step)
       int n = first;
       // the list builder puts the sequence's last block (the only one that can be ragged) into the last tile
       const int n_rag = item_ragged ? n_tiles - 1 : -1;
       if (!exact) {
-        for (; n < n_tiles; n += 2) {
-          if (n == n_rag || (!kPacked && ref_of == kRefFirst && n <= 1)) do_tile(std::true_type{}, std::false_type{}, n);
+        for (; n < n_tiles; n += C::kWGs) {
+          if (n == n_rag || (!kPacked && ref_of == kRefFirst && n < C::kWGs)) do_tile(std::true_type{}, std::false_type{}, n);
           else do_tile(std::false_type{}, std::false_type{}, n);
           if (exact) break;  // what the first tile says
         }
       }
       if (exact)
-        for (; n < n_tiles; n += 2) do_tile(std::true_type{}, std::true_type{}, n);
+        for (; n < n_tiles; n += C::kWGs) do_tile(std::true_type{}, std::true_type{}, n);
 
       g0 += n_tiles;
+      w0 = (w0 + n_tiles) % C::kWGs;
       // ---- item epilogue: the warpgroup of the item's last tile writes the rows, the other one goes on ----
-      if (first >= n_tiles && ref_of != kRefExact) learn_ref();
       const int last = g0 - 1;
-      if ((last & 1) != wg) {
-        if (exact) take_turn();  // (the last tile was the other warp's)
+      if ((w0 == 0 ? C::kWGs - 1 : w0 - 1) != wg) {
         if (__any_sync(0xffffffffu, !exact && !(i_max <= kMaxExponent)) && lane == 0) s_failed[buf] = 1;
         __syncwarp();
         if (p.in_place) {
@@ -1617,7 +1770,20 @@ static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
   const unsigned grid = (unsigned)std::min<int64_t>(most, sms);
-  SPARSP_CUDA_OK(launch_kernel(kern, grid, kAttnThreads, smem, st, tq, tk, tv, tp, p));
+  // The warpgroups share out the registers that the block is launched with; should a build of the kernel be given fewer, some
+  // of them would wait for good.
+  constexpr int kShared = 128 * (SPARSP_REGS_UTILITY + SPARSP_REGS_UTILITY2 + AttnCfg<D, BLK>::kWGs * AttnCfg<D, BLK>::kRegsSoftmax);
+  static std::atomic<int> launched_with{0};
+  if (launched_with.load(std::memory_order_relaxed) < kShared) {
+    cudaFuncAttributes attr;
+    SPARSP_CUDA_OK(cudaFuncGetAttributes(&attr, (const void*)kern));
+    launched_with.store(attr.numRegs * AttnCfg<D, BLK>::kThreads, std::memory_order_relaxed);
+    if (attr.numRegs * AttnCfg<D, BLK>::kThreads < kShared) {
+      set_error("the attention kernel was built with %d registers a thread: too few to share out", attr.numRegs);
+      return SPARSP_ERR_UNSUPPORTED;
+    }
+  }
+  SPARSP_CUDA_OK(launch_kernel(kern, grid, AttnCfg<D, BLK>::kThreads, smem, st, tq, tk, tv, tp, p));
   return SPARSP_OK;
 }
 
