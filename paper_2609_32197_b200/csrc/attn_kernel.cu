@@ -1421,13 +1421,13 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
 // tile's work is masked away.
 // Packed source: neighbours in the consumer's ascending list of blocks (D = 1), so that a row's result depends on its
 // neighbour's list at most, not on what the consumer's other blocks keep.
-// (Mask rows in shared memory have an odd pitch: the threads' offsets differ by one row, a pitch of 32 words would put
-// them all on one bank.)
+// (Mask rows in shared memory have a pitch of an odd number of 16-byte units, which are read whole: the threads' offsets differ
+// by one row, an even pitch would put many of them on the same banks.)
 // Items of one (batch, head) are handed out longest list first: the items still running when the queue
 // runs dry are then the short ones, which matters when list lengths vary (threshold selection, unions of two
 // stacked blocks).  Key = (list length << 10) | (1023 - index): equal lengths keep their index order.
 // Latency-bound integer work, so what matters is how many loads and barriers wait for each other: rows are counted by a
-// warp each with eight in flight, up to 256 items are put in order without rounds, offsets are scored by all threads, and
+// warp each with sixteen in flight, items are put in order without rounds, offsets are scored by all threads, and
 // slots have CTAs of their own and no shared-memory atomics.  One hop of 40 heads x 591 blocks, 8 ranks 5.9 us (23 with
 // 256 threads, a thread per row, a bitonic sort for any number and the slots behind the items), 24 x 384 stacked blocks
 // 15.5, 2 x 64 4.5 (attention calls 72 -> 66-74, 617 -> 594 and 21.2 -> 19.4 us).
@@ -1453,7 +1453,7 @@ struct PrepParams {
   int P, consumer;
 };
 
-// Sorts n keys (n a power of two, <= 1024; distinct but for zeros) in shared memory into descending order; all threads call it.
+// Sorts n keys (n a power of two, <= 1024) in shared memory by length, the longest first; all threads call it.
 __device__ __forceinline__ void sort_keys_descending(uint32_t* keys, int n) {
   if (n <= kPrepThreads / 2) {
     // Few keys: a key's place is the number of larger ones, counted by two threads.  No rounds that wait for each other.
@@ -1470,21 +1470,55 @@ __device__ __forceinline__ void sort_keys_descending(uint32_t* keys, int n) {
     __syncthreads();
     return;
   }
-  for (int k = 2; k <= n; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < n; t += kPrepThreads) {
-        const int u = t ^ j;
-        if (u > t) {
-          const uint32_t a = keys[t], b = keys[u];
-          if (((t & k) == 0) ? a < b : a > b) {
-            keys[t] = b;
-            keys[u] = a;
-          }
-        }
-      }
-      __syncthreads();
-    }
+  // Many keys: a place for every length, by counting; equal lengths in any order, a warp's together.
+  constexpr int kLens = kMaxBlocks + 1, kPer = (kLens + kPrepThreads - 1) / kPrepThreads, kWarps = kPrepThreads / 32;
+  constexpr int kKeys = kMaxBlocks / kPrepThreads;
+  __shared__ int at_s[kPer * kPrepThreads], sum_s[kWarps];  // place kLens - 1 - length: keys of that length, then where they begin
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int t = 0; t < kPer; ++t) at_s[threadIdx.x + t * kPrepThreads] = 0;
+  uint32_t key[kKeys], peers[kKeys];
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kKeys; ++t) {
+    const int i = threadIdx.x + t * kPrepThreads;
+    key[t] = i < n ? keys[i] : 0u;
+    peers[t] = __match_any_sync(0xffffffffu, key[t] >> 10);
+    if (lane == __ffs(peers[t]) - 1) atomicAdd(&at_s[kLens - 1 - (key[t] >> 10)], __popc(peers[t]));
   }
+  __syncthreads();
+  int mine[kPer], sum = 0;
+#pragma unroll
+  for (int t = 0; t < kPer; ++t) {
+    mine[t] = at_s[threadIdx.x * kPer + t];
+    sum += mine[t];
+  }
+  int incl = sum;
+#pragma unroll
+  for (int s = 1; s < 32; s <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, s);
+    if (lane >= s) incl += v;
+  }
+  if (lane == 31) sum_s[warp] = incl;
+  __syncthreads();
+  int begin = incl - sum;
+#pragma unroll
+  for (int k = 0; k < kWarps; ++k) begin += k < warp ? sum_s[k] : 0;
+#pragma unroll
+  for (int t = 0; t < kPer; ++t) {
+    at_s[threadIdx.x * kPer + t] = begin;
+    begin += mine[t];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kKeys; ++t) {
+    const int leader = __ffs(peers[t]) - 1;
+    int place = 0;
+    if (lane == leader) place = atomicAdd(&at_s[kLens - 1 - (key[t] >> 10)], __popc(peers[t]));
+    place = __shfl_sync(0xffffffffu, place, leader) + __popc(peers[t] & ((1u << lane) - 1u));
+    if (place < n) keys[place] = key[t];
+  }
+  __syncthreads();
 }
 
 __device__ __forceinline__ int next_pow2(int n) {
@@ -1506,13 +1540,36 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
   int n_keys;
   bool live = false;  // any of my keys is an item's
   if (p.b == 64) {
-    uint32_t* m = reinterpret_cast<uint32_t*>(smem_raw);  // [n][pitch]
-    const int Wd = p.Wd, pitch = Wd | 1;
+    uint32_t* m = reinterpret_cast<uint32_t*>(smem_raw);  // [n][pitch], zeros behind a row's words
+    const uint4* m4 = reinterpret_cast<const uint4*>(smem_raw);
+    const int Wd = p.Wd, units = (Wd + 3) / 4, pitch4 = units | 1, pitch = 4 * pitch4;
     if (threadIdx.x == 0) s_best = 1023u - 1u;  // default D = 1
-    for (int idx = threadIdx.x; idx < n * Wd; idx += kPrepThreads) {
-      const int i = idx / Wd, w = idx - i * Wd;
-      m[i * pitch + w] = rows[(int64_t)block(i) * Wd + w];
+    for (int i = threadIdx.x; i < n; i += kPrepThreads)
+      for (int w = Wd; w < 4 * units; ++w) m[i * pitch + w] = 0u;
+    constexpr int kFlight = 8;
+    for (int idx0 = threadIdx.x; idx0 < n * Wd; idx0 += kFlight * kPrepThreads) {
+      uint32_t v[kFlight];
+      int at[kFlight];
+#pragma unroll
+      for (int u = 0; u < kFlight; ++u) {
+        const int idx = idx0 + u * kPrepThreads, i = idx / Wd, w = idx - i * Wd;
+        at[u] = idx < n * Wd ? i * pitch + w : -1;
+        v[u] = at[u] >= 0 ? rows[(int64_t)block(i) * Wd + w] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < kFlight; ++u)
+        if (at[u] >= 0) m[at[u]] = v[u];
     }
+    // bits that two rows share, or that either has
+    auto common = [&](int a, int b2, bool either) {
+      int bits = 0;
+      for (int u = 0; u < units; ++u) {
+        const uint4 x = m4[a * pitch4 + u], y = m4[b2 * pitch4 + u];
+        bits += either ? __popc(x.x | y.x) + __popc(x.y | y.y) + __popc(x.z | y.z) + __popc(x.w | y.w)
+                       : __popc(x.x & y.x) + __popc(x.y & y.y) + __popc(x.z & y.z) + __popc(x.w & y.w);
+      }
+      return bits;
+    };
     __syncthreads();
     if (!list && n > 1) {
       const int n_off = n / 2, parts = max(1, kPrepThreads / n_off);  // threads per offset
@@ -1523,7 +1580,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
         unsigned int score = 0;
         // every kPairSample-th row is enough to rank offsets
         for (int i = part * kPairSample; i + d < n; i += kPairSample * parts)
-          for (int w = 0; w < Wd; ++w) score += __popc(m[i * pitch + w] & m[(i + d) * pitch + w]);
+          score += (unsigned int)common(i, i + d, false);
         atomicAdd(&s_score[d - 1], score);
       }
       __syncthreads();
@@ -1554,8 +1611,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
       uint32_t key = 0;
       if (c < n_keys) {
         const int a = (int)(s_pair[c] & 0xffffu), b2 = (int)(s_pair[c] >> 16);
-        int len = 0;
-        for (int w = 0; w < Wd; ++w) len += __popc(m[a * pitch + w] | (b2 != 0xffff ? m[b2 * pitch + w] : 0u));
+        const int len = common(a, b2 != 0xffff ? b2 : a, true);
         key = ((uint32_t)len << 10) | (uint32_t)(1023 - c);
       }
       s_keys[c] = key;
@@ -1564,7 +1620,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
   } else {
     // a warp per row, kPrepRows rows of loads in flight
     n_keys = n;
-    constexpr int kPrepRows = 8, kWarps = kPrepThreads / 32;
+    constexpr int kPrepRows = 16, kWarps = kPrepThreads / 32;
     const int lane = threadIdx.x & 31, n_pow2 = next_pow2(n_keys);
     for (int i0 = threadIdx.x >> 5; i0 < n_pow2; i0 += kWarps * kPrepRows) {
       uint32_t v[kPrepRows];
@@ -1816,7 +1872,7 @@ static int launch_attn_common(const sparsp_shape& s, const Geometry& g, const vo
 template <bool kPacked>
 static int launch_prep(const Geometry& g, const PrepParams& p, cudaStream_t st) {
   auto kern = attn_prep_kernel<kPacked>;
-  const int smem = g.b == 64 ? g.NB * (g.Wd | 1) * 4 : 0;
+  const int smem = g.b == 64 ? g.NB * (((g.Wd + 3) / 4) | 1) * 16 : 0;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
   SPARSP_CUDA_OK(launch_kernel(kern, (unsigned)(kPacked ? 2 * p.BH : p.BH), kPrepThreads, smem, st, p));
   return SPARSP_OK;
