@@ -176,10 +176,13 @@ constexpr int kHeadEntries = 0xffff, kHeadRagged = 1 << 16, kHeadRefShift = 17, 
 
 // Where items and their K / V tiles come from.
 //   kQueue         a queue of items made by the preparatory launch, the sequence's own K and V
-//   kDirect        the same K and V, but every query block has a CTA of its own and is its item (64-token blocks: not stacked)
+//   kDirect        the same K and V, but every query block is an item (64-token blocks: not stacked), of which there are so few
+//                  that the CTAs put them in order for themselves
 //   kPacked        a queue of the consumer's items, a packed buffer and the consumer's own K and V
 //   kPackedDirect  the same tiles, but the CTAs number the consumer's items and places in the buffer for themselves
 enum class Source { kQueue, kDirect, kPacked, kPackedDirect };
+
+constexpr int kMaxDirect = 2 * 148;  // items of a call without a queue
 
 template <int D, int BLK>
 struct AttnCfg {
@@ -227,6 +230,8 @@ struct AttnCfg {
   static constexpr int kOffOwn = kTotal, kOffFirst = kOffOwn + kMaxRanks * kMaxWords * 4;
   static constexpr int kOffUnion = kOffFirst + kMaxRanks * kMaxWords * 4, kOffRank = kOffUnion + kMaxWords * 4;
   static constexpr int kDynamicDirect = kOffRank + kMaxBlocks + 1024;
+  // kDirect: uint32 length of every item's list and its number, uint16 items in order
+  static constexpr int kOffLength = kTotal, kOffOrder = kOffLength + 4 * kMaxDirect;
   static_assert(kDynamicDirect <= 232448, "shared memory budget");
 };
 
@@ -410,6 +415,46 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
   enter_grid();  // (barriers, tensor memory and constants are set up while the launch before still runs)
   uint32_t* sOwn = reinterpret_cast<uint32_t*>(smem + C::kOffOwn);
   uint8_t* sRank = smem + C::kOffRank;
+  uint32_t* sLength = reinterpret_cast<uint32_t*>(smem + C::kOffLength);
+  uint16_t* sOrder = reinterpret_cast<uint16_t*>(smem + C::kOffOrder);
+  if constexpr (kDirect) {
+    // More items than CTAs: every CTA puts all of them in order, the longest list first.  A mask row is an item; short rows
+    // share a warp's load.
+    const int n = p.BH * p.NB;
+    if (n > (int)gridDim.x) {
+      int width = 1;  // lanes per row: the next power of two
+      while (width < p.Wd) width <<= 1;
+      const int per_warp = 32 / width, w = lane & (width - 1);
+      constexpr int kFlight = 4, kWarps = C::kThreads / 32;
+      for (int first = warp * per_warp; first < n; first += kFlight * kWarps * per_warp) {  // (the same for all lanes)
+        const int row0 = first + lane / width;
+        uint32_t v[kFlight];
+#pragma unroll
+        for (int u = 0; u < kFlight; ++u) {
+          const int row = row0 + u * kWarps * per_warp;
+          v[u] = row < n && w < p.Wd ? p.mask[(int64_t)row * p.Wd + w] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < kFlight; ++u) {
+          const int row = row0 + u * kWarps * per_warp;
+          int len = __popc(v[u]);
+          for (int s = 1; s < width; s <<= 1) len += __shfl_xor_sync(0xffffffffu, len, s);
+          if (w == 0 && row < n) sLength[row] = (uint32_t)len << 16 | (uint32_t)(0xffff - row);
+        }
+      }
+      if (tid < 4 && n + tid < ((n + 3) & ~3)) sLength[n + tid] = 0u;
+      __syncthreads();
+      for (int t = tid; t < n; t += C::kThreads) {
+        const uint32_t key = sLength[t];
+        int place = 0;
+        for (int k = 0; k < (n + 3) / 4; ++k) {
+          const uint4 x = reinterpret_cast<const uint4*>(sLength)[k];
+          place += (x.x > key) + (x.y > key) + (x.z > key) + (x.w > key);
+        }
+        sOrder[place] = (uint16_t)t;
+      }
+    }
+  }
   if constexpr (kPackedDirect) {
     constexpr int kWarps = C::kThreads / 32, kRounds = (kMaxWords + kWarps - 1) / kWarps;
     int rk[kRounds];
@@ -672,11 +717,14 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         rb1 = lane < p.Wd && blk1 >= 0 ? rows[blk1 * p.Wd + lane] : 0u;
       };
       auto fetch = [&](int it) {
-        if (kDirect) {  // my item is the query block of my number, if it keeps anything
-          bh = it / p.NB;
-          blk0 = it - bh * p.NB;
-          if (bh < p.BH) load_rows();
-          if (!__any_sync(0xffffffffu, rb0 != 0u)) bh = p.BH;
+        if constexpr (kDirect) {  // the CTAs take places in order from the front and from behind in turn
+          bh = p.BH;
+          if (it >= p.BH * p.NB) return;
+          const int item = p.BH * p.NB > (int)gridDim.x ? sOrder[it] : it;
+          bh = item / p.NB;
+          blk0 = item - bh * p.NB;
+          load_rows();
+          if (!__any_sync(0xffffffffu, rb0 != 0u)) bh = p.BH;  // (and so do all behind it)
           return;
         }
         if constexpr (kPackedDirect) {  // every gridDim.x-th one; those that keep nothing are left out
@@ -722,7 +770,10 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         load_rows();
       };
       auto next_item = [&]() {
-        if (kDirect) return p.BH * p.NB;
+        if (kDirect) {
+          const int turn_no = ++number, c = (int)blockIdx.x, G = (int)gridDim.x;
+          return turn_no * G + (turn_no & 1 ? G - 1 - c : c);
+        }
         if (kPackedDirect) return number + (int)gridDim.x;
         int it = 0;
         if (lane == 0) it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
@@ -1819,7 +1870,7 @@ static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q
     tp = tk;  // never used
   }
   auto kern = attn_fwd_kernel<D, BLK, kSource>;
-  const int smem = kSource == Source::kPackedDirect ? AttnCfg<D, BLK>::kDynamicDirect : AttnCfg<D, BLK>::kDynamic;
+  const int smem = kSource == Source::kPackedDirect || kSource == Source::kDirect ? AttnCfg<D, BLK>::kDynamicDirect : AttnCfg<D, BLK>::kDynamic;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
   // work item = one 128-row Q tile (a 128-token block, a pair of 64-token blocks, or one of them); one persistent CTA per SM
   const int64_t most = (int64_t)g.B * g.H * (BLK == 128 || kSource == Source::kDirect ? g.NB : (g.NB + 1) / 2);
@@ -1897,14 +1948,16 @@ int launch_attn(const sparsp_shape& s, const Geometry& g, const void* Q, const v
                 cudaStream_t st) {
   AttnParams p = {};
   p.mask = mask;
-  // Where every query block can have an SM of its own, its CTA needs no queue, no order and no partner for it: one launch.
-  // Two query blocks share a Q tile for the sake of throughput, and alone one is done sooner with its own list than with the
-  // union of two.  (us a call with the launch that makes items, stacked / single / without it: 2 heads x 64 blocks of 64 x 64,
-  // 16 kept 19.4 / 14.9 / 11.5; 7 x 21 of 64 x 128 - / 15.7 / 10.4.  An instance of the kernel of its own, because the
-  // question inside the queue's made 64-token blocks 1-2 % slower.)
+  // Up to two query blocks an SM need no queue and no launch that fills it: every CTA puts them in order for itself and takes
+  // one from the front and one from behind.  Two query blocks share a Q tile for the sake of throughput, and so few are done
+  // sooner each with its own list than with the union of two.  (us a call with the launch that makes items / without it: 2 heads
+  // x 64 blocks of 64 x 64, 16 kept 14.9 / 11.5 (stacked 19.4); 7 x 21 of 64 x 128 15.7 / 10.4; 19 x 9 of 128 x 128 14.5 / 12.0;
+  // 2 x 128 of 128 x 128, 10 % kept 33.5 / 32.1, threshold lists 67 / 54; 2 x 120 of 128 x 64, threshold lists 77 / 52; in order of
+  // their numbers 10.1 for 19 x 9, but 70 and 82 for the last two.  Up to three an SM 0.90 to 1.10 times as fast, up to four 0.80
+  // to 1.04.  An instance of the kernel of its own, because the question inside the queue's made 64-token blocks 1-2 % slower.)
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
-  if ((int64_t)g.B * g.H * g.NB <= sms)
+  if ((int64_t)g.B * g.H * g.NB <= std::min(2 * sms, kMaxDirect))
     return launch_attn_common<Source::kDirect>(s, g, Q, K, V, nullptr, 0, p, scale, O, lse, ws, L, st);
   const PrepParams pre = prep_params(g, mask, ws, L);
   const int rc = launch_prep<false>(g, pre, st);
