@@ -1478,7 +1478,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
 // runs dry are then the short ones, which matters when list lengths vary (threshold selection, unions of two
 // stacked blocks).  Key = (list length << 10) | (1023 - index): equal lengths keep their index order.
 // Latency-bound integer work, so what matters is how many loads and barriers wait for each other: rows are counted by a
-// warp each with sixteen in flight, items are put in order without rounds, offsets are scored by all threads, and
+// warp each with eight in flight, items are put in order without rounds, offsets are scored by all threads, and
 // slots have CTAs of their own and no shared-memory atomics.  One hop of 40 heads x 591 blocks, 8 ranks 5.9 us (23 with
 // 256 threads, a thread per row, a bitonic sort for any number and the slots behind the items), 24 x 384 stacked blocks
 // 15.5, 2 x 64 4.5 (attention calls 72 -> 66-74, 617 -> 594 and 21.2 -> 19.4 us).
@@ -1504,9 +1504,11 @@ struct PrepParams {
   int P, consumer;
 };
 
-// Sorts n keys (n a power of two, <= 1024) in shared memory by length, the longest first; all threads call it.
+// Sorts n keys (n a power of two; up to kPrepThreads / 2, or kMany: 1024) in shared memory by length, the longest first; all threads
+// call it.
+template <bool kMany>
 __device__ __forceinline__ void sort_keys_descending(uint32_t* keys, int n) {
-  if (n <= kPrepThreads / 2) {
+  if constexpr (!kMany) {
     // Few keys: a key's place is the number of larger ones, counted by two threads.  No rounds that wait for each other.
     const int k = threadIdx.x >> 1;
     const uint32_t key = k < n ? keys[k] : 0u;
@@ -1519,57 +1521,57 @@ __device__ __forceinline__ void sort_keys_descending(uint32_t* keys, int n) {
     __syncthreads();
     if (key != 0u && (threadIdx.x & 1) == 0) keys[place] = key;
     __syncthreads();
-    return;
+  } else {
+    // Many keys: a place for every length, by counting; equal lengths in any order, a warp's together.
+    constexpr int kLens = kMaxBlocks + 1, kPer = (kLens + kPrepThreads - 1) / kPrepThreads, kWarps = kPrepThreads / 32;
+    constexpr int kKeys = kMaxBlocks / kPrepThreads;
+    __shared__ int at_s[kPer * kPrepThreads], sum_s[kWarps];  // place kLens - 1 - length: keys of that length, then where they begin
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int t = 0; t < kPer; ++t) at_s[threadIdx.x + t * kPrepThreads] = 0;
+    uint32_t key[kKeys], peers[kKeys];
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kKeys; ++t) {
+      const int i = threadIdx.x + t * kPrepThreads;
+      key[t] = i < n ? keys[i] : 0u;
+      peers[t] = __match_any_sync(0xffffffffu, key[t] >> 10);
+      if (lane == __ffs(peers[t]) - 1) atomicAdd(&at_s[kLens - 1 - (key[t] >> 10)], __popc(peers[t]));
+    }
+    __syncthreads();
+    int mine[kPer], sum = 0;
+#pragma unroll
+    for (int t = 0; t < kPer; ++t) {
+      mine[t] = at_s[threadIdx.x * kPer + t];
+      sum += mine[t];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, s);
+      if (lane >= s) incl += v;
+    }
+    if (lane == 31) sum_s[warp] = incl;
+    __syncthreads();
+    int begin = incl - sum;
+#pragma unroll
+    for (int k = 0; k < kWarps; ++k) begin += k < warp ? sum_s[k] : 0;
+#pragma unroll
+    for (int t = 0; t < kPer; ++t) {
+      at_s[threadIdx.x * kPer + t] = begin;
+      begin += mine[t];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kKeys; ++t) {
+      const int leader = __ffs(peers[t]) - 1;
+      int place = 0;
+      if (lane == leader) place = atomicAdd(&at_s[kLens - 1 - (key[t] >> 10)], __popc(peers[t]));
+      place = __shfl_sync(0xffffffffu, place, leader) + __popc(peers[t] & ((1u << lane) - 1u));
+      if (place < n) keys[place] = key[t];
+    }
+    __syncthreads();
   }
-  // Many keys: a place for every length, by counting; equal lengths in any order, a warp's together.
-  constexpr int kLens = kMaxBlocks + 1, kPer = (kLens + kPrepThreads - 1) / kPrepThreads, kWarps = kPrepThreads / 32;
-  constexpr int kKeys = kMaxBlocks / kPrepThreads;
-  __shared__ int at_s[kPer * kPrepThreads], sum_s[kWarps];  // place kLens - 1 - length: keys of that length, then where they begin
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int t = 0; t < kPer; ++t) at_s[threadIdx.x + t * kPrepThreads] = 0;
-  uint32_t key[kKeys], peers[kKeys];
-  __syncthreads();
-#pragma unroll
-  for (int t = 0; t < kKeys; ++t) {
-    const int i = threadIdx.x + t * kPrepThreads;
-    key[t] = i < n ? keys[i] : 0u;
-    peers[t] = __match_any_sync(0xffffffffu, key[t] >> 10);
-    if (lane == __ffs(peers[t]) - 1) atomicAdd(&at_s[kLens - 1 - (key[t] >> 10)], __popc(peers[t]));
-  }
-  __syncthreads();
-  int mine[kPer], sum = 0;
-#pragma unroll
-  for (int t = 0; t < kPer; ++t) {
-    mine[t] = at_s[threadIdx.x * kPer + t];
-    sum += mine[t];
-  }
-  int incl = sum;
-#pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, s);
-    if (lane >= s) incl += v;
-  }
-  if (lane == 31) sum_s[warp] = incl;
-  __syncthreads();
-  int begin = incl - sum;
-#pragma unroll
-  for (int k = 0; k < kWarps; ++k) begin += k < warp ? sum_s[k] : 0;
-#pragma unroll
-  for (int t = 0; t < kPer; ++t) {
-    at_s[threadIdx.x * kPer + t] = begin;
-    begin += mine[t];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int t = 0; t < kKeys; ++t) {
-    const int leader = __ffs(peers[t]) - 1;
-    int place = 0;
-    if (lane == leader) place = atomicAdd(&at_s[kLens - 1 - (key[t] >> 10)], __popc(peers[t]));
-    place = __shfl_sync(0xffffffffu, place, leader) + __popc(peers[t] & ((1u << lane) - 1u));
-    if (place < n) keys[place] = key[t];
-  }
-  __syncthreads();
 }
 
 __device__ __forceinline__ int next_pow2(int n) {
@@ -1580,6 +1582,7 @@ __device__ __forceinline__ int next_pow2(int n) {
 
 // Work items of one (batch, head) among the n query blocks list[0..n) (packed source; NULL: all blocks, K / V source);
 // returns their number.
+template <bool kStacked, bool kMany>
 __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uint16_t* list, int n,
                                           unsigned char* smem_raw) {
   __shared__ uint32_t s_keys[kMaxBlocks];
@@ -1590,7 +1593,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
   auto block = [&](int pos) -> int { return list ? list[pos] : pos; };
   int n_keys;
   bool live = false;  // any of my keys is an item's
-  if (p.b == 64) {
+  if constexpr (kStacked) {
     uint32_t* m = reinterpret_cast<uint32_t*>(smem_raw);  // [n][pitch], zeros behind a row's words
     const uint4* m4 = reinterpret_cast<const uint4*>(smem_raw);
     const int Wd = p.Wd, units = (Wd + 3) / 4, pitch4 = units | 1, pitch = 4 * pitch4;
@@ -1671,7 +1674,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
   } else {
     // a warp per row, kPrepRows rows of loads in flight
     n_keys = n;
-    constexpr int kPrepRows = 16, kWarps = kPrepThreads / 32;
+    constexpr int kPrepRows = 8, kWarps = kPrepThreads / 32;
     const int lane = threadIdx.x & 31, n_pow2 = next_pow2(n_keys);
     for (int i0 = threadIdx.x >> 5; i0 < n_pow2; i0 += kWarps * kPrepRows) {
       uint32_t v[kPrepRows];
@@ -1689,7 +1692,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
     }
   }
   if (!__syncthreads_or(live)) return 0;
-  sort_keys_descending(s_keys, next_pow2(n_keys));
+  sort_keys_descending<kMany>(s_keys, next_pow2(n_keys));
   int32_t* out = p.pairs + (int64_t)bh * (2 * ((p.NB + 1) / 2));
   int n_live = 0;
   for (int x0 = 0; x0 < n_keys; x0 += kPrepThreads) {
@@ -1697,7 +1700,7 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
     const bool is_item = x < n_keys && (s_keys[x] >> 10) != 0u;
     if (is_item) {
       const int c = 1023 - (int)(s_keys[x] & 1023u);
-      if (p.b == 64) {
+      if (kStacked) {
         const int a = (int)(s_pair[c] & 0xffffu), b2 = (int)(s_pair[c] >> 16);
         out[2 * x] = block(a);
         out[2 * x + 1] = b2 != 0xffff ? block(b2) : -1;
@@ -1749,7 +1752,9 @@ __device__ __forceinline__ void make_slots(const PrepParams& p, int bh) {
   }
 }
 
-template <bool kPacked>
+// (An instance for each form, because the launch waits for the code it is given: with all of it in one, layers of a few thousand
+// tokens took 6 us longer.)
+template <bool kPacked, bool kStacked, bool kMany>
 __global__ void __launch_bounds__(kPrepThreads) attn_prep_kernel(const PrepParams p) {
   enter_grid();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1766,7 +1771,7 @@ __global__ void __launch_bounds__(kPrepThreads) attn_prep_kernel(const PrepParam
     __shared__ uint16_t s_list[kMaxBlocks];
     rank_words(p.rank, p.NB, p.consumer, s_words);
     const int n = list_blocks(s_words, p.NB, s_list);
-    n_live = make_items(p, bh, s_list, n, smem_raw);
+    n_live = make_items<kStacked, kMany>(p, bh, s_list, n, smem_raw);
     if (bh % p.H == 0 && warp == 0) {  // first tile of the consumer's buffer for this batch item
       const int64_t br = (int64_t)(bh / p.H) * p.P + p.consumer;
       int64_t first = 0;
@@ -1780,7 +1785,7 @@ __global__ void __launch_bounds__(kPrepThreads) attn_prep_kernel(const PrepParam
       if (lane == 0) p.tile_base[bh / p.H] = first;
     }
   } else {
-    n_live = make_items(p, bh, nullptr, p.NB, smem_raw);
+    n_live = make_items<kStacked, kMany>(p, bh, nullptr, p.NB, smem_raw);
   }
   if (threadIdx.x == 0) p.n_items[bh] = n_live;
 }
@@ -1922,7 +1927,9 @@ static int launch_attn_common(const sparsp_shape& s, const Geometry& g, const vo
 
 template <bool kPacked>
 static int launch_prep(const Geometry& g, const PrepParams& p, cudaStream_t st) {
-  auto kern = attn_prep_kernel<kPacked>;
+  const bool many = (g.b == 64 ? (g.NB + 1) / 2 : g.NB) > kPrepThreads / 2;
+  auto kern = g.b == 64 ? (many ? attn_prep_kernel<kPacked, true, true> : attn_prep_kernel<kPacked, true, false>)
+                        : (many ? attn_prep_kernel<kPacked, false, true> : attn_prep_kernel<kPacked, false, false>);
   const int smem = g.b == 64 ? g.NB * (((g.Wd + 3) / 4) | 1) * 16 : 0;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
   SPARSP_CUDA_OK(launch_kernel(kern, (unsigned)(kPacked ? 2 * p.BH : p.BH), kPrepThreads, smem, st, p));
