@@ -133,21 +133,16 @@ constexpr float kSafeSumZero = 1.8446744073709552e19f;  // 2^64
 constexpr float kSafeSumFirst = 33554432.0f;            // 2^25: kGrowThreshold and 2^17 keys
 constexpr float kZeroSample = 48.0f, kFirstSample = 64.0f;
 constexpr int kZeroMinTiles = 4;  // K / V source: shorter items take kRefFirst, whose largest terms are exact
-// Tuning switch (compile-time): how many of the exponentials go to the FMA pipe instead of the
-// special-function unit (every n-th pair; 0 = none).  us per attention call with every 3rd / 4th / 6th / none:
-//   d = 128, K / V source    40 heads x 75600, 10 % kept 9884 / 9816 / 9903 / 10596, 24 x 24576 of 64-token blocks with
-//                            threshold lists 671 / 665 / 681 / 690, 2 x 13560 38.9 / 37.8 / 37.8 / 37.3
-//   ... packed source, 128-token blocks (hops: 2 to 8 tiles an item)    62.5 / 61.4 / 61.2 / 60.5; with none lists as long
-//                            as those above would be 5-10 % slower
-//   d = 64                   48 x 17776 1393 / 1410 / 1429 / 1488, 13 x 2 x 6034 77.8 / 80.0 / 79.5 / 84.2, every 2nd 85
+// Tuning switch (compile-time): how many of the exponentials go to the FMA pipe instead of the special-function unit (every
+// n-th pair; 0 = none).  The same share everywhere, so that a row's result does not depend on where its tiles come from.  us
+// per attention call with every 3rd / 4th / 6th pair:
+//   d = 64                   48 heads x 17776 tokens 1393 / 1410 / 1429 (none 1488, every 2nd 3 % slower than every 3rd)
+//   d = 128, 64-token blocks 24 x 24576, half of the blocks kept, neighbours alike 3094 / 3219 / -, 8 x 16384 with all kept 912 /
+//                            948 / -, 24 x 24576 with threshold lists 671 / 665 / 681
+//   ... 128-token blocks     under the power cap a smaller share is up to 1 % faster: 40 x 75600, 10 % kept 9884 / 9816 / 9903
+//                            (none 10596), one hop of it over 8 ranks 60.8 / - / 60.2
 #ifndef SPARSP_TUNE_POLY
-#define SPARSP_TUNE_POLY 4
-#endif
-#ifndef SPARSP_TUNE_POLY_HOP
-#define SPARSP_TUNE_POLY_HOP 6
-#endif
-#ifndef SPARSP_TUNE_POLY_D64
-#define SPARSP_TUNE_POLY_D64 3
+#define SPARSP_TUNE_POLY 3
 #endif
 
 // Lists that the list builder keeps: the current item's and the next one's.  (With 3 or 4 a CTA takes items that one with
@@ -1200,7 +1195,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
             const float2 x = ffma2(make_float2(v[2 * e], v[2 * e + 1]), sc2, nm2);
-            constexpr int kPoly = SPARSP_TUNE_POLY_D64;
+            constexpr int kPoly = SPARSP_TUNE_POLY;
             const float2 pp = (kPoly > 0 && (((q & 1) * 16 + e) % (kPoly > 0 ? kPoly : 1)) == 1)
                                   ? exp2_poly2<kRagged || kExact, !kExact>(x, &i_max)
                                   : make_float2(ex2(x.x), ex2(x.y));
@@ -1289,7 +1284,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
               const float2 x = ffma2(make_float2(svh[2 * e], svh[2 * e + 1]), sc2, nm2);
-              constexpr int kPoly = kPacked && BLK == 128 ? SPARSP_TUNE_POLY_HOP : SPARSP_TUNE_POLY;
+              constexpr int kPoly = SPARSP_TUNE_POLY;
               const float2 pp = (kPoly > 0 && (e % (kPoly > 0 ? kPoly : 1)) == 1)
                                     ? exp2_poly2<kRagged || kExact, !kExact>(x, &i_max)
                                     : make_float2(ex2(x.x), ex2(x.y));
