@@ -168,6 +168,8 @@ struct Entry<true> {
 // Item header, one load for each role: x = batch * H + head; y = entries | kHead... flags (0: there are no more items);
 // z = query blocks, first | second << 16 (0xffff: none); w = batch.
 constexpr int kHeadEntries = 0xffff, kHeadRagged = 1 << 16, kHeadRefShift = 17, kHeadNoneShift = 19;
+// ... and whether all softmax warps meet before the item's rows are written (`placed`), with the parity of that meeting.
+constexpr int kHeadMeet = 1 << 21, kHeadMeetParityShift = 22;
 
 // Where items and their K / V tiles come from.
 //   kQueue         a queue of items made by the preparatory launch, the sequence's own K and V
@@ -353,7 +355,10 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
   // cannot be bounded: after a wait that has run out two warps need not agree on who takes turns.  Every lane arrives: with
   // one lane behind a __syncwarp and the count of waits in shared memory 13 heads x 2 x 6034, Q times 8, took 138 us, not 132.)
   uint64_t* turn = ref_ready + 4;
-  uint64_t* placed = turn + 8 * C::kWGs;  // in-place calls: all softmax warps know whether the item is to be computed again
+  // All softmax warps have come to the end of an item that they meet at.  In-place calls: all items, so that it is known whether
+  // the item is to be computed again.  Else: items that are computed again, so that the rows of the first pass, which another
+  // warpgroup may have written, and written behind its arrival on list_free, come before those of the second.
+  uint64_t* placed = turn + 8 * C::kWGs;
   int4* s_head = reinterpret_cast<int4*>(smem + C::kOffHead);  // [kLists] item headers
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
@@ -777,6 +782,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
       // An item that has failed is handed out again.  Its verdict is there once its list buffer is free: before the buffer is
       // used again, or, when there are no more items, one outstanding item after the other.
       int checked = 0;  // items whose verdict has been seen
+      int meetings = 0;  // items so far whose rows are written behind a meeting
       auto verdict = [&]() -> int {
         const int b = checked % kLists;
         mbar_wait_bounded_inline(list_free + b, (checked / kLists) & 1, s_abort, 50, p.wait_limit);
@@ -966,8 +972,11 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         }
         int ref_of = kPacked || running <= (kZeroMinTiles - 1) * C::kEPT ? kRefFirst : kRefZero;
         if (again >= 0) ref_of = kRefExact;
+        int meet = 0;
+        if (p.in_place || again >= 0) meet = kHeadMeet | (meetings++ & 1) << kHeadMeetParityShift;
         if (lane == 0) {
-          s_head[buf] = make_int4(bh, running | (rag_pos >= 0 ? kHeadRagged : 0) | ref_of << kHeadRefShift | none << kHeadNoneShift,
+          s_head[buf] = make_int4(bh, running | (rag_pos >= 0 ? kHeadRagged : 0) | ref_of << kHeadRefShift |
+                                          none << kHeadNoneShift | meet,
                                   blk0 | (blk1 < 0 ? 0xffff : blk1) << 16, batch);
           s_failed[buf] = 0;
         }
@@ -1374,9 +1383,9 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
       if ((w0 == 0 ? C::kWGs - 1 : w0 - 1) != wg) {
         if (__any_sync(0xffffffffu, !exact && !(i_max <= kMaxExponent)) && lane == 0) s_failed[buf] = 1;
         __syncwarp();
-        if (p.in_place) {
+        if (hd.y & kHeadMeet) {
           if (lane == 0) mbar_arrive(placed);
-          mbar_wait_bounded_inline(placed, i & 1, s_abort, 45, p.wait_limit);
+          mbar_wait_bounded_inline(placed, (hd.y >> kHeadMeetParityShift) & 1, s_abort, 45, p.wait_limit);
         }
         if (lane == 0) mbar_arrive(list_free + buf);
       } else {
@@ -1406,7 +1415,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         // (an ordinary item asks one question here)
         const float safe = ref_of == kRefZero ? kSafeSumZero : kSafeSumFirst;
         const bool asks = !exact && mine_to_write && !(i_max <= kMaxExponent && l >= kMinSum && l <= safe);
-        if (__any_sync(0xffffffffu, asks) || p.in_place) {
+        if (__any_sync(0xffffffffu, asks) || (hd.y & kHeadMeet)) {
           bool failed = asks && !(i_max <= kMaxExponent && l >= kMinSum && l <= kMaxSum);
           if (asks) {
             float most = 0.0f;  // has a column run out of fp32?
@@ -1416,9 +1425,9 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
           }
           if (__any_sync(0xffffffffu, failed) && lane == 0) s_failed[buf] = 1;
           __syncwarp();
-          if (p.in_place) {  // the rows of an item that is computed again are still its queries
+          if (hd.y & kHeadMeet) {  // (in place, the rows of an item that is to be computed again are still its queries)
             if (lane == 0) mbar_arrive(placed);
-            mbar_wait_bounded_inline(placed, i & 1, s_abort, 45, p.wait_limit);
+            mbar_wait_bounded_inline(placed, (hd.y >> kHeadMeetParityShift) & 1, s_abort, 45, p.wait_limit);
             if (s_failed[buf]) mine_to_write = 0;
           }
         }
