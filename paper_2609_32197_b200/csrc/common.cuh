@@ -17,7 +17,6 @@ namespace sparsp {
 constexpr int kMaxBlocks = 1024;  // NB limit (score rows are held in shared memory)
 constexpr int kMaxRanks = 64;
 constexpr int kStatusWords = 64;  // workspace header: word 0 = status code, 1.. = detail
-constexpr int kPlanTicketWord = 16, kPlanTickets = 48;  // words of the header that count a plan's finished CTAs, 0 between launches
 
 struct Geometry {
   int64_t N;         // tokens
@@ -57,22 +56,30 @@ template <typename T>
 struct same_type {
   using type = T;
 };
+// ... in clusters of `cluster` CTAs (the grid is a multiple of it)
 template <typename... P>
-inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
-                                 typename same_type<P>::type... args) {
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+inline cudaError_t launch_clusters(void (*kernel)(P...), dim3 grid, int cluster, int threads, size_t smem, cudaStream_t st,
+                                   typename same_type<P>::type... args) {
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim = {(unsigned)cluster, 1, 1};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
   if (e == cudaSuccess) count_launch();
   return e;
+}
+template <typename... P>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                 typename same_type<P>::type... args) {
+  return launch_clusters(kernel, grid, 1, threads, smem, st, args...);
 }
 
 #ifdef __CUDACC__

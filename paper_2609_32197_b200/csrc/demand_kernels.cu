@@ -19,133 +19,38 @@ namespace sparsp {
 // request, shorter rows share one), so a mask row is read once in all and B*H*P CTAs are in flight; the ownership
 // words are rebuilt per CTA from the rank table.  Latency-bound: the mask is a few MB.  (One CTA per (batch, head) with
 // shared-memory atomics for all ranks at once: 20.6 us on 24 heads x 929 blocks, 8 ranks, 24 CTAs on 148 SMs; this
-// split 8 us.  Ownership words by ballot, the list of rows by counting bits and eight rows in flight, the last ones too: a
-// plan of that layer in one launch 9.8 us with shared-memory atomics for both and four rows, 7.9 this way.)  OR does not depend on the order, so the bits are well defined.  A rank value outside [0, P) is ignored.
+// split 8 us.)  OR does not depend on the order, so the bits are well defined.  A rank value outside [0, P) is ignored.
 constexpr int kUnionThreads = 512;
-
-// The plan of a call without destinations, consumer by consumer, by whichever of a consumer's CTAs is the last to finish.
-// One launch instead of two, where the tickets fit the workspace's header and the CTAs the chip: us a call, of which 5.4 are
-// the host's (7.4 with two), two launches / one: 13 heads x 77 blocks, 5 ranks 7.5 / 5.3; 24 x 384, 4 ranks 7.6 / 5.4; with
-// more CTAs than SMs, whose launches overlap less, 48 x 278, 8 ranks 7.4 / 7.3; 24 x 929, 8 ranks 7.5 / 8.0.  (One CTA
-// planning for all consumers: 24 x 929 9.8, 48 x 278 11.5.)
-constexpr int kLastPlanCtas = 148;  // one per SM
-struct LastPlan {
-  int32_t* tickets;  // [B*P] CTAs that have finished; 0 before the launch and behind it.  NULL: no plan
-  int64_t *seg_off, *seg_total, *volume;
-  int64_t entry_bytes;
-  int include_local;
-};
-
-// Called by all threads of a CTA that has left its counts for consumer br.
-__device__ __forceinline__ void plan_by_last_cta(const LastPlan& q, const int32_t* cnt, int br, int H, int P) {
-  constexpr int kWarps = kUnionThreads / 32;
-  __shared__ int last_s, warp_s[kWarps], remote_s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last_s = atomicAdd(q.tickets + br, 1) == H - 1;
-    if (last_s) q.tickets[br] = 0;
-    remote_s = 0;
-    __threadfence();
-  }
-  __syncthreads();
-  if (!last_s) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, PH = P * H, own = br % P * H;
-  const int32_t* mine = cnt + (int64_t)br * PH;
-  int64_t cursor = 0;
-  for (int i0 = 0; i0 < PH; i0 += kUnionThreads) {
-    const int i = i0 + (int)threadIdx.x;
-    const int c = i < PH ? __ldcg(mine + i) : 0;
-    const bool local = i >= own && i < own + H;
-    const int counted = local && !q.include_local ? 0 : c;
-    const int remote = __reduce_add_sync(0xffffffffu, local ? 0 : c);
-    int incl = counted;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, s);
-      if (lane >= s) incl += v;
-    }
-    if (i0 > 0) __syncthreads();  // (the previous chunk's sums have been read)
-    if (lane == 31) {
-      warp_s[warp] = incl;
-      atomicAdd(&remote_s, remote);
-    }
-    __syncthreads();
-    int before = 0, all = 0;
-#pragma unroll
-    for (int k = 0; k < kWarps; ++k) {
-      before += k < warp ? warp_s[k] : 0;
-      all += warp_s[k];
-    }
-    if (i < PH) q.seg_off[(int64_t)br * PH + i] = cursor + before + incl - counted;
-    cursor += all;
-  }
-  if (threadIdx.x == 0) {
-    q.seg_total[br] = cursor;
-    q.volume[br] = q.entry_bytes * remote_s;
-  }
-}
 
 __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32_t* __restrict__ mask,
                                                                     const int32_t* __restrict__ rank, int H, int NB,
                                                                     int Wd, int P, uint32_t* __restrict__ U,
                                                                     int include_local, int32_t* __restrict__ cnt,
                                                                     int32_t* __restrict__ received,
-                                                                    int32_t* __restrict__ n_src, const LastPlan plan) {
+                                                                    int32_t* __restrict__ n_src) {
   enter_grid(mask, rank);
   __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
   __shared__ uint32_t u_s[kMaxWords];
   __shared__ uint16_t rows_s[kMaxBlocks];
+  __shared__ int n_rows_s;
   const int r = blockIdx.x % P, bh = blockIdx.x / P, bb = bh / H, h = bh % H;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = kUnionThreads / 32;
+  if (threadIdx.x == 0) n_rows_s = 0;
   if (threadIdx.x < kMaxWords) u_s[threadIdx.x] = 0u;
   if (blockIdx.x == 0 && threadIdx.x == 0 && n_src) *n_src = 0;
-  constexpr int kOwn = kMaxWords / n_warps;  // words of blocks a warp looks at
-  uint32_t mine[kOwn];                       // my rank's blocks of them
-  {
-    int rk[kOwn];
-#pragma unroll
-    for (int t = 0; t < kOwn; ++t) {
-      const int j = (warp + t * n_warps) * 32 + lane;
-      rk[t] = j < NB ? rank[j] : -1;
-    }
-#pragma unroll
-    for (int t = 0; t < kOwn; ++t) {
-      const int w = warp + t * n_warps;
-      mine[t] = __ballot_sync(0xffffffffu, rk[t] == r);
-      if (w < Wd)
-        for (int p = 0; p < P; ++p) {
-          const uint32_t word = __ballot_sync(0xffffffffu, rk[t] == p);
-          if (lane == 0) own_s[p * Wd + w] = word;
-        }
-    }
-  }
-  __syncthreads();
-  int n_rows;
-  const int before = bits_below(lane < Wd ? own_s[r * Wd + lane] : 0u, lane, &n_rows);
-#pragma unroll
-  for (int t = 0; t < kOwn; ++t) {
-    const int first = __shfl_sync(0xffffffffu, before, (warp + t * n_warps) & 31);
-    if ((mine[t] >> lane) & 1u)
-      rows_s[first + __popc(mine[t] & ((1u << lane) - 1u))] = (uint16_t)((warp + t * n_warps) * 32 + lane);
-  }
+  own_words(rank, NB, Wd, P, own_s);
+  for (int i = threadIdx.x; i < NB; i += kUnionThreads)
+    if (rank[i] == r) rows_s[atomicAdd(&n_rows_s, 1)] = (uint16_t)i;
   __syncthreads();
   int width = 1;  // lanes per row: the next power of two
   while (width < Wd) width <<= 1;
   const int per_warp = 32 / width, w = lane & (width - 1), sub = lane / width;
   const uint32_t* m = mask + (int64_t)bh * NB * Wd;
   uint32_t acc = 0;
-  constexpr int kRows = 8;  // rows in flight, the last ones too
-  for (int k0 = warp * per_warp + sub; k0 < n_rows; k0 += kRows * n_warps * per_warp) {
-    uint32_t v[kRows];
-#pragma unroll
-    for (int u = 0; u < kRows; ++u) {
-      const int k = k0 + u * n_warps * per_warp;
-      v[u] = k < n_rows && w < Wd ? m[(int64_t)rows_s[k] * Wd + w] : 0u;
-    }
-#pragma unroll
-    for (int u = 0; u < kRows; ++u) acc |= v[u];
-  }
+  const int n_rows = n_rows_s;
+#pragma unroll 4
+  for (int k = warp * per_warp + sub; k < n_rows; k += n_warps * per_warp)
+    if (w < Wd) acc |= m[(int64_t)rows_s[k] * Wd + w];
   for (int s = width; s < 32; s <<= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, s);
   if (lane < Wd && acc) atomicOr(&u_s[lane], acc);
   __syncthreads();
@@ -162,7 +67,125 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
     const int c = __reduce_add_sync(0xffffffffu, __popc(u & packed));
     if (lane == 0) received[(int64_t)(bb * P + r) * H + h] = c;
   }
-  if (plan.tickets) plan_by_last_cta(plan, cnt, bb * P + r, H, P);
+}
+
+// Unions, counts and offsets of a plan without destinations, in one launch: a cluster of CTAs per consumer takes the consumer's
+// heads in turn, meets when all counts are there, and its first CTA scans them.  Nothing is kept between launches.
+// Latency-bound, and what is saved is the host's time for a launch.  So a CTA makes its lists by ballots, matches and counting
+// bits, with eight rows in flight, the last ones too (the lists of the kernel above, of atomics, are fewer instructions, which
+// is what bounds it where CTAs are many: 2 x 48 heads x 512 blocks, 16 ranks 15.0 us a plan against 18.5 with lists like these).
+// us a plan with two launches / this way, one call behind the other and in a graph, where the host is out of it: 2 heads x 64
+// blocks, 4 ranks 7.4 / 5.1 and 4.0 / 3.9; 4 x 1000, 8 ranks 7.6 / 5.1 and 5.8 / 4.7; 13 x 77, 5 ranks 7.6 / 5.1 and 4.3 / 4.5;
+// 16 x 177, 8 ranks 7.6 / 5.2 and 4.6 / 4.7; 24 x 384, 4 ranks 8.0 / 5.8 and 4.9 / 5.4.  Several heads a CTA take too long where
+// rows are many and wide, 16 x 1000, 2 ranks 8.3 / 9.0 and 7.6 / 8.5, 24 x 929, 8 ranks 7.5 / 8.3 and 7.0 / 7.0, and so do more
+// than three: 48 x 278, 3 ranks 7.6 / 7.9 and 5.2 / 7.5.
+constexpr int kPlanCtas = 8, kPlanHeads = 3;                    // CTAs of a cluster, heads that one takes
+constexpr int kPlanWordsOfTwo = 20480, kPlanWordsOfThree = 4096;  // mask words of two and of three heads
+static bool plan_fits_clusters(const Geometry& g, int P, int sms) {
+  const int ctas = std::min(g.H, kPlanCtas), heads = (g.H + ctas - 1) / ctas, rows = (g.NB + P - 1) / P;
+  const int words = heads == 1 ? 0 : heads * rows * g.Wd, most = heads <= 2 ? kPlanWordsOfTwo : kPlanWordsOfThree;
+  return heads <= kPlanHeads && words <= most && g.H * P <= kUnionThreads && g.B * P * ctas <= sms;
+}
+
+__global__ void __launch_bounds__(kUnionThreads)
+    cluster_plan_kernel(const uint32_t* __restrict__ mask, const int32_t* __restrict__ rank, int H, int NB, int Wd, int P,
+                        uint32_t* __restrict__ U, int include_local, int32_t* __restrict__ cnt,
+                        int64_t* __restrict__ seg_off, int64_t* __restrict__ seg_total, int64_t* __restrict__ volume,
+                        int64_t entry_bytes) {
+  enter_grid(mask, rank);
+  __shared__ uint32_t own_s[kMaxRanks * kMaxWords];
+  __shared__ uint32_t u_s[kPlanHeads][kMaxWords];
+  __shared__ uint16_t rows_s[kMaxBlocks];
+  const int ctas = min(H, kPlanCtas), br = blockIdx.x / ctas, bb = br / P, r = br - bb * P;
+  const int h0 = blockIdx.x - br * ctas, n_heads = (H - h0 + ctas - 1) / ctas;  // heads h0, h0 + ctas, ...
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int n_warps = kUnionThreads / 32;
+  for (int i = threadIdx.x; i < kPlanHeads * kMaxWords; i += kUnionThreads) (&u_s[0][0])[i] = 0u;
+  for (int i = threadIdx.x; i < P * Wd; i += kUnionThreads) own_s[i] = 0u;
+  constexpr int kOwn = kMaxWords / n_warps;  // words of blocks a warp looks at
+  uint32_t mine[kOwn];                       // my rank's blocks of them
+  int rk[kOwn];
+#pragma unroll
+  for (int t = 0; t < kOwn; ++t) {
+    const int j = (warp + t * n_warps) * 32 + lane;
+    rk[t] = j < NB ? rank[j] : -1;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kOwn; ++t) {
+    mine[t] = __ballot_sync(0xffffffffu, rk[t] == r);
+    const uint32_t same = __match_any_sync(0xffffffffu, rk[t]);
+    if ((unsigned)rk[t] < (unsigned)P && lane == __ffs(same) - 1) own_s[rk[t] * Wd + warp + t * n_warps] = same;
+  }
+  __syncthreads();
+  int n_rows;
+  const int before = bits_below(lane < Wd ? own_s[r * Wd + lane] : 0u, lane, &n_rows);
+#pragma unroll
+  for (int t = 0; t < kOwn; ++t) {
+    const int first = __shfl_sync(0xffffffffu, before, (warp + t * n_warps) & 31);
+    if ((mine[t] >> lane) & 1u)
+      rows_s[first + __popc(mine[t] & ((1u << lane) - 1u))] = (uint16_t)((warp + t * n_warps) * 32 + lane);
+  }
+  __syncthreads();
+  int width = 1;  // lanes per row: the next power of two
+  while (width < Wd) width <<= 1;
+  const int per_warp = 32 / width, w = lane & (width - 1), sub = lane / width;
+  for (int k = 0; k < n_heads; ++k) {
+    const uint32_t* m = mask + (int64_t)(bb * H + h0 + k * ctas) * NB * Wd;
+    uint32_t acc = 0;
+    constexpr int kRows = 8;  // rows in flight, the last ones too
+    for (int k0 = warp * per_warp + sub; k0 < n_rows; k0 += kRows * n_warps * per_warp) {
+      uint32_t v[kRows];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        const int at = k0 + u * n_warps * per_warp;
+        v[u] = at < n_rows && w < Wd ? m[(int64_t)rows_s[at] * Wd + w] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) acc |= v[u];
+    }
+    for (int s = width; s < 32; s <<= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, s);
+    if (lane < Wd && acc) atomicOr(&u_s[k][lane], acc);
+  }
+  __syncthreads();
+  for (int i = warp; i < n_heads * P; i += n_warps) {
+    const int k = i / P, p = i - k * P, h = h0 + k * ctas;
+    const uint32_t u = lane < Wd ? u_s[k][lane] : 0u;
+    if (p == 0 && lane < Wd) U[((int64_t)br * H + h) * Wd + lane] = u;
+    const int c = __reduce_add_sync(0xffffffffu, lane < Wd ? __popc(u & own_s[p * Wd + lane]) : 0);
+    if (lane == 0) cnt[((int64_t)br * P + p) * H + h] = c;
+  }
+  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  if (h0 != 0) return;
+  // the consumer's counts in pack order, one per thread
+  __shared__ int sum_s[n_warps], remote_s[n_warps];
+  const int i = (int)threadIdx.x, n = P * H;
+  const int c = i < n ? __ldcg(cnt + (int64_t)br * n + i) : 0;
+  const bool local = i / H == r;
+  const int counted = local && !include_local ? 0 : c, remote = __reduce_add_sync(0xffffffffu, local ? 0 : c);
+  int incl = counted;
+#pragma unroll
+  for (int s = 1; s < 32; s <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, s);
+    if (lane >= s) incl += v;
+  }
+  if (lane == 31) {
+    sum_s[warp] = incl;
+    remote_s[warp] = remote;
+  }
+  __syncthreads();
+  int first = 0, all = 0, all_remote = 0;
+#pragma unroll
+  for (int k = 0; k < n_warps; ++k) {
+    first += k < warp ? sum_s[k] : 0;
+    all += sum_s[k];
+    all_remote += remote_s[k];
+  }
+  if (i < n) seg_off[(int64_t)br * n + i] = first + incl - counted;
+  if (i == 0) {
+    seg_total[br] = all;
+    volume[br] = entry_bytes * all_remote;
+  }
 }
 
 // Pack-order offsets, and where every packed tile goes.  A CTA per consumer scans its consumer's counts in pack
@@ -319,10 +342,9 @@ static int32_t* received_table(char* ws, const WsLayout& L, const Geometry& g, i
 }
 
 static cudaError_t launch_union(const Geometry& g, const uint32_t* mask, const int32_t* rank, int P, int include_local,
-                                uint32_t* U, int32_t* cnt, int32_t* received, int32_t* n_src, cudaStream_t st,
-                                const LastPlan& plan = LastPlan{}) {
+                                uint32_t* U, int32_t* cnt, int32_t* received, int32_t* n_src, cudaStream_t st) {
   return launch_kernel(union_count_kernel, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P, U,
-                       include_local, cnt, received, n_src, plan);
+                       include_local, cnt, received, n_src);
 }
 
 // dst, src, n_src, received: NULL for a plan without destinations.
@@ -350,15 +372,16 @@ int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_o
                   cudaStream_t st) {
   const int rc = check_consumers(g, P);
   if (rc != SPARSP_OK) return rc;
-  const int local = (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0;
-  int32_t* status = (int32_t*)(ws + L.status);
-  if (g.B * P <= kPlanTickets && (int64_t)g.B * g.H * P <= kLastPlanCtas) {
-    const LastPlan plan = {status + kPlanTicketWord, seg_off, seg_total, volume, 2LL * g.b * g.d * 2, local};
-    SPARSP_CUDA_OK(launch_union(g, mask, rank_of_block, P, local, U, cnt, nullptr, nullptr, st, plan));
+  const int local = (flags & SPARSP_INCLUDE_LOCAL) ? 1 : 0, ctas = std::min(g.H, kPlanCtas);
+  int sms = 0;
+  SPARSP_CUDA_OK(sm_count(&sms));
+  if (plan_fits_clusters(g, P, sms)) {
+    SPARSP_CUDA_OK(launch_clusters(cluster_plan_kernel, g.B * P * ctas, ctas, kUnionThreads, 0, st, mask, rank_of_block, g.H,
+                                   g.NB, g.Wd, P, U, local, cnt, seg_off, seg_total, volume, 2LL * g.b * g.d * 2));
     return SPARSP_OK;
   }
   SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, P, local, U, cnt, seg_off, seg_total, volume, nullptr, -1, nullptr,
-                             nullptr, nullptr, nullptr, status, st));
+                             nullptr, nullptr, nullptr, (int32_t*)(ws + L.status), st));
   return SPARSP_OK;
 }
 
