@@ -1959,16 +1959,17 @@ int launch_attn(const sparsp_shape& s, const Geometry& g, const void* Q, const v
                 cudaStream_t st) {
   AttnParams p = {};
   p.mask = mask;
-  // Up to two query blocks an SM need no queue and no launch that fills it: every CTA puts them in order for itself and takes
-  // one from the front and one from behind.  Two query blocks share a Q tile for the sake of throughput, and so few are done
-  // sooner each with its own list than with the union of two.  (us a call with the launch that makes items / without it: 2 heads
-  // x 64 blocks of 64 x 64, 16 kept 14.9 / 11.5 (stacked 19.4); 7 x 21 of 64 x 128 15.7 / 10.4; 19 x 9 of 128 x 128 14.5 / 12.0;
-  // 2 x 128 of 128 x 128, 10 % kept 33.5 / 32.1, threshold lists 67 / 54; 2 x 120 of 128 x 64, threshold lists 77 / 52; in order of
-  // their numbers 10.1 for 19 x 9, but 70 and 82 for the last two.  Up to three an SM 0.90 to 1.10 times as fast, up to four 0.80
-  // to 1.04.  An instance of the kernel of its own, because the question inside the queue's made 64-token blocks 1-2 % slower.)
+  // So few query blocks need no queue and no launch that fills it.  64-token blocks: one an SM; an item is then done sooner with
+  // its own list than with the union of two (us a call with the launch that makes items / without it: 2 heads x 64 blocks of 64
+  // x 64, 16 kept 14.9 / 11.5, stacked 19.4).  More of them have to share Q tiles where neighbours keep the same blocks: 2 x 100
+  // of 64 x 128, a quarter kept in windows 22.5 with the queue, 30.9 unstacked, all kept 50 / 83 (threshold lists, whose unions
+  // are long, would gain: 2 x 120 77 / 52).  128-token blocks: two an SM; every CTA puts them in order for itself and takes one
+  // from the front and one from behind (7 x 21 of 64 x 128 15.7 / 10.4, 2 x 148 of 128 x 128, 15 % kept 58.5 / 52.9, threshold
+  // lists 67 / 54; up to three an SM 0.90 to 1.10 times as fast, up to four 0.80 to 1.04).  An instance of the kernel of its own,
+  // because the question inside the queue's made 64-token blocks 1-2 % slower.
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
-  if ((int64_t)g.B * g.H * g.NB <= std::min(2 * sms, kMaxDirect))
+  if ((int64_t)g.B * g.H * g.NB <= std::min((g.b == 64 ? 1 : 2) * sms, kMaxDirect))
     return launch_attn_common<Source::kDirect>(s, g, Q, K, V, nullptr, 0, p, scale, O, lse, ws, L, st);
   const PrepParams pre = prep_params(g, mask, ws, L);
   const int rc = launch_prep<false>(g, pre, st);
