@@ -1992,15 +1992,15 @@ int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, 
   p.mask = mask;
   p.rank = rank;
   p.consumer = consumer;
-  // Where the consumer has hardly more items than there are SMs (if it has its share of the blocks; otherwise the CTAs just
-  // take more of them), their order and a queue are worth less than the launch that makes them: us a call over a whole
-  // buffer, with the launch / without, 1 head x 43 blocks, 5 ranks 18.5 / 16.4; 4 x 97 of 64 x 128, 8 ranks 20.0 / 17.9; 8 x 128,
-  // 4 ranks (1.7 items an SM) 37.6 / 33.4; 9 hops of 6 x 140 with all that belongs to them 238 / 214.  With 2.2 items an SM it
-  // depends: 80.5 / 77.3 for a whole buffer of 10 x 128, but 222 / 227 for its hops, half of whose items are empty.
+  // Where every CTA has one item at most, even if the consumer should own all blocks, neither their order nor a queue matters, and
+  // the launch that makes them is left out: us a call over a whole buffer, with the launch / without, 1 head x 43 blocks, 5 ranks
+  // 18.5 / 16.4; 2 x 140 of 64 x 128, 8 ranks, 15 % kept 27.5 / 25.0.  (With two items an SM by an even share of the blocks 4 x 97
+  // of 64 x 128 gains as much, 15.3 / 12.6, but lists of unequal length lose, 4 x 300 of 128 x 128 34 / 44, and more so where the
+  // consumer owns more than its share: a third of the blocks of 1 x 1024 of 64 x 128, 15 % kept on average 294 / 505.)
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
-  const int64_t blocks = (g.NB + P - 1) / P, per_item = 128 / g.b;
-  if ((int64_t)g.B * g.H * ((blocks + per_item - 1) / per_item) <= 2 * sms) {
+  const int64_t per_item = 128 / g.b;
+  if ((int64_t)g.B * g.H * ((g.NB + per_item - 1) / per_item) <= sms) {
     p.P = P;
     p.U = U;
     p.seg_off = seg_off;
