@@ -44,8 +44,10 @@
 // item that left the range is computed again (kRefZero ... below).  Only such an item, and rows whose first scores are out
 // of range, take their maxima as they go: the threads that own the same row (one per warpgroup) then share the reference
 // through shared memory and take their decisions strictly in tile order (mbarriers of the row group hand the turn from one to
-// the next), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since the reference last moved --
-// the thread that decides so first waits for every P V issued so far.
+// the next), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since the reference last moved.
+// The thread that decides so waits for every P V issued so far, but only behind its exponentials, which need nothing but the
+// new reference: those of neighbouring tiles overlap.  (Waiting and rescaling before them, us a call with Q times 40: 5 heads x
+// 492 blocks of 64 x 64, 15 % kept 930, now 632; 9 x 324 of 64 x 128 1787 / 1039; 4 x 300 of 128 x 128, 10 % 554 / 363.)
 // (The range used to be proved beforehand, by Cauchy-Schwarz from key norms that a pass over K took ahead of every call
 // and row norms taken from the Q tile of every item, and not at all for a packed source, whose tiles all took their
 // maximum in turns.  us per call then and now: one hop of 40 heads x 75600 over 8 ranks, 7 tiles an item, 97-112 -> 75;
@@ -1097,42 +1099,39 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         }
       };
 
-      // the row's reference follows its running maximum; the accumulator is rescaled
-      auto move_ref = [&](const float mx, const int n) {
-        const int g = g0 + n;
+      // The row's reference follows its running maximum; what has been added up so far shrinks by the factor that is returned.
+      auto move_ref = [&](const float mx) -> float {
         const float m_new = fmaxf(m_ref, mx);
-        const bool grow = m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY);
-        if (__any_sync(0xffffffffu, grow)) {
-          const float alpha = grow ? ex2(m_ref - m_new) : 1.0f;  // m_ref = -inf -> 0
-          if (n > 0) {
-            // every P V of the item issued so far must have landed in O before the row is rescaled; they
-            // complete in order, so the one of tile g-1 suffices
-            mbar_wait_bounded_inline(o_full + ((g - 1) & 3), ((g - 1) >> 2) & 1, s_abort, 38, p.wait_limit);
-            tc_fence_after();
+        if (!(m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY))) return 1.0f;
+        const float alpha = ex2(m_ref - m_new);  // m_ref = -inf -> 0
+        m_ref = m_new;
+        ref[row] = m_new;
+        return alpha;
+      };
+      // Rescales the row's accumulator, after the exponentials of the tile, which need the new reference only, and before its P
+      // is handed over.  Every P V of the item issued so far must have landed in O; they complete in order, so the one of tile
+      // g-1 suffices, and the tile behind, which may have a factor of its own by now, waits for the P V of this one.
+      auto rescale = [&](const float alpha, const int n) {
+        if (n == 0 || !__any_sync(0xffffffffu, alpha != 1.0f)) return;
+        const int g = g0 + n;
+        mbar_wait_bounded_inline(o_full + ((g - 1) & 3), ((g - 1) >> 2) & 1, s_abort, 38, p.wait_limit);
+        tc_fence_after();
 #pragma unroll 1
-            for (int c = 0; c < C::kAccCols / 16; ++c) {  // the row's accumulator, 16 columns at a time (rare: kept small)
-              uint32_t o[16];
-              tmem_ld16(tO + c * 16, o);
-              tmem_ld_wait();
+        for (int c = 0; c < C::kAccCols / 16; ++c) {  // the row's accumulator, 16 columns at a time (rare: kept small)
+          uint32_t o[16];
+          tmem_ld16(tO + c * 16, o);
+          tmem_ld_wait();
 #pragma unroll
-              for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-              tmem_st16(tO + c * 16, o);
-            }
-            if (C::kSum128) {  // the row sums live in columns of their own
-              uint32_t o[16];
-              tmem_ld16(tmem_base + C::kColL + lane_off, o);
-              tmem_ld_wait();
+          for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+          tmem_st16(tO + c * 16, o);
+        }
+        if (C::kSum128) {  // the row sums live in columns of their own
+          uint32_t o[16];
+          tmem_ld16(tmem_base + C::kColL + lane_off, o);
+          tmem_ld_wait();
 #pragma unroll
-              for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-              tmem_st16(tmem_base + C::kColL + lane_off, o);
-            }
-            tmem_st_wait();
-            tc_fence_before();
-          }
-          if (grow) {
-            m_ref = m_new;
-            ref[row] = m_new;
-          }
+          for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+          tmem_st16(tmem_base + C::kColL + lane_off, o);
         }
       };
       // A tile whose P takes the place of its scores: 32 columns at a time, the next ones on their way from tensor memory.
@@ -1150,6 +1149,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
             for (int e = 0; e < 32; ++e) v[e] = (q & 1) * 32 + e < vh[q >> 1] ? v[e] : -INFINITY;
           }
         };
+        float alpha = 1.0f;
         if (kExact || n == 0) {  // a look at the whole tile first
           float mx = -INFINITY, most = 0.0f;
 #pragma unroll
@@ -1175,7 +1175,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
           mx *= p.scale_log2;
           if (kExact) {
             if (n > 0) take_turn();
-            move_ref(mx, n);
+            alpha = move_ref(mx);
             if (n == 0 && m_ref == -INFINITY) ref[row] = m_ref;
             if (n + 1 < n_tiles) give_turn();
           } else {
@@ -1238,6 +1238,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
             tmem_st16(tP + (2 * h + 1) * 16, none);
           }
         }
+        if (kExact) rescale(alpha, n);
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
@@ -1273,11 +1274,12 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(s_free + wg);
 
+        float alpha = 1.0f;
         if (kExact) {
           const float mx = row_max(sv, vh);
           // ---- my turn to look at / move the row's reference maximum (strictly in tile order) ----
           if (n > 0) take_turn();
-          move_ref(mx, n);
+          alpha = move_ref(mx);
           if (n == 0 && m_ref == -INFINITY) ref[row] = m_ref;
           if (n + 1 < n_tiles) give_turn();
         }
@@ -1318,6 +1320,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_st16(tP + c * 16, pk + c * 16);
+        if (kExact) rescale(alpha, n);
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
