@@ -1120,7 +1120,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         for (int c = 0; c < C::kAccCols / 16; ++c) {  // the row's accumulator, 16 columns at a time (rare: kept small)
           uint32_t o[16];
           tmem_ld16(tO + c * 16, o);
-          tmem_ld_wait();
+          tmem_ld_wait(o);
 #pragma unroll
           for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
           tmem_st16(tO + c * 16, o);
@@ -1128,7 +1128,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         if (C::kSum128) {  // the row sums live in columns of their own
           uint32_t o[16];
           tmem_ld16(tmem_base + C::kColL + lane_off, o);
-          tmem_ld_wait();
+          tmem_ld_wait(o);
 #pragma unroll
           for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
           tmem_st16(tmem_base + C::kColL + lane_off, o);
@@ -1139,10 +1139,6 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         constexpr bool kRagged = decltype(ragged_tag)::value, kExact = decltype(exact_tag)::value;
         float va[32], vb[32];
         auto load = [&](float(&v)[32], const int q) { tmem_ld32(tS + q * 32, reinterpret_cast<uint32_t*>(v)); };
-        auto loaded = [&](float(&v)[32]) {  // nothing of v is looked at ahead of the wait before this
-#pragma unroll
-          for (int e = 0; e < 32; ++e) asm volatile("" : "+f"(v[e]));
-        };
         auto cut = [&](float(&v)[32], const int q) {  // columns past the end of the sequence count as -inf
           if (kRagged && vh[q >> 1] < 64) {
 #pragma unroll
@@ -1156,7 +1152,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
           for (int q = 0; q < 4; ++q) {
             if (vh[q >> 1] > 0) {
               load(va, q);
-              tmem_ld_wait();
+              tmem_ld_wait(va);
               cut(va, q);
               if (kExact || ((kRagged || kPacked) && ref_of == kRefFirst)) {
                 float m0 = va[0], m1 = va[1];
@@ -1224,11 +1220,10 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         for (int h = 0; h < 2; ++h) {
           if (vh[h] > 0) {
             load(va, 2 * h);
-            tmem_ld_wait();
+            tmem_ld_wait(va);
             load(vb, 2 * h + 1);
             exponentials(va, 2 * h);
-            tmem_ld_wait();
-            loaded(vb);
+            tmem_ld_wait(vb);
             exponentials(vb, 2 * h + 1);
           } else {
             uint32_t none[16];
@@ -1253,7 +1248,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         float sv[128];
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, reinterpret_cast<uint32_t*>(sv) + c * 32);
-        tmem_ld_wait();
+        tmem_ld_wait(sv);
         if (kRagged) {
           // the sequence ends inside this tile: columns past the end count as -inf
 #pragma unroll
@@ -1405,16 +1400,16 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         asm volatile("" : "+l"(orow), "+l"(lrow), "+r"(wide), "+r"(mine_to_write));
         mbar_wait_bounded_inline(o_full + (last & 3), (last >> 2) & 1, s_abort, 40, p.wait_limit);
         tc_fence_after();
-        uint32_t sum, o[D];
-        tmem_ld1(tmem_base + C::kColL + lane_off, &sum);
+        uint32_t o[D + 1];  // the row's accumulator and its sum
+        tmem_ld1(tmem_base + C::kColL + lane_off, o + D);
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) tmem_ld32(tO + c * 32, o + c * 32);
-        tmem_ld_wait();
+        tmem_ld_wait(o);
         // the accumulator is in registers: the next item's first P V may overwrite it
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(o_drained);
-        const float l = __uint_as_float(sum);  // the row sum is a tensor-memory column
+        const float l = __uint_as_float(o[D]);
         // (an ordinary item asks one question here)
         const float safe = ref_of == kRefZero ? kSafeSumZero : kSafeSumFirst;
         const bool asks = !exact && mine_to_write && !(i_max <= kMaxExponent && l >= kMinSum && l <= safe);

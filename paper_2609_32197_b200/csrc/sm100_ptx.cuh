@@ -162,6 +162,20 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t n_cols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(n_cols) : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// ... for loads into these registers: nothing computed from them can be moved ahead of the wait, with which the compiler sees
+// no connection otherwise.
+template <int N>
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[N]) {
+  tmem_ld_wait();
+#pragma unroll
+  for (int e = 0; e < N; ++e) asm volatile("" : "+r"(r[e]));
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld_wait(float (&r)[N]) {
+  tmem_ld_wait();
+#pragma unroll
+  for (int e = 0; e < N; ++e) asm volatile("" : "+f"(r[e]));
+}
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp receives lane (base + i).
