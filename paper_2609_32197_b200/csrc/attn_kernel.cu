@@ -181,7 +181,7 @@ constexpr int kHeadMeet = 1 << 21, kHeadMeetParityShift = 22;
 //   kPackedDirect  the same tiles, but the CTAs number the consumer's items and places in the buffer for themselves
 enum class Source { kQueue, kDirect, kPacked, kPackedDirect };
 
-constexpr int kMaxDirect = 2 * 148;  // items of a call without a queue
+constexpr int kMaxDirect = 2 * 148, kMaxPackedDirect = 512;  // items of a call without a queue
 
 template <int D, int BLK>
 struct AttnCfg {
@@ -228,8 +228,11 @@ struct AttnCfg {
   // kPackedDirect: uint32 own[P][Wd], int32 first[P][Wd] (places of a head's blocks), uint32 union[32], uint8 rank[1024]
   static constexpr int kOffOwn = kTotal, kOffFirst = kOffOwn + kMaxRanks * kMaxWords * 4;
   static constexpr int kOffUnion = kOffFirst + kMaxRanks * kMaxWords * 4, kOffRank = kOffUnion + kMaxWords * 4;
-  static constexpr int kDynamicDirect = kOffRank + kMaxBlocks + 1024;
-  // kDirect: uint32 length of every item's list and its number, uint16 items in order
+  static constexpr int kOffPackedOrder = kOffRank + kMaxBlocks;  // uint16 items in order
+  static constexpr int kDynamicDirect = kOffPackedOrder + 2 * kMaxPackedDirect + 1024;
+  // (while items are put in order, the places of entries and `first` hold counts and the list of own blocks)
+  static_assert(4 * (kMaxBlocks + 1) <= kLists * kMaxBlocks * 4 && 2 * kMaxBlocks <= kMaxRanks * kMaxWords * 4, "room for both");
+  // kDirect: the same lengths, uint16 items in order
   static constexpr int kOffLength = kTotal, kOffOrder = kOffLength + 4 * kMaxDirect;
   static_assert(kDynamicDirect <= 232448, "shared memory budget");
 };
@@ -418,7 +421,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
   uint32_t* sOwn = reinterpret_cast<uint32_t*>(smem + C::kOffOwn);
   uint8_t* sRank = smem + C::kOffRank;
   uint32_t* sLength = reinterpret_cast<uint32_t*>(smem + C::kOffLength);
-  uint16_t* sOrder = reinterpret_cast<uint16_t*>(smem + C::kOffOrder);
+  uint16_t* sOrder = reinterpret_cast<uint16_t*>(smem + (kPackedDirect ? C::kOffPackedOrder : C::kOffOrder));
   if constexpr (kDirect) {
     // More items than CTAs: every CTA puts all of them in order, the longest list first.  A mask row is an item; short rows
     // share a warp's load.
@@ -473,6 +476,70 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         for (int r = 0; r < p.P; ++r) {
           const uint32_t word = __ballot_sync(0xffffffffu, rk[t] == r);
           if (lane == 0) sOwn[r * p.Wd + w] = word;
+        }
+      }
+    }
+    // More items than CTAs, because the consumer has more than its share of the blocks: every CTA puts them in order by
+    // counting their lengths.  An item is a block or two neighbours, a thread has one at most.  Items of one length stay in order
+    // of their numbers: all CTAs have to come to the same order.
+    int n_own = 0, own_before = 0, per_head = 0, n = p.BH * ((p.NB + C::kEPT - 1) / C::kEPT);
+    uint32_t own = 0u;
+    if (n > (int)gridDim.x) {  // (as many as if all blocks were the consumer's)
+      __syncthreads();
+      own = lane < p.Wd ? sOwn[p.consumer * p.Wd + lane] : 0u;
+      own_before = bits_below(own, lane, &n_own);
+      per_head = (n_own + C::kEPT - 1) / C::kEPT;
+      n = p.BH * per_head;
+    }
+    if (n > (int)gridDim.x) {
+      int* at = reinterpret_cast<int*>(smem + C::kOffEnt);  // [NB + 1] place NB - length: items of that length, then where they begin
+      uint16_t* blocks = reinterpret_cast<uint16_t*>(smem + C::kOffFirst);
+      for (int t = tid; t <= p.NB; t += C::kThreads) at[t] = 0;
+      for (int w = warp; w < p.Wd; w += kWarps) {  // (the same for all lanes)
+        const uint32_t word = __shfl_sync(0xffffffffu, own, w);
+        const int first = __shfl_sync(0xffffffffu, own_before, w);
+        if ((word >> lane) & 1u) blocks[first + __popc(word & ((1u << lane) - 1u))] = (uint16_t)(w * 32 + lane);
+      }
+      __syncthreads();
+      static_assert(kMaxPackedDirect <= C::kThreads, "a thread per item");
+      int place = -1;  // NB - length, where I have an item
+      if (tid < n) {
+        const int bh = tid / per_head, x = (tid - bh * per_head) * C::kEPT;
+        const uint32_t* rows = p.mask + (int64_t)bh * p.NB * p.Wd;
+        const uint32_t *row0 = rows + blocks[x] * p.Wd, *row1 = rows + blocks[min(x + C::kEPT - 1, n_own - 1)] * p.Wd;
+        place = p.NB;
+#pragma unroll 8
+        for (int w = 0; w < p.Wd; ++w) place -= __popc(C::kStacked ? row0[w] | row1[w] : row0[w]);
+        place = max(place, 0);  // (a mask has no bits behind its NB-th)
+      }
+      const uint32_t peers = __match_any_sync(0xffffffffu, place);
+      const int leader = __ffs(peers) - 1;
+      if (tid < n && lane == leader) atomicAdd(at + place, __popc(peers));
+      __syncthreads();
+      if (warp == 0) {
+        int before = 0;
+        for (int t0 = 0; t0 <= p.NB; t0 += 32) {  // (the same for all lanes)
+          const int count = t0 + lane <= p.NB ? at[t0 + lane] : 0;
+          int incl = count;
+#pragma unroll
+          for (int s = 1; s < 32; s <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, s);
+            if (lane >= s) incl += v;
+          }
+          if (t0 + lane <= p.NB) at[t0 + lane] = before + incl - count;
+          before += __shfl_sync(0xffffffffu, incl, 31);
+        }
+      }
+      for (int k = 0; k * 32 < n; ++k) {  // warp by warp
+        __syncthreads();
+        if (warp == k) {
+          int first = 0;
+          if (tid < n && lane == leader) {
+            first = at[place];
+            at[place] = first + __popc(peers);
+          }
+          first = __shfl_sync(0xffffffffu, first, leader);
+          if (tid < n) sOrder[first + __popc(peers & ((1u << lane) - 1u))] = (uint16_t)tid;
         }
       }
     }
@@ -719,27 +786,17 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         rb1 = lane < p.Wd && blk1 >= 0 ? rows[blk1 * p.Wd + lane] : 0u;
       };
       auto fetch = [&](int it) {
-        if constexpr (kDirect) {  // the CTAs take places in order from the front and from behind in turn
+        if constexpr (kDirect || kPackedDirect) {  // the CTAs take places in order from the front and from behind in turn
+          const int per_head = kDirect ? p.NB : (n_own + C::kEPT - 1) / C::kEPT, n = p.BH * per_head;
           bh = p.BH;
-          if (it >= p.BH * p.NB) return;
-          const int item = p.BH * p.NB > (int)gridDim.x ? sOrder[it] : it;
-          bh = item / p.NB;
-          blk0 = item - bh * p.NB;
+          if (it >= n) return;
+          const int item = n > (int)gridDim.x ? sOrder[it] : it, at = item / per_head, x = item - at * per_head;
+          bh = at;
+          blk0 = kDirect ? x : own_block(x * C::kEPT);
+          blk1 = kPackedDirect && C::kStacked && x * C::kEPT + 1 < n_own ? own_block(x * C::kEPT + 1) : -1;
           load_rows();
-          if (!__any_sync(0xffffffffu, rb0 != 0u)) bh = p.BH;  // (and so do all behind it)
+          if (!__any_sync(0xffffffffu, (rb0 | rb1) != 0u)) bh = p.BH;  // (and so do all behind it)
           return;
-        }
-        if constexpr (kPackedDirect) {  // every gridDim.x-th one; those that keep nothing are left out
-          const int per_head = (n_own + C::kEPT - 1) / C::kEPT;
-          for (number = it;; number += (int)gridDim.x) {
-            bh = per_head > 0 ? min(number / per_head, p.BH) : p.BH;
-            if (bh >= p.BH) return;
-            const int x = (number - bh * per_head) * C::kEPT;
-            blk0 = own_block(x);
-            blk1 = C::kStacked && x + 1 < n_own ? own_block(x + 1) : -1;
-            load_rows();
-            if (__any_sync(0xffffffffu, (rb0 | rb1) != 0u)) return;
-          }
         }
         int x;
         if (kPacked) {
@@ -772,11 +829,10 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         load_rows();
       };
       auto next_item = [&]() {
-        if (kDirect) {
+        if (kDirect || kPackedDirect) {
           const int turn_no = ++number, c = (int)blockIdx.x, G = (int)gridDim.x;
           return turn_no * G + (turn_no & 1 ? G - 1 - c : c);
         }
-        if (kPackedDirect) return number + (int)gridDim.x;
         int it = 0;
         if (lane == 0) it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
         return __shfl_sync(0xffffffffu, it, 0);
@@ -1990,15 +2046,18 @@ int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, 
   p.mask = mask;
   p.rank = rank;
   p.consumer = consumer;
-  // Where every CTA has one item at most, even if the consumer should own all blocks, neither their order nor a queue matters, and
-  // the launch that makes them is left out: us a call over a whole buffer, with the launch / without, 1 head x 43 blocks, 5 ranks
-  // 18.5 / 16.4; 2 x 140 of 64 x 128, 8 ranks, 15 % kept 27.5 / 25.0.  (With two items an SM by an even share of the blocks 4 x 97
-  // of 64 x 128 gains as much, 15.3 / 12.6, but lists of unequal length lose, 4 x 300 of 128 x 128 34 / 44, and more so where the
-  // consumer owns more than its share: a third of the blocks of 1 x 1024 of 64 x 128, 15 % kept on average 294 / 505.)
+  // Where the consumer has one item an SM at most, if it has its share of the blocks, neither their order nor a queue matters,
+  // and the launch that makes them is left out: us a call over a whole buffer, with the launch / without, 1 head x 43 blocks, 5
+  // ranks 18.5 / 16.4; an even share of 8 ranks, 15 % kept, 2 x 140 of 64 x 128 26.8 / 25.0, 4 x 97 of 64 x 128 21.2 / 19.1, 8 x 128
+  // of 64 x 128 27.1 / 24.7; a hop of 6 x 140 15.2 / 13.0.  If the consumer has more than its share, the CTAs put its items in
+  // order for themselves, up to 512 of them: 30 % of 8 x 128 42.9 / 42.0, with lists of unequal length 49.3 / 37.9, all of it 80.7
+  // / 79.4, but short lists, 4 % kept, 39.9 / 43.3.  (In order of their numbers lists of unequal length took up to 1.7 times as
+  // long, half of 1 x 300 of 128 x 128 75 / 110.  With two items an SM by an even share 4 x 300 of 128 x 128 34 / 44; with up to 1024
+  // to put in order 2 x 1000 of 64 x 128 240 / 265.)
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
-  const int64_t per_item = 128 / g.b;
-  if ((int64_t)g.B * g.H * ((g.NB + per_item - 1) / per_item) <= sms) {
+  const int64_t BH = (int64_t)g.B * g.H, share = (g.NB + P - 1) / P, per_item = 128 / g.b;
+  if (BH * ((share + per_item - 1) / per_item) <= sms && BH * ((g.NB + per_item - 1) / per_item) <= kMaxPackedDirect) {
     p.P = P;
     p.U = U;
     p.seg_off = seg_off;

@@ -1,6 +1,6 @@
 """Which attention calls do without the launch that makes their items, seen from the number of launches: 64-token blocks up to
-one an SM (more of them share Q tiles), 128-token blocks up to two, and a packed source only where every CTA has one item at
-most, whoever owns the blocks."""
+one an SM (more of them share Q tiles), 128-token blocks up to two, and a packed source where a CTA has one item at most if the
+consumer has its share of the blocks, and the items can be put in order if it has more."""
 import pytest
 import torch
 
@@ -35,12 +35,13 @@ def test_own_keys(binding, b, per_sm, more):
     assert binding.sparsp_status(ws) == binding.SPARSP_OK
 
 
-@pytest.mark.parametrize("b,per_item", [(64, 2), (128, 1)])
-@pytest.mark.parametrize("more", [0, 1])
-def test_packed(binding, b, per_item, more):
-    sms, P = torch.cuda.get_device_properties(0).multi_processor_count, 4
-    NB = per_item * sms + more
-    shape, Q, K, V, mask = _inputs(binding, b, 1, NB)
+@pytest.mark.parametrize("b,H,NB,P,launches", [
+    # one item an SM (148) by an even share of the blocks, and one more
+    (128, 1, 148, 1, 1), (128, 1, 149, 1, 2), (64, 1, 296, 1, 1), (64, 1, 297, 1, 2), (128, 4, 74, 2, 1), (128, 4, 76, 2, 2),
+    # 512 items if it owns all blocks, and more
+    (128, 4, 128, 4, 1), (128, 4, 129, 4, 2), (64, 4, 256, 8, 1), (64, 4, 257, 8, 2)])
+def test_packed(binding, b, H, NB, P, launches):
+    shape, Q, K, V, mask = _inputs(binding, b, H, NB)
     ws = binding.make_workspace(shape, P)
     rank = torch.zeros(NB, dtype=torch.int32, device="cuda")
     do = binding.alloc_demand_outputs(shape, P)
@@ -50,5 +51,5 @@ def test_packed(binding, b, per_item, more):
     before = binding.sparsp_launch_count()
     binding.sparsp_sparse_attn_fwd_packed(shape, Q, K, V, mask, rank, P, 0, do["union_mask"], do["seg_offset"],
                                           do["seg_total"], packed, packed.numel(), None, 0.0, O, None, ws)
-    assert binding.sparsp_launch_count() - before == 1 + more
+    assert binding.sparsp_launch_count() - before == launches
     assert binding.sparsp_status(ws) == binding.SPARSP_OK

@@ -75,3 +75,14 @@ def test_packed_rows(binding, d, b, B, H, NB, P, owner, bases, far):
             # bf16 output and bf16 probabilities, |V| up to 5
             assert live.sum() == 0 or (O[bb, h, live].double() - want).abs().max().item() <= pu.ATTN_MAX_ABS
             assert bool((O[bb, h, mine & ~live] == 0).all()) and bool((lse[bb, h, mine & ~live] == float("-inf")).all())
+
+
+# consumers with far more than their share, whose items the CTAs put in order: as many as there is room for, one more, batches
+@pytest.mark.parametrize("d,b", [(64, 64), (128, 64), (64, 128), (128, 128)])
+@pytest.mark.parametrize("B,H,NB,P", [(1, 8, 60, 8), (1, 8, 64, 8), (2, 4, 64, 8), (1, 16, 64, 8), (1, 16, 65, 8), (1, 2, 200, 16),
+                                      (3, 5, 34, 4), (1, 1, 480, 8)])
+@pytest.mark.parametrize("far", [1.0, 60.0])
+def test_more_than_its_share(binding, d, b, B, H, NB, P, far):
+    if NB > 260 and b == 128:
+        pytest.skip("64-bit scores of as many tokens")
+    test_packed_rows(binding, d, b, B, H, NB, P, "most", False, far)
