@@ -77,14 +77,16 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
 // us a plan with two launches / this way, one call behind the other and in a graph, where the host is out of it: 2 heads x 64
 // blocks, 4 ranks 7.4 / 5.1 and 4.0 / 3.9; 4 x 1000, 8 ranks 7.6 / 5.1 and 5.8 / 4.7; 13 x 77, 5 ranks 7.6 / 5.1 and 4.3 / 4.5;
 // 16 x 177, 8 ranks 7.6 / 5.2 and 4.6 / 4.7; 24 x 384, 4 ranks 8.0 / 5.8 and 4.9 / 5.4.  Several heads a CTA take too long where
-// rows are many and wide, 16 x 1000, 2 ranks 8.3 / 9.0 and 7.6 / 8.5, 24 x 929, 8 ranks 7.5 / 8.3 and 7.0 / 7.0, and so do more
-// than three: 48 x 278, 3 ranks 7.6 / 7.9 and 5.2 / 7.5.
+// rows are many and wide, 16 x 1000, 2 ranks 8.3 / 9.0 and 7.6 / 8.5, 24 x 929, 8 ranks 7.5 / 8.3 and 7.0 / 7.0, where there are
+// more than eight clusters, 16 x 300, 11 ranks 7.6 / 6.7 and 5.0 / 6.8, 24 x 300 7.8 / 8.7 and 6.1 / 8.1, and so do more than three:
+// 48 x 278, 3 ranks 7.6 / 7.9 and 5.2 / 7.5.
 constexpr int kPlanCtas = 8, kPlanHeads = 3;                    // CTAs of a cluster, heads that one takes
+constexpr int kPlanAtOnce = 64;                                // CTAs of a launch, where they take several heads
 constexpr int kPlanWordsOfTwo = 20480, kPlanWordsOfThree = 4096;  // mask words of two and of three heads
 static bool plan_fits_clusters(const Geometry& g, int P, int sms) {
   const int ctas = std::min(g.H, kPlanCtas), heads = (g.H + ctas - 1) / ctas, rows = (g.NB + P - 1) / P;
   const int words = heads == 1 ? 0 : heads * rows * g.Wd, most = heads <= 2 ? kPlanWordsOfTwo : kPlanWordsOfThree;
-  return heads <= kPlanHeads && words <= most && g.H * P <= kUnionThreads && g.B * P * ctas <= sms;
+  return heads <= kPlanHeads && words <= most && g.H * P <= kUnionThreads && g.B * P * ctas <= (heads == 1 ? sms : kPlanAtOnce);
 }
 
 __global__ void __launch_bounds__(kUnionThreads)
