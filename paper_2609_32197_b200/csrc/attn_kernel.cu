@@ -1658,20 +1658,24 @@ __device__ __forceinline__ int make_items(const PrepParams& p, int bh, const uin
     if (threadIdx.x == 0) s_best = 1023u - 1u;  // default D = 1
     for (int i = threadIdx.x; i < n; i += kPrepThreads)
       for (int w = Wd; w < 4 * units; ++w) m[i * pitch + w] = 0u;
-    constexpr int kFlight = 8;
-    for (int idx0 = threadIdx.x; idx0 < n * Wd; idx0 += kFlight * kPrepThreads) {
-      uint32_t v[kFlight];
-      int at[kFlight];
+    auto read = [&](auto in_flight) {
+      constexpr int kFlight = decltype(in_flight)::value;
+      for (int idx0 = threadIdx.x; idx0 < n * Wd; idx0 += kFlight * kPrepThreads) {
+        uint32_t v[kFlight];
+        int at[kFlight];
 #pragma unroll
-      for (int u = 0; u < kFlight; ++u) {
-        const int idx = idx0 + u * kPrepThreads, i = idx / Wd, w = idx - i * Wd;
-        at[u] = idx < n * Wd ? i * pitch + w : -1;
-        v[u] = at[u] >= 0 ? rows[(int64_t)block(i) * Wd + w] : 0u;
+        for (int u = 0; u < kFlight; ++u) {
+          const int idx = idx0 + u * kPrepThreads, i = idx / Wd, w = idx - i * Wd;
+          at[u] = idx < n * Wd ? i * pitch + w : -1;
+          v[u] = at[u] >= 0 ? rows[(int64_t)block(i) * Wd + w] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < kFlight; ++u)
+          if (at[u] >= 0) m[at[u]] = v[u];
       }
-#pragma unroll
-      for (int u = 0; u < kFlight; ++u)
-        if (at[u] >= 0) m[at[u]] = v[u];
-    }
+    };
+    if (n * Wd <= kPrepThreads) read(std::integral_constant<int, 1>{});
+    else read(std::integral_constant<int, 8>{});
     // bits that two rows share, or that either has
     auto common = [&](int a, int b2, bool either) {
       int bits = 0;
