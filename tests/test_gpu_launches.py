@@ -1,6 +1,7 @@
-"""Which attention calls do without the launch that makes their items, seen from the number of launches: 64-token blocks up to
+"""Which calls do without a launch, seen from the number of launches.  Attention without the one that makes its items: 64-token blocks up to
 one an SM (more of them share Q tiles), 128-token blocks up to two, and a packed source where a CTA has one item at most if the
-consumer has its share of the blocks, and the items can be put in order if it has more."""
+consumer has its share of the blocks, and the items can be put in order if it has more.  The gather without the one that makes
+the unions: up to 4096 mask words and four blocks a warp, or half of the words and six."""
 import pytest
 import torch
 
@@ -51,5 +52,20 @@ def test_packed(binding, b, H, NB, P, launches):
     before = binding.sparsp_launch_count()
     binding.sparsp_sparse_attn_fwd_packed(shape, Q, K, V, mask, rank, P, 0, do["union_mask"], do["seg_offset"],
                                           do["seg_total"], packed, packed.numel(), None, 0.0, O, None, ws)
+    assert binding.sparsp_launch_count() - before == launches
+    assert binding.sparsp_status(ws) == binding.SPARSP_OK
+
+
+@pytest.mark.parametrize("H,NB,launches", [(4, 128, 1), (5, 118, 1), (5, 119, 2), (13, 60, 1), (13, 64, 1), (14, 64, 2), (1, 362, 2)])
+def test_gather(binding, H, NB, launches):
+    b, d, P = 128, 128, 3  # one warp copies a block
+    shape, _, K, V, mask = _inputs(binding, b, H, NB, d)
+    ws = binding.make_workspace(shape, P)
+    rank = torch.arange(NB, dtype=torch.int32, device="cuda").remainder(P)
+    do = binding.alloc_demand_outputs(shape, P)
+    packed = torch.zeros(4 * b * d * H * P, dtype=torch.uint8, device="cuda")
+    before = binding.sparsp_launch_count()
+    binding.sparsp_demand_pack(shape, mask, rank, P, 0, K, V, do["union_mask"], do["cnt"], do["seg_offset"], do["seg_total"],
+                               do["volume_bytes"], packed, packed.numel(), None, ws)
     assert binding.sparsp_launch_count() - before == launches
     assert binding.sparsp_status(ws) == binding.SPARSP_OK
