@@ -1,7 +1,7 @@
 """Attention calls of few query blocks, whose CTAs put the items in order for themselves: one and two an SM and one more than
 that, rows of one to eight mask words, lists of every length in any order, rows and heads that keep nothing; and calls of many
-blocks in few heads, whose items are put in order by counting.  Rows against a masked softmax in 64 bits, also with scores that
-leave the range."""
+blocks in few heads, whose items are put in order by counting.  Rows and their log-sum-exps against a masked softmax in 64
+bits, also with scores that leave the range."""
 import math
 
 import pytest
@@ -53,4 +53,7 @@ def test_few_items(binding, d, b, B, H, NB, far):
                 want = torch.softmax(s, -1) @ V[bb, h].double()
                 # bf16 output and bf16 probabilities, |V| up to 5
                 assert not live.any() or (O[bb, h, rows].double() - want)[live].abs().max().item() <= pu.ATTN_MAX_ABS
+                # sums of bf16 probabilities; an fp32 number of up to hundreds: eight units in the last place on top
+                wl = torch.logsumexp(s, -1)[live]
+                assert bool(((lse[bb, h, rows][live].double() - wl).abs() <= 2e-2 + wl.abs() * 2.0 ** -20).all())
                 assert bool((O[bb, h, rows][~live] == 0).all()) and bool((lse[bb, h, rows][~live] == float("-inf")).all())

@@ -1,7 +1,7 @@
 """Attention over a packed buffer with and without the launch that numbers items and places: both sides of the rule between
-them (2 items an SM if the consumer has its share of the blocks), consumers that own nearly all, one or none of the blocks, 64
-ranks, batches, explicit slot bases, empty rows and heads, keys far out of range.  Foreign K and V are not numbers; rows
-against a masked softmax in 64 bits."""
+them (an item an SM if the consumer has its share of the blocks, 512 if it has all of them), consumers that own nearly all, one
+or none of the blocks, 64 ranks, batches, explicit slot bases, empty rows and heads, keys far out of range.  Foreign K and V are
+not numbers; rows and their log-sum-exps against a masked softmax in 64 bits."""
 import math
 
 import pytest
@@ -74,6 +74,9 @@ def test_packed_rows(binding, d, b, B, H, NB, P, owner, bases, far):
             want = torch.softmax(s[live], -1) @ V[bb, h].double()
             # bf16 output and bf16 probabilities, |V| up to 5
             assert live.sum() == 0 or (O[bb, h, live].double() - want).abs().max().item() <= pu.ATTN_MAX_ABS
+            # sums of bf16 probabilities; an fp32 number of up to hundreds: eight units in the last place on top
+            wl = torch.logsumexp(s[live], -1)
+            assert bool(((lse[bb, h, live].double() - wl).abs() <= 2e-2 + wl.abs() * 2.0 ** -20).all())
             assert bool((O[bb, h, mine & ~live] == 0).all()) and bool((lse[bb, h, mine & ~live] == float("-inf")).all())
 
 

@@ -1,6 +1,6 @@
-"""Plans made by the last CTA of the union's launch against the two launches of the call that has no workspace: both sides of
-the line between them (batch x ranks = 48, batch x heads x ranks = the number of SMs, 148), more counts of a consumer than one round takes, own blocks packed or not, and
-calls one behind the other on the same workspace."""
+"""Plans made in one launch, by a cluster of CTAs per consumer, against the two launches of the call that has no workspace: one to
+three heads a CTA and more, few and many consumers, own blocks packed or not, and calls one behind the other on the same
+workspace."""
 import pytest
 import torch
 
