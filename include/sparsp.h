@@ -15,7 +15,9 @@
  *   - Unless a parameter says "host", every data pointer is a DEVICE pointer owned by the caller.
  *     The library never allocates, frees or keeps caller memory; scratch lives in a caller-provided
  *     device workspace of sparsp_workspace_bytes() bytes (256-byte aligned).  Calls that share a
- *     workspace must be ordered on one stream.
+ *     workspace must be ordered on one stream.  No result depends on what the workspace holds
+ *     before a call, except the status that sparsp_status() returns: zero its first 256 bytes once,
+ *     or call sparsp_status() once, before the first status that matters.
  *   - `stream` is a cudaStream_t passed as void*; all work is enqueued on it asynchronously.
  *     Conditions only the device can detect (packed buffer too small, a bounded wait inside a
  *     kernel running out) are written to a status word in the workspace; sparsp_status()

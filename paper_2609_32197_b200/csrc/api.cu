@@ -306,7 +306,9 @@ int sparsp_exchange_plan(const sparsp_shape* shape, int32_t n_ranks, const int32
           *out++ = t;
         }
         // most blocks first, lower head first among equals (the chunks were produced in head order)
-        std::stable_sort(hop, out, [](const sparsp_transfer& a, const sparsp_transfer& b) { return a.n_entries > b.n_entries; });
+        std::stable_sort(hop, out, [](const sparsp_transfer& a, const sparsp_transfer& b) {
+          return a.n_entries > b.n_entries;
+        });
         for (int c = 0; c < C; ++c) hop[c].order = c;
       }
   return SPARSP_OK;
@@ -553,7 +555,8 @@ int sparsp_hop_chunk_mask(const sparsp_shape* shape, const uint32_t* mask, const
 
 int sparsp_hop_mask(const sparsp_shape* shape, const uint32_t* mask, const int32_t* rank_of_block, int32_t n_ranks,
                     int32_t consumer, int32_t producer, uint32_t* hop_mask, void* stream) {
-  if (!shape) return sparsp_hop_chunk_mask(shape, mask, rank_of_block, n_ranks, consumer, producer, 0, 0, hop_mask, stream);
+  if (!shape)
+    return sparsp_hop_chunk_mask(shape, mask, rank_of_block, n_ranks, consumer, producer, 0, 0, hop_mask, stream);
   return sparsp_hop_chunk_mask(shape, mask, rank_of_block, n_ranks, consumer, producer, 0, shape->heads, hop_mask,
                                stream);
 }

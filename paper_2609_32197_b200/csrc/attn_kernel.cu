@@ -2,30 +2,31 @@
 //
 // Work item = ONE 128-row Q tile of one (batch, head) with one fp32 accumulator O in tensor memory:
 //   block = 128: the Q tile is one query block; the item walks that block's kept KV blocks.
-//   block = 64 : two query blocks (chosen by a pairing pass so that their kept lists overlap) are stacked
-//                into the Q tile (full-rate M = 128 MMAs); a KV tile is two entries of the UNION of their
-//                kept lists (128 keys, full-rate N = 128); each 64x64 quadrant the mask does not keep is
-//                zeroed in P.
-// The kernel is persistent: one CTA per SM takes items from a global counter; the next item's kept
-// list, Q tile and first K/V tiles overlap the current item's last tiles, its first Q K^T the epilogue.
-// Where an item ends, only the warpgroup of its last tile waits for the accumulator and writes the rows; the other one is
+//   block = 64 : two query blocks (chosen by a pairing pass so that their kept lists overlap) are stacked into the Q
+//                tile (full-rate M = 128 MMAs); a KV tile is two entries of the UNION of their kept lists (128 keys,
+//                full-rate N = 128); each 64x64 quadrant the mask does not keep is zeroed in P.
+// The kernel is persistent: one CTA per SM takes items from a global counter (or in turn, see Source); the next item's
+// kept list, Q tile and first K/V tiles overlap the current item's last tiles, its first Q K^T the epilogue.  Where an
+// item ends, only the warpgroup of its last tile waits for the accumulator and writes the rows; the other one is
 // already at the next item, whose Q tile has a buffer of its own: the next one of the K ring, which gets the finished
-// item's Q buffer in exchange.  (Both warpgroups writing half of the columns, the Q tile behind the last Q K^T in a buffer
-// that is always Q's: 13 heads x 2 x 6034 tokens, 9 tiles an item, 86.9 us a call, now 78.2; 16 x 18600 with 6 to 30 tiles
-// 306 / 282; 40 x 75600, 59 tiles, 10.05 / 9.82 ms; one hop of it over 8 ranks, 2 to 8 tiles, 64.1 / 61.1.  Tried on top and
-// no better: rows through shared memory and a TMA store, lists for one or two items more, tiles dealt so that the
-// warpgroups take turns at writing.)
-// Every softmax warpgroup has a buffer of its own for scores S = Q K^T in tensor memory (128 fp32 columns), so that the tensor
-// pipe always has the next tiles' MMAs queued while the softmax of the current tile runs.  Tiles are numbered g = 0, 1, 2, ...
-// across the CTA's items; every ring, buffer and barrier phase follows g.
-//   d = 128: two warpgroups.  S 2 x 128 columns, P 64 columns of packed bf16, O 128 columns, 16 columns for the row sums.
-//            Q K^T of tile g+2 starts as soon as the scores of tile g have been READ.  A tile moves 160 KB through shared memory
-//            (64 KB of TMA writes, 96 KB of operands), 1250 clocks at 128 bytes a clock; ordinary tiles take 1400.
-//   d = 64:  three warpgroups.  A tile is half of that and its 16384 exponentials bound it, with two warps a scheduler more by
-//            their latencies (1495 clocks) than by the special-function unit (683), so there is a third one.  S 3 x 128
-//            columns, P in the place of the scores it was made from, O 64 + 16 columns; Q K^T of tile g+3 starts when P V of
-//            tile g has read P.  Two warpgroups with P buffers of their own / three: 13 heads x 2 x 6034 tokens 78.7 / 76.0 us
-//            a call, 48 x 17776 1380 / 1321, 16 x 18600 with threshold lists 282 / 258, 27 x 27403 from a packed buffer 279 / 244.
+// item's Q buffer in exchange.  (Both warpgroups writing half of the columns, the Q tile behind the last Q K^T in a
+// buffer that is always Q's: 13 heads x 2 x 6034 tokens, 9 tiles an item, 86.9 us a call, now 78.2; 16 x 18600 with 6
+// to 30 tiles 306 / 282; 40 x 75600, 59 tiles, 10.05 / 9.82 ms; one hop of it over 8 ranks, 2 to 8 tiles, 64.1 / 61.1.
+// Tried on top and no better: rows through shared memory and a TMA store, lists for one or two items more, tiles dealt
+// so that the warpgroups take turns at writing.)
+// Every softmax warpgroup has a buffer of its own for scores S = Q K^T in tensor memory (128 fp32 columns), so that the
+// tensor pipe always has the next tiles' MMAs queued while the softmax of the current tile runs.  Tiles are numbered g
+// = 0, 1, 2, ...  across the CTA's items; every ring, buffer and barrier phase follows g.
+//   d = 128: two warpgroups.  S 2 x 128 columns, P 64 columns of packed bf16, O 128 columns, 16 columns for the row
+//            sums.  Q K^T of tile g+2 starts as soon as the scores of tile g have been READ.  A tile moves 160 KB
+//            through shared memory (64 KB of TMA writes, 96 KB of operands), 1250 clocks at 128 bytes a clock; ordinary
+//            tiles take 1400.
+//   d = 64:  three warpgroups.  A tile is half of that and its 16384 exponentials bound it, with two warps a scheduler
+//            more by their latencies (1495 clocks) than by the special-function unit (683), so there is a third one.  S
+//            3 x 128 columns, P in the place of the scores it was made from, O 64 + 16 columns; Q K^T of tile g+3
+//            starts when P V of tile g has read P.  Two warpgroups with P buffers of their own / three: 13 heads x 2 x
+//            6034 tokens 78.7 / 76.0 us a call, 48 x 17776 1380 / 1321, 16 x 18600 with threshold lists 282 / 258, 27 x
+//            27403 from a packed buffer 279 / 244.
 // P V of tile g is issued as soon as P_g is written.
 // Warp roles (512 or 640 threads = 4 or 5 warpgroups; the first two hand most of their registers to the others):
 //   warp 0      TMA producer of Q (per item) and K, which share a ring of buffers
@@ -34,26 +35,27 @@
 //   warp 4      builds the kept / union list of the NEXT items (two list buffers)
 //   warps 5-7   clear the output rows of query blocks that keep nothing
 //   warps 8-    softmax: warpgroup w of kWGs takes the tiles with g % kWGs = w
-// (A producer is one thread running a chain of dependent instructions next to busy softmax warps: it gets
-// an instruction issued every ~8 cycles, so K and V loads have a warp each and keep per-tile work minimal.)
-// A softmax thread owns one query row of its tile: at d = 128 the whole 128-column row of S sits in registers, at d = 64, with
+// (A producer is one thread running a chain of dependent instructions next to busy softmax warps: it gets an
+// instruction issued every ~8 cycles, so K and V loads have a warp each and keep per-tile work minimal.)  A softmax
+// thread owns one query row of its tile: at d = 128 the whole 128-column row of S sits in registers, at d = 64, with
 // fewer registers a thread, 32 columns and the next 32 on their way.  Ordinary items run
 // without a row maximum: load scores -> exponentials -> store P, relative to 0 (K / V source) or to the row's maximum
 // over the item's first tile (packed source), which the warpgroup of that tile hands to the others; the tensor pipe
 // takes the row sums.  Whether that was right is seen from the finished row sums and the exponents on the way, and an
-// item that left the range is computed again (kRefZero ... below).  Only such an item, and rows whose first scores are out
-// of range, take their maxima as they go: the threads that own the same row (one per warpgroup) then share the reference
-// through shared memory and take their decisions strictly in tile order (mbarriers of the row group hand the turn from one to
-// the next), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since the reference last moved.
-// The thread that decides so waits for every P V issued so far, but only behind its exponentials, which need nothing but the
-// new reference: those of neighbouring tiles overlap.  (Waiting and rescaling before them, us a call with Q times 40: 5 heads x
-// 492 blocks of 64 x 64, 15 % kept 930, now 632; 9 x 324 of 64 x 128 1787 / 1039; 4 x 300 of 128 x 128, 10 % 554 / 363.)
-// (The range used to be proved beforehand, by Cauchy-Schwarz from key norms that a pass over K took ahead of every call
-// and row norms taken from the Q tile of every item, and not at all for a packed source, whose tiles all took their
-// maximum in turns.  us per call then and now: one hop of 40 heads x 75600 over 8 ranks, 7 tiles an item, 97-112 -> 75;
-// 24 x 24576 from one rank's whole buffer 437-445 -> 415-425; 13 heads x 2 x 6034 92-101 -> 85-93; all of 40 x 75600
-// 10.1-10.5 -> 9.7-10.2 ms.)
-// The block-64 pairing and the order of a head's items (longest list first) come from attn_prep_kernel.
+// item that left the range is computed again (kRefZero ... below).  Only such an item, and rows whose first scores are
+// out of range, take their maxima as they go: the threads that own the same row (one per warpgroup) then share the
+// reference through shared memory and take their decisions strictly in tile order (mbarriers of the row group hand the
+// turn from one to the next), and O is rescaled lazily, only when a row's maximum has grown by more than 2^8 since the
+// reference last moved.  The thread that decides so waits for every P V issued so far, but only behind its
+// exponentials, which need nothing but the new reference: those of neighbouring tiles overlap.  (Waiting and rescaling
+// before them, us a call with Q times 40: 5 heads x 492 blocks of 64 x 64, 15 % kept 930, now 632; 9 x 324 of 64 x 128
+// 1787 / 1039; 4 x 300 of 128 x 128, 10 % 554 / 363.)  (The range used to be proved beforehand, by Cauchy-Schwarz from
+// key norms that a pass over K took ahead of every call and row norms taken from the Q tile of every item, and not at
+// all for a packed source, whose tiles all took their maximum in turns.  us per call then and now: one hop of 40 heads
+// x 75600 over 8 ranks, 7 tiles an item, 97-112 -> 75; 24 x 24576 from one rank's whole buffer 437-445 -> 415-425; 13
+// heads x 2 x 6034 92-101 -> 85-93; all of 40 x 75600 10.1-10.5 -> 9.7-10.2 ms.)
+// The block-64 pairing and the order of a head's items (longest list first) come from attn_prep_kernel; calls of few
+// items have their CTAs put them in order (kDirect, kPackedDirect below).
 // Every mbarrier wait is bounded; a wait that runs out sets SPARSP_ERR_TIMEOUT in the status word
 // and raises a CTA-wide flag that makes all later waits fall through, so the CTA still drains.
 #include <algorithm>
@@ -98,8 +100,9 @@ struct AttnParams {
   long long wait_limit;
 };
 
-// register budget per thread after the warpgroups re-balance (d = 128: 256 * 48 + 256 * 208 = 512 * 128; d = 64: 256 * 48 + 384 *
-// 128 = 640 * 96, which is what a block of 640 threads is launched with; hardly anything spills)
+// register budget per thread after the warpgroups re-balance (d = 128: 256 * 48 + 256 * 208 = 512 * 128; d = 64: 256 *
+// 48 + 384 * 128 = 640 * 96, which is what a block of 640 threads is launched with; the softmax warps and the list
+// builder spill up to 130 bytes)
 #ifndef SPARSP_REGS_UTILITY
 #define SPARSP_REGS_UTILITY 48
 #define SPARSP_REGS_UTILITY2 48
@@ -114,19 +117,19 @@ constexpr float kGrowThreshold = 8.0f;
 //   kRefExact  the row's running maximum, moved lazily and strictly in tile order.
 // The first two look at no score behind the first tile, so they are right only for rows whose scores stay near the
 // reference.  That is seen at the end of the item: no exponential left the range of normal numbers on the FMA pipe
-// (kMaxExponent; the special-function unit saturates to 0 and infinity by itself), the row sum lies within
-// [kMinSum, kMaxSum], and no output column ran out of fp32 where the sum is so large that a finite V could do that (above
-// kSafeSumZero or kSafeSumFirst; below them it takes |V| > 2^63 or 2^102, and the running maximum allows no more than the
-// latter).  Then every term is a normal fp32 and bf16 number of full relative precision, or at most 2^-36 of the sum.  An
-// item with a row that fails, one with scores that are no numbers included, is computed again as kRefExact.
-// So that this is rare, the four warps of the item's first tile look at it first: rows whose first scores are far from 0
-// take the running maximum from the start, the 32 rows of a warp together (kZeroSample: every eighth score; kFirstSample:
-// the maximum that the reference is anyway).  Ordinary scores pass both: with unit-variance Q and K at d = 128 they are
-// within +-16.  (us per call of 13 heads x 2 x 6034 tokens, Q times 1, 4 and 60: 87, 144 and 136; looking for +-64 only 183
-// with Q times 4; with range proofs from the norms of rows and keys instead of all this 91, 131 and 140.)
-// All of this follows from the item alone, so a call repeats itself bit for bit whichever CTA takes which item.  (A CTA that
-// remembered failures and began its next items further on was right too, but let rows of ordinary heads change in their
-// last bit from call to call.)
+// (kMaxExponent; the special-function unit saturates to 0 and infinity by itself), the row sum lies within [kMinSum,
+// kMaxSum], and no output column ran out of fp32 where the sum is so large that a finite V could do that (above
+// kSafeSumZero or kSafeSumFirst; below them it takes |V| > 2^63 or 2^102, and the running maximum allows no more than
+// the latter).  Then every term is a normal fp32 and bf16 number of full relative precision, or at most 2^-36 of the
+// sum.  An item with a row that fails, one with scores that are no numbers included, is computed again as kRefExact.
+// So that this is rare, the four warps of the item's first tile look at it first: rows whose first scores are far from
+// 0 take the running maximum from the start, the 32 rows of a warp together (kZeroSample: every eighth score;
+// kFirstSample: the maximum that the reference is anyway).  Ordinary scores pass both: with unit-variance Q and K at d
+// = 128 they are within +-16.  (us per call of 13 heads x 2 x 6034 tokens, Q times 1, 4 and 60: 87, 144 and 136;
+// looking for +-64 only 183 with Q times 4; with range proofs from the norms of rows and keys instead of all this 91,
+// 131 and 140.)  All of this follows from the item alone, so a call repeats itself bit for bit whichever CTA takes
+// which item.  (A CTA that remembered failures and began its next items further on was right too, but let rows of
+// ordinary heads change in their last bit from call to call.)
 constexpr int kRefZero = 0, kRefFirst = 1, kRefExact = 2;
 constexpr float kMaxExponent = 126.0f;
 constexpr float kMinSum = 8.077935669463161e-28f;  // 2^-90
@@ -135,24 +138,25 @@ constexpr float kSafeSumZero = 1.8446744073709552e19f;  // 2^64
 constexpr float kSafeSumFirst = 33554432.0f;            // 2^25: kGrowThreshold and 2^17 keys
 constexpr float kZeroSample = 48.0f, kFirstSample = 64.0f;
 constexpr int kZeroMinTiles = 4;  // K / V source: shorter items take kRefFirst, whose largest terms are exact
-// Tuning switch (compile-time): how many of the exponentials go to the FMA pipe instead of the special-function unit (every
-// n-th pair; 0 = none).  The same share everywhere, so that a row's result does not depend on where its tiles come from.  us
-// per attention call with every 3rd / 4th / 6th pair:
-//   d = 64                   48 heads x 17776 tokens 1393 / 1410 / 1429 (none 1488, every 2nd 3 % slower than every 3rd)
-//   d = 128, 64-token blocks 24 x 24576, half of the blocks kept, neighbours alike 3094 / 3219 / -, 8 x 16384 with all kept 912 /
-//                            948 / -, 24 x 24576 with threshold lists 671 / 665 / 681
-//   ... 128-token blocks     under the power cap a smaller share is up to 1 % faster: 40 x 75600, 10 % kept 9884 / 9816 / 9903
-//                            (none 10596), one hop of it over 8 ranks 60.8 / - / 60.2
+// Tuning switch (compile-time): how many of the exponentials go to the FMA pipe instead of the special-function unit
+// (every n-th pair; 0 = none).  The same share everywhere, so that a row's result does not depend on where its tiles
+// come from.  us per attention call with every 3rd / 4th / 6th pair:
+//   d = 64                   48 heads x 17776 tokens 1393 / 1410 / 1429 (none 1488, every 2nd 3 % slower than every
+//                            3rd)
+//   d = 128, 64-token blocks 24 x 24576, half of the blocks kept, neighbours alike 3094 / 3219 / -, 8 x 16384 with all
+//                            kept 912 / 948 / -, 24 x 24576 with threshold lists 671 / 665 / 681
+//   ... 128-token blocks     under the power cap a smaller share is up to 1 % faster: 40 x 75600, 10 % kept 9884 / 9816
+//                            / 9903 (none 10596), one hop of it over 8 ranks 60.8 / - / 60.2
 #ifndef SPARSP_TUNE_POLY
 #define SPARSP_TUNE_POLY 3
 #endif
 
-// Lists that the list builder keeps: the current item's and the next one's.  (With 3 or 4 a CTA takes items that one with
-// nothing left to do cannot take any more: 9 heads x 10602 tokens 60.8 us a call, 62.2 with 3, 63.2 with 4.)
+// Lists that the list builder keeps: the current item's and the next one's.  (With 3 or 4 a CTA takes items that one
+// with nothing left to do cannot take any more: 9 heads x 10602 tokens 60.8 us a call, 62.2 with 3, 63.2 with 4.)
 constexpr int kLists = 2;
-// One list entry: a KV block and which of the item's two query blocks keep it (64-token blocks); for a packed source the
-// tile index of a remote block in its place.  (A word, or half of one, for both of a tile's entries: with the block, the
-// valid keys per query block and the slot in three arrays 48 heads x 17776 took 2 % longer.)
+// One list entry: a KV block and which of the item's two query blocks keep it (64-token blocks); for a packed source
+// the tile index of a remote block in its place.  (A word, or half of one, for both of a tile's entries: with the
+// block, the valid keys per query block and the slot in three arrays 48 heads x 17776 took 2 % longer.)
 template <bool kPacked>
 struct Entry;
 template <>
@@ -164,21 +168,24 @@ template <>
 struct Entry<true> {
   using type = uint32_t;
   static constexpr int kFlagShift = 30;
-  static constexpr uint32_t kRemote = 1u << 29;  // bits 0-28 are the block's K tile in the packed buffer (its V tile is next)
+  // bits 0-28 are the block's K tile in the packed buffer (its V tile is next)
+  static constexpr uint32_t kRemote = 1u << 29;
   static constexpr uint32_t kValue = kRemote - 1u;
 };
 // Item header, one load for each role: x = batch * H + head; y = entries | kHead... flags (0: there are no more items);
 // z = query blocks, first | second << 16 (0xffff: none); w = batch.
 constexpr int kHeadEntries = 0xffff, kHeadRagged = 1 << 16, kHeadRefShift = 17, kHeadNoneShift = 19;
-// ... and whether all softmax warps meet before the item's rows are written (`placed`), with the parity of that meeting.
+// ... and whether all softmax warps meet before the item's rows are written (`placed`), with the parity of that
+// meeting.
 constexpr int kHeadMeet = 1 << 21, kHeadMeetParityShift = 22;
 
 // Where items and their K / V tiles come from.
 //   kQueue         a queue of items made by the preparatory launch, the sequence's own K and V
-//   kDirect        the same K and V, but every query block is an item (64-token blocks: not stacked), of which there are so few
-//                  that the CTAs put them in order for themselves
+//   kDirect        the same K and V, but every query block is an item (64-token blocks: not stacked), of which there
+//                  are so few that the CTAs take them in turn, in order if there are more of them than CTAs
 //   kPacked        a queue of the consumer's items, a packed buffer and the consumer's own K and V
-//   kPackedDirect  the same tiles, but the CTAs number the consumer's items and places in the buffer for themselves
+//   kPackedDirect  the same tiles, but the CTAs number the consumer's items and places in the buffer for themselves,
+//                  and put the items in order if there are more of them than CTAs
 enum class Source { kQueue, kDirect, kPacked, kPackedDirect };
 
 constexpr int kMaxDirect = 2 * 148, kMaxPackedDirect = 512;  // items of a call without a queue
@@ -190,8 +197,8 @@ struct AttnCfg {
   static constexpr int kStagesK = (D == 64) ? 4 : 3;
   static constexpr int kStagesV = (D == 64) ? 4 : 2;
   static constexpr int kTileBytes = 128 * D * 2;  // one K or V tile
-  // Q tile and K ring share kStagesK + 1 buffers: an item's Q tile takes the next buffer of the ring for as long as the item
-  // lasts, the buffer of the item before it joins the ring behind (QKRing).
+  // Q tile and K ring share kStagesK + 1 buffers: an item's Q tile takes the next buffer of the ring for as long as the
+  // item lasts, the buffer of the item before it joins the ring behind (QKRing).
   static constexpr int kBufsQK = kStagesK + 1;
   static constexpr int kOffQK = 0;
   static constexpr int kOffV = kOffQK + kBufsQK * kTileBytes;
@@ -205,8 +212,8 @@ struct AttnCfg {
   // keys against a [16 keys][column 0 = 1] block (2 KB, 128-byte swizzle like a V box), into 16 tensor-memory columns
   // of its own -- which exist only if P keeps ONE buffer instead of two (tensor memory is full otherwise)
   static constexpr bool kSum128 = (D == 128);
-  // Softmax warpgroups, each of which takes every kWGs-th tile and has an S buffer.  Three: P takes the place of the scores it
-  // was made from.  Two: one P buffer for both.
+  // Softmax warpgroups, each of which takes every kWGs-th tile and has an S buffer.  Three: P takes the place of the
+  // scores it was made from.  Two: one P buffer for both.
   static constexpr int kWGs = D == 64 ? 3 : 2;
   static constexpr bool kInPlaceP = kWGs == 3;
   static constexpr int kThreads = (2 + kWGs) * 128;  // two warpgroups of utility warps before them
@@ -225,13 +232,15 @@ struct AttnCfg {
   static constexpr int kOffMisc = kOffHead + 16 * kLists;
   static constexpr int kTotal = kOffMisc + 64;
   static constexpr int kDynamic = kTotal + 1024;  // slack for the 1024-byte alignment of the base
-  // kPackedDirect: uint32 own[P][Wd], int32 first[P][Wd] (places of a head's blocks), uint32 union[32], uint8 rank[1024]
+  // kPackedDirect: uint32 own[P][Wd], int32 first[P][Wd] (places of a head's blocks), uint32 union[32], uint8
+  // rank[1024]
   static constexpr int kOffOwn = kTotal, kOffFirst = kOffOwn + kMaxRanks * kMaxWords * 4;
   static constexpr int kOffUnion = kOffFirst + kMaxRanks * kMaxWords * 4, kOffRank = kOffUnion + kMaxWords * 4;
   static constexpr int kOffPackedOrder = kOffRank + kMaxBlocks;  // uint16 items in order
   static constexpr int kDynamicDirect = kOffPackedOrder + 2 * kMaxPackedDirect + 1024;
   // (while items are put in order, the places of entries and `first` hold counts and the list of own blocks)
-  static_assert(4 * (kMaxBlocks + 1) <= kLists * kMaxBlocks * 4 && 2 * kMaxBlocks <= kMaxRanks * kMaxWords * 4, "room for both");
+  static_assert(4 * (kMaxBlocks + 1) <= kLists * kMaxBlocks * 4, "room for the counts");
+  static_assert(2 * kMaxBlocks <= kMaxRanks * kMaxWords * 4, "room for the list");
   // kDirect: the same lengths, uint16 items in order
   static constexpr int kOffLength = kTotal, kOffOrder = kOffLength + 4 * kMaxDirect;
   static_assert(kDynamicDirect <= 232448, "shared memory budget");
@@ -274,8 +283,9 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 
 // 2^x for a pair of fp32 values on the FMA/ALU pipes (no special-function unit): round-to-nearest
 // split x = i + f, f in [-0.5, 0.5], cubic minimax polynomial for 2^f (relative error 7.5e-5, far
-// below bf16 rounding), exponent added into the bit pattern.  The result is right for |i| <= 126, and infinite in bf16 where
-// x is not a number.  kTrack: *i_max collects the largest |i|.  kClamp: x is clamped at -126 first (result >= 2^-126).
+// below bf16 rounding), exponent added into the bit pattern.  The result is right for |i| <= 126, and infinite in bf16
+// where x is not a number.  kTrack: *i_max collects the largest |i|.  kClamp: x is clamped at -126 first (result >=
+// 2^-126).
 template <bool kClamp, bool kTrack>
 __device__ __forceinline__ float2 exp2_poly2(float2 x, float* i_max) {
   const float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
@@ -295,7 +305,8 @@ __device__ __forceinline__ float2 exp2_poly2(float2 x, float* i_max) {
   return q;
 }
 
-// The output rows of query block i: zeros and a log-sum-exp of -inf.  One warp, 32 bytes a lane where the layout allows.
+// The output rows of query block i: zeros and a log-sum-exp of -inf.  One warp, 32 bytes a lane where the layout
+// allows.
 template <int D, int BLK>
 __device__ __forceinline__ void clear_rows(const AttnParams& p, int bh, int i) {
   const int lane = threadIdx.x & 31;
@@ -342,34 +353,39 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
   uint64_t* qk_empty = qk_full + C::kBufsQK;  // ... and every Q K^T that reads it has completed
   uint64_t* v_full = qk_empty + C::kBufsQK;
   uint64_t* v_empty = v_full + SV;
-  uint64_t* s_full = v_empty + SV;  // [2] S buffer written by a Q K^T
-  uint64_t* s_free = s_full + C::kWGs;  // [kWGs] S buffer read into registers by its 4 softmax warps (not where P takes its place)
+  uint64_t* s_full = v_empty + SV;  // [kWGs] S buffer written by a Q K^T
+  // [kWGs] S buffer read into registers by its 4 softmax warps (not where P takes its place)
+  uint64_t* s_free = s_full + C::kWGs;
   uint64_t* p_full = s_free + C::kWGs;  // [kWGs] P of a tile written by its 4 softmax warps
-  // [4] the P V of tile g arrives on o_full[g % 4].  Four barriers, because a parity wait can only tell the phase a barrier is
-  // in from the one before.  d = 128: a softmax thread that wants P V g-1 has itself seen P V g-3 complete, and P V g+2 cannot
-  // complete before that thread has stored P_g.  d = 64: P V g-3 was complete when the Q K^T whose scores it holds was issued.
+  // [4] the P V of tile g arrives on o_full[g % 4].  Four barriers, because a parity wait can only tell the phase a
+  // barrier is in from the one before.  d = 128: a softmax thread that wants P V g-1 has itself seen P V g-3 complete,
+  // and P V g+2 cannot complete before that thread has stored P_g.  d = 64: P V g-3 was complete when the Q K^T whose
+  // scores it holds was issued.
   uint64_t* o_full = p_full + C::kWGs;
   uint64_t* o_drained = o_full + 4;      // the item's accumulator has been read out by the four warps that write it
   uint64_t* list_ready = o_drained + 1;  // [kLists] list buffer filled
   uint64_t* list_free = list_ready + kLists;  // [kLists] list buffer no longer needed by its kListReaders
-  // [4] the four warps that own an item's first tile have left what it says in s_exact and, if that is the reference, in
-  // sRef.  Four, because a warpgroup that waits for it may be up to three tiles and as many items behind.
+  // [4] the four warps that own an item's first tile have left what it says in s_exact and, if that is the reference,
+  // in sRef.  Four, because a warpgroup that waits for it may be up to three tiles and as many items behind.
   uint64_t* ref_ready = list_free + kLists;
-  // [2][kWGs][4] the warpgroup's warp of a row group has decided about the running maximum of a tile.  Two in turn, because it may
-  // decide about the first tile of the next item before the warp behind it has noticed.  (Not named barriers, which
-  // cannot be bounded: after a wait that has run out two warps need not agree on who takes turns.  Every lane arrives: with
-  // one lane behind a __syncwarp and the count of waits in shared memory 13 heads x 2 x 6034, Q times 8, took 138 us, not 132.)
+  // [2][kWGs][4] the warpgroup's warp of a row group has decided about the running maximum of a tile.  Two in turn,
+  // because it may decide about the first tile of the next item before the warp behind it has noticed.  (Not named
+  // barriers, which cannot be bounded: after a wait that has run out two warps need not agree on who takes turns.
+  // Every lane arrives: with one lane behind a __syncwarp and the count of waits in shared memory 13 heads x 2 x 6034,
+  // Q times 8, took 138 us, not 132.)
   uint64_t* turn = ref_ready + 4;
-  // All softmax warps have come to the end of an item that they meet at.  In-place calls: all items, so that it is known whether
-  // the item is to be computed again.  Else: items that are computed again, so that the rows of the first pass, which another
-  // warpgroup may have written, and written behind its arrival on list_free, come before those of the second.
+  // All softmax warps have come to the end of an item that they meet at.  In-place calls: all items, so that it is
+  // known whether the item is to be computed again.  Else: items that are computed again, so that the rows of the first
+  // pass, which another warpgroup may have written, and written behind its arrival on list_free, come before those of
+  // the second.
   uint64_t* placed = turn + 8 * C::kWGs;
   int4* s_head = reinterpret_cast<int4*>(smem + C::kOffHead);  // [kLists] item headers
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 4);
   // [4 items][4 row groups] the group's rows take the running maximum
   volatile uint8_t* s_exact = reinterpret_cast<volatile uint8_t*>(smem + C::kOffMisc + 16);
-  volatile int* s_failed = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 32);  // [kLists] the item is to be computed again
+  // [kLists] the item is to be computed again
+  volatile int* s_failed = reinterpret_cast<volatile int*>(smem + C::kOffMisc + 32);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -423,8 +439,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
   uint32_t* sLength = reinterpret_cast<uint32_t*>(smem + C::kOffLength);
   uint16_t* sOrder = reinterpret_cast<uint16_t*>(smem + (kPackedDirect ? C::kOffPackedOrder : C::kOffOrder));
   if constexpr (kDirect) {
-    // More items than CTAs: every CTA puts all of them in order, the longest list first.  A mask row is an item; short rows
-    // share a warp's load.
+    // More items than CTAs: every CTA puts all of them in order, the longest list first.  A mask row is an item; short
+    // rows share a warp's load.
     const int n = p.BH * p.NB;
     if (n > (int)gridDim.x) {
       int width = 1;  // lanes per row: the next power of two
@@ -480,8 +496,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
       }
     }
     // More items than CTAs, because the consumer has more than its share of the blocks: every CTA puts them in order by
-    // counting their lengths.  An item is a block or two neighbours, a thread has one at most.  Items of one length stay in order
-    // of their numbers: all CTAs have to come to the same order.
+    // counting their lengths.  An item is a block or two neighbours, a thread has one at most.  Items of one length
+    // stay in order of their numbers: all CTAs have to come to the same order.
     int n_own = 0, own_before = 0, per_head = 0, n = p.BH * ((p.NB + C::kEPT - 1) / C::kEPT);
     uint32_t own = 0u;
     if (n > (int)gridDim.x) {  // (as many as if all blocks were the consumer's)
@@ -492,7 +508,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
       n = p.BH * per_head;
     }
     if (n > (int)gridDim.x) {
-      int* at = reinterpret_cast<int*>(smem + C::kOffEnt);  // [NB + 1] place NB - length: items of that length, then where they begin
+      // [NB + 1] place NB - length: items of that length, then where they begin
+      int* at = reinterpret_cast<int*>(smem + C::kOffEnt);
       uint16_t* blocks = reinterpret_cast<uint16_t*>(smem + C::kOffFirst);
       for (int t = tid; t <= p.NB; t += C::kThreads) at[t] = 0;
       for (int w = warp; w < p.Wd; w += kWarps) {  // (the same for all lanes)
@@ -555,8 +572,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SPARSP_REGS_UTILITY));
     // K (of_v = 0) or V tile n of an item's list; an absent second half re-reads the last entry
-    auto load_kv = [&](const CUtensorMap* tm, uint64_t* bar, unsigned char* dst, const EntT* ent, int n, int n_ent, int head,
-                       int batch, int of_v) {
+    auto load_kv = [&](const CUtensorMap* tm, uint64_t* bar, unsigned char* dst, const EntT* ent, int n, int n_ent,
+                       int head, int batch, int of_v) {
 #pragma unroll
       for (int e = 0; e < C::kEPT; ++e) {
         const uint32_t v = ent[min(n * C::kEPT + e, n_ent - 1)];
@@ -573,7 +590,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         if (!remote) {
           const int tok = (int)(v & (kMaxBlocks - 1)) * BLK;
 #pragma unroll
-          for (int c = 0; c < D / 64; ++c) tma_load_4d(dst + c * 16384 + e * (BLK * 128), tm, bar, c * 64, tok, head, batch);
+          for (int c = 0; c < D / 64; ++c)
+            tma_load_4d(dst + c * 16384 + e * (BLK * 128), tm, bar, c * 64, tok, head, batch);
         }
       }
     };
@@ -585,7 +603,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
           const int buf = i % kLists;
           mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 58, p.wait_limit);
           const int4 hd = s_head[buf];
-          if (hd.y == 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
+          if (hd.y == 0) break;  // (only the list builder decides when to stop: all roles stop at the same item)
           const int n_ent = hd.y & kHeadEntries, n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
           const int batch = hd.w, head = hd.x - batch * p.H;
           const EntT* ent = sEnt + buf * kMaxBlocks;
@@ -606,7 +624,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
           const int buf = i % kLists;
           mbar_wait_bounded_inline(list_ready + buf, (i / kLists) & 1, s_abort, 51, p.wait_limit);
           const int4 hd = s_head[buf];
-          if (hd.y == 0) break;  // (only the list builder decides when to stop, so that all roles stop at the same item)
+          if (hd.y == 0) break;  // (only the list builder decides when to stop: all roles stop at the same item)
           const int n_ent = hd.y & kHeadEntries, n_tiles = (n_ent + C::kEPT - 1) / C::kEPT;
           const int batch = hd.w, head = hd.x - batch * p.H;
           const EntT* ent = sEnt + buf * kMaxBlocks;
@@ -621,8 +639,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
               const int b1 = (int)((uint32_t)hd.z >> 16), bq = q && b1 != 0xffff ? b1 : hd.z & 0xffff;
 #pragma unroll
               for (int c = 0; c < D / 64; ++c)
-                tma_load_4d(sQK + b * C::kTileBytes + c * 16384 + q * (BLK * 128), &tmQ, qk_full + b, c * 64, bq * BLK, head,
-                            batch);
+                tma_load_4d(sQK + b * C::kTileBytes + c * 16384 + q * (BLK * 128), &tmQ, qk_full + b, c * 64, bq * BLK,
+                            head, batch);
             }
           }
           for (int n = 0; n < n_tiles; ++n) {
@@ -643,7 +661,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
       const uint32_t hi = (uint32_t)(desc0 >> 32);
       uint32_t lo[D / 16];
 #pragma unroll
-      for (int kk = 0; kk < D / 16; ++kk) lo[kk] = (uint32_t)desc0 + (uint32_t)(((kk / 4) * 16384 + (kk % 4) * 32) >> 4);
+      for (int kk = 0; kk < D / 16; ++kk)
+        lo[kk] = (uint32_t)desc0 + (uint32_t)(((kk / 4) * 16384 + (kk % 4) * 32) >> 4);
       QKRing<C::kStagesK> at;
       int g = 0, w = 0;     // tiles so far, the next one's warpgroup
       uint32_t round = 0u;  // parity of that warpgroup's tiles so far
@@ -659,11 +678,12 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         for (int n = 0; n < n_tiles; ++n, ++g) {
           const uint32_t bk = at.next_k();
           mbar_wait_bounded_inline(qk_full + bk, at.use(bk), s_abort, 12, p.wait_limit);
-          // an S buffer is free once its warpgroup has loaded the scores of its tile before, or the P V has read the P that
-          // took their place
+          // an S buffer is free once its warpgroup has loaded the scores of its tile before, or the P V has read the P
+          // that took their place
           if (g >= C::kWGs) {
             if (C::kInPlaceP)
-              mbar_wait_bounded_inline(o_full + ((g - C::kWGs) & 3), ((g - C::kWGs) >> 2) & 1, s_abort, 24, p.wait_limit);
+              mbar_wait_bounded_inline(o_full + ((g - C::kWGs) & 3), ((g - C::kWGs) >> 2) & 1, s_abort, 24,
+                                       p.wait_limit);
             else
               mbar_wait_bounded_inline(s_free + w, round ^ 1u, s_abort, 24, p.wait_limit);
           }
@@ -786,7 +806,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         rb1 = lane < p.Wd && blk1 >= 0 ? rows[blk1 * p.Wd + lane] : 0u;
       };
       auto fetch = [&](int it) {
-        if constexpr (kDirect || kPackedDirect) {  // the CTAs take places in order from the front and from behind in turn
+        if constexpr (kDirect || kPackedDirect) {  // the CTAs take places from the front and from behind in turn
           const int per_head = kDirect ? p.NB : (n_own + C::kEPT - 1) / C::kEPT, n = p.BH * per_head;
           bh = p.BH;
           if (it >= n) return;
@@ -837,8 +857,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         if (lane == 0) it = (int)gridDim.x + atomicAdd(p.work_counter, 1);
         return __shfl_sync(0xffffffffu, it, 0);
       };
-      // An item that has failed is handed out again.  Its verdict is there once its list buffer is free: before the buffer is
-      // used again, or, when there are no more items, one outstanding item after the other.
+      // An item that has failed is handed out again.  Its verdict is there once its list buffer is free: before the
+      // buffer is used again, or, when there are no more items, one outstanding item after the other.
       int checked = 0;  // items whose verdict has been seen
       int meetings = 0;  // items so far whose rows are written behind a meeting
       auto verdict = [&]() -> int {
@@ -1011,7 +1031,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
               if (r >= p.P || r == p.consumer) return -1;
               const uint32_t set = reinterpret_cast<const uint32_t*>(smem + C::kOffUnion)[w] & sOwn[r * p.Wd + w];
               if (!((set >> (j & 31)) & 1u)) return -1;
-              return reinterpret_cast<const int32_t*>(smem + C::kOffFirst)[r * p.Wd + w] + __popc(set & ((1u << (j & 31)) - 1u));
+              const int32_t* first = reinterpret_cast<const int32_t*>(smem + C::kOffFirst);
+              return first[r * p.Wd + w] + __popc(set & ((1u << (j & 31)) - 1u));
             } else {
               return slot[j];
             }
@@ -1047,8 +1068,9 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
       // They have nothing to do with the items, so three idle warps write them while the others work: 677 MB of an
       // attention of 40 heads x 75600 to one rank's own blocks.  A lane looks at a query block of its own, since a look
       // is one or two loads that wait for each other; neighbours go to different warps.
-      // (They are alone with it where hardly anything is kept, so no 64-bit division is in their way: nothing kept by 16 heads
-      // x 591 blocks of 128 x 64 is 49.5 us a call; 76.9 with such divisions, 16-byte stores and a sort of no items.)
+      // (They are alone with it where hardly anything is kept, so no 64-bit division is in their way: nothing kept by
+      // 16 heads x 591 blocks of 128 x 64 is 49.5 us a call; 76.9 with such divisions, 16-byte stores and a sort of no
+      // items.)
       const unsigned n_rows = (unsigned)p.BH * p.NB, warps = gridDim.x * 3, mine = blockIdx.x * 3 + warp - 5;
       for (unsigned u0 = mine; u0 < n_rows; u0 += 32 * warps) {
         const unsigned u = u0 + lane * warps;  // (batch, head, block)
@@ -1103,13 +1125,14 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         if (ref_of == kRefFirst && !exact) m_ref = ref[row];
       };
       auto take_turn = [&]() {  // the other warp has decided about the tile before, and may have moved the reference
-        mbar_wait_bounded_inline(turn + before + (turns & 1) * 4 * C::kWGs, (turns >> 1) & 1, s_abort, 44, p.wait_limit);
+        mbar_wait_bounded_inline(turn + before + (turns & 1) * 4 * C::kWGs, (turns >> 1) & 1, s_abort, 44,
+                                 p.wait_limit);
         ++turns;
         m_ref = ref[row];
       };
       auto give_turn = [&]() { mbar_arrive(turn + mine + (given++ & 1) * 4 * C::kWGs); };
-      // the row's largest score of a tile: one flat instruction stream per 64-key half, an absent half (not kept by this
-      // row's query block) is skipped
+      // the row's largest score of a tile: one flat instruction stream per 64-key half, an absent half (not kept by
+      // this row's query block) is skipped
       auto row_max = [&](const float* sv, const int* vh) {
         float mx = -INFINITY;
 #pragma unroll
@@ -1155,7 +1178,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         }
       };
 
-      // The row's reference follows its running maximum; what has been added up so far shrinks by the factor that is returned.
+      // The row's reference follows its running maximum; what has been added up so far shrinks by the factor that is
+      // returned.
       auto move_ref = [&](const float mx) -> float {
         const float m_new = fmaxf(m_ref, mx);
         if (!(m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY))) return 1.0f;
@@ -1164,9 +1188,10 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         ref[row] = m_new;
         return alpha;
       };
-      // Rescales the row's accumulator, after the exponentials of the tile, which need the new reference only, and before its P
-      // is handed over.  Every P V of the item issued so far must have landed in O; they complete in order, so the one of tile
-      // g-1 suffices, and the tile behind, which may have a factor of its own by now, waits for the P V of this one.
+      // Rescales the row's accumulator, after the exponentials of the tile, which need the new reference only, and
+      // before its P is handed over.  Every P V of the item issued so far must have landed in O; they complete in
+      // order, so the one of tile g-1 suffices, and the tile behind, which may have a factor of its own by now, waits
+      // for the P V of this one.
       auto rescale = [&](const float alpha, const int n) {
         if (n == 0 || !__any_sync(0xffffffffu, alpha != 1.0f)) return;
         const int g = g0 + n;
@@ -1190,7 +1215,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
           tmem_st16(tmem_base + C::kColL + lane_off, o);
         }
       };
-      // A tile whose P takes the place of its scores: 32 columns at a time, the next ones on their way from tensor memory.
+      // A tile whose P takes the place of its scores: 32 columns at a time, the next ones on their way from tensor
+      // memory.
       auto in_place_tile = [&](auto ragged_tag, auto exact_tag, const int n, const int* vh) {
         constexpr bool kRagged = decltype(ragged_tag)::value, kExact = decltype(exact_tag)::value;
         float va[32], vb[32];
@@ -1357,7 +1383,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
               // columns past the end of the sequence: exactly zero in P (the polynomial path returns
               // 2^-126 for them, which the row sum may keep)
 #pragma unroll
-              for (int e = 0; e < 32; ++e) pkh[e] = 2 * e + 1 < vh[h] ? pkh[e] : (2 * e < vh[h] ? (pkh[e] & 0xffffu) : 0u);
+              for (int e = 0; e < 32; ++e)
+                pkh[e] = 2 * e + 1 < vh[h] ? pkh[e] : (2 * e < vh[h] ? (pkh[e] & 0xffffu) : 0u);
             }
           } else {
 #pragma unroll
@@ -1379,9 +1406,9 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         round ^= 1u;
       };
 
-      // One tile of this warpgroup.  kRagged = the sequence ends inside the tile (possible only for the item's last one), or
-      // (K / V source) the reference comes from the first tile and this is it: that variant carries the column masking;
-      // kExact: the one with the turns.  The common variant stays small.
+      // One tile of this warpgroup.  kRagged = the sequence ends inside the tile (possible only for the item's last
+      // one), or (K / V source) the reference comes from the first tile and this is it: that variant carries the column
+      // masking; kExact: the one with the turns.  The common variant stays small.
       auto do_tile = [&](auto ragged_tag, auto exact_tag, const int n) {
         constexpr bool kRagged = decltype(ragged_tag)::value;
         // kept / valid key columns of each 64-column half of the tile (warp-uniform), as the list builder left them
@@ -1416,14 +1443,17 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         if constexpr (C::kInPlaceP) in_place_tile(ragged_tag, exact_tag, n, vh);
         else own_buffer_tile(ragged_tag, exact_tag, n, vh);
       };
-      if (exact && first == 0 && lane == 0) mbar_arrive(ref_ready + (i & 3));  // (nothing to learn: the barriers keep step)
+      // (nothing to learn: the barriers keep step)
+      if (exact && first == 0 && lane == 0) mbar_arrive(ref_ready + (i & 3));
       int n = first;
       // the list builder puts the sequence's last block (the only one that can be ragged) into the last tile
       const int n_rag = item_ragged ? n_tiles - 1 : -1;
       if (!exact) {
         for (; n < n_tiles; n += C::kWGs) {
-          if (n == n_rag || (!kPacked && ref_of == kRefFirst && n < C::kWGs)) do_tile(std::true_type{}, std::false_type{}, n);
-          else do_tile(std::false_type{}, std::false_type{}, n);
+          if (n == n_rag || (!kPacked && ref_of == kRefFirst && n < C::kWGs))
+            do_tile(std::true_type{}, std::false_type{}, n);
+          else
+            do_tile(std::false_type{}, std::false_type{}, n);
           if (exact) break;  // what the first tile says
         }
       }
@@ -1520,8 +1550,8 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
 }
 
 // ------------------------------------------------------------------------------------------------
-// Preparation of an attention call: a CTA per (batch, head) fixes its work items and, packed source, another one its table
-// of packed slots.  A query block that keeps nothing never becomes a work item.
+// Preparation of an attention call: a CTA per (batch, head) fixes its work items and, packed source, another one its
+// table of packed slots.  A query block that keeps nothing never becomes a work item.
 //
 // Block 64: which two query blocks share a Q tile.  K / V source: blocks i and i+D are paired in stripes (i mod 2D <
 // D), leftovers pair up consecutively; the offset D in 1..n/2 that maximises the summed overlap |M[i] & M[i+D]| of the
@@ -1530,15 +1560,16 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
 // tile's work is masked away.
 // Packed source: neighbours in the consumer's ascending list of blocks (D = 1), so that a row's result depends on its
 // neighbour's list at most, not on what the consumer's other blocks keep.
-// (Mask rows in shared memory have a pitch of an odd number of 16-byte units, which are read whole: the threads' offsets differ
-// by one row, an even pitch would put many of them on the same banks.)
-// Items of one (batch, head) are handed out longest list first: the items still running when the queue
-// runs dry are then the short ones, which matters when list lengths vary (threshold selection, unions of two
-// stacked blocks).  Key = (list length << 10) | (1023 - index): equal lengths keep their index order.
+// (Mask rows in shared memory have a pitch of an odd number of 16-byte units, which are read whole: the threads'
+// offsets differ by one row, an even pitch would put many of them on the same banks.)
+// Items of one (batch, head) are handed out longest list first: the items still running when the queue runs dry are
+// then the short ones, which matters when list lengths vary (threshold selection, unions of two stacked blocks).  Key =
+// (list length << 10) | (1023 - index): up to kPrepThreads / 2 items of equal length keep their index order, more of
+// them are in any order.
 // Latency-bound integer work, so what matters is how many loads and barriers wait for each other: rows are counted by a
-// warp each with eight in flight, items are put in order without rounds, offsets are scored by all threads, and
-// slots have CTAs of their own and no shared-memory atomics.  One hop of 40 heads x 591 blocks, 8 ranks 5.9 us (23 with
-// 256 threads, a thread per row, a bitonic sort for any number and the slots behind the items), 24 x 384 stacked blocks
+// warp each with eight in flight, items are put in order without rounds, offsets are scored by all threads, and slots
+// have CTAs of their own and no shared-memory atomics.  One hop of 40 heads x 591 blocks, 8 ranks 5.9 us (23 with 256
+// threads, a thread per row, a bitonic sort for any number and the slots behind the items), 24 x 384 stacked blocks
 // 15.5, 2 x 64 4.5 (attention calls 72 -> 66-74, 617 -> 594 and 21.2 -> 19.4 us).
 // ------------------------------------------------------------------------------------------------
 constexpr int kPrepThreads = 512;
@@ -1562,12 +1593,13 @@ struct PrepParams {
   int P, consumer;
 };
 
-// Sorts n keys (n a power of two; up to kPrepThreads / 2, or kMany: 1024) in shared memory by length, the longest first; all threads
-// call it.
+// Sorts n keys (n a power of two; up to kPrepThreads / 2, or kMany: 1024) in shared memory by length, the longest
+// first; all threads call it.
 template <bool kMany>
 __device__ __forceinline__ void sort_keys_descending(uint32_t* keys, int n) {
   if constexpr (!kMany) {
-    // Few keys: a key's place is the number of larger ones, counted by two threads.  No rounds that wait for each other.
+    // Few keys: a key's place is the number of larger ones, counted by two threads.  No rounds that wait for each
+    // other.
     const int k = threadIdx.x >> 1;
     const uint32_t key = k < n ? keys[k] : 0u;
     int place = 0;
@@ -1583,7 +1615,8 @@ __device__ __forceinline__ void sort_keys_descending(uint32_t* keys, int n) {
     // Many keys: a place for every length, by counting; equal lengths in any order, a warp's together.
     constexpr int kLens = kMaxBlocks + 1, kPer = (kLens + kPrepThreads - 1) / kPrepThreads, kWarps = kPrepThreads / 32;
     constexpr int kKeys = kMaxBlocks / kPrepThreads;
-    __shared__ int at_s[kPer * kPrepThreads], sum_s[kWarps];  // place kLens - 1 - length: keys of that length, then where they begin
+    // place kLens - 1 - length: keys of that length, then where they begin
+    __shared__ int at_s[kPer * kPrepThreads], sum_s[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int t = 0; t < kPer; ++t) at_s[threadIdx.x + t * kPrepThreads] = 0;
@@ -1814,8 +1847,8 @@ __device__ __forceinline__ void make_slots(const PrepParams& p, int bh) {
   }
 }
 
-// (An instance for each form, because the launch waits for the code it is given: with all of it in one, layers of a few thousand
-// tokens took 6 us longer.)
+// (An instance for each form, because the launch waits for the code it is given: with all of it in one, layers of a few
+// thousand tokens took 6 us longer.)
 template <bool kPacked, bool kStacked, bool kMany>
 __global__ void __launch_bounds__(kPrepThreads) attn_prep_kernel(const PrepParams p) {
   enter_grid();
@@ -1937,16 +1970,19 @@ static int launch_attn_t(const sparsp_shape& s, const Geometry& g, const void* Q
     tp = tk;  // never used
   }
   auto kern = attn_fwd_kernel<D, BLK, kSource>;
-  const int smem = kSource == Source::kPackedDirect || kSource == Source::kDirect ? AttnCfg<D, BLK>::kDynamicDirect : AttnCfg<D, BLK>::kDynamic;
+  constexpr bool kNoQueue = kSource == Source::kPackedDirect || kSource == Source::kDirect;
+  const int smem = kNoQueue ? AttnCfg<D, BLK>::kDynamicDirect : AttnCfg<D, BLK>::kDynamic;
   SPARSP_CUDA_OK(ensure_dynamic_smem((const void*)kern, smem));
-  // work item = one 128-row Q tile (a 128-token block, a pair of 64-token blocks, or one of them); one persistent CTA per SM
+  // work item = one 128-row Q tile (a 128-token block, a pair of 64-token blocks, or one of them); one persistent CTA
+  // per SM
   const int64_t most = (int64_t)g.B * g.H * (BLK == 128 || kSource == Source::kDirect ? g.NB : (g.NB + 1) / 2);
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
   const unsigned grid = (unsigned)std::min<int64_t>(most, sms);
-  // The warpgroups share out the registers that the block is launched with; should a build of the kernel be given fewer, some
-  // of them would wait for good.
-  constexpr int kShared = 128 * (SPARSP_REGS_UTILITY + SPARSP_REGS_UTILITY2 + AttnCfg<D, BLK>::kWGs * AttnCfg<D, BLK>::kRegsSoftmax);
+  // The warpgroups share out the registers that the block is launched with; should a build of the kernel be given
+  // fewer, some of them would wait for good.
+  constexpr int kSoftmax = AttnCfg<D, BLK>::kWGs * AttnCfg<D, BLK>::kRegsSoftmax;
+  constexpr int kShared = 128 * (SPARSP_REGS_UTILITY + SPARSP_REGS_UTILITY2 + kSoftmax);
   static std::atomic<int> launched_with{0};
   if (launched_with.load(std::memory_order_relaxed) < kShared) {
     cudaFuncAttributes attr;
@@ -2017,14 +2053,15 @@ int launch_attn(const sparsp_shape& s, const Geometry& g, const void* Q, const v
                 cudaStream_t st) {
   AttnParams p = {};
   p.mask = mask;
-  // So few query blocks need no queue and no launch that fills it.  64-token blocks: one an SM; an item is then done sooner with
-  // its own list than with the union of two (us a call with the launch that makes items / without it: 2 heads x 64 blocks of 64
-  // x 64, 16 kept 14.9 / 11.5, stacked 19.4).  More of them have to share Q tiles where neighbours keep the same blocks: 2 x 100
-  // of 64 x 128, a quarter kept in windows 22.5 with the queue, 30.9 unstacked, all kept 50 / 83 (threshold lists, whose unions
-  // are long, would gain: 2 x 120 77 / 52).  128-token blocks: two an SM; every CTA puts them in order for itself and takes one
-  // from the front and one from behind (7 x 21 of 64 x 128 15.7 / 10.4, 2 x 148 of 128 x 128, 15 % kept 58.5 / 52.9, threshold
-  // lists 67 / 54; up to three an SM 0.90 to 1.10 times as fast, up to four 0.80 to 1.04).  An instance of the kernel of its own,
-  // because the question inside the queue's made 64-token blocks 1-2 % slower.
+  // So few query blocks need no queue and no launch that fills it.  64-token blocks: one an SM; an item is then done
+  // sooner with its own list than with the union of two (us a call with the launch that makes items / without it: 2
+  // heads x 64 blocks of 64 x 64, 16 kept 14.9 / 11.5, stacked 19.4).  More of them have to share Q tiles where
+  // neighbours keep the same blocks: 2 x 100 of 64 x 128, a quarter kept in windows 22.5 with the queue, 30.9
+  // unstacked, all kept 50 / 83 (threshold lists, whose unions are long, would gain: 2 x 120 77 / 52).  128-token
+  // blocks: two an SM; every CTA puts them in order for itself and takes one from the front and one from behind (7 x 21
+  // of 64 x 128 15.7 / 10.4, 2 x 148 of 128 x 128, 15 % kept 58.5 / 52.9, threshold lists 67 / 54; up to three an SM
+  // 0.90 to 1.10 times as fast, up to four 0.80 to 1.04).  An instance of the kernel of its own, because the question
+  // inside the queue's made 64-token blocks 1-2 % slower.
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
   if ((int64_t)g.B * g.H * g.NB <= std::min((g.b == 64 ? 1 : 2) * sms, kMaxDirect))
@@ -2050,14 +2087,15 @@ int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, 
   p.mask = mask;
   p.rank = rank;
   p.consumer = consumer;
-  // Where the consumer has one item an SM at most, if it has its share of the blocks, neither their order nor a queue matters,
-  // and the launch that makes them is left out: us a call over a whole buffer, with the launch / without, 1 head x 43 blocks, 5
-  // ranks 18.5 / 16.4; an even share of 8 ranks, 15 % kept, 2 x 140 of 64 x 128 26.8 / 25.0, 4 x 97 of 64 x 128 21.2 / 19.1, 8 x 128
-  // of 64 x 128 27.1 / 24.7; a hop of 6 x 140 15.2 / 13.0.  If the consumer has more than its share, the CTAs put its items in
-  // order for themselves, up to 512 of them: 30 % of 8 x 128 42.9 / 42.0, with lists of unequal length 49.3 / 37.9, all of it 80.7
-  // / 79.4, but short lists, 4 % kept, 39.9 / 43.3.  (In order of their numbers lists of unequal length took up to 1.7 times as
-  // long, half of 1 x 300 of 128 x 128 75 / 110.  With two items an SM by an even share 4 x 300 of 128 x 128 34 / 44; with up to 1024
-  // to put in order 2 x 1000 of 64 x 128 240 / 265.)
+  // Where the consumer has one item an SM at most, if it has its share of the blocks, neither their order nor a queue
+  // matters, and the launch that makes them is left out: us a call over a whole buffer, with the launch / without, 1
+  // head x 43 blocks, 5 ranks 18.5 / 16.4; an even share of 8 ranks, 15 % kept, 2 x 140 of 64 x 128 26.8 / 25.0, 4 x 97
+  // of 64 x 128 21.2 / 19.1, 8 x 128 of 64 x 128 27.1 / 24.7; a hop of 6 x 140 15.2 / 13.0.  If the consumer has more
+  // than its share, the CTAs put its items in order for themselves, up to 512 of them: 30 % of 8 x 128 42.9 / 42.0,
+  // with lists of unequal length 49.3 / 37.9, all of it 80.7 / 79.4, but short lists, 4 % kept, 39.9 / 43.3.  (In order
+  // of their numbers lists of unequal length took up to 1.7 times as long, half of 1 x 300 of 128 x 128 75 / 110.  With
+  // two items an SM by an even share 4 x 300 of 128 x 128 34 / 44; with up to 1024 to put in order 2 x 1000 of 64 x 128
+  // 240 / 265.)
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
   const int64_t BH = (int64_t)g.B * g.H, share = (g.NB + P - 1) / P, per_item = 128 / g.b;

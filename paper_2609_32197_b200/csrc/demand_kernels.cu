@@ -69,29 +69,31 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
   }
 }
 
-// Unions, counts and offsets of a plan without destinations, in one launch: a cluster of CTAs per consumer takes the consumer's
-// heads in turn, meets when all counts are there, and its first CTA scans them.  Nothing is kept between launches.
-// Latency-bound, and what is saved is the host's time for a launch.  So a CTA makes its lists by ballots, matches and counting
-// bits, with eight rows in flight, the last ones too (the lists of the kernel above, of atomics, are fewer instructions, which
-// is what bounds it where CTAs are many: 2 x 48 heads x 512 blocks, 16 ranks 15.0 us a plan against 18.5 with lists like these).
-// us a plan with two launches / this way, one call behind the other and in a graph, where the host is out of it: 2 heads x 64
-// blocks, 4 ranks 7.4 / 5.1 and 4.0 / 3.9; 4 x 1000, 8 ranks 7.6 / 5.1 and 5.8 / 4.7; 13 x 77, 5 ranks 7.6 / 5.1 and 4.3 / 4.5;
-// 16 x 177, 8 ranks 7.6 / 5.2 and 4.6 / 4.7; 24 x 384, 4 ranks 8.0 / 5.8 and 4.9 / 5.4.  Several heads a CTA take too long where
-// rows are many and wide, 16 x 1000, 2 ranks 8.3 / 9.0 and 7.6 / 8.5, 24 x 929, 8 ranks 7.5 / 8.3 and 7.0 / 7.0, where there are
-// more than eight clusters, 16 x 300, 11 ranks 7.6 / 6.7 and 5.0 / 6.8, 24 x 300 7.8 / 8.7 and 6.1 / 8.1, and so do more than three:
-// 48 x 278, 3 ranks 7.6 / 7.9 and 5.2 / 7.5.
+// Unions, counts and offsets of a plan without destinations, in one launch: a cluster of CTAs per consumer takes the
+// consumer's heads in turn, meets when all counts are there, and its first CTA scans them.  Nothing is kept between
+// launches.  Latency-bound, and what is saved is the host's time for a launch.  So a CTA makes its lists by ballots,
+// matches and counting bits, with eight rows in flight, the last ones too (the lists of the kernel above, of atomics,
+// are fewer instructions, which is what bounds it where CTAs are many: 2 x 48 heads x 512 blocks, 16 ranks 15.0 us a
+// plan against 18.5 with lists like these).  us a plan with two launches / this way, one call behind the other and in a
+// graph, where the host is out of it: 2 heads x 64 blocks, 4 ranks 7.4 / 5.1 and 4.0 / 3.9; 4 x 1000, 8 ranks 7.6 / 5.1
+// and 5.8 / 4.7; 13 x 77, 5 ranks 7.6 / 5.1 and 4.3 / 4.5; 16 x 177, 8 ranks 7.6 / 5.2 and 4.6 / 4.7; 24 x 384, 4 ranks
+// 8.0 / 5.8 and 4.9 / 5.4.  Several heads a CTA take too long where rows are many and wide, 16 x 1000, 2 ranks 8.3 /
+// 9.0 and 7.6 / 8.5, 24 x 929, 8 ranks 7.5 / 8.3 and 7.0 / 7.0, where there are more than eight clusters, 16 x 300, 11
+// ranks 7.6 / 6.7 and 5.0 / 6.8, 24 x 300 7.8 / 8.7 and 6.1 / 8.1, and so do more than three: 48 x 278, 3 ranks 7.6 /
+// 7.9 and 5.2 / 7.5.
 constexpr int kPlanCtas = 8, kPlanHeads = 3;                    // CTAs of a cluster, heads that one takes
 constexpr int kPlanAtOnce = 64;                                // CTAs of a launch, where they take several heads
 constexpr int kPlanWordsOfTwo = 20480, kPlanWordsOfThree = 4096;  // mask words of two and of three heads
 static bool plan_fits_clusters(const Geometry& g, int P, int sms) {
   const int ctas = std::min(g.H, kPlanCtas), heads = (g.H + ctas - 1) / ctas, rows = (g.NB + P - 1) / P;
   const int words = heads == 1 ? 0 : heads * rows * g.Wd, most = heads <= 2 ? kPlanWordsOfTwo : kPlanWordsOfThree;
-  return heads <= kPlanHeads && words <= most && g.H * P <= kUnionThreads && g.B * P * ctas <= (heads == 1 ? sms : kPlanAtOnce);
+  return heads <= kPlanHeads && words <= most && g.H * P <= kUnionThreads &&
+         g.B * P * ctas <= (heads == 1 ? sms : kPlanAtOnce);
 }
 
 __global__ void __launch_bounds__(kUnionThreads)
-    cluster_plan_kernel(const uint32_t* __restrict__ mask, const int32_t* __restrict__ rank, int H, int NB, int Wd, int P,
-                        uint32_t* __restrict__ U, int include_local, int32_t* __restrict__ cnt,
+    cluster_plan_kernel(const uint32_t* __restrict__ mask, const int32_t* __restrict__ rank, int H, int NB, int Wd,
+                        int P, uint32_t* __restrict__ U, int include_local, int32_t* __restrict__ cnt,
                         int64_t* __restrict__ seg_off, int64_t* __restrict__ seg_total, int64_t* __restrict__ volume,
                         int64_t entry_bytes) {
   enter_grid(mask, rank);
@@ -378,8 +380,8 @@ int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_o
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
   if (plan_fits_clusters(g, P, sms)) {
-    SPARSP_CUDA_OK(launch_clusters(cluster_plan_kernel, g.B * P * ctas, ctas, kUnionThreads, 0, st, mask, rank_of_block, g.H,
-                                   g.NB, g.Wd, P, U, local, cnt, seg_off, seg_total, volume, 2LL * g.b * g.d * 2));
+    SPARSP_CUDA_OK(launch_clusters(cluster_plan_kernel, g.B * P * ctas, ctas, kUnionThreads, 0, st, mask, rank_of_block,
+                                   g.H, g.NB, g.Wd, P, U, local, cnt, seg_off, seg_total, volume, 2LL * g.b * g.d * 2));
     return SPARSP_OK;
   }
   SPARSP_CUDA_OK(launch_plan(g, mask, rank_of_block, P, local, U, cnt, seg_off, seg_total, volume, nullptr, -1, nullptr,
@@ -402,9 +404,9 @@ int launch_demand(const Geometry& g, const uint32_t* mask, const int32_t* rank_o
 constexpr int kPackStages = 5;
 constexpr int kPackMaxWarps = 4;
 
-// Nobody reads the copies before a consumer fetches them, so the L2 cache need not keep them: the sources, which are read
-// again for other consumers, and K and V stay there longer (demand and gather of 24 heads x 24576 226.5 -> 224 us, of 48 x
-// 17776 328.5 -> 325.5, of 40 x 75600 2221 -> 2207; seven segments 394.7 -> 392).
+// Nobody reads the copies before a consumer fetches them, so the L2 cache need not keep them: the sources, which are
+// read again for other consumers, and K and V stay there longer (demand and gather of 24 heads x 24576 226.5 -> 224 us,
+// of 48 x 17776 328.5 -> 325.5, of 40 x 75600 2221 -> 2207; seven segments 394.7 -> 392).
 __device__ __forceinline__ void bulk_store(void* gdst, const void* smem_src, uint32_t bytes) {
   uint64_t policy;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
@@ -469,7 +471,8 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps) pack_kernel(const __grid_c
   for (int q = 0; q < n_local; ++q) {
     const int64_t half = which(q) ? tile_bytes : 0;
     const unsigned char* buf = ring + (size_t)(q % kPackStages) * tile_bytes;
-    ptx::mbar_wait_bounded(full + q % kPackStages, (uint32_t)((q / kPackStages) & 1), &s_abort, status, 50, 200000000LL);
+    ptx::mbar_wait_bounded(full + q % kPackStages, (uint32_t)((q / kPackStages) & 1), &s_abort, status, 50,
+                           200000000LL);
     if (d0 >= 0) bulk_store(packed + d0 + half, buf, tile_bytes);
     if (d1 >= 0) bulk_store(packed + d1 + half, buf, tile_bytes);
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -513,35 +516,35 @@ static int prepare_pack(const sparsp_shape& s, const Geometry& g, const void* K,
 }
 
 // ------------------------------------------------------------------------------------------------
-// Offsets and gather in one launch, for plans of up to kScanMax counts: every CTA scans the counts of all consumers into
-// shared memory (their flat order is the order of the packed buffers), and a copy's place is its segment's first entry
-// plus the blocks of the segment below it, counted in the union words by the lane of its consumer.  The other half of its
-// warps meanwhile numbers the blocks that anybody receives, of all heads, so that only those are handed out.  No tables, no
-// list of sources in memory and no launch that makes them.  The first CTAs also write the offsets, totals and volumes.  Tiles
-// move as in pack_kernel, a block's K and V together (an entry is one store), kGatherStages - 1 blocks of loads in flight.
-// us of the whole call with tables and the n-th source of the list for the n-th warp / this way: 40 heads x 75600, 8 ranks
-// 2176 / 1931 (6.4 TB/s), 24 x 118800 1714 / 1522, 48 x 17776 322 / 287, 24 x 24576, 4 ranks 223 / 200, 2 x 13 x 6034, 3
-// ranks 18.0 / 13.9, 2 x 4096 18.3 / 10.3.  What held it back was not memory but warps whose blocks happened to have many
-// consumers.  Where little is wanted, with tables / this way / with every block handed out and looked up, wanted or not: 40
-// heads x 591 blocks of 128 x 128, a band of two blocks either side, 8 ranks 38 / 38 / 158, one rank 12.6 / 11 / 96, two heads
-// of all 129 / 115 / 231.
-// The counts, the words of live blocks and a table of owners have to fit beside the rings, and every CTA scans all of them: a
-// few us at 6144 counts (24 heads, 16 ranks 1712 / 1483; one more head, by tables, 1784 / 1770).
+// Offsets and gather in one launch, for plans of up to kScanMax counts: every CTA scans the counts of all consumers
+// into shared memory (their flat order is the order of the packed buffers), and a copy's place is its segment's first
+// entry plus the blocks of the segment below it, counted in the union words by the lane of its consumer.  The other
+// half of its warps meanwhile numbers the blocks that anybody receives, of all heads, so that only those are handed
+// out.  No tables, no list of sources in memory and no launch that makes them.  The first CTAs also write the offsets,
+// totals and volumes.  Tiles move as in pack_kernel, a block's K and V together (an entry is one store), kGatherStages
+// - 1 blocks of loads in flight.  us of the whole call with tables and the n-th source of the list for the n-th warp /
+// this way: 40 heads x 75600, 8 ranks 2176 / 1931 (6.4 TB/s), 24 x 118800 1714 / 1522, 48 x 17776 322 / 287, 24 x
+// 24576, 4 ranks 223 / 200, 2 x 13 x 6034, 3 ranks 18.0 / 13.9, 2 x 4096 18.3 / 10.3.  What held it back was not memory
+// but warps whose blocks happened to have many consumers.  Where little is wanted, with tables / this way / with every
+// block handed out and looked up, wanted or not: 40 heads x 591 blocks of 128 x 128, a band of two blocks either side,
+// 8 ranks 38 / 38 / 158, one rank 12.6 / 11 / 96, two heads of all 129 / 115 / 231.
+// The counts, the words of live blocks and a table of owners have to fit beside the rings, and every CTA scans all of
+// them: a few us at 6144 counts (24 heads, 16 ranks 1712 / 1483; one more head, by tables, 1784 / 1770).
 // ------------------------------------------------------------------------------------------------
 constexpr int kScanMax = 6144;
-// Masks of up to kMaskMax words are read by every CTA, which makes the unions and counts for itself (kFromMask): no launch of
-// the union before it.  A warp then gets every n-th block, of which there are few enough for that.  us of the whole call with
-// the union's launch / without: 2 heads x 64 blocks, 4 ranks 10.2 / 8.1; 7 x 21 of d = 128, 7 ranks 11.5 / 8.5; 48 x 13 of 128
-// x 128, 7 ranks 27.0 / 23.0; 2 x 13 x 48, 3 ranks 13.3 / 11.6; 40 x 40, 8 ranks 29.9 / 28.4 (3200 words); beyond the line 24 x
-// 80 (5760 words) 20.2 / 22.7, 9 x 166 (8964) 27.9 / 31.2; 16 x 64 of 128 x 128 in 7 blocks a warp 43.8 / 44.3.  Between four and six
-// blocks a warp only with half of the words: 13 x 60 of 128 x 128, 4 ranks (1560 words) 38.2 / 36.3, but 5 x 144, 14 ranks (3600)
-// 78.3 / 81.1, 7 x 120, 8 ranks (3360) 69.0 / 72.5.
+// Masks of up to kMaskMax words are read by every CTA, which makes the unions and counts for itself (kFromMask): no
+// launch of the union before it.  A warp then gets every n-th block, of which there are few enough for that.  us of the
+// whole call with the union's launch / without: 2 heads x 64 blocks, 4 ranks 10.2 / 8.1; 7 x 21 of d = 128, 7 ranks
+// 11.5 / 8.5; 48 x 13 of 128 x 128, 7 ranks 27.0 / 23.0; 2 x 13 x 48, 3 ranks 13.3 / 11.6; 40 x 40, 8 ranks 29.9 / 28.4
+// (3200 words); beyond the line 24 x 80 (5760 words) 20.2 / 22.7, 9 x 166 (8964) 27.9 / 31.2; 16 x 64 of 128 x 128 in 7
+// blocks a warp 43.8 / 44.3.  Between four and six blocks a warp only with half of the words: 13 x 60 of 128 x 128, 4
+// ranks (1560 words) 38.2 / 36.3, but 5 x 144, 14 ranks (3600) 78.3 / 81.1, 7 x 120, 8 ranks (3360) 69.0 / 72.5.
 constexpr int kMaskMax = 4096, kFromMaskBlocks = 6, kFromMaskFew = 4;
 constexpr int kGatherStages = 3, kGatherThreads = 512;
 constexpr int kGatherSmem = 232448 - 7 * 1024;  // dynamic shared memory, next to less than 7 KB of its own
 
-// out[i] = sum of value(0 .. i - 1) for i <= n, in two steps with a barrier between them and one behind: n_warps warps, of
-// which this one is `warp`, scan a part each, then add what lies before it.
+// out[i] = sum of value(0 .. i - 1) for i <= n, in two steps with a barrier between them and one behind: n_warps warps,
+// of which this one is `warp`, scan a part each, then add what lies before it.
 template <int kUnroll, typename F>
 __device__ __forceinline__ void scan_part(int n, int warp, int n_warps, int32_t* out, int* warp_s, F value) {
   const int lane = threadIdx.x & 31;
@@ -605,9 +608,9 @@ __global__ void __launch_bounds__(kGatherThreads)
     ptx::mbar_init(full_all + threadIdx.x, 1);
     ptx::mbar_init_fence();
   }
-  // The launches behind this one begin when its CTAs end: an attention that takes its places while CTAs are still copying
-  // makes the step longer (mask, demand and gather, attention of 2 x 13 x 6034 tokens 138 us, 131 this way, 141 with the
-  // gather by tables; of 2 x 4096 39.2, 38.8 and 41).
+  // The launches behind this one begin when its CTAs end: an attention that takes its places while CTAs are still
+  // copying makes the step longer (mask, demand and gather, attention of 2 x 13 x 6034 tokens 138 us, 131 this way, 141
+  // with the gather by tables; of 2 x 4096 39.2, 38.8 and 41).
   const uint32_t* U = U_out;
   const int32_t* cnt = cnt_out;
   wait_previous_grids(mask, U, rank, cnt, dst_base);
@@ -722,7 +725,8 @@ __global__ void __launch_bounds__(kGatherThreads)
       const int bit = __ffs(left) - 1, bh = word / Wd, w = word - bh * Wd, j = w * 32 + bit;
       // its owner, looked for by a lane per rank
       int p = __ffs(__ballot_sync(0xffffffffu, lane < P && ((own_s[lane * Wd + w] >> bit) & 1u))) - 1;
-      if (p < 0) p = 31 + __ffs(__ballot_sync(0xffffffffu, lane + 32 < P && ((own_s[(lane + 32) * Wd + w] >> bit) & 1u)));
+      if (p < 0)
+        p = 31 + __ffs(__ballot_sync(0xffffffffu, lane + 32 < P && ((own_s[(lane + 32) * Wd + w] >> bit) & 1u)));
       const int bb = bh / H, h = bh - bb * H;
       bool any = false;
 #pragma unroll 1
@@ -809,15 +813,16 @@ int launch_demand_pack(const sparsp_shape& s, const Geometry& g, const uint32_t*
 }
 
 // ------------------------------------------------------------------------------------------------
-// Pack of ONE (consumer, producer) segment (Section 6.1: the producer packs the payload of one consumer into
-// the slot designated for that pair).  Entry (h, j) sits where it sits inside the consumer's buffer, minus the segment's
-// first entry, so that consumer and producer derive the same byte ranges from the demand counts.
+// Pack of ONE (consumer, producer) segment (Section 6.1: the producer packs the payload of one consumer into the slot
+// designated for that pair).  Entry (h, j) sits where it sits inside the consumer's buffer, minus the segment's first
+// entry, so that consumer and producer derive the same byte ranges from the demand counts.
 // The entries are U[consumer][h] & own[producer], head by head, blocks ascending.  Their places in the slot are
 // consecutive, so a warp that takes every n-th entry finds its head in the offsets and its block by counting bits: no
 // tables and no launch that fills them.  Tiles move as in pack_kernel.  HBM-bound: seven segments of 175 MB, read and
 // written, 426 us with tables, 382-384 this way (6.4 TB/s); 421 with a run of consecutive entries per warp instead of
-// every n-th.  Three tiles per warp: with two loads in flight reads and writes alternate best (four 390, five 394).  Small
-// segments, 80 entries of 40 heads / 400 of 200: 9.2 / 9.0 us with tables, 6.2 / 6.2; walking from head to head 18 / 52.
+// every n-th.  Three tiles per warp: with two loads in flight reads and writes alternate best (four 390, five 394).
+// Small segments, 80 entries of 40 heads / 400 of 200: 9.2 / 9.0 us with tables, 6.2 / 6.2; walking from head to head
+// 18 / 52.
 // ------------------------------------------------------------------------------------------------
 constexpr int kSegmentStages = 3;
 
@@ -870,8 +875,8 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps)
       return lo;
     };
     auto head_words = [&](int h) { return lane < Wd ? u_row[(int64_t)h * Wd + lane] & own : 0u; };
-    // The head of the next entry to load, its first entry, and its words on their way.  Where the heads begin is kept a lane
-    // per head, 32 of them in the direction of the walk, so that a look needs no load.
+    // The head of the next entry to load, its first entry, and its words on their way.  Where the heads begin is kept a
+    // lane per head, 32 of them in the direction of the walk, so that a look needs no load.
     int h, at, h0, x_at;
     uint32_t words;
     auto keep_heads = [&](int from) {
@@ -892,8 +897,8 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps)
     };
     keep_heads(head_of(entry(0)));
     look_up(entry(0));
-    // head * NB + block of entry e, which has been looked up; -1 where there is none, should the counts promise more than
-    // there are
+    // head * NB + block of entry e, which has been looked up; -1 where there is none, should the counts promise more
+    // than there are
     auto block_of = [&](int e) -> int {
       int total;
       const int below = bits_below(words, lane, &total), k = e - at;
@@ -922,7 +927,8 @@ __global__ void __launch_bounds__(32 * kPackMaxWarps)
     for (int q = 0; q < kSegmentStages - 1 && q < n_local; ++q) issue_load(q);
     for (int q = 0; q < n_local; ++q) {
       const int64_t e = entry(q);
-      ptx::mbar_wait_bounded(full + q % kSegmentStages, (uint32_t)((q / kSegmentStages) & 1), &s_abort, status, 50, 200000000LL);
+      ptx::mbar_wait_bounded(full + q % kSegmentStages, (uint32_t)((q / kSegmentStages) & 1), &s_abort, status, 50,
+                             200000000LL);
       if (lane == 0) {
         if ((e + 1) * 2 * tile_bytes <= capacity)
           bulk_store(slot + (2 * e + (q & 1)) * tile_bytes, ring + (size_t)(q % kSegmentStages) * tile_bytes, tile_bytes);

@@ -1,5 +1,5 @@
-// Which work item a number of the attention kernel's queue stands for (K / V source), and which buffer a tile of an item
-// lies in.  Plain integer code, apart from the kernel so that it can be run on a host as well.
+// Which work item a number of the attention kernel's queue stands for (K / V source), and which buffer a tile of an
+// item lies in.  Plain integer code, apart from the kernel so that it can be run on a host as well.
 #pragma once
 
 #include <stdint.h>
@@ -29,8 +29,8 @@ SPARSP_QUEUE_FN int find_item(int it, int per_head, int n_heads, const int32_t* 
   return head;
 }
 
-// Which of the kRing + 1 shared buffers the next Q or K tile lies in, and the parity of its use: the producer and the Q K^T
-// issuer both follow the same sequence of tiles.  A nibble per buffer, the next one lowest.
+// Which of the kRing + 1 shared buffers the next Q or K tile lies in, and the parity of its use: the producer and the Q
+// K^T issuer both follow the same sequence of tiles.  A nibble per buffer, the next one lowest.
 template <int kRing>
 struct QKRing {
   uint32_t ring = kRing == 4 ? 0x3210u : 0x210u;

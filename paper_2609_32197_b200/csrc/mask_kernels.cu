@@ -12,13 +12,13 @@
 namespace sparsp {
 
 // ------------------------------------------------------------------------------------------------
-// pool: a warp per (tensor, batch*head, block) tile, a CTA of its own.  The tile comes into shared memory as one TMA load
-// (any token stride; rows behind the last token arrive as zeros), so all of it is in flight at once and as many tiles per
-// multiprocessor as fit there; a lane then adds its 2 or 4 channels row by row, every channel one sequential chain.
-// HBM-bound where there are many tiles, one memory latency and the chain of `block` additions where there are few.
-// us of a whole mask call with loads through registers (8 to 32 rows in flight a lane) / this way: 40 heads x 75600 x 128
-// 486 / 419, 24 x 24576 115 / 100 (pool alone 53.6 -> about 46, 6.5 TB/s), 48 x 17776 x 64 89 / 81, 2 x 13 x 6034 x 64
-// token-major 18.6 / 13.1, 48 heads x 1558 token-major 23.9 / 14.5, 2 x 4096 x 64 11.7 / 9.9.
+// pool: a warp per (tensor, batch*head, block) tile, a CTA of its own.  The tile comes into shared memory as one TMA
+// load (any token stride; rows behind the last token arrive as zeros), so all of it is in flight at once and as many
+// tiles per multiprocessor as fit there; a lane then adds its 2 or 4 channels row by row, every channel one sequential
+// chain.  HBM-bound where there are many tiles, one memory latency and the chain of `block` additions where there are
+// few.  us of a whole mask call with loads through registers (8 to 32 rows in flight a lane) / this way: 40 heads x
+// 75600 x 128 486 / 419, 24 x 24576 115 / 100 (pool alone 53.6 -> about 46, 6.5 TB/s), 48 x 17776 x 64 89 / 81, 2 x 13
+// x 6034 x 64 token-major 18.6 / 13.1, 48 heads x 1558 token-major 23.9 / 14.5, 2 x 4096 x 64 11.7 / 9.9.
 // ------------------------------------------------------------------------------------------------
 template <int D>
 __global__ void __launch_bounds__(32) pool_kernel(const __grid_constant__ CUtensorMap tmQ,
@@ -406,13 +406,14 @@ __global__ void __launch_bounds__(kTopkWarps * 32, WMAX <= 12 ? 4 : WMAX <= 20 ?
 }
 
 // ------------------------------------------------------------------------------------------------
-// Scores and selection of short rows (up to 128 blocks) in one launch: a CTA keeps the pooled K of its head in shared memory
-// and takes a few rows of it, a warp each, whose scores never leave the registers they are selected from.  Same chains, same
-// selection.  What bounds it is the latency of the launch, of bringing pooled K in (16 warps, more than have a row) and of one
-// row: few rows a CTA while all CTAs run at once, more where pooled K would be read too often.  us of a whole mask call, two
-// launches / this way: 2 heads x 64 blocks of d = 64 9.7 / 7.6, 7 x 21 of d = 128 13.5 / 7.7, 2 x 68 15.2 / 9.6, 5 x 108 18.3 /
-// 12.0, 26 x 48 of d = 64 13.2 / 10.6, 48 x 128 of d = 128 85 / 82.  (8 warps and rows whatever the size: 7.6, 7.6, 12.8, 15.1,
-// 10.9, 84.  Rows of up to 256 blocks: 7 x 147 21.1 -> 18.5, but 2 x 200 14.2 -> 17.5 and 24 x 256 60 -> 79.)
+// Scores and selection of short rows (up to 128 blocks) in one launch: a CTA keeps the pooled K of its head in shared
+// memory and takes a few rows of it, a warp each, whose scores never leave the registers they are selected from.  Same
+// chains, same selection.  What bounds it is the latency of the launch, of bringing pooled K in (16 warps, more than
+// have a row) and of one row: few rows a CTA while all CTAs run at once, more where pooled K would be read too often.
+// us of a whole mask call, two launches / this way: 2 heads x 64 blocks of d = 64 9.7 / 7.6, 7 x 21 of d = 128 13.5 /
+// 7.7, 2 x 68 15.2 / 9.6, 5 x 108 18.3 / 12.0, 26 x 48 of d = 64 13.2 / 10.6, 48 x 128 of d = 128 85 / 82.  (8 warps
+// and rows whatever the size: 7.6, 7.6, 12.8, 15.1, 10.9, 84.  Rows of up to 256 blocks: 7 x 147 21.1 -> 18.5, but 2 x
+// 200 14.2 -> 17.5 and 24 x 256 60 -> 79.)
 // ------------------------------------------------------------------------------------------------
 constexpr int kShortWords = 4;
 constexpr int kShortWarps = 16;
@@ -459,7 +460,8 @@ __global__ void __launch_bounds__(kShortWarps * 32)
 }
 
 template <typename Params>
-static cudaError_t launch_short_rows(const Geometry& g, const float* pq, const float* pk, const Params& p, cudaStream_t st) {
+static cudaError_t launch_short_rows(const Geometry& g, const float* pq, const float* pk, const Params& p,
+                                     cudaStream_t st) {
   const int64_t BH = (int64_t)g.B * g.H;
   auto groups = [&](int rows) { return (g.NB + rows - 1) / rows; };
   const int rows = BH * groups(4) <= 148 ? 4 : BH * groups(8) <= 2 * 148 ? 8 : kShortWarps;

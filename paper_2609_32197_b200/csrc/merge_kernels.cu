@@ -8,10 +8,10 @@
 
 namespace sparsp {
 
-// hop[b][h][i][w] = (rank[i] == consumer and head_begin <= h < head_end) ? mask[b][h][i][w] & own_producer[w] : 0.
-// A lane handles one word of kHopRows rows (rows of fewer than 32 words share a warp); the producer's ownership words
-// and the consumer's rows are bits in shared memory, built once per CTA.  A mask is a few MB, so this is latency: 40
-// heads x 591 rows x 19 words in 5.0 us (11.3 us with a thread per word that walked 32 ranks for its ownership bits, 7.5 with
+// hop[b][h][i][w] = (rank[i] == consumer and head_begin <= h < head_end) ? mask[b][h][i][w] & own_producer[w] : 0.  A
+// lane handles one word of kHopRows rows (rows of fewer than 32 words share a warp); the producer's ownership words and
+// the consumer's rows are bits in shared memory, built once per CTA.  A mask is a few MB, so this is latency: 40 heads
+// x 591 rows x 19 words in 5.0 us (11.3 us with a thread per word that walked 32 ranks for its ownership bits, 7.5 with
 // a pass over the ranks for each of the two sets, 6.5 with eight rows a lane).
 constexpr int kHopThreads = 256;
 constexpr int kHopRows = 4;
@@ -77,8 +77,8 @@ __global__ void __launch_bounds__(kHopThreads) hop_mask_kernel(const uint32_t* _
 // its blocks 60 / 71 / 73; 24 x 384 of 64 x 128 75 / 91 / 75, a quarter of them 13 / 14 / 17; 48 x 279 of 64 x 64 62 /
 // 97 / 65, an eighth 11 / 15 / 13.  (Listing 1024 blocks takes longer than the merge of few heads in L2: half of the
 // blocks of 8 heads x 1024 of 64 x 64 22 / 34 / 18.)
-// A consumer's blocks are walked from behind: the attention before the merge wrote the last ones last, and they are still in
-// L2 (an attention of 40 heads x 75600 hop by hop 2539 us, 2515 this way).
+// A consumer's blocks are walked from behind: the attention before the merge wrote the last ones last, and they are
+// still in L2 (an attention of 40 heads x 75600 hop by hop 2539 us, 2515 this way).
 // O may be O_a or O_b and lse may be lse_a or lse_b (no pointer is declared restrict): a thread reads the 16 bytes it
 // later writes, and the D/8 threads of a row are consecutive lanes of one warp, all of which have read the row's
 // log-sum-exp values before its first thread writes the merged one.

@@ -162,8 +162,8 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t n_cols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(n_cols) : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// ... for loads into these registers: nothing computed from them can be moved ahead of the wait, with which the compiler sees
-// no connection otherwise.
+// ... for loads into these registers: nothing computed from them can be moved ahead of the wait, with which the
+// compiler sees no connection otherwise.
 template <int N>
 __device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[N]) {
   tmem_ld_wait();
