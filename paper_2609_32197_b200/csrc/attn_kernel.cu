@@ -49,11 +49,12 @@
 // reference last moved.  The thread that decides so waits for every P V issued so far, but only behind its
 // exponentials, which need nothing but the new reference: those of neighbouring tiles overlap.  (Waiting and rescaling
 // before them, us a call with Q times 40: 5 heads x 492 blocks of 64 x 64, 15 % kept 930, now 632; 9 x 324 of 64 x 128
-// 1787 / 1039; 4 x 300 of 128 x 128, 10 % 554 / 363.)  (The range used to be proved beforehand, by Cauchy-Schwarz from
-// key norms that a pass over K took ahead of every call and row norms taken from the Q tile of every item, and not at
-// all for a packed source, whose tiles all took their maximum in turns.  us per call then and now: one hop of 40 heads
-// x 75600 over 8 ranks, 7 tiles an item, 97-112 -> 75; 24 x 24576 from one rank's whole buffer 437-445 -> 415-425; 13
-// heads x 2 x 6034 92-101 -> 85-93; all of 40 x 75600 10.1-10.5 -> 9.7-10.2 ms.)
+// 1787 / 1039; 4 x 300 of 128 x 128, 10 % 554 / 363.  16 columns of the accumulator at a time also at d = 128: 24 x
+// 24576 from a packed buffer, Q times 60 638, now 578.)  (The range used to be proved beforehand, by Cauchy-Schwarz
+// from key norms that a pass over K took ahead of every call and row norms taken from the Q tile of every item, and not
+// at all for a packed source, whose tiles all took their maximum in turns.  us per call then and now: one hop of 40
+// heads x 75600 over 8 ranks, 7 tiles an item, 97-112 -> 75; 24 x 24576 from one rank's whole buffer 437-445 ->
+// 415-425; 13 heads x 2 x 6034 92-101 -> 85-93; all of 40 x 75600 10.1-10.5 -> 9.7-10.2 ms.)
 // The block-64 pairing and the order of a head's items (longest list first) come from attn_prep_kernel; calls of few
 // items have their CTAs put them in order (kDirect, kPackedDirect below).
 // Every mbarrier wait is bounded; a wait that runs out sets SPARSP_ERR_TIMEOUT in the status word
@@ -1182,10 +1183,15 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
       // returned.
       auto move_ref = [&](const float mx) -> float {
         const float m_new = fmaxf(m_ref, mx);
-        if (!(m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY))) return 1.0f;
-        const float alpha = ex2(m_ref - m_new);  // m_ref = -inf -> 0
-        m_ref = m_new;
-        ref[row] = m_new;
+        const bool grow = m_new > m_ref + kGrowThreshold || (m_ref == -INFINITY && m_new > -INFINITY);
+        float alpha = 1.0f;
+        if (__any_sync(0xffffffffu, grow)) {
+          alpha = grow ? ex2(m_ref - m_new) : 1.0f;  // m_ref = -inf -> 0
+          if (grow) {
+            m_ref = m_new;
+            ref[row] = m_new;
+          }
+        }
         return alpha;
       };
       // Rescales the row's accumulator, after the exponentials of the tile, which need the new reference only, and
@@ -1197,23 +1203,22 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         const int g = g0 + n;
         mbar_wait_bounded_inline(o_full + ((g - 1) & 3), ((g - 1) >> 2) & 1, s_abort, 38, p.wait_limit);
         tc_fence_after();
+        constexpr int kAtOnce = D == 128 ? 64 : 16;  // columns in flight (d = 64 has half the registers)
 #pragma unroll 1
-        for (int c = 0; c < C::kAccCols / 16; ++c) {  // the row's accumulator, 16 columns at a time (rare: kept small)
-          uint32_t o[16];
-          tmem_ld16(tO + c * 16, o);
+        for (int c = 0; c < D / kAtOnce; ++c) {  // the row's accumulator
+          uint32_t o[kAtOnce];
+#pragma unroll
+          for (int q = 0; q < kAtOnce; q += 16) tmem_ld16(tO + c * kAtOnce + q, o + q);
           tmem_ld_wait(o);
 #pragma unroll
-          for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-          tmem_st16(tO + c * 16, o);
-        }
-        if (C::kSum128) {  // the row sums live in columns of their own
-          uint32_t o[16];
-          tmem_ld16(tmem_base + C::kColL + lane_off, o);
-          tmem_ld_wait(o);
+          for (int e = 0; e < kAtOnce; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
 #pragma unroll
-          for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-          tmem_st16(tmem_base + C::kColL + lane_off, o);
+          for (int q = 0; q < kAtOnce; q += 16) tmem_st16(tO + c * kAtOnce + q, o + q);
         }
+        uint32_t sum[1];  // the row's sum (nobody reads the columns beside it)
+        tmem_ld1(tmem_base + C::kColL + lane_off, sum);
+        tmem_ld_wait(sum);
+        tmem_st1(tmem_base + C::kColL + lane_off, __float_as_uint(__uint_as_float(sum[0]) * alpha));
       };
       // A tile whose P takes the place of its scores: 32 columns at a time, the next ones on their way from tensor
       // memory.
