@@ -537,9 +537,10 @@ constexpr int kScanMax = 6144;
 // whole call with the union's launch / without: 2 heads x 64 blocks, 4 ranks 10.2 / 8.1; 7 x 21 of d = 128, 7 ranks
 // 11.5 / 8.5; 48 x 13 of 128 x 128, 7 ranks 27.0 / 23.0; 2 x 13 x 48, 3 ranks 13.3 / 11.6; 40 x 40, 8 ranks 29.9 / 28.4
 // (3200 words); beyond the line 24 x 80 (5760 words) 20.2 / 22.7, 9 x 166 (8964) 27.9 / 31.2; 16 x 64 of 128 x 128 in 7
-// blocks a warp 43.8 / 44.3.  Between four and six blocks a warp only with half of the words: 13 x 60 of 128 x 128, 4
-// ranks (1560 words) 38.2 / 36.3, but 5 x 144, 14 ranks (3600) 78.3 / 81.1, 7 x 120, 8 ranks (3360) 69.0 / 72.5.
-constexpr int kMaskMax = 4096, kFromMaskBlocks = 6, kFromMaskFew = 4;
+// blocks a warp 43.8 / 44.3.  Between four and six blocks a warp only with 2560 words at most: 13 x 60 of 128 x 128, 4
+// ranks (1560 words) 38.2 / 36.3, 9 x 80, 5 ranks (2160) 41.0 / 40.6, 2 x 13 x 48 of 64 x 128 (2496), but 5 x 144, 14
+// ranks (3600) 78.3 / 81.1, 7 x 120, 8 ranks (3360) 69.0 / 72.5, 22 x 64 of 64 x 128 (2816) 47.5 / 50.0.
+constexpr int kMaskMax = 4096, kMaskMaxMany = 2560, kFromMaskBlocks = 6, kFromMaskFew = 4;
 constexpr int kGatherStages = 3, kGatherThreads = 512;
 constexpr int kGatherSmem = 232448 - 7 * 1024;  // dynamic shared memory, next to less than 7 KB of its own
 
@@ -785,7 +786,7 @@ int launch_demand_pack(const sparsp_shape& s, const Geometry& g, const uint32_t*
   const int64_t n_words = (int64_t)g.B * g.H * g.Wd;
   int64_t smem = n_copy * kGatherStages * 2 * tile_bytes + (T + 1 + 2 * n_words + 1 + (int64_t)P * g.Wd) * 4;
   const int64_t n_mask = n_words * g.NB, blocks = (int64_t)g.B * g.H * g.NB, a_block_a_warp = 148 * n_copy;
-  const bool from_mask = n_mask <= (blocks <= kFromMaskFew * a_block_a_warp ? kMaskMax : kMaskMax / 2) &&
+  const bool from_mask = n_mask <= (blocks <= kFromMaskFew * a_block_a_warp ? kMaskMax : kMaskMaxMany) &&
                          blocks <= kFromMaskBlocks * a_block_a_warp &&
                          smem + n_words * P * 4 <= kGatherSmem;
   PackLaunch c;

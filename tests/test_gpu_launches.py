@@ -1,7 +1,7 @@
 """Which calls do without a launch, seen from the number of launches.  Attention without the one that makes its items: 64-token blocks up to
 one an SM (more of them share Q tiles), 128-token blocks up to two, and a packed source where a CTA has one item at most if the
 consumer has its share of the blocks, and the items can be put in order if it has more.  The gather without the one that makes
-the unions: up to 4096 mask words and four blocks a warp, or half of the words and six."""
+the unions: up to 4096 mask words and four blocks a warp, or 2560 words and six blocks."""
 import pytest
 import torch
 
@@ -56,7 +56,8 @@ def test_packed(binding, b, H, NB, P, launches):
     assert binding.sparsp_status(ws) == binding.SPARSP_OK
 
 
-@pytest.mark.parametrize("H,NB,launches", [(4, 128, 1), (5, 118, 1), (5, 119, 2), (13, 60, 1), (13, 64, 1), (14, 64, 2), (1, 362, 2)])
+@pytest.mark.parametrize("H,NB,launches", [(4, 144, 1), (5, 118, 1), (5, 128, 1), (5, 129, 2), (13, 64, 1), (14, 64, 2),
+                                           (1, 362, 2)])
 def test_gather(binding, H, NB, launches):
     b, d, P = 128, 128, 3  # one warp copies a block
     shape, _, K, V, mask = _inputs(binding, b, H, NB, d)
