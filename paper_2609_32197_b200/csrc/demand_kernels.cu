@@ -20,8 +20,84 @@ namespace sparsp {
 // words are rebuilt per CTA from the rank table.  Latency-bound: the mask is a few MB.  (One CTA per (batch, head) with
 // shared-memory atomics for all ranks at once: 20.6 us on 24 heads x 929 blocks, 8 ranks, 24 CTAs on 148 SMs; this
 // split 8 us.)  OR does not depend on the order, so the bits are well defined.  A rank value outside [0, P) is ignored.
-constexpr int kUnionThreads = 512;
+// Where a lane has several rows one behind the other (kLong) the lists are made without atomics and eight rows are in
+// flight, the last ones too: us a plan in a graph, atomics and four rows / this way, 24 x 929, 8 ranks 7.6 / 5.6, 40 x
+// 591, 8 ranks 8.2 / 7.4, 48 x 1000, 3 ranks 8.3 / 7.1.  With few rows the instructions that takes are what bounds many
+// CTAs: 16 x 500, 16 ranks 6.2 / 6.8, 2 x 32 x 246, 10 ranks 7.7 / 8.9, 2 x 48 x 512, 16 ranks 15.0 / 18.5.
+constexpr int kUnionThreads = 512, kUnionWarps = kUnionThreads / 32;
+constexpr int kLongRows = 4;  // rows a lane from which on
 
+__host__ __device__ __forceinline__ int lanes_per_row(int Wd) {  // the next power of two
+  int width = 1;
+  while (width < Wd) width <<= 1;
+  return width;
+}
+static bool rows_are_long(const Geometry& g, int P) {
+  return (g.NB + P - 1) / P >= kLongRows * kUnionWarps * (32 / lanes_per_row(g.Wd));
+}
+
+// own[p][Wd] of all ranks and the list of rank r's rows; returns their number.  Called by all threads, own_s zeroed
+// before.
+__device__ __forceinline__ int list_rows(const int32_t* __restrict__ rank, int NB, int Wd, int P, int r,
+                                         uint32_t* own_s, uint16_t* rows_s) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kOwn = kMaxWords / kUnionWarps;  // words of blocks a warp looks at
+  uint32_t mine[kOwn];                           // my rank's blocks of them
+  int rk[kOwn];
+#pragma unroll
+  for (int t = 0; t < kOwn; ++t) {
+    const int j = (warp + t * kUnionWarps) * 32 + lane;
+    rk[t] = j < NB ? rank[j] : -1;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kOwn; ++t) {
+    mine[t] = __ballot_sync(0xffffffffu, rk[t] == r);
+    const uint32_t same = __match_any_sync(0xffffffffu, rk[t]);
+    if ((unsigned)rk[t] < (unsigned)P && lane == __ffs(same) - 1) own_s[rk[t] * Wd + warp + t * kUnionWarps] = same;
+  }
+  __syncthreads();
+  int n_rows;
+  const int before = bits_below(lane < Wd ? own_s[r * Wd + lane] : 0u, lane, &n_rows);
+#pragma unroll
+  for (int t = 0; t < kOwn; ++t) {
+    const int first = __shfl_sync(0xffffffffu, before, (warp + t * kUnionWarps) & 31);
+    if ((mine[t] >> lane) & 1u)
+      rows_s[first + __popc(mine[t] & ((1u << lane) - 1u))] = (uint16_t)((warp + t * kUnionWarps) * 32 + lane);
+  }
+  __syncthreads();
+  return n_rows;
+}
+
+// OR of the listed rows of one mask m[NB][Wd], a word per lane.  Called by all lanes of a warp, which takes its share.
+template <int kInFlight>
+__device__ __forceinline__ uint32_t or_rows(const uint32_t* __restrict__ m, const uint16_t* rows_s, int n_rows, int Wd,
+                                            int width) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per_warp = 32 / width, w = lane & (width - 1), first = warp * per_warp + lane / width;
+  const int step = kUnionWarps * per_warp;
+  uint32_t acc = 0;
+  if constexpr (kInFlight == 4) {
+#pragma unroll 4
+    for (int k = first; k < n_rows; k += step)
+      if (w < Wd) acc |= m[(int64_t)rows_s[k] * Wd + w];
+  } else {
+    for (int k0 = first; k0 < n_rows; k0 += kInFlight * step) {
+      uint32_t v[kInFlight];
+#pragma unroll
+      for (int u = 0; u < kInFlight; ++u) {
+        const int k = k0 + u * step;
+        v[u] = k < n_rows && w < Wd ? m[(int64_t)rows_s[k] * Wd + w] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < kInFlight; ++u) acc |= v[u];
+    }
+  }
+  for (int s = width; s < 32; s <<= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, s);
+  return acc;
+}
+
+template <bool kLong>
 __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32_t* __restrict__ mask,
                                                                     const int32_t* __restrict__ rank, int H, int NB,
                                                                     int Wd, int P, uint32_t* __restrict__ U,
@@ -38,20 +114,19 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
   if (threadIdx.x == 0) n_rows_s = 0;
   if (threadIdx.x < kMaxWords) u_s[threadIdx.x] = 0u;
   if (blockIdx.x == 0 && threadIdx.x == 0 && n_src) *n_src = 0;
-  own_words(rank, NB, Wd, P, own_s);
-  for (int i = threadIdx.x; i < NB; i += kUnionThreads)
-    if (rank[i] == r) rows_s[atomicAdd(&n_rows_s, 1)] = (uint16_t)i;
-  __syncthreads();
-  int width = 1;  // lanes per row: the next power of two
-  while (width < Wd) width <<= 1;
-  const int per_warp = 32 / width, w = lane & (width - 1), sub = lane / width;
   const uint32_t* m = mask + (int64_t)bh * NB * Wd;
-  uint32_t acc = 0;
-  const int n_rows = n_rows_s;
-#pragma unroll 4
-  for (int k = warp * per_warp + sub; k < n_rows; k += n_warps * per_warp)
-    if (w < Wd) acc |= m[(int64_t)rows_s[k] * Wd + w];
-  for (int s = width; s < 32; s <<= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, s);
+  uint32_t acc;
+  if constexpr (kLong) {
+    for (int i = threadIdx.x; i < P * Wd; i += kUnionThreads) own_s[i] = 0u;
+    const int n_rows = list_rows(rank, NB, Wd, P, r, own_s, rows_s);
+    acc = or_rows<8>(m, rows_s, n_rows, Wd, lanes_per_row(Wd));
+  } else {
+    own_words(rank, NB, Wd, P, own_s);
+    for (int i = threadIdx.x; i < NB; i += kUnionThreads)
+      if (rank[i] == r) rows_s[atomicAdd(&n_rows_s, 1)] = (uint16_t)i;
+    __syncthreads();
+    acc = or_rows<4>(m, rows_s, n_rows_s, Wd, lanes_per_row(Wd));
+  }
   if (lane < Wd && acc) atomicOr(&u_s[lane], acc);
   __syncthreads();
   const uint32_t u = lane < Wd ? u_s[lane] : 0u;
@@ -71,16 +146,13 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
 
 // Unions, counts and offsets of a plan without destinations, in one launch: a cluster of CTAs per consumer takes the
 // consumer's heads in turn, meets when all counts are there, and its first CTA scans them.  Nothing is kept between
-// launches.  Latency-bound, and what is saved is the host's time for a launch.  So a CTA makes its lists by ballots,
-// matches and counting bits, with eight rows in flight, the last ones too (the lists of the kernel above, of atomics,
-// are fewer instructions, which is what bounds it where CTAs are many: 2 x 48 heads x 512 blocks, 16 ranks 15.0 us a
-// plan against 18.5 with lists like these).  us a plan with two launches / this way, one call behind the other and in a
-// graph, where the host is out of it: 2 heads x 64 blocks, 4 ranks 7.4 / 5.1 and 4.0 / 3.9; 4 x 1000, 8 ranks 7.6 / 5.1
-// and 5.8 / 4.7; 13 x 77, 5 ranks 7.6 / 5.1 and 4.3 / 4.5; 16 x 177, 8 ranks 7.6 / 5.2 and 4.6 / 4.7; 24 x 384, 4 ranks
-// 8.0 / 5.8 and 4.9 / 5.4.  Several heads a CTA take too long where rows are many and wide, 16 x 1000, 2 ranks 8.3 /
-// 9.0 and 7.6 / 8.5, 24 x 929, 8 ranks 7.5 / 8.3 and 7.0 / 7.0, where there are more than eight clusters, 16 x 300, 11
-// ranks 7.6 / 6.7 and 5.0 / 6.8, 24 x 300 7.8 / 8.7 and 6.1 / 8.1, and so do more than three: 48 x 278, 3 ranks 7.6 /
-// 7.9 and 5.2 / 7.5.
+// launches.  Latency-bound, and what is saved is the host's time for a launch.  us a plan with two launches / this way,
+// one call behind the other and in a graph, where the host is out of it: 2 heads x 64 blocks, 4 ranks 7.4 / 5.1 and 4.0
+// / 3.9; 4 x 1000, 8 ranks 7.6 / 5.1 and 5.8 / 4.7; 13 x 77, 5 ranks 7.6 / 5.1 and 4.3 / 4.5; 16 x 177, 8 ranks 7.6 /
+// 5.2 and 4.6 / 4.7; 24 x 384, 4 ranks 8.0 / 5.8 and 4.9 / 5.4.  Several heads a CTA take too long where rows are many
+// and wide, 16 x 1000, 2 ranks 8.3 / 9.0 and 7.6 / 8.5, 24 x 929, 8 ranks 7.5 / 8.3 and 7.0 / 7.0, where there are more
+// than eight clusters, 16 x 300, 11 ranks 7.6 / 6.7 and 5.0 / 6.8, 24 x 300 7.8 / 8.7 and 6.1 / 8.1, and so do more
+// than three: 48 x 278, 3 ranks 7.6 / 7.9 and 5.2 / 7.5.
 constexpr int kPlanCtas = 8, kPlanHeads = 3;                    // CTAs of a cluster, heads that one takes
 constexpr int kPlanAtOnce = 64;                                // CTAs of a launch, where they take several heads
 constexpr int kPlanWordsOfTwo = 20480, kPlanWordsOfThree = 4096;  // mask words of two and of three heads
@@ -103,52 +175,13 @@ __global__ void __launch_bounds__(kUnionThreads)
   const int ctas = min(H, kPlanCtas), br = blockIdx.x / ctas, bb = br / P, r = br - bb * P;
   const int h0 = blockIdx.x - br * ctas, n_heads = (H - h0 + ctas - 1) / ctas;  // heads h0, h0 + ctas, ...
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int n_warps = kUnionThreads / 32;
+  constexpr int n_warps = kUnionWarps;
   for (int i = threadIdx.x; i < kPlanHeads * kMaxWords; i += kUnionThreads) (&u_s[0][0])[i] = 0u;
   for (int i = threadIdx.x; i < P * Wd; i += kUnionThreads) own_s[i] = 0u;
-  constexpr int kOwn = kMaxWords / n_warps;  // words of blocks a warp looks at
-  uint32_t mine[kOwn];                       // my rank's blocks of them
-  int rk[kOwn];
-#pragma unroll
-  for (int t = 0; t < kOwn; ++t) {
-    const int j = (warp + t * n_warps) * 32 + lane;
-    rk[t] = j < NB ? rank[j] : -1;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int t = 0; t < kOwn; ++t) {
-    mine[t] = __ballot_sync(0xffffffffu, rk[t] == r);
-    const uint32_t same = __match_any_sync(0xffffffffu, rk[t]);
-    if ((unsigned)rk[t] < (unsigned)P && lane == __ffs(same) - 1) own_s[rk[t] * Wd + warp + t * n_warps] = same;
-  }
-  __syncthreads();
-  int n_rows;
-  const int before = bits_below(lane < Wd ? own_s[r * Wd + lane] : 0u, lane, &n_rows);
-#pragma unroll
-  for (int t = 0; t < kOwn; ++t) {
-    const int first = __shfl_sync(0xffffffffu, before, (warp + t * n_warps) & 31);
-    if ((mine[t] >> lane) & 1u)
-      rows_s[first + __popc(mine[t] & ((1u << lane) - 1u))] = (uint16_t)((warp + t * n_warps) * 32 + lane);
-  }
-  __syncthreads();
-  int width = 1;  // lanes per row: the next power of two
-  while (width < Wd) width <<= 1;
-  const int per_warp = 32 / width, w = lane & (width - 1), sub = lane / width;
+  const int n_rows = list_rows(rank, NB, Wd, P, r, own_s, rows_s);
+  const int width = lanes_per_row(Wd);
   for (int k = 0; k < n_heads; ++k) {
-    const uint32_t* m = mask + (int64_t)(bb * H + h0 + k * ctas) * NB * Wd;
-    uint32_t acc = 0;
-    constexpr int kRows = 8;  // rows in flight, the last ones too
-    for (int k0 = warp * per_warp + sub; k0 < n_rows; k0 += kRows * n_warps * per_warp) {
-      uint32_t v[kRows];
-#pragma unroll
-      for (int u = 0; u < kRows; ++u) {
-        const int at = k0 + u * n_warps * per_warp;
-        v[u] = at < n_rows && w < Wd ? m[(int64_t)rows_s[at] * Wd + w] : 0u;
-      }
-#pragma unroll
-      for (int u = 0; u < kRows; ++u) acc |= v[u];
-    }
-    for (int s = width; s < 32; s <<= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, s);
+    const uint32_t acc = or_rows<8>(mask + (int64_t)(bb * H + h0 + k * ctas) * NB * Wd, rows_s, n_rows, Wd, width);
     if (lane < Wd && acc) atomicOr(&u_s[k][lane], acc);
   }
   __syncthreads();
@@ -347,7 +380,8 @@ static int32_t* received_table(char* ws, const WsLayout& L, const Geometry& g, i
 
 static cudaError_t launch_union(const Geometry& g, const uint32_t* mask, const int32_t* rank, int P, int include_local,
                                 uint32_t* U, int32_t* cnt, int32_t* received, int32_t* n_src, cudaStream_t st) {
-  return launch_kernel(union_count_kernel, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P, U,
+  auto kern = rows_are_long(g, P) ? union_count_kernel<true> : union_count_kernel<false>;
+  return launch_kernel(kern, g.B * g.H * P, kUnionThreads, 0, st, mask, rank, g.H, g.NB, g.Wd, P, U,
                        include_local, cnt, received, n_src);
 }
 
