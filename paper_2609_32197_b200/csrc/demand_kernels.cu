@@ -69,32 +69,35 @@ __device__ __forceinline__ int list_rows(const int32_t* __restrict__ rank, int N
   return n_rows;
 }
 
-// OR of the listed rows of one mask m[NB][Wd], a word per lane.  Called by all lanes of a warp, which takes its share.
-template <int kInFlight>
-__device__ __forceinline__ uint32_t or_rows(const uint32_t* __restrict__ m, const uint16_t* rows_s, int n_rows, int Wd,
-                                            int width) {
+// OR of the listed rows of kHeads masks m[NB][Wd], `pitch` words apart, of which the first n_heads are there, a word
+// per lane and mask.  Called by all lanes of a warp, which takes its share of the rows, kInFlight of every mask at a
+// time.
+template <int kHeads, int kInFlight>
+__device__ __forceinline__ void or_rows(const uint32_t* __restrict__ m, int64_t pitch, int n_heads,
+                                        const uint16_t* rows_s, int n_rows, int Wd, int width,
+                                        uint32_t (&acc)[kHeads]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int per_warp = 32 / width, w = lane & (width - 1), first = warp * per_warp + lane / width;
-  const int step = kUnionWarps * per_warp;
-  uint32_t acc = 0;
-  if constexpr (kInFlight == 4) {
-#pragma unroll 4
-    for (int k = first; k < n_rows; k += step)
-      if (w < Wd) acc |= m[(int64_t)rows_s[k] * Wd + w];
-  } else {
-    for (int k0 = first; k0 < n_rows; k0 += kInFlight * step) {
-      uint32_t v[kInFlight];
+  const int per_warp = 32 / width, w = lane & (width - 1), step = kUnionWarps * per_warp;
 #pragma unroll
-      for (int u = 0; u < kInFlight; ++u) {
-        const int k = k0 + u * step;
-        v[u] = k < n_rows && w < Wd ? m[(int64_t)rows_s[k] * Wd + w] : 0u;
-      }
+  for (int h = 0; h < kHeads; ++h) acc[h] = 0u;
+  for (int k0 = warp * per_warp + lane / width; k0 < n_rows; k0 += kInFlight * step) {
+    uint32_t v[kHeads][kInFlight];
 #pragma unroll
-      for (int u = 0; u < kInFlight; ++u) acc |= v[u];
+    for (int u = 0; u < kInFlight; ++u) {
+      const int k = k0 + u * step;
+      const bool there = k < n_rows && w < Wd;
+      const uint32_t* at = m + (there ? (int64_t)rows_s[k] * Wd + w : 0);
+#pragma unroll
+      for (int h = 0; h < kHeads; ++h) v[h][u] = there && h < n_heads ? at[h * pitch] : 0u;
     }
+#pragma unroll
+    for (int h = 0; h < kHeads; ++h)
+#pragma unroll
+      for (int u = 0; u < kInFlight; ++u) acc[h] |= v[h][u];
   }
-  for (int s = width; s < 32; s <<= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, s);
-  return acc;
+#pragma unroll
+  for (int h = 0; h < kHeads; ++h)
+    for (int s = width; s < 32; s <<= 1) acc[h] |= __shfl_xor_sync(0xffffffffu, acc[h], s);
 }
 
 template <bool kLong>
@@ -115,17 +118,24 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
   if (threadIdx.x < kMaxWords) u_s[threadIdx.x] = 0u;
   if (blockIdx.x == 0 && threadIdx.x == 0 && n_src) *n_src = 0;
   const uint32_t* m = mask + (int64_t)bh * NB * Wd;
-  uint32_t acc;
+  const int width = lanes_per_row(Wd);
+  uint32_t acc = 0;
   if constexpr (kLong) {
     for (int i = threadIdx.x; i < P * Wd; i += kUnionThreads) own_s[i] = 0u;
     const int n_rows = list_rows(rank, NB, Wd, P, r, own_s, rows_s);
-    acc = or_rows<8>(m, rows_s, n_rows, Wd, lanes_per_row(Wd));
+    uint32_t all[1];
+    or_rows<1, 8>(m, 0, 1, rows_s, n_rows, Wd, width, all);
+    acc = all[0];
   } else {
     own_words(rank, NB, Wd, P, own_s);
     for (int i = threadIdx.x; i < NB; i += kUnionThreads)
       if (rank[i] == r) rows_s[atomicAdd(&n_rows_s, 1)] = (uint16_t)i;
     __syncthreads();
-    acc = or_rows<4>(m, rows_s, n_rows_s, Wd, lanes_per_row(Wd));
+    const int n_rows = n_rows_s, per_warp = 32 / width, w = lane & (width - 1);
+#pragma unroll 4
+    for (int k = warp * per_warp + lane / width; k < n_rows; k += n_warps * per_warp)
+      if (w < Wd) acc |= m[(int64_t)rows_s[k] * Wd + w];
+    for (int s = width; s < 32; s <<= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, s);
   }
   if (lane < Wd && acc) atomicOr(&u_s[lane], acc);
   __syncthreads();
@@ -148,19 +158,17 @@ __global__ void __launch_bounds__(kUnionThreads) union_count_kernel(const uint32
 // consumer's heads in turn, meets when all counts are there, and its first CTA scans them.  Nothing is kept between
 // launches.  Latency-bound, and what is saved is the host's time for a launch.  us a plan with two launches / this way,
 // one call behind the other and in a graph, where the host is out of it: 2 heads x 64 blocks, 4 ranks 7.4 / 5.1 and 4.0
-// / 3.9; 4 x 1000, 8 ranks 7.6 / 5.1 and 5.8 / 4.7; 13 x 77, 5 ranks 7.6 / 5.1 and 4.3 / 4.5; 16 x 177, 8 ranks 7.6 /
-// 5.2 and 4.6 / 4.7; 24 x 384, 4 ranks 8.0 / 5.8 and 4.9 / 5.4.  Several heads a CTA take too long where rows are many
-// and wide, 16 x 1000, 2 ranks 8.3 / 9.0 and 7.6 / 8.5, 24 x 929, 8 ranks 7.5 / 8.3 and 7.0 / 7.0, where there are more
-// than eight clusters, 16 x 300, 11 ranks 7.6 / 6.7 and 5.0 / 6.8, 24 x 300 7.8 / 8.7 and 6.1 / 8.1, and so do more
-// than three: 48 x 278, 3 ranks 7.6 / 7.9 and 5.2 / 7.5.
-constexpr int kPlanCtas = 8, kPlanHeads = 3;                    // CTAs of a cluster, heads that one takes
-constexpr int kPlanAtOnce = 64;                                // CTAs of a launch, where they take several heads
-constexpr int kPlanWordsOfTwo = 20480, kPlanWordsOfThree = 4096;  // mask words of two and of three heads
+// / 3.8; 4 x 1000, 8 ranks 7.6 / 5.1 and 5.6 / 4.4; 13 x 77, 5 ranks 7.6 / 5.4 and 4.3 / 4.3; 24 x 384, 4 ranks 8.2 /
+// 5.3 and 4.9 / 4.4; 24 x 300, 11 ranks 7.9 / 5.4 and 6.1 / 6.0; 16 x 500, 2 ranks 7.7 / 5.2 and 4.4 / 5.2.  Beyond the
+// line 24 x 929, 8 ranks (10530 words a CTA) 7.6 / 6.8 and 5.8 / 6.5, 12 x 600, 2 ranks (11400) 7.5 / 7.3 and 5.3 /
+// 7.1, 9 x 1000, 3 ranks (21376) 7.5 / 8.0 and 5.5 / 7.8.  (The heads of a CTA one after the other: 24 x 384 5.8 and
+// 5.5, 21 x 22, 7 ranks 6.1 and 5.4, now 5.3 and 4.9.)
+constexpr int kPlanCtas = 8, kPlanHeads = 3;  // CTAs of a cluster, heads that one takes
+constexpr int kPlanWords = 10240;             // mask words of two or three heads
 static bool plan_fits_clusters(const Geometry& g, int P, int sms) {
   const int ctas = std::min(g.H, kPlanCtas), heads = (g.H + ctas - 1) / ctas, rows = (g.NB + P - 1) / P;
-  const int words = heads == 1 ? 0 : heads * rows * g.Wd, most = heads <= 2 ? kPlanWordsOfTwo : kPlanWordsOfThree;
-  return heads <= kPlanHeads && words <= most && g.H * P <= kUnionThreads &&
-         g.B * P * ctas <= (heads == 1 ? sms : kPlanAtOnce);
+  return heads <= kPlanHeads && (heads == 1 || heads * rows * g.Wd <= kPlanWords) && g.H * P <= kUnionThreads &&
+         g.B * P * ctas <= sms;
 }
 
 __global__ void __launch_bounds__(kUnionThreads)
@@ -180,9 +188,18 @@ __global__ void __launch_bounds__(kUnionThreads)
   for (int i = threadIdx.x; i < P * Wd; i += kUnionThreads) own_s[i] = 0u;
   const int n_rows = list_rows(rank, NB, Wd, P, r, own_s, rows_s);
   const int width = lanes_per_row(Wd);
-  for (int k = 0; k < n_heads; ++k) {
-    const uint32_t acc = or_rows<8>(mask + (int64_t)(bb * H + h0 + k * ctas) * NB * Wd, rows_s, n_rows, Wd, width);
-    if (lane < Wd && acc) atomicOr(&u_s[k][lane], acc);
+  const uint32_t* m = mask + (int64_t)(bb * H + h0) * NB * Wd;
+  const int64_t pitch = (int64_t)ctas * NB * Wd;
+  if (n_heads == 1) {
+    uint32_t acc[1];
+    or_rows<1, 8>(m, pitch, 1, rows_s, n_rows, Wd, width, acc);
+    if (lane < Wd && acc[0]) atomicOr(&u_s[0][lane], acc[0]);
+  } else {
+    uint32_t acc[kPlanHeads];
+    or_rows<kPlanHeads, 4>(m, pitch, n_heads, rows_s, n_rows, Wd, width, acc);
+#pragma unroll
+    for (int k = 0; k < kPlanHeads; ++k)
+      if (lane < Wd && acc[k]) atomicOr(&u_s[k][lane], acc[k]);
   }
   __syncthreads();
   for (int i = warp; i < n_heads * P; i += n_warps) {

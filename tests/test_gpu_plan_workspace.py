@@ -16,7 +16,8 @@ def binding():
 
 
 @pytest.mark.parametrize("B,P,H,NB", [(1, 1, 1, 1), (1, 2, 3, 33), (1, 4, 2, 64), (2, 9, 8, 70), (1, 18, 8, 90), (1, 19, 8, 90), (1, 5, 9, 100),
-                                      (1, 18, 16, 40), (1, 8, 17, 929), (1, 8, 16, 1024), (1, 2, 16, 1024), (1, 2, 12, 800), (1, 4, 24, 384), (1, 2, 25, 64),
+                                      (1, 18, 16, 40), (1, 8, 17, 929), (1, 8, 16, 1024), (1, 2, 16, 1024), (1, 2, 12, 600), (1, 8, 24, 929),
+                                      (1, 11, 21, 130), (1, 2, 16, 500), (1, 4, 24, 384), (1, 2, 25, 64),
                                       (1, 37, 4, 96), (1, 64, 2, 200), (49, 3, 1, 20), (1, 2, 48, 300)])
 @pytest.mark.parametrize("fill", [0, -1, 2])
 def test_plan_on_any_workspace(binding, B, P, H, NB, fill):
