@@ -189,7 +189,8 @@ constexpr int kHeadMeet = 1 << 21, kHeadMeetParityShift = 22;
 //                  and put the items in order if there are more of them than CTAs
 enum class Source { kQueue, kDirect, kPacked, kPackedDirect };
 
-constexpr int kMaxDirect = 2 * 148, kMaxPackedDirect = 512;  // items of a call without a queue
+constexpr int kMaxDirect = 2 * 148, kMaxPackedDirect = 1024;  // items of a call without a queue
+constexpr int kPackedDirectBlocks = 512;  // blocks of a head up to which that many
 
 template <int D, int BLK>
 struct AttnCfg {
@@ -497,7 +498,7 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
       }
     }
     // More items than CTAs, because the consumer has more than its share of the blocks: every CTA puts them in order by
-    // counting their lengths.  An item is a block or two neighbours, a thread has one at most.  Items of one length
+    // counting their lengths.  An item is a block or two neighbours, a thread has up to kPer.  Items of one length
     // stay in order of their numbers: all CTAs have to come to the same order.
     int n_own = 0, own_before = 0, per_head = 0, n = p.BH * ((p.NB + C::kEPT - 1) / C::kEPT);
     uint32_t own = 0u;
@@ -519,20 +520,26 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
         if ((word >> lane) & 1u) blocks[first + __popc(word & ((1u << lane) - 1u))] = (uint16_t)(w * 32 + lane);
       }
       __syncthreads();
-      static_assert(kMaxPackedDirect <= C::kThreads, "a thread per item");
-      int place = -1;  // NB - length, where I have an item
-      if (tid < n) {
-        const int bh = tid / per_head, x = (tid - bh * per_head) * C::kEPT;
-        const uint32_t* rows = p.mask + (int64_t)bh * p.NB * p.Wd;
-        const uint32_t *row0 = rows + blocks[x] * p.Wd, *row1 = rows + blocks[min(x + C::kEPT - 1, n_own - 1)] * p.Wd;
-        place = p.NB;
+      constexpr int kPer = (kMaxPackedDirect + C::kThreads - 1) / C::kThreads;
+      int place[kPer];  // NB - length, -1 where there is no item
+      uint32_t peers[kPer];
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const int t = tid + u * C::kThreads;
+        place[u] = -1;
+        if (t < n) {
+          const int bh = t / per_head, x = (t - bh * per_head) * C::kEPT;
+          const uint32_t* rows = p.mask + (int64_t)bh * p.NB * p.Wd;
+          const uint32_t* row0 = rows + blocks[x] * p.Wd;
+          const uint32_t* row1 = rows + blocks[min(x + C::kEPT - 1, n_own - 1)] * p.Wd;
+          int left = p.NB;
 #pragma unroll 8
-        for (int w = 0; w < p.Wd; ++w) place -= __popc(C::kStacked ? row0[w] | row1[w] : row0[w]);
-        place = max(place, 0);  // (a mask has no bits behind its NB-th)
+          for (int w = 0; w < p.Wd; ++w) left -= __popc(C::kStacked ? row0[w] | row1[w] : row0[w]);
+          place[u] = max(left, 0);  // (a mask has no bits behind its NB-th)
+        }
+        peers[u] = __match_any_sync(0xffffffffu, place[u]);
+        if (t < n && lane == __ffs(peers[u]) - 1) atomicAdd(at + place[u], __popc(peers[u]));
       }
-      const uint32_t peers = __match_any_sync(0xffffffffu, place);
-      const int leader = __ffs(peers) - 1;
-      if (tid < n && lane == leader) atomicAdd(at + place, __popc(peers));
       __syncthreads();
       if (warp == 0) {
         int before = 0;
@@ -548,16 +555,20 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
           before += __shfl_sync(0xffffffffu, incl, 31);
         }
       }
-      for (int k = 0; k * 32 < n; ++k) {  // warp by warp
-        __syncthreads();
-        if (warp == k) {
-          int first = 0;
-          if (tid < n && lane == leader) {
-            first = at[place];
-            at[place] = first + __popc(peers);
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const int t = tid + u * C::kThreads, leader = __ffs(peers[u]) - 1;
+        for (int k = 0; k < kWarps && u * C::kThreads + k * 32 < n; ++k) {  // warp by warp
+          __syncthreads();
+          if (warp == k) {
+            int first = 0;
+            if (t < n && lane == leader) {
+              first = at[place[u]];
+              at[place[u]] = first + __popc(peers[u]);
+            }
+            first = __shfl_sync(0xffffffffu, first, leader);
+            if (t < n) sOrder[first + __popc(peers[u] & ((1u << lane) - 1u))] = (uint16_t)t;
           }
-          first = __shfl_sync(0xffffffffu, first, leader);
-          if (tid < n) sOrder[first + __popc(peers & ((1u << lane) - 1u))] = (uint16_t)tid;
         }
       }
     }
@@ -2095,16 +2106,18 @@ int launch_attn_packed(const sparsp_shape& s, const Geometry& g, const void* Q, 
   // Where the consumer has one item an SM at most, if it has its share of the blocks, neither their order nor a queue
   // matters, and the launch that makes them is left out: us a call over a whole buffer, with the launch / without, 1
   // head x 43 blocks, 5 ranks 18.5 / 16.4; an even share of 8 ranks, 15 % kept, 2 x 140 of 64 x 128 26.8 / 25.0, 4 x 97
-  // of 64 x 128 21.2 / 19.1, 8 x 128 of 64 x 128 27.1 / 24.7; a hop of 6 x 140 15.2 / 13.0.  If the consumer has more
-  // than its share, the CTAs put its items in order for themselves, up to 512 of them: 30 % of 8 x 128 42.9 / 42.0,
-  // with lists of unequal length 49.3 / 37.9, all of it 80.7 / 79.4, but short lists, 4 % kept, 39.9 / 43.3.  (In order
-  // of their numbers lists of unequal length took up to 1.7 times as long, half of 1 x 300 of 128 x 128 75 / 110.  With
-  // two items an SM by an even share 4 x 300 of 128 x 128 34 / 44; with up to 1024 to put in order 2 x 1000 of 64 x 128
-  // 240 / 265.)
+  // of 64 x 128 21.2 / 19.1, 8 x 256 of 64 x 64 32.0 / 30.1, 7 x 146 of 128 x 128 33.2 / 30.1; a hop of 6 x 140 15.2 /
+  // 13.0.  If the consumer has more than its share, the CTAs put its items in order for themselves, up to 1024 of them
+  // (512 of heads of more than 512 blocks): 30 % of 8 x 128 of 64 x 128 42.9 / 42.0, with lists of unequal length 49.3
+  // / 37.9, 30 % of 7 x 146 81.2 / 82.5 and 91.6 / 74.6, but all of short lists, 4 % kept, 8 x 128 39.9 / 43.3, 8 x 256
+  // 64.8 / 76.6.  (In order of their numbers lists of unequal length took up to 1.7 times as long, half of 1 x 300 of
+  // 128 x 128 75 / 110.  With two items an SM by an even share 4 x 300 of 128 x 128 34 / 44; 30 % of 2 x 1000 of 64 x
+  // 128, whose rows are wide, 240 / 265.)
   int sms = 0;
   SPARSP_CUDA_OK(sm_count(&sms));
   const int64_t BH = (int64_t)g.B * g.H, share = (g.NB + P - 1) / P, per_item = 128 / g.b;
-  if (BH * ((share + per_item - 1) / per_item) <= sms && BH * ((g.NB + per_item - 1) / per_item) <= kMaxPackedDirect) {
+  const int64_t most = g.NB <= kPackedDirectBlocks ? kMaxPackedDirect : kMaxPackedDirect / 2;
+  if (BH * ((share + per_item - 1) / per_item) <= sms && BH * ((g.NB + per_item - 1) / per_item) <= most) {
     p.P = P;
     p.U = U;
     p.seg_off = seg_off;

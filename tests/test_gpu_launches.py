@@ -39,8 +39,9 @@ def test_own_keys(binding, b, per_sm, more):
 @pytest.mark.parametrize("b,H,NB,P,launches", [
     # one item an SM (148) by an even share of the blocks, and one more
     (128, 1, 148, 1, 1), (128, 1, 149, 1, 2), (64, 1, 296, 1, 1), (64, 1, 297, 1, 2), (128, 4, 74, 2, 1), (128, 4, 76, 2, 2),
-    # 512 items if it owns all blocks, and more
-    (128, 4, 128, 4, 1), (128, 4, 129, 4, 2), (64, 4, 256, 8, 1), (64, 4, 257, 8, 2)])
+    # 1024 items if it owns all blocks, and more; half of that with more than 512 blocks a head
+    (128, 8, 128, 8, 1), (128, 8, 129, 8, 2), (64, 4, 512, 8, 1), (64, 2, 513, 8, 2), (128, 1, 512, 8, 1),
+    (128, 1, 513, 8, 2), (64, 1, 1024, 8, 1)])
 def test_packed(binding, b, H, NB, P, launches):
     shape, Q, K, V, mask = _inputs(binding, b, H, NB)
     ws = binding.make_workspace(shape, P)

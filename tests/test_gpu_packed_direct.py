@@ -1,5 +1,5 @@
 """Attention over a packed buffer with and without the launch that numbers items and places: both sides of the rule between
-them (an item an SM if the consumer has its share of the blocks, 512 if it has all of them), consumers that own nearly all, one
+them (an item an SM if the consumer has its share of the blocks, 1024 if it has all of them), consumers that own nearly all, one
 or none of the blocks, 64 ranks, batches, explicit slot bases, empty rows and heads, keys far out of range.  Foreign K and V are
 not numbers; rows and their log-sum-exps against a masked softmax in 64 bits."""
 import math
@@ -83,7 +83,7 @@ def test_packed_rows(binding, d, b, B, H, NB, P, owner, bases, far):
 # consumers with far more than their share, whose items the CTAs put in order: as many as there is room for, one more, batches
 @pytest.mark.parametrize("d,b", [(64, 64), (128, 64), (64, 128), (128, 128)])
 @pytest.mark.parametrize("B,H,NB,P", [(1, 8, 60, 8), (1, 8, 64, 8), (2, 4, 64, 8), (1, 16, 64, 8), (1, 16, 65, 8), (1, 2, 200, 16),
-                                      (3, 5, 34, 4), (1, 1, 480, 8)])
+                                      (3, 5, 34, 4), (1, 1, 480, 8), (1, 16, 128, 16)])
 @pytest.mark.parametrize("far", [1.0, 60.0])
 def test_more_than_its_share(binding, d, b, B, H, NB, P, far):
     if NB > 260 and b == 128:
