@@ -500,16 +500,17 @@ __global__ void __launch_bounds__(AttnCfg<D, BLK>::kThreads, 1)
     // More items than CTAs, because the consumer has more than its share of the blocks: every CTA puts them in order by
     // counting their lengths.  An item is a block or two neighbours, a thread has up to kPer.  Items of one length
     // stay in order of their numbers: all CTAs have to come to the same order.
-    int n_own = 0, own_before = 0, per_head = 0, n = p.BH * ((p.NB + C::kEPT - 1) / C::kEPT);
-    uint32_t own = 0u;
+    int n_own = 0, per_head = 0, n = p.BH * ((p.NB + C::kEPT - 1) / C::kEPT);
     if (n > (int)gridDim.x) {  // (as many as if all blocks were the consumer's)
-      __syncthreads();
-      own = lane < p.Wd ? sOwn[p.consumer * p.Wd + lane] : 0u;
-      own_before = bits_below(own, lane, &n_own);
+#pragma unroll
+      for (int t = 0; t < kRounds; ++t)
+        if (t * C::kThreads < p.NB) n_own += __syncthreads_count(rk[t] == p.consumer);
       per_head = (n_own + C::kEPT - 1) / C::kEPT;
       n = p.BH * per_head;
     }
     if (n > (int)gridDim.x) {
+      const uint32_t own = lane < p.Wd ? sOwn[p.consumer * p.Wd + lane] : 0u;
+      const int own_before = bits_below(own, lane, &n_own);
       // [NB + 1] place NB - length: items of that length, then where they begin
       int* at = reinterpret_cast<int*>(smem + C::kOffEnt);
       uint16_t* blocks = reinterpret_cast<uint16_t*>(smem + C::kOffFirst);
